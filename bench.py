@@ -420,7 +420,8 @@ def run_ours(args):
                            "l2": f"{N_ROTATE} rotating input/output buffer sets ({N_ROTATE * 2 * B * T * D * 2 / 1e6:.0f} MB) > 126 MB L2",
                            "prewarm": f"{PREWARM_S * 1e3:.0f} ms of untimed launches of the step before the {args.warmup} warm-up steps",
                            "launch": f"the {args.steps} timed steps are {args.steps} API calls captured in one CUDA graph and replayed once",
-                           "kernel_path": "sm100" if binding.workspace_bytes(shape, binding.OP_PREFILL) > 256 else "generic"},
+                           "kernel_path": "sm100" if (binding.workspace_bytes(shape, binding.OP_PREFILL) != binding.workspace_bytes(
+                               binding.make_shape(*(getattr(shape, k) for k in "BTDH"), torch.bfloat16, flags=binding.FLAG_FORCE_GENERIC), binding.OP_PREFILL)) else "generic"},
                 "clocks": clocks, "gpu_launches": args.steps,
                 "e2e": {"value": world * B * T / (e2e_ms * 1e-3), "unit": "tokens/s", "h2d_bytes_per_step": h2d,
                         "d2h_bytes_per_step": d2h, "ms_per_step": e2e_ms, "steps": e2e_steps},

@@ -112,7 +112,7 @@ size_t rglru_workspace_bytes(const rglru_shape_t *s, int32_t op) {
     size_t body = 0;
     switch (op) {
         case RGLRU_OP_PREFILL:
-            if (use_sm100_prefill(s)) body = sm100_prefill_workspace_bytes(s->B, s->T, s->D, s->H);
+            body = use_sm100_prefill(s) ? sm100_prefill_workspace_bytes(s->B, s->T, s->D, s->H) : generic_prefill_workspace_bytes(s->B, s->D, s->io);
             break;
         case RGLRU_OP_DECODE: break;
         case RGLRU_OP_BACKWARD:
@@ -156,7 +156,7 @@ int32_t rglru_prefill_ex(const rglru_shape_t *s, const rglru_params_t *p, const 
     if (use_sm100_prefill(s))
         e = sm100_prefill(a, (char *)workspace + WS_HEADER_BYTES, workspace_bytes - WS_HEADER_BYTES, st);
     else
-        e = generic_prefill(a, s->io, st);
+        e = generic_prefill(a, s->io, (char *)workspace + WS_HEADER_BYTES, st);
     return e == cudaSuccess ? RGLRU_OK : RGLRU_ERR_CUDA;
 }
 

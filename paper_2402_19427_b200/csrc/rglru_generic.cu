@@ -1,24 +1,50 @@
 // Shape-generic CUDA-core kernels for the RG-LRU temporal core: any head width up to
-// GENERIC_MAX_DH, fp32 or bf16 io, accurate libm-grade transcendental functions.
-// They serve the fp32 configuration, head widths without a tensor-core kernel, and the
-// backward.  One block walks one (sequence, head) pair through time; the gate products
-// W_a u, W_x u (Eq. 1-2) run on FP32 FMAs with the weights staged through shared memory.
+// GENERIC_MAX_DH, fp32 or bf16 io, accurate libm-grade transcendental functions, fp32 throughout.
+// They serve the fp32 configurations, bf16 heads without a tensor-core kernel, and the backward of both.
+//
+// Every contraction (gate products W_a u, W_x u of Eq. 1-2; du = W^T dz; dW = dz^T u) is a register-blocked fp32 product on
+// packed FMAs: 128 threads own BM x 2 BM results, 2 TM NH = BM * BM / 64 each (64 for BM = 64), operands staged K-major
+// through double-buffered shared memory with the next slab's global loads in flight.  At BM = 64 a thread does 64 FMAs per
+// four 16-byte shared loads, so the FMA pipe and not shared memory bounds it.  BM = 32 is the same code with a quarter of the
+// work per block, for problems whose 64-tiles would not fill the SMs twice (see tile_rows).
+// Time is cut into chunks of BM tokens.  The forward and the reverse scan run from zero state inside a chunk, in registers,
+// and the chunks of a channel are chained through one 16-byte record per (sequence, channel): block order is chunk-major, so
+// a block only ever waits for blocks that were dispatched before it.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
 #include "rglru_internal.h"
+#include "sm100_ptx.cuh"
 
 namespace rglru {
 namespace {
 
-constexpr int NT = 256;  // threads per block
-constexpr int GT = 16;   // tokens (or sequences, for decode) per tile
-constexpr int NB = 16;   // input channels per staged weight slab
+using ptx::f32x2;
+using ptx::fma2;
+using ptx::pack2;
 
+constexpr int NT = 256;  // threads per block of the element-wise and decode kernels
+constexpr int GT = 16;   // sequences per tile of the decode kernel
+constexpr int NB = 16;   // input channels per staged weight slab of the decode kernel
+constexpr int MT = 128;  // threads per block of the contractions
+constexpr int BK = 16;   // K slab of the contractions
+
+__device__ __forceinline__ float tof(float v) { return v; }
+__device__ __forceinline__ float tof(__nv_bfloat16 v) { return __bfloat162float(v); }
 __device__ __forceinline__ float ldf(const float *p, size_t i) { return p[i]; }
 __device__ __forceinline__ float ldf(const __nv_bfloat16 *p, size_t i) { return __bfloat162float(p[i]); }
 __device__ __forceinline__ void stf(float *p, size_t i, float v) { p[i] = v; }
 __device__ __forceinline__ void stf(__nv_bfloat16 *p, size_t i, float v) { p[i] = __float2bfloat16_rn(v); }
+// four consecutive elements (address a multiple of four elements)
+__device__ __forceinline__ void ld4(const float *p, float *v) {
+    const float4 t = *(const float4 *)p;
+    v[0] = t.x; v[1] = t.y; v[2] = t.z; v[3] = t.w;
+}
+__device__ __forceinline__ void ld4(const __nv_bfloat16 *p, float *v) {
+    const uint2 t = *(const uint2 *)p;
+    v[0] = __uint_as_float(t.x << 16); v[1] = __uint_as_float(t.x & 0xFFFF0000u);
+    v[2] = __uint_as_float(t.y << 16); v[3] = __uint_as_float(t.y & 0xFFFF0000u);
+}
 
 __device__ __forceinline__ float sigmoid_acc(float z) { return 1.0f / (1.0f + expf(-z)); }
 // GeLU(v) = v Phi(v), the non-linearity on the second branch of the recurrent block (Section 2.3)
@@ -35,6 +61,322 @@ __device__ __forceinline__ void decay(float s, float r, float &a, float &m) {
     float L = -s * r;
     a = expf(L);
     m = sqrtf(fmaxf(0.0f, -expm1f(2.0f * L)));
+}
+
+// x_{tau} of sequence b for tau in [-3, T): history comes from conv_state_in (oldest first) or is zero
+template <typename IOT>
+__device__ __forceinline__ float x_at(const IOT *x, const IOT *cs_in, int T, int D, int b, int tau, int d) {
+    if (tau >= 0) return ldf(x, ((size_t)b * T + tau) * D + d);
+    if (cs_in == nullptr) return 0.0f;
+    return ldf(cs_in, ((size_t)b * 3 + (3 + tau)) * D + d);
+}
+template <typename IOT>
+__device__ __forceinline__ IOT x_raw_at(const IOT *x, const IOT *cs_in, int T, int D, int b, int tau, int d) {
+    if (tau >= 0) return x[((size_t)b * T + tau) * D + d];
+    if (cs_in == nullptr) return IOT(0.0f);
+    return cs_in[((size_t)b * 3 + (3 + tau)) * D + d];
+}
+
+// ------------------------------------------------------------------ register-blocked fp32 product
+// Geometry of a block: 128 threads as 8 (rows) x 16 (columns); BM rows x 2 BM columns of results.  Thread (ty, tx) owns rows
+// TM ty .. TM ty + TM - 1 and columns NH tx .. + NH - 1 of each half of the columns (in the forward the halves are the two
+// gates of the same channels).
+template <int BM> struct Tile {
+    static constexpr int BN = 2 * BM, TM = BM / 8, NH = BM / 16;
+    static constexpr int AS = BM + 4, BS = BN + 4;   // row strides in shared memory (floats): 16-byte rows, shifted by one bank group
+    float As[2][BK][AS], Bs[2][BK][BS];
+};
+
+template <int BM>
+__device__ __forceinline__ void mul_slab(const Tile<BM> &s, int buf, int ty, int tx, f32x2 (&acc)[Tile<BM>::TM][Tile<BM>::NH]) {
+    constexpr int TM = Tile<BM>::TM, NH = Tile<BM>::NH;
+#pragma unroll
+    for (int k = 0; k < BK; ++k) {
+        float a[TM];
+        f32x2 b[NH];
+#pragma unroll
+        for (int i = 0; i < TM; i += 4) {
+            const float4 t = *(const float4 *)&s.As[buf][k][ty * TM + i];
+            a[i] = t.x; a[i + 1] = t.y; a[i + 2] = t.z; a[i + 3] = t.w;
+        }
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+#pragma unroll
+            for (int j = 0; j < NH; j += 2) b[half * (NH / 2) + j / 2] = *(const f32x2 *)&s.Bs[buf][k][half * BM + tx * NH + j];
+        }
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+#pragma unroll
+            for (int j = 0; j < NH; ++j) acc[i][j] = fma2(pack2(a[i], a[i]), b[j], acc[i][j]);
+        }
+    }
+}
+// column j (0 .. NH - 1) of half `half` of this thread's row i
+template <int NH> __device__ __forceinline__ float col(const f32x2 (&row)[NH], int half, int j) {
+    const f32x2 p = row[half * (NH / 2) + j / 2];
+    return (j & 1) ? p.y : p.x;
+}
+// A BK x W block of a row-major matrix (rows = K index, W contiguous columns) on its way to shared memory: 128 threads, W / 8
+// values each, by fours of one row when the addresses allow it.
+template <int W, bool VEC, typename T>
+__device__ __forceinline__ void fetch_rows(const T *src, size_t stride, int rows_valid, int cols_valid, int tid, float (&v)[W / 8]) {
+    if (VEC) {
+#pragma unroll
+        for (int i = 0; i < W / 32; ++i) {
+            const int e = tid + MT * i, k = e / (W / 4), n = (e % (W / 4)) * 4;
+            if (k < rows_valid && n < cols_valid) ld4(src + (size_t)k * stride + n, v + 4 * i);
+            else { v[4 * i] = 0.f; v[4 * i + 1] = 0.f; v[4 * i + 2] = 0.f; v[4 * i + 3] = 0.f; }
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < W / 8; ++i) {
+            const int e = tid + MT * i, k = e / W, n = e % W;
+            v[i] = k < rows_valid && n < cols_valid ? tof(src[(size_t)k * stride + n]) : 0.0f;
+        }
+    }
+}
+template <int W, bool VEC, int S>
+__device__ __forceinline__ void put_rows(float (&dst)[BK][S], int tid, const float (&v)[W / 8]) {
+    if (VEC) {
+#pragma unroll
+        for (int i = 0; i < W / 32; ++i) {
+            const int e = tid + MT * i, k = e / (W / 4), n = (e % (W / 4)) * 4;
+            *(float4 *)&dst[k][n] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < W / 8; ++i) { const int e = tid + MT * i; dst[e / W][e % W] = v[i]; }
+    }
+}
+// E consecutive K values of one row of a matrix whose rows run along K (it is transposed on its way to shared memory)
+template <int E, bool VEC, typename T> __device__ __forceinline__ void fetch_k(const T *row, bool row_valid, int k_valid, float (&v)[E]) {
+    if (VEC) {
+#pragma unroll
+        for (int i = 0; i < E; i += 4) {
+            if (row_valid && i < k_valid) ld4(row + i, v + i);
+            else { v[i] = 0.f; v[i + 1] = 0.f; v[i + 2] = 0.f; v[i + 3] = 0.f; }
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < E; ++i) v[i] = row_valid && i < k_valid ? tof(row[i]) : 0.0f;
+    }
+}
+
+// ------------------------------------------------------------------ chain of chunks
+// One record {A, tag, B, tag2} per (sequence, channel): what the chunks so far hand to the next one.  Chunk c waits for the
+// tags of its predecessor and overwrites the record with its own; nobody else reads it, so one slot serves the whole chain
+// (and what a finished call leaves behind carries the tag of the last chunk, which no chunk ever waits for).
+struct Chain {
+    uint4 *slot;        // [B][D]
+    uint32_t tag, tag2;
+    unsigned long long spin_ns;
+    uint32_t *status;
+};
+// All lanes of the warp call it (a lane without a channel passes need = false); false if the wait ran out.
+__device__ __forceinline__ bool chain_wait(const Chain &ch, const uint4 *slot, bool need, int link, float &A, float &B) {
+    uint64_t t0 = 0;
+    for (uint32_t n = 0;; ++n) {
+        uint4 r = make_uint4(0u, 0u, 0u, 0u);
+        if (need) asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(slot) : "memory");
+        const bool ready = !need || (r.y == ch.tag + (uint32_t)link && r.w == (ch.tag2 ^ (uint32_t)link));
+        if (__all_sync(0xffffffffu, ready)) {
+            A = __uint_as_float(r.x); B = __uint_as_float(r.z);
+            return true;
+        }
+        if ((n & 31u) == 31u) {
+            const uint64_t t = ptx::gtimer();
+            if (t0 == 0) t0 = t;
+            if (__any_sync(0xffffffffu, t - t0 > ch.spin_ns)) {
+                if ((threadIdx.x & 31) == 0) atomicExch(ch.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT);
+                return false;
+            }
+        }
+    }
+}
+__device__ __forceinline__ void chain_put(const Chain &ch, uint4 *slot, int link, float A, float B) {
+    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(slot), "r"(__float_as_uint(A)), "r"(ch.tag + (uint32_t)link), "r"(__float_as_uint(B)),
+                 "r"(ch.tag2 ^ (uint32_t)link) : "memory");
+}
+
+// ------------------------------------------------------------------ forward
+// Block = (chunk of BM tokens, sequence, head, BM output channels): Conv1D on the way into shared memory, both gate products,
+// gates and decay on the results in registers, scan of each thread's TM tokens from zero state, the 8 row groups combined
+// through shared memory, chain to the previous chunk, y.  u, r, i, a, v never leave the block.  With SAVE (the backward's
+// forward sweep) u, r, i and h_{t-1} go to fp32 arrays instead of y.
+// Against one block per (head, sequence) walking the whole of T: 4 x 1024 x 1024 (4 heads), fp32, ran at 1.8 TFLOP/s there.
+template <typename IOT, bool SAVE, int BM, bool VEC>
+__global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(FwdArgs a, Chain ch, int nchunk, int ntile) {
+    using TL = Tile<BM>;
+    constexpr int TM = TL::TM, NH = TL::NH, EB = TL::BN / 8;
+    __shared__ __align__(16) TL s;
+    __shared__ float agg_P[8][BM], agg_h[8][BM], in_h[8][BM];
+    __shared__ int ok_s;
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const int Dh = a.D / a.H, D = a.D, T = a.T;
+    int bid = blockIdx.x;
+    const int nt = bid % ntile; bid /= ntile;
+    const int head = bid % a.H; bid /= a.H;
+    const int b = bid % a.B, chunk = bid / a.B;
+    const int d0 = head * Dh, n0 = nt * BM, t0 = chunk * BM;
+    const IOT *x = (const IOT *)a.x, *cw = (const IOT *)a.conv_w, *cs_in = (const IOT *)a.cs_in;
+    const IOT *xb = x + (size_t)b * T * D;
+    if (tid == 0) ok_s = 1;
+
+    // A operand: this thread convolves channel kk of each slab for tokens TM seg .. + TM - 1 of the chunk
+    const int kk = tid & 15, seg = tid >> 4, ta = t0 + seg * TM;
+    // B operand: row br of the 2 BM weight rows (both gates), EB consecutive input channels from koff
+    constexpr int ROWS_PER_PASS = MT < TL::BN ? MT : TL::BN;
+    static_assert(ROWS_PER_PASS * EB * (MT / ROWS_PER_PASS) == TL::BN * BK, "weight slab is covered exactly once");
+    const int br = tid % TL::BN, koff = (tid / TL::BN) * EB;
+    const int bch = n0 + (br % BM);
+    const IOT *wrow = (const IOT *)(br < BM ? a.W_a : a.W_x) + ((size_t)head * Dh + (bch < Dh ? bch : 0)) * Dh + koff;
+    float xr[TM + 3], taps[4], cb, wv[EB];
+    auto fetch = [&](int k0) {
+        const int k = k0 + kk, d = d0 + k;
+        const bool kv = k < Dh;
+#pragma unroll
+        for (int i = 0; i < TM + 3; ++i) {
+            const int t = ta - 3 + i;
+            float v = 0.0f;
+            if (kv) {
+                if (t >= 0) { if (t < T) v = ldf(xb, (size_t)t * D + d); }
+                else if (cs_in) v = ldf(cs_in, ((size_t)b * 3 + (3 + t)) * D + d);
+            }
+            xr[i] = v;
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) taps[j] = kv ? ldf(cw, (size_t)j * D + d) : 0.0f;
+        cb = kv && a.conv_b ? a.conv_b[d] : 0.0f;
+        fetch_k<EB, VEC>(wrow + k0, bch < Dh, Dh - k0 - koff, wv);
+    };
+    auto stage = [&](int buf) {
+        float u[TM];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) {
+            u[i] = fmaf(taps[0], xr[i + 3], cb);
+#pragma unroll
+            for (int j = 1; j < 4; ++j) u[i] = fmaf(taps[j], xr[i + 3 - j], u[i]);
+        }
+#pragma unroll
+        for (int i = 0; i < TM; i += 4) *(float4 *)&s.As[buf][kk][seg * TM + i] = make_float4(u[i], u[i + 1], u[i + 2], u[i + 3]);
+#pragma unroll
+        for (int i = 0; i < EB; ++i) s.Bs[buf][koff + i][br] = wv[i];
+    };
+    f32x2 acc[TM][NH];
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+#pragma unroll
+        for (int j = 0; j < NH; ++j) acc[i][j] = pack2(0.f, 0.f);
+    }
+    const int nk = (Dh + BK - 1) / BK;
+    fetch(0);
+    stage(0);
+    __syncthreads();
+    for (int kc = 0; kc < nk; ++kc) {
+        if (kc + 1 < nk) fetch((kc + 1) * BK);
+        mul_slab<BM>(s, kc & 1, ty, tx, acc);
+        if (kc + 1 < nk) stage((kc + 1) & 1);
+        __syncthreads();
+    }
+
+    // ---- gates, decay, scan of this thread's TM tokens x NH channels from zero state
+    const int tr = t0 + ty * TM, c0 = n0 + tx * NH, dc = d0 + c0;
+    float P[TM][NH], h[TM][NH];
+    {
+#pragma unroll
+        for (int j = 0; j < NH; ++j) {
+            const bool cv = c0 + j < Dh;
+            const int d = cv ? dc + j : d0;
+            float u[TM];
+            {
+                float w[4], xv[TM + 3];
+#pragma unroll
+                for (int i = 0; i < TM + 3; ++i) {
+                    const int t = tr - 3 + i;
+                    xv[i] = t >= 0 ? (t < T ? ldf(xb, (size_t)t * D + d) : 0.0f) : (cs_in ? ldf(cs_in, ((size_t)b * 3 + (3 + t)) * D + d) : 0.0f);
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) w[q] = ldf(cw, (size_t)q * D + d);
+                const float cbj = a.conv_b ? a.conv_b[d] : 0.0f;
+#pragma unroll
+                for (int i = 0; i < TM; ++i) {
+                    u[i] = fmaf(w[0], xv[i + 3], cbj);
+#pragma unroll
+                    for (int q = 1; q < 4; ++q) u[i] = fmaf(w[q], xv[i + 3 - q], u[i]);
+                }
+            }
+            const float sr = decay_rate(a.lambda[d], a.c), ba = a.b_a[d], bx = a.b_x[d];
+            float Pc = 1.0f, hc = 0.0f;
+#pragma unroll
+            for (int i = 0; i < TM; ++i) {
+                const float r = sigmoid_acc(col<NH>(acc[i], 0, j) + ba), g = sigmoid_acc(col<NH>(acc[i], 1, j) + bx);
+                float at, mt;
+                decay(sr, r, at, mt);
+                const bool tv = tr + i < T;
+                if (SAVE) {
+                    if (tv && cv) {
+                        const size_t e = ((size_t)b * T + tr + i) * D + d;
+                        a.save_u[e] = u[i]; a.save_r[e] = r; a.save_i[e] = g;
+                    }
+                    P[i][j] = Pc; h[i][j] = hc;   // state before the token
+                }
+                if (tv) { Pc *= at; hc = fmaf(at, hc, mt * (g * u[i])); }
+                if (!SAVE) { P[i][j] = Pc; h[i][j] = hc; }
+            }
+            agg_P[ty][tx * NH + j] = Pc;
+            agg_h[ty][tx * NH + j] = hc;
+        }
+    }
+    __syncthreads();
+    // ---- chain: one thread per channel takes the state the previous chunk reached and hands its own on
+    if (tid < BM) {
+        const bool cv = n0 + tid < Dh;
+        const int d = cv ? d0 + n0 + tid : d0;
+        uint4 *slot = ch.slot + (size_t)b * D + d;
+        float hs = 0.0f, Ps = 1.0f;
+        bool ok = true;
+        if (chunk == 0) hs = a.h0 ? a.h0[(size_t)b * D + d] : 0.0f;
+        else ok = chain_wait(ch, slot, cv, chunk - 1, hs, Ps);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+            in_h[q][tid] = hs;
+            hs = fmaf(agg_P[q][tid], hs, agg_h[q][tid]);
+            Ps *= agg_P[q][tid];
+        }
+        if (ok && cv) {
+            if (chunk + 1 < nchunk) chain_put(ch, slot, chunk, hs, Ps);
+            else if (!SAVE) {
+                a.h_T[(size_t)b * D + d] = hs;
+                if (a.a_prod) a.a_prod[(size_t)b * D + d] = Ps;
+                // the last three raw inputs of concat(conv_state_in, x), bit-exact
+                IOT *cs_out = (IOT *)a.cs_out;
+                IOT keep[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) keep[q] = x_raw_at(x, cs_in, T, D, b, T - 3 + q, d);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) cs_out[((size_t)b * 3 + q) * D + d] = keep[q];
+            }
+        }
+        if (!ok) ok_s = 0;
+    }
+    __syncthreads();
+    if (!ok_s) return;
+    const IOT *gb = (const IOT *)a.gate_branch;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int t = tr + i;
+        if (t >= T) break;
+        const size_t e = ((size_t)b * T + t) * D + dc;
+#pragma unroll
+        for (int j = 0; j < NH; ++j) {
+            if (c0 + j < Dh) {
+                const float hv = fmaf(P[i][j], in_h[ty][tx * NH + j], h[i][j]);
+                if (SAVE) a.save_hprev[e + j] = hv;
+                // merged output of the recurrent block (Section 2.3): GeLU on the second branch, then the product
+                else stf((IOT *)a.y, e + j, gb ? hv * gelu(ldf(gb, e + j)) : hv);
+            }
+        }
+    }
 }
 
 // acc_a[tt] += sum_n W_a[o][n] u_s[tt][n] (same for W_x) for this thread's output channel o.
@@ -74,98 +416,6 @@ __device__ __forceinline__ void gate_accumulate(const IOT *__restrict__ Wa, cons
                     acc_x[tt] = fmaf(wx, uv, acc_x[tt]);
                 }
             }
-        }
-    }
-}
-
-// x_{tau} of sequence b for tau in [-3, T): history comes from conv_state_in (oldest first) or is zero
-template <typename IOT>
-__device__ __forceinline__ float x_at(const IOT *x, const IOT *cs_in, int T, int D, int b, int tau, int d) {
-    if (tau >= 0) return ldf(x, ((size_t)b * T + tau) * D + d);
-    if (cs_in == nullptr) return 0.0f;
-    return ldf(cs_in, ((size_t)b * 3 + (3 + tau)) * D + d);
-}
-template <typename IOT>
-__device__ __forceinline__ IOT x_raw_at(const IOT *x, const IOT *cs_in, int T, int D, int b, int tau, int d) {
-    if (tau >= 0) return x[((size_t)b * T + tau) * D + d];
-    if (cs_in == nullptr) return IOT(0.0f);
-    return cs_in[((size_t)b * 3 + (3 + tau)) * D + d];
-}
-
-// Forward over T tokens for one (head, sequence) per block.  grid = (H, B).
-// Dynamic shared memory: u_s[GT][Dh] | h_s[Dh] | w_s[2*NB][NT+1].
-template <typename IOT, bool SAVE>
-__global__ void __launch_bounds__(NT) generic_prefill_kernel(FwdArgs a) {
-    extern __shared__ float smem[];
-    const int Dh = a.D / a.H, D = a.D, T = a.T;
-    const int k = blockIdx.x, b = blockIdx.y, d0 = k * Dh, tid = threadIdx.x;
-    float *u_s = smem, *h_s = u_s + GT * Dh, *w_s = h_s + Dh;
-    const IOT *x = (const IOT *)a.x, *cw = (const IOT *)a.conv_w, *cs_in = (const IOT *)a.cs_in;
-    const IOT *Wa = (const IOT *)a.W_a + (size_t)k * Dh * Dh, *Wx = (const IOT *)a.W_x + (size_t)k * Dh * Dh;
-    IOT *y = (IOT *)a.y;
-    const IOT *gb = (const IOT *)a.gate_branch;
-    const int nob = (Dh + NT - 1) / NT;
-
-    for (int n = tid; n < Dh; n += NT) h_s[n] = a.h0 ? a.h0[(size_t)b * D + d0 + n] : 0.0f;
-
-    for (int t0 = 0; t0 < T; t0 += GT) {
-        const int len = min(GT, T - t0);
-        __syncthreads();
-        // Conv1D, width 4, causal: u_t = b_c + sum_j w[j] x_{t-j}
-        for (int idx = tid; idx < GT * Dh; idx += NT) {
-            int tt = idx / Dh, n = idx % Dh, d = d0 + n;
-            float u = 0.0f;
-            if (tt < len) {
-                u = a.conv_b ? a.conv_b[d] : 0.0f;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) u = fmaf(ldf(cw, (size_t)j * D + d), x_at(x, cs_in, T, D, b, t0 + tt - j, d), u);
-                if (SAVE) a.save_u[((size_t)b * T + t0 + tt) * D + d] = u;
-            }
-            u_s[tt * Dh + n] = u;
-        }
-        __syncthreads();
-        for (int ob = 0; ob < nob; ++ob) {
-            float acc_a[GT], acc_x[GT];
-            gate_accumulate<IOT>(Wa, Wx, Dh, ob, u_s, w_s, acc_a, acc_x);
-            const int o = ob * NT + tid;
-            if (o < Dh) {
-                const int d = d0 + o;
-                const float s = decay_rate(a.lambda[d], a.c), ba = a.b_a[d], bx = a.b_x[d];
-                float h = h_s[o];
-                // prod_t a_t of the call, carried from one time group to the next in the output itself (same thread each time)
-                float ap = (a.a_prod && t0 > 0) ? a.a_prod[(size_t)b * D + d] : 1.0f;
-#pragma unroll
-                for (int tt = 0; tt < GT; ++tt) {
-                    if (tt < len) {
-                        float r = sigmoid_acc(acc_a[tt] + ba), g = sigmoid_acc(acc_x[tt] + bx), at, mt;
-                        decay(s, r, at, mt);
-                        size_t e = ((size_t)b * T + t0 + tt) * D + d;
-                        if (SAVE) { a.save_r[e] = r; a.save_i[e] = g; a.save_hprev[e] = h; }
-                        h = fmaf(at, h, mt * (g * u_s[tt * Dh + o]));
-                        ap *= at;
-                        // merged output of the recurrent block (Section 2.3): GeLU on the second branch, then the product
-                        if (!SAVE) stf(y, e, gb ? h * gelu(ldf(gb, e)) : h);
-                    }
-                }
-                h_s[o] = h;
-                if (!SAVE && a.a_prod) a.a_prod[(size_t)b * D + d] = ap;
-            }
-        }
-    }
-    __syncthreads();
-    if (!SAVE) {
-        for (int n = tid; n < Dh; n += NT) a.h_T[(size_t)b * D + d0 + n] = h_s[n];
-        // conv_state_out = last three raw inputs of concat(conv_state_in, x); staged so that it may alias conv_state_in
-        IOT *stage = (IOT *)u_s;
-        for (int idx = tid; idx < 3 * Dh; idx += NT) {
-            int kk = idx / Dh, n = idx % Dh;
-            stage[idx] = x_raw_at(x, cs_in, T, D, b, T - 3 + kk, d0 + n);
-        }
-        __syncthreads();
-        IOT *cs_out = (IOT *)a.cs_out;
-        for (int idx = tid; idx < 3 * Dh; idx += NT) {
-            int kk = idx / Dh, n = idx % Dh;
-            cs_out[((size_t)b * 3 + kk) * D + d0 + n] = stage[idx];
         }
     }
 }
@@ -225,129 +475,211 @@ __global__ void __launch_bounds__(NT) generic_decode_kernel(FwdArgs a) {
 }
 
 // ------------------------------------------------------------------ backward
-// Reverse-time scan and element-wise adjoints.  One thread per (b, d); grid = (ceil(D/NT), B).
+// Reverse-time scan and element-wise adjoints.  Block = (chunk of 64 tokens, 32 channels, sequence): thread (lane, seg) holds
+// the eight tokens of its segment in registers, runs the recurrence from zero, the segments are combined through shared
+// memory, the chunks are chained last chunk first.
 //   g_t = dy_t + a_{t+1} g_{t+1};  dL = g (a h_{t-1} - a^2 v / m);  dv = g m;  di = dv u;  du = dv i;
 //   dr = -s dL;  dz_a = dr r (1-r);  dz_x = di i (1-i).
 // In place: r -> dz_a, i -> dz_x, hprev -> du (direct part).
+constexpr int RCHUNK = 64;
 template <typename IOT>
-__global__ void __launch_bounds__(NT) generic_bwd_scan_kernel(BwdArgs q) {
-    const int d = blockIdx.x * NT + threadIdx.x, b = blockIdx.y;
-    if (d >= q.D) return;
-    const int T = q.T, D = q.D;
+__global__ void __launch_bounds__(NT) generic_bwd_scan_kernel(BwdArgs q, Chain ch, int nchunk, int ctiles) {
+    __shared__ float agg_Q[8][32], agg_g[8][32], in_g[8][32], sums[3][8][32];
+    __shared__ int ok_s;
+    const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+    int bid = blockIdx.x;
+    const int ct = bid % ctiles; bid /= ctiles;
+    const int b = bid % q.B, link = bid / q.B, chunk = nchunk - 1 - link;   // last chunk first
+    const int T = q.T, D = q.D, d = ct * 32 + lane;
+    const bool cv = d < D;
+    const int dc = cv ? d : 0, t0 = chunk * RCHUNK + seg * 8;
     const IOT *dy = (const IOT *)q.dy;
-    const float lam = q.lambda[d];
-    const float s = decay_rate(lam, q.c);
+    const float lam = q.lambda[dc], s = decay_rate(lam, q.c);
     const float dsdlam_neg = q.c * sigmoid_acc(-lam);  // dL/dLambda = c r sigmoid(-Lambda)
-    // past the last token g holds the gradient arriving on h_T (h_T = h_{T-1}, so it is carried with factor 1)
-    float g = q.dh_T ? q.dh_T[(size_t)b * D + d] : 0.0f, a_next = 1.0f, s_lam = 0.0f, s_ba = 0.0f, s_bx = 0.0f;
-    for (int t = T - 1; t >= 0; --t) {
-        size_t e = ((size_t)b * T + t) * D + d;
-        float r = q.r[e], gi = q.gi[e], u = q.u[e], hp = q.hp[e], at, mt;
-        decay(s, r, at, mt);
-        g = fmaf(a_next, g, ldf(dy, e));
-        float v = gi * u;
-        float dm_term = mt > 0.0f ? at * at * v / mt : 0.0f;
-        float dL = g * (at * hp - dm_term);
-        float dv = g * mt;
-        float di = dv * u;
-        float dr = -s * dL;
-        float dza = dr * r * (1.0f - r), dzx = di * gi * (1.0f - gi);
-        s_lam = fmaf(dL * r, dsdlam_neg, s_lam);
-        s_ba += dza;
-        s_bx += dzx;
-        q.r[e] = dza;
-        q.gi[e] = dzx;
-        q.hp[e] = dv * gi;
-        a_next = at;
+    if (threadIdx.x == 0) ok_s = 1;
+    float r[8], at[8], mt[8], dyv[8];
+    const size_t e0 = ((size_t)b * T + t0) * D + dc;
+    const int nv = min(8, T - t0);   // tokens of the segment that exist (may be <= 0); a token that does not passes g through
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { r[i] = i < nv ? q.r[e0 + (size_t)i * D] : 0.0f; dyv[i] = i < nv ? ldf(dy, e0 + (size_t)i * D) : 0.0f; }
+    float Q = 1.0f, G = 0.0f;
+#pragma unroll
+    for (int i = 7; i >= 0; --i) {
+        if (i < nv) decay(s, r[i], at[i], mt[i]); else { at[i] = 1.0f; mt[i] = 0.0f; }
+        G = at[i] * (dyv[i] + G);
+        Q *= at[i];
     }
-    if (q.dh0) q.dh0[(size_t)b * D + d] = a_next * g;   // a_0 g_0: h0 enters Eq. 4 only at t = 0
-    q.part_vec[((size_t)b * 3 + 0) * D + d] = s_lam;
-    q.part_vec[((size_t)b * 3 + 1) * D + d] = s_ba;
-    q.part_vec[((size_t)b * 3 + 2) * D + d] = s_bx;
-}
-
-// du[tok][n] += sum_o W_a[o][n] dz_a[tok][o] + W_x[o][n] dz_x[tok][o].  grid = (H, ceil(B*T/GT)).
-// Dynamic shared memory: dz_s[2][GT][Dh].
-template <typename IOT>
-__global__ void __launch_bounds__(NT) generic_bwd_du_kernel(BwdArgs q) {
-    extern __shared__ float smem[];
-    const int Dh = q.D / q.H, D = q.D, k = blockIdx.x, d0 = k * Dh, tid = threadIdx.x;
-    const size_t ntok = (size_t)q.B * q.T, tok0 = (size_t)blockIdx.y * GT;
-    const int len = (int)min((size_t)GT, ntok - tok0);
-    float *dza_s = smem, *dzx_s = smem + GT * Dh;
-    const IOT *Wa = (const IOT *)q.W_a + (size_t)k * Dh * Dh, *Wx = (const IOT *)q.W_x + (size_t)k * Dh * Dh;
-    for (int idx = tid; idx < GT * Dh; idx += NT) {
-        int tt = idx / Dh, o = idx % Dh;
-        float va = 0.0f, vx = 0.0f;
-        if (tt < len) { va = q.r[(tok0 + tt) * D + d0 + o]; vx = q.gi[(tok0 + tt) * D + d0 + o]; }
-        dza_s[idx] = va; dzx_s[idx] = vx;
+    agg_Q[seg][lane] = Q; agg_g[seg][lane] = G;
+    __syncthreads();
+    if (seg == 0) {
+        uint4 *slot = ch.slot + (size_t)b * D + dc;
+        // past the last token g holds the gradient arriving on h_T (h_T = h_{T-1}, so it is carried with factor 1)
+        float X = 0.0f, unused;
+        bool ok = true;
+        if (link == 0) X = q.dh_T ? q.dh_T[(size_t)b * D + dc] : 0.0f;
+        else ok = chain_wait(ch, slot, cv, link - 1, X, unused);
+#pragma unroll
+        for (int k = 7; k >= 0; --k) { in_g[k][lane] = X; X = fmaf(agg_Q[k][lane], X, agg_g[k][lane]); }
+        if (ok && cv) {
+            if (chunk > 0) chain_put(ch, slot, link, X, 0.0f);
+            else if (q.dh0) q.dh0[(size_t)b * D + d] = X;   // a_0 g_0: h0 enters Eq. 4 only at t = 0
+        }
+        if (!ok) ok_s = 0;
     }
     __syncthreads();
-    for (int n = tid; n < Dh; n += NT) {
-        float acc[GT];
+    if (!ok_s) return;
+    float carry = in_g[seg][lane], s_lam = 0.0f, s_ba = 0.0f, s_bx = 0.0f;
 #pragma unroll
-        for (int tt = 0; tt < GT; ++tt) acc[tt] = 0.0f;
-        for (int o = 0; o < Dh; ++o) {
-            float wa = ldf(Wa, (size_t)o * Dh + n), wx = ldf(Wx, (size_t)o * Dh + n);
-#pragma unroll
-            for (int tt = 0; tt < GT; ++tt) acc[tt] = fmaf(wa, dza_s[tt * Dh + o], fmaf(wx, dzx_s[tt * Dh + o], acc[tt]));
+    for (int i = 7; i >= 0; --i) {
+        if (i < nv && cv) {
+            const size_t e = e0 + (size_t)i * D;
+            const float gi = q.gi[e], u = q.u[e], hp = q.hp[e], a = at[i], m = mt[i];
+            const float g = dyv[i] + carry;
+            const float v = gi * u;
+            const float dm_term = m > 0.0f ? a * a * v / m : 0.0f;
+            const float dL = g * (a * hp - dm_term);
+            const float dv = g * m;
+            const float di = dv * u;
+            const float dr = -s * dL;
+            const float dza = dr * r[i] * (1.0f - r[i]), dzx = di * gi * (1.0f - gi);
+            s_lam = fmaf(dL * r[i], dsdlam_neg, s_lam);
+            s_ba += dza;
+            s_bx += dzx;
+            q.r[e] = dza;
+            q.gi[e] = dzx;
+            q.hp[e] = dv * gi;
+            carry = a * g;
         }
+    }
+    sums[0][seg][lane] = s_lam; sums[1][seg][lane] = s_ba; sums[2][seg][lane] = s_bx;
+    __syncthreads();
+    if (seg < 3 && cv) {
+        float t = 0.0f;
 #pragma unroll
-        for (int tt = 0; tt < GT; ++tt)
-            if (tt < len) q.hp[(tok0 + tt) * D + d0 + n] += acc[tt];
+        for (int k = 0; k < 8; ++k) t += sums[seg][k][lane];
+        q.part_vec[((size_t)(b * nchunk + chunk) * 3 + seg) * D + d] = t;
     }
 }
 
-// Partial dW_a, dW_x: part[s][g][k][o][n] = sum over the tokens of split s of dz_g[tok][o] u[tok][n].
-// grid = (H * ceil(Dh/GT), ceil(Dh/NT), S): a block owns GT output rows and NT input columns.
-__global__ void __launch_bounds__(NT) generic_bwd_dw_kernel(BwdArgs q) {
-    __shared__ float dz_s[2][GT][GT];
-    const int Dh = q.D / q.H, D = q.D, tid = threadIdx.x;
-    const int nobk = (Dh + GT - 1) / GT;
-    const int k = blockIdx.x / nobk, o0 = (blockIdx.x % nobk) * GT, n = blockIdx.y * NT + tid, s = blockIdx.z;
-    const int d0 = k * Dh;
-    const size_t ntok = (size_t)q.B * q.T;
-    const size_t per = (ntok + q.S - 1) / q.S;
-    const size_t lo = (size_t)s * per, hi = min(ntok, lo + per);
-    float acc_a[GT], acc_x[GT];
+// du[tok][n] += sum_o W_a[o][n] dz_a[tok][o] + W_x[o][n] dz_x[tok][o].  Block = (BM tokens, head, 2 BM input channels); K runs
+// over the output channels of both gates.
+template <typename IOT, int BM, bool VEC>
+__global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_du_kernel(BwdArgs q, int ntile) {
+    using TL = Tile<BM>;
+    constexpr int TM = TL::TM, NH = TL::NH, EA = BM / 8;
+    __shared__ __align__(16) TL s;
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const int Dh = q.D / q.H, D = q.D;
+    int bid = blockIdx.x;
+    const int n0 = (bid % ntile) * TL::BN; bid /= ntile;
+    const int head = bid % q.H, d0 = head * Dh;
+    const size_t ntok = (size_t)q.B * q.T, tok0 = (size_t)(bid / q.H) * BM;
+    const int am = tid % BM, koff = (tid / BM) * EA;
+    const bool arow = tok0 + am < ntok;
+    const size_t aoff = (tok0 + (arow ? am : 0)) * D + d0 + koff;
+    const int nkg = (Dh + BK - 1) / BK;   // slabs per gate
+    float av[EA], bv[TL::BN / 8];
+    auto fetch = [&](int kc) {
+        const int gate = kc >= nkg, k0 = (kc - gate * nkg) * BK;
+        fetch_k<EA, VEC>((gate ? q.gi : q.r) + aoff + k0, arow, Dh - k0 - koff, av);
+        const IOT *W = (const IOT *)(gate ? q.W_x : q.W_a) + ((size_t)head * Dh + k0) * Dh + n0;
+        fetch_rows<TL::BN, VEC>(W, (size_t)Dh, Dh - k0, Dh - n0, tid, bv);
+    };
+    auto stage = [&](int buf) {
 #pragma unroll
-    for (int oo = 0; oo < GT; ++oo) { acc_a[oo] = 0.0f; acc_x[oo] = 0.0f; }
-    for (size_t tok0 = lo; tok0 < hi; tok0 += GT) {
-        __syncthreads();
-        for (int idx = tid; idx < 2 * GT * GT; idx += NT) {
-            int g = idx / (GT * GT), tt = (idx / GT) % GT, oo = idx % GT;
-            float v = 0.0f;
-            if (tok0 + tt < hi && o0 + oo < Dh) v = (g ? q.gi : q.r)[(tok0 + tt) * D + d0 + o0 + oo];
-            dz_s[g][tt][oo] = v;
-        }
-        __syncthreads();
-        if (n < Dh) {
-            const int len = (int)min((size_t)GT, hi - tok0);
-            for (int tt = 0; tt < len; ++tt) {
-                float uv = q.u[(tok0 + tt) * D + d0 + n];
+        for (int i = 0; i < EA; ++i) s.As[buf][koff + i][am] = av[i];
+        put_rows<TL::BN, VEC>(s.Bs[buf], tid, bv);
+    };
+    f32x2 acc[TM][NH];
 #pragma unroll
-                for (int oo = 0; oo < GT; ++oo) {
-                    acc_a[oo] = fmaf(dz_s[0][tt][oo], uv, acc_a[oo]);
-                    acc_x[oo] = fmaf(dz_s[1][tt][oo], uv, acc_x[oo]);
-                }
-            }
+    for (int i = 0; i < TM; ++i) {
+#pragma unroll
+        for (int j = 0; j < NH; ++j) acc[i][j] = pack2(0.f, 0.f);
+    }
+    fetch(0);
+    stage(0);
+    __syncthreads();
+    for (int kc = 0; kc < 2 * nkg; ++kc) {
+        if (kc + 1 < 2 * nkg) fetch(kc + 1);
+        mul_slab<BM>(s, kc & 1, ty, tx, acc);
+        if (kc + 1 < 2 * nkg) stage((kc + 1) & 1);
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const size_t tok = tok0 + ty * TM + i;
+        if (tok >= ntok) break;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int n = n0 + half * BM + tx * NH;
+            float *dst = q.hp + tok * D + d0 + n;
+#pragma unroll
+            for (int j = 0; j < NH; ++j)
+                if (n + j < Dh) dst[j] += col<NH>(acc[i], half, j);
         }
     }
-    if (n < Dh) {
-        const size_t wsz = (size_t)q.H * Dh * Dh;
+}
+
+// Partial dW_a, dW_x: part[s][gate][head][o][n] = sum over the tokens of split s of dz_gate[tok][o] u[tok][n].
+// Block = (split, gate, head, BM output rows, 2 BM input columns).
+template <int BM, bool VEC>
+__global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_dw_kernel(BwdArgs q, int mtile, int ntile) {
+    using TL = Tile<BM>;
+    constexpr int TM = TL::TM, NH = TL::NH;
+    __shared__ __align__(16) TL s;
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
+    const int Dh = q.D / q.H, D = q.D;
+    int bid = blockIdx.x;
+    const int n0 = (bid % ntile) * TL::BN; bid /= ntile;
+    const int m0 = (bid % mtile) * BM; bid /= mtile;
+    const int head = bid % q.H; bid /= q.H;
+    const int gate = bid & 1, split = bid >> 1, d0 = head * Dh;
+    const size_t ntok = (size_t)q.B * q.T, per = (ntok + q.S - 1) / q.S;
+    const size_t lo = (size_t)split * per, hi = lo + per < ntok ? lo + per : ntok;
+    const float *dz = (gate ? q.gi : q.r) + d0 + m0, *u = q.u + d0 + n0;
+    float av[BM / 8], bv[TL::BN / 8];
+    auto fetch = [&](size_t k0) {
+        const int rows = (int)(hi - k0 < (size_t)BK ? hi - k0 : (size_t)BK);
+        fetch_rows<BM, VEC>(dz + k0 * D, (size_t)D, rows, Dh - m0, tid, av);
+        fetch_rows<TL::BN, VEC>(u + k0 * D, (size_t)D, rows, Dh - n0, tid, bv);
+    };
+    auto stage = [&](int buf) {
+        put_rows<BM, VEC>(s.As[buf], tid, av);
+        put_rows<TL::BN, VEC>(s.Bs[buf], tid, bv);
+    };
+    f32x2 acc[TM][NH];
 #pragma unroll
-        for (int oo = 0; oo < GT; ++oo) {
-            if (o0 + oo < Dh) {
-                size_t w = ((size_t)k * Dh + o0 + oo) * Dh + n;
-                q.part_dw[((size_t)s * 2 + 0) * wsz + w] = acc_a[oo];
-                q.part_dw[((size_t)s * 2 + 1) * wsz + w] = acc_x[oo];
-            }
+    for (int i = 0; i < TM; ++i) {
+#pragma unroll
+        for (int j = 0; j < NH; ++j) acc[i][j] = pack2(0.f, 0.f);
+    }
+    const int nk = lo < hi ? (int)((hi - lo + BK - 1) / BK) : 0;
+    if (nk > 0) { fetch(lo); stage(0); }
+    __syncthreads();
+    for (int kc = 0; kc < nk; ++kc) {
+        if (kc + 1 < nk) fetch(lo + (size_t)(kc + 1) * BK);
+        mul_slab<BM>(s, kc & 1, ty, tx, acc);
+        if (kc + 1 < nk) stage((kc + 1) & 1);
+        __syncthreads();
+    }
+    const size_t wsz = (size_t)q.H * Dh * Dh;
+#pragma unroll
+    for (int i = 0; i < TM; ++i) {
+        const int o = m0 + ty * TM + i;
+        if (o >= Dh) break;
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const int n = n0 + half * BM + tx * NH;
+            float *dst = q.part_dw + ((size_t)split * 2 + gate) * wsz + ((size_t)head * Dh + o) * Dh + n;
+#pragma unroll
+            for (int j = 0; j < NH; ++j)
+                if (n + j < Dh) dst[j] = col<NH>(acc[i], half, j);
         }
     }
 }
 
 // Conv1D adjoint: dx_t = sum_j w[j] du_{t+j} (t+j < T); partial dw[j] = sum_t du_t x_{t-j}; partial db_c = sum_t du_t.
-// One thread per (b, chunk, d); grid = (ceil(D/NT), nchunk, B).
+// One thread per (b, chunk of GENERIC_BWD_CHUNK tokens, d) walks forward with sliding windows; grid = (ceil(D/NT), nchunk, B).
 template <typename IOT>
 __global__ void __launch_bounds__(NT) generic_bwd_conv_kernel(BwdArgs q) {
     const int d = blockIdx.x * NT + threadIdx.x, ch = blockIdx.y, b = blockIdx.z;
@@ -359,16 +691,25 @@ __global__ void __launch_bounds__(NT) generic_bwd_conv_kernel(BwdArgs q) {
 #pragma unroll
     for (int j = 0; j < 4; ++j) w[j] = ldf(cw, (size_t)j * D + d);
     const int t_lo = ch * GENERIC_BWD_CHUNK, t_hi = min(T, t_lo + GENERIC_BWD_CHUNK);
-    for (int t = t_lo; t < t_hi; ++t) {
-        float acc = 0.0f;
+    const float *du = q.hp + (size_t)b * T * D + d;
+    auto duat = [&](int t) -> float { return t < T ? du[(size_t)t * D] : 0.0f; };
+    float x1 = x_at(x, cs_in, T, D, b, t_lo - 1, d), x2 = x_at(x, cs_in, T, D, b, t_lo - 2, d), x3 = x_at(x, cs_in, T, D, b, t_lo - 3, d);
+    float g0 = duat(t_lo), g1 = duat(t_lo + 1), g2 = duat(t_lo + 2);
+    for (int tb = t_lo; tb < t_hi; tb += 8) {
+        float xs[8], gs[8];
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            if (t + j < T) acc = fmaf(w[j], q.hp[((size_t)b * T + t + j) * D + d], acc);
-        stf(dx, ((size_t)b * T + t) * D + d, acc);
-        float dut = q.hp[((size_t)b * T + t) * D + d];
+        for (int k = 0; k < 8; ++k) { xs[k] = tb + k < t_hi ? x_at(x, cs_in, T, D, b, tb + k, d) : 0.0f; gs[k] = duat(tb + k + 3); }
 #pragma unroll
-        for (int j = 0; j < 4; ++j) sw[j] = fmaf(dut, x_at(x, cs_in, T, D, b, t - j, d), sw[j]);
-        sb += dut;
+        for (int k = 0; k < 8; ++k) {
+            if (tb + k < t_hi) {
+                const float g3 = gs[k], x0 = xs[k];
+                stf(dx, ((size_t)b * T + tb + k) * D + d, fmaf(w[3], g3, fmaf(w[2], g2, fmaf(w[1], g1, w[0] * g0))));
+                sw[0] = fmaf(g0, x0, sw[0]); sw[1] = fmaf(g0, x1, sw[1]); sw[2] = fmaf(g0, x2, sw[2]); sw[3] = fmaf(g0, x3, sw[3]);
+                sb += g0;
+                g0 = g1; g1 = g2; g2 = g3;
+                x3 = x2; x2 = x1; x1 = x0;
+            }
+        }
     }
     float *p = q.part_conv + ((size_t)(b * q.nchunk + ch) * 5) * D + d;
 #pragma unroll
@@ -412,41 +753,45 @@ __global__ void __launch_bounds__(NT) state_conv_grads_kernel(BwdArgs q, const D
     }
 }
 
-// out[i] = sum_p in[p * stride + i], p ascending (fixed order => run-to-run identical results)
-__global__ void reduce_partials_kernel(const float *in, int nparts, size_t stride, float *out, size_t n) {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || out == nullptr) return;
+// out[i] = sum over the parts of in[p * stride + i] in a fixed order (run-to-run identical results), the row of each job being
+// split over up to three output arrays; all jobs of a call in one launch.  A block owns 32 columns with eight slices of the
+// parts (slice k sums parts k, k + 8, ... ascending, then the slices are added in order) or, for few parts, 256 columns.
+__global__ void __launch_bounds__(256) reduce_jobs_kernel(ReduceJobs jobs) {
+    __shared__ float part[8][32];
+    int blk = blockIdx.x, j = 0;
+    while (j + 1 < jobs.n && blk >= jobs.job[j].blocks) { blk -= jobs.job[j].blocks; ++j; }
+    const ReduceJob &q = jobs.job[j];
+    const size_t n = q.n0 + q.n1 + q.n2;
+    const bool sliced = q.sliced != 0;
+    const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+    const size_t i = sliced ? (size_t)blk * 32 + lane : (size_t)blk * 256 + threadIdx.x;
+    const int p0 = sliced ? slice : 0, dp = sliced ? 8 : 1;
     float acc = 0.0f;
-    for (int p = 0; p < nparts; ++p) acc += in[(size_t)p * stride + i];
-    out[i] = acc;
+    if (i < n) {
+        int p = p0;
+        for (; p + 7 * dp < q.nparts; p += 8 * dp) {   // eight loads in flight
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = q.in[(size_t)(p + k * dp) * q.stride + i];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc += v[k];
+        }
+        for (; p < q.nparts; p += dp) acc += q.in[(size_t)p * q.stride + i];
+    }
+    if (sliced) {
+        part[slice][lane] = acc;
+        __syncthreads();
+        if (slice != 0) return;
+        acc = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) acc += part[k][lane];
+    }
+    if (i >= n) return;
+    float *out = i < q.n0 ? (q.out0 ? q.out0 + i : nullptr) : i < q.n0 + q.n1 ? (q.out1 ? q.out1 + (i - q.n0) : nullptr) : (q.out2 ? q.out2 + (i - q.n0 - q.n1) : nullptr);
+    if (out) *out = acc;
 }
 
-// out[i] = sum over p of in[p * stride + i] in a fixed order (four interleaved running sums, added at the end), the row being
-// split over three output arrays
-__global__ void reduce_partials3_kernel(const float *in, int nparts, size_t stride, float *out0, size_t n0, float *out1, size_t n1,
-                                        float *out2, size_t n2) {
-    const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n0 + n1 + n2) return;
-    float *out = i < n0 ? (out0 ? out0 + i : nullptr) : i < n0 + n1 ? (out1 ? out1 + (i - n0) : nullptr) : (out2 ? out2 + (i - n0 - n1) : nullptr);
-    if (out == nullptr) return;
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-    int p = 0;
-    for (; p + 16 <= nparts; p += 16) {   // sixteen loads in flight, still four running sums in a fixed order
-        float v[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = in[(size_t)(p + j) * stride + i];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) acc[j & 3] += v[j];
-    }
-    for (; p + 4 <= nparts; p += 4) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[j] += in[(size_t)(p + j) * stride + i];
-    }
-    for (; p < nparts; ++p) acc[0] += in[(size_t)p * stride + i];
-    *out = (acc[0] + acc[1]) + (acc[2] + acc[3]);
-}
-
-size_t fwd_smem_bytes(int Dh) { return sizeof(float) * ((size_t)GT * Dh + Dh + 2 * NB * (NT + 1)); }
+size_t decode_smem_bytes(int Dh) { return sizeof(float) * ((size_t)GT * Dh + Dh + 2 * NB * (NT + 1)); }
 
 template <typename K>
 cudaError_t set_smem(K kernel, size_t bytes) {
@@ -455,34 +800,87 @@ cudaError_t set_smem(K kernel, size_t bytes) {
 }
 
 size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
+inline int ceil_div(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 
-int dw_splits(size_t ntok) {
-    size_t s = (ntok + 1023) / 1024;
+// Rows per block of a contraction with `blocks64` blocks of 64 rows x 128 columns: three of those fit an SM, and below two per
+// SM the machine is better filled by four times as many blocks of 32 x 64 (config 0, B1 T256 D256 H2: 8 -> 64 blocks).
+constexpr int FILL_BLOCKS = 296;
+inline int tile_rows(size_t blocks64) { return blocks64 >= (size_t)FILL_BLOCKS ? 64 : 32; }
+
+// Token splits of the dW products: enough blocks for two waves of three per SM, at least 128 tokens each, at most 32
+int dw_splits(size_t ntok, int H, int Dh) {
+    const size_t tiles = (size_t)2 * H * ceil_div(Dh, 64) * ceil_div(Dh, 128);
+    size_t s = (888 + tiles - 1) / tiles;
+    const size_t most = (ntok + 127) / 128;
+    if (s > most) s = most;
     return (int)(s < 1 ? 1 : (s > 32 ? 32 : s));
 }
 
 }  // namespace
 
-cudaError_t generic_prefill(const FwdArgs &a, int io, cudaStream_t st) {
-    const int Dh = a.D / a.H;
-    const size_t smem = fwd_smem_bytes(Dh);
-    dim3 grid(a.H, a.B);
-    cudaError_t e;
-    const bool save = a.save_u != nullptr;
-#define LAUNCH_PREFILL(IOT, SAVE)                                                     \
-    do {                                                                              \
-        if ((e = set_smem(generic_prefill_kernel<IOT, SAVE>, smem)) != cudaSuccess) return e; \
-        generic_prefill_kernel<IOT, SAVE><<<grid, NT, smem, st>>>(a);                 \
-    } while (0)
-    if (io == RGLRU_F32) { if (save) LAUNCH_PREFILL(float, true); else LAUNCH_PREFILL(float, false); }
-    else { if (save) LAUNCH_PREFILL(__nv_bfloat16, true); else LAUNCH_PREFILL(__nv_bfloat16, false); }
-#undef LAUNCH_PREFILL
+size_t generic_prefill_workspace_bytes(int B, int D, int io) {
+    return align256((size_t)B * D * sizeof(uint4)) + align256((size_t)B * 3 * D * (io == RGLRU_F32 ? 4 : 2));
+}
+
+namespace {
+template <typename IOT, bool SAVE, int BM>
+cudaError_t launch_forward(const FwdArgs &a, const Chain &ch, cudaStream_t st) {
+    const int Dh = a.D / a.H, nchunk = ceil_div(a.T, BM), ntile = ceil_div(Dh, BM);
+    const size_t grid = (size_t)nchunk * a.B * a.H * ntile;
+    if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    if (Dh % 4 == 0) generic_forward_kernel<IOT, SAVE, BM, true><<<(unsigned)grid, MT, 0, st>>>(a, ch, nchunk, ntile);
+    else generic_forward_kernel<IOT, SAVE, BM, false><<<(unsigned)grid, MT, 0, st>>>(a, ch, nchunk, ntile);
     return cudaGetLastError();
+}
+template <typename IOT, bool SAVE>
+cudaError_t forward_any(const FwdArgs &a, const Chain &ch, cudaStream_t st) {
+    const int Dh = a.D / a.H;
+    const size_t blocks64 = (size_t)ceil_div(a.T, 64) * a.B * a.H * ceil_div(Dh, 64);
+    return tile_rows(blocks64) == 64 ? launch_forward<IOT, SAVE, 64>(a, ch, st) : launch_forward<IOT, SAVE, 32>(a, ch, st);
+}
+Chain make_chain(uint4 *slots, uint32_t *status) {
+    const uint32_t tag = next_call_tag();
+    return Chain{slots, tag, tag * 0x85EBCA6Bu + 0x27220A95u, g_spin_limit_ns, status};
+}
+template <typename IOT, int BM>
+cudaError_t launch_du(const BwdArgs &q, cudaStream_t st) {
+    const int Dh = q.D / q.H, ntile = ceil_div(Dh, 2 * BM);
+    const size_t grid = (size_t)ceil_div((size_t)q.B * q.T, BM) * q.H * ntile;
+    if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    if (Dh % 4 == 0) generic_bwd_du_kernel<IOT, BM, true><<<(unsigned)grid, MT, 0, st>>>(q, ntile);
+    else generic_bwd_du_kernel<IOT, BM, false><<<(unsigned)grid, MT, 0, st>>>(q, ntile);
+    return cudaGetLastError();
+}
+template <int BM>
+cudaError_t launch_dw(const BwdArgs &q, cudaStream_t st) {
+    const int Dh = q.D / q.H, mtile = ceil_div(Dh, BM), ntile = ceil_div(Dh, 2 * BM);
+    const unsigned grid = (unsigned)((size_t)q.S * 2 * q.H * mtile * ntile);
+    if (Dh % 4 == 0) generic_bwd_dw_kernel<BM, true><<<grid, MT, 0, st>>>(q, mtile, ntile);
+    else generic_bwd_dw_kernel<BM, false><<<grid, MT, 0, st>>>(q, mtile, ntile);
+    return cudaGetLastError();
+}
+}  // namespace
+
+// Workspace body: chain records | private copy of conv_state_in.  The copy is used only when the caller's conv_state_out
+// aliases it: blocks of the first chunk read the carried inputs of the whole head while blocks of the last chunk write theirs.
+// (h0 needs none: the only block that reads a channel's h0 precedes the one that writes its h_T in the chain.)
+cudaError_t generic_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_t st) {
+    FwdArgs f = a;
+    const Chain ch = make_chain((uint4 *)ws_body, a.status);
+    const size_t cs_bytes = (size_t)a.B * 3 * a.D * (io == RGLRU_F32 ? 4 : 2);
+    const uintptr_t ci = (uintptr_t)a.cs_in, co = (uintptr_t)a.cs_out;
+    if (ci && ci < co + cs_bytes && co < ci + cs_bytes) {
+        void *copy = (char *)ws_body + align256((size_t)a.B * a.D * sizeof(uint4));
+        cudaError_t e = cudaMemcpyAsync(copy, a.cs_in, cs_bytes, cudaMemcpyDeviceToDevice, st);
+        if (e != cudaSuccess) return e;
+        f.cs_in = copy;
+    }
+    return io == RGLRU_F32 ? forward_any<float, false>(f, ch, st) : forward_any<__nv_bfloat16, false>(f, ch, st);
 }
 
 cudaError_t generic_decode(const FwdArgs &a, int io, cudaStream_t st) {
     const int Dh = a.D / a.H;
-    const size_t smem = fwd_smem_bytes(Dh);
+    const size_t smem = decode_smem_bytes(Dh);
     dim3 grid(a.H, (a.B + GT - 1) / GT);
     cudaError_t e;
     if (io == RGLRU_F32) {
@@ -504,83 +902,80 @@ cudaError_t state_conv_grads(const BwdArgs &q, int io, const void *du, bool du_i
     return cudaGetLastError();
 }
 
-cudaError_t reduce_partials(const float *in, int nparts, size_t stride, float *out, size_t n, cudaStream_t st) {
-    if (out == nullptr || n == 0) return cudaSuccess;
-    reduce_partials_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(in, nparts, stride, out, n);
-    return cudaGetLastError();
-}
-
-cudaError_t reduce_partials3(const float *in, int nparts, size_t stride, float *out0, size_t n0, float *out1, size_t n1, float *out2,
-                             size_t n2, cudaStream_t st) {
+void add_reduce_job(ReduceJobs &jobs, const float *in, int nparts, size_t stride, float *out0, size_t n0, float *out1, size_t n1, float *out2, size_t n2) {
     const size_t n = n0 + n1 + n2;
-    if (n == 0 || (out0 == nullptr && out1 == nullptr && out2 == nullptr)) return cudaSuccess;
-    reduce_partials3_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(in, nparts, stride, out0, n0, out1, n1, out2, n2);
+    if (n == 0 || (out0 == nullptr && out1 == nullptr && out2 == nullptr)) return;
+    ReduceJob &q = jobs.job[jobs.n++];
+    q = ReduceJob{in, stride, out0, out1, out2, n0, n1, n2, nparts, nparts > 16, 0};   // up to 16 parts are two rounds of loads for one thread
+    q.blocks = ceil_div(n, q.sliced ? 32 : 256);
+}
+cudaError_t run_reduce_jobs(const ReduceJobs &jobs, cudaStream_t st) {
+    int blocks = 0;
+    for (int i = 0; i < jobs.n; ++i) blocks += jobs.job[i].blocks;
+    if (blocks == 0) return cudaSuccess;
+    reduce_jobs_kernel<<<blocks, 256, 0, st>>>(jobs);
     return cudaGetLastError();
 }
 
 size_t generic_backward_workspace_bytes(int B, int T, int D, int H) {
     const size_t btd = (size_t)B * T * D, Dh = D / H;
-    const int nchunk = (T + GENERIC_BWD_CHUNK - 1) / GENERIC_BWD_CHUNK;
-    const int S = dw_splits((size_t)B * T);
     size_t bytes = 4 * align256(btd * sizeof(float));
-    bytes += align256((size_t)B * 3 * D * sizeof(float));
-    bytes += align256((size_t)B * nchunk * 5 * D * sizeof(float));
-    bytes += align256((size_t)S * 2 * H * Dh * Dh * sizeof(float));
+    bytes += align256((size_t)B * ceil_div(T, RCHUNK) * 3 * D * sizeof(float));
+    bytes += align256((size_t)B * ceil_div(T, GENERIC_BWD_CHUNK) * 5 * D * sizeof(float));
+    bytes += align256((size_t)dw_splits((size_t)B * T, H, (int)Dh) * 2 * H * Dh * Dh * sizeof(float));
+    bytes += 2 * align256((size_t)B * D * sizeof(uint4));
     return bytes;
 }
 
 cudaError_t generic_backward(const FwdArgs &fwd_in, BwdArgs &q, int io, void *ws_body, cudaStream_t st) {
     const int B = q.B, T = q.T, D = q.D, H = q.H, Dh = D / H;
-    const size_t btd = (size_t)B * T * D;
+    const size_t btd = (size_t)B * T * D, wsz = (size_t)H * Dh * Dh;
     char *p = (char *)ws_body;
-    q.u = (float *)p; p += align256(btd * sizeof(float));
-    q.r = (float *)p; p += align256(btd * sizeof(float));
-    q.gi = (float *)p; p += align256(btd * sizeof(float));
-    q.hp = (float *)p; p += align256(btd * sizeof(float));
-    q.nchunk = (T + GENERIC_BWD_CHUNK - 1) / GENERIC_BWD_CHUNK;
-    q.S = dw_splits((size_t)B * T);
-    q.part_vec = (float *)p; p += align256((size_t)B * 3 * D * sizeof(float));
-    q.part_conv = (float *)p; p += align256((size_t)B * q.nchunk * 5 * D * sizeof(float));
-    q.part_dw = (float *)p;
+    auto take = [&](size_t bytes) { char *at = p; p += align256(bytes); return at; };
+    q.u = (float *)take(btd * sizeof(float));
+    q.r = (float *)take(btd * sizeof(float));
+    q.gi = (float *)take(btd * sizeof(float));
+    q.hp = (float *)take(btd * sizeof(float));
+    const int rchunks = ceil_div(T, RCHUNK);
+    q.nchunk = ceil_div(T, GENERIC_BWD_CHUNK);
+    q.S = dw_splits((size_t)B * T, H, Dh);
+    q.part_vec = (float *)take((size_t)B * rchunks * 3 * D * sizeof(float));
+    q.part_conv = (float *)take((size_t)B * q.nchunk * 5 * D * sizeof(float));
+    q.part_dw = (float *)take((size_t)q.S * 2 * wsz * sizeof(float));
+    uint4 *slots_f = (uint4 *)take((size_t)B * D * sizeof(uint4)), *slots_r = (uint4 *)take((size_t)B * D * sizeof(uint4));
+    const bool f32 = io == RGLRU_F32;
 
     // 1. forward sweep, keeping u, r, i and h_{t-1} in fp32
     FwdArgs f = fwd_in;
     f.save_u = q.u; f.save_r = q.r; f.save_i = q.gi; f.save_hprev = q.hp;
-    cudaError_t e = generic_prefill(f, io, st);
+    const Chain chf = make_chain(slots_f, fwd_in.status), chr = make_chain(slots_r, fwd_in.status);
+    cudaError_t e = f32 ? forward_any<float, true>(f, chf, st) : forward_any<__nv_bfloat16, true>(f, chf, st);
     if (e != cudaSuccess) return e;
     // 2. reverse-time scan + element-wise adjoints
-    dim3 g2((D + NT - 1) / NT, B);
-    if (io == RGLRU_F32) generic_bwd_scan_kernel<float><<<g2, NT, 0, st>>>(q);
-    else generic_bwd_scan_kernel<__nv_bfloat16><<<g2, NT, 0, st>>>(q);
+    const int ctiles = ceil_div(D, 32);
+    const size_t g2 = (size_t)rchunks * B * ctiles;
+    if (g2 > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    if (f32) generic_bwd_scan_kernel<float><<<(unsigned)g2, NT, 0, st>>>(q, chr, rchunks, ctiles);
+    else generic_bwd_scan_kernel<__nv_bfloat16><<<(unsigned)g2, NT, 0, st>>>(q, chr, rchunks, ctiles);
     // 3. du += W^T dz
-    const size_t smem3 = sizeof(float) * 2 * GT * Dh;
-    dim3 g3(H, (unsigned)((btd / D + GT - 1) / GT));
-    if (io == RGLRU_F32) {
-        if ((e = set_smem(generic_bwd_du_kernel<float>, smem3)) != cudaSuccess) return e;
-        generic_bwd_du_kernel<float><<<g3, NT, smem3, st>>>(q);
-    } else {
-        if ((e = set_smem(generic_bwd_du_kernel<__nv_bfloat16>, smem3)) != cudaSuccess) return e;
-        generic_bwd_du_kernel<__nv_bfloat16><<<g3, NT, smem3, st>>>(q);
-    }
-    // 4. dW partials and their reduction
-    dim3 g4(H * ((Dh + GT - 1) / GT), (Dh + NT - 1) / NT, q.S);
-    generic_bwd_dw_kernel<<<g4, NT, 0, st>>>(q);
-    const size_t wsz = (size_t)H * Dh * Dh;
-    reduce_partials_kernel<<<(unsigned)((wsz + 255) / 256), 256, 0, st>>>(q.part_dw, q.S, 2 * wsz, q.dW_a, wsz);
-    reduce_partials_kernel<<<(unsigned)((wsz + 255) / 256), 256, 0, st>>>(q.part_dw + wsz, q.S, 2 * wsz, q.dW_x, wsz);
+    const size_t blocks3 = (size_t)ceil_div((size_t)B * T, 64) * H * ceil_div(Dh, 128);
+    if (tile_rows(blocks3) == 64) e = f32 ? launch_du<float, 64>(q, st) : launch_du<__nv_bfloat16, 64>(q, st);
+    else e = f32 ? launch_du<float, 32>(q, st) : launch_du<__nv_bfloat16, 32>(q, st);
+    if (e != cudaSuccess) return e;
+    // 4. dW partial sums
+    const size_t blocks4 = (size_t)q.S * 2 * H * ceil_div(Dh, 64) * ceil_div(Dh, 128);
+    if ((e = tile_rows(blocks4) == 64 ? launch_dw<64>(q, st) : launch_dw<32>(q, st)) != cudaSuccess) return e;
     // 5. Conv1D adjoint
     dim3 g5((D + NT - 1) / NT, q.nchunk, B);
-    if (io == RGLRU_F32) generic_bwd_conv_kernel<float><<<g5, NT, 0, st>>>(q);
+    if (f32) generic_bwd_conv_kernel<float><<<g5, NT, 0, st>>>(q);
     else generic_bwd_conv_kernel<__nv_bfloat16><<<g5, NT, 0, st>>>(q);
     if ((e = state_conv_grads(q, io, q.hp, false, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
-    // 6. deterministic reductions of the per-channel partial sums
-    const unsigned gd = (D + 255) / 256;
-    reduce_partials_kernel<<<gd, 256, 0, st>>>(q.part_vec, B, (size_t)3 * D, q.dlambda, D);
-    reduce_partials_kernel<<<gd, 256, 0, st>>>(q.part_vec + D, B, (size_t)3 * D, q.db_a, D);
-    reduce_partials_kernel<<<gd, 256, 0, st>>>(q.part_vec + 2 * (size_t)D, B, (size_t)3 * D, q.db_x, D);
-    reduce_partials_kernel<<<(4 * D + 255) / 256, 256, 0, st>>>(q.part_conv, B * q.nchunk, (size_t)5 * D, q.dconv_w, (size_t)4 * D);
-    reduce_partials_kernel<<<gd, 256, 0, st>>>(q.part_conv + 4 * (size_t)D, B * q.nchunk, (size_t)5 * D, q.dconv_b, D);
-    return cudaGetLastError();
+    // 6. deterministic reductions of the partial sums
+    ReduceJobs jobs{};
+    add_reduce_job(jobs, q.part_dw, q.S, 2 * wsz, q.dW_a, wsz, q.dW_x, wsz, nullptr, 0);
+    add_reduce_job(jobs, q.part_vec, B * rchunks, (size_t)3 * D, q.dlambda, D, q.db_a, D, q.db_x, D);
+    add_reduce_job(jobs, q.part_conv, B * q.nchunk, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
+    return run_reduce_jobs(jobs, st);
 }
 
 }  // namespace rglru

@@ -74,17 +74,18 @@ struct BwdArgs {
     void *dcs_in;
     // workspace arrays, each [B,T,D] fp32: u, r -> dz_a, i -> dz_x, hprev -> du
     float *u, *r, *gi, *hp;
-    float *part_vec;   // [B][3][D]        partial sums of dlambda, db_a, db_x
+    float *part_vec;   // [B*chunks][3][D] partial sums of dlambda, db_a, db_x
     float *part_conv;  // [B*nchunk][5][D] partial sums of dconv_w (4 rows) and dconv_b
     float *part_dw;    // [S][2][H*Dh*Dh]  partial sums of dW_a, dW_x
-    int nchunk, S;
+    int nchunk, S;     // chunks of the conv adjoint, token splits of dW
 };
 
 // ---- shape-generic CUDA-core kernels (any D_h <= GENERIC_MAX_DH, fp32 or bf16 io) ----
 constexpr int GENERIC_MAX_DH = 1024;
-constexpr int GENERIC_BWD_CHUNK = 64;  // tokens per thread in the conv backward
+constexpr int GENERIC_BWD_CHUNK = 32;  // tokens per thread in the conv backward
 size_t generic_backward_workspace_bytes(int B, int T, int D, int H);
-cudaError_t generic_prefill(const FwdArgs &a, int io, cudaStream_t st);
+size_t generic_prefill_workspace_bytes(int B, int D, int io);
+cudaError_t generic_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_t st);
 cudaError_t generic_decode(const FwdArgs &a, int io, cudaStream_t st);
 cudaError_t generic_backward(const FwdArgs &fwd, BwdArgs &b, int io, void *ws_body, cudaStream_t st);
 
@@ -112,11 +113,19 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &b, const void *y_saved, 
 // on conv_state_out added to the rows it copies (dx_{T-3+k} is recomputed from du with the term added, so it is rounded once;
 // rows of conv_state_in when T < 3).  du is [B,T,D] of DUT (float or __half); io tensors are IOT.  No-op without dcs_in / dcs_out.
 cudaError_t state_conv_grads(const BwdArgs &q, int io, const void *du, bool du_is_half, cudaStream_t st);
-// out[i] = sum over p of in[p * stride + i] in ascending p (fixed order: run-to-run identical results)
-cudaError_t reduce_partials(const float *in, int nparts, size_t stride, float *out, size_t n, cudaStream_t st);
-// A row of n0 + n1 + n2 values summed over the parts and split over up to three output arrays (any of them may be null or
-// empty); four interleaved running sums over ascending p, added at the end: also a fixed order.
-cudaError_t reduce_partials3(const float *in, int nparts, size_t stride, float *out0, size_t n0, float *out1, size_t n1, float *out2,
-                             size_t n2, cudaStream_t st);
+// Sums over partial results, all of a call in one launch: out[i] = sum over p of in[p * stride + i] in a fixed order (run-to-run
+// identical results), the row of n0 + n1 + n2 values being split over up to three output arrays (any may be null or empty).
+struct ReduceJob {
+    const float *in;
+    size_t stride;
+    float *out0, *out1, *out2;
+    size_t n0, n1, n2;
+    int nparts, sliced, blocks;
+};
+struct ReduceJobs { ReduceJob job[3]; int n; };
+void add_reduce_job(ReduceJobs &jobs, const float *in, int nparts, size_t stride, float *out0, size_t n0, float *out1, size_t n1, float *out2, size_t n2);
+cudaError_t run_reduce_jobs(const ReduceJobs &jobs, cudaStream_t st);
+// A tag no other call uses: validity tag of the carry records a call publishes
+uint32_t next_call_tag();
 
 }  // namespace rglru

@@ -713,13 +713,13 @@ bool make_activation_map(CUtensorMap *tm, const void *ptr, int B, int T, int D, 
 
 std::atomic<uint32_t> g_call_counter{0};
 
-uint32_t next_tag() {
+}  // namespace
+
+uint32_t next_call_tag() {
     static const uint32_t salt = (uint32_t)std::chrono::steady_clock::now().time_since_epoch().count() * 2654435761u;
     uint32_t t = salt + 0x9E3779B9u * (g_call_counter.fetch_add(1) + 1u);
     return t == 0 ? 1u : t;
 }
-
-}  // namespace
 
 unsigned long long g_spin_limit_ns = 2000000000ull;  // bounded waits give up after this long
 
@@ -817,7 +817,7 @@ cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes,
     if (S > a.B * p.tps) S = a.B * p.tps;
     p.S = S;
     p.tiles_total = record_slots(a.B, G) * p.tps;
-    p.tag = next_tag();
+    p.tag = next_call_tag();
     p.tag_wait = (a.flags & RGLRU_FLAG_TEST_CARRY_NEVER_ARRIVES) ? ~p.tag : p.tag;
     p.agg = (uint4 *)ws_body;
     p.spin_ns = g_spin_limit_ns;

@@ -582,7 +582,7 @@ inline int groups_of_heads(int D, int H) { const int k = DH / (D / H); return (H
 struct BwdLayout {
     size_t BT, BTp, off_u, off_z, off_dz, off_du, off_y, off_hT, off_cs, off_fold, off_xin, off_pvec, off_pconv, off_pdw,
         off_wt, off_w16, off_fws, total;
-    int nchunk, nchunk_conv, S, kb_per_split;
+    int nchunk, S, kb_per_split;
 };
 
 BwdLayout bwd_layout(int B, int T, int D, int Hl) {
@@ -592,7 +592,6 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     L.BT = (size_t)B * T;
     L.BTp = (L.BT + 63) & ~(size_t)63;
     L.nchunk = (T + CHUNK - 1) / CHUNK;
-    L.nchunk_conv = (T + GENERIC_BWD_CHUNK - 1) / GENERIC_BWD_CHUNK;
     const int kblocks = (int)(L.BTp / 64);
     L.S = kblocks < 8 ? kblocks : 8;
     L.kb_per_split = (kblocks + L.S - 1) / L.S;
@@ -678,6 +677,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     const dim3 grid_ew((D + 255) / 256, L.nchunk, B);
     conv_forward_kernel<<<grid_ew, 256, 0, st>>>(a);
 
+    ReduceJobs jobs{};
     GemmArgs g{};
     g.H = H; g.D = D; g.hstride = hstride; g.cvalid = hstride; g.status = status; g.spin_ns = g_spin_limit_ns;
     const unsigned mtiles = (unsigned)((L.BT + 127) / 128);
@@ -725,7 +725,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
         tc_gemm_kernel<<<gemm_grid(g), GEMM_THREADS, GEMM_SMEM_ALLOC, st>>>(g);
         const size_t wsz = (size_t)H * DH * DH;
         if (dh == DH) {   // one head per group: the partial sums already have the layout of dW
-            if ((e = reduce_partials3(part, L.S, 2 * wsz, q.dW_a, wsz, q.dW_x, wsz, nullptr, 0, st)) != cudaSuccess) return e;
+            add_reduce_job(jobs, part, L.S, 2 * wsz, q.dW_a, wsz, q.dW_x, wsz, nullptr, 0);
         } else {
             const size_t nout = (size_t)2 * q.H * dh * dh;
             reduce_dw_blocks_kernel<<<(unsigned)((nout + 255) / 256), 256, 0, st>>>(part, L.S, H, dh, q.H, q.dW_a, q.dW_x);
@@ -733,15 +733,15 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     }
     // 6. per-channel sums, Conv1D adjoint
     const int nparts = B * L.nchunk;
-    if ((e = reduce_partials3(a.part_vec, nparts, (size_t)3 * D, q.dlambda, D, q.db_a, D, q.db_x, D, st)) != cudaSuccess) return e;
+    add_reduce_job(jobs, a.part_vec, nparts, (size_t)3 * D, q.dlambda, D, q.db_a, D, q.db_x, D);
     ConvBwdArgs cb{};
     cb.B = B; cb.T = T; cb.D = D; cb.nchunk = L.nchunk;
     cb.x = a.x; cb.conv_w = a.conv_w; cb.cs_in = a.cs_in; cb.du = du; cb.dx = (__nv_bfloat16 *)q.dx;
     cb.part_conv = (float *)(ws + L.off_pconv);
     conv_backward_kernel<<<grid_ew, 256, 0, st>>>(cb);
     if ((e = state_conv_grads(q, RGLRU_BF16, du, true, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
-    if ((e = reduce_partials3(cb.part_conv, nparts, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0, st)) != cudaSuccess) return e;
-    return cudaGetLastError();
+    add_reduce_job(jobs, cb.part_conv, nparts, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
+    return run_reduce_jobs(jobs, st);
 }
 
 }  // namespace rglru

@@ -1,0 +1,46 @@
+"""GPU parity at the sizes where a kernel variant can go wrong: edges of its tiles, remainders, the smallest and largest of its
+range.  Every case is compared with the fp64 oracle under the tolerances of util.py."""
+import numpy as np
+import pytest
+
+from paper_2402_19427_b200 import inputs as synth
+from util import assert_close, f64, oracle_prefill, to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+GENERIC = 1  # RGLRU_FLAG_FORCE_GENERIC
+
+
+def forward_and_backward(oracle, B, T, D, H, io, flags, seed, in_place=True):
+    """Forward with in-place state and backward through the carried state, both against the oracle."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    inp = synth.make_inputs(B, T, D, H, io=io, seed=seed, with_dy=True, with_state=True, bias_scale=0.2)
+    params = binding.Params.from_numpy(inp["params"], io)
+    x, h0, cs = to_dev(inp["x"], io), to_dev(inp["h0"]), to_dev(inp["conv_state"], io)
+    h, c = (h0.clone(), cs.clone())
+    y, _, _ = binding.prefill(x, params, h0=h, conv_state_in=c, h_T=h, conv_state_out=c, flags=flags)
+    ws = binding.alloc_workspace(binding.make_shape(B, T, D, H, x.dtype, flags=flags), binding.OP_BACKWARD, x.device)
+    ws[256:].fill_(0xFF)   # NaN patterns: nothing may depend on what the workspace held
+    g = binding.backward(x, params, to_dev(inp["dy"], io), h0=h0, conv_state_in=cs, flags=flags, state_grads=True, workspace=ws)
+    torch.cuda.synchronize()
+    assert binding.query_status(ws) == binding.OK
+    h064, cs64 = inp["h0"].astype(np.float64), inp["conv_state"].astype(np.float64)
+    yr, hr, cr = oracle_prefill(oracle, inp, h0=h064, cs=cs64)
+    assert_close("y", to_np(y), yr, io); assert_close("h_T", to_np(h), hr, io)
+    assert np.array_equal(to_np(c), cr)
+    gr = oracle.backward(inp["x"].astype(np.float64), f64(inp["params"]), H, inp["dy"].astype(np.float64), h0=h064, conv_state_in=cs64, state_grads=True)
+    for k in gr:
+        # fp32: the 1e-4 bound is absolute for values of order one; gradients that sum over many tokens scale with their size
+        scale = max(1.0, float(np.abs(gr[k]).max())) if io == "f32" else 1.0
+        assert_close("d" + k, to_np(g[k]), gr[k], io, scale=scale)
+
+
+@pytest.mark.parametrize("B,T,D,H,io", [
+    (2, 321, 1600, 5, "f32"),    # 64-row blocks, six chunks with a one-token tail
+    (2, 321, 1610, 5, "f32"),    # the same with a head width that is no multiple of four (322: scalar loads)
+    (2, 257, 1610, 5, "bf16"),
+    (1, 32, 32, 1, "f32"), (1, 33, 33, 1, "f32"), (3, 65, 132, 2, "f32"),   # 32-row blocks at their edges
+    (1, 70, 1024, 1, "f32"),     # the widest head
+])
+def test_cuda_core_blocks_and_chunk_chain(oracle, B, T, D, H, io):
+    forward_and_backward(oracle, B, T, D, H, io, GENERIC, seed=900 + T)
