@@ -1,6 +1,8 @@
-"""Thin ctypes binding over the C ABI in ``include/rglru.h``.
+"""Thin binding over the C ABI in ``include/rglru.h``.
 
-Argument marshalling only: every step of the path (Conv1D, gates, decay, scan, state hand-off,
+``prefill``, ``decode_step`` and ``backward`` go through the native extension ``_host`` (csrc/host_binding.cpp), which checks
+the arguments, allocates the outputs and calls the library; calls that it does not take, because an argument is wrong or
+unusual, go through the ctypes path below, which names what is wrong.  Argument marshalling only: every step of the path (Conv1D, gates, decay, scan, state hand-off,
 backward) runs inside the CUDA library.  PyTorch appears here for device memory and streams.
 There is no fallback: if the shared library is missing or a call fails, an exception is raised.
 """
@@ -14,6 +16,7 @@ import torch
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "librglru_b200.so")
+HOST_PATH = os.path.join(_PKG, "_host.so")
 
 OK, ERR_NULL, ERR_SHAPE, ERR_UNSUPPORTED, ERR_ALIGN, ERR_WORKSPACE, ERR_CUDA, ERR_TIMEOUT, ERR_ALIAS = range(9)
 F32, BF16 = 0, 1
@@ -44,6 +47,19 @@ class RglruError(RuntimeError):
 
 
 _lib = None
+_host = None
+
+
+def _native():
+    """The native host extension; raises if it has not been built."""
+    global _host
+    if _host is None:
+        load()
+        if not os.path.exists(HOST_PATH):
+            raise RuntimeError(f"{HOST_PATH} is missing: build it with `python -m paper_2402_19427_b200.build`")
+        from . import _host as ext
+        _host = ext
+    return _host
 
 
 def load() -> ctypes.CDLL:
@@ -129,6 +145,8 @@ class Params:
         self.H, self.D, self.io = H, D, io
         self.ptrs = ParamPtrs(conv_w.data_ptr(), 0 if conv_b is None else conv_b.data_ptr(), W_a.data_ptr(),
                               b_a.data_ptr(), W_x.data_ptr(), b_x.data_ptr(), lam.data_ptr())
+        self.native = _native()
+        self.handle = self.native.params_handle(conv_w, conv_b, W_a, b_a, W_x, b_x, lam)
 
     @classmethod
     def from_numpy(cls, p: dict, io: str, device="cuda"):
@@ -163,6 +181,9 @@ def prefill(x, params: Params, h0=None, conv_state_in=None, c=8.0, flags=0, y=No
             workspace=None, gate_branch=None, a_prod=None):
     """y, h_T, conv_state_out = Conv1D(4) + RG-LRU over x[B,T,D] (rglru_prefill; rglru_prefill_ex when an extra is given).
     ``gate_branch`` [B,T,D]: y_t = h_t * GeLU(gate_branch_t); ``a_prod`` [B,D] fp32 receives prod_t a_t."""
+    out = params.native.prefill(params.handle, x, h0, conv_state_in, c, flags, y, h_T, conv_state_out, workspace, gate_branch, a_prod)
+    if out is not None:
+        return out
     lib = load()
     B, T, D = x.shape
     shape = make_shape(B, T, D, params.H, x.dtype, c, flags)
@@ -215,6 +236,9 @@ def prefill_static_scratch(x, params: Params, y, h_T, conv_state_out, h0=None, c
 
 def decode_step(x, params: Params, h, conv_state, c=8.0, flags=0, y=None, workspace=None):
     """One token for B sequences; h[B,D] fp32 and conv_state[B,3,D] are updated in place; returns y[B,D]."""
+    out = params.native.decode_step(params.handle, x, h, conv_state, c, flags, y, workspace)
+    if out is not None:
+        return out
     lib = load()
     B, D = x.shape
     shape = make_shape(B, 1, D, params.H, x.dtype, c, flags)
@@ -239,6 +263,10 @@ def backward(x, params: Params, dy, h0=None, conv_state_in=None, y=None, c=8.0, 
              dh_T=None, dconv_state_out=None, state_grads=False):
     """Gradients of sum(dy*y) [+ sum(dh_T*h_T) + sum(dconv_state_out*conv_state_out)] (rglru_backward): dict with x (io dtype)
     and fp32 conv_w, conv_b, W_a, b_a, W_x, b_x, lam; with ``state_grads`` also h0 [B,D] fp32 and conv_state [B,3,D] io."""
+    if out is None:
+        g = params.native.backward(params.handle, x, dy, h0, conv_state_in, y, c, flags, workspace, dh_T, dconv_state_out, state_grads)
+        if g is not None:
+            return g
     lib = load()
     B, T, D = x.shape
     H, Dh = params.H, D // params.H

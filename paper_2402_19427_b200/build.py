@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import os
 import subprocess
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
@@ -10,6 +11,8 @@ _ROOT = os.path.dirname(_PKG)
 CSRC = os.path.join(_PKG, "csrc")
 INCLUDE = os.path.join(_ROOT, "include")
 LIB_PATH = os.path.join(_PKG, "librglru_b200.so")
+HOST_PATH = os.path.join(_PKG, "_host.so")       # CPython extension behind binding.py (links against the library above)
+HOST_SOURCE = os.path.join(CSRC, "host_binding.cpp")
 SOURCES = ["rglru_api.cu", "rglru_generic.cu", "rglru_sm100.cu", "rglru_sm100_decode.cu", "rglru_sm100_bwd.cu", "rglru_static_scratch.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -29,8 +32,27 @@ def _stale(target: str, deps) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def _host_command():
+    """g++ command of the host extension: Python and torch headers, the CUDA library found beside it at run time."""
+    import torch
+    root = os.path.dirname(os.path.abspath(torch.__file__))
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.path.isabs(_nvcc()) else "/usr/local/cuda"
+    return ["g++", "-O2", "-std=c++20", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", HOST_SOURCE,
+            "-o", HOST_PATH, "-I", INCLUDE, "-I", sysconfig.get_paths()["include"], "-I", os.path.join(root, "include"),
+            "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"), "-I", os.path.join(cuda, "include"),
+            "-L", _PKG, "-l:librglru_b200.so", "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda",
+            "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"]
+
+
+def _run(cmd):
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("build failed:\n" + " ".join(cmd) + "\n" + r.stdout + r.stderr)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
-    """Compile every .cu under csrc/ and link ``librglru_b200.so`` next to this file.  Returns its path."""
+    """Compile every .cu under csrc/ and link ``librglru_b200.so`` next to this file, then the host extension ``_host.so``.
+    Returns the library's path."""
     headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     headers.append(os.path.join(INCLUDE, "rglru.h"))
     objdir = os.path.join(_PKG, "_build")
@@ -58,6 +80,9 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("link failed:\n" + r.stdout + r.stderr)
+    # the extension refers to the library by name only, so a rebuilt library does not make it stale
+    if force or _stale(HOST_PATH, [HOST_SOURCE, os.path.join(INCLUDE, "rglru.h")]):
+        _run(_host_command())
     return LIB_PATH
 
 

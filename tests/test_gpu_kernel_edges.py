@@ -44,3 +44,24 @@ def forward_and_backward(oracle, B, T, D, H, io, flags, seed, in_place=True):
 ])
 def test_cuda_core_blocks_and_chunk_chain(oracle, B, T, D, H, io):
     forward_and_backward(oracle, B, T, D, H, io, GENERIC, seed=900 + T)
+
+
+@pytest.mark.parametrize("change,error", [
+    (dict(h0=lambda t: t.double()), ValueError), (dict(x=lambda t: t.transpose(0, 1)), ValueError), (dict(workspace=lambda t: t[:128]), RuntimeError),
+    (dict(flags=lambda v: 1 << 40), RuntimeError), (dict(conv_state_in=lambda t: t.cpu()), ValueError)])
+def test_calls_the_native_path_does_not_take(change, error):
+    """A call with an argument that is wrong raises what the checked path raises, launches nothing, and leaves the next call fine."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    inp = synth.make_inputs(2, 2, 64, 2, io="f32", seed=3, with_state=True)
+    params = binding.Params.from_numpy(inp["params"], "f32")
+    args = dict(x=to_dev(inp["x"]), h0=to_dev(inp["h0"]), conv_state_in=to_dev(inp["conv_state"]), flags=0,
+                workspace=binding.alloc_workspace(binding.make_shape(2, 2, 64, 2, torch.float32), binding.OP_PREFILL, torch.device("cuda", 0)))
+    good = binding.prefill(params=params, **args)[0].clone()
+    name, make = next(iter(change.items()))
+    if name == "flags":   # a flag word wider than 32 bits is truncated as ctypes does, not an error
+        assert torch.equal(binding.prefill(params=params, **dict(args, flags=make(0)))[0], good)
+        return
+    with pytest.raises(error):
+        binding.prefill(params=params, **dict(args, **{name: make(args[name])}))
+    assert torch.equal(binding.prefill(params=params, **args)[0], good)
