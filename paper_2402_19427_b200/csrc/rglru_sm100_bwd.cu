@@ -1,5 +1,5 @@
 // sm_100a backward of the RG-LRU temporal core (bf16 io, head width a multiple of 32 up to 256 -- narrower heads in groups of
-// 256 channel slots --, T a multiple of 8).
+// 256 channel slots --, any T).
 //
 // The paper gives no backward; this is reverse-mode differentiation of Eq. 1-4 and the Conv1D.  The three dense
 // contractions run on tcgen05 tensor cores through one small GEMM kernel, the rest is element-wise and HBM-bound:
@@ -7,10 +7,9 @@
 //                        (every tensor-core operand here is fp16: 11 significant bits instead of bf16's 8 keep the
 //                        rounding of u and dz out of the gradients; finite overflow saturates at +-65504)
 //   2. GEMM              z_a | z_x = u W_a^T | u W_x^T per head (Eq. 1-2 before the sigmoid), fp16 out
-//   3. scan_fold / scan_carry / scan_apply
-//                        reverse-time scan g_t = dy_t + a_{t+1} g_{t+1} over chunks of 128 tokens (fold, carry across
-//                        chunks, re-run with the carry), then the element-wise adjoints: dz_a, dz_x (fp16, token-major),
-//                        the direct part of du (fp16), partial sums of dLambda, db_a, db_x
+//   3. scan              reverse-time scan g_t = dy_t + a_{t+1} g_{t+1} over chunks of 64 tokens with decoupled look-back, and
+//                        the element-wise adjoints: dz_a, dz_x (fp16, token-major), the direct part of du (fp16), partial
+//                        sums of dLambda, db_a, db_x
 //   4. GEMM              du += dz_a W_a + dz_x W_x
 //   5. GEMM (split K)    dW_a | dW_x = dz^T u over all tokens: both operands are read token-major as steps 1 and 3 wrote them
 //                        and handed to the tensor core as MN-major operands (no transposed copies exist); fp32 partial sums
@@ -23,6 +22,7 @@
 
 #include "rglru_internal.h"
 #include "sm100_ptx.cuh"
+#include "sm100_gates.cuh"
 
 namespace rglru {
 namespace {
@@ -30,7 +30,9 @@ namespace {
 using namespace ptx;
 
 constexpr int DH = 256;
-constexpr int CHUNK = 128;                 // tokens per scan chunk = rows of a GEMM tile
+constexpr int SCAN_CHUNK = 64;             // tokens per block of the reverse scan (eight warps x eight tokens)
+constexpr int CONV_CHUNK = 32;             // tokens per thread of the two Conv1D kernels
+constexpr float LOG2E = 1.44269504f;
 constexpr int GEMM_THREADS = 192;          // TMA warp, MMA warp, four epilogue warps
 constexpr int GEMM_STAGES = 4;
 constexpr uint32_t A_STAGE_BYTES = 128 * 128;   // 128 rows x 64 bf16
@@ -242,12 +244,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
 }
 
 // ------------------------------------------------------------------ element-wise kernels
-__device__ __forceinline__ float bf2f(__nv_bfloat16 v) { return __bfloat162float(v); }
 __device__ __forceinline__ float sigmoid_acc(float z) { return 1.0f / (1.0f + expf(-z)); }
 // Hardware-approximate versions for the per-element work (relative error ~1e-6, far inside the gradient tolerance)
 __device__ __forceinline__ float rcp_fast(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float rsqrt_fast(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
-__device__ __forceinline__ float sigmoid_fast(float z) { return rcp_fast(1.0f + __expf(-z)); }
 // 1 - exp(x) for x <= 0 without cancellation near 0
 __device__ __forceinline__ float one_minus_exp(float x) {
     if (x > -0.25f) {   // -x (1 + x/2 + x^2/6 + x^3/24 + x^4/120 + x^5/720): relative truncation error < 2e-7
@@ -270,11 +270,14 @@ struct EwArgs {
     const __nv_bfloat16 *x, *conv_w, *cs_in, *dy, *y;
     const float *conv_b, *b_a, *b_x, *lambda, *h0;
     __half *u, *dz;
-    const __half *z;
+    const __half *z;                  // [tok][H][2][256] before the sigmoid, without the bias
     __half *du;                       // [tok][D]
-    float2 *fold;                     // [B][nchunk][D]: (prod a_t, carry out of the chunk for zero carry in)
-    float *xin;                       // [B][nchunk][D]: a_{t+1} g_{t+1} entering the chunk from later tokens
-    float *part_vec;                  // [B*nchunk][3][D]
+    uint4 *rec;                       // [nchunk][B][D] carry records of the reverse scan
+    uint32_t *epoch;                  // launch counter in the workspace (any starting value): part of the records' tag
+    uint32_t tag;
+    unsigned long long spin_ns;
+    uint32_t *status;
+    float *part_vec;                  // [B*S][3][D]
     const float *dh_T;                // [B][D] gradient arriving on h_T, or null
     float *dh0;                       // [B][D] gradient of h0, or null
 };
@@ -325,253 +328,356 @@ __global__ void reduce_dw_blocks_kernel(const float *part, int S, int G, int dh,
     (gate ? dWx : dWa)[i % per_gate] = acc;
 }
 
-__device__ __forceinline__ __half to_half_sat(float v) { return __float2half_rn(fminf(fmaxf(v, -65504.0f), 65504.0f)); }
+__device__ __forceinline__ f32x2 bf2x(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
+__device__ __forceinline__ f32x2 hf2x(uint32_t w) { return __half22float2(*(const __half2 *)&w); }
+__device__ __forceinline__ f32x2 ld2f(const float *p) { return *(const float2 *)p; }
 
-// u_t = b_c + sum_j w[j] x_{t-j}: one thread per (sequence, chunk, channel), forward in time.  grid (D/256, nchunk, B)
-__global__ void __launch_bounds__(256) conv_forward_kernel(EwArgs a) {
-    const int d = blockIdx.x * 256 + threadIdx.x, c = blockIdx.y, b = blockIdx.z;
-    const int T = a.T, D = a.D;
+// u_t = b_c + sum_j w[j] x_{t-j}: one thread per (sequence, 32 tokens, two adjacent channels), forward in time, eight tokens'
+// loads in flight.  Bound by its 4 bytes per element.  grid (ceil(D/512), ceil(T/CONV_CHUNK), B)
+__global__ void __launch_bounds__(256, 6) conv_forward_kernel(EwArgs a) {
+    const int d = (blockIdx.x * 256 + threadIdx.x) * 2, b = blockIdx.z;
+    const int T = a.T, D = a.D, t0 = blockIdx.y * CONV_CHUNK, t1 = min(T, t0 + CONV_CHUNK);
+    // the scan's carry records are told apart from those an earlier launch with the same host tag (a graph replay) left behind
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *a.epoch += 1u;
     if (d >= D) return;
-    const int t0 = c * CHUNK, t1 = min(T, t0 + CHUNK);
-    float w[4];
+    f32x2 w[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] = bf2f(a.conv_w[(size_t)j * D + d]);
-    const float cb = a.conv_b ? a.conv_b[d] : 0.0f;
-    auto xat = [&](int t) -> float {
-        if (t >= 0) return bf2f(a.x[((size_t)b * T + t) * D + d]);
-        return a.cs_in ? bf2f(a.cs_in[((size_t)b * 3 + (3 + t)) * D + d]) : 0.0f;
+    for (int j = 0; j < 4; ++j) w[j] = bf2x(*(const uint32_t *)(a.conv_w + (size_t)j * D + d));
+    const f32x2 cb = a.conv_b ? ld2f(a.conv_b + d) : pack2(0.f, 0.f);
+    auto xat = [&](int t) -> f32x2 {
+        if (t >= 0) return bf2x(*(const uint32_t *)(a.x + ((size_t)b * T + t) * D + d));
+        return a.cs_in ? bf2x(*(const uint32_t *)(a.cs_in + ((size_t)b * 3 + (3 + t)) * D + d)) : pack2(0.f, 0.f);
     };
-    float x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
-    // eight tokens at a time, all loads first: u token-major (coalesced across the block)
-    const uint32_t sD = (uint32_t)D;   // token stride; sixteen tokens' worth fits 32 bits
-    auto batch8 = [&](__half *pu, const float (&xs)[8]) {
+    f32x2 x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
+    const uint32_t sD = (uint32_t)D / 2;   // token stride in channel pairs
+    for (int t = t0; t < t1; t += 8) {
+        const uint32_t *px = (const uint32_t *)(a.x + ((size_t)b * T + t) * D + d);
+        uint32_t *pu = (uint32_t *)(a.u + ((size_t)b * T + t) * D + d);
+        const int n = t1 - t;
+        uint32_t xs[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) xs[k] = k < n ? px[k * sD] : 0u;
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            const float uv = fmaf(w[3], x3, fmaf(w[2], x2, fmaf(w[1], x1, fmaf(w[0], xs[k], cb))));
-            pu[k * sD] = to_half_sat(uv);
-            x3 = x2; x2 = x1; x1 = xs[k];
-        }
-    };
-    int t = t0;
-    for (; t + 16 <= t1; t += 16) {
-        float xa[8], xb[8];
-        const __nv_bfloat16 *px = a.x + ((size_t)b * T + t) * D + d;
-        __half *pu = a.u + ((size_t)b * T + t) * D + d;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) { xa[k] = bf2f(px[k * sD]); xb[k] = bf2f(px[(8 + k) * sD]); }
-        batch8(pu, xa);
-        batch8(pu + 8 * (size_t)sD, xb);
-    }
-    if (t < t1) {
-        float xa[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) xa[k] = bf2f(a.x[((size_t)b * T + t + k) * D + d]);
-        batch8(a.u + ((size_t)b * T + t) * D + d, xa);
-    }
-}
-
-// Reverse scan, pass 1: per chunk the product of a_t and the carry a_first g_first it hands to earlier tokens when
-// nothing comes in from later ones.  grid (D/256, nchunk, B)
-__global__ void __launch_bounds__(256) scan_fold_kernel(EwArgs a) {
-    const int d = blockIdx.x * 256 + threadIdx.x, c = blockIdx.y, b = blockIdx.z;
-    if (d >= a.D) return;
-    const int T = a.T, D = a.D, h = d / a.hstride, n = d % a.hstride;   // group of heads and channel slot within it
-    const int t0 = c * CHUNK, t1 = min(T, t0 + CHUNK);
-    const float s = decay_rate(a.lambda[d], a.c), ba = a.b_a[d];
-    float carry = 0.0f, Q = 1.0f;
-    const size_t tokb = (size_t)b * T + (t1 - 8);
-    const uint32_t sD = (uint32_t)D, sZ = (uint32_t)a.H * 2 * DH;
-    const __nv_bfloat16 *p_dy = a.dy + tokb * (size_t)sD + d;
-    const __half *p_z = a.z + tokb * sZ + (size_t)h * 2 * DH + n;
-    int tb = t1 - 8;
-    // the kernel waits on memory: 16-token rounds keep 32 loads per thread in flight at 60 registers (32-token rounds
-    // need 128 and measured the same); the pointers sit 8 tokens below the top of the round
-    for (; tb - 8 >= t0; tb -= 16) {
-        float dyv[16], zav[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) { dyv[k] = bf2f(p_dy[(k - 8) * (int)sD]); zav[k] = __half2float(p_z[(k - 8) * (int)sZ]); }
-#pragma unroll
-        for (int k = 15; k >= 0; --k) {
-            const float at = __expf(-s * sigmoid_fast(zav[k] + ba));
-            const float g = dyv[k] + carry;
-            carry = at * g;
-            Q *= at;
-        }
-        p_dy -= 16 * (size_t)sD; p_z -= 16 * (size_t)sZ;
-    }
-    for (; tb >= t0; tb -= 8) {
-        float dyv[8], zav[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) { dyv[k] = bf2f(p_dy[k * sD]); zav[k] = __half2float(p_z[k * sZ]); }
-#pragma unroll
-        for (int k = 7; k >= 0; --k) {
-            const float at = __expf(-s * sigmoid_fast(zav[k] + ba));
-            const float g = dyv[k] + carry;
-            carry = at * g;
-            Q *= at;
-        }
-        p_dy -= 8 * (size_t)sD; p_z -= 8 * (size_t)sZ;
-    }
-    a.fold[((size_t)b * a.nchunk + c) * D + d] = make_float2(Q, carry);
-}
-
-// pass 2: carries across chunks, last chunk first.  grid (D/256, B)
-__global__ void __launch_bounds__(256) scan_carry_kernel(EwArgs a) {
-    const int d = blockIdx.x * 256 + threadIdx.x, b = blockIdx.y;
-    if (d >= a.D) return;
-    // what later tokens hand to the last chunk: the gradient arriving on h_T (h_T = h_{T-1}, factor 1), else nothing
-    float X = a.dh_T ? a.dh_T[(size_t)b * a.D + d] : 0.0f;
-    // sixteen folds are requested at once (loads interleaved with the stores below would go out one at a time)
-    for (int c1 = a.nchunk; c1 > 0; c1 -= 16) {
-        float2 f[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int c = c1 - 1 - j;
-            f[j] = c >= 0 ? a.fold[((size_t)b * a.nchunk + c) * a.D + d] : make_float2(1.0f, 0.0f);
-        }
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int c = c1 - 1 - j;
-            if (c >= 0) {
-                a.xin[((size_t)b * a.nchunk + c) * a.D + d] = X;
-                X = fmaf(f[j].x, X, f[j].y);
-            }
-        }
-    }
-    if (a.dh0) a.dh0[(size_t)b * a.D + d] = X;   // what the first chunk hands on is a_0 g_0, the gradient of h0
-}
-
-// pass 3: the scan with its carry and every element-wise adjoint (derived from Eq. 1-4):
-//   g_t = dy_t + a_{t+1} g_{t+1};  dL = g a (h_{t-1} - a v / m);  dv = g m;  di = dv u;  du = dv i;
-//   dr = -s dL;  dz_a = dr r (1-r);  dz_x = di i (1-i);  dLambda += dL c r sigmoid(-Lambda).   grid (D/256, nchunk, B)
-__global__ void __launch_bounds__(256, 3) scan_apply_kernel(EwArgs a) {
-    const int d = blockIdx.x * 256 + threadIdx.x, c = blockIdx.y, b = blockIdx.z;
-    if (d >= a.D) return;
-    const int T = a.T, D = a.D, h = d / a.hstride, n = d % a.hstride;   // group of heads and channel slot within it
-    const int t0 = c * CHUNK, t1 = min(T, t0 + CHUNK);
-    const float lam = a.lambda[d];
-    const float s = decay_rate(lam, a.c), ba = a.b_a[d], bx = a.b_x[d];
-    const float dsdlam_neg = a.c * sigmoid_acc(-lam);
-    float carry = a.xin[((size_t)b * a.nchunk + c) * D + d];
-    float s_lam = 0.0f, s_ba = 0.0f, s_bx = 0.0f;
-    // running pointers at token t1 - 8 (the loop walks backwards in steps of eight tokens)
-    const size_t tokb = (size_t)b * T + (t1 - 8);
-    const uint32_t sD = (uint32_t)D, sZ = (uint32_t)a.H * 2 * DH;      // token strides of [tok][D] and [tok][H][2][256] arrays; eight tokens' worth fits 32 bits
-    const __nv_bfloat16 *p_dy = a.dy + tokb * (size_t)sD + d, *p_y = a.y + (tokb - 1) * (size_t)sD + d;
-    const __half *p_z = a.z + tokb * (size_t)sZ + (size_t)h * 2 * DH + n, *p_u = a.u + tokb * (size_t)sD + d;
-    __half *p_dz = a.dz + tokb * (size_t)sZ + (size_t)h * 2 * DH + n;
-    __half *p_du = a.du + tokb * (size_t)sD + d;
-    const float h0v = a.h0 ? a.h0[(size_t)b * D + d] : 0.0f;
-    // eight tokens at the running pointers, newest first
-    auto batch8 = [&](int tb) {
-        float dza_hi = 0.0f, dzx_hi = 0.0f;
-        float dyv[8], hpv[8], zav[8], zxv[8], uv[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            dyv[k] = bf2f(p_dy[k * sD]);
-            hpv[k] = (tb + k) > 0 ? bf2f(p_y[k * sD]) : h0v;
-            zav[k] = __half2float(p_z[k * sZ]);
-            zxv[k] = __half2float(p_z[k * sZ + DH]);
-            uv[k] = __half2float(p_u[k * sD]);
-        }
-#pragma unroll
-        for (int k = 7; k >= 0; --k) {
-            const float r = sigmoid_fast(zav[k] + ba), gi = sigmoid_fast(zxv[k] + bx);
-            const float L = -s * r, at = __expf(L), m2 = one_minus_exp(2.0f * L);
-            const float rm = m2 > 0.0f ? rsqrt_fast(m2) : 0.0f, mt = m2 * rm;   // 1/sqrt(1 - a^2) and sqrt(1 - a^2) from one MUFU
-            const float g = dyv[k] + carry;
-            carry = at * g;
-            const float v = gi * uv[k];
-            const float dL = g * (at * hpv[k] - at * at * v * rm);
-            const float dv = g * mt;
-            const float dza = -s * dL * r * (1.0f - r), dzx = dv * uv[k] * gi * (1.0f - gi);
-            s_lam = fmaf(dL * r, dsdlam_neg, s_lam);
-            s_ba += dza; s_bx += dzx;
-            p_du[k * sD] = to_half_sat(dv * gi);
-            // tokens k (odd) and k - 1 share one packed conversion
-            if (k & 1) { dza_hi = dza; dzx_hi = dzx; }
-            else {
-                const uint32_t wa = pack_f16_sat(dza, dza_hi), wx = pack_f16_sat(dzx, dzx_hi);
-                p_dz[k * sZ] = __ushort_as_half((unsigned short)(wa & 0xFFFFu));
-                p_dz[(k + 1) * sZ] = __ushort_as_half((unsigned short)(wa >> 16));
-                p_dz[k * sZ + DH] = __ushort_as_half((unsigned short)(wx & 0xFFFFu));
-                p_dz[(k + 1) * sZ + DH] = __ushort_as_half((unsigned short)(wx >> 16));
-            }
-        }
-        p_dy -= 8 * (size_t)sD; p_y -= 8 * (size_t)sD; p_z -= 8 * (size_t)sZ; p_u -= 8 * (size_t)sD; p_dz -= 8 * (size_t)sZ; p_du -= 8 * (size_t)sD;
-    };
-    int tb = t1 - 8;
-    // sixteen tokens per round: the loads of the second eight are requested while the first eight are worked on
-    for (; tb - 8 >= t0; tb -= 16) {
-        batch8(tb);
-        batch8(tb - 8);
-    }
-    if (tb >= t0) batch8(tb);
-    float *pv = a.part_vec + ((size_t)b * a.nchunk + c) * 3 * D + d;
-    pv[0] = s_lam; pv[(size_t)D] = s_ba; pv[(size_t)2 * D] = s_bx;
-}
-
-// Conv1D adjoint: dx_t = sum_j w[j] du_{t+j} (t + j < T); per-chunk partial sums of dw[j] = sum_t du_t x_{t-j} and
-// db_c = sum_t du_t.  One thread per (sequence, chunk, channel) walks forward with sliding windows, so that every du and
-// every x is loaded once.  grid (D/256, nchunk, B)
-struct ConvBwdArgs {
-    int B, T, D, nchunk;
-    const __nv_bfloat16 *x, *conv_w, *cs_in;
-    const __half *du;
-    __nv_bfloat16 *dx;
-    float *part_conv;   // [B*nchunk][5][D]
-};
-
-__global__ void __launch_bounds__(256) conv_backward_kernel(ConvBwdArgs a) {
-    const int d = blockIdx.x * 256 + threadIdx.x, c = blockIdx.y, b = blockIdx.z;
-    const int T = a.T, D = a.D;
-    if (d >= D) return;
-    const int t0 = c * CHUNK, t1 = min(T, t0 + CHUNK);
-    float w[4], sw[4] = {0.f, 0.f, 0.f, 0.f}, sb = 0.0f;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] = bf2f(a.conv_w[(size_t)j * D + d]);
-    auto xat = [&](int t) -> float {
-        if (t >= 0) return bf2f(a.x[((size_t)b * T + t) * D + d]);
-        return a.cs_in ? bf2f(a.cs_in[((size_t)b * 3 + (3 + t)) * D + d]) : 0.0f;
-    };
-    auto duat = [&](int t) -> float { return t < T ? __half2float(a.du[((size_t)b * T + t) * D + d]) : 0.0f; };
-    float x1 = xat(t0 - 1), x2 = xat(t0 - 2), x3 = xat(t0 - 3);     // x_{t-1}, x_{t-2}, x_{t-3}
-    float g0 = duat(t0), g1 = duat(t0 + 1), g2 = duat(t0 + 2);     // du_t, du_{t+1}, du_{t+2}
-    const uint32_t sD = (uint32_t)D;   // token stride; eleven tokens' worth fits 32 bits
-    for (int tb = t0; tb < t1; tb += 8) {
-        float xs[8], gs[8];
-        const size_t row = ((size_t)b * T + tb) * D + d;
-        const __nv_bfloat16 *px = a.x + row;
-        const __half *pg = a.du + row;
-        __nv_bfloat16 *pdx = a.dx + row;
-        if (tb + 11 <= T) {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) { xs[k] = bf2f(px[k * sD]); gs[k] = __half2float(pg[(k + 3) * sD]); }
-        } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) { xs[k] = bf2f(px[k * sD]); gs[k] = duat(tb + k + 3); }
-        }
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const float g3 = gs[k], x0 = xs[k];
-            pdx[k * sD] = __float2bfloat16_rn(fmaf(w[3], g3, fmaf(w[2], g2, fmaf(w[1], g1, w[0] * g0))));
-            sw[0] = fmaf(g0, x0, sw[0]); sw[1] = fmaf(g0, x1, sw[1]); sw[2] = fmaf(g0, x2, sw[2]); sw[3] = fmaf(g0, x3, sw[3]);
-            sb += g0;
-            g0 = g1; g1 = g2; g2 = g3;
+            const f32x2 x0 = bf2x(xs[k]);
+            const f32x2 uv = fma2(w[3], x3, fma2(w[2], x2, fma2(w[1], x1, fma2(w[0], x0, cb))));
+            if (k < n) pu[k * sD] = pack_f16_sat(uv.x, uv.y);
             x3 = x2; x2 = x1; x1 = x0;
         }
     }
-    float *pc = a.part_conv + ((size_t)(b * a.nchunk + c) * 5) * D + d;
+}
+
+// 1 - exp(-x) for 0 <= x <= S_POLY without cancellation: x (1 - x/2 + x^2/6 - x^3/24 + x^4/120), relative truncation error < 1.5e-6
+__device__ __forceinline__ f32x2 one_minus_exp_neg2(f32x2 x) {
+    f32x2 p = fma2(x, pack2(1.0f / 120.0f, 1.0f / 120.0f), pack2(-1.0f / 24.0f, -1.0f / 24.0f));
+    p = fma2(p, x, pack2(1.0f / 6.0f, 1.0f / 6.0f));
+    p = fma2(p, x, pack2(-0.5f, -0.5f));
+    p = fma2(p, x, pack2(1.0f, 1.0f));
+    return mul2(p, x);
+}
+
+// r = sigmoid(z_a + b_a) and f = 1 - a_t of two channels; a_t = 1 - f, 1 - a_t^2 = f (2 - f)
+template <bool POLY> __device__ __forceinline__ void gate_f2(f32x2 za, f32x2 nba, f32x2 s2, f32x2 &r, f32x2 &f) {
+    const f32x2 e = fma2(za, pack2(-LOG2E, -LOG2E), nba);   // -(z + b) log2 e
+    const f32x2 q = __fadd2_rn(pack2(ex2_approx(e.x), ex2_approx(e.y)), pack2(1.0f, 1.0f));
+    r = pack2(rcp_fast(q.x), rcp_fast(q.y));
+    const f32x2 x = mul2(s2, r);
+    f = POLY ? one_minus_exp_neg2(x) : pack2(one_minus_exp(-x.x), one_minus_exp(-x.y));
+}
+
+// The reverse scan g_t = dy_t + a_{t+1} g_{t+1} and every element-wise adjoint (derived from Eq. 1-4):
+//   dL = g a (h_{t-1} - a v / m);  dv = g m;  di = dv u;  du = dv i;
+//   dr = -s dL;  dz_a = dr r (1-r);  dz_x = di i (1-i);  dLambda += dL c r sigmoid(-Lambda).
+// A block walks a column of 64 channels of one sequence backwards in chunks of 64 tokens; dy, y, u, z_a, z_x of the next chunk
+// arrive by tiled TMA while it works on this one (two stages of 40 KB, two blocks per SM).  A thread holds two adjacent channels
+// x the eight tokens of its warp's segment: fold from zero carry, segments combined through shared memory, adjoints.
+// Bound by its 16 bytes per element: z and dy are read once.  (The fold, carry and apply passes of one channel per thread that
+// it replaces: 79 + 5 + 309 us on B4 T4096 D4096.  One block per chunk with decoupled look-back for every chunk, all loads
+// straight into registers: 525 us, each block a serial chain of load, look-back and store.)
+// A column with idle SMs beside it is shared by S blocks that take its chunks round-robin: each chunk's step {Q, G} is
+// published before anyone waits, and a block forms its incoming carry from the one it reached S chunks ago and the S - 1
+// steps in between, in fixed order (run-to-run identical results).  The blocks of a column are neighbours in block order, so
+// with at most one partly dispatched column the resident ones always finish.
+struct ScanArgs {
+    alignas(64) CUtensorMap tm_dy, tm_y, tm_u;   // [B][T][D], box 64 tokens x 64 channels
+    alignas(64) CUtensorMap tm_z;                // [B][T][groups x 2 x 256], the same box
+    EwArgs e;
+    int S;          // blocks per column
+    int tiles;      // columns per group of heads
+    int cvalid;     // channel slots of a group that exist
+};
+constexpr uint32_t SCAN_TILE_BYTES = SCAN_CHUNK * 128;
+constexpr uint32_t SCAN_STAGE_BYTES = 5 * SCAN_TILE_BYTES;
+constexpr uint32_t SCAN_SMEM_ALLOC = 2 * SCAN_STAGE_BYTES + 1024;
+constexpr int SCAN_MAX_S = 16;
+constexpr int SCAN_WINDOW = 4;   // records requested at once
+
+struct ScanShared {
+    f32x2 agg[2][8][32];   // steps of the eight segments: Q, G
+    f32x2 xin[32];
+    uint64_t full[2];
+    int ok, abort;
+};
+
+template <bool POLY>
+__device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, const uint8_t *stage, uint32_t stage_addr, int b, int k0, int group, int n0, f32x2 s2) {
+    const EwArgs &a = p.e;
+    const int tid = threadIdx.x, lane = tid & 31, seg = tid >> 5;
+    const int T = a.T, D = a.D, S = p.S, n = n0 + 2 * lane, d = group * a.hstride + n;
+    const bool cv = n < p.cvalid && d < D;
+    const uint32_t sD = (uint32_t)D / 2, sZ = (uint32_t)a.H * DH;   // token strides in channel pairs
+    const f32x2 ba = cv ? ld2f(a.b_a + d) : pack2(0.f, 0.f), bx = cv ? ld2f(a.b_x + d) : pack2(0.f, 0.f);
+    const f32x2 nba = mul2(ba, pack2(-LOG2E, -LOG2E)), nbx = mul2(bx, pack2(-LOG2E, -LOG2E));
+    const f32x2 ONE = pack2(1.0f, 1.0f), TWO = pack2(2.0f, 2.0f), NEG = pack2(-1.0f, -1.0f), ns2 = mul2(s2, NEG);
+    const uint32_t full0 = smem_u32(&sh.full[0]);
+    // this block's chunks are links k0, k0 + S, ... counted from the end of the sequence
+    auto issue = [&](int link, int st) {
+        const int t0 = (a.nchunk - 1 - link) * SCAN_CHUNK, c = group * a.hstride + n0, zc = group * 2 * DH + n0;
+        const uint32_t bar = full0 + 8u * st, dst = stage_addr + st * SCAN_STAGE_BYTES;
+        mbar_expect_tx(bar, SCAN_STAGE_BYTES);
+        tma_load_3d(dst, &p.tm_z, zc, t0, b, bar);
+        tma_load_3d(dst + SCAN_TILE_BYTES, &p.tm_dy, c, t0, b, bar);
+        tma_load_3d(dst + 2 * SCAN_TILE_BYTES, &p.tm_z, zc + DH, t0, b, bar);
+        tma_load_3d(dst + 3 * SCAN_TILE_BYTES, &p.tm_u, c, t0, b, bar);
+        tma_load_3d(dst + 4 * SCAN_TILE_BYTES, &p.tm_y, c, t0 - 1, b, bar);   // h_{t-1}; the row before the sequence reads as zero
+    };
+    if (tid == 0) {
+        issue(k0, 0);
+        if (k0 + S < a.nchunk) issue(k0 + S, 1);
+    }
+    // past the last token the carry is the gradient arriving on h_T (h_T = h_{T-1}, so it enters with factor 1), else nothing
+    f32x2 X = a.dh_T && cv ? ld2f(a.dh_T + (size_t)b * D + d) : pack2(0.f, 0.f);
+    f32x2 s_lam = pack2(0.f, 0.f), s_ba = s_lam, s_bx = s_lam;
+    const uint32_t tag = S > 1 ? a.tag + *a.epoch * 0x9E3779B1u : 0u;
+    bool ok = true;
+    int it = 0;
+    for (int link = k0; link < a.nchunk; link += S, ++it) {
+        const int st = it & 1, chunk = a.nchunk - 1 - link, t0 = chunk * SCAN_CHUNK + seg * 8;
+        const int nv = T - t0;     // tokens of the segment that exist, if fewer than eight
+        ok = warp_wait(full0 + 8u * st, (it >> 1) & 1, a.spin_ns, &sh.abort);
+        const uint32_t *sm = (const uint32_t *)(stage + st * SCAN_STAGE_BYTES) + seg * 8 * 32 + lane;
+        constexpr int TW = SCAN_TILE_BYTES / 4;
+        f32x2 r[8], f[8];
+        f32x2 Q = ONE, G = pack2(0.0f, 0.0f);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) pc[(size_t)j * D] = sw[j];
-    pc[(size_t)4 * D] = sb;
+        for (int k = 7; k >= 0; --k) {
+            gate_f2<POLY>(hf2x(sm[k * 32]), nba, s2, r[k], f[k]);
+            if (k >= nv) { r[k] = pack2(0.f, 0.f); f[k] = pack2(0.f, 0.f); }   // a token that does not exist passes the carry through (its dy reads as zero)
+            const f32x2 at = fma2(f[k], NEG, ONE);
+            G = mul2(at, __fadd2_rn(bf2x(sm[TW + k * 32]), G));
+            Q = mul2(Q, at);
+        }
+        sh.agg[0][seg][lane] = Q; sh.agg[1][seg][lane] = G;
+        if (!ok) sh.abort = 1;
+        __syncthreads();
+        if (S > 1) {
+            if (seg == 0 && !sh.abort) {
+                uint4 *rec = a.rec + ((size_t)chunk * a.B + b) * D + d;
+                const size_t rstride = (size_t)a.B * D;   // the next later chunk
+                f32x2 Qt = ONE, Gt = pack2(0.0f, 0.0f);
+#pragma unroll
+                for (int k = 7; k >= 0; --k) { Gt = fma2(sh.agg[0][k][lane], Gt, sh.agg[1][k][lane]); Qt = mul2(Qt, sh.agg[0][k][lane]); }
+                if (cv) {
+                    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec), "r"(__float_as_uint(Qt.x)), "r"(tag), "r"(__float_as_uint(Gt.x)), "r"(tag) : "memory");
+                    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec + 1), "r"(__float_as_uint(Qt.y)), "r"(tag), "r"(__float_as_uint(Gt.y)), "r"(tag) : "memory");
+                }
+                for (int jb = min(link, S - 1); jb > 0 && ok; jb -= SCAN_WINDOW) {   // records jb, jb - 1, ... chunks later, farthest first
+                    uint4 w0[SCAN_WINDOW], w1[SCAN_WINDOW];
+                    uint64_t tstart = 0;
+                    for (uint32_t npoll = 0;; ++npoll) {
+                        bool ready = true;
+#pragma unroll
+                        for (int k = 0; k < SCAN_WINDOW; ++k) {
+                            if (k < jb && cv) {
+                                const uint4 *src = rec + (size_t)(jb - k) * rstride;
+                                asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w0[k].x), "=r"(w0[k].y), "=r"(w0[k].z), "=r"(w0[k].w) : "l"(src) : "memory");
+                                asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w1[k].x), "=r"(w1[k].y), "=r"(w1[k].z), "=r"(w1[k].w) : "l"(src + 1) : "memory");
+                                // 8-byte words are written atomically: a record with this launch's tag in both halves is whole
+                                ready = ready && w0[k].y == tag && w0[k].w == tag && w1[k].y == tag && w1[k].w == tag;
+                            }
+                        }
+                        if (__all_sync(0xffffffffu, ready)) break;
+                        if ((npoll & 31u) == 31u) {
+                            const uint64_t tnow = gtimer();
+                            if (tstart == 0) tstart = tnow;
+                            if (__any_sync(0xffffffffu, tnow - tstart > a.spin_ns)) { ok = false; break; }
+                        }
+                    }
+                    if (!ok) break;
+#pragma unroll
+                    for (int k = 0; k < SCAN_WINDOW; ++k)
+                        if (k < jb && cv) X = fma2(pack2(__uint_as_float(w0[k].x), __uint_as_float(w1[k].x)), X, pack2(__uint_as_float(w0[k].z), __uint_as_float(w1[k].z)));
+                }
+                sh.xin[lane] = X;
+                if (!ok) sh.abort = 1;
+            }
+            __syncthreads();
+            X = sh.xin[lane];
+        }
+        if (sh.abort) break;   // uniform: set before the barrier above
+        f32x2 carry = X;
+#pragma unroll
+        for (int k = 7; k >= 0; --k) {
+            if (k == seg) carry = X;
+            X = fma2(sh.agg[0][k][lane], X, sh.agg[1][k][lane]);
+        }
+        uint32_t *p_dz = (uint32_t *)(a.dz + ((size_t)b * T + t0) * (size_t)(2 * sZ) + (size_t)group * 2 * DH + n);
+        uint32_t *p_du = (uint32_t *)(a.du + ((size_t)b * T + t0) * D + d);
+#pragma unroll
+        for (int k = 7; k >= 0; --k) {
+            const f32x2 u = hf2x(sm[3 * TW + k * 32]);
+            f32x2 hp = bf2x(sm[4 * TW + k * 32]);
+            if (k == 0 && t0 == 0 && a.h0 && cv) hp = ld2f(a.h0 + (size_t)b * D + d);
+            const f32x2 e = fma2(hf2x(sm[2 * TW + k * 32]), pack2(-LOG2E, -LOG2E), nbx);
+            const f32x2 q = __fadd2_rn(pack2(ex2_approx(e.x), ex2_approx(e.y)), ONE);
+            const f32x2 gi = pack2(rcp_fast(q.x), rcp_fast(q.y));
+            const f32x2 at = fma2(f[k], NEG, ONE), m2 = mul2(f[k], fma2(f[k], NEG, TWO));
+            const f32x2 rm = pack2(m2.x > 0.0f ? rsqrt_fast(m2.x) : 0.0f, m2.y > 0.0f ? rsqrt_fast(m2.y) : 0.0f);   // 1 / sqrt(1 - a^2)
+            const f32x2 g = __fadd2_rn(bf2x(sm[TW + k * 32]), carry);
+            carry = mul2(at, g);
+            const f32x2 v = mul2(gi, u);
+            const f32x2 hh = fma2(mul2(at, v), mul2(rm, NEG), hp);          // h_{t-1} - a v / m
+            const f32x2 dLr = mul2(mul2(carry, hh), r[k]);                   // dL r,  dL = g a (h_{t-1} - a v / m)
+            const f32x2 du = mul2(mul2(g, mul2(m2, rm)), gi);
+            const f32x2 dza = mul2(mul2(dLr, ns2), fma2(r[k], NEG, ONE));
+            const f32x2 dzx = mul2(mul2(du, u), fma2(gi, NEG, ONE));
+            s_lam = __fadd2_rn(s_lam, dLr);
+            s_ba = __fadd2_rn(s_ba, dza); s_bx = __fadd2_rn(s_bx, dzx);      // tokens that do not exist add zeros (r = 0, u = 0)
+            if (cv && k < nv) {
+                p_du[k * sD] = pack_f16_sat(du.x, du.y);
+                p_dz[k * sZ] = pack_f16_sat(dza.x, dza.y);
+                p_dz[k * sZ + DH / 2] = pack_f16_sat(dzx.x, dzx.y);
+            }
+        }
+        __syncthreads();   // everybody has read the stage and the segments' steps
+        if (tid == 0 && link + 2 * S < a.nchunk) issue(link + 2 * S, st);
+        if (chunk == 0 && seg == 0 && cv && a.dh0) *(float2 *)(a.dh0 + (size_t)b * D + d) = X;   // a_0 g_0, the gradient of h0
+    }
+    if (sh.abort) {
+        if (tid == 0) {
+            atomicExch(a.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT);
+            const uint64_t tw = gtimer();   // let copies in flight land before shared memory is given back
+            while (gtimer() - tw < 50000ull) __nanosleep(1000);
+        }
+        __syncthreads();
+        return;
+    }
+    // sums over this block's tokens, segment by segment
+    f32x2(*sums)[8][32] = (f32x2(*)[8][32])stage;
+    sums[0][seg][lane] = s_lam; sums[1][seg][lane] = s_ba; sums[2][seg][lane] = s_bx;
+    __syncthreads();
+    if (seg < 3 && cv) {
+        f32x2 t = pack2(0.f, 0.f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t = __fadd2_rn(t, sums[seg][k][lane]);
+        if (seg == 0) {   // dL/dLambda = c r sigmoid(-Lambda)
+            const f32x2 lam = ld2f(a.lambda + d);
+            t = mul2(t, pack2(a.c * sigmoid_acc(-lam.x), a.c * sigmoid_acc(-lam.y)));
+        }
+        *(float2 *)(a.part_vec + ((size_t)(b * S + k0) * 3 + seg) * D + d) = t;
+    }
+}
+
+__global__ void __launch_bounds__(256, 2) scan_kernel(const __grid_constant__ ScanArgs p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ ScanShared sh;
+    const uint32_t raw = smem_u32(smem_raw), base = (raw + 127u) & ~127u;
+    const EwArgs &a = p.e;
+    if (threadIdx.x == 0) {
+        mbar_init(smem_u32(&sh.full[0]), 1); mbar_init(smem_u32(&sh.full[1]), 1);
+        sh.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    int bid = blockIdx.x;
+    const int k0 = bid % p.S; bid /= p.S;
+    const int tile = bid % p.tiles; bid /= p.tiles;
+    const int group = bid % a.H, b = bid / a.H;
+    const int n = tile * 64 + (threadIdx.x & 31) * 2, d = group * a.hstride + n;
+    const bool cv = n < p.cvalid && d < a.D;
+    const f32x2 lam = cv ? ld2f(a.lambda + d) : pack2(0.f, 0.f);
+    const f32x2 s2 = cv ? pack2(decay_rate(lam.x, a.c), decay_rate(lam.y, a.c)) : pack2(0.f, 0.f);
+    uint8_t *stage = smem_raw + (base - raw);
+    // uniform over the block: every warp holds the same channels
+    if (__all_sync(0xffffffffu, s2.x <= S_POLY && s2.y <= S_POLY)) scan_column<true>(p, sh, stage, base, b, k0, group, tile * 64, s2);
+    else scan_column<false>(p, sh, stage, base, b, k0, group, tile * 64, s2);
+}
+
+// Blocks per column: two blocks fit an SM; the fewest rounds of chunks over all waves, a shared column paying for its look-back
+int scan_split(int columns, int nchunk, int slots) {
+    int best = 1;
+    double best_cost = 1e30;
+    for (int S = 1; S <= SCAN_MAX_S && S <= nchunk; ++S) {
+        const double waves = (double)(((size_t)columns * S + slots - 1) / slots), rounds = (nchunk + S - 1) / S;
+        const double cost = waves * (S == 1 ? rounds : 1.2 * rounds + 1.0);
+        if (cost < best_cost) { best_cost = cost; best = S; }
+    }
+    return best;
+}
+
+// Conv1D adjoint: dx_t = sum_j w[j] du_{t+j} (t + j < T); per-chunk partial sums of dw[j] = sum_t du_t x_{t-j} and
+// db_c = sum_t du_t.  One thread per (sequence, 32 tokens, two adjacent channels) walks forward with sliding windows, so that
+// every du and every x is loaded once.  Bound by its 6 bytes per element.  grid (ceil(D/512), ceil(T/CONV_CHUNK), B)
+struct ConvBwdArgs {
+    int B, T, D;
+    const __nv_bfloat16 *x, *conv_w, *cs_in;
+    const __half *du;
+    __nv_bfloat16 *dx;
+    float *part_conv;   // [B*chunks][5][D]
+};
+
+__global__ void __launch_bounds__(256, 4) conv_backward_kernel(ConvBwdArgs a) {
+    const int d = (blockIdx.x * 256 + threadIdx.x) * 2, b = blockIdx.z;
+    const int T = a.T, D = a.D, t0 = blockIdx.y * CONV_CHUNK, t1 = min(T, t0 + CONV_CHUNK);
+    if (d >= D) return;
+    f32x2 w[4], sw[4], sb = pack2(0.f, 0.f);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) { w[j] = bf2x(*(const uint32_t *)(a.conv_w + (size_t)j * D + d)); sw[j] = pack2(0.f, 0.f); }
+    auto xat = [&](int t) -> f32x2 {
+        if (t >= 0) return bf2x(*(const uint32_t *)(a.x + ((size_t)b * T + t) * D + d));
+        return a.cs_in ? bf2x(*(const uint32_t *)(a.cs_in + ((size_t)b * 3 + (3 + t)) * D + d)) : pack2(0.f, 0.f);
+    };
+    auto duat = [&](int t) -> f32x2 { return t < T ? hf2x(*(const uint32_t *)(a.du + ((size_t)b * T + t) * D + d)) : pack2(0.f, 0.f); };
+    f32x2 x1 = xat(t0 - 1), x2 = xat(t0 - 2), x3 = xat(t0 - 3);
+    f32x2 g0 = duat(t0), g1 = duat(t0 + 1), g2 = duat(t0 + 2);
+    const uint32_t sD = (uint32_t)D / 2;
+    for (int t = t0; t < t1; t += 4) {
+        const size_t row = ((size_t)b * T + t) * D + d;
+        const uint32_t *px = (const uint32_t *)(a.x + row), *pg = (const uint32_t *)(a.du + row);
+        uint32_t *pdx = (uint32_t *)(a.dx + row);
+        const int n = t1 - t, ng = T - t - 3;
+        uint32_t xs[4], gs[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) { xs[k] = k < n ? px[k * sD] : 0u; gs[k] = k < ng ? pg[(k + 3) * sD] : 0u; }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (k < n) {
+                const f32x2 g3 = hf2x(gs[k]), x0 = bf2x(xs[k]);
+                const f32x2 o = fma2(w[3], g3, fma2(w[2], g2, fma2(w[1], g1, mul2(w[0], g0))));
+                const __nv_bfloat162 ob = __floats2bfloat162_rn(o.x, o.y);
+                pdx[k * sD] = *(const uint32_t *)&ob;
+                sw[0] = fma2(g0, x0, sw[0]); sw[1] = fma2(g0, x1, sw[1]); sw[2] = fma2(g0, x2, sw[2]); sw[3] = fma2(g0, x3, sw[3]);
+                sb = __fadd2_rn(sb, g0);
+                g0 = g1; g1 = g2; g2 = g3;
+                x3 = x2; x2 = x1; x1 = x0;
+            }
+        }
+    }
+    float *pc = a.part_conv + ((size_t)(b * gridDim.y + blockIdx.y) * 5) * D + d;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) *(float2 *)(pc + (size_t)j * D) = sw[j];
+    *(float2 *)(pc + (size_t)4 * D) = sb;
 }
 
 inline size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-unsigned gemm_grid(const GemmArgs &g) {
+int num_sms() {
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 148;
+    return nsm;
+}
+unsigned gemm_grid(const GemmArgs &g) {
+    const int nsm = num_sms();
     const int ntiles = g.nx * g.ny * g.H;
     return (unsigned)(ntiles < nsm ? ntiles : nsm);
 }
@@ -580,9 +686,9 @@ unsigned gemm_grid(const GemmArgs &g) {
 inline int groups_of_heads(int D, int H) { const int k = DH / (D / H); return (H + k - 1) / k; }
 
 struct BwdLayout {
-    size_t BT, BTp, off_u, off_z, off_dz, off_du, off_y, off_hT, off_cs, off_fold, off_xin, off_pvec, off_pconv, off_pdw,
+    size_t BT, BTp, off_u, off_z, off_dz, off_du, off_y, off_hT, off_cs, off_rec, off_pvec, off_pconv, off_pdw,
         off_wt, off_w16, off_fws, total;
-    int nchunk, S, kb_per_split;
+    int nchunk, nchunk_conv, S, kb_per_split;
 };
 
 BwdLayout bwd_layout(int B, int T, int D, int Hl) {
@@ -591,7 +697,8 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     const size_t Dg = (size_t)H * DH;         // channel slots of all groups (>= D)
     L.BT = (size_t)B * T;
     L.BTp = (L.BT + 63) & ~(size_t)63;
-    L.nchunk = (T + CHUNK - 1) / CHUNK;
+    L.nchunk = (T + SCAN_CHUNK - 1) / SCAN_CHUNK;
+    L.nchunk_conv = (T + CONV_CHUNK - 1) / CONV_CHUNK;
     const int kblocks = (int)(L.BTp / 64);
     L.S = kblocks < 8 ? kblocks : 8;
     L.kb_per_split = (kblocks + L.S - 1) / L.S;
@@ -604,10 +711,9 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     L.off_y = take(L.BT * D * 2);
     L.off_hT = take((size_t)B * D * 4);
     L.off_cs = take((size_t)B * 3 * D * 2);
-    L.off_fold = take((size_t)B * L.nchunk * D * 8);
-    L.off_xin = take((size_t)B * L.nchunk * D * 4);
-    L.off_pvec = take((size_t)B * L.nchunk * 3 * D * 4);
-    L.off_pconv = take((size_t)B * L.nchunk * 5 * D * 4);
+    L.off_rec = take((size_t)B * L.nchunk * D * sizeof(uint4) + 256);   // the records, then the launch counter
+    L.off_pvec = take((size_t)B * (L.nchunk < SCAN_MAX_S ? L.nchunk : SCAN_MAX_S) * 3 * D * 4);
+    L.off_pconv = take((size_t)B * L.nchunk_conv * 5 * D * 4);
     L.off_pdw = take((size_t)L.S * 2 * H * DH * DH * 4);
     L.off_wt = take((size_t)H * DH * 2 * DH * 2);
     L.off_w16 = take((size_t)H * DH * 2 * DH * 2);
@@ -623,7 +729,7 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
 // and only the diagonal blocks of its gradient are kept (reduce_dw_blocks_kernel).  Slots beyond k width do not exist: they
 // read neighbouring channels against zero weights and nothing of them is written to du.
 bool sm100_backward_supported(int B, int T, int D, int H, int io) {
-    if (io != RGLRU_BF16 || B <= 0 || T <= 0 || H <= 0 || D % H != 0 || T % 8 != 0) return false;
+    if (io != RGLRU_BF16 || B <= 0 || T <= 0 || H <= 0 || D % H != 0) return false;
     const int dh = D / H;
     return dh <= DH && dh % 32 == 0;
 }
@@ -669,13 +775,14 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     a.dy = (const __nv_bfloat16 *)q.dy; a.y = (const __nv_bfloat16 *)y;
     a.conv_b = fwd.conv_b; a.b_a = fwd.b_a; a.b_x = fwd.b_x; a.lambda = q.lambda; a.h0 = fwd.h0;
     a.u = u; a.dz = dz; a.z = z; a.du = du;
-    a.fold = (float2 *)(ws + L.off_fold); a.xin = (float *)(ws + L.off_xin); a.part_vec = (float *)(ws + L.off_pvec);
+    a.rec = (uint4 *)(ws + L.off_rec); a.epoch = (uint32_t *)(a.rec + (size_t)B * L.nchunk * D);
+    a.tag = next_call_tag(); a.spin_ns = g_spin_limit_ns; a.status = status; a.part_vec = (float *)(ws + L.off_pvec);
     a.dh_T = q.dh_T; a.dh0 = q.dh0;
 
     // 1. W^T for the du contraction, conv output
     convert_w_kernel<<<dim3(DH / 32, DH / 32, 2 * H), dim3(32, 8), 0, st>>>((const __nv_bfloat16 *)q.W_a, (const __nv_bfloat16 *)q.W_x, W16, WT, H, dh, q.H);
-    const dim3 grid_ew((D + 255) / 256, L.nchunk, B);
-    conv_forward_kernel<<<grid_ew, 256, 0, st>>>(a);
+    const dim3 grid_conv((D + 511) / 512, L.nchunk_conv, B);
+    conv_forward_kernel<<<grid_conv, 256, 0, st>>>(a);
 
     ReduceJobs jobs{};
     GemmArgs g{};
@@ -696,9 +803,23 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
         tc_gemm_kernel<<<gemm_grid(g), GEMM_THREADS, GEMM_SMEM_ALLOC, st>>>(g);
     }
     // 3. reverse scan and element-wise adjoints
-    scan_fold_kernel<<<grid_ew, 256, 0, st>>>(a);
-    scan_carry_kernel<<<dim3((D + 255) / 256, B), 256, 0, st>>>(a);
-    scan_apply_kernel<<<grid_ew, 256, 0, st>>>(a);
+    ScanArgs sc{};
+    sc.e = a;
+    sc.tiles = (hstride + 63) / 64; sc.cvalid = hstride;
+    sc.S = scan_split(B * H * sc.tiles, L.nchunk, 2 * num_sms());
+    {
+        const uint64_t dx[3] = {(uint64_t)D, (uint64_t)T, (uint64_t)B}, sx[2] = {(uint64_t)D * 2, (uint64_t)D * T * 2};
+        const uint64_t wz = (uint64_t)H * 2 * DH, dzm[3] = {wz, (uint64_t)T, (uint64_t)B}, szm[2] = {wz * 2, wz * T * 2};
+        const uint32_t box[3] = {64, SCAN_CHUNK, 1};
+        if (!encode_map16_3d(&sc.tm_dy, q.dy, dx, sx, box, false) || !encode_map16_3d(&sc.tm_y, y, dx, sx, box, false) ||
+            !encode_map16_3d(&sc.tm_u, u, dx, sx, box, false) || !encode_map16_3d(&sc.tm_z, z, dzm, szm, box, false))
+            return cudaErrorNotSupported;
+        static PerDeviceOptIn scan_opt_in;
+        if ((e = scan_opt_in.ensure(scan_kernel, (int)SCAN_SMEM_ALLOC)) != cudaSuccess) return e;
+    }
+    const size_t scan_blocks = (size_t)B * H * sc.tiles * sc.S;
+    if (scan_blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    scan_kernel<<<(unsigned)scan_blocks, 256, SCAN_SMEM_ALLOC, st>>>(sc);
     // 4. du += dz W
     {
         const uint64_t da[3] = {2 * DH, (uint64_t)H, BT}, sa[2] = {2 * DH * 2, (uint64_t)H * 2 * DH * 2};
@@ -732,15 +853,14 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
         }
     }
     // 6. per-channel sums, Conv1D adjoint
-    const int nparts = B * L.nchunk;
-    add_reduce_job(jobs, a.part_vec, nparts, (size_t)3 * D, q.dlambda, D, q.db_a, D, q.db_x, D);
+    add_reduce_job(jobs, a.part_vec, B * sc.S, (size_t)3 * D, q.dlambda, D, q.db_a, D, q.db_x, D);
     ConvBwdArgs cb{};
-    cb.B = B; cb.T = T; cb.D = D; cb.nchunk = L.nchunk;
+    cb.B = B; cb.T = T; cb.D = D;
     cb.x = a.x; cb.conv_w = a.conv_w; cb.cs_in = a.cs_in; cb.du = du; cb.dx = (__nv_bfloat16 *)q.dx;
     cb.part_conv = (float *)(ws + L.off_pconv);
-    conv_backward_kernel<<<grid_ew, 256, 0, st>>>(cb);
+    conv_backward_kernel<<<grid_conv, 256, 0, st>>>(cb);
     if ((e = state_conv_grads(q, RGLRU_BF16, du, true, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
-    add_reduce_job(jobs, cb.part_conv, nparts, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
+    add_reduce_job(jobs, cb.part_conv, B * L.nchunk_conv, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
     return run_reduce_jobs(jobs, st);
 }
 

@@ -46,6 +46,15 @@ def test_cuda_core_blocks_and_chunk_chain(oracle, B, T, D, H, io):
     forward_and_backward(oracle, B, T, D, H, io, GENERIC, seed=900 + T)
 
 
+@pytest.mark.parametrize("B,T,Dh,H", [
+    (2, 1, 256, 1), (1, 63, 256, 1), (2, 65, 128, 3), (1, 127, 96, 3),   # one chunk, tails, a partial last group of heads
+    (1, 1203, 160, 2),    # a column shared by many blocks (look-back over their steps), channels beyond the last 64
+    (3, 1030, 64, 5),
+])
+def test_tensor_core_backward_of_ragged_sequences(oracle, B, T, Dh, H):
+    forward_and_backward(oracle, B, T, Dh * H, H, "bf16", 0, seed=700 + T)
+
+
 @pytest.mark.parametrize("change,error", [
     (dict(h0=lambda t: t.double()), ValueError), (dict(x=lambda t: t.transpose(0, 1)), ValueError), (dict(workspace=lambda t: t[:128]), RuntimeError),
     (dict(flags=lambda v: 1 << 40), RuntimeError), (dict(conv_state_in=lambda t: t.cpu()), ValueError)])
