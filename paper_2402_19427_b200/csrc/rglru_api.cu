@@ -42,6 +42,10 @@ bool use_sm100_prefill(const rglru_shape_t *s) {
     return !(s->flags & RGLRU_FLAG_FORCE_GENERIC) && sm100_prefill_supported(s->B, s->T, s->D, s->H, s->io);
 }
 
+bool use_sm100_wide_prefill(const rglru_shape_t *s) {
+    return !(s->flags & RGLRU_FLAG_FORCE_GENERIC) && sm100_wide_prefill_supported(s->B, s->T, s->D, s->H, s->io);
+}
+
 // Two helper streams and the events that tie them to the caller's stream for rglru_prefill_host, one set per device,
 // created on first use (streams and events are not device memory).  Calls on one device are serialised by the mutex.
 struct HostPipe {
@@ -112,7 +116,9 @@ size_t rglru_workspace_bytes(const rglru_shape_t *s, int32_t op) {
     size_t body = 0;
     switch (op) {
         case RGLRU_OP_PREFILL:
-            body = use_sm100_prefill(s) ? sm100_prefill_workspace_bytes(s->B, s->T, s->D, s->H) : generic_prefill_workspace_bytes(s->B, s->D, s->io);
+            body = use_sm100_prefill(s)        ? sm100_prefill_workspace_bytes(s->B, s->T, s->D, s->H)
+                   : use_sm100_wide_prefill(s) ? sm100_wide_prefill_workspace_bytes(s->B, s->T, s->D, s->H)
+                                               : generic_prefill_workspace_bytes(s->B, s->D, s->io);
             break;
         case RGLRU_OP_DECODE: break;
         case RGLRU_OP_BACKWARD:
@@ -155,6 +161,8 @@ int32_t rglru_prefill_ex(const rglru_shape_t *s, const rglru_params_t *p, const 
     cudaError_t e;
     if (use_sm100_prefill(s))
         e = sm100_prefill(a, (char *)workspace + WS_HEADER_BYTES, workspace_bytes - WS_HEADER_BYTES, st);
+    else if (use_sm100_wide_prefill(s))
+        e = sm100_wide_prefill(a, (char *)workspace + WS_HEADER_BYTES, workspace_bytes - WS_HEADER_BYTES, st);
     else
         e = generic_prefill(a, s->io, (char *)workspace + WS_HEADER_BYTES, st);
     return e == cudaSuccess ? RGLRU_OK : RGLRU_ERR_CUDA;

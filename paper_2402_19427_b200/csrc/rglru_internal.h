@@ -93,6 +93,10 @@ cudaError_t generic_backward(const FwdArgs &fwd, BwdArgs &b, int io, void *ws_bo
 bool sm100_prefill_supported(int B, int T, int D, int H, int io);
 size_t sm100_prefill_workspace_bytes(int B, int T, int D, int H);
 cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes, cudaStream_t st);
+// the same for heads wider than 256, as separate kernels
+bool sm100_wide_prefill_supported(int B, int T, int D, int H, int io);
+size_t sm100_wide_prefill_workspace_bytes(int B, int T, int D, int H);
+cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes, cudaStream_t st);
 bool sm100_decode_supported(int B, int D, int H, int io);
 cudaError_t sm100_decode(const FwdArgs &a, cudaStream_t st);
 extern unsigned long long g_spin_limit_ns;  // every device-side wait gives up after this many nanoseconds
@@ -104,7 +108,7 @@ bool encode_bf16_map_3d(CUtensorMap *tm, const void *ptr, uint64_t d0, uint64_t 
 // The general form for any 16-bit element type: dims (innermost first), byte strides of dims 1 and 2, box extents.
 bool encode_map16_3d(CUtensorMap *tm, const void *ptr, const uint64_t dims[3], const uint64_t strides_bytes[2], const uint32_t box[3],
                      bool swizzle128);
-// ---- sm_100a backward (bf16 io, D_h a multiple of 32 up to 256): tensor-core GEMMs around element-wise scan kernels
+// ---- sm_100a backward (bf16 io, D_h a multiple of 32): tensor-core GEMMs around element-wise scan kernels
 bool sm100_backward_supported(int B, int T, int D, int H, int io);
 size_t sm100_backward_workspace_bytes(int B, int T, int D, int H);
 cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &b, const void *y_saved, void *ws_body, size_t ws_body_bytes, uint32_t *status,

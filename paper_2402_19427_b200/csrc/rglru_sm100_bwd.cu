@@ -49,24 +49,24 @@ struct GemmArgs {
     alignas(64) CUtensorMap tm_a;    // A rows (M side), K innermost
     alignas(64) CUtensorMap tm_b0;   // B rows (N side), K innermost
     alignas(64) CUtensorMap tm_b1;   // MODE_Z: the second gate's weights (grid.y selects)
-    int mode, H, D;    // H: 256-slot groups of heads
-    int hstride;       // channels from one group to the next in the layer's [.., D] arrays (k dh with k = 256 / dh heads per group)
-    int cvalid;        // channel slots of a group that exist (k dh; fewer in a partial last group)
+    int mode, H, D;    // H: groups of heads
+    int NS, NT, nt;    // channel slots of a group; they are nt column tiles of NT
+    int hstride;       // channels of a group that exist (fewer in a partial last group) = channels from one group to the next in [.., D] arrays
     int nx, ny;        // tile grid: nx x ny x H
-    int kblocks;       // 64-wide K blocks per CTA
-    int rows_valid;    // MODE_Z / MODE_DU: number of tokens; MODE_DW: 512
-    void *out;         // MODE_Z: __half z[tok][H][2][256]; MODE_DU: __half du[tok][D] (+=); MODE_DW: float part[split][2][H][256][256]
+    int kblocks;       // MODE_DW: 64-token K blocks of a split.  MODE_Z / MODE_DU: K runs over the existing 64-slot blocks of the group
+    int rows_valid;    // MODE_Z / MODE_DU: number of tokens; MODE_DW: 2 NS
+    void *out;         // MODE_Z: __half z[tok][H][2][NS]; MODE_DU: __half du[tok][D] (+=); MODE_DW: float part[split][2][H][NS][NS]
     uint32_t *status;
     unsigned long long spin_ns;
 };
 
-// C[128 x 256] = A[128 x K] B[256 x K]^T per tile; A and B tiles arrive by tiled TMA in the 128-byte-swizzled K-major
+// C[128 x NT] = A[128 x K] B[NT x K]^T per tile; A and B tiles arrive by tiled TMA in the 128-byte-swizzled K-major
 // layout, accumulate in tensor memory (fp32), and leave through the four epilogue warps.  CTAs are persistent: each
 // walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... with two accumulators, so that the epilogue of one tile overlaps
 // the loads and MMAs of the next.  Tile number -> (x, y, z) with x fastest:
-//   MODE_Z : (token tiles, 2 gates, H)   A = u[tok][h][k]        B = W_gate[h][out][k]
-//   MODE_DU: (token tiles, 1, H)         A = dz[tok][h][k=512]   B = W^T[h][in][k=512]
-//   MODE_DW: (4 row tiles, splits, H)    A = dz[tok][h][row]     B = u[tok][h][in], both MN-major, K = this split's tokens
+//   MODE_Z : (token tiles, 2 gates x nt, H)   A = u[tok][h][k]        B = W_gate[h][out][k]
+//   MODE_DU: (token tiles, nt, H)             A = dz[tok][h][k=2 NS]  B = W^T[h][in][k=2 NS]
+//   MODE_DW: (2 NS / 128, splits x nt, H)     A = dz[tok][h][row]     B = u[tok][h][in], both MN-major, K = this split's tokens
 // 32-byte accesses: one whole DRAM sector per thread and instruction where a thread owns a row (pointers 32-byte aligned)
 __device__ __forceinline__ void st_global_v8(void *ptr, const uint32_t (&r)[8]) {
     asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(ptr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]),
@@ -76,6 +76,10 @@ __device__ __forceinline__ void ld_global_v8(const void *ptr, uint32_t (&r)[8]) 
     asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
                  "=r"(r[6]), "=r"(r[7]) : "l"(ptr) : "memory");
 }
+
+// 64-slot blocks of group h that hold channels, and the number of K blocks of a tile of that group
+__device__ __forceinline__ int slot_blocks(const GemmArgs &p, int h) { return (min(p.hstride, p.D - h * p.hstride) + 63) / 64; }
+__device__ __forceinline__ int tile_kblocks(const GemmArgs &p, int h) { return p.mode == MODE_DW ? p.kblocks : (p.mode == MODE_DU ? 2 : 1) * slot_blocks(p, h); }
 
 __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_constant__ GemmArgs p) {
     extern __shared__ uint8_t smem_raw[];
@@ -112,29 +116,33 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
         // ---- TMA producer
         if (lane == 0) {
             int kbg = 0;   // K blocks issued so far, over all tiles (ring position)
+            const int ncopies = (p.NT + 63) / 64;   // MODE_DW: 64-channel copies of the B operand
+            const uint32_t tx_bytes = A_STAGE_BYTES + (p.mode == MODE_DW ? (uint32_t)ncopies * MN_BLOCK_BYTES : (uint32_t)p.NT * 128u);
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                 const int tx = tile % p.nx, ty = (tile / p.nx) % p.ny, h = tile / (p.nx * p.ny);
-                const CUtensorMap *tb = (p.mode == MODE_Z && ty == 1) ? &p.tm_b1 : &p.tm_b0;
-                for (int kb = 0; kb < p.kblocks; ++kb, ++kbg) {
+                const int col0 = (ty % p.nt) * p.NT, sel = ty / p.nt;   // sel: gate (MODE_Z), split (MODE_DW)
+                const CUtensorMap *tb = (p.mode == MODE_Z && sel == 1) ? &p.tm_b1 : &p.tm_b0;
+                const int kslots = slot_blocks(p, h), kblocks = tile_kblocks(p, h);
+                for (int kb = 0; kb < kblocks; ++kb, ++kbg) {
                     const int s = kbg % GEMM_STAGES;
                     ok = mbar_wait(BAR_EMPTY(s), ((kbg / GEMM_STAGES) & 1) ^ 1, spin, abort_flag);
                     if (!ok) break;
-                    mbar_expect_tx(BAR_FULL(s), STAGE_BYTES);
+                    mbar_expect_tx(BAR_FULL(s), tx_bytes);
                     const uint32_t a_dst = base + s * STAGE_BYTES, b_dst = a_dst + A_STAGE_BYTES;
                     if (p.mode == MODE_DW) {
                         // both operands token-major as the scan wrote them: 64 tokens (K) x 64 channels per copy, the channels
                         // innermost; tokens at or beyond B T read as zero
-                        const int k0 = (ty * p.kblocks + kb) * 64;
+                        const int k0 = (sel * p.kblocks + kb) * 64;
 #pragma unroll
                         for (int j = 0; j < 2; ++j) tma_load_3d(a_dst + j * MN_BLOCK_BYTES, &p.tm_a, tx * 128 + j * 64, h, k0, BAR_FULL(s));
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) tma_load_3d(b_dst + j * MN_BLOCK_BYTES, tb, h * p.hstride + j * 64, k0, 0, BAR_FULL(s));
+                        for (int j = 0; j < ncopies; ++j) tma_load_3d(b_dst + j * MN_BLOCK_BYTES, tb, h * p.hstride + col0 + j * 64, k0, 0, BAR_FULL(s));
                     } else {
                         // u is read out of the layer's [tok][D] array at the group's first channel (channels past the group's own
-                        // meet zero weights; past D they read as zero); dz has the groups' own [tok][group][2][256] layout
+                        // meet zero weights; past D they read as zero); dz has the groups' own [tok][group][2][NS] layout
+                        const int kc = kb < kslots ? kb * 64 : p.NS + (kb - kslots) * 64;   // MODE_DU: the second gate's slots follow the first's
                         if (p.mode == MODE_Z) tma_load_3d(a_dst, &p.tm_a, h * p.hstride + kb * 64, tx * 128, 0, BAR_FULL(s));
-                        else tma_load_3d(a_dst, &p.tm_a, kb * 64, h, tx * 128, BAR_FULL(s));
-                        tma_load_3d(b_dst, tb, kb * 64, 0, h, BAR_FULL(s));
+                        else tma_load_3d(a_dst, &p.tm_a, kc, h, tx * 128, BAR_FULL(s));
+                        tma_load_3d(b_dst, tb, kc, col0, h, BAR_FULL(s));
                     }
                 }
             }
@@ -143,13 +151,14 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
     } else if (warp == 1) {
         // ---- MMA issuer
         if (lane == 0) {
-            constexpr uint32_t idesc = make_idesc_f16(128, 256), idesc_mn = make_idesc_f16_mn(128, 256);
+            const uint32_t idesc = make_idesc_f16(128, p.NT), idesc_mn = make_idesc_f16_mn(128, p.NT);
             int kbg = 0, it = 0;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
                 const int acc = it & 1;
                 ok = mbar_wait(BAR_ACCEMPTY(acc), ((it >> 1) & 1) ^ 1, spin, abort_flag);   // epilogue of tile it - 2 done
                 if (!ok) break;
-                for (int kb = 0; kb < p.kblocks; ++kb, ++kbg) {
+                const int kblocks = tile_kblocks(p, tile / (p.nx * p.ny));
+                for (int kb = 0; kb < kblocks; ++kb, ++kbg) {
                     const int s = kbg % GEMM_STAGES;
                     ok = mbar_wait(BAR_FULL(s), (kbg / GEMM_STAGES) & 1, spin, abort_flag);
                     if (!ok) break;
@@ -178,6 +187,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
         int it = 0;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
             const int tx = tile % p.nx, ty = (tile / p.nx) % p.ny, h = tile / (p.nx * p.ny);
+            const int col0 = (ty % p.nt) * p.NT, sel = ty / p.nt;
             const int acc = it & 1;
             const int row = tx * 128 + q * 32 + lane;
             ok = warp_wait(BAR_ACCFULL(acc), (it >> 1) & 1, spin, abort_flag);
@@ -185,15 +195,15 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
             tc_fence_after();
             const uint32_t tm_lane = tmem + ((uint32_t)(q * 32) << 16) + acc * 256;
             const bool valid = row < p.rows_valid;
-            const int cv = min(p.cvalid, p.D - h * p.hstride);   // channel slots of this group that exist
+            const int cv = min(p.hstride, p.D - h * p.hstride);   // channel slots of this group that exist
 #pragma unroll 1
-            for (int c0 = 0; c0 < 256; c0 += 32) {
+            for (int c0 = 0; c0 < p.NT; c0 += 32) {
                 f32x2 v[16];
                 tmem_ld32(tm_lane + c0, v);
                 tmem_ld_wait();
                 if (!valid) continue;
                 if (p.mode == MODE_Z) {
-                    __half *dst = (__half *)p.out + (((size_t)row * p.H + h) * 2 + ty) * 256 + c0;
+                    __half *dst = (__half *)p.out + (((size_t)row * p.H + h) * 2 + sel) * p.NS + col0 + c0;
 #pragma unroll
                     for (int j8 = 0; j8 < 2; ++j8) {
                         uint32_t w[8];
@@ -203,8 +213,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                     }
                 } else if (p.mode == MODE_DU) {
                     // du is kept in fp16 like dz (bf16 failed the dx tolerance where the taps of the Conv1D adjoint cancel)
-                    if (c0 >= cv) continue;   // a slot that does not exist: nothing of du belongs to it
-                    __half *dst = (__half *)p.out + (size_t)row * p.D + h * p.hstride + c0;
+                    if (col0 + c0 >= cv) continue;   // a slot that does not exist: nothing of du belongs to it
+                    __half *dst = (__half *)p.out + (size_t)row * p.D + h * p.hstride + col0 + c0;
                     uint32_t o0[8], o1[8];
                     ld_global_v8(dst, o0);
                     ld_global_v8(dst + 16, o1);
@@ -217,8 +227,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                     st_global_v8(dst, o0);
                     st_global_v8(dst + 16, o1);
                 } else {
-                    const int g = row >> 8, o_row = row & 255;
-                    float *dst = (float *)p.out + ((((size_t)ty * 2 + g) * p.H + h) * 256 + o_row) * 256 + c0;
+                    const int g = row >= p.NS, o_row = row - g * p.NS;
+                    float *dst = (float *)p.out + ((((size_t)sel * 2 + g) * p.H + h) * p.NS + o_row) * p.NS + col0 + c0;
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         uint32_t w[8];
@@ -265,12 +275,12 @@ __device__ __forceinline__ float decay_rate(float lambda, float c) {
 
 struct EwArgs {
     int B, T, D, H, nchunk;
-    int hstride;                      // channels from one 256-slot group of heads to the next
+    int hstride, NS;                  // channels of a group of heads = channels from one group to the next; its channel slots
     float c;
     const __nv_bfloat16 *x, *conv_w, *cs_in, *dy, *y;
     const float *conv_b, *b_a, *b_x, *lambda, *h0;
     __half *u, *dz;
-    const __half *z;                  // [tok][H][2][256] before the sigmoid, without the bias
+    const __half *z;                  // [tok][H][2][NS] before the sigmoid, without the bias
     __half *du;                       // [tok][D]
     uint4 *rec;                       // [nchunk][B][D] carry records of the reverse scan
     uint32_t *epoch;                  // launch counter in the workspace (any starting value): part of the records' tag
@@ -282,37 +292,37 @@ struct EwArgs {
     float *dh0;                       // [B][D] gradient of h0, or null
 };
 
-// fp16 copies of the gate weights: W16[g][h][o][n] = W_g[h][o][n] and WT[h][n][g*256 + o] = W_g[h][o][n]
-// One block per 32 x 32 tile of one (gate, head) matrix; the transposed copy goes through shared memory so that both
-// copies are written with consecutive threads on consecutive addresses.  grid (8, 8, 2 H), block (32, 8)
-// H counts 256-slot groups; dh is the width of a head of the layer (a multiple of 32 up to 256): a group holds k = 256 / dh
-// (rounded down) heads on its diagonal -- fewer in a partial last group of a layer of Hl heads -- and every tile outside
-// those blocks is written as zeros.
-__global__ void convert_w_kernel(const __nv_bfloat16 *Wa, const __nv_bfloat16 *Wx, __half *W16, __half *WT, int H, int dh, int Hl) {
+// fp16 copies of the gate weights: W16[g][h][o][n] = W_g[h][o][n] and, unless null, WT[h][n][g*NS + o] = W_g[h][o][n]
+// One block per 32 x 32 tile of one (gate, group) matrix; the transposed copy goes through shared memory so that both
+// copies are written with consecutive threads on consecutive addresses.  grid (NS/32, NS/32, 2 H), block (32, 8)
+// H counts groups; dh is the width of a head of the layer (a multiple of 32): a group holds k heads on its diagonal -- fewer
+// in a partial last group of a layer of Hl heads -- and every tile outside those blocks is written as zeros.
+__global__ void convert_w_kernel(const __nv_bfloat16 *Wa, const __nv_bfloat16 *Wx, __half *W16, __half *WT, int H, int NS, int k, int dh, int Hl) {
     __shared__ __half tile[32][33];
     const int g = blockIdx.z / H, h = blockIdx.z % H;
     const int o0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
-    const int k = DH / dh, sub = o0 / dh;            // heads per group; head of the group that owns these output rows
+    const int sub = o0 / dh;                         // head of the group that owns these output rows
     const int heads_here = min(k, Hl - h * k);
     const bool on_diagonal = sub < heads_here && n0 / dh == sub;
     const __nv_bfloat16 *W = (g ? Wx : Wa) + ((size_t)h * k + sub) * dh * dh + (size_t)(o0 - sub * dh) * dh + (n0 - sub * dh);
-    __half *W16m = W16 + ((size_t)g * H + h) * DH * DH;
+    __half *W16m = W16 + ((size_t)g * H + h) * NS * NS;
 #pragma unroll
     for (int r = threadIdx.y; r < 32; r += 8) {
         const float v = on_diagonal ? __bfloat162float(W[(size_t)r * dh + threadIdx.x]) : 0.0f;
         const __half hv = __float2half_rn(fminf(fmaxf(v, -65504.0f), 65504.0f));
-        W16m[(size_t)(o0 + r) * DH + n0 + threadIdx.x] = hv;
+        W16m[(size_t)(o0 + r) * NS + n0 + threadIdx.x] = hv;
         tile[r][threadIdx.x] = hv;
     }
+    if (WT == nullptr) return;
     __syncthreads();
 #pragma unroll
     for (int r = threadIdx.y; r < 32; r += 8)
-        WT[((size_t)h * DH + n0 + r) * (2 * DH) + g * DH + o0 + threadIdx.x] = tile[threadIdx.x][r];
+        WT[((size_t)h * NS + n0 + r) * (2 * NS) + g * NS + o0 + threadIdx.x] = tile[threadIdx.x][r];
 }
 
-// Fixed-order sum over the token splits of the diagonal blocks of the groups' 256 x 256 weight gradients: one thread per
-// element of dW_a / dW_x [H_layer][dh][dh].  part: [S][2 gates][G groups][256][256]
-__global__ void reduce_dw_blocks_kernel(const float *part, int S, int G, int dh, int Hl, float *dWa, float *dWx) {
+// Fixed-order sum over the token splits of the diagonal blocks of the groups' weight gradients: one thread per
+// element of dW_a / dW_x [H_layer][dh][dh].  part: [S][2 gates][G groups][NS][NS]
+__global__ void reduce_dw_blocks_kernel(const float *part, int S, int G, int NS, int k, int dh, int Hl, float *dWa, float *dWx) {
     const size_t per_gate = (size_t)Hl * dh * dh;
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 2 * per_gate) return;
@@ -320,9 +330,9 @@ __global__ void reduce_dw_blocks_kernel(const float *part, int S, int G, int dh,
     size_t r = i % per_gate;
     const int n = (int)(r % dh); r /= dh;
     const int o = (int)(r % dh); r /= dh;
-    const int head = (int)r, group = head / (DH / dh), sub = head % (DH / dh);
-    const size_t src = (((size_t)gate * G + group) * DH + sub * dh + o) * DH + sub * dh + n;
-    const size_t stride = (size_t)2 * G * DH * DH;
+    const int head = (int)r, group = head / k, sub = head % k;
+    const size_t src = (((size_t)gate * G + group) * NS + sub * dh + o) * NS + sub * dh + n;
+    const size_t stride = (size_t)2 * G * NS * NS;
     float acc = 0.0f;
     for (int s = 0; s < S; ++s) acc += part[(size_t)s * stride + src];
     (gate ? dWx : dWa)[i % per_gate] = acc;
@@ -332,12 +342,20 @@ __device__ __forceinline__ f32x2 bf2x(uint32_t w) { return make_float2(__uint_as
 __device__ __forceinline__ f32x2 hf2x(uint32_t w) { return __half22float2(*(const __half2 *)&w); }
 __device__ __forceinline__ f32x2 ld2f(const float *p) { return *(const float2 *)p; }
 
-// u_t = b_c + sum_j w[j] x_{t-j}: one thread per (sequence, 32 tokens, two adjacent channels), forward in time, eight tokens'
-// loads in flight.  Bound by its 4 bytes per element.  grid (ceil(D/512), ceil(T/CONV_CHUNK), B)
-__global__ void __launch_bounds__(256, 6) conv_forward_kernel(EwArgs a) {
-    const int d = (blockIdx.x * 256 + threadIdx.x) * 2, b = blockIdx.z;
-    const int T = a.T, D = a.D, t0 = blockIdx.y * CONV_CHUNK, t1 = min(T, t0 + CONV_CHUNK);
-    // the scan's carry records are told apart from those an earlier launch with the same host tag (a graph replay) left behind
+// u_t = b_c + sum_j w[j] x_{t-j} of tokens [tb, tb + n) of sequences b0, b0 + 1, ... as u[sequence][n][D]: one thread per
+// (sequence, 32 tokens, two adjacent channels), forward in time, eight tokens' loads in flight.  Bound by its 4 bytes per
+// element.  grid (ceil(D/512), ceil(n/CONV_CHUNK), sequences)
+struct ConvArgs {
+    int T, D, b0, tb, n;
+    const __nv_bfloat16 *x, *conv_w, *cs_in;
+    const float *conv_b;
+    __half *u;
+    uint32_t *epoch;
+};
+__global__ void __launch_bounds__(256, 6) conv_forward_kernel(ConvArgs a) {
+    const int d = (blockIdx.x * 256 + threadIdx.x) * 2, b = a.b0 + blockIdx.z;
+    const int T = a.T, D = a.D, t0 = a.tb + blockIdx.y * CONV_CHUNK, t1 = min(a.tb + a.n, t0 + CONV_CHUNK);
+    // the scans' carry records are told apart from those an earlier launch with the same host tag (a graph replay) left behind
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *a.epoch += 1u;
     if (d >= D) return;
     f32x2 w[4];
@@ -350,9 +368,9 @@ __global__ void __launch_bounds__(256, 6) conv_forward_kernel(EwArgs a) {
     };
     f32x2 x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
     const uint32_t sD = (uint32_t)D / 2;   // token stride in channel pairs
+    const uint32_t *px = (const uint32_t *)(a.x + ((size_t)b * T + t0) * D + d);
+    uint32_t *pu = (uint32_t *)(a.u + ((size_t)blockIdx.z * a.n + (t0 - a.tb)) * D + d);
     for (int t = t0; t < t1; t += 8) {
-        const uint32_t *px = (const uint32_t *)(a.x + ((size_t)b * T + t) * D + d);
-        uint32_t *pu = (uint32_t *)(a.u + ((size_t)b * T + t) * D + d);
         const int n = t1 - t;
         uint32_t xs[8];
 #pragma unroll
@@ -364,6 +382,7 @@ __global__ void __launch_bounds__(256, 6) conv_forward_kernel(EwArgs a) {
             if (k < n) pu[k * sD] = pack_f16_sat(uv.x, uv.y);
             x3 = x2; x2 = x1; x1 = x0;
         }
+        px += 8 * (size_t)sD; pu += 8 * (size_t)sD;
     }
 }
 
@@ -400,11 +419,10 @@ template <bool POLY> __device__ __forceinline__ void gate_f2(f32x2 za, f32x2 nba
 // with at most one partly dispatched column the resident ones always finish.
 struct ScanArgs {
     alignas(64) CUtensorMap tm_dy, tm_y, tm_u;   // [B][T][D], box 64 tokens x 64 channels
-    alignas(64) CUtensorMap tm_z;                // [B][T][groups x 2 x 256], the same box
+    alignas(64) CUtensorMap tm_z;                // [B][T][groups x 2 x NS], the same box
     EwArgs e;
     int S;          // blocks per column
     int tiles;      // columns per group of heads
-    int cvalid;     // channel slots of a group that exist
 };
 constexpr uint32_t SCAN_TILE_BYTES = SCAN_CHUNK * 128;
 constexpr uint32_t SCAN_STAGE_BYTES = 5 * SCAN_TILE_BYTES;
@@ -414,30 +432,55 @@ constexpr int SCAN_WINDOW = 4;   // records requested at once
 
 struct ScanShared {
     f32x2 agg[2][8][32];   // steps of the eight segments: Q, G
-    f32x2 xin[32];
+    f32x2 xin[32], pin[32];
     uint64_t full[2];
-    int ok, abort;
+    int abort;
 };
+
+// The first W of `left` records of a pair of channels (two adjacent ones), `stride` apart, polled until every lane sees this
+// launch's tag in both halves of each (8-byte words are written atomically: such a record is whole).  False if the wait ran out.
+template <int W>
+__device__ __forceinline__ bool read_records(const uint4 *rec, ptrdiff_t stride, int left, bool cv, uint32_t tag, unsigned long long spin_ns, uint4 (&w0)[W], uint4 (&w1)[W]) {
+    uint64_t tstart = 0;
+    for (uint32_t npoll = 0;; ++npoll) {
+        bool ready = true;
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+            if (k < left && cv) {
+                const uint4 *src = rec + (ptrdiff_t)k * stride;
+                asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w0[k].x), "=r"(w0[k].y), "=r"(w0[k].z), "=r"(w0[k].w) : "l"(src) : "memory");
+                asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w1[k].x), "=r"(w1[k].y), "=r"(w1[k].z), "=r"(w1[k].w) : "l"(src + 1) : "memory");
+                ready = ready && w0[k].y == tag && w0[k].w == tag && w1[k].y == tag && w1[k].w == tag;
+            }
+        }
+        if (__all_sync(0xffffffffu, ready)) return true;
+        if ((npoll & 31u) == 31u) {
+            const uint64_t tnow = gtimer();
+            if (tstart == 0) tstart = tnow;
+            if (__any_sync(0xffffffffu, tnow - tstart > spin_ns)) return false;
+        }
+    }
+}
 
 template <bool POLY>
 __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, const uint8_t *stage, uint32_t stage_addr, int b, int k0, int group, int n0, f32x2 s2) {
     const EwArgs &a = p.e;
     const int tid = threadIdx.x, lane = tid & 31, seg = tid >> 5;
     const int T = a.T, D = a.D, S = p.S, n = n0 + 2 * lane, d = group * a.hstride + n;
-    const bool cv = n < p.cvalid && d < D;
-    const uint32_t sD = (uint32_t)D / 2, sZ = (uint32_t)a.H * DH;   // token strides in channel pairs
+    const bool cv = n < a.hstride && d < D;
+    const uint32_t sD = (uint32_t)D / 2, sZ = (uint32_t)a.H * a.NS;   // token strides in channel pairs
     const f32x2 ba = cv ? ld2f(a.b_a + d) : pack2(0.f, 0.f), bx = cv ? ld2f(a.b_x + d) : pack2(0.f, 0.f);
     const f32x2 nba = mul2(ba, pack2(-LOG2E, -LOG2E)), nbx = mul2(bx, pack2(-LOG2E, -LOG2E));
     const f32x2 ONE = pack2(1.0f, 1.0f), TWO = pack2(2.0f, 2.0f), NEG = pack2(-1.0f, -1.0f), ns2 = mul2(s2, NEG);
     const uint32_t full0 = smem_u32(&sh.full[0]);
     // this block's chunks are links k0, k0 + S, ... counted from the end of the sequence
     auto issue = [&](int link, int st) {
-        const int t0 = (a.nchunk - 1 - link) * SCAN_CHUNK, c = group * a.hstride + n0, zc = group * 2 * DH + n0;
+        const int t0 = (a.nchunk - 1 - link) * SCAN_CHUNK, c = group * a.hstride + n0, zc = group * 2 * a.NS + n0;
         const uint32_t bar = full0 + 8u * st, dst = stage_addr + st * SCAN_STAGE_BYTES;
         mbar_expect_tx(bar, SCAN_STAGE_BYTES);
         tma_load_3d(dst, &p.tm_z, zc, t0, b, bar);
         tma_load_3d(dst + SCAN_TILE_BYTES, &p.tm_dy, c, t0, b, bar);
-        tma_load_3d(dst + 2 * SCAN_TILE_BYTES, &p.tm_z, zc + DH, t0, b, bar);
+        tma_load_3d(dst + 2 * SCAN_TILE_BYTES, &p.tm_z, zc + a.NS, t0, b, bar);
         tma_load_3d(dst + 3 * SCAN_TILE_BYTES, &p.tm_u, c, t0, b, bar);
         tma_load_3d(dst + 4 * SCAN_TILE_BYTES, &p.tm_y, c, t0 - 1, b, bar);   // h_{t-1}; the row before the sequence reads as zero
     };
@@ -483,26 +526,7 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
                 }
                 for (int jb = min(link, S - 1); jb > 0 && ok; jb -= SCAN_WINDOW) {   // records jb, jb - 1, ... chunks later, farthest first
                     uint4 w0[SCAN_WINDOW], w1[SCAN_WINDOW];
-                    uint64_t tstart = 0;
-                    for (uint32_t npoll = 0;; ++npoll) {
-                        bool ready = true;
-#pragma unroll
-                        for (int k = 0; k < SCAN_WINDOW; ++k) {
-                            if (k < jb && cv) {
-                                const uint4 *src = rec + (size_t)(jb - k) * rstride;
-                                asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w0[k].x), "=r"(w0[k].y), "=r"(w0[k].z), "=r"(w0[k].w) : "l"(src) : "memory");
-                                asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w1[k].x), "=r"(w1[k].y), "=r"(w1[k].z), "=r"(w1[k].w) : "l"(src + 1) : "memory");
-                                // 8-byte words are written atomically: a record with this launch's tag in both halves is whole
-                                ready = ready && w0[k].y == tag && w0[k].w == tag && w1[k].y == tag && w1[k].w == tag;
-                            }
-                        }
-                        if (__all_sync(0xffffffffu, ready)) break;
-                        if ((npoll & 31u) == 31u) {
-                            const uint64_t tnow = gtimer();
-                            if (tstart == 0) tstart = tnow;
-                            if (__any_sync(0xffffffffu, tnow - tstart > a.spin_ns)) { ok = false; break; }
-                        }
-                    }
+                    ok = read_records<SCAN_WINDOW>(rec + (size_t)jb * rstride, -(ptrdiff_t)rstride, jb, cv, tag, a.spin_ns, w0, w1);
                     if (!ok) break;
 #pragma unroll
                     for (int k = 0; k < SCAN_WINDOW; ++k)
@@ -521,7 +545,7 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
             if (k == seg) carry = X;
             X = fma2(sh.agg[0][k][lane], X, sh.agg[1][k][lane]);
         }
-        uint32_t *p_dz = (uint32_t *)(a.dz + ((size_t)b * T + t0) * (size_t)(2 * sZ) + (size_t)group * 2 * DH + n);
+        uint32_t *p_dz = (uint32_t *)(a.dz + ((size_t)b * T + t0) * (size_t)(2 * sZ) + (size_t)group * 2 * a.NS + n);
         uint32_t *p_du = (uint32_t *)(a.du + ((size_t)b * T + t0) * D + d);
 #pragma unroll
         for (int k = 7; k >= 0; --k) {
@@ -543,10 +567,11 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
             const f32x2 dzx = mul2(mul2(du, u), fma2(gi, NEG, ONE));
             s_lam = __fadd2_rn(s_lam, dLr);
             s_ba = __fadd2_rn(s_ba, dza); s_bx = __fadd2_rn(s_bx, dzx);      // tokens that do not exist add zeros (r = 0, u = 0)
-            if (cv && k < nv) {
-                p_du[k * sD] = pack_f16_sat(du.x, du.y);
-                p_dz[k * sZ] = pack_f16_sat(dza.x, dza.y);
-                p_dz[k * sZ + DH / 2] = pack_f16_sat(dzx.x, dzx.y);
+            if (k < nv) {
+                if (cv) p_du[k * sD] = pack_f16_sat(du.x, du.y);
+                // slots of this 64-slot block that do not exist get zeros: the du product multiplies the whole block
+                p_dz[k * sZ] = cv ? pack_f16_sat(dza.x, dza.y) : 0u;
+                p_dz[k * sZ + a.NS / 2] = cv ? pack_f16_sat(dzx.x, dzx.y) : 0u;
             }
         }
         __syncthreads();   // everybody has read the stage and the segments' steps
@@ -594,7 +619,7 @@ __global__ void __launch_bounds__(256, 2) scan_kernel(const __grid_constant__ Sc
     const int tile = bid % p.tiles; bid /= p.tiles;
     const int group = bid % a.H, b = bid / a.H;
     const int n = tile * 64 + (threadIdx.x & 31) * 2, d = group * a.hstride + n;
-    const bool cv = n < p.cvalid && d < a.D;
+    const bool cv = n < a.hstride && d < a.D;
     const f32x2 lam = cv ? ld2f(a.lambda + d) : pack2(0.f, 0.f);
     const f32x2 s2 = cv ? pack2(decay_rate(lam.x, a.c), decay_rate(lam.y, a.c)) : pack2(0.f, 0.f);
     uint8_t *stage = smem_raw + (base - raw);
@@ -682,8 +707,24 @@ unsigned gemm_grid(const GemmArgs &g) {
     return (unsigned)(ntiles < nsm ? ntiles : nsm);
 }
 
-// 256-slot groups of k = 256 / width (rounded down) consecutive heads: the unit of the GEMMs
-inline int groups_of_heads(int D, int H) { const int k = DH / (D / H); return (H + k - 1) / k; }
+// Groups of heads, the unit of the GEMMs and of the z / dz arrays: k = 256 / width (rounded down) consecutive heads, or one head
+// wider than 256.  Its NS channel slots (the channels rounded up) are nt column tiles of NT <= 256.
+struct Groups {
+    int dh, k, G, hstride, NS, NT, nt;
+    size_t W16_bytes() const { return (size_t)2 * G * NS * NS * 2; }
+};
+Groups make_groups(int D, int H) {
+    Groups g{};
+    g.dh = D / H;
+    g.k = g.dh < DH ? DH / g.dh : 1;
+    g.G = (H + g.k - 1) / g.k;
+    g.hstride = g.k * g.dh;
+    g.nt = (g.hstride + DH - 1) / DH;
+    const int unit = g.nt % 2 ? 64 : 32;   // NS has to be a multiple of 64, the K block
+    g.NT = (((g.hstride + g.nt - 1) / g.nt + unit - 1) / unit) * unit;
+    g.NS = g.nt * g.NT;
+    return g;
+}
 
 struct BwdLayout {
     size_t BT, BTp, off_u, off_z, off_dz, off_du, off_y, off_hT, off_cs, off_rec, off_pvec, off_pconv, off_pdw,
@@ -693,8 +734,8 @@ struct BwdLayout {
 
 BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     BwdLayout L{};
-    const int H = groups_of_heads(D, Hl);   // the GEMMs work on 256-slot groups of heads
-    const size_t Dg = (size_t)H * DH;         // channel slots of all groups (>= D)
+    const Groups gr = make_groups(D, Hl);
+    const size_t Dg = (size_t)gr.G * gr.NS;   // channel slots of all groups (>= D)
     L.BT = (size_t)B * T;
     L.BTp = (L.BT + 63) & ~(size_t)63;
     L.nchunk = (T + SCAN_CHUNK - 1) / SCAN_CHUNK;
@@ -714,38 +755,267 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     L.off_rec = take((size_t)B * L.nchunk * D * sizeof(uint4) + 256);   // the records, then the launch counter
     L.off_pvec = take((size_t)B * (L.nchunk < SCAN_MAX_S ? L.nchunk : SCAN_MAX_S) * 3 * D * 4);
     L.off_pconv = take((size_t)B * L.nchunk_conv * 5 * D * 4);
-    L.off_pdw = take((size_t)L.S * 2 * H * DH * DH * 4);
-    L.off_wt = take((size_t)H * DH * 2 * DH * 2);
-    L.off_w16 = take((size_t)H * DH * 2 * DH * 2);
-    L.off_fws = take(WS_HEADER_BYTES + sm100_prefill_workspace_bytes(B, T, D, Hl));
+    L.off_pdw = take((size_t)L.S * 2 * gr.G * gr.NS * gr.NS * 4);
+    L.off_wt = take(gr.W16_bytes());
+    L.off_w16 = take(gr.W16_bytes());
+    L.off_fws = take(gr.dh <= DH ? sm100_prefill_workspace_bytes(B, T, D, Hl) : sm100_wide_prefill_workspace_bytes(B, T, D, Hl));
+    L.total = o;
+    return L;
+}
+
+GemmArgs gemm_args(const Groups &gr, int D, uint32_t *status) {
+    GemmArgs g{};
+    g.H = gr.G; g.D = D; g.NS = gr.NS; g.NT = gr.NT; g.nt = gr.nt; g.hstride = gr.hstride; g.status = status; g.spin_ns = g_spin_limit_ns;
+    return g;
+}
+cudaError_t run_gemm(const GemmArgs &g, cudaStream_t st) {
+    static PerDeviceOptIn opt_in;
+    cudaError_t e = opt_in.ensure(tc_gemm_kernel, (int)GEMM_SMEM_ALLOC);
+    if (e != cudaSuccess) return e;
+    tc_gemm_kernel<<<gemm_grid(g), GEMM_THREADS, GEMM_SMEM_ALLOC, st>>>(g);
+    return cudaGetLastError();
+}
+// z = u W^T per group and gate: u [ntok][D], z [ntok][G][2][NS]
+cudaError_t gemm_z(const Groups &gr, int D, size_t ntok, const __half *u, const __half *W16, __half *z, uint32_t *status, cudaStream_t st) {
+    GemmArgs g = gemm_args(gr, D, status);
+    const uint64_t NS = gr.NS;
+    const uint64_t da[3] = {(uint64_t)D, ntok, 1}, sa[2] = {(uint64_t)D * 2, (uint64_t)D * ntok * 2};
+    const uint32_t ba[3] = {64, 128, 1};
+    const uint64_t db[3] = {NS, NS, (uint64_t)gr.G}, sb[2] = {NS * 2, NS * NS * 2};
+    const uint32_t bb[3] = {64, (uint32_t)gr.NT, 1};
+    if (!encode_map16_3d(&g.tm_a, u, da, sa, ba, true) || !encode_map16_3d(&g.tm_b0, W16, db, sb, bb, true) ||
+        !encode_map16_3d(&g.tm_b1, W16 + (size_t)gr.G * NS * NS, db, sb, bb, true))
+        return cudaErrorNotSupported;
+    g.mode = MODE_Z; g.rows_valid = (int)ntok; g.out = z;
+    g.nx = (int)((ntok + 127) / 128); g.ny = 2 * gr.nt;
+    return run_gemm(g, st);
+}
+
+// ------------------------------------------------------------------ forward of heads wider than 256
+// The fused prefill keeps a head's weights in the tensor memory of a CTA pair, which holds 256 channels.  A wider head runs as
+// conv_forward -> z product -> the kernel below, over at most WIDE_TOKENS tokens at a time so that the workspace stays small
+// (~7 bytes per element of a pass) and z mostly in L2; the state goes from pass to pass through h_T (and a_prod).
+// Forward scan: a block walks a 64-channel column forwards in chunks of 64 tokens, u, z_a, z_x (and the gate branch) of the
+// next chunk arriving by tiled TMA meanwhile; same shape as the reverse scan.  Bound by its 8 bytes per element.
+struct WideScanArgs {
+    alignas(64) CUtensorMap tm_u, tm_z, tm_g;   // of the pass: [sequences][n][D], [sequences][n][G x 2 x NS]; the branch: [B][T][D]
+    FwdArgs f;
+    int G, hstride, NS, tiles, S, nchunk;
+    int b0, nb, tb, n;                   // sequences b0 .. b0 + nb - 1, tokens tb .. tb + n - 1
+    uint4 *rec;                          // [nchunk][nb][D] carry records
+    uint32_t *epoch;
+    uint32_t tag;
+    unsigned long long spin_ns;
+};
+constexpr uint32_t WIDE_STAGE_BYTES = 4 * SCAN_TILE_BYTES;
+constexpr uint32_t WIDE_SMEM_ALLOC = 2 * WIDE_STAGE_BYTES + 1024;
+constexpr size_t WIDE_TOKENS = 8192;
+
+template <bool POLY>
+__device__ __forceinline__ void wide_scan_column(const WideScanArgs &p, ScanShared &sh, const uint8_t *stage, uint32_t stage_addr, int bl, int k0, int group, int n0, f32x2 s2) {
+    const FwdArgs &f = p.f;
+    const int tid = threadIdx.x, lane = tid & 31, seg = tid >> 5;
+    const int T = f.T, D = f.D, S = p.S, n = n0 + 2 * lane, d = group * p.hstride + n, b = p.b0 + bl;
+    const bool cv = n < p.hstride && d < D, first = p.tb == 0, last = p.tb + p.n == T;
+    const f32x2 ba = cv ? ld2f(f.b_a + d) : pack2(0.f, 0.f), bx = cv ? ld2f(f.b_x + d) : pack2(0.f, 0.f);
+    const f32x2 nba = mul2(ba, pack2(-LOG2E, -LOG2E)), nbx = mul2(bx, pack2(-LOG2E, -LOG2E));
+    const f32x2 ONE = pack2(1.0f, 1.0f), TWO = pack2(2.0f, 2.0f), NEG = pack2(-1.0f, -1.0f);
+    const bool merged = f.gate_branch != nullptr;
+    const uint32_t full0 = smem_u32(&sh.full[0]);
+    auto issue = [&](int chunk, int st) {
+        const int t0 = chunk * SCAN_CHUNK, c = group * p.hstride + n0, zc = group * 2 * p.NS + n0;
+        const uint32_t bar = full0 + 8u * st, dst = stage_addr + st * WIDE_STAGE_BYTES;
+        mbar_expect_tx(bar, (merged ? 4 : 3) * SCAN_TILE_BYTES);
+        tma_load_3d(dst, &p.tm_z, zc, t0, bl, bar);
+        tma_load_3d(dst + SCAN_TILE_BYTES, &p.tm_z, zc + p.NS, t0, bl, bar);
+        tma_load_3d(dst + 2 * SCAN_TILE_BYTES, &p.tm_u, c, t0, bl, bar);
+        if (merged) tma_load_3d(dst + 3 * SCAN_TILE_BYTES, &p.tm_g, c, p.tb + t0, b, bar);
+    };
+    if (tid == 0) {
+        issue(k0, 0);
+        if (k0 + S < p.nchunk) issue(k0 + S, 1);
+    }
+    const float *hin = first ? f.h0 : f.h_T;
+    f32x2 X = hin && cv ? ld2f(hin + (size_t)b * D + d) : pack2(0.f, 0.f);
+    f32x2 Pc = !first && f.a_prod && cv ? ld2f(f.a_prod + (size_t)b * D + d) : ONE;   // product of a_t up to the chunk
+    // through shared memory, so that the loads above have returned before this block publishes anything: the block that reaches
+    // the end of the column overwrites h_T (and a_prod) once it has seen every other block's records
+    if (seg == 0) { sh.xin[lane] = X; sh.pin[lane] = Pc; }
+    __syncthreads();
+    X = sh.xin[lane]; Pc = sh.pin[lane];
+    const uint32_t tag = S > 1 ? p.tag + *p.epoch * 0x9E3779B1u : 0u;
+    bool ok = true;
+    int it = 0;
+    for (int chunk = k0; chunk < p.nchunk; chunk += S, ++it) {
+        const int st = it & 1, t0 = chunk * SCAN_CHUNK + seg * 8, nv = p.n - t0;
+        ok = warp_wait(full0 + 8u * st, (it >> 1) & 1, p.spin_ns, &sh.abort);
+        const uint32_t *sm = (const uint32_t *)(stage + st * WIDE_STAGE_BYTES) + seg * 8 * 32 + lane;
+        constexpr int TW = SCAN_TILE_BYTES / 4;
+        f32x2 P[8], h[8];
+        f32x2 Q = ONE, Hc = pack2(0.0f, 0.0f);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            f32x2 r, fa;
+            gate_f2<POLY>(hf2x(sm[k * 32]), nba, s2, r, fa);
+            if (k >= nv) fa = pack2(0.f, 0.f);   // a token that does not exist holds the state: a = 1, m = 0
+            const f32x2 e = fma2(hf2x(sm[TW + k * 32]), pack2(-LOG2E, -LOG2E), nbx);
+            const f32x2 q = __fadd2_rn(pack2(ex2_approx(e.x), ex2_approx(e.y)), ONE);
+            const f32x2 gi = pack2(rcp_fast(q.x), rcp_fast(q.y));
+            const f32x2 at = fma2(fa, NEG, ONE), m2 = mul2(fa, fma2(fa, NEG, TWO));
+            const f32x2 m = pack2(sqrt_approx(m2.x), sqrt_approx(m2.y));
+            Hc = fma2(at, Hc, mul2(m, mul2(gi, hf2x(sm[2 * TW + k * 32]))));
+            Q = mul2(Q, at);
+            P[k] = Q; h[k] = Hc;
+        }
+        sh.agg[0][seg][lane] = Q; sh.agg[1][seg][lane] = Hc;
+        if (!ok) sh.abort = 1;
+        __syncthreads();
+        if (S > 1) {
+            if (seg == 0 && !sh.abort) {
+                uint4 *rec = p.rec + ((size_t)chunk * p.nb + bl) * D + d;
+                const size_t rstride = (size_t)p.nb * D;
+                f32x2 Qt = ONE, Gt = pack2(0.0f, 0.0f);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) { Gt = fma2(sh.agg[0][k][lane], Gt, sh.agg[1][k][lane]); Qt = mul2(Qt, sh.agg[0][k][lane]); }
+                if (cv) {
+                    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec), "r"(__float_as_uint(Qt.x)), "r"(tag), "r"(__float_as_uint(Gt.x)), "r"(tag) : "memory");
+                    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec + 1), "r"(__float_as_uint(Qt.y)), "r"(tag), "r"(__float_as_uint(Gt.y)), "r"(tag) : "memory");
+                }
+                for (int jb = min(chunk, S - 1); jb > 0 && ok; jb -= SCAN_WINDOW) {   // records jb, jb - 1, ... chunks earlier, farthest first
+                    uint4 w0[SCAN_WINDOW], w1[SCAN_WINDOW];
+                    ok = read_records<SCAN_WINDOW>(rec - (size_t)jb * rstride, rstride, jb, cv, tag, p.spin_ns, w0, w1);
+                    if (!ok) break;
+#pragma unroll
+                    for (int k = 0; k < SCAN_WINDOW; ++k) {
+                        if (k < jb && cv) {
+                            const f32x2 q = pack2(__uint_as_float(w0[k].x), __uint_as_float(w1[k].x));
+                            X = fma2(q, X, pack2(__uint_as_float(w0[k].z), __uint_as_float(w1[k].z)));
+                            Pc = mul2(Pc, q);
+                        }
+                    }
+                }
+                sh.xin[lane] = X; sh.pin[lane] = Pc;
+                if (!ok) sh.abort = 1;
+            }
+            __syncthreads();
+            X = sh.xin[lane]; Pc = sh.pin[lane];
+        }
+        if (sh.abort) break;   // uniform: set before the barrier above
+        f32x2 carry = X;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            if (k == seg) carry = X;
+            X = fma2(sh.agg[0][k][lane], X, sh.agg[1][k][lane]);
+            Pc = mul2(Pc, sh.agg[0][k][lane]);
+        }
+        uint32_t *p_y = (uint32_t *)((__nv_bfloat16 *)f.y + ((size_t)b * T + p.tb + t0) * D + d);
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            f32x2 y = fma2(P[k], carry, h[k]);
+            if (merged) {
+                const f32x2 g = bf2x(sm[3 * TW + k * 32]);   // y_t = h_t GeLU(branch_t), GeLU(v) = v Phi(v) (Section 2.3)
+                y = mul2(y, pack2(0.5f * g.x * (1.0f + erff(g.x * 0.70710678f)), 0.5f * g.y * (1.0f + erff(g.y * 0.70710678f))));
+            }
+            if (cv && k < nv) {
+                const __nv_bfloat162 o = __floats2bfloat162_rn(y.x, y.y);
+                p_y[(size_t)k * (D / 2)] = *(const uint32_t *)&o;
+            }
+        }
+        __syncthreads();   // everybody has read the stage and the segments' steps
+        if (tid == 0 && chunk + 2 * S < p.nchunk) issue(chunk + 2 * S, st);
+        if (chunk == p.nchunk - 1 && seg == 0 && cv) {
+            *(float2 *)(f.h_T + (size_t)b * D + d) = X;
+            if (f.a_prod) *(float2 *)(f.a_prod + (size_t)b * D + d) = Pc;
+            if (last) {   // the last three raw inputs of concat(conv_state_in, x), bit-exact
+                uint32_t keep[3];
+#pragma unroll
+                for (int kk = 0; kk < 3; ++kk) {
+                    const int t = T - 3 + kk;
+                    keep[kk] = t >= 0 ? *(const uint32_t *)((const __nv_bfloat16 *)f.x + ((size_t)b * T + t) * D + d)
+                                      : (f.cs_in ? *(const uint32_t *)((const __nv_bfloat16 *)f.cs_in + ((size_t)b * 3 + (3 + t)) * D + d) : 0u);
+                }
+#pragma unroll
+                for (int kk = 0; kk < 3; ++kk) *(uint32_t *)((__nv_bfloat16 *)f.cs_out + ((size_t)b * 3 + kk) * D + d) = keep[kk];
+            }
+        }
+    }
+    if (sh.abort && tid == 0) {
+        atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT);
+        const uint64_t tw = gtimer();   // let copies in flight land before shared memory is given back
+        while (gtimer() - tw < 50000ull) __nanosleep(1000);
+    }
+    __syncthreads();
+}
+
+__global__ void __launch_bounds__(256, 2) wide_scan_kernel(const __grid_constant__ WideScanArgs p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ ScanShared sh;
+    const uint32_t raw = smem_u32(smem_raw), base = (raw + 127u) & ~127u;
+    if (threadIdx.x == 0) {
+        mbar_init(smem_u32(&sh.full[0]), 1); mbar_init(smem_u32(&sh.full[1]), 1);
+        sh.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    int bid = blockIdx.x;
+    const int k0 = bid % p.S; bid /= p.S;
+    const int tile = bid % p.tiles; bid /= p.tiles;
+    const int group = bid % p.G, bl = bid / p.G;
+    const int n = tile * 64 + (threadIdx.x & 31) * 2, d = group * p.hstride + n;
+    const bool cv = n < p.hstride && d < p.f.D;
+    const f32x2 lam = cv ? ld2f(p.f.lambda + d) : pack2(0.f, 0.f);
+    const f32x2 s2 = cv ? pack2(decay_rate(lam.x, p.f.c), decay_rate(lam.y, p.f.c)) : pack2(0.f, 0.f);
+    uint8_t *stage = smem_raw + (base - raw);
+    if (__all_sync(0xffffffffu, s2.x <= S_POLY && s2.y <= S_POLY)) wide_scan_column<true>(p, sh, stage, base, bl, k0, group, tile * 64, s2);
+    else wide_scan_column<false>(p, sh, stage, base, bl, k0, group, tile * 64, s2);
+}
+
+// Passes over the batch: whole sequences while they fit WIDE_TOKENS, else one sequence in pieces of that length
+struct WideLayout {
+    int nb, n;   // sequences and tokens of a pass, at most
+    size_t off_u, off_z, off_w16, off_rec, off_h0, total;
+};
+WideLayout wide_layout(int B, int T, int D, int H) {
+    WideLayout L{};
+    const Groups gr = make_groups(D, H);
+    L.n = (size_t)T < WIDE_TOKENS ? T : (int)WIDE_TOKENS;
+    const size_t fit = WIDE_TOKENS / L.n;
+    L.nb = (size_t)B < fit ? B : (int)fit;
+    const size_t tok = (size_t)L.nb * L.n;
+    size_t o = 0;
+    auto take = [&](size_t bytes) { const size_t at = o; o += up256(bytes); return at; };
+    L.off_u = take(tok * D * 2);
+    L.off_z = take(tok * gr.G * gr.NS * 2 * 2);
+    L.off_w16 = take(gr.W16_bytes());
+    L.off_rec = take((size_t)((L.n + SCAN_CHUNK - 1) / SCAN_CHUNK) * L.nb * D * sizeof(uint4) + 256);   // the records, then the launch counter
+    L.off_h0 = take((size_t)B * D * 4);
     L.total = o;
     return L;
 }
 
 }  // namespace
 
-// Head width: any multiple of 32 up to 256.  k = 256 / width (rounded down) consecutive heads form a group of 256 channel slots
-// whose weight matrix is block-diagonal; it is multiplied as a dense 256 x 256 matrix (convert_w_kernel writes the zeros),
-// and only the diagonal blocks of its gradient are kept (reduce_dw_blocks_kernel).  Slots beyond k width do not exist: they
-// read neighbouring channels against zero weights and nothing of them is written to du.
+// Head width: any multiple of 32.  Up to 256, k = 256 / width (rounded down) consecutive heads form a group whose weight
+// matrix is block-diagonal; it is multiplied as a dense matrix (convert_w_kernel writes the zeros), and only the diagonal blocks
+// of its gradient are kept (reduce_dw_blocks_kernel).  A wider head is a group of its own, several column tiles wide.  Slots
+// beyond the group's channels do not exist: they meet zero weights, the scan writes zeros for those that share a 64-slot block
+// with real ones, the other blocks are left out of the products, and nothing of them is written to du.
 bool sm100_backward_supported(int B, int T, int D, int H, int io) {
     if (io != RGLRU_BF16 || B <= 0 || T <= 0 || H <= 0 || D % H != 0) return false;
     const int dh = D / H;
-    return dh <= DH && dh % 32 == 0;
+    return dh <= GENERIC_MAX_DH && dh % 32 == 0;
 }
 
 size_t sm100_backward_workspace_bytes(int B, int T, int D, int H) { return bwd_layout(B, T, D, H).total; }
 
 cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, void *ws_body, size_t ws_body_bytes, uint32_t *status,
                            cudaStream_t st) {
-    const int B = q.B, T = q.T, D = q.D, dh = q.D / q.H;
-    const int H = groups_of_heads(D, q.H);   // 256-slot groups of heads: the unit of the GEMMs and of the z / dz arrays
-    const int hstride = (DH / dh) * dh;      // channels from one group to the next
+    const int B = q.B, T = q.T, D = q.D;
+    const Groups gr = make_groups(D, q.H);
+    const int H = gr.G, NS = gr.NS, hstride = gr.hstride;
     const BwdLayout L = bwd_layout(B, T, D, q.H);
     if (ws_body_bytes < L.total) return cudaErrorInvalidValue;
-    static PerDeviceOptIn opt_in;
-    cudaError_t e = opt_in.ensure(tc_gemm_kernel, (int)GEMM_SMEM_ALLOC);
-    if (e != cudaSuccess) return e;
+    cudaError_t e;
     char *ws = (char *)ws_body;
     __half *u = (__half *)(ws + L.off_u), *z = (__half *)(ws + L.off_z);
     __half *dz = (__half *)(ws + L.off_dz), *WT = (__half *)(ws + L.off_wt), *W16 = (__half *)(ws + L.off_w16);
@@ -757,20 +1027,14 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
         FwdArgs f = fwd;
         f.y = ws + L.off_y; f.h_T = (float *)(ws + L.off_hT); f.cs_out = ws + L.off_cs;
         f.status = status;
-        char *fws = ws + L.off_fws;
-        e = sm100_prefill(f, fws + WS_HEADER_BYTES, sm100_prefill_workspace_bytes(B, T, D, q.H), st);
+        void *fws = ws + L.off_fws;
+        e = gr.dh <= DH ? sm100_prefill(f, fws, sm100_prefill_workspace_bytes(B, T, D, q.H), st) : sm100_wide_prefill(f, fws, sm100_wide_prefill_workspace_bytes(B, T, D, q.H), st);
         if (e != cudaSuccess) return e;
         y = f.y;
     }
 
-    if ((size_t)H * DH != (size_t)D) {
-        // Some channel slots of the groups do not exist.  Nothing writes their dz, and although their weights are zero a NaN
-        // bit pattern left in the workspace would still poison du = dz W: clear dz once.
-        if ((e = cudaMemsetAsync(dz, 0, L.BT * (size_t)H * DH * 2 * 2, st)) != cudaSuccess) return e;
-    }
-
     EwArgs a{};
-    a.B = B; a.T = T; a.D = D; a.H = H; a.nchunk = L.nchunk; a.c = q.c; a.hstride = hstride;
+    a.B = B; a.T = T; a.D = D; a.H = H; a.nchunk = L.nchunk; a.c = q.c; a.hstride = hstride; a.NS = NS;
     a.x = (const __nv_bfloat16 *)q.x; a.conv_w = (const __nv_bfloat16 *)q.conv_w; a.cs_in = (const __nv_bfloat16 *)q.cs_in;
     a.dy = (const __nv_bfloat16 *)q.dy; a.y = (const __nv_bfloat16 *)y;
     a.conv_b = fwd.conv_b; a.b_a = fwd.b_a; a.b_x = fwd.b_x; a.lambda = q.lambda; a.h0 = fwd.h0;
@@ -780,36 +1044,24 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     a.dh_T = q.dh_T; a.dh0 = q.dh0;
 
     // 1. W^T for the du contraction, conv output
-    convert_w_kernel<<<dim3(DH / 32, DH / 32, 2 * H), dim3(32, 8), 0, st>>>((const __nv_bfloat16 *)q.W_a, (const __nv_bfloat16 *)q.W_x, W16, WT, H, dh, q.H);
+    convert_w_kernel<<<dim3(NS / 32, NS / 32, 2 * H), dim3(32, 8), 0, st>>>((const __nv_bfloat16 *)q.W_a, (const __nv_bfloat16 *)q.W_x, W16, WT, H, NS, gr.k, gr.dh, q.H);
     const dim3 grid_conv((D + 511) / 512, L.nchunk_conv, B);
-    conv_forward_kernel<<<grid_conv, 256, 0, st>>>(a);
+    conv_forward_kernel<<<grid_conv, 256, 0, st>>>(ConvArgs{T, D, 0, 0, T, a.x, a.conv_w, a.cs_in, a.conv_b, u, a.epoch});
 
     ReduceJobs jobs{};
-    GemmArgs g{};
-    g.H = H; g.D = D; g.hstride = hstride; g.cvalid = hstride; g.status = status; g.spin_ns = g_spin_limit_ns;
-    const unsigned mtiles = (unsigned)((L.BT + 127) / 128);
     const uint64_t BT = L.BT;
     // 2. z = u W^T per head and gate
-    {
-        const uint64_t da[3] = {(uint64_t)D, BT, 1}, sa[2] = {(uint64_t)D * 2, (uint64_t)D * BT * 2};   // u [tok][D]
-        const uint32_t ba[3] = {64, 128, 1};
-        const uint64_t db[3] = {DH, DH, (uint64_t)H}, sb[2] = {DH * 2, (uint64_t)DH * DH * 2};
-        const uint32_t bb[3] = {64, 256, 1};
-        if (!encode_map16_3d(&g.tm_a, u, da, sa, ba, true) || !encode_map16_3d(&g.tm_b0, W16, db, sb, bb, true) ||
-            !encode_map16_3d(&g.tm_b1, W16 + (size_t)H * DH * DH, db, sb, bb, true))
-            return cudaErrorNotSupported;
-        g.mode = MODE_Z; g.kblocks = DH / 64; g.rows_valid = (int)BT; g.out = z;
-        g.nx = (int)mtiles; g.ny = 2;
-        tc_gemm_kernel<<<gemm_grid(g), GEMM_THREADS, GEMM_SMEM_ALLOC, st>>>(g);
-    }
+    if ((e = gemm_z(gr, D, L.BT, u, W16, z, status, st)) != cudaSuccess) return e;
+    GemmArgs g = gemm_args(gr, D, status);
+    const unsigned mtiles = (unsigned)((L.BT + 127) / 128);
     // 3. reverse scan and element-wise adjoints
     ScanArgs sc{};
     sc.e = a;
-    sc.tiles = (hstride + 63) / 64; sc.cvalid = hstride;
+    sc.tiles = (hstride + 63) / 64;
     sc.S = scan_split(B * H * sc.tiles, L.nchunk, 2 * num_sms());
     {
         const uint64_t dx[3] = {(uint64_t)D, (uint64_t)T, (uint64_t)B}, sx[2] = {(uint64_t)D * 2, (uint64_t)D * T * 2};
-        const uint64_t wz = (uint64_t)H * 2 * DH, dzm[3] = {wz, (uint64_t)T, (uint64_t)B}, szm[2] = {wz * 2, wz * T * 2};
+        const uint64_t wz = (uint64_t)H * 2 * NS, dzm[3] = {wz, (uint64_t)T, (uint64_t)B}, szm[2] = {wz * 2, wz * T * 2};
         const uint32_t box[3] = {64, SCAN_CHUNK, 1};
         if (!encode_map16_3d(&sc.tm_dy, q.dy, dx, sx, box, false) || !encode_map16_3d(&sc.tm_y, y, dx, sx, box, false) ||
             !encode_map16_3d(&sc.tm_u, u, dx, sx, box, false) || !encode_map16_3d(&sc.tm_z, z, dzm, szm, box, false))
@@ -821,35 +1073,34 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     if (scan_blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
     scan_kernel<<<(unsigned)scan_blocks, 256, SCAN_SMEM_ALLOC, st>>>(sc);
     // 4. du += dz W
+    const uint64_t K2 = 2 * (uint64_t)NS, ddz[3] = {K2, (uint64_t)H, BT}, sdz[2] = {K2 * 2, (uint64_t)H * K2 * 2};   // dz [tok][group][gate, slot]
     {
-        const uint64_t da[3] = {2 * DH, (uint64_t)H, BT}, sa[2] = {2 * DH * 2, (uint64_t)H * 2 * DH * 2};
         const uint32_t ba[3] = {64, 1, 128};
-        const uint64_t db[3] = {2 * DH, DH, (uint64_t)H}, sb[2] = {2 * DH * 2, (uint64_t)DH * 2 * DH * 2};
-        const uint32_t bb[3] = {64, 256, 1};
-        if (!encode_map16_3d(&g.tm_a, dz, da, sa, ba, true) || !encode_map16_3d(&g.tm_b0, WT, db, sb, bb, true)) return cudaErrorNotSupported;
+        const uint64_t db[3] = {K2, (uint64_t)NS, (uint64_t)H}, sb[2] = {K2 * 2, (uint64_t)NS * K2 * 2};
+        const uint32_t bb[3] = {64, (uint32_t)gr.NT, 1};
+        if (!encode_map16_3d(&g.tm_a, dz, ddz, sdz, ba, true) || !encode_map16_3d(&g.tm_b0, WT, db, sb, bb, true)) return cudaErrorNotSupported;
         g.tm_b1 = g.tm_b0;
-        g.mode = MODE_DU; g.kblocks = 2 * DH / 64; g.rows_valid = (int)BT; g.out = du;
-        g.nx = (int)mtiles; g.ny = 1;
-        tc_gemm_kernel<<<gemm_grid(g), GEMM_THREADS, GEMM_SMEM_ALLOC, st>>>(g);
+        g.mode = MODE_DU; g.rows_valid = (int)BT; g.out = du;
+        g.nx = (int)mtiles; g.ny = gr.nt;
+        if ((e = run_gemm(g, st)) != cudaSuccess) return e;
     }
     // 5. dW = dz^T u, split over the tokens, then a fixed-order sum of the splits
     {
-        const uint64_t da[3] = {2 * DH, (uint64_t)H, BT}, sa[2] = {2 * DH * 2, (uint64_t)H * 2 * DH * 2};   // dz [tok][h][gate, channel]
         const uint32_t ba[3] = {64, 1, 64};
         const uint64_t db[3] = {(uint64_t)D, BT, 1}, sb[2] = {(uint64_t)D * 2, (uint64_t)D * BT * 2};         // u [tok][D]
         const uint32_t bb[3] = {64, 64, 1};
-        if (!encode_map16_3d(&g.tm_a, dz, da, sa, ba, true) || !encode_map16_3d(&g.tm_b0, u, db, sb, bb, true)) return cudaErrorNotSupported;
+        if (!encode_map16_3d(&g.tm_a, dz, ddz, sdz, ba, true) || !encode_map16_3d(&g.tm_b0, u, db, sb, bb, true)) return cudaErrorNotSupported;
         g.tm_b1 = g.tm_b0;
         float *part = (float *)(ws + L.off_pdw);
-        g.mode = MODE_DW; g.kblocks = L.kb_per_split; g.rows_valid = 2 * DH; g.out = part;
-        g.nx = 4; g.ny = L.S;
-        tc_gemm_kernel<<<gemm_grid(g), GEMM_THREADS, GEMM_SMEM_ALLOC, st>>>(g);
-        const size_t wsz = (size_t)H * DH * DH;
-        if (dh == DH) {   // one head per group: the partial sums already have the layout of dW
+        g.mode = MODE_DW; g.kblocks = L.kb_per_split; g.rows_valid = 2 * NS; g.out = part;
+        g.nx = 2 * NS / 128; g.ny = L.S * gr.nt;
+        if ((e = run_gemm(g, st)) != cudaSuccess) return e;
+        const size_t wsz = (size_t)H * NS * NS;
+        if (gr.dh == NS) {   // one head per group and every slot exists: the partial sums already have the layout of dW
             add_reduce_job(jobs, part, L.S, 2 * wsz, q.dW_a, wsz, q.dW_x, wsz, nullptr, 0);
         } else {
-            const size_t nout = (size_t)2 * q.H * dh * dh;
-            reduce_dw_blocks_kernel<<<(unsigned)((nout + 255) / 256), 256, 0, st>>>(part, L.S, H, dh, q.H, q.dW_a, q.dW_x);
+            const size_t nout = (size_t)2 * q.H * gr.dh * gr.dh;
+            reduce_dw_blocks_kernel<<<(unsigned)((nout + 255) / 256), 256, 0, st>>>(part, L.S, H, NS, gr.k, gr.dh, q.H, q.dW_a, q.dW_x);
         }
     }
     // 6. per-channel sums, Conv1D adjoint
@@ -862,6 +1113,62 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     if ((e = state_conv_grads(q, RGLRU_BF16, du, true, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
     add_reduce_job(jobs, cb.part_conv, B * L.nchunk_conv, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
     return run_reduce_jobs(jobs, st);
+}
+
+// Heads wider than 256 (a multiple of 32): see wide_scan_kernel
+bool sm100_wide_prefill_supported(int B, int T, int D, int H, int io) {
+    if (io != RGLRU_BF16 || B <= 0 || T <= 0 || H <= 0 || D % H != 0) return false;
+    const int dh = D / H;
+    return dh > DH && dh <= GENERIC_MAX_DH && dh % 32 == 0;
+}
+
+size_t sm100_wide_prefill_workspace_bytes(int B, int T, int D, int H) { return wide_layout(B, T, D, H).total; }
+
+cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes, cudaStream_t st) {
+    const int B = a.B, T = a.T, D = a.D;
+    const Groups gr = make_groups(D, a.H);
+    const WideLayout L = wide_layout(B, T, D, a.H);
+    if (ws_body_bytes < L.total) return cudaErrorInvalidValue;
+    char *ws = (char *)ws_body;
+    __half *u = (__half *)(ws + L.off_u), *z = (__half *)(ws + L.off_z), *W16 = (__half *)(ws + L.off_w16);
+    cudaError_t e;
+    WideScanArgs p{};
+    p.f = a;
+    // blocks that share a column read the incoming state at unrelated times: an in-place update works on a copy
+    const size_t hb = (size_t)B * D * sizeof(float);
+    if (a.h0 && (uintptr_t)a.h0 < (uintptr_t)a.h_T + hb && (uintptr_t)a.h_T < (uintptr_t)a.h0 + hb) {
+        if ((e = cudaMemcpyAsync(ws + L.off_h0, a.h0, hb, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+        p.f.h0 = (const float *)(ws + L.off_h0);
+    }
+    p.G = gr.G; p.hstride = gr.hstride; p.NS = gr.NS; p.tiles = (gr.hstride + 63) / 64;
+    p.rec = (uint4 *)(ws + L.off_rec);
+    p.epoch = (uint32_t *)(p.rec + (size_t)((L.n + SCAN_CHUNK - 1) / SCAN_CHUNK) * L.nb * D);
+    p.tag = next_call_tag(); p.spin_ns = g_spin_limit_ns;
+    static PerDeviceOptIn opt_in;
+    if ((e = opt_in.ensure(wide_scan_kernel, (int)WIDE_SMEM_ALLOC)) != cudaSuccess) return e;
+    const uint32_t box[3] = {64, SCAN_CHUNK, 1};
+    if (a.gate_branch) {
+        if (!encode_bf16_map_3d(&p.tm_g, a.gate_branch, (uint64_t)D, (uint64_t)T, (uint64_t)B, 64, SCAN_CHUNK, false)) return cudaErrorNotSupported;
+    }
+    convert_w_kernel<<<dim3(gr.NS / 32, gr.NS / 32, 2 * gr.G), dim3(32, 8), 0, st>>>((const __nv_bfloat16 *)a.W_a, (const __nv_bfloat16 *)a.W_x, W16, nullptr, gr.G, gr.NS, gr.k, gr.dh, a.H);
+    const int slots = 2 * num_sms();
+    for (int b0 = 0; b0 < B; b0 += L.nb) {
+        for (int tb = 0; tb < T; tb += L.n) {
+            p.b0 = b0; p.nb = B - b0 < L.nb ? B - b0 : L.nb;
+            p.tb = tb; p.n = T - tb < L.n ? T - tb : L.n;
+            p.nchunk = (p.n + SCAN_CHUNK - 1) / SCAN_CHUNK;
+            conv_forward_kernel<<<dim3((D + 511) / 512, (p.n + CONV_CHUNK - 1) / CONV_CHUNK, p.nb), 256, 0, st>>>(
+                ConvArgs{T, D, b0, tb, p.n, (const __nv_bfloat16 *)a.x, (const __nv_bfloat16 *)a.conv_w, (const __nv_bfloat16 *)a.cs_in, a.conv_b, u, p.epoch});
+            if ((e = gemm_z(gr, D, (size_t)p.nb * p.n, u, W16, z, a.status, st)) != cudaSuccess) return e;
+            const uint64_t wz = (uint64_t)gr.G * 2 * gr.NS;
+            const uint64_t du[3] = {(uint64_t)D, (uint64_t)p.n, (uint64_t)p.nb}, su[2] = {(uint64_t)D * 2, (uint64_t)D * p.n * 2};
+            const uint64_t dz[3] = {wz, (uint64_t)p.n, (uint64_t)p.nb}, sz[2] = {wz * 2, wz * p.n * 2};
+            if (!encode_map16_3d(&p.tm_u, u, du, su, box, false) || !encode_map16_3d(&p.tm_z, z, dz, sz, box, false)) return cudaErrorNotSupported;
+            p.S = scan_split(p.nb * gr.G * p.tiles, p.nchunk, slots);
+            wide_scan_kernel<<<(unsigned)(p.nb * gr.G * p.tiles * p.S), 256, WIDE_SMEM_ALLOC, st>>>(p);
+        }
+    }
+    return cudaGetLastError();
 }
 
 }  // namespace rglru

@@ -55,6 +55,29 @@ def test_tensor_core_backward_of_ragged_sequences(oracle, B, T, Dh, H):
     forward_and_backward(oracle, B, T, Dh * H, H, "bf16", 0, seed=700 + T)
 
 
+@pytest.mark.parametrize("B,T,Dh,H", [
+    (2, 77, 352, 2), (3, 1, 288, 1), (1, 64, 320, 3), (1, 200, 1024, 1),   # 2 x 192, 2 x 160 and 4 x 256 column tiles
+    (1, 515, 544, 1),      # 3 x 192; a column shared by several blocks
+    (2, 8300, 288, 1),     # more tokens than one pass of the wide forward: state carried from pass to pass
+])
+def test_tensor_core_kernels_of_heads_wider_than_256(oracle, B, T, Dh, H):
+    forward_and_backward(oracle, B, T, Dh * H, H, "bf16", 0, seed=300 + T)
+
+
+def test_wide_heads_with_gate_branch_and_decay_product(oracle):
+    import torch
+    from paper_2402_19427_b200 import binding
+    B, T, D, H = 2, 150, 704, 2
+    inp = synth.make_inputs(B, T, D, H, io="bf16", seed=41, with_state=True, with_dy=True)
+    params = binding.Params.from_numpy(inp["params"], "bf16")
+    ap = torch.empty(B, D, dtype=torch.float32, device="cuda")
+    y, hT, _ = binding.prefill(to_dev(inp["x"], "bf16"), params, h0=to_dev(inp["h0"]), gate_branch=to_dev(inp["dy"], "bf16"), a_prod=ap)
+    torch.cuda.synchronize()
+    branch = inp["dy"].astype(np.float64)
+    yr, hr, _, apr = oracle.prefill(inp["x"].astype(np.float64), f64(inp["params"]), H, h0=inp["h0"].astype(np.float64), gate_branch=branch, with_a_prod=True)
+    assert_close("y", to_np(y), yr, "bf16"); assert_close("h_T", to_np(hT), hr, "bf16"); assert_close("a_prod", to_np(ap), apr, "bf16")
+
+
 @pytest.mark.parametrize("change,error", [
     (dict(h0=lambda t: t.double()), ValueError), (dict(x=lambda t: t.transpose(0, 1)), ValueError), (dict(workspace=lambda t: t[:128]), RuntimeError),
     (dict(flags=lambda v: 1 << 40), RuntimeError), (dict(conv_state_in=lambda t: t.cpu()), ValueError)])
