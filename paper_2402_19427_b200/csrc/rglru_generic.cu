@@ -206,6 +206,7 @@ __device__ __forceinline__ void chain_put(const Chain &ch, uint4 *slot, int link
 // Against one block per (head, sequence) walking the whole of T: 4 x 1024 x 1024 (4 heads), fp32, ran at 1.8 TFLOP/s there.
 template <typename IOT, bool SAVE, int BM, bool VEC>
 __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(FwdArgs a, Chain ch, int nchunk, int ntile) {
+    ptx::dependency_wait();
     using TL = Tile<BM>;
     constexpr int TM = TL::TM, NH = TL::NH, EB = TL::BN / 8;
     __shared__ __align__(16) TL s;
@@ -279,6 +280,7 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(F
         __syncthreads();
     }
 
+    ptx::dependency_trigger();
     // ---- gates, decay, scan of this thread's TM tokens x NH channels from zero state
     const int tr = t0 + ty * TM, c0 = n0 + tx * NH, dc = d0 + c0;
     float P[TM][NH], h[TM][NH];
@@ -423,6 +425,7 @@ __device__ __forceinline__ void gate_accumulate(const IOT *__restrict__ Wa, cons
 // One decode step.  grid = (H, ceil(B / GT)); a block handles GT sequences of one head.
 template <typename IOT>
 __global__ void __launch_bounds__(NT) generic_decode_kernel(FwdArgs a) {
+    ptx::dependency_wait();
     extern __shared__ float smem[];
     const int Dh = a.D / a.H, D = a.D, B = a.B;
     const int k = blockIdx.x, b0 = blockIdx.y * GT, d0 = k * Dh, tid = threadIdx.x;
@@ -484,6 +487,7 @@ __global__ void __launch_bounds__(NT) generic_decode_kernel(FwdArgs a) {
 constexpr int RCHUNK = 64;
 template <typename IOT>
 __global__ void __launch_bounds__(NT) generic_bwd_scan_kernel(BwdArgs q, Chain ch, int nchunk, int ctiles) {
+    ptx::dependency_wait();
     __shared__ float agg_Q[8][32], agg_g[8][32], in_g[8][32], sums[3][8][32];
     __shared__ int ok_s;
     const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
@@ -528,6 +532,7 @@ __global__ void __launch_bounds__(NT) generic_bwd_scan_kernel(BwdArgs q, Chain c
     }
     __syncthreads();
     if (!ok_s) return;
+    ptx::dependency_trigger();
     float carry = in_g[seg][lane], s_lam = 0.0f, s_ba = 0.0f, s_bx = 0.0f;
 #pragma unroll
     for (int i = 7; i >= 0; --i) {
@@ -565,6 +570,7 @@ __global__ void __launch_bounds__(NT) generic_bwd_scan_kernel(BwdArgs q, Chain c
 // over the output channels of both gates.
 template <typename IOT, int BM, bool VEC>
 __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_du_kernel(BwdArgs q, int ntile) {
+    ptx::dependency_wait();
     using TL = Tile<BM>;
     constexpr int TM = TL::TM, NH = TL::NH, EA = BM / 8;
     __shared__ __align__(16) TL s;
@@ -605,6 +611,7 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_du_kernel(Bw
         if (kc + 1 < 2 * nkg) stage((kc + 1) & 1);
         __syncthreads();
     }
+    ptx::dependency_trigger();
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
         const size_t tok = tok0 + ty * TM + i;
@@ -624,6 +631,7 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_du_kernel(Bw
 // Block = (split, gate, head, BM output rows, 2 BM input columns).
 template <int BM, bool VEC>
 __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_dw_kernel(BwdArgs q, int mtile, int ntile) {
+    ptx::dependency_wait();
     using TL = Tile<BM>;
     constexpr int TM = TL::TM, NH = TL::NH;
     __shared__ __align__(16) TL s;
@@ -662,6 +670,7 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_dw_kernel(Bw
         if (kc + 1 < nk) stage((kc + 1) & 1);
         __syncthreads();
     }
+    ptx::dependency_trigger();
     const size_t wsz = (size_t)q.H * Dh * Dh;
 #pragma unroll
     for (int i = 0; i < TM; ++i) {
@@ -682,6 +691,7 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_dw_kernel(Bw
 // One thread per (b, chunk of GENERIC_BWD_CHUNK tokens, d) walks forward with sliding windows; grid = (ceil(D/NT), nchunk, B).
 template <typename IOT>
 __global__ void __launch_bounds__(NT) generic_bwd_conv_kernel(BwdArgs q) {
+    ptx::dependency_wait();
     const int d = blockIdx.x * NT + threadIdx.x, ch = blockIdx.y, b = blockIdx.z;
     if (d >= q.D) return;
     const int T = q.T, D = q.D;
@@ -720,6 +730,7 @@ __global__ void __launch_bounds__(NT) generic_bwd_conv_kernel(BwdArgs q) {
 // Gradient through the carried conv inputs and through the copies in conv_state_out.  One thread per (b, d); grid (ceil(D/NT), B).
 template <typename IOT, typename DUT>
 __global__ void __launch_bounds__(NT) state_conv_grads_kernel(BwdArgs q, const DUT *du) {
+    ptx::dependency_wait();
     const int d = blockIdx.x * NT + threadIdx.x, b = blockIdx.y;
     if (d >= q.D) return;
     const int T = q.T, D = q.D;
@@ -757,6 +768,7 @@ __global__ void __launch_bounds__(NT) state_conv_grads_kernel(BwdArgs q, const D
 // split over up to three output arrays; all jobs of a call in one launch.  A block owns 32 columns with eight slices of the
 // parts (slice k sums parts k, k + 8, ... ascending, then the slices are added in order) or, for few parts, 256 columns.
 __global__ void __launch_bounds__(256) reduce_jobs_kernel(ReduceJobs jobs) {
+    ptx::dependency_wait();
     __shared__ float part[8][32];
     int blk = blockIdx.x, j = 0;
     while (j + 1 < jobs.n && blk >= jobs.job[j].blocks) { blk -= jobs.job[j].blocks; ++j; }
@@ -828,8 +840,8 @@ cudaError_t launch_forward(const FwdArgs &a, const Chain &ch, cudaStream_t st) {
     const int Dh = a.D / a.H, nchunk = ceil_div(a.T, BM), ntile = ceil_div(Dh, BM);
     const size_t grid = (size_t)nchunk * a.B * a.H * ntile;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    if (Dh % 4 == 0) generic_forward_kernel<IOT, SAVE, BM, true><<<(unsigned)grid, MT, 0, st>>>(a, ch, nchunk, ntile);
-    else generic_forward_kernel<IOT, SAVE, BM, false><<<(unsigned)grid, MT, 0, st>>>(a, ch, nchunk, ntile);
+    if (Dh % 4 == 0) launch_dependent(generic_forward_kernel<IOT, SAVE, BM, true>, dim3((unsigned)grid), dim3(MT), 0, st, a, ch, nchunk, ntile);
+    else launch_dependent(generic_forward_kernel<IOT, SAVE, BM, false>, dim3((unsigned)grid), dim3(MT), 0, st, a, ch, nchunk, ntile);
     return cudaGetLastError();
 }
 template <typename IOT, bool SAVE>
@@ -847,16 +859,16 @@ cudaError_t launch_du(const BwdArgs &q, cudaStream_t st) {
     const int Dh = q.D / q.H, ntile = ceil_div(Dh, 2 * BM);
     const size_t grid = (size_t)ceil_div((size_t)q.B * q.T, BM) * q.H * ntile;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    if (Dh % 4 == 0) generic_bwd_du_kernel<IOT, BM, true><<<(unsigned)grid, MT, 0, st>>>(q, ntile);
-    else generic_bwd_du_kernel<IOT, BM, false><<<(unsigned)grid, MT, 0, st>>>(q, ntile);
+    if (Dh % 4 == 0) launch_dependent(generic_bwd_du_kernel<IOT, BM, true>, dim3((unsigned)grid), dim3(MT), 0, st, q, ntile);
+    else launch_dependent(generic_bwd_du_kernel<IOT, BM, false>, dim3((unsigned)grid), dim3(MT), 0, st, q, ntile);
     return cudaGetLastError();
 }
 template <int BM>
 cudaError_t launch_dw(const BwdArgs &q, cudaStream_t st) {
     const int Dh = q.D / q.H, mtile = ceil_div(Dh, BM), ntile = ceil_div(Dh, 2 * BM);
     const unsigned grid = (unsigned)((size_t)q.S * 2 * q.H * mtile * ntile);
-    if (Dh % 4 == 0) generic_bwd_dw_kernel<BM, true><<<grid, MT, 0, st>>>(q, mtile, ntile);
-    else generic_bwd_dw_kernel<BM, false><<<grid, MT, 0, st>>>(q, mtile, ntile);
+    if (Dh % 4 == 0) launch_dependent(generic_bwd_dw_kernel<BM, true>, grid, dim3(MT), 0, st, q, mtile, ntile);
+    else launch_dependent(generic_bwd_dw_kernel<BM, false>, grid, dim3(MT), 0, st, q, mtile, ntile);
     return cudaGetLastError();
 }
 }  // namespace
@@ -885,10 +897,10 @@ cudaError_t generic_decode(const FwdArgs &a, int io, cudaStream_t st) {
     cudaError_t e;
     if (io == RGLRU_F32) {
         if ((e = set_smem(generic_decode_kernel<float>, smem)) != cudaSuccess) return e;
-        generic_decode_kernel<float><<<grid, NT, smem, st>>>(a);
+        launch_dependent(generic_decode_kernel<float>, grid, dim3(NT), smem, st, a);
     } else {
         if ((e = set_smem(generic_decode_kernel<__nv_bfloat16>, smem)) != cudaSuccess) return e;
-        generic_decode_kernel<__nv_bfloat16><<<grid, NT, smem, st>>>(a);
+        launch_dependent(generic_decode_kernel<__nv_bfloat16>, grid, dim3(NT), smem, st, a);
     }
     return cudaGetLastError();
 }
@@ -896,9 +908,9 @@ cudaError_t generic_decode(const FwdArgs &a, int io, cudaStream_t st) {
 cudaError_t state_conv_grads(const BwdArgs &q, int io, const void *du, bool du_is_half, cudaStream_t st) {
     if (!q.dcs_in && !q.dcs_out) return cudaSuccess;
     dim3 grid((q.D + NT - 1) / NT, q.B);
-    if (io == RGLRU_F32) state_conv_grads_kernel<float, float><<<grid, NT, 0, st>>>(q, (const float *)du);
-    else if (du_is_half) state_conv_grads_kernel<__nv_bfloat16, __half><<<grid, NT, 0, st>>>(q, (const __half *)du);
-    else state_conv_grads_kernel<__nv_bfloat16, float><<<grid, NT, 0, st>>>(q, (const float *)du);
+    if (io == RGLRU_F32) launch_dependent(state_conv_grads_kernel<float, float>, grid, dim3(NT), 0, st, q, (const float *)du);
+    else if (du_is_half) launch_dependent(state_conv_grads_kernel<__nv_bfloat16, __half>, grid, dim3(NT), 0, st, q, (const __half *)du);
+    else launch_dependent(state_conv_grads_kernel<__nv_bfloat16, float>, grid, dim3(NT), 0, st, q, (const float *)du);
     return cudaGetLastError();
 }
 
@@ -913,7 +925,7 @@ cudaError_t run_reduce_jobs(const ReduceJobs &jobs, cudaStream_t st) {
     int blocks = 0;
     for (int i = 0; i < jobs.n; ++i) blocks += jobs.job[i].blocks;
     if (blocks == 0) return cudaSuccess;
-    reduce_jobs_kernel<<<blocks, 256, 0, st>>>(jobs);
+    launch_dependent(reduce_jobs_kernel, dim3(blocks), dim3(256), 0, st, jobs);
     return cudaGetLastError();
 }
 
@@ -955,8 +967,8 @@ cudaError_t generic_backward(const FwdArgs &fwd_in, BwdArgs &q, int io, void *ws
     const int ctiles = ceil_div(D, 32);
     const size_t g2 = (size_t)rchunks * B * ctiles;
     if (g2 > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    if (f32) generic_bwd_scan_kernel<float><<<(unsigned)g2, NT, 0, st>>>(q, chr, rchunks, ctiles);
-    else generic_bwd_scan_kernel<__nv_bfloat16><<<(unsigned)g2, NT, 0, st>>>(q, chr, rchunks, ctiles);
+    if (f32) launch_dependent(generic_bwd_scan_kernel<float>, dim3((unsigned)g2), dim3(NT), 0, st, q, chr, rchunks, ctiles);
+    else launch_dependent(generic_bwd_scan_kernel<__nv_bfloat16>, dim3((unsigned)g2), dim3(NT), 0, st, q, chr, rchunks, ctiles);
     // 3. du += W^T dz
     const size_t blocks3 = (size_t)ceil_div((size_t)B * T, 64) * H * ceil_div(Dh, 128);
     if (tile_rows(blocks3) == 64) e = f32 ? launch_du<float, 64>(q, st) : launch_du<__nv_bfloat16, 64>(q, st);
@@ -967,8 +979,8 @@ cudaError_t generic_backward(const FwdArgs &fwd_in, BwdArgs &q, int io, void *ws
     if ((e = tile_rows(blocks4) == 64 ? launch_dw<64>(q, st) : launch_dw<32>(q, st)) != cudaSuccess) return e;
     // 5. Conv1D adjoint
     dim3 g5((D + NT - 1) / NT, q.nchunk, B);
-    if (f32) generic_bwd_conv_kernel<float><<<g5, NT, 0, st>>>(q);
-    else generic_bwd_conv_kernel<__nv_bfloat16><<<g5, NT, 0, st>>>(q);
+    if (f32) launch_dependent(generic_bwd_conv_kernel<float>, g5, dim3(NT), 0, st, q);
+    else launch_dependent(generic_bwd_conv_kernel<__nv_bfloat16>, g5, dim3(NT), 0, st, q);
     if ((e = state_conv_grads(q, io, q.hp, false, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
     // 6. deterministic reductions of the partial sums
     ReduceJobs jobs{};

@@ -33,6 +33,22 @@ struct PerDeviceOptIn {
     }
 };
 
+// Launch with programmatic dependent launch: the kernel may be scheduled as CTAs of the one before it on the stream finish, does
+// its set-up (barriers, tensor memory) and then waits (dependency_wait) before it touches global memory, so that the launch
+// latency and the set-up overlap the tail of its predecessor.  A kernel lets its successor in (dependency_trigger) when its main
+// work is done, or simply by ending: triggered at the start, the successors of several small kernels came to sit beside them
+// (forward and backward of B1 T256 D256, seven launches: 81 us without, 84 us triggered at the start, 70 us at the end).
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // The first 256 bytes of every workspace hold the device-side status: word 0 carries
 // STATUS_MAGIC | code once a kernel has recorded a condition.  A word without the magic
 // (fresh, uninitialised scratch) reads as "nothing recorded".

@@ -22,8 +22,9 @@
 // dealt out whole go to the S pairs of a head tile by tile, round-robin.  The scan warp folds such a tile to the
 // aggregate (prod a_t, h_end from zero state), publishes it, and obtains its incoming state from its own previous
 // tile plus the S-1 aggregates published by the other pairs (decoupled look-back); only then does it run the scan.
-// Waits are bounded and end in RGLRU_ERR_TIMEOUT; the launch is cooperative so that all CTAs are co-resident.
-#include <cooperative_groups.h>
+// Waits are bounded and end in RGLRU_ERR_TIMEOUT.  With a time split the grid fits the SMs at once, and the pairs of a head are
+// neighbours in block order, so at most one head is partly dispatched while others still hold SMs, and those finish.
+// (A cooperative launch, which would ask for all SMs at once, measured the same but does not combine with dependent launch.)
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -190,9 +191,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 5) { tmem_alloc2(smem_u32(tmem_base_s), 512); tmem_relinquish2(); }
+    if (warp == 4 && lane == 0) { prefetch_tensormap(&p.tm_x); prefetch_tensormap(&p.tm_y); }
     tc_fence_before();
     cluster_arrive();   // the peer's barriers must exist before anything arrives on them
     cluster_wait();
+    // nothing in global memory is touched before the previous kernel of the stream is done (see launch_dependent)
+    dependency_wait();
     tc_fence_after();
     const uint32_t tmem = *tmem_base_s;
 
@@ -644,6 +648,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
         if (!ok && lane == 0) record_timeout();
     }
 
+    dependency_trigger();
     // ---- teardown: every role falls through to here, also after a timeout
     if (*abort_flag) {
         // let copies and MMAs in flight land before shared and tensor memory are given back
@@ -832,13 +837,7 @@ cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes,
         if ((e = cudaMemcpyAsync(cs_copy, a.cs_in, cs_bytes, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
         p.f.cs_in = cs_copy;
     }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(2 * G * S); cfg.blockDim = dim3(NUM_THREADS); cfg.dynamicSmemBytes = SMEM_ALLOC; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;   // pairs wait on one another's aggregates: they must all be resident
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr; cfg.numAttrs = (S > 1 && a.B % S != 0) ? 1 : 0;
-    return a.gate_branch ? cudaLaunchKernelEx(&cfg, sm100_prefill_kernel<true>, p) : cudaLaunchKernelEx(&cfg, sm100_prefill_kernel<false>, p);
+    return launch_dependent(a.gate_branch ? sm100_prefill_kernel<true> : sm100_prefill_kernel<false>, dim3(2 * G * S), dim3(NUM_THREADS), SMEM_ALLOC, st, p);
 }
 
 }  // namespace rglru

@@ -106,11 +106,13 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 1) { tmem_alloc(smem_u32(tmem_base_s), 512); tmem_relinquish(); }
+    if (warp == 0 && lane == 0) { prefetch_tensormap(&p.tm_a); prefetch_tensormap(&p.tm_b0); prefetch_tensormap(&p.tm_b1); }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_base_s;
     bool ok = true;
+    dependency_wait();
 
     if (warp == 0) {
         // ---- TMA producer
@@ -244,6 +246,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
         }
         if (!ok && lane == 0) { *abort_flag = 1; atomicExch(p.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
     }
+    dependency_trigger();
     if (*abort_flag) {   // let copies and MMAs in flight land before shared and tensor memory are given back
         const uint64_t tw = gtimer();
         while (gtimer() - tw < 50000ull) __nanosleep(1000);
@@ -299,6 +302,7 @@ struct EwArgs {
 // in a partial last group of a layer of Hl heads -- and every tile outside those blocks is written as zeros.
 __global__ void convert_w_kernel(const __nv_bfloat16 *Wa, const __nv_bfloat16 *Wx, __half *W16, __half *WT, int H, int NS, int k, int dh, int Hl) {
     __shared__ __half tile[32][33];
+    dependency_wait();
     const int g = blockIdx.z / H, h = blockIdx.z % H;
     const int o0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
     const int sub = o0 / dh;                         // head of the group that owns these output rows
@@ -323,6 +327,7 @@ __global__ void convert_w_kernel(const __nv_bfloat16 *Wa, const __nv_bfloat16 *W
 // Fixed-order sum over the token splits of the diagonal blocks of the groups' weight gradients: one thread per
 // element of dW_a / dW_x [H_layer][dh][dh].  part: [S][2 gates][G groups][NS][NS]
 __global__ void reduce_dw_blocks_kernel(const float *part, int S, int G, int NS, int k, int dh, int Hl, float *dWa, float *dWx) {
+    dependency_wait();
     const size_t per_gate = (size_t)Hl * dh * dh;
     const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= 2 * per_gate) return;
@@ -353,6 +358,7 @@ struct ConvArgs {
     uint32_t *epoch;
 };
 __global__ void __launch_bounds__(256, 6) conv_forward_kernel(ConvArgs a) {
+    dependency_wait();
     const int d = (blockIdx.x * 256 + threadIdx.x) * 2, b = a.b0 + blockIdx.z;
     const int T = a.T, D = a.D, t0 = a.tb + blockIdx.y * CONV_CHUNK, t1 = min(a.tb + a.n, t0 + CONV_CHUNK);
     // the scans' carry records are told apart from those an earlier launch with the same host tag (a graph replay) left behind
@@ -587,6 +593,7 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
         __syncthreads();
         return;
     }
+    dependency_trigger();
     // sums over this block's tokens, segment by segment
     f32x2(*sums)[8][32] = (f32x2(*)[8][32])stage;
     sums[0][seg][lane] = s_lam; sums[1][seg][lane] = s_ba; sums[2][seg][lane] = s_bx;
@@ -614,6 +621,7 @@ __global__ void __launch_bounds__(256, 2) scan_kernel(const __grid_constant__ Sc
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    dependency_wait();
     int bid = blockIdx.x;
     const int k0 = bid % p.S; bid /= p.S;
     const int tile = bid % p.tiles; bid /= p.tiles;
@@ -652,6 +660,7 @@ struct ConvBwdArgs {
 };
 
 __global__ void __launch_bounds__(256, 4) conv_backward_kernel(ConvBwdArgs a) {
+    dependency_wait();
     const int d = (blockIdx.x * 256 + threadIdx.x) * 2, b = blockIdx.z;
     const int T = a.T, D = a.D, t0 = blockIdx.y * CONV_CHUNK, t1 = min(T, t0 + CONV_CHUNK);
     if (d >= D) return;
@@ -772,8 +781,7 @@ cudaError_t run_gemm(const GemmArgs &g, cudaStream_t st) {
     static PerDeviceOptIn opt_in;
     cudaError_t e = opt_in.ensure(tc_gemm_kernel, (int)GEMM_SMEM_ALLOC);
     if (e != cudaSuccess) return e;
-    tc_gemm_kernel<<<gemm_grid(g), GEMM_THREADS, GEMM_SMEM_ALLOC, st>>>(g);
-    return cudaGetLastError();
+    return launch_dependent(tc_gemm_kernel, dim3(gemm_grid(g)), dim3(GEMM_THREADS), GEMM_SMEM_ALLOC, st, g);
 }
 // z = u W^T per group and gate: u [ntok][D], z [ntok][G][2][NS]
 cudaError_t gemm_z(const Groups &gr, int D, size_t ntok, const __half *u, const __half *W16, __half *z, uint32_t *status, cudaStream_t st) {
@@ -957,6 +965,7 @@ __global__ void __launch_bounds__(256, 2) wide_scan_kernel(const __grid_constant
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    dependency_wait();
     int bid = blockIdx.x;
     const int k0 = bid % p.S; bid /= p.S;
     const int tile = bid % p.tiles; bid /= p.tiles;
@@ -1044,9 +1053,9 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     a.dh_T = q.dh_T; a.dh0 = q.dh0;
 
     // 1. W^T for the du contraction, conv output
-    convert_w_kernel<<<dim3(NS / 32, NS / 32, 2 * H), dim3(32, 8), 0, st>>>((const __nv_bfloat16 *)q.W_a, (const __nv_bfloat16 *)q.W_x, W16, WT, H, NS, gr.k, gr.dh, q.H);
+    if ((e = launch_dependent(convert_w_kernel, dim3(NS / 32, NS / 32, 2 * H), dim3(32, 8), 0, st, (const __nv_bfloat16 *)q.W_a, (const __nv_bfloat16 *)q.W_x, W16, WT, H, NS, gr.k, gr.dh, q.H)) != cudaSuccess) return e;
     const dim3 grid_conv((D + 511) / 512, L.nchunk_conv, B);
-    conv_forward_kernel<<<grid_conv, 256, 0, st>>>(ConvArgs{T, D, 0, 0, T, a.x, a.conv_w, a.cs_in, a.conv_b, u, a.epoch});
+    if ((e = launch_dependent(conv_forward_kernel, grid_conv, dim3(256), 0, st, ConvArgs{T, D, 0, 0, T, a.x, a.conv_w, a.cs_in, a.conv_b, u, a.epoch})) != cudaSuccess) return e;
 
     ReduceJobs jobs{};
     const uint64_t BT = L.BT;
@@ -1071,7 +1080,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     }
     const size_t scan_blocks = (size_t)B * H * sc.tiles * sc.S;
     if (scan_blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    scan_kernel<<<(unsigned)scan_blocks, 256, SCAN_SMEM_ALLOC, st>>>(sc);
+    if ((e = launch_dependent(scan_kernel, dim3((unsigned)scan_blocks), dim3(256), SCAN_SMEM_ALLOC, st, sc)) != cudaSuccess) return e;
     // 4. du += dz W
     const uint64_t K2 = 2 * (uint64_t)NS, ddz[3] = {K2, (uint64_t)H, BT}, sdz[2] = {K2 * 2, (uint64_t)H * K2 * 2};   // dz [tok][group][gate, slot]
     {
@@ -1100,7 +1109,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
             add_reduce_job(jobs, part, L.S, 2 * wsz, q.dW_a, wsz, q.dW_x, wsz, nullptr, 0);
         } else {
             const size_t nout = (size_t)2 * q.H * gr.dh * gr.dh;
-            reduce_dw_blocks_kernel<<<(unsigned)((nout + 255) / 256), 256, 0, st>>>(part, L.S, H, NS, gr.k, gr.dh, q.H, q.dW_a, q.dW_x);
+            if ((e = launch_dependent(reduce_dw_blocks_kernel, dim3((unsigned)((nout + 255) / 256)), dim3(256), 0, st, part, L.S, H, NS, gr.k, gr.dh, q.H, q.dW_a, q.dW_x)) != cudaSuccess) return e;
         }
     }
     // 6. per-channel sums, Conv1D adjoint
@@ -1109,7 +1118,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     cb.B = B; cb.T = T; cb.D = D;
     cb.x = a.x; cb.conv_w = a.conv_w; cb.cs_in = a.cs_in; cb.du = du; cb.dx = (__nv_bfloat16 *)q.dx;
     cb.part_conv = (float *)(ws + L.off_pconv);
-    conv_backward_kernel<<<grid_conv, 256, 0, st>>>(cb);
+    if ((e = launch_dependent(conv_backward_kernel, grid_conv, dim3(256), 0, st, cb)) != cudaSuccess) return e;
     if ((e = state_conv_grads(q, RGLRU_BF16, du, true, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
     add_reduce_job(jobs, cb.part_conv, B * L.nchunk_conv, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
     return run_reduce_jobs(jobs, st);
@@ -1150,22 +1159,21 @@ cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_b
     if (a.gate_branch) {
         if (!encode_bf16_map_3d(&p.tm_g, a.gate_branch, (uint64_t)D, (uint64_t)T, (uint64_t)B, 64, SCAN_CHUNK, false)) return cudaErrorNotSupported;
     }
-    convert_w_kernel<<<dim3(gr.NS / 32, gr.NS / 32, 2 * gr.G), dim3(32, 8), 0, st>>>((const __nv_bfloat16 *)a.W_a, (const __nv_bfloat16 *)a.W_x, W16, nullptr, gr.G, gr.NS, gr.k, gr.dh, a.H);
+    if ((e = launch_dependent(convert_w_kernel, dim3(gr.NS / 32, gr.NS / 32, 2 * gr.G), dim3(32, 8), 0, st, (const __nv_bfloat16 *)a.W_a, (const __nv_bfloat16 *)a.W_x, W16, (__half *)nullptr, gr.G, gr.NS, gr.k, gr.dh, a.H)) != cudaSuccess) return e;
     const int slots = 2 * num_sms();
     for (int b0 = 0; b0 < B; b0 += L.nb) {
         for (int tb = 0; tb < T; tb += L.n) {
             p.b0 = b0; p.nb = B - b0 < L.nb ? B - b0 : L.nb;
             p.tb = tb; p.n = T - tb < L.n ? T - tb : L.n;
             p.nchunk = (p.n + SCAN_CHUNK - 1) / SCAN_CHUNK;
-            conv_forward_kernel<<<dim3((D + 511) / 512, (p.n + CONV_CHUNK - 1) / CONV_CHUNK, p.nb), 256, 0, st>>>(
-                ConvArgs{T, D, b0, tb, p.n, (const __nv_bfloat16 *)a.x, (const __nv_bfloat16 *)a.conv_w, (const __nv_bfloat16 *)a.cs_in, a.conv_b, u, p.epoch});
+            if ((e = launch_dependent(conv_forward_kernel, dim3((D + 511) / 512, (p.n + CONV_CHUNK - 1) / CONV_CHUNK, p.nb), dim3(256), 0, st, ConvArgs{T, D, b0, tb, p.n, (const __nv_bfloat16 *)a.x, (const __nv_bfloat16 *)a.conv_w, (const __nv_bfloat16 *)a.cs_in, a.conv_b, u, p.epoch})) != cudaSuccess) return e;
             if ((e = gemm_z(gr, D, (size_t)p.nb * p.n, u, W16, z, a.status, st)) != cudaSuccess) return e;
             const uint64_t wz = (uint64_t)gr.G * 2 * gr.NS;
             const uint64_t du[3] = {(uint64_t)D, (uint64_t)p.n, (uint64_t)p.nb}, su[2] = {(uint64_t)D * 2, (uint64_t)D * p.n * 2};
             const uint64_t dz[3] = {wz, (uint64_t)p.n, (uint64_t)p.nb}, sz[2] = {wz * 2, wz * p.n * 2};
             if (!encode_map16_3d(&p.tm_u, u, du, su, box, false) || !encode_map16_3d(&p.tm_z, z, dz, sz, box, false)) return cudaErrorNotSupported;
             p.S = scan_split(p.nb * gr.G * p.tiles, p.nchunk, slots);
-            wide_scan_kernel<<<(unsigned)(p.nb * gr.G * p.tiles * p.S), 256, WIDE_SMEM_ALLOC, st>>>(p);
+            if ((e = launch_dependent(wide_scan_kernel, dim3((unsigned)(p.nb * gr.G * p.tiles * p.S)), dim3(256), WIDE_SMEM_ALLOC, st, p)) != cudaSuccess) return e;
         }
     }
     return cudaGetLastError();

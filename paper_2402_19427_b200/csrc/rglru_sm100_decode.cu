@@ -90,7 +90,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) sm100_d
     // Programmatic dependent launch: the next kernel on the stream (typically the next decode step) may be scheduled
     // as SMs free up, and runs its own prologue -- barrier set-up, tensor-memory allocation, the weight copies, the
     // conv taps -- while this step is still finishing; it touches x, h and the conv state only after griddepcontrol.wait.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    dependency_trigger();
     if (tid == 0) {
         mbar_init(BAR_W, 1);
         mbar_init(BAR_ACC, 1);
@@ -199,7 +199,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) sm100_d
         const uint32_t chunk = (uint32_t)(cdl & 63) >> 3;
         // everything above reads only parameters; x and the state may have been written by the kernel just before this
         // one on the stream, whose completion (and visibility of its stores) is awaited here
-        asm volatile("griddepcontrol.wait;" ::: "memory");
+        dependency_wait();
         // all global loads of the phase are issued before anything waits on them
         constexpr int NIT = NB_MAX / 32;
         uint4 xv[NIT], r0[NIT], r1[NIT], r2[NIT];   // x_t and x_{t-3}, x_{t-2}, x_{t-1} per sequence
@@ -408,14 +408,7 @@ cudaError_t sm100_decode(const FwdArgs &a, cudaStream_t st) {
     p.NB = NB;
     p.ntile = (a.B + NB - 1) / NB;
     p.spin_ns = g_spin_limit_ns;
-    dim3 grid(2u * (unsigned)G * (unsigned)p.ntile), block(NTHREADS);
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = SMEM_ALLOC; cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;   // see griddepcontrol in the kernel
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, sm100_decode_kernel, p);
+    return launch_dependent(sm100_decode_kernel, dim3(2u * (unsigned)G * (unsigned)p.ntile), dim3(NTHREADS), SMEM_ALLOC, st, p);   // see griddepcontrol in the kernel
 }
 
 }  // namespace rglru

@@ -126,6 +126,9 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
     asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
 }
+// Programmatic dependent launch (see launch_dependent): let the next kernel of the stream be scheduled; wait for the previous one
+__device__ __forceinline__ void dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 // Two fp32 values in an aligned register pair; arithmetic through the packed-fp32 builtins (fma.rn.f32x2 and friends).
 typedef float2 f32x2;
 // D[tmem] (+)= A[smem] * B[smem]^T, kind::f16 (A and B of one 16-bit type, fp32 accumulate), one CTA
@@ -186,6 +189,8 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst_smem, const CUtensorMap
     asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
                  ::"r"(dst_smem), "l"(tm), "r"(c0), "r"(t), "r"(b), "r"(bar) : "memory");
 }
+// the descriptor of a tiled copy on its way to the descriptor cache (its fetch is the longest part of a first copy)
+__device__ __forceinline__ void prefetch_tensormap(const CUtensorMap *tm) { asm volatile("prefetch.tensormap [%0];" ::"l"(tm) : "memory"); }
 // one tiled TMA store; rows at or beyond T are clipped by the tensor bounds
 __device__ __forceinline__ void tma_store_3d(const CUtensorMap *tm, int c0, int t, int b, uint32_t src_smem) {
     asm volatile("cp.async.bulk.tensor.3d.global.shared::cta.tile.bulk_group [%0, {%1, %2, %3}], [%4];"
