@@ -47,7 +47,8 @@ constexpr int HALF = 32;           // tokens of a tile one CTA convolves (one TM
 constexpr int SLAB_ROWS = HALF + 3;
 constexpr int XS = 4;              // x slab ring depth
 constexpr int US = 6;              // U tile stages
-constexpr int NUM_THREADS = 640;
+constexpr int NUM_THREADS = 640;          // 20 warps; the merged forward has four scan warps more
+constexpr int MERGED_THREADS = 768;
 constexpr int MAX_S = 16;          // at most this many pairs share one head's time axis
 constexpr int LOOKBACK_BATCH = 8;  // carry records requested at once by the look-back
 constexpr uint32_t U_STAGE_BYTES = HALF * DH * 2;          // 16384
@@ -60,7 +61,7 @@ constexpr uint32_t Y_BUF_BYTES = TILE * 32 * 2;            // 4096: one scan war
 constexpr uint32_t SMEM_Y = SMEM_X + XS * X_SLAB_BYTES;    // bf16 y_s[4 warps][2 buffers][64][32], staged for tiled stores
 constexpr uint32_t SMEM_AGG = SMEM_Y + 4 * 2 * Y_BUF_BYTES;   // float2 agg_s[2 buffers][2 half tiles][128 channels]
 constexpr uint32_t SMEM_BAR = SMEM_AGG + 2 * 2 * CH * 8;
-constexpr int NUM_BARS = 2 * XS + 2 * US + 4 + 8 + 1 + 4;
+constexpr int NUM_BARS = 2 * XS + 2 * US + 4 + 8 + 1 + 8;
 constexpr uint32_t SMEM_MISC = SMEM_BAR + NUM_BARS * 8;    // tmem base, abort flag
 constexpr uint32_t SMEM_TOTAL = SMEM_MISC + 16;
 constexpr uint32_t SMEM_ALLOC = SMEM_TOTAL + 1024;         // slack for 1024-byte alignment
@@ -71,27 +72,27 @@ __host__ __device__ constexpr uint32_t tm_acc(int bf, int gate) { return (uint32
 
 // y * GeLU(g) for two tokens at once, GeLU(v) = v Phi(v) = v (1 + erf(v / sqrt 2)) / 2 (Section 2.3).  erf by the rational
 // approximation 7.1.26 of Abramowitz & Stegun (|error| < 1.5e-7):
-// 1 - erf(z) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-z^2), t = 1 / (1 + p z), z >= 0.
+// 1 - erf(z) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-z^2), t = 1 / (1 + p z), z >= 0,
+// used as 1 - Phi(|v|) = (1 - erf) / 2 (coefficients halved) and GeLU(v) = max(v, 0) - |v| (1 - Phi(|v|)), which needs no selects.
 __device__ __forceinline__ f32x2 gelu_times2(f32x2 y, float g0, float g1) {
-    const f32x2 g = pack2(g0, g1);
-    const f32x2 z = mul2(pack2(fabsf(g0), fabsf(g1)), pack2(0.70710678f, 0.70710678f));
-    const f32x2 den = fma2(z, pack2(0.3275911f, 0.3275911f), pack2(1.0f, 1.0f));
-    const f32x2 t = pack2(__fdividef(1.0f, lo2(den)), __fdividef(1.0f, hi2(den)));
-    f32x2 q = fma2(t, pack2(1.061405429f, 1.061405429f), pack2(-1.453152027f, -1.453152027f));
-    q = fma2(q, t, pack2(1.421413741f, 1.421413741f));
-    q = fma2(q, t, pack2(-0.284496736f, -0.284496736f));
-    q = fma2(q, t, pack2(0.254829592f, 0.254829592f));
-    const f32x2 ez = mul2(mul2(z, z), pack2(-1.44269504f, -1.44269504f));
-    q = mul2(mul2(q, t), pack2(ex2_approx(lo2(ez)), ex2_approx(hi2(ez))));   // 1 - erf(z)
-    const f32x2 two_phi = pack2(g0 >= 0.0f ? 2.0f - lo2(q) : lo2(q), g1 >= 0.0f ? 2.0f - hi2(q) : hi2(q));   // 1 + erf(g / sqrt 2)
-    return mul2(y, mul2(mul2(g, pack2(0.5f, 0.5f)), two_phi));
+    const f32x2 g = pack2(g0, g1), ga = pack2(fabsf(g0), fabsf(g1));
+    const f32x2 den = fma2(ga, pack2(0.3275911f * 0.70710678f, 0.3275911f * 0.70710678f), pack2(1.0f, 1.0f));
+    const f32x2 t = pack2(rcp_approx(lo2(den)), rcp_approx(hi2(den)));
+    const f32x2 ez = mul2(mul2(g, g), pack2(-0.72134752f, -0.72134752f));   // -v^2 / 2 log2 e
+    f32x2 q = fma2(t, pack2(0.5307027145f, 0.5307027145f), pack2(-0.7265760135f, -0.7265760135f));
+    q = fma2(q, t, pack2(0.7107068705f, 0.7107068705f));
+    q = fma2(q, t, pack2(-0.142248368f, -0.142248368f));
+    q = fma2(q, t, pack2(0.127414796f, 0.127414796f));
+    q = mul2(mul2(q, t), pack2(ex2_approx(lo2(ez)), ex2_approx(hi2(ez))));   // 1 - Phi(|v|)
+    const f32x2 gelu = fma2(pack2(-lo2(ga), -hi2(ga)), q, pack2(fmaxf(g0, 0.0f), fmaxf(g1, 0.0f)));
+    return mul2(y, gelu);
 }
 
 struct Sm100Args {
     // x as [B][T][D] with a box of SLAB_ROWS token rows x one head; y with a box of TILE rows x 32 channels
     alignas(64) CUtensorMap tm_x;
     alignas(64) CUtensorMap tm_y;
-    alignas(64) CUtensorMap tm_g;   // gate branch, same geometry as y (encoded only when the call has one)
+    alignas(64) CUtensorMap tm_g;   // gate branch, same geometry as y (encoded only when the call has one; both then with boxes of HALF rows)
     FwdArgs f;
     int dh;            // width of a head of the layer, a multiple of 32 up to 256.  A "head" below is a group of k = 256 / dh
                        // (rounded down) consecutive layer heads: its weight matrices are block-diagonal with k blocks
@@ -109,9 +110,10 @@ struct Sm100Args {
 using namespace ptx;
 
 // MERGED: the call has a gate branch and writes y_t = h_t GeLU(branch_t); a separate instantiation so that the plain forward
-// carries none of its code.
+// carries none of its code.  GeLU triples the scan warps' work per element, so there are eight of them, half a tile each (four
+// warps with whole tiles: 180 us on B8 T2048 D2560, twice the plain forward).
 template <bool MERGED>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm100_prefill_kernel(const __grid_constant__ Sm100Args p) {
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THREADS : NUM_THREADS, 1) sm100_prefill_kernel(const __grid_constant__ Sm100Args p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t base = (raw_addr + 1023u) & ~1023u;
@@ -126,7 +128,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
     auto BAR_ACCEMPTY = [&](int bf) { return bar0 + 8u * (2 * XS + 2 * US + 2 + bf); };   // leader CTA only
     auto BAR_GDONE = [&](int bf, int q) { return bar0 + 8u * (2 * XS + 2 * US + 4 + bf * 4 + q); };
     const uint32_t BAR_WREADY = bar0 + 8u * (2 * XS + 2 * US + 12);               // leader CTA only: both CTAs' weights are in tensor memory
-    auto BAR_BRANCH = [&](int q) { return bar0 + 8u * (2 * XS + 2 * US + 13 + q); };   // scan warp q's block of the gate branch has landed
+    auto BAR_BRANCH = [&](int w) { return bar0 + 8u * (2 * XS + 2 * US + 13 + w); };   // scan warp w's block of the gate branch has landed
     uint32_t *tmem_base_s = (uint32_t *)(smem + SMEM_MISC);
     volatile int *abort_flag = (volatile int *)(smem + SMEM_MISC + 4);
 
@@ -182,11 +184,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
         for (int s = 0; s < US; ++s) { mbar_init(BAR_UFULL(s), 8); mbar_init(BAR_UEMPTY(s), 10); }
         for (int bf = 0; bf < 2; ++bf) {
             mbar_init(BAR_ACCFULL(bf), 2);    // one commit per MMA issuer
-            mbar_init(BAR_ACCEMPTY(bf), 8);   // the four scan warps of both CTAs
+            mbar_init(BAR_ACCEMPTY(bf), MERGED ? 16 : 8);   // the scan warps of both CTAs
             for (int q = 0; q < 4; ++q) mbar_init(BAR_GDONE(bf, q), 2);
         }
         mbar_init(BAR_WREADY, 16);
-        for (int q = 0; q < 4; ++q) mbar_init(BAR_BRANCH(q), 1);
+        for (int w = 0; w < 8; ++w) mbar_init(BAR_BRANCH(w), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -235,8 +237,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
     }
 
     // Register budget per warpgroup (the four warps of a group execute the same setmaxnreg; the increases draw on
-    // what the decreases release: 128 (96-64) + 128 (96-40) = 256 (112-96) + 128 (152-96)):
-    // conv producers 64, loader / MMA issuers / idle 40, gate warps 112, scan warps 152.
+    // what the decreases release).  20 warps start at 96: conv producers 64, loader / MMA issuers / idle 40, gate warps 112, scan
+    // warps 152: 128 (96-64) + 128 (96-40) = 256 (112-96) + 128 (152-96).  24 warps (merged) start at 80: 64 / 40 / 104 / 80, and
+    // 4 * 32 * (64 + 40) + 8 * 32 * (104 + 80) = 60416 <= 768 * 80.
     if (warp < 4) {
         // ================================================================ conv producers
         reg_dec<64>();
@@ -401,7 +404,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
       }
     } else if (warp < 16) {
         // ================================================================ gate warps
-        reg_inc<112>();
+        if constexpr (MERGED) reg_inc<104>(); else reg_inc<112>();
         const int q = warp & 3, g = (warp - 8) >> 2;     // lane quarter; tokens [32 g, 32 g + 32) of every tile, convolved by CTA g
         const int hc = (int)rank * CH + q * 32 + lane;   // channel within the head
         const int d = cbase + hc;                        // global channel
@@ -485,14 +488,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
         if (!ok && lane == 0) record_timeout();
     } else {
         // ================================================================ scan warps
-        reg_inc<152>();
+        if constexpr (!MERGED) reg_inc<152>();
         const int q = warp & 3;
+        constexpr int SPAN = MERGED ? HALF : TILE;       // tokens of a tile one scan warp writes
+        const int part = (warp - 16) >> 2;               // merged: which half tile
         const int c_own = q * 32 + lane;                 // channel within the CTA
         const int d = cbase + (int)rank * CH + c_own;    // global channel
         const bool exists = (int)rank * CH + c_own < cvalid;   // uniform over the warp; a warp of channel slots that do not exist
                                                                 // keeps the barriers going but reads and writes no global memory
         const uint32_t tm_lane = tmem + ((uint32_t)(q * 32) << 16);
-        const uint32_t y_warp_off = SMEM_Y + (uint32_t)q * 2 * Y_BUF_BYTES;
+        constexpr uint32_t Y_BYTES = SPAN * 32 * 2;
+        const uint32_t y_warp_off = SMEM_Y + (uint32_t)(warp - 16) * 2 * Y_BYTES;
         const float2 *agg_s = (const float2 *)(smem + SMEM_AGG) + c_own;
         const __nv_bfloat16 *x = (const __nv_bfloat16 *)f.x;
         const __nv_bfloat16 *cs_in = (const __nv_bfloat16 *)f.cs_in;
@@ -507,14 +513,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
             const int gidx = (b - B_whole) * p.tps + ti;   // index of the tile's carry record (shared tiles only)
             const int t0 = ti * TILE;
             const int bf = it & 1;
-            const uint32_t y_off = y_warp_off + (uint32_t)bf * Y_BUF_BYTES;
+            const uint32_t y_off = y_warp_off + (uint32_t)bf * Y_BYTES;
             if constexpr (merged) {
-                // The warp's 64 x 32 block of the gate branch is fetched into the y staging buffer of this tile (free once
+                // The warp's 32 x 32 block of the gate branch is fetched into the y staging buffer of this tile (free once
                 // the store of two tiles ago has read it) while the gate warps still work; y then overwrites it in place.
                 if (lane == 0 && exists) {
                     bulk_wait_read1();
-                    mbar_expect_tx(BAR_BRANCH(q), Y_BUF_BYTES);
-                    tma_load_3d(base + y_off, &p.tm_g, cbase + (int)rank * CH + q * 32, t0, b, BAR_BRANCH(q));
+                    mbar_expect_tx(BAR_BRANCH(warp - 16), Y_BYTES);
+                    tma_load_3d(base + y_off, &p.tm_g, cbase + (int)rank * CH + q * 32, t0 + part * HALF, b, BAR_BRANCH(warp - 16));
                 }
                 __syncwarp();
             }
@@ -534,7 +540,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
                 uint4 rec;
                 rec.x = __float_as_uint(e0.x * e1.x); rec.y = p.tag; rec.z = __float_as_uint(fmaf(e1.x, e0.y, e1.y)); rec.w = p.tag;
                 uint4 *dst = p.agg + ((size_t)group * p.tiles_total + gidx) * CH + c_own;
-                asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "r"(rec.x), "r"(rec.y), "r"(rec.z), "r"(rec.w) : "memory");
+                if (part == 0) asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "r"(rec.x), "r"(rec.y), "r"(rec.z), "r"(rec.w) : "memory");
                 int nback;
                 if (ti < S) { h = f.h0 && exists ? f.h0[(size_t)b * D + d] : 0.0f; P = 1.0f; nback = ti; }
                 else { h = h_prev_own; P = P_prev_own; nback = S - 1; }
@@ -583,33 +589,45 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
             __syncwarp();
             // ---- y_t = h_t = (h_t from zero) + (prod a up to t) h_in  (Eq. 4 unrolled over the half tile), 16 tokens at a time
             uint16_t *y_s = (uint16_t *)(smem + y_off) + lane;   // this thread's column of the warp's y block [64 tokens][32 channels]
-            // The whole tile is pulled into registers and the accumulator buffer handed back before any arithmetic: the buffer's
-            // round trip (MMA -> gate warps -> here -> MMA) is what paces the kernel.
-            float C[TILE], H[TILE];
             const uint32_t tc = tm_lane + tm_acc(bf, 0), th = tm_lane + tm_acc(bf, 1);
-#pragma unroll
-            for (int c0 = 0; c0 < TILE; c0 += 16) { tmem_ld16f(tc + c0, C + c0); tmem_ld16f(th + c0, H + c0); }
-            tmem_ld_wait();
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_at(BAR_ACCEMPTY(bf), 0);
             if constexpr (merged) {
                 // merged output of the recurrent block (Section 2.3): y_t = h_t GeLU(branch_t); the state is not touched
                 if (exists) {
-                    ok = warp_wait(BAR_BRANCH(q), it & 1, spin, abort_flag);
+                    ok = warp_wait(BAR_BRANCH(warp - 16), it & 1, spin, abort_flag);
                     if (!ok) break;
                 }
+                const f32x2 hb = part ? pack2(h_mid, h_mid) : pack2(h, h);
 #pragma unroll
-                for (int j = 0; j < TILE; j += 2) {
-                    const float hb = j < HALF ? h : h_mid;
-                    const float g0 = __uint_as_float((uint32_t)y_s[j * 32] << 16), g1 = __uint_as_float((uint32_t)y_s[(j + 1) * 32] << 16);
-                    const f32x2 ym = gelu_times2(fma2(pack2(C[j], C[j + 1]), pack2(hb, hb), pack2(H[j], H[j + 1])), g0, g1);
-                    const __nv_bfloat162 o = __floats2bfloat162_rn(lo2(ym), hi2(ym));
-                    const uint32_t ow = *(const uint32_t *)&o;
-                    y_s[j * 32] = (uint16_t)(ow & 0xFFFFu);
-                    y_s[(j + 1) * 32] = (uint16_t)(ow >> 16);
+                for (int bt = 0; bt < 2; ++bt) {
+                    f32x2 C[8], H[8];
+                    tmem_ld16(tc + part * HALF + 16 * bt, C);
+                    tmem_ld16(th + part * HALF + 16 * bt, H);
+                    tmem_ld_wait();
+                    if (bt == 1) {   // the buffer goes back before the arithmetic of its last tokens
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_at(BAR_ACCEMPTY(bf), 0);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        uint16_t *y0 = y_s + (16 * bt + 2 * j) * 32, *y1 = y0 + 32;
+                        const f32x2 ym = gelu_times2(fma2(C[j], hb, H[j]), __uint_as_float((uint32_t)*y0 << 16), __uint_as_float((uint32_t)*y1 << 16));
+                        const __nv_bfloat162 o = __floats2bfloat162_rn(lo2(ym), hi2(ym));
+                        const uint32_t ow = *(const uint32_t *)&o;
+                        *y0 = (uint16_t)(ow & 0xFFFFu);
+                        *y1 = (uint16_t)(ow >> 16);
+                    }
                 }
             } else {
+                // The whole tile is pulled into registers and the accumulator buffer handed back before any arithmetic: the buffer's
+                // round trip (MMA -> gate warps -> here -> MMA) is what paces the kernel.
+                float C[TILE], H[TILE];
+#pragma unroll
+                for (int c0 = 0; c0 < TILE; c0 += 16) { tmem_ld16f(tc + c0, C + c0); tmem_ld16f(th + c0, H + c0); }
+                tmem_ld_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_at(BAR_ACCEMPTY(bf), 0);
 #pragma unroll
                 for (int j = 0; j < TILE; j += 2) {
                     const float hb = j < HALF ? h : h_mid;
@@ -623,11 +641,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NUM_THREADS, 1) sm10
             fence_async_smem();   // y rows become visible to the bulk-copy engine
             __syncwarp();
             if (lane == 0 && exists) {
-                // the warp's 64 tokens x 32 channels go out as one tiled store; rows at or beyond T are clipped
-                tma_store_3d(&p.tm_y, cbase + (int)rank * CH + q * 32, t0, b, base + y_off);
+                // the warp's tokens x 32 channels go out as one tiled store; rows at or beyond T are clipped
+                if (!merged || t0 + part * HALF < T) tma_store_3d(&p.tm_y, cbase + (int)rank * CH + q * 32, t0 + part * HALF, b, base + y_off);
                 bulk_commit();
             }
-            if (ti == p.tps - 1 && exists) {
+            if (ti == p.tps - 1 && exists && part == 0) {
                 // end of a sequence: h_T (unrounded state) and the last three raw inputs, bit-exact
                 f.h_T[(size_t)b * D + d] = h_prev_own;
                 if (f.a_prod) f.a_prod[(size_t)b * D + d] = P_prev_own;
@@ -803,10 +821,10 @@ cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes,
     DeviceInfo di;
     if ((e = device_info(&di)) != cudaSuccess) return e;
     Sm100Args p;
-    if (!make_activation_map(&p.tm_x, a.x, a.B, a.T, a.D, DH, SLAB_ROWS) || !make_activation_map(&p.tm_y, a.y, a.B, a.T, a.D, 32, TILE))
+    if (!make_activation_map(&p.tm_x, a.x, a.B, a.T, a.D, DH, SLAB_ROWS) || !make_activation_map(&p.tm_y, a.y, a.B, a.T, a.D, 32, a.gate_branch ? HALF : TILE))
         return cudaErrorNotSupported;
     if (a.gate_branch) {
-        if (!make_activation_map(&p.tm_g, a.gate_branch, a.B, a.T, a.D, 32, TILE)) return cudaErrorNotSupported;
+        if (!make_activation_map(&p.tm_g, a.gate_branch, a.B, a.T, a.D, 32, HALF)) return cudaErrorNotSupported;
     } else {
         p.tm_g = p.tm_y;   // never used by the kernel
     }
@@ -837,7 +855,7 @@ cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes,
         if ((e = cudaMemcpyAsync(cs_copy, a.cs_in, cs_bytes, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
         p.f.cs_in = cs_copy;
     }
-    return launch_dependent(a.gate_branch ? sm100_prefill_kernel<true> : sm100_prefill_kernel<false>, dim3(2 * G * S), dim3(NUM_THREADS), SMEM_ALLOC, st, p);
+    return launch_dependent(a.gate_branch ? sm100_prefill_kernel<true> : sm100_prefill_kernel<false>, dim3(2 * G * S), dim3(a.gate_branch ? MERGED_THREADS : NUM_THREADS), SMEM_ALLOC, st, p);
 }
 
 }  // namespace rglru

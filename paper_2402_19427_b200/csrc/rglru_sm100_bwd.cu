@@ -259,7 +259,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
 // ------------------------------------------------------------------ element-wise kernels
 __device__ __forceinline__ float sigmoid_acc(float z) { return 1.0f / (1.0f + expf(-z)); }
 // Hardware-approximate versions for the per-element work (relative error ~1e-6, far inside the gradient tolerance)
-__device__ __forceinline__ float rcp_fast(float x) { float y; asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 __device__ __forceinline__ float rsqrt_fast(float x) { float y; asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x)); return y; }
 // 1 - exp(x) for x <= 0 without cancellation near 0
 __device__ __forceinline__ float one_minus_exp(float x) {
@@ -405,7 +404,7 @@ __device__ __forceinline__ f32x2 one_minus_exp_neg2(f32x2 x) {
 template <bool POLY> __device__ __forceinline__ void gate_f2(f32x2 za, f32x2 nba, f32x2 s2, f32x2 &r, f32x2 &f) {
     const f32x2 e = fma2(za, pack2(-LOG2E, -LOG2E), nba);   // -(z + b) log2 e
     const f32x2 q = __fadd2_rn(pack2(ex2_approx(e.x), ex2_approx(e.y)), pack2(1.0f, 1.0f));
-    r = pack2(rcp_fast(q.x), rcp_fast(q.y));
+    r = pack2(rcp_approx(q.x), rcp_approx(q.y));
     const f32x2 x = mul2(s2, r);
     f = POLY ? one_minus_exp_neg2(x) : pack2(one_minus_exp(-x.x), one_minus_exp(-x.y));
 }
@@ -560,7 +559,7 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
             if (k == 0 && t0 == 0 && a.h0 && cv) hp = ld2f(a.h0 + (size_t)b * D + d);
             const f32x2 e = fma2(hf2x(sm[2 * TW + k * 32]), pack2(-LOG2E, -LOG2E), nbx);
             const f32x2 q = __fadd2_rn(pack2(ex2_approx(e.x), ex2_approx(e.y)), ONE);
-            const f32x2 gi = pack2(rcp_fast(q.x), rcp_fast(q.y));
+            const f32x2 gi = pack2(rcp_approx(q.x), rcp_approx(q.y));
             const f32x2 at = fma2(f[k], NEG, ONE), m2 = mul2(f[k], fma2(f[k], NEG, TWO));
             const f32x2 rm = pack2(m2.x > 0.0f ? rsqrt_fast(m2.x) : 0.0f, m2.y > 0.0f ? rsqrt_fast(m2.y) : 0.0f);   // 1 / sqrt(1 - a^2)
             const f32x2 g = __fadd2_rn(bf2x(sm[TW + k * 32]), carry);
@@ -868,7 +867,7 @@ __device__ __forceinline__ void wide_scan_column(const WideScanArgs &p, ScanShar
             if (k >= nv) fa = pack2(0.f, 0.f);   // a token that does not exist holds the state: a = 1, m = 0
             const f32x2 e = fma2(hf2x(sm[TW + k * 32]), pack2(-LOG2E, -LOG2E), nbx);
             const f32x2 q = __fadd2_rn(pack2(ex2_approx(e.x), ex2_approx(e.y)), ONE);
-            const f32x2 gi = pack2(rcp_fast(q.x), rcp_fast(q.y));
+            const f32x2 gi = pack2(rcp_approx(q.x), rcp_approx(q.y));
             const f32x2 at = fma2(fa, NEG, ONE), m2 = mul2(fa, fma2(fa, NEG, TWO));
             const f32x2 m = pack2(sqrt_approx(m2.x), sqrt_approx(m2.y));
             Hc = fma2(at, Hc, mul2(m, mul2(gi, hf2x(sm[2 * TW + k * 32]))));
