@@ -65,7 +65,7 @@ struct GemmArgs {
 // walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... with two accumulators, so that the epilogue of one tile overlaps
 // the loads and MMAs of the next.  Tile number -> (x, y, z) with x fastest:
 //   MODE_Z : (token tiles, 2 gates x nt, H)   A = u[tok][h][k]        B = W_gate[h][out][k]
-//   MODE_DU: (token tiles, nt, H)             A = dz[tok][h][k=2 NS]  B = W^T[h][in][k=2 NS]
+//   MODE_DU: (token tiles, nt, H)             A = dz[tok][h][k=2 NS]  B = W[gate][h][k=out][in], MN-major
 //   MODE_DW: (2 NS / 128, splits x nt, H)     A = dz[tok][h][row]     B = u[tok][h][in], both MN-major, K = this split's tokens
 // 32-byte accesses: one whole DRAM sector per thread and instruction where a thread owns a row (pointers 32-byte aligned)
 __device__ __forceinline__ void st_global_v8(void *ptr, const uint32_t (&r)[8]) {
@@ -118,8 +118,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
         // ---- TMA producer
         if (lane == 0) {
             int kbg = 0;   // K blocks issued so far, over all tiles (ring position)
-            const int ncopies = (p.NT + 63) / 64;   // MODE_DW: 64-channel copies of the B operand
-            const uint32_t tx_bytes = A_STAGE_BYTES + (p.mode == MODE_DW ? (uint32_t)ncopies * MN_BLOCK_BYTES : (uint32_t)p.NT * 128u);
+            const int ncopies = (p.NT + 63) / 64;   // 64-channel copies of an MN-major B operand
+            const uint32_t tx_bytes = A_STAGE_BYTES + (p.mode != MODE_Z ? (uint32_t)ncopies * MN_BLOCK_BYTES : (uint32_t)p.NT * 128u);
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
                 const int tx = tile % p.nx, ty = (tile / p.nx) % p.ny, h = tile / (p.nx * p.ny);
                 const int col0 = (ty % p.nt) * p.NT, sel = ty / p.nt;   // sel: gate (MODE_Z), split (MODE_DW)
@@ -142,9 +142,14 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                         // u is read out of the layer's [tok][D] array at the group's first channel (channels past the group's own
                         // meet zero weights; past D they read as zero); dz has the groups' own [tok][group][2][NS] layout
                         const int kc = kb < kslots ? kb * 64 : p.NS + (kb - kslots) * 64;   // MODE_DU: the second gate's slots follow the first's
-                        if (p.mode == MODE_Z) tma_load_3d(a_dst, &p.tm_a, h * p.hstride + kb * 64, tx * 128, 0, BAR_FULL(s));
-                        else tma_load_3d(a_dst, &p.tm_a, kc, h, tx * 128, BAR_FULL(s));
-                        tma_load_3d(b_dst, tb, kc, col0, h, BAR_FULL(s));
+                        if (p.mode == MODE_Z) {
+                            tma_load_3d(a_dst, &p.tm_a, h * p.hstride + kb * 64, tx * 128, 0, BAR_FULL(s));
+                            tma_load_3d(b_dst, tb, kb * 64, col0, h, BAR_FULL(s));
+                        } else {
+                            tma_load_3d(a_dst, &p.tm_a, kc, h, tx * 128, BAR_FULL(s));
+                            const int gate = kb >= kslots, o0 = (kb - gate * kslots) * 64;
+                            for (int j = 0; j < ncopies; ++j) tma_load_3d(b_dst + j * MN_BLOCK_BYTES, tb, col0 + j * 64, o0, gate * p.H + h, BAR_FULL(s));
+                        }
                     }
                 }
             }
@@ -153,7 +158,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
     } else if (warp == 1) {
         // ---- MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = make_idesc_f16(128, p.NT), idesc_mn = make_idesc_f16_mn(128, p.NT);
+            const uint32_t idesc = make_idesc_f16(128, p.NT), idesc_mn = make_idesc_f16_mn(128, p.NT), idesc_bmn = make_idesc_f16_bmn(128, p.NT);
             int kbg = 0, it = 0;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
                 const int acc = it & 1;
@@ -172,6 +177,10 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                         for (int ks = 0; ks < 4; ++ks)
                             mma_ss(tmem + acc * 256, make_desc_sw128_mn(a_src + ks * 2048, MN_BLOCK_BYTES), make_desc_sw128_mn(b_src + ks * 2048, MN_BLOCK_BYTES),
                                    idesc_mn, (kb | ks) != 0);
+                    } else if (p.mode == MODE_DU) {
+#pragma unroll
+                        for (int ks = 0; ks < 4; ++ks)
+                            mma_ss(tmem + acc * 256, make_desc_sw128(a_src + ks * 32), make_desc_sw128_mn(b_src + ks * 2048, MN_BLOCK_BYTES), idesc_bmn, (kb | ks) != 0);
                     } else {
 #pragma unroll
                         for (int ks = 0; ks < 4; ++ks)
@@ -294,33 +303,27 @@ struct EwArgs {
     float *dh0;                       // [B][D] gradient of h0, or null
 };
 
-// fp16 copies of the gate weights: W16[g][h][o][n] = W_g[h][o][n] and, unless null, WT[h][n][g*NS + o] = W_g[h][o][n]
-// One block per 32 x 32 tile of one (gate, group) matrix; the transposed copy goes through shared memory so that both
-// copies are written with consecutive threads on consecutive addresses.  grid (NS/32, NS/32, 2 H), block (32, 8)
-// H counts groups; dh is the width of a head of the layer (a multiple of 32): a group holds k heads on its diagonal -- fewer
-// in a partial last group of a layer of Hl heads -- and every tile outside those blocks is written as zeros.
-__global__ void convert_w_kernel(const __nv_bfloat16 *Wa, const __nv_bfloat16 *Wx, __half *W16, __half *WT, int H, int NS, int k, int dh, int Hl) {
-    __shared__ __half tile[32][33];
+// fp16 copy of the gate weights, W16[g][h][o][n] = W_g[h][o][n], eight elements per thread.  H counts groups; dh is the width of a
+// head of the layer (a multiple of 32): a group holds k heads on its diagonal -- fewer in a partial last group of a layer of Hl
+// heads -- and everything outside those blocks is written as zeros.  Both the z product (K-major) and the du product (MN-major)
+// read this one copy.
+__global__ void __launch_bounds__(256) convert_w_kernel(const __nv_bfloat16 *Wa, const __nv_bfloat16 *Wx, __half *W16, int H, int NS, int k, int dh, int Hl) {
     dependency_wait();
-    const int g = blockIdx.z / H, h = blockIdx.z % H;
-    const int o0 = blockIdx.y * 32, n0 = blockIdx.x * 32;
-    const int sub = o0 / dh;                         // head of the group that owns these output rows
-    const int heads_here = min(k, Hl - h * k);
-    const bool on_diagonal = sub < heads_here && n0 / dh == sub;
-    const __nv_bfloat16 *W = (g ? Wx : Wa) + ((size_t)h * k + sub) * dh * dh + (size_t)(o0 - sub * dh) * dh + (n0 - sub * dh);
-    __half *W16m = W16 + ((size_t)g * H + h) * NS * NS;
-#pragma unroll
-    for (int r = threadIdx.y; r < 32; r += 8) {
-        const float v = on_diagonal ? __bfloat162float(W[(size_t)r * dh + threadIdx.x]) : 0.0f;
-        const __half hv = __float2half_rn(fminf(fmaxf(v, -65504.0f), 65504.0f));
-        W16m[(size_t)(o0 + r) * NS + n0 + threadIdx.x] = hv;
-        tile[r][threadIdx.x] = hv;
+    const int per_row = NS / 8;
+    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= (size_t)2 * H * NS * per_row) return;
+    const int n0 = (int)(i % per_row) * 8;
+    size_t r = i / per_row;
+    const int o = (int)(r % NS); r /= NS;
+    const int h = (int)(r % H), g = (int)(r / H);
+    const int sub = o / dh;                          // head of the group that owns this output row
+    uint4 out = make_uint4(0u, 0u, 0u, 0u);
+    if (sub < min(k, Hl - h * k) && n0 / dh == sub) {
+        const uint4 v = *(const uint4 *)((g ? Wx : Wa) + (((size_t)h * k + sub) * dh + (o - sub * dh)) * dh + (n0 - sub * dh));
+        auto cvt2 = [](uint32_t w) { return pack_f16_sat(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); };
+        out = make_uint4(cvt2(v.x), cvt2(v.y), cvt2(v.z), cvt2(v.w));
     }
-    if (WT == nullptr) return;
-    __syncthreads();
-#pragma unroll
-    for (int r = threadIdx.y; r < 32; r += 8)
-        WT[((size_t)h * NS + n0 + r) * (2 * NS) + g * NS + o0 + threadIdx.x] = tile[threadIdx.x][r];
+    *(uint4 *)(W16 + i * 8) = out;
 }
 
 // Fixed-order sum over the token splits of the diagonal blocks of the groups' weight gradients: one thread per
@@ -736,7 +739,7 @@ Groups make_groups(int D, int H) {
 
 struct BwdLayout {
     size_t BT, BTp, off_u, off_z, off_dz, off_du, off_y, off_hT, off_cs, off_rec, off_pvec, off_pconv, off_pdw,
-        off_wt, off_w16, off_fws, total;
+        off_w16, off_fws, total;
     int nchunk, nchunk_conv, S, kb_per_split;
 };
 
@@ -764,7 +767,6 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     L.off_pvec = take((size_t)B * (L.nchunk < SCAN_MAX_S ? L.nchunk : SCAN_MAX_S) * 3 * D * 4);
     L.off_pconv = take((size_t)B * L.nchunk_conv * 5 * D * 4);
     L.off_pdw = take((size_t)L.S * 2 * gr.G * gr.NS * gr.NS * 4);
-    L.off_wt = take(gr.W16_bytes());
     L.off_w16 = take(gr.W16_bytes());
     L.off_fws = take(gr.dh <= DH ? sm100_prefill_workspace_bytes(B, T, D, Hl) : sm100_wide_prefill_workspace_bytes(B, T, D, Hl));
     L.total = o;
@@ -781,6 +783,10 @@ cudaError_t run_gemm(const GemmArgs &g, cudaStream_t st) {
     cudaError_t e = opt_in.ensure(tc_gemm_kernel, (int)GEMM_SMEM_ALLOC);
     if (e != cudaSuccess) return e;
     return launch_dependent(tc_gemm_kernel, dim3(gemm_grid(g)), dim3(GEMM_THREADS), GEMM_SMEM_ALLOC, st, g);
+}
+cudaError_t convert_w(const Groups &gr, const void *Wa, const void *Wx, int Hl, __half *W16, cudaStream_t st) {
+    const size_t n = (size_t)2 * gr.G * gr.NS * (gr.NS / 8);
+    return launch_dependent(convert_w_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, (const __nv_bfloat16 *)Wa, (const __nv_bfloat16 *)Wx, W16, gr.G, gr.NS, gr.k, gr.dh, Hl);
 }
 // z = u W^T per group and gate: u [ntok][D], z [ntok][G][2][NS]
 cudaError_t gemm_z(const Groups &gr, int D, size_t ntok, const __half *u, const __half *W16, __half *z, uint32_t *status, cudaStream_t st) {
@@ -1026,7 +1032,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     cudaError_t e;
     char *ws = (char *)ws_body;
     __half *u = (__half *)(ws + L.off_u), *z = (__half *)(ws + L.off_z);
-    __half *dz = (__half *)(ws + L.off_dz), *WT = (__half *)(ws + L.off_wt), *W16 = (__half *)(ws + L.off_w16);
+    __half *dz = (__half *)(ws + L.off_dz), *W16 = (__half *)(ws + L.off_w16);
     __half *du = (__half *)(ws + L.off_du);
 
     // 0. h_{t-1} comes from the forward output; run the forward when the caller kept none
@@ -1051,8 +1057,8 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     a.tag = next_call_tag(); a.spin_ns = g_spin_limit_ns; a.status = status; a.part_vec = (float *)(ws + L.off_pvec);
     a.dh_T = q.dh_T; a.dh0 = q.dh0;
 
-    // 1. W^T for the du contraction, conv output
-    if ((e = launch_dependent(convert_w_kernel, dim3(NS / 32, NS / 32, 2 * H), dim3(32, 8), 0, st, (const __nv_bfloat16 *)q.W_a, (const __nv_bfloat16 *)q.W_x, W16, WT, H, NS, gr.k, gr.dh, q.H)) != cudaSuccess) return e;
+    // 1. fp16 weights, conv output
+    if ((e = convert_w(gr, q.W_a, q.W_x, q.H, W16, st)) != cudaSuccess) return e;
     const dim3 grid_conv((D + 511) / 512, L.nchunk_conv, B);
     if ((e = launch_dependent(conv_forward_kernel, grid_conv, dim3(256), 0, st, ConvArgs{T, D, 0, 0, T, a.x, a.conv_w, a.cs_in, a.conv_b, u, a.epoch})) != cudaSuccess) return e;
 
@@ -1084,9 +1090,9 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     const uint64_t K2 = 2 * (uint64_t)NS, ddz[3] = {K2, (uint64_t)H, BT}, sdz[2] = {K2 * 2, (uint64_t)H * K2 * 2};   // dz [tok][group][gate, slot]
     {
         const uint32_t ba[3] = {64, 1, 128};
-        const uint64_t db[3] = {K2, (uint64_t)NS, (uint64_t)H}, sb[2] = {K2 * 2, (uint64_t)NS * K2 * 2};
-        const uint32_t bb[3] = {64, (uint32_t)gr.NT, 1};
-        if (!encode_map16_3d(&g.tm_a, dz, ddz, sdz, ba, true) || !encode_map16_3d(&g.tm_b0, WT, db, sb, bb, true)) return cudaErrorNotSupported;
+        const uint64_t db[3] = {(uint64_t)NS, (uint64_t)NS, 2 * (uint64_t)H}, sb[2] = {(uint64_t)NS * 2, (uint64_t)NS * NS * 2};   // W16 [gate, group][out][in]
+        const uint32_t bb[3] = {64, 64, 1};
+        if (!encode_map16_3d(&g.tm_a, dz, ddz, sdz, ba, true) || !encode_map16_3d(&g.tm_b0, W16, db, sb, bb, true)) return cudaErrorNotSupported;
         g.tm_b1 = g.tm_b0;
         g.mode = MODE_DU; g.rows_valid = (int)BT; g.out = du;
         g.nx = (int)mtiles; g.ny = gr.nt;
@@ -1158,7 +1164,7 @@ cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_b
     if (a.gate_branch) {
         if (!encode_bf16_map_3d(&p.tm_g, a.gate_branch, (uint64_t)D, (uint64_t)T, (uint64_t)B, 64, SCAN_CHUNK, false)) return cudaErrorNotSupported;
     }
-    if ((e = launch_dependent(convert_w_kernel, dim3(gr.NS / 32, gr.NS / 32, 2 * gr.G), dim3(32, 8), 0, st, (const __nv_bfloat16 *)a.W_a, (const __nv_bfloat16 *)a.W_x, W16, (__half *)nullptr, gr.G, gr.NS, gr.k, gr.dh, a.H)) != cudaSuccess) return e;
+    if ((e = convert_w(gr, a.W_a, a.W_x, a.H, W16, st)) != cudaSuccess) return e;
     const int slots = 2 * num_sms();
     for (int b0 = 0; b0 < B; b0 += L.nb) {
         for (int tb = 0; tb < T; tb += L.n) {

@@ -222,6 +222,10 @@ __device__ __forceinline__ uint64_t make_desc_sw128_mn(uint32_t saddr, uint32_t 
 __host__ __device__ constexpr uint32_t make_idesc_f16_mn(int M, int N) {
     return (1u << 4) | (1u << 15) | (1u << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
+// the same with only B MN-major (bit 16)
+__host__ __device__ constexpr uint32_t make_idesc_f16_bmn(int M, int N) {
+    return (1u << 4) | (1u << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
 // kind::f16 instruction descriptor: fp32 accumulator, fp16 A and B, both K-major, M x N
 __host__ __device__ constexpr uint32_t make_idesc_f16(int M, int N) {
     return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
