@@ -27,7 +27,6 @@ constexpr int NT = 256;  // threads per block of the element-wise and decode ker
 constexpr int GT = 16;   // sequences per tile of the decode kernel
 constexpr int NB = 16;   // input channels per staged weight slab of the decode kernel
 constexpr int MT = 128;  // threads per block of the contractions
-constexpr int BK = 16;   // K slab of the contractions
 
 __device__ __forceinline__ float tof(float v) { return v; }
 __device__ __forceinline__ float tof(__nv_bfloat16 v) { return __bfloat162float(v); }
@@ -81,8 +80,11 @@ __device__ __forceinline__ IOT x_raw_at(const IOT *x, const IOT *cs_in, int T, i
 // Geometry of a block: 128 threads as 8 (rows) x 16 (columns); BM rows x 2 BM columns of results.  Thread (ty, tx) owns rows
 // TM ty .. TM ty + TM - 1 and columns NH tx .. + NH - 1 of each half of the columns (in the forward the halves are the two
 // gates of the same channels).
+// A slab is BK deep: small blocks, of which an SM holds one or two, take twice the depth so that fewer rounds of load latency
+// are exposed.
 template <int BM> struct Tile {
-    static constexpr int BN = 2 * BM, TM = BM / 8, NH = BM / 16;
+    static constexpr int BN = 2 * BM, TM = BM / 8, NH = BM / 16, BK = BM == 64 ? 16 : 32;
+    static constexpr int TA = BM * BK / MT, EB = BN * BK / MT;   // values of the A and B slab a thread brings in
     static constexpr int AS = BM + 4, BS = BN + 4;   // row strides in shared memory (floats): 16-byte rows, shifted by one bank group
     float As[2][BK][AS], Bs[2][BK][BS];
 };
@@ -91,7 +93,7 @@ template <int BM>
 __device__ __forceinline__ void mul_slab(const Tile<BM> &s, int buf, int ty, int tx, f32x2 (&acc)[Tile<BM>::TM][Tile<BM>::NH]) {
     constexpr int TM = Tile<BM>::TM, NH = Tile<BM>::NH;
 #pragma unroll
-    for (int k = 0; k < BK; ++k) {
+    for (int k = 0; k < Tile<BM>::BK; ++k) {
         float a[TM];
         f32x2 b[NH];
 #pragma unroll
@@ -116,36 +118,36 @@ template <int NH> __device__ __forceinline__ float col(const f32x2 (&row)[NH], i
     const f32x2 p = row[half * (NH / 2) + j / 2];
     return (j & 1) ? p.y : p.x;
 }
-// A BK x W block of a row-major matrix (rows = K index, W contiguous columns) on its way to shared memory: 128 threads, W / 8
-// values each, by fours of one row when the addresses allow it.
-template <int W, bool VEC, typename T>
-__device__ __forceinline__ void fetch_rows(const T *src, size_t stride, int rows_valid, int cols_valid, int tid, float (&v)[W / 8]) {
+// A BK x W block of a row-major matrix (rows = K index, W contiguous columns) on its way to shared memory: 128 threads,
+// BK W / 128 values each, by fours of one row when the addresses allow it.
+template <int W, int N, bool VEC, typename T>
+__device__ __forceinline__ void fetch_rows(const T *src, size_t stride, int rows_valid, int cols_valid, int tid, float (&v)[N]) {
     if (VEC) {
 #pragma unroll
-        for (int i = 0; i < W / 32; ++i) {
+        for (int i = 0; i < N / 4; ++i) {
             const int e = tid + MT * i, k = e / (W / 4), n = (e % (W / 4)) * 4;
             if (k < rows_valid && n < cols_valid) ld4(src + (size_t)k * stride + n, v + 4 * i);
             else { v[4 * i] = 0.f; v[4 * i + 1] = 0.f; v[4 * i + 2] = 0.f; v[4 * i + 3] = 0.f; }
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < W / 8; ++i) {
+        for (int i = 0; i < N; ++i) {
             const int e = tid + MT * i, k = e / W, n = e % W;
             v[i] = k < rows_valid && n < cols_valid ? tof(src[(size_t)k * stride + n]) : 0.0f;
         }
     }
 }
-template <int W, bool VEC, int S>
-__device__ __forceinline__ void put_rows(float (&dst)[BK][S], int tid, const float (&v)[W / 8]) {
+template <int W, int N, bool VEC, int K, int S>
+__device__ __forceinline__ void put_rows(float (&dst)[K][S], int tid, const float (&v)[N]) {
     if (VEC) {
 #pragma unroll
-        for (int i = 0; i < W / 32; ++i) {
+        for (int i = 0; i < N / 4; ++i) {
             const int e = tid + MT * i, k = e / (W / 4), n = (e % (W / 4)) * 4;
             *(float4 *)&dst[k][n] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         }
     } else {
 #pragma unroll
-        for (int i = 0; i < W / 8; ++i) { const int e = tid + MT * i; dst[e / W][e % W] = v[i]; }
+        for (int i = 0; i < N; ++i) { const int e = tid + MT * i; dst[e / W][e % W] = v[i]; }
     }
 }
 // E consecutive K values of one row of a matrix whose rows run along K (it is transposed on its way to shared memory)
@@ -164,8 +166,9 @@ template <int E, bool VEC, typename T> __device__ __forceinline__ void fetch_k(c
 
 // ------------------------------------------------------------------ chain of chunks
 // One record {A, tag, B, tag2} per (sequence, channel): what the chunks so far hand to the next one.  Chunk c waits for the
-// tags of its predecessor and overwrites the record with its own; nobody else reads it, so one slot serves the whole chain
-// (and what a finished call leaves behind carries the tag of the last chunk, which no chunk ever waits for).
+// tags of its predecessor and overwrites the record with its own; nobody else reads it, so one slot serves the whole chain.
+// The last chunk writes too: what a finished call leaves behind carries a tag that no chunk waits for, also when a CUDA graph
+// replays the call with the same tags.
 struct Chain {
     uint4 *slot;        // [B][D]
     uint32_t tag, tag2;
@@ -208,7 +211,7 @@ template <typename IOT, bool SAVE, int BM, bool VEC>
 __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(FwdArgs a, Chain ch, int nchunk, int ntile) {
     ptx::dependency_wait();
     using TL = Tile<BM>;
-    constexpr int TM = TL::TM, NH = TL::NH, EB = TL::BN / 8;
+    constexpr int TM = TL::TM, NH = TL::NH, BK = TL::BK, TA = TL::TA, EB = TL::EB;
     __shared__ __align__(16) TL s;
     __shared__ float agg_P[8][BM], agg_h[8][BM], in_h[8][BM];
     __shared__ int ok_s;
@@ -223,20 +226,18 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(F
     const IOT *xb = x + (size_t)b * T * D;
     if (tid == 0) ok_s = 1;
 
-    // A operand: this thread convolves channel kk of each slab for tokens TM seg .. + TM - 1 of the chunk
-    const int kk = tid & 15, seg = tid >> 4, ta = t0 + seg * TM;
+    // A operand: this thread convolves channel kk of each slab for tokens TA seg .. + TA - 1 of the chunk
+    const int kk = tid % BK, seg = tid / BK, ta = t0 + seg * TA;
     // B operand: row br of the 2 BM weight rows (both gates), EB consecutive input channels from koff
-    constexpr int ROWS_PER_PASS = MT < TL::BN ? MT : TL::BN;
-    static_assert(ROWS_PER_PASS * EB * (MT / ROWS_PER_PASS) == TL::BN * BK, "weight slab is covered exactly once");
     const int br = tid % TL::BN, koff = (tid / TL::BN) * EB;
     const int bch = n0 + (br % BM);
     const IOT *wrow = (const IOT *)(br < BM ? a.W_a : a.W_x) + ((size_t)head * Dh + (bch < Dh ? bch : 0)) * Dh + koff;
-    float xr[TM + 3], taps[4], cb, wv[EB];
+    float xr[TA + 3], taps[4], cb, wv[EB];
     auto fetch = [&](int k0) {
         const int k = k0 + kk, d = d0 + k;
         const bool kv = k < Dh;
 #pragma unroll
-        for (int i = 0; i < TM + 3; ++i) {
+        for (int i = 0; i < TA + 3; ++i) {
             const int t = ta - 3 + i;
             float v = 0.0f;
             if (kv) {
@@ -251,15 +252,15 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(F
         fetch_k<EB, VEC>(wrow + k0, bch < Dh, Dh - k0 - koff, wv);
     };
     auto stage = [&](int buf) {
-        float u[TM];
+        float u[TA];
 #pragma unroll
-        for (int i = 0; i < TM; ++i) {
+        for (int i = 0; i < TA; ++i) {
             u[i] = fmaf(taps[0], xr[i + 3], cb);
 #pragma unroll
             for (int j = 1; j < 4; ++j) u[i] = fmaf(taps[j], xr[i + 3 - j], u[i]);
         }
 #pragma unroll
-        for (int i = 0; i < TM; i += 4) *(float4 *)&s.As[buf][kk][seg * TM + i] = make_float4(u[i], u[i + 1], u[i + 2], u[i + 3]);
+        for (int i = 0; i < TA; i += 4) *(float4 *)&s.As[buf][kk][seg * TA + i] = make_float4(u[i], u[i + 1], u[i + 2], u[i + 3]);
 #pragma unroll
         for (int i = 0; i < EB; ++i) s.Bs[buf][koff + i][br] = wv[i];
     };
@@ -335,19 +336,21 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(F
         const bool cv = n0 + tid < Dh;
         const int d = cv ? d0 + n0 + tid : d0;
         uint4 *slot = ch.slot + (size_t)b * D + d;
-        float hs = 0.0f, Ps = 1.0f;
-        bool ok = true;
-        if (chunk == 0) hs = a.h0 ? a.h0[(size_t)b * D + d] : 0.0f;
-        else ok = chain_wait(ch, slot, cv, chunk - 1, hs, Ps);
+        // the chunk as one step first, so that a link of the chain is one FMA between the record that arrives and the one that leaves
+        float cP = 1.0f, cH = 0.0f;
 #pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            in_h[q][tid] = hs;
-            hs = fmaf(agg_P[q][tid], hs, agg_h[q][tid]);
-            Ps *= agg_P[q][tid];
-        }
+        for (int q = 0; q < 8; ++q) { cH = fmaf(agg_P[q][tid], cH, agg_h[q][tid]); cP *= agg_P[q][tid]; }
+        float h_in = 0.0f, P_in = 1.0f;
+        bool ok = true;
+        if (chunk == 0) h_in = a.h0 ? a.h0[(size_t)b * D + d] : 0.0f;
+        else ok = chain_wait(ch, slot, cv, chunk - 1, h_in, P_in);
+        const float hs = fmaf(cP, h_in, cH), Ps = cP * P_in;
+        if (ok && cv) chain_put(ch, slot, chunk, hs, Ps);
+        float hq = h_in;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) { in_h[q][tid] = hq; hq = fmaf(agg_P[q][tid], hq, agg_h[q][tid]); }
         if (ok && cv) {
-            if (chunk + 1 < nchunk) chain_put(ch, slot, chunk, hs, Ps);
-            else if (!SAVE) {
+            if (!SAVE && chunk + 1 == nchunk) {
                 a.h_T[(size_t)b * D + d] = hs;
                 if (a.a_prod) a.a_prod[(size_t)b * D + d] = Ps;
                 // the last three raw inputs of concat(conv_state_in, x), bit-exact
@@ -518,16 +521,20 @@ __global__ void __launch_bounds__(NT) generic_bwd_scan_kernel(BwdArgs q, Chain c
     if (seg == 0) {
         uint4 *slot = ch.slot + (size_t)b * D + dc;
         // past the last token g holds the gradient arriving on h_T (h_T = h_{T-1}, so it is carried with factor 1)
+        float cQ = 1.0f, cG = 0.0f;   // the chunk as one step, before the wait
+#pragma unroll
+        for (int k = 7; k >= 0; --k) { cG = fmaf(agg_Q[k][lane], cG, agg_g[k][lane]); cQ *= agg_Q[k][lane]; }
         float X = 0.0f, unused;
         bool ok = true;
         if (link == 0) X = q.dh_T ? q.dh_T[(size_t)b * D + dc] : 0.0f;
         else ok = chain_wait(ch, slot, cv, link - 1, X, unused);
+        const float Xout = fmaf(cQ, X, cG);
+        if (ok && cv) {
+            chain_put(ch, slot, link, Xout, 0.0f);
+            if (chunk == 0 && q.dh0) q.dh0[(size_t)b * D + d] = Xout;   // a_0 g_0: h0 enters Eq. 4 only at t = 0
+        }
 #pragma unroll
         for (int k = 7; k >= 0; --k) { in_g[k][lane] = X; X = fmaf(agg_Q[k][lane], X, agg_g[k][lane]); }
-        if (ok && cv) {
-            if (chunk > 0) chain_put(ch, slot, link, X, 0.0f);
-            else if (q.dh0) q.dh0[(size_t)b * D + d] = X;   // a_0 g_0: h0 enters Eq. 4 only at t = 0
-        }
         if (!ok) ok_s = 0;
     }
     __syncthreads();
@@ -572,7 +579,7 @@ template <typename IOT, int BM, bool VEC>
 __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_du_kernel(BwdArgs q, int ntile) {
     ptx::dependency_wait();
     using TL = Tile<BM>;
-    constexpr int TM = TL::TM, NH = TL::NH, EA = BM / 8;
+    constexpr int TM = TL::TM, NH = TL::NH, BK = TL::BK, EA = TL::TA;
     __shared__ __align__(16) TL s;
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
     const int Dh = q.D / q.H, D = q.D;
@@ -584,17 +591,17 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_du_kernel(Bw
     const bool arow = tok0 + am < ntok;
     const size_t aoff = (tok0 + (arow ? am : 0)) * D + d0 + koff;
     const int nkg = (Dh + BK - 1) / BK;   // slabs per gate
-    float av[EA], bv[TL::BN / 8];
+    float av[EA], bv[TL::EB];
     auto fetch = [&](int kc) {
         const int gate = kc >= nkg, k0 = (kc - gate * nkg) * BK;
         fetch_k<EA, VEC>((gate ? q.gi : q.r) + aoff + k0, arow, Dh - k0 - koff, av);
         const IOT *W = (const IOT *)(gate ? q.W_x : q.W_a) + ((size_t)head * Dh + k0) * Dh + n0;
-        fetch_rows<TL::BN, VEC>(W, (size_t)Dh, Dh - k0, Dh - n0, tid, bv);
+        fetch_rows<TL::BN, TL::EB, VEC>(W, (size_t)Dh, Dh - k0, Dh - n0, tid, bv);
     };
     auto stage = [&](int buf) {
 #pragma unroll
         for (int i = 0; i < EA; ++i) s.As[buf][koff + i][am] = av[i];
-        put_rows<TL::BN, VEC>(s.Bs[buf], tid, bv);
+        put_rows<TL::BN, TL::EB, VEC>(s.Bs[buf], tid, bv);
     };
     f32x2 acc[TM][NH];
 #pragma unroll
@@ -633,7 +640,7 @@ template <int BM, bool VEC>
 __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_dw_kernel(BwdArgs q, int mtile, int ntile) {
     ptx::dependency_wait();
     using TL = Tile<BM>;
-    constexpr int TM = TL::TM, NH = TL::NH;
+    constexpr int TM = TL::TM, NH = TL::NH, BK = TL::BK;
     __shared__ __align__(16) TL s;
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
     const int Dh = q.D / q.H, D = q.D;
@@ -645,15 +652,15 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_bwd_dw_kernel(Bw
     const size_t ntok = (size_t)q.B * q.T, per = (ntok + q.S - 1) / q.S;
     const size_t lo = (size_t)split * per, hi = lo + per < ntok ? lo + per : ntok;
     const float *dz = (gate ? q.gi : q.r) + d0 + m0, *u = q.u + d0 + n0;
-    float av[BM / 8], bv[TL::BN / 8];
+    float av[TL::TA], bv[TL::EB];
     auto fetch = [&](size_t k0) {
         const int rows = (int)(hi - k0 < (size_t)BK ? hi - k0 : (size_t)BK);
-        fetch_rows<BM, VEC>(dz + k0 * D, (size_t)D, rows, Dh - m0, tid, av);
-        fetch_rows<TL::BN, VEC>(u + k0 * D, (size_t)D, rows, Dh - n0, tid, bv);
+        fetch_rows<BM, TL::TA, VEC>(dz + k0 * D, (size_t)D, rows, Dh - m0, tid, av);
+        fetch_rows<TL::BN, TL::EB, VEC>(u + k0 * D, (size_t)D, rows, Dh - n0, tid, bv);
     };
     auto stage = [&](int buf) {
-        put_rows<BM, VEC>(s.As[buf], tid, av);
-        put_rows<TL::BN, VEC>(s.Bs[buf], tid, bv);
+        put_rows<BM, TL::TA, VEC>(s.As[buf], tid, av);
+        put_rows<TL::BN, TL::EB, VEC>(s.Bs[buf], tid, bv);
     };
     f32x2 acc[TM][NH];
 #pragma unroll
