@@ -361,6 +361,186 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) sm100_d
     if (warp == 0) tmem_dealloc(tmem, TMEM_COLS);
 }
 
+// ------------------------------------------------------------------ few sequences
+// A step of a few sequences is a chain of latencies, and the kernel above has a long one: weight copies, U tile, hand-over to
+// the peer, 32 MMAs, accumulator read (5.3 us per step at B = 1 from a CUDA graph, 5.7 as launches).  Here up to eight CTAs (a
+// cluster) own a head, 32 of its channels each: a CTA's 64 gate rows wait in registers, as mma fragments, before the previous
+// kernel of the stream has finished; every CTA convolves all channels of the head itself, so nothing is exchanged; the products
+// are a handful of mma.sync of 16 rows (8 channels x 2 gates) x 8 sequences, K split over two warps.  The cluster barrier only
+// keeps a CTA from shifting its channels' conv state before its siblings have read it.  Precision as above: the gate products
+// take bf16(u), i_t u_t takes u (in fp32 here).
+constexpr int FS_THREADS = 256;
+constexpr int FS_CH = 32;           // channels per CTA
+constexpr int FS_ROW = DH + 32;     // bf16 per row of u: 576 bytes, so that the eight lanes of a phase hit different banks
+
+__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ float fs_sigmoid(float z) { return __fdividef(1.0f, 1.0f + __expf(-z)); }
+
+template <int NB>   // sequences per batch tile: 8 or 16 (32: 5.8 us at B = 32 where two tiles of 16 take 4.4)
+__global__ void __launch_bounds__(FS_THREADS, 2) sm100_decode_few_kernel(FwdArgs f, int dh, int C) {
+    constexpr int NTILE = NB / 8, NIT = NB / 8;
+    __shared__ __align__(16) __nv_bfloat16 u_s[NB][FS_ROW];
+    __shared__ __align__(16) float u_own[NB][FS_CH];
+    __shared__ float4 red[4][NTILE][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, D = f.D, B = f.B;
+    const int rank = (int)cluster_ctarank(), item = blockIdx.x / C, head = item % f.H, b0 = (item / f.H) * NB;
+    const int ngroup = dh >> 5, nchunk = dh >> 3, cbase = head * dh;
+    // product: warp (mt, kh) takes channels 8 mt .. + 7 of the CTA and every second group of 32 input channels; a thread holds 16
+    // bytes of a row (K is permuted alike in both operands: the mma sums over it)
+    const int mt = warp >> 1, kh = warp & 1, g = lane >> 2, t = lane & 3;
+    const int d = cbase + rank * FS_CH + mt * 8 + g;
+    uint4 wa[4], wx[4];
+    float lam = 0.0f, ba = 0.0f, bx = 0.0f;
+    {
+        const uint4 *ra = (const uint4 *)((const __nv_bfloat16 *)f.W_a + (size_t)d * dh), *rx = (const uint4 *)((const __nv_bfloat16 *)f.W_x + (size_t)d * dh);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int grp = kh + 2 * j;
+            wa[j] = grp < ngroup ? ra[grp * 4 + t] : make_uint4(0u, 0u, 0u, 0u);
+            wx[j] = grp < ngroup ? rx[grp * 4 + t] : make_uint4(0u, 0u, 0u, 0u);
+        }
+        lam = f.lambda[d]; ba = f.b_a[d]; bx = f.b_x[d];
+    }
+    // conv: thread (8-channel chunk c, sequences bi, bi + 8, ...)
+    const int c = lane, bi = warp, cd = cbase + c * 8;
+    const bool cexists = c < nchunk;
+    uint4 tap[4];
+    float cb[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) tap[j] = cexists ? *(const uint4 *)((const __nv_bfloat16 *)f.conv_w + (size_t)j * D + cd) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) cb[e] = f.conv_b && cexists ? f.conv_b[cd + e] : 0.0f;
+    const float zl = -lam, s = f.c * (zl > 0.0f ? zl + log1pf(expf(-zl)) : log1pf(expf(zl)));
+    dependency_wait();   // everything above reads only parameters
+
+    const __nv_bfloat16 *x = (const __nv_bfloat16 *)f.x;
+    __nv_bfloat16 *cs = (__nv_bfloat16 *)f.cs_out;   // in/out
+    float *h = f.h_T;                                 // in/out
+    uint4 xv[NIT], r0[NIT], r1[NIT], r2[NIT];
+#pragma unroll
+    for (int i = 0; i < NIT; ++i) {
+        const int b = b0 + bi + 8 * i;
+        xv[i] = r0[i] = r1[i] = r2[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (b < B && cexists) {
+            xv[i] = *(const uint4 *)(x + (size_t)b * D + cd);
+            r0[i] = *(const uint4 *)(cs + ((size_t)b * 3 + 0) * D + cd);
+            r1[i] = *(const uint4 *)(cs + ((size_t)b * 3 + 1) * D + cd);
+            r2[i] = *(const uint4 *)(cs + ((size_t)b * 3 + 2) * D + cd);
+        }
+    }
+    // the thread finishes channel d of sequences 2 t, 2 t + 1 of the sequence tiles its warp owns (alternate ones)
+    constexpr int OWN = NTILE > 1 ? NTILE / 2 : 1;
+    const bool finishes = NTILE > 1 || kh == 0;
+    float hv[OWN][2];
+#pragma unroll
+    for (int i = 0; i < OWN; ++i) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const int b = b0 + (NTILE > 1 ? 2 * i + kh : 0) * 8 + 2 * t + e;
+            hv[i][e] = finishes && b < B ? h[(size_t)b * D + d] : 0.0f;
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < NIT; ++i) {
+        const int n = bi + 8 * i;
+        if (c < nchunk) {
+            const uint32_t xw[4] = {xv[i].x, xv[i].y, xv[i].z, xv[i].w}, a0[4] = {r0[i].x, r0[i].y, r0[i].z, r0[i].w},
+                           a1[4] = {r1[i].x, r1[i].y, r1[i].z, r1[i].w}, a2[4] = {r2[i].x, r2[i].y, r2[i].z, r2[i].w};
+            const uint32_t w0[4] = {tap[0].x, tap[0].y, tap[0].z, tap[0].w}, w1[4] = {tap[1].x, tap[1].y, tap[1].z, tap[1].w},
+                           w2[4] = {tap[2].x, tap[2].y, tap[2].z, tap[2].w}, w3[4] = {tap[3].x, tap[3].y, tap[3].z, tap[3].w};
+            float u[8];
+            uint32_t o[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                float ul = cb[2 * e], uh = cb[2 * e + 1];
+                ul = fmaf(bf_lo(w0[e]), bf_lo(xw[e]), ul); uh = fmaf(bf_hi(w0[e]), bf_hi(xw[e]), uh);
+                ul = fmaf(bf_lo(w1[e]), bf_lo(a2[e]), ul); uh = fmaf(bf_hi(w1[e]), bf_hi(a2[e]), uh);
+                ul = fmaf(bf_lo(w2[e]), bf_lo(a1[e]), ul); uh = fmaf(bf_hi(w2[e]), bf_hi(a1[e]), uh);
+                ul = fmaf(bf_lo(w3[e]), bf_lo(a0[e]), ul); uh = fmaf(bf_hi(w3[e]), bf_hi(a0[e]), uh);
+                u[2 * e] = ul; u[2 * e + 1] = uh;
+                o[e] = pack_bf16(ul, uh);
+            }
+            *(uint4 *)&u_s[n][c * 8] = make_uint4(o[0], o[1], o[2], o[3]);
+            if (c >= rank * (FS_CH / 8) && c < (rank + 1) * (FS_CH / 8)) {
+                float *dst = &u_own[n][(c - rank * (FS_CH / 8)) * 8];
+                *(float4 *)dst = make_float4(u[0], u[1], u[2], u[3]);
+                *(float4 *)(dst + 4) = make_float4(u[4], u[5], u[6], u[7]);
+            }
+        }
+    }
+    __syncthreads();
+    cluster_arrive();    // this CTA has read the conv state of the whole head
+    float acc[NTILE][4];
+#pragma unroll
+    for (int nt = 0; nt < NTILE; ++nt) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[nt][e] = 0.0f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int grp = kh + 2 * j;
+            if (grp < ngroup) {
+                const uint4 ub = *(const uint4 *)&u_s[nt * 8 + g][grp * 32 + t * 8];
+                mma_bf16(acc[nt], wa[j].x, wx[j].x, wa[j].y, wx[j].y, ub.x, ub.y);
+                mma_bf16(acc[nt], wa[j].z, wx[j].z, wa[j].w, wx[j].w, ub.z, ub.w);
+            }
+        }
+        if (NTILE > 1 ? (nt & 1) != kh : kh == 1) red[mt][nt][lane] = make_float4(acc[nt][0], acc[nt][1], acc[nt][2], acc[nt][3]);
+    }
+    dependency_trigger();
+    __syncthreads();     // the other half of K
+#pragma unroll
+    for (int i = 0; i < OWN; ++i) {
+        if (finishes) {
+            const int nt = NTILE > 1 ? 2 * i + kh : 0;
+            const float4 o = red[mt][nt][lane];
+            constexpr int LAST = NTILE - 1;
+            float z[4];   // the accumulator of tile nt, picked without a dynamic register index
+#pragma unroll
+            for (int e = 0; e < 4; ++e) z[e] = NTILE > 1 && kh ? acc[2 * i + 1 < NTILE ? 2 * i + 1 : LAST][e] : acc[2 * i < NTILE ? 2 * i : LAST][e];
+            z[0] += o.x; z[1] += o.y; z[2] += o.z; z[3] += o.w;   // z_a of sequences 2 t, 2 t + 1, then z_x
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int n = nt * 8 + 2 * t + e, b = b0 + n;
+                if (b < B) {
+                    const float r = fs_sigmoid(z[e] + ba), gi = fs_sigmoid(z[2 + e] + bx), L = -s * r;
+                    const float a = expf(L), m = sqrtf(fmaxf(0.0f, -expm1f(2.0f * L)));
+                    const float hn = fmaf(a, hv[i][e], m * (gi * u_own[n][mt * 8 + g]));
+                    h[(size_t)b * D + d] = hn;
+                    ((__nv_bfloat16 *)f.y)[(size_t)b * D + d] = __float2bfloat16_rn(hn);
+                }
+            }
+        }
+    }
+    cluster_wait();      // all CTAs of the head have read its conv state: shift this CTA's channels by one row, bit-exact
+    if (cexists && c >= rank * (FS_CH / 8) && c < (rank + 1) * (FS_CH / 8)) {
+#pragma unroll
+        for (int i = 0; i < NIT; ++i) {
+            const int b = b0 + bi + 8 * i;
+            if (b < B) {
+                *(uint4 *)(cs + ((size_t)b * 3 + 0) * D + cd) = r1[i];
+                *(uint4 *)(cs + ((size_t)b * 3 + 1) * D + cd) = r2[i];
+                *(uint4 *)(cs + ((size_t)b * 3 + 2) * D + cd) = xv[i];
+            }
+        }
+    }
+}
+
+cudaError_t decode_few(const FwdArgs &a, int C, int NB, cudaStream_t st) {
+    const int dh = a.D / a.H;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(a.H * C * ((a.B + NB - 1) / NB))); cfg.blockDim = dim3(FS_THREADS); cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)C; attr[1].val.clusterDim.y = 1; attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 2;
+    return NB == 8 ? cudaLaunchKernelEx(&cfg, sm100_decode_few_kernel<8>, a, dh, C) : cudaLaunchKernelEx(&cfg, sm100_decode_few_kernel<16>, a, dh, C);
+}
+
 int num_sms() {
     int dev = 0, n = 0;
     if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) return n;
@@ -381,6 +561,13 @@ bool sm100_decode_supported(int B, int D, int H, int io) {
 }
 
 cudaError_t sm100_decode(const FwdArgs &a, cudaStream_t st) {
+    {
+        // Two blocks of the few-sequences kernel fit an SM.  While all of a step fit at once it is the faster kernel (D 2560, ten
+        // heads of 256: 3.0 against 5.7 us at B = 1, 4.0 / 6.0 at 16, 4.7 / 5.9 at 48); a second round of blocks costs a whole
+        // step more (8.6 / 6.2 at 56).
+        const int C = (a.D / a.H + FS_CH - 1) / FS_CH, NB = a.B <= 8 ? 8 : 16;
+        if ((long long)a.H * C * ((a.B + NB - 1) / NB) <= 2ll * num_sms()) return decode_few(a, C, NB, st);
+    }
     static PerDeviceOptIn opt_in;
     cudaError_t e = opt_in.ensure(sm100_decode_kernel, (int)SMEM_ALLOC);
     if (e != cudaSuccess) return e;

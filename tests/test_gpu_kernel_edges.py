@@ -78,6 +78,58 @@ def test_wide_heads_with_gate_branch_and_decay_product(oracle):
     assert_close("y", to_np(y), yr, "bf16"); assert_close("h_T", to_np(hT), hr, "bf16"); assert_close("a_prod", to_np(ap), apr, "bf16")
 
 
+@pytest.mark.parametrize("B,Dh,H", [(1, 256, 1), (8, 160, 3), (9, 32, 2), (16, 96, 2), (17, 224, 2), (48, 256, 10), (49, 256, 10), (64, 96, 16)])
+def test_decode_step_at_the_edges_of_its_two_kernels(oracle, B, Dh, H):
+    """Batch tiles of 8 and 16 sequences with remainders, widths that leave a cluster of one to eight blocks, and the batch at
+    which the step changes kernels; state in place, biases, several steps."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    T0, steps, D = 2, 3, Dh * H
+    inp = synth.make_inputs(B, T0 + steps, D, H, io="bf16", seed=50 + B, bias_scale=0.3)
+    params = binding.Params.from_numpy(inp["params"], "bf16")
+    x = to_dev(inp["x"], "bf16")
+    _, h, cs = binding.prefill(x[:, :T0].contiguous(), params)
+    ys = [binding.decode_step(x[:, t].contiguous(), params, h, cs) for t in range(T0, T0 + steps)]
+    torch.cuda.synchronize()
+    yr, hr, cr = oracle_prefill(oracle, inp)
+    assert_close("y", np.stack([to_np(v) for v in ys], 1), yr[:, T0:], "bf16")
+    assert_close("h", to_np(h), hr, "bf16")
+    assert np.array_equal(to_np(cs), cr)
+
+
+def test_replayed_graph_of_chained_chunks(oracle):
+    """A CUDA graph replays a call with the tags of its capture: records that the first replay left in the workspace must not be
+    taken for those of the second, which works on other inputs."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    for io, Dh, flags in (("f32", 64, GENERIC), ("bf16", 288, 0)):
+        B, T, H = 1, 700, 1
+        first, second = [synth.make_inputs(B, T, Dh * H, H, io=io, seed=60 + k, with_dy=True) for k in range(2)]
+        params = binding.Params.from_numpy(first["params"], io)
+        x, dy = to_dev(first["x"], io), to_dev(first["dy"], io)
+        shape = binding.make_shape(B, T, Dh * H, H, x.dtype, flags=flags)
+        ws, wsb = [binding.alloc_workspace(shape, op, x.device) for op in (binding.OP_PREFILL, binding.OP_BACKWARD)]
+        y = torch.empty_like(x)
+        stream = torch.cuda.Stream()
+        with torch.cuda.stream(stream):
+            binding.prefill(x, params, y=y, workspace=ws, flags=flags)   # first use outside the capture
+            binding.backward(x, params, dy, y=y, workspace=wsb, flags=flags)
+            stream.synchronize()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream):
+                binding.prefill(x, params, y=y, workspace=ws, flags=flags)
+                g = binding.backward(x, params, dy, y=y, workspace=wsb, flags=flags)
+            graph.replay()
+            x.copy_(to_dev(second["x"], io)); dy.copy_(to_dev(second["dy"], io))
+            graph.replay()
+        torch.cuda.synchronize()
+        second["params"] = first["params"]
+        yr, _, _ = oracle_prefill(oracle, second)
+        gr = oracle.backward(second["x"].astype(np.float64), f64(first["params"]), H, second["dy"].astype(np.float64))
+        assert_close("y", to_np(y), yr, io)
+        assert_close("dx", to_np(g["x"]), gr["x"], io, scale=max(1.0, float(np.abs(gr["x"]).max())) if io == "f32" else 1.0)
+
+
 @pytest.mark.parametrize("change,error", [
     (dict(h0=lambda t: t.double()), ValueError), (dict(x=lambda t: t.transpose(0, 1)), ValueError), (dict(workspace=lambda t: t[:128]), RuntimeError),
     (dict(flags=lambda v: 1 << 40), RuntimeError), (dict(conv_state_in=lambda t: t.cpu()), ValueError)])
