@@ -61,7 +61,7 @@ constexpr uint32_t Y_BUF_BYTES = TILE * 32 * 2;            // 4096: one scan war
 constexpr uint32_t SMEM_Y = SMEM_X + XS * X_SLAB_BYTES;    // bf16 y_s[4 warps][2 buffers][64][32], staged for tiled stores
 constexpr uint32_t SMEM_AGG = SMEM_Y + 4 * 2 * Y_BUF_BYTES;   // float2 agg_s[2 buffers][2 half tiles][128 channels]
 constexpr uint32_t SMEM_BAR = SMEM_AGG + 2 * 2 * CH * 8;
-constexpr int NUM_BARS = 2 * XS + 2 * US + 4 + 8 + 1 + 8;
+constexpr int NUM_BARS = 2 * XS + 2 * US + 4 + 8 + 1 + 8 + 2;
 constexpr uint32_t SMEM_MISC = SMEM_BAR + NUM_BARS * 8;    // tmem base, abort flag
 constexpr uint32_t SMEM_TOTAL = SMEM_MISC + 16;
 constexpr uint32_t SMEM_ALLOC = SMEM_TOTAL + 1024;         // slack for 1024-byte alignment
@@ -92,6 +92,7 @@ struct Sm100Args {
     // x as [B][T][D] with a box of SLAB_ROWS token rows x one head; y with a box of TILE rows x 32 channels
     alignas(64) CUtensorMap tm_x;
     alignas(64) CUtensorMap tm_y;
+    alignas(64) CUtensorMap tm_wa, tm_wx;   // the layer's weights as [D][dh], box 128 rows x 64 columns, 128-byte swizzle
     alignas(64) CUtensorMap tm_g;   // gate branch, same geometry as y (encoded only when the call has one; both then with boxes of HALF rows)
     FwdArgs f;
     int dh;            // width of a head of the layer, a multiple of 32 up to 256.  A "head" below is a group of k = 256 / dh
@@ -108,6 +109,62 @@ struct Sm100Args {
 };
 
 using namespace ptx;
+
+// Where the weights are staged on their way to tensor memory: 128 rows x 64 input channels of gate g, in U stages, x slots and y
+// buffers that the first two tiles do not use.
+static_assert(US >= 6 && XS >= 4 && U_STAGE_BYTES == 16384 && (SMEM_X + 2 * X_SLAB_BYTES) % 1024 == 0 && SMEM_Y % 1024 == 0 && 2 * X_SLAB_BYTES >= 32768 &&
+              8 * Y_BUF_BYTES >= 32768, "weight staging");
+__device__ __forceinline__ uint32_t weight_stage_off(int g, int kt) {
+    const int blk = g * 4 + kt;
+    return blk < 4 ? SMEM_U + 2 * U_STAGE_BYTES + (uint32_t)blk * 16384u : blk < 6 ? SMEM_X + 2 * X_SLAB_BYTES + (uint32_t)(blk - 4) * 16384u : SMEM_Y + (uint32_t)(blk - 6) * 16384u;
+}
+// Gate weights of a half-head into tensor memory, by warps 8 .. 15: lane = output channel, 32-bit column j holds input channels 2j
+// (low half) and 2j+1 (high half).  The tensor core multiplies them with the conv output u, which is kept in fp16 (11 significant
+// bits instead of bf16's 8, because u also enters i_t * u_t of Eq. 4 directly), and both operands of one MMA must have one type:
+// the bf16 weights are converted to fp16 here, which is exact for every weight of magnitude within [2^-14, 65504] and rounds
+// tinier ones to a multiple of 2^-24.
+// They come by tiled copies of 128 rows x 64 input channels.  (Each thread reading its own 512-byte row touched 32 sectors per
+// load: weights in place 5.2 us after the previous kernel's end, where the first conv tile is there after 3.4.)  The conversion
+// loop is rolled, because it runs once per launch and unrolled the fetch of its code was half of its time, and all of it is a
+// function of its own, because inlined it changed the register assignment of the gate warps' loop: B4 T4096 D4096 148 instead of
+// 146 us.  B1 T197 D2560: 12.0 -> 11.4 us; B3 T1213 width 160: 41.5 -> 39.9.
+__device__ __noinline__ bool stage_weights(const CUtensorMap *tm_wa, const CUtensorMap *tm_wx, int D, int dh, unsigned long long spin, uint8_t *smem, uint32_t base,
+                                           int rank, int cbase, int cvalid, uint32_t tmem, uint32_t bar, volatile int *abort_flag) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, g = (warp - 8) >> 2;
+    if (warp == 8 && lane == 0) {
+        const int ktiles = (dh + 63) >> 6, row0 = cbase + rank * CH;
+        if (row0 < D) {
+            mbar_expect_tx(bar, (uint32_t)(2 * ktiles) * 16384u);
+            for (int kt = 0; kt < ktiles; ++kt) {
+                tma_load_3d(base + weight_stage_off(0, kt), tm_wa, kt * 64, row0, 0, bar);
+                tma_load_3d(base + weight_stage_off(1, kt), tm_wx, kt * 64, row0, 0, bar);
+            }
+        } else mbar_arrive(bar);   // a last group whose channels all belong to the other CTA
+    }
+    __syncwarp();
+    // Narrower heads run as groups that fill the 256 x 256 block: the block is then block-diagonal, and a row holds its own head's
+    // weights in that head's input channels (16-byte chunks c_first .. + c_count - 1; none for a slot that does not exist) and zeros
+    // elsewhere.
+    const int row = q * 32 + lane, row_in_group = rank * CH + row;
+    const int sub = row_in_group / dh;
+    const int c_first = sub * (dh >> 3), c_count = row_in_group < cvalid ? dh >> 3 : 0;
+    const bool w_ok = warp_wait(bar, 0, spin, abort_flag);
+    const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (g ? TM_W_X : TM_W_A);
+    auto cvt2 = [](uint32_t w) { return pack_f16_sat(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); };
+    const uint8_t *src = smem + (uint32_t)row * 128u;
+    const uint32_t sw = ((uint32_t)row & 7u) << 4;
+    auto chunk = [&](int cc) -> uint4 {
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if ((uint32_t)cc < (uint32_t)c_count) v = *(const uint4 *)(src + weight_stage_off(g, cc >> 3) + ((((uint32_t)cc & 7u) << 4) ^ sw));
+        return make_uint4(cvt2(v.x), cvt2(v.y), cvt2(v.z), cvt2(v.w));
+    };
+#pragma unroll 1
+    for (int c = 0; c < 16; ++c) tmem_st8(taddr + c * 8, chunk(2 * c - c_first), chunk(2 * c + 1 - c_first));
+    tmem_st_wait();
+    tc_fence_before();
+    __syncwarp();
+    return w_ok;
+}
 
 // MERGED: the call has a gate branch and writes y_t = h_t GeLU(branch_t); a separate instantiation so that the plain forward
 // carries none of its code.  GeLU triples the scan warps' work per element, so there are eight of them, half a tile each (four
@@ -129,6 +186,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
     auto BAR_GDONE = [&](int bf, int q) { return bar0 + 8u * (2 * XS + 2 * US + 4 + bf * 4 + q); };
     const uint32_t BAR_WREADY = bar0 + 8u * (2 * XS + 2 * US + 12);               // leader CTA only: both CTAs' weights are in tensor memory
     auto BAR_BRANCH = [&](int w) { return bar0 + 8u * (2 * XS + 2 * US + 13 + w); };   // scan warp w's block of the gate branch has landed
+    const uint32_t BAR_WLOAD = bar0 + 8u * (2 * XS + 2 * US + 21), BAR_WDONE = BAR_WLOAD + 8;   // weights staged in shared memory; read out of it again
     uint32_t *tmem_base_s = (uint32_t *)(smem + SMEM_MISC);
     volatile int *abort_flag = (volatile int *)(smem + SMEM_MISC + 4);
 
@@ -188,12 +246,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
             for (int q = 0; q < 4; ++q) mbar_init(BAR_GDONE(bf, q), 2);
         }
         mbar_init(BAR_WREADY, 16);
+        mbar_init(BAR_WLOAD, 1); mbar_init(BAR_WDONE, 8);
         for (int w = 0; w < 8; ++w) mbar_init(BAR_BRANCH(w), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 5) { tmem_alloc2(smem_u32(tmem_base_s), 512); tmem_relinquish2(); }
-    if (warp == 4 && lane == 0) { prefetch_tensormap(&p.tm_x); prefetch_tensormap(&p.tm_y); }
+    if (warp == 4 && lane == 0) { prefetch_tensormap(&p.tm_x); prefetch_tensormap(&p.tm_wa); prefetch_tensormap(&p.tm_wx); prefetch_tensormap(&p.tm_y); }
     tc_fence_before();
     cluster_arrive();   // the peer's barriers must exist before anything arrives on them
     cluster_wait();
@@ -202,38 +261,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
     tc_fence_after();
     const uint32_t tmem = *tmem_base_s;
 
-    // Gate weights of this half-head into tensor memory: lane = output channel, 32-bit column j holds
-    // input channels 2j (low half) and 2j+1 (high half).  The tensor core multiplies them with the conv output
-    // u, which is kept in fp16 (11 significant bits instead of bf16's 8, because u also enters i_t * u_t of
-    // Eq. 4 directly), and both operands of one MMA must have one type: the bf16 weights are converted to
-    // fp16 here, which is exact for every weight of magnitude within [2^-14, 65504] and rounds tinier ones
-    // to a multiple of 2^-24.
+    // only the MMA issuers wait for the weights: loads and the conv of the first tiles run meanwhile
     if (warp >= 8 && warp < 16) {
-        const int q = warp & 3, g = (warp - 8) >> 2;  // g = 0: W_a, 1: W_x
-        const __nv_bfloat16 *W = (const __nv_bfloat16 *)(g ? f.W_x : f.W_a);
-        // Narrower heads (128 or 64 channels) run as groups of 2 or 4 heads that fill the 256 x 256 block: the block is then
-        // block-diagonal, and a row holds its own head's weights in that head's input channels and zeros elsewhere.
-        const int dh = p.dh, row_in_group = (int)rank * CH + q * 32 + lane;
-        const int sub = row_in_group / dh;                     // head of the group this output channel belongs to
-        const uint4 *row = (const uint4 *)(W + ((size_t)cbase + row_in_group) * dh);   // (head * 256 / dh + sub) * dh + row_in_group % dh rows of dh
-        // the 16-byte chunks of the 256 input channels that are this head's (none for a channel slot that does not exist)
-        const int c_first = sub * (dh >> 3), c_count = row_in_group < cvalid ? dh >> 3 : 0;
-        const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + (g ? TM_W_X : TM_W_A);
-        auto cvt2 = [](uint32_t w) { return pack_f16_sat(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); };
-        const uint4 zero4 = make_uint4(0u, 0u, 0u, 0u);
-#pragma unroll 4
-        for (int c = 0; c < 16; ++c) {
-            const int c0 = 2 * c - c_first, c1 = c0 + 1;
-            uint4 lo = (c0 >= 0 && c0 < c_count) ? __ldg(row + c0) : zero4, hi = (c1 >= 0 && c1 < c_count) ? __ldg(row + c1) : zero4;
-            lo.x = cvt2(lo.x); lo.y = cvt2(lo.y); lo.z = cvt2(lo.z); lo.w = cvt2(lo.w);
-            hi.x = cvt2(hi.x); hi.y = cvt2(hi.y); hi.z = cvt2(hi.z); hi.w = cvt2(hi.w);
-            tmem_st8(taddr + c * 8, lo, hi);
+        const bool w_ok = stage_weights(&p.tm_wa, &p.tm_wx, D, p.dh, spin, smem, base, (int)rank, cbase, cvalid, tmem, BAR_WLOAD, abort_flag);
+        if (lane == 0) {
+            if (!w_ok) record_timeout();
+            mbar_arrive(BAR_WDONE);
+            mbar_arrive_at(BAR_WREADY, 0);
         }
-        tmem_st_wait();
-        // only the MMA issuers wait for the weights: loads and the conv of the first tiles run meanwhile
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_at(BAR_WREADY, 0);
     }
 
     // Register budget per warpgroup (the four warps of a group execute the same setmaxnreg; the increases draw on
@@ -272,6 +307,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
         for (int it = 0; it < n_my_tiles; ++it) {
             const int st = it % US, slot = it % XS;
             ok = warp_wait_far(BAR_UEMPTY(st), ((it / US) & 1) ^ 1, spin, abort_flag);
+            if (it == 2) ok = ok && warp_wait(BAR_WDONE, 0, spin, abort_flag);   // the weights were staged in U stages 2 .. 5
             if (!ok) break;
             ok = warp_wait(BAR_XFULL(slot), (it / XS) & 1, spin, abort_flag);
             if (!ok) break;
@@ -333,6 +369,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
         for (int it = 0; it < n_my_tiles; tile_next(it, b, ti), ++it) {
             const int slot = it % XS;
             ok = warp_wait_far(BAR_XEMPTY(slot), ((it / XS) & 1) ^ 1, spin, abort_flag);
+            if (it == 2) ok = ok && warp_wait(BAR_WDONE, 0, spin, abort_flag);   // and in x slots 2 and 3
             if (!ok) break;
             const int ts0 = ti * TILE + (int)rank * HALF;   // first token this CTA convolves
             const uint32_t dst = base + SMEM_X + slot * X_SLAB_BYTES;
@@ -506,9 +543,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
         float P_prev_own = 1.0f;  // prod of a_t from the start of the sequence to the end of this pair's previous tile
         constexpr bool merged = MERGED;
         bool ok = true;
+        if constexpr (merged) ok = warp_wait(BAR_WDONE, 0, spin, abort_flag);   // and in the y buffers, where the branch arrives
+        const int n_scan = !merged || ok ? n_my_tiles : 0;
         int b, ti;
         tile_first(b, ti);
-        for (int it = 0; it < n_my_tiles; tile_next(it, b, ti), ++it) {
+        for (int it = 0; it < n_scan; tile_next(it, b, ti), ++it) {
             const bool shared = it < n_shared;
             const int gidx = (b - B_whole) * p.tps + ti;   // index of the tile's carry record (shared tiles only)
             const int t0 = ti * TILE;
@@ -661,7 +700,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
                 for (int kk = 0; kk < 3; ++kk) cs_out[((size_t)b * 3 + kk) * D + d] = keep[kk];
             }
         }
-        if (lane == 0) bulk_wait0();
+        if (lane == 0) bulk_wait_read0();   // shared memory has been read; the writes complete with the kernel
         ok = __all_sync(0xffffffffu, ok);
         if (!ok && lane == 0) record_timeout();
     }
@@ -822,6 +861,9 @@ cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes,
     if ((e = device_info(&di)) != cudaSuccess) return e;
     Sm100Args p;
     if (!make_activation_map(&p.tm_x, a.x, a.B, a.T, a.D, DH, SLAB_ROWS) || !make_activation_map(&p.tm_y, a.y, a.B, a.T, a.D, 32, a.gate_branch ? HALF : TILE))
+        return cudaErrorNotSupported;
+    if (!encode_bf16_map_3d(&p.tm_wa, a.W_a, (uint64_t)(a.D / a.H), (uint64_t)a.D, 1, 64, CH, true) ||
+        !encode_bf16_map_3d(&p.tm_wx, a.W_x, (uint64_t)(a.D / a.H), (uint64_t)a.D, 1, 64, CH, true))
         return cudaErrorNotSupported;
     if (a.gate_branch) {
         if (!make_activation_map(&p.tm_g, a.gate_branch, a.B, a.T, a.D, 32, HALF)) return cudaErrorNotSupported;
