@@ -15,10 +15,12 @@
 //                        and handed to the tensor core as MN-major operands (no transposed copies exist); fp32 partial sums
 //                        per split, reduced in fixed order
 //   6. Conv1D adjoint    dx, dconv_w, dconv_b with sliding windows, fixed-order reductions
-// h_{t-1} comes from the forward output y (bf16); when the caller has none the forward is run first.
+// h_{t-1} comes from the forward output y (bf16); when the caller has none, a forward scan over u and z makes it (between 2 and 3).
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <type_traits>
 
 #include "rglru_internal.h"
 #include "sm100_ptx.cuh"
@@ -31,7 +33,9 @@ using namespace ptx;
 
 constexpr int DH = 256;
 constexpr int SCAN_CHUNK = 64;             // tokens per block of the reverse scan (eight warps x eight tokens)
-constexpr int CONV_CHUNK = 32;             // tokens per thread of the two Conv1D kernels
+constexpr int CONV_SEG = 32;               // tokens per thread of the two Conv1D kernels ...
+constexpr int CONV_CHUNK = 4 * CONV_SEG;   // ... and per block: 64 threads x 4 channels, four segments
+constexpr int CONV_CH = 256;
 constexpr float LOG2E = 1.44269504f;
 constexpr int GEMM_THREADS = 192;          // TMA warp, MMA warp, four epilogue warps
 constexpr int GEMM_STAGES = 4;
@@ -349,9 +353,18 @@ __device__ __forceinline__ f32x2 bf2x(uint32_t w) { return make_float2(__uint_as
 __device__ __forceinline__ f32x2 hf2x(uint32_t w) { return __half22float2(*(const __half2 *)&w); }
 __device__ __forceinline__ f32x2 ld2f(const float *p) { return *(const float2 *)p; }
 
+// four adjacent channels
+struct f32x4 { f32x2 a, b; };
+__device__ __forceinline__ f32x4 bf4x(uint2 w) { return f32x4{bf2x(w.x), bf2x(w.y)}; }
+__device__ __forceinline__ f32x4 hf4x(uint2 w) { return f32x4{hf2x(w.x), hf2x(w.y)}; }
+__device__ __forceinline__ f32x4 zero4() { return f32x4{pack2(0.f, 0.f), pack2(0.f, 0.f)}; }
+__device__ __forceinline__ f32x4 fma4(const f32x4 &x, const f32x4 &y, const f32x4 &z) { return f32x4{fma2(x.a, y.a, z.a), fma2(x.b, y.b, z.b)}; }
+__device__ __forceinline__ f32x4 mul4(const f32x4 &x, const f32x4 &y) { return f32x4{mul2(x.a, y.a), mul2(x.b, y.b)}; }
+
 // u_t = b_c + sum_j w[j] x_{t-j} of tokens [tb, tb + n) of sequences b0, b0 + 1, ... as u[sequence][n][D]: one thread per
-// (sequence, 32 tokens, two adjacent channels), forward in time, eight tokens' loads in flight.  Bound by its 4 bytes per
-// element.  grid (ceil(D/512), ceil(n/CONV_CHUNK), sequences)
+// (sequence, 32 tokens, four adjacent channels), forward in time, eight tokens' loads in flight.  Bound by its 4 bytes per
+// element: with two channels per thread and a predicate on every token it executed 26 instructions per element (66 % of the issue
+// slots) and took 66 us on B4 T4096 D4096.  grid (ceil(D/256), ceil(n/128), sequences)
 struct ConvArgs {
     int T, D, b0, tb, n;
     const __nv_bfloat16 *x, *conv_w, *cs_in;
@@ -359,39 +372,43 @@ struct ConvArgs {
     __half *u;
     uint32_t *epoch;
 };
-__global__ void __launch_bounds__(256, 6) conv_forward_kernel(ConvArgs a) {
+__global__ void __launch_bounds__(256, 4) conv_forward_kernel(ConvArgs a) {
     dependency_wait();
-    const int d = (blockIdx.x * 256 + threadIdx.x) * 2, b = a.b0 + blockIdx.z;
-    const int T = a.T, D = a.D, t0 = a.tb + blockIdx.y * CONV_CHUNK, t1 = min(a.tb + a.n, t0 + CONV_CHUNK);
+    const int d = blockIdx.x * CONV_CH + (threadIdx.x & 63) * 4, b = a.b0 + blockIdx.z;
+    const int T = a.T, D = a.D, t0 = a.tb + blockIdx.y * CONV_CHUNK + (threadIdx.x >> 6) * CONV_SEG, t1 = min(a.tb + a.n, t0 + CONV_SEG);
     // the scans' carry records are told apart from those an earlier launch with the same host tag (a graph replay) left behind
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *a.epoch += 1u;
-    if (d >= D) return;
-    f32x2 w[4];
+    if (d >= D || t0 >= t1) return;
+    f32x4 w[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] = bf2x(*(const uint32_t *)(a.conv_w + (size_t)j * D + d));
-    const f32x2 cb = a.conv_b ? ld2f(a.conv_b + d) : pack2(0.f, 0.f);
-    auto xat = [&](int t) -> f32x2 {
-        if (t >= 0) return bf2x(*(const uint32_t *)(a.x + ((size_t)b * T + t) * D + d));
-        return a.cs_in ? bf2x(*(const uint32_t *)(a.cs_in + ((size_t)b * 3 + (3 + t)) * D + d)) : pack2(0.f, 0.f);
+    for (int j = 0; j < 4; ++j) w[j] = bf4x(*(const uint2 *)(a.conv_w + (size_t)j * D + d));
+    const f32x4 cb = a.conv_b ? f32x4{ld2f(a.conv_b + d), ld2f(a.conv_b + d + 2)} : zero4();
+    auto xat = [&](int t) -> f32x4 {
+        if (t >= 0) return bf4x(*(const uint2 *)(a.x + ((size_t)b * T + t) * D + d));
+        return a.cs_in ? bf4x(*(const uint2 *)(a.cs_in + ((size_t)b * 3 + (3 + t)) * D + d)) : zero4();
     };
-    f32x2 x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
-    const uint32_t sD = (uint32_t)D / 2;   // token stride in channel pairs
-    const uint32_t *px = (const uint32_t *)(a.x + ((size_t)b * T + t0) * D + d);
-    uint32_t *pu = (uint32_t *)(a.u + ((size_t)blockIdx.z * a.n + (t0 - a.tb)) * D + d);
-    for (int t = t0; t < t1; t += 8) {
-        const int n = t1 - t;
-        uint32_t xs[8];
+    f32x4 x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
+    const uint32_t sD = (uint32_t)D / 4;   // token stride in groups of four channels
+    const uint2 *px = (const uint2 *)(a.x + ((size_t)b * T + t0) * D + d);
+    uint2 *pu = (uint2 *)(a.u + ((size_t)blockIdx.z * a.n + (t0 - a.tb)) * D + d);
+    auto token = [&](uint2 xw) {
+        const f32x4 x0 = bf4x(xw);
+        const f32x4 uv = fma4(w[3], x3, fma4(w[2], x2, fma4(w[1], x1, fma4(w[0], x0, cb))));
+        *pu = make_uint2(pack_f16_sat(uv.a.x, uv.a.y), pack_f16_sat(uv.b.x, uv.b.y));
+        pu += sD;
+        x3 = x2; x2 = x1; x1 = x0;
+    };
+    int t = t0;
+#pragma unroll 1
+    for (; t + 8 <= t1; t += 8) {
+        uint2 xs[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) xs[k] = k < n ? px[k * sD] : 0u;
+        for (int k = 0; k < 8; ++k) { xs[k] = *px; px += sD; }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            const f32x2 x0 = bf2x(xs[k]);
-            const f32x2 uv = fma2(w[3], x3, fma2(w[2], x2, fma2(w[1], x1, fma2(w[0], x0, cb))));
-            if (k < n) pu[k * sD] = pack_f16_sat(uv.x, uv.y);
-            x3 = x2; x2 = x1; x1 = x0;
-        }
-        px += 8 * (size_t)sD; pu += 8 * (size_t)sD;
+        for (int k = 0; k < 8; ++k) token(xs[k]);
     }
+#pragma unroll 1
+    for (; t < t1; ++t) { token(*px); px += sD; }
 }
 
 // 1 - exp(-x) for 0 <= x <= S_POLY without cancellation: x (1 - x/2 + x^2/6 - x^3/24 + x^4/120), relative truncation error < 1.5e-6
@@ -476,7 +493,7 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
     const int tid = threadIdx.x, lane = tid & 31, seg = tid >> 5;
     const int T = a.T, D = a.D, S = p.S, n = n0 + 2 * lane, d = group * a.hstride + n;
     const bool cv = n < a.hstride && d < D;
-    const uint32_t sD = (uint32_t)D / 2, sZ = (uint32_t)a.H * a.NS;   // token strides in channel pairs
+    const uint32_t sD = (uint32_t)D / 2, sZ = (uint32_t)a.H * a.NS, sN = (uint32_t)a.NS / 2;   // strides in channel pairs: tokens, gates
     const f32x2 ba = cv ? ld2f(a.b_a + d) : pack2(0.f, 0.f), bx = cv ? ld2f(a.b_x + d) : pack2(0.f, 0.f);
     const f32x2 nba = mul2(ba, pack2(-LOG2E, -LOG2E)), nbx = mul2(bx, pack2(-LOG2E, -LOG2E));
     const f32x2 ONE = pack2(1.0f, 1.0f), TWO = pack2(2.0f, 2.0f), NEG = pack2(-1.0f, -1.0f), ns2 = mul2(s2, NEG);
@@ -510,14 +527,18 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
         constexpr int TW = SCAN_TILE_BYTES / 4;
         f32x2 r[8], f[8];
         f32x2 Q = ONE, G = pack2(0.0f, 0.0f);
+        auto fold = [&](auto all) {   // all: all tokens of the chunk exist
 #pragma unroll
-        for (int k = 7; k >= 0; --k) {
-            gate_f2<POLY>(hf2x(sm[k * 32]), nba, s2, r[k], f[k]);
-            if (k >= nv) { r[k] = pack2(0.f, 0.f); f[k] = pack2(0.f, 0.f); }   // a token that does not exist passes the carry through (its dy reads as zero)
-            const f32x2 at = fma2(f[k], NEG, ONE);
-            G = mul2(at, __fadd2_rn(bf2x(sm[TW + k * 32]), G));
-            Q = mul2(Q, at);
-        }
+            for (int k = 7; k >= 0; --k) {
+                gate_f2<POLY>(hf2x(sm[k * 32]), nba, s2, r[k], f[k]);
+                if (!decltype(all)::value && k >= nv) { r[k] = pack2(0.f, 0.f); f[k] = pack2(0.f, 0.f); }   // a token that does not exist passes the carry through (its dy reads as zero)
+                const f32x2 at = fma2(f[k], NEG, ONE);
+                G = mul2(at, __fadd2_rn(bf2x(sm[TW + k * 32]), G));
+                Q = mul2(Q, at);
+            }
+        };
+        const bool whole = (chunk + 1) * SCAN_CHUNK <= T;
+        if (whole) fold(std::true_type{}); else fold(std::false_type{});
         sh.agg[0][seg][lane] = Q; sh.agg[1][seg][lane] = G;
         if (!ok) sh.abort = 1;
         __syncthreads();
@@ -555,8 +576,7 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
         }
         uint32_t *p_dz = (uint32_t *)(a.dz + ((size_t)b * T + t0) * (size_t)(2 * sZ) + (size_t)group * 2 * a.NS + n);
         uint32_t *p_du = (uint32_t *)(a.du + ((size_t)b * T + t0) * D + d);
-#pragma unroll
-        for (int k = 7; k >= 0; --k) {
+        auto adjoint = [&](auto all, int k) {
             const f32x2 u = hf2x(sm[3 * TW + k * 32]);
             f32x2 hp = bf2x(sm[4 * TW + k * 32]);
             if (k == 0 && t0 == 0 && a.h0 && cv) hp = ld2f(a.h0 + (size_t)b * D + d);
@@ -564,7 +584,8 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
             const f32x2 q = __fadd2_rn(pack2(ex2_approx(e.x), ex2_approx(e.y)), ONE);
             const f32x2 gi = pack2(rcp_approx(q.x), rcp_approx(q.y));
             const f32x2 at = fma2(f[k], NEG, ONE), m2 = mul2(f[k], fma2(f[k], NEG, TWO));
-            const f32x2 rm = pack2(m2.x > 0.0f ? rsqrt_fast(m2.x) : 0.0f, m2.y > 0.0f ? rsqrt_fast(m2.y) : 0.0f);   // 1 / sqrt(1 - a^2)
+            // 1 / sqrt(1 - a^2).  Where that is below 1e-15, r is below 1e-30 and makes dL r vanish as it should
+            const f32x2 rm = pack2(rsqrt_fast(fmaxf(m2.x, 1e-30f)), rsqrt_fast(fmaxf(m2.y, 1e-30f)));
             const f32x2 g = __fadd2_rn(bf2x(sm[TW + k * 32]), carry);
             carry = mul2(at, g);
             const f32x2 v = mul2(gi, u);
@@ -575,12 +596,19 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
             const f32x2 dzx = mul2(mul2(du, u), fma2(gi, NEG, ONE));
             s_lam = __fadd2_rn(s_lam, dLr);
             s_ba = __fadd2_rn(s_ba, dza); s_bx = __fadd2_rn(s_bx, dzx);      // tokens that do not exist add zeros (r = 0, u = 0)
-            if (k < nv) {
+            if (decltype(all)::value || k < nv) {
                 if (cv) p_du[k * sD] = pack_f16_sat(du.x, du.y);
                 // slots of this 64-slot block that do not exist get zeros: the du product multiplies the whole block
                 p_dz[k * sZ] = cv ? pack_f16_sat(dza.x, dza.y) : 0u;
-                p_dz[k * sZ + a.NS / 2] = cv ? pack_f16_sat(dzx.x, dzx.y) : 0u;
+                p_dz[k * sZ + sN] = cv ? pack_f16_sat(dzx.x, dzx.y) : 0u;
             }
+        };
+        if (whole) {
+#pragma unroll
+            for (int k = 7; k >= 0; --k) adjoint(std::true_type{}, k);
+        } else {
+#pragma unroll
+            for (int k = 7; k >= 0; --k) adjoint(std::false_type{}, k);
         }
         __syncthreads();   // everybody has read the stage and the segments' steps
         if (tid == 0 && link + 2 * S < a.nchunk) issue(link + 2 * S, st);
@@ -651,8 +679,9 @@ int scan_split(int columns, int nchunk, int slots) {
 }
 
 // Conv1D adjoint: dx_t = sum_j w[j] du_{t+j} (t + j < T); per-chunk partial sums of dw[j] = sum_t du_t x_{t-j} and
-// db_c = sum_t du_t.  One thread per (sequence, 32 tokens, two adjacent channels) walks forward with sliding windows, so that
-// every du and every x is loaded once.  Bound by its 6 bytes per element.  grid (ceil(D/512), ceil(T/CONV_CHUNK), B)
+// db_c = sum_t du_t.  One thread per (sequence, 32 tokens, four adjacent channels) walks forward with sliding windows, so that
+// every du and every x is loaded once; a block adds its four segments' sums.  Bound by its 6 bytes per element (two channels per
+// thread, a predicate on every token and sums per 32 tokens: 104 us on B4 T4096 D4096).  grid (ceil(D/256), ceil(T/128), B)
 struct ConvBwdArgs {
     int B, T, D;
     const __nv_bfloat16 *x, *conv_w, *cs_in;
@@ -661,48 +690,67 @@ struct ConvBwdArgs {
     float *part_conv;   // [B*chunks][5][D]
 };
 
-__global__ void __launch_bounds__(256, 4) conv_backward_kernel(ConvBwdArgs a) {
+__global__ void __launch_bounds__(256, 2) conv_backward_kernel(ConvBwdArgs a) {
+    __shared__ float4 red[3][5][64];
     dependency_wait();
-    const int d = (blockIdx.x * 256 + threadIdx.x) * 2, b = blockIdx.z;
-    const int T = a.T, D = a.D, t0 = blockIdx.y * CONV_CHUNK, t1 = min(T, t0 + CONV_CHUNK);
-    if (d >= D) return;
-    f32x2 w[4], sw[4], sb = pack2(0.f, 0.f);
+    const int c = threadIdx.x & 63, sg = threadIdx.x >> 6, d = blockIdx.x * CONV_CH + c * 4, b = blockIdx.z;
+    const int T = a.T, D = a.D, t0 = blockIdx.y * CONV_CHUNK + sg * CONV_SEG, t1 = min(T, t0 + CONV_SEG);
+    f32x4 sw[5];   // four taps, bias
 #pragma unroll
-    for (int j = 0; j < 4; ++j) { w[j] = bf2x(*(const uint32_t *)(a.conv_w + (size_t)j * D + d)); sw[j] = pack2(0.f, 0.f); }
-    auto xat = [&](int t) -> f32x2 {
-        if (t >= 0) return bf2x(*(const uint32_t *)(a.x + ((size_t)b * T + t) * D + d));
-        return a.cs_in ? bf2x(*(const uint32_t *)(a.cs_in + ((size_t)b * 3 + (3 + t)) * D + d)) : pack2(0.f, 0.f);
-    };
-    auto duat = [&](int t) -> f32x2 { return t < T ? hf2x(*(const uint32_t *)(a.du + ((size_t)b * T + t) * D + d)) : pack2(0.f, 0.f); };
-    f32x2 x1 = xat(t0 - 1), x2 = xat(t0 - 2), x3 = xat(t0 - 3);
-    f32x2 g0 = duat(t0), g1 = duat(t0 + 1), g2 = duat(t0 + 2);
-    const uint32_t sD = (uint32_t)D / 2;
-    for (int t = t0; t < t1; t += 4) {
-        const size_t row = ((size_t)b * T + t) * D + d;
-        const uint32_t *px = (const uint32_t *)(a.x + row), *pg = (const uint32_t *)(a.du + row);
-        uint32_t *pdx = (uint32_t *)(a.dx + row);
-        const int n = t1 - t, ng = T - t - 3;
-        uint32_t xs[4], gs[4];
+    for (int j = 0; j < 5; ++j) sw[j] = zero4();
+    if (d < D && t0 < t1) {
+        f32x4 w[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) { xs[k] = k < n ? px[k * sD] : 0u; gs[k] = k < ng ? pg[(k + 3) * sD] : 0u; }
+        for (int j = 0; j < 4; ++j) w[j] = bf4x(*(const uint2 *)(a.conv_w + (size_t)j * D + d));
+        auto xat = [&](int t) -> f32x4 {
+            if (t >= 0) return bf4x(*(const uint2 *)(a.x + ((size_t)b * T + t) * D + d));
+            return a.cs_in ? bf4x(*(const uint2 *)(a.cs_in + ((size_t)b * 3 + (3 + t)) * D + d)) : zero4();
+        };
+        const uint32_t sD = (uint32_t)D / 4;
+        const uint2 *px = (const uint2 *)(a.x + ((size_t)b * T + t0) * D + d), *pg = (const uint2 *)(a.du + ((size_t)b * T + t0) * D + d);
+        uint2 *pdx = (uint2 *)(a.dx + ((size_t)b * T + t0) * D + d);
+        f32x4 x1 = xat(t0 - 1), x2 = xat(t0 - 2), x3 = xat(t0 - 3);
+        f32x4 g0 = hf4x(pg[0]), g1 = t0 + 1 < T ? hf4x(pg[sD]) : zero4(), g2 = t0 + 2 < T ? hf4x(pg[2 * sD]) : zero4();
+        pg += 3 * (size_t)sD;
+        auto token = [&](uint2 xw, uint2 gw) {   // gw: du_{t+3}, zero bits past the end
+            const f32x4 x0 = bf4x(xw), g3 = hf4x(gw);
+            const f32x4 o = fma4(w[3], g3, fma4(w[2], g2, fma4(w[1], g1, mul4(w[0], g0))));
+            const __nv_bfloat162 oa = __floats2bfloat162_rn(o.a.x, o.a.y), ob = __floats2bfloat162_rn(o.b.x, o.b.y);
+            *pdx = make_uint2(*(const uint32_t *)&oa, *(const uint32_t *)&ob);
+            pdx += sD;
+            sw[0] = fma4(g0, x0, sw[0]); sw[1] = fma4(g0, x1, sw[1]); sw[2] = fma4(g0, x2, sw[2]); sw[3] = fma4(g0, x3, sw[3]);
+            sw[4].a = __fadd2_rn(sw[4].a, g0.a); sw[4].b = __fadd2_rn(sw[4].b, g0.b);
+            g0 = g1; g1 = g2; g2 = g3;
+            x3 = x2; x2 = x1; x1 = x0;
+        };
+        int t = t0;
+#pragma unroll 1
+        for (; t + 8 <= t1 && t + 11 <= T; t += 8) {
+            uint2 xs[8], gs[8];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            if (k < n) {
-                const f32x2 g3 = hf2x(gs[k]), x0 = bf2x(xs[k]);
-                const f32x2 o = fma2(w[3], g3, fma2(w[2], g2, fma2(w[1], g1, mul2(w[0], g0))));
-                const __nv_bfloat162 ob = __floats2bfloat162_rn(o.x, o.y);
-                pdx[k * sD] = *(const uint32_t *)&ob;
-                sw[0] = fma2(g0, x0, sw[0]); sw[1] = fma2(g0, x1, sw[1]); sw[2] = fma2(g0, x2, sw[2]); sw[3] = fma2(g0, x3, sw[3]);
-                sb = __fadd2_rn(sb, g0);
-                g0 = g1; g1 = g2; g2 = g3;
-                x3 = x2; x2 = x1; x1 = x0;
-            }
+            for (int k = 0; k < 8; ++k) { xs[k] = *px; px += sD; gs[k] = *pg; pg += sD; }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) token(xs[k], gs[k]);
+        }
+#pragma unroll 1
+        for (; t < t1; ++t) { token(*px, t + 3 < T ? *pg : make_uint2(0u, 0u)); px += sD; pg += sD; }
+    }
+    // segments added in order: run-to-run identical
+    if (sg > 0) {
+#pragma unroll
+        for (int j = 0; j < 5; ++j) red[sg - 1][j][c] = make_float4(sw[j].a.x, sw[j].a.y, sw[j].b.x, sw[j].b.y);
+    }
+    __syncthreads();
+    if (sg == 0 && d < D) {
+        float *pc = a.part_conv + ((size_t)(b * gridDim.y + blockIdx.y) * 5) * D + d;
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            float4 t = make_float4(sw[j].a.x, sw[j].a.y, sw[j].b.x, sw[j].b.y);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) { const float4 o = red[k][j][c]; t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w; }
+            *(float4 *)(pc + (size_t)j * D) = t;
         }
     }
-    float *pc = a.part_conv + ((size_t)(b * gridDim.y + blockIdx.y) * 5) * D + d;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) *(float2 *)(pc + (size_t)j * D) = sw[j];
-    *(float2 *)(pc + (size_t)4 * D) = sb;
 }
 
 inline size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
@@ -739,9 +787,25 @@ Groups make_groups(int D, int H) {
 
 struct BwdLayout {
     size_t BT, BTp, off_u, off_z, off_dz, off_du, off_y, off_hT, off_cs, off_rec, off_pvec, off_pconv, off_pdw,
-        off_w16, off_fws, total;
+        off_w16, total;
     int nchunk, nchunk_conv, S, kb_per_split;
 };
+
+// Token splits of the dW products.  A K block (48 KB per SM) takes ~0.6 us, a tile four of them more for filling and epilogue, and
+// each split's partial sums are written and read again at ~5 TB/s.  Counted in whole rounds of 148 SMs (whatever the device: the
+// workspace size has to agree with the launch): 2 splits for 16 heads of 256 (64 tiles a split; eight of them took four rounds
+// and 67 MB of partial sums, dW and its reduction 110 us on B4 T4096).
+int dw_split(const Groups &gr, int kblocks) {
+    const int tiles = gr.G * gr.nt * (2 * gr.NS / 128), most = kblocks < 16 ? kblocks : 16;
+    const double part_us = 2.0 * 2 * gr.G * gr.NS * gr.NS * 4 / 5e6;
+    int best = 1;
+    double best_us = 1e30;
+    for (int S = 1; S <= most; ++S) {
+        const double us = ((tiles * S + 147) / 148) * 0.6 * ((kblocks + S - 1) / S + 4) + S * part_us;
+        if (us < best_us) { best_us = us; best = S; }
+    }
+    return best;
+}
 
 BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     BwdLayout L{};
@@ -752,7 +816,7 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     L.nchunk = (T + SCAN_CHUNK - 1) / SCAN_CHUNK;
     L.nchunk_conv = (T + CONV_CHUNK - 1) / CONV_CHUNK;
     const int kblocks = (int)(L.BTp / 64);
-    L.S = kblocks < 8 ? kblocks : 8;
+    L.S = dw_split(gr, kblocks);
     L.kb_per_split = (kblocks + L.S - 1) / L.S;
     size_t o = 0;
     auto take = [&](size_t bytes) { const size_t at = o; o += up256(bytes); return at; };
@@ -768,7 +832,6 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     L.off_pconv = take((size_t)B * L.nchunk_conv * 5 * D * 4);
     L.off_pdw = take((size_t)L.S * 2 * gr.G * gr.NS * gr.NS * 4);
     L.off_w16 = take(gr.W16_bytes());
-    L.off_fws = take(gr.dh <= DH ? sm100_prefill_workspace_bytes(B, T, D, Hl) : sm100_wide_prefill_workspace_bytes(B, T, D, Hl));
     L.total = o;
     return L;
 }
@@ -921,6 +984,7 @@ __device__ __forceinline__ void wide_scan_column(const WideScanArgs &p, ScanShar
             X = fma2(sh.agg[0][k][lane], X, sh.agg[1][k][lane]);
             Pc = mul2(Pc, sh.agg[0][k][lane]);
         }
+        const uint32_t sD = (uint32_t)D / 2;
         uint32_t *p_y = (uint32_t *)((__nv_bfloat16 *)f.y + ((size_t)b * T + p.tb + t0) * D + d);
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
@@ -931,7 +995,7 @@ __device__ __forceinline__ void wide_scan_column(const WideScanArgs &p, ScanShar
             }
             if (cv && k < nv) {
                 const __nv_bfloat162 o = __floats2bfloat162_rn(y.x, y.y);
-                p_y[(size_t)k * (D / 2)] = *(const uint32_t *)&o;
+                p_y[k * sD] = *(const uint32_t *)&o;
             }
         }
         __syncthreads();   // everybody has read the stage and the segments' steps
@@ -982,6 +1046,32 @@ __global__ void __launch_bounds__(256, 2) wide_scan_kernel(const __grid_constant
     uint8_t *stage = smem_raw + (base - raw);
     if (__all_sync(0xffffffffu, s2.x <= S_POLY && s2.y <= S_POLY)) wide_scan_column<true>(p, sh, stage, base, bl, k0, group, tile * 64, s2);
     else wide_scan_column<false>(p, sh, stage, base, bl, k0, group, tile * 64, s2);
+}
+
+WideScanArgs wide_scan_args(const Groups &gr, const FwdArgs &f, uint4 *rec, uint32_t *epoch) {
+    WideScanArgs p{};
+    p.f = f;
+    p.G = gr.G; p.hstride = gr.hstride; p.NS = gr.NS; p.tiles = (gr.hstride + 63) / 64;
+    p.rec = rec; p.epoch = epoch;
+    p.tag = next_call_tag(); p.spin_ns = g_spin_limit_ns;
+    return p;
+}
+// The scan of one pass (p.b0, nb, tb, n) over its u and z
+cudaError_t run_wide_scan(WideScanArgs &p, const __half *u, const __half *z, cudaStream_t st) {
+    static PerDeviceOptIn opt_in;
+    cudaError_t e = opt_in.ensure(wide_scan_kernel, (int)WIDE_SMEM_ALLOC);
+    if (e != cudaSuccess) return e;
+    const uint64_t D = p.f.D, n = p.n, wz = (uint64_t)p.G * 2 * p.NS;
+    const uint64_t du[3] = {D, n, (uint64_t)p.nb}, su[2] = {D * 2, D * n * 2};
+    const uint64_t dz[3] = {wz, n, (uint64_t)p.nb}, sz[2] = {wz * 2, wz * n * 2};
+    const uint32_t box[3] = {64, SCAN_CHUNK, 1};
+    if (!encode_map16_3d(&p.tm_u, u, du, su, box, false) || !encode_map16_3d(&p.tm_z, z, dz, sz, box, false)) return cudaErrorNotSupported;
+    if (p.f.gate_branch && !encode_bf16_map_3d(&p.tm_g, p.f.gate_branch, D, (uint64_t)p.f.T, (uint64_t)p.f.B, 64, SCAN_CHUNK, false)) return cudaErrorNotSupported;
+    p.nchunk = (p.n + SCAN_CHUNK - 1) / SCAN_CHUNK;
+    p.S = scan_split(p.nb * p.G * p.tiles, p.nchunk, 2 * num_sms());
+    const size_t blocks = (size_t)p.nb * p.G * p.tiles * p.S;
+    if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    return launch_dependent(wide_scan_kernel, dim3((unsigned)blocks), dim3(256), WIDE_SMEM_ALLOC, st, p);
 }
 
 // Passes over the batch: whole sequences while they fit WIDE_TOKENS, else one sequence in pieces of that length
@@ -1035,22 +1125,10 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     __half *dz = (__half *)(ws + L.off_dz), *W16 = (__half *)(ws + L.off_w16);
     __half *du = (__half *)(ws + L.off_du);
 
-    // 0. h_{t-1} comes from the forward output; run the forward when the caller kept none
-    const void *y = y_saved;
-    if (y == nullptr) {
-        FwdArgs f = fwd;
-        f.y = ws + L.off_y; f.h_T = (float *)(ws + L.off_hT); f.cs_out = ws + L.off_cs;
-        f.status = status;
-        void *fws = ws + L.off_fws;
-        e = gr.dh <= DH ? sm100_prefill(f, fws, sm100_prefill_workspace_bytes(B, T, D, q.H), st) : sm100_wide_prefill(f, fws, sm100_wide_prefill_workspace_bytes(B, T, D, q.H), st);
-        if (e != cudaSuccess) return e;
-        y = f.y;
-    }
-
     EwArgs a{};
     a.B = B; a.T = T; a.D = D; a.H = H; a.nchunk = L.nchunk; a.c = q.c; a.hstride = hstride; a.NS = NS;
     a.x = (const __nv_bfloat16 *)q.x; a.conv_w = (const __nv_bfloat16 *)q.conv_w; a.cs_in = (const __nv_bfloat16 *)q.cs_in;
-    a.dy = (const __nv_bfloat16 *)q.dy; a.y = (const __nv_bfloat16 *)y;
+    a.dy = (const __nv_bfloat16 *)q.dy;
     a.conv_b = fwd.conv_b; a.b_a = fwd.b_a; a.b_x = fwd.b_x; a.lambda = q.lambda; a.h0 = fwd.h0;
     a.u = u; a.dz = dz; a.z = z; a.du = du;
     a.rec = (uint4 *)(ws + L.off_rec); a.epoch = (uint32_t *)(a.rec + (size_t)B * L.nchunk * D);
@@ -1059,7 +1137,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
 
     // 1. fp16 weights, conv output
     if ((e = convert_w(gr, q.W_a, q.W_x, q.H, W16, st)) != cudaSuccess) return e;
-    const dim3 grid_conv((D + 511) / 512, L.nchunk_conv, B);
+    const dim3 grid_conv((D + CONV_CH - 1) / CONV_CH, L.nchunk_conv, B);
     if ((e = launch_dependent(conv_forward_kernel, grid_conv, dim3(256), 0, st, ConvArgs{T, D, 0, 0, T, a.x, a.conv_w, a.cs_in, a.conv_b, u, a.epoch})) != cudaSuccess) return e;
 
     ReduceJobs jobs{};
@@ -1068,7 +1146,19 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     if ((e = gemm_z(gr, D, L.BT, u, W16, z, status, st)) != cudaSuccess) return e;
     GemmArgs g = gemm_args(gr, D, status);
     const unsigned mtiles = (unsigned)((L.BT + 127) / 128);
+    // h_{t-1} comes from the forward output; when the caller kept none, u and z are what the forward scan needs
+    const void *y = y_saved;
+    if (y == nullptr) {
+        FwdArgs f = fwd;
+        f.y = ws + L.off_y; f.h_T = (float *)(ws + L.off_hT); f.cs_out = ws + L.off_cs;
+        f.gate_branch = nullptr; f.a_prod = nullptr; f.status = status;
+        WideScanArgs w = wide_scan_args(gr, f, a.rec, a.epoch);
+        w.nb = B; w.n = T;
+        if ((e = run_wide_scan(w, u, z, st)) != cudaSuccess) return e;
+        y = f.y;
+    }
     // 3. reverse scan and element-wise adjoints
+    a.y = (const __nv_bfloat16 *)y;
     ScanArgs sc{};
     sc.e = a;
     sc.tiles = (hstride + 63) / 64;
@@ -1146,39 +1236,22 @@ cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_b
     char *ws = (char *)ws_body;
     __half *u = (__half *)(ws + L.off_u), *z = (__half *)(ws + L.off_z), *W16 = (__half *)(ws + L.off_w16);
     cudaError_t e;
-    WideScanArgs p{};
-    p.f = a;
+    WideScanArgs p = wide_scan_args(gr, a, (uint4 *)(ws + L.off_rec), nullptr);
+    p.epoch = (uint32_t *)(p.rec + (size_t)((L.n + SCAN_CHUNK - 1) / SCAN_CHUNK) * L.nb * D);
     // blocks that share a column read the incoming state at unrelated times: an in-place update works on a copy
     const size_t hb = (size_t)B * D * sizeof(float);
     if (a.h0 && (uintptr_t)a.h0 < (uintptr_t)a.h_T + hb && (uintptr_t)a.h_T < (uintptr_t)a.h0 + hb) {
         if ((e = cudaMemcpyAsync(ws + L.off_h0, a.h0, hb, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
         p.f.h0 = (const float *)(ws + L.off_h0);
     }
-    p.G = gr.G; p.hstride = gr.hstride; p.NS = gr.NS; p.tiles = (gr.hstride + 63) / 64;
-    p.rec = (uint4 *)(ws + L.off_rec);
-    p.epoch = (uint32_t *)(p.rec + (size_t)((L.n + SCAN_CHUNK - 1) / SCAN_CHUNK) * L.nb * D);
-    p.tag = next_call_tag(); p.spin_ns = g_spin_limit_ns;
-    static PerDeviceOptIn opt_in;
-    if ((e = opt_in.ensure(wide_scan_kernel, (int)WIDE_SMEM_ALLOC)) != cudaSuccess) return e;
-    const uint32_t box[3] = {64, SCAN_CHUNK, 1};
-    if (a.gate_branch) {
-        if (!encode_bf16_map_3d(&p.tm_g, a.gate_branch, (uint64_t)D, (uint64_t)T, (uint64_t)B, 64, SCAN_CHUNK, false)) return cudaErrorNotSupported;
-    }
     if ((e = convert_w(gr, a.W_a, a.W_x, a.H, W16, st)) != cudaSuccess) return e;
-    const int slots = 2 * num_sms();
     for (int b0 = 0; b0 < B; b0 += L.nb) {
         for (int tb = 0; tb < T; tb += L.n) {
             p.b0 = b0; p.nb = B - b0 < L.nb ? B - b0 : L.nb;
             p.tb = tb; p.n = T - tb < L.n ? T - tb : L.n;
-            p.nchunk = (p.n + SCAN_CHUNK - 1) / SCAN_CHUNK;
-            if ((e = launch_dependent(conv_forward_kernel, dim3((D + 511) / 512, (p.n + CONV_CHUNK - 1) / CONV_CHUNK, p.nb), dim3(256), 0, st, ConvArgs{T, D, b0, tb, p.n, (const __nv_bfloat16 *)a.x, (const __nv_bfloat16 *)a.conv_w, (const __nv_bfloat16 *)a.cs_in, a.conv_b, u, p.epoch})) != cudaSuccess) return e;
+            if ((e = launch_dependent(conv_forward_kernel, dim3((D + CONV_CH - 1) / CONV_CH, (p.n + CONV_CHUNK - 1) / CONV_CHUNK, p.nb), dim3(256), 0, st, ConvArgs{T, D, b0, tb, p.n, (const __nv_bfloat16 *)a.x, (const __nv_bfloat16 *)a.conv_w, (const __nv_bfloat16 *)a.cs_in, a.conv_b, u, p.epoch})) != cudaSuccess) return e;
             if ((e = gemm_z(gr, D, (size_t)p.nb * p.n, u, W16, z, a.status, st)) != cudaSuccess) return e;
-            const uint64_t wz = (uint64_t)gr.G * 2 * gr.NS;
-            const uint64_t du[3] = {(uint64_t)D, (uint64_t)p.n, (uint64_t)p.nb}, su[2] = {(uint64_t)D * 2, (uint64_t)D * p.n * 2};
-            const uint64_t dz[3] = {wz, (uint64_t)p.n, (uint64_t)p.nb}, sz[2] = {wz * 2, wz * p.n * 2};
-            if (!encode_map16_3d(&p.tm_u, u, du, su, box, false) || !encode_map16_3d(&p.tm_z, z, dz, sz, box, false)) return cudaErrorNotSupported;
-            p.S = scan_split(p.nb * gr.G * p.tiles, p.nchunk, slots);
-            if ((e = launch_dependent(wide_scan_kernel, dim3((unsigned)(p.nb * gr.G * p.tiles * p.S)), dim3(256), WIDE_SMEM_ALLOC, st, p)) != cudaSuccess) return e;
+            if ((e = run_wide_scan(p, u, z, st)) != cudaSuccess) return e;
         }
     }
     return cudaGetLastError();
