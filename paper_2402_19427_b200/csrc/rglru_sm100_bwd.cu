@@ -37,7 +37,7 @@ constexpr int CONV_SEG = 32;               // tokens per thread of the two Conv1
 constexpr int CONV_CHUNK = 4 * CONV_SEG;   // ... and per block: 64 threads x 4 channels, four segments
 constexpr int CONV_CH = 256;
 constexpr float LOG2E = 1.44269504f;
-constexpr int GEMM_THREADS = 192;          // TMA warp, MMA warp, four epilogue warps
+constexpr int GEMM_THREADS = 320;          // TMA warp, MMA warp, eight epilogue warps
 constexpr int GEMM_STAGES = 4;
 constexpr uint32_t A_STAGE_BYTES = 128 * 128;   // 128 rows x 64 bf16
 constexpr uint32_t B_STAGE_BYTES = 256 * 128;   // 256 rows x 64 bf16
@@ -65,7 +65,7 @@ struct GemmArgs {
 };
 
 // C[128 x NT] = A[128 x K] B[NT x K]^T per tile; A and B tiles arrive by tiled TMA in the 128-byte-swizzled K-major
-// layout, accumulate in tensor memory (fp32), and leave through the four epilogue warps.  CTAs are persistent: each
+// layout, accumulate in tensor memory (fp32), and leave through the eight epilogue warps.  CTAs are persistent: each
 // walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... with two accumulators, so that the epilogue of one tile overlaps
 // the loads and MMAs of the next.  Tile number -> (x, y, z) with x fastest:
 //   MODE_Z : (token tiles, 2 gates x nt, H)   A = u[tok][h][k]        B = W_gate[h][out][k]
@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
 
     if (tid == 0) {
         for (int s = 0; s < GEMM_STAGES; ++s) { mbar_init(BAR_FULL(s), 1); mbar_init(BAR_EMPTY(s), 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(BAR_ACCFULL(a), 1); mbar_init(BAR_ACCEMPTY(a), 4); }
+        for (int a = 0; a < 2; ++a) { mbar_init(BAR_ACCFULL(a), 1); mbar_init(BAR_ACCEMPTY(a), 8); }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -197,59 +197,81 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
             if (!ok) { *abort_flag = 1; atomicExch(p.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
         }
     } else {
-        // ---- epilogue: warp owns TMEM lanes 32 (warp & 3) .. +31 = rows of the tile
-        const int q = warp & 3;
+        // ---- epilogue: warp owns TMEM lanes 32 (warp & 3) .. +31 = rows of the tile, and every other 32 columns.  With four warps and
+        // the du values read between the accumulator loads, the du product waited for memory once per 32 columns (118 us on B4 T4096
+        // D4096); now a tile's du values are requested while its products run.
+        const int q = warp & 3, half = (warp - 2) >> 2;
         int it = 0;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
             const int tx = tile % p.nx, ty = (tile / p.nx) % p.ny, h = tile / (p.nx * p.ny);
             const int col0 = (ty % p.nt) * p.NT, sel = ty / p.nt;
             const int acc = it & 1;
             const int row = tx * 128 + q * 32 + lane;
-            ok = warp_wait(BAR_ACCFULL(acc), (it >> 1) & 1, spin, abort_flag);
-            if (!ok) break;
-            tc_fence_after();
-            const uint32_t tm_lane = tmem + ((uint32_t)(q * 32) << 16) + acc * 256;
             const bool valid = row < p.rows_valid;
             const int cv = min(p.hstride, p.D - h * p.hstride);   // channel slots of this group that exist
+            const uint32_t tm_lane = tmem + ((uint32_t)(q * 32) << 16) + acc * 256;
+            auto wait_acc = [&]() { ok = warp_wait(BAR_ACCFULL(acc), (it >> 1) & 1, spin, abort_flag); tc_fence_after(); };
+            if (p.mode == MODE_DU) {
+                // du is kept in fp16 like dz (bf16 failed the dx tolerance where the taps of the Conv1D adjoint cancel)
+                __half *dst0 = (__half *)p.out + (size_t)row * p.D + h * p.hstride + col0;
+                uint32_t o[4][2][8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int c0 = j * 64 + half * 32;
+                    if (valid && c0 < p.NT && col0 + c0 < cv) {   // a slot that does not exist: nothing of du belongs to it
+                        ld_global_v8(dst0 + c0, o[j][0]);
+                        ld_global_v8(dst0 + c0 + 16, o[j][1]);
+                    }
+                }
+                wait_acc();
+                if (!ok) break;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int c0 = j * 64 + half * 32;
+                    if (c0 < p.NT) {
+                        f32x2 v[16];
+                        tmem_ld32(tm_lane + c0, v);
+                        tmem_ld_wait();
+                        if (valid && col0 + c0 < cv) {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) {
+                                const float2 a0 = __half22float2(*(const __half2 *)&o[j][0][e]), a1 = __half22float2(*(const __half2 *)&o[j][1][e]);
+                                o[j][0][e] = pack_f16_sat(a0.x + lo2(v[e]), a0.y + hi2(v[e]));
+                                o[j][1][e] = pack_f16_sat(a1.x + lo2(v[8 + e]), a1.y + hi2(v[8 + e]));
+                            }
+                            st_global_v8(dst0 + c0, o[j][0]);
+                            st_global_v8(dst0 + c0 + 16, o[j][1]);
+                        }
+                    }
+                }
+            } else {
+                wait_acc();
+                if (!ok) break;
 #pragma unroll 1
-            for (int c0 = 0; c0 < p.NT; c0 += 32) {
-                f32x2 v[16];
-                tmem_ld32(tm_lane + c0, v);
-                tmem_ld_wait();
-                if (!valid) continue;
-                if (p.mode == MODE_Z) {
-                    __half *dst = (__half *)p.out + (((size_t)row * p.H + h) * 2 + sel) * p.NS + col0 + c0;
+                for (int c0 = half * 32; c0 < p.NT; c0 += 64) {
+                    f32x2 v[16];
+                    tmem_ld32(tm_lane + c0, v);
+                    tmem_ld_wait();
+                    if (!valid) continue;
+                    if (p.mode == MODE_Z) {
+                        __half *dst = (__half *)p.out + (((size_t)row * p.H + h) * 2 + sel) * p.NS + col0 + c0;
 #pragma unroll
-                    for (int j8 = 0; j8 < 2; ++j8) {
-                        uint32_t w[8];
+                        for (int j8 = 0; j8 < 2; ++j8) {
+                            uint32_t w[8];
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) { const __half2 hh = __floats2half2_rn(lo2(v[8 * j8 + j]), hi2(v[8 * j8 + j])); w[j] = *(const uint32_t *)&hh; }
-                        st_global_v8(dst + 16 * j8, w);
-                    }
-                } else if (p.mode == MODE_DU) {
-                    // du is kept in fp16 like dz (bf16 failed the dx tolerance where the taps of the Conv1D adjoint cancel)
-                    if (col0 + c0 >= cv) continue;   // a slot that does not exist: nothing of du belongs to it
-                    __half *dst = (__half *)p.out + (size_t)row * p.D + h * p.hstride + col0 + c0;
-                    uint32_t o0[8], o1[8];
-                    ld_global_v8(dst, o0);
-                    ld_global_v8(dst + 16, o1);
+                            for (int j = 0; j < 8; ++j) { const __half2 hh = __floats2half2_rn(lo2(v[8 * j8 + j]), hi2(v[8 * j8 + j])); w[j] = *(const uint32_t *)&hh; }
+                            st_global_v8(dst + 16 * j8, w);
+                        }
+                    } else {
+                        const int g = row >= p.NS, o_row = row - g * p.NS;
+                        float *dst = (float *)p.out + ((((size_t)sel * 2 + g) * p.H + h) * p.NS + o_row) * p.NS + col0 + c0;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float2 a0 = __half22float2(*(const __half2 *)&o0[j]), a1 = __half22float2(*(const __half2 *)&o1[j]);
-                        o0[j] = pack_f16_sat(a0.x + lo2(v[j]), a0.y + hi2(v[j]));
-                        o1[j] = pack_f16_sat(a1.x + lo2(v[8 + j]), a1.y + hi2(v[8 + j]));
-                    }
-                    st_global_v8(dst, o0);
-                    st_global_v8(dst + 16, o1);
-                } else {
-                    const int g = row >= p.NS, o_row = row - g * p.NS;
-                    float *dst = (float *)p.out + ((((size_t)sel * 2 + g) * p.H + h) * p.NS + o_row) * p.NS + col0 + c0;
+                        for (int j = 0; j < 4; ++j) {
+                            uint32_t w[8];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        uint32_t w[8];
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) { w[2 * e] = __float_as_uint(lo2(v[4 * j + e])); w[2 * e + 1] = __float_as_uint(hi2(v[4 * j + e])); }
-                        st_global_v8(dst + 8 * j, w);
+                            for (int e = 0; e < 4; ++e) { w[2 * e] = __float_as_uint(lo2(v[4 * j + e])); w[2 * e + 1] = __float_as_uint(hi2(v[4 * j + e])); }
+                            st_global_v8(dst + 8 * j, w);
+                        }
                     }
                 }
             }
