@@ -76,6 +76,15 @@ __device__ __forceinline__ IOT x_raw_at(const IOT *x, const IOT *cs_in, int T, i
     return cs_in[((size_t)b * 3 + (3 + tau)) * D + d];
 }
 
+// r, i, a, m of Eq. 1-4 for one token of one channel.  A function of its own: inlined for each of a thread's 8 x 4 results it was
+// some five thousand instructions, which every block fetched once.
+__device__ __noinline__ float4 gates_acc(float za, float zx, float s) {
+    const float r = sigmoid_acc(za), g = sigmoid_acc(zx);
+    float a, m;
+    decay(s, r, a, m);
+    return make_float4(r, g, a, m);
+}
+
 // ------------------------------------------------------------------ register-blocked fp32 product
 // Geometry of a block: 128 threads as 8 (rows) x 16 (columns); BM rows x 2 BM columns of results.  Thread (ty, tx) owns rows
 // TM ty .. TM ty + TM - 1 and columns NH tx .. + NH - 1 of each half of the columns (in the forward the halves are the two
@@ -312,9 +321,8 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(F
             float Pc = 1.0f, hc = 0.0f;
 #pragma unroll
             for (int i = 0; i < TM; ++i) {
-                const float r = sigmoid_acc(col<NH>(acc[i], 0, j) + ba), g = sigmoid_acc(col<NH>(acc[i], 1, j) + bx);
-                float at, mt;
-                decay(sr, r, at, mt);
+                const float4 gt = gates_acc(col<NH>(acc[i], 0, j) + ba, col<NH>(acc[i], 1, j) + bx, sr);
+                const float r = gt.x, g = gt.y, at = gt.z, mt = gt.w;
                 const bool tv = tr + i < T;
                 if (SAVE) {
                     if (tv && cv) {
@@ -826,10 +834,10 @@ inline int ceil_div(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 constexpr int FILL_BLOCKS = 296;
 inline int tile_rows(size_t blocks64) { return blocks64 >= (size_t)FILL_BLOCKS ? 64 : 32; }
 
-// Token splits of the dW products: enough blocks for two waves of three per SM, at least 128 tokens each, at most 32
+// Token splits of the dW products: as many blocks as fill two waves of three per SM (one split more began a third wave), at least 128 tokens each, at most 32
 int dw_splits(size_t ntok, int H, int Dh) {
     const size_t tiles = (size_t)2 * H * ceil_div(Dh, 64) * ceil_div(Dh, 128);
-    size_t s = (888 + tiles - 1) / tiles;
+    size_t s = 888 / tiles;
     const size_t most = (ntok + 127) / 128;
     if (s > most) s = most;
     return (int)(s < 1 ? 1 : (s > 32 ? 32 : s));
