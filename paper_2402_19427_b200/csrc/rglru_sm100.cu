@@ -50,7 +50,6 @@ constexpr int US = 6;              // U tile stages
 constexpr int NUM_THREADS = 640;          // 20 warps; the merged forward has four scan warps more
 constexpr int MERGED_THREADS = 768;
 constexpr int MAX_S = 16;          // at most this many pairs share one head's time axis
-constexpr int LOOKBACK_BATCH = 8;  // carry records requested at once by the look-back
 constexpr uint32_t U_STAGE_BYTES = HALF * DH * 2;          // 16384
 constexpr uint32_t U_KBLOCK_BYTES = HALF * 128;            // 4096: one 64-channel K block
 constexpr uint32_t X_ROW_BYTES = DH * 2;                   // 512
@@ -542,6 +541,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
         float h_prev_own = 0.0f;  // state at the end of this pair's previous tile
         float P_prev_own = 1.0f;  // prod of a_t from the start of the sequence to the end of this pair's previous tile
         constexpr bool merged = MERGED;
+        // carry records requested at once by the look-back: few, because their registers are live beside the tile's (eight for both:
+        // B8 T2048 D2560 with the gate branch 126 instead of 122 us, B3 T1213 width 160 39.9 instead of 39.6)
+        constexpr int LOOKBACK_BATCH = MERGED ? 2 : 4;
         bool ok = true;
         if constexpr (merged) ok = warp_wait(BAR_WDONE, 0, spin, abort_flag);   // and in the y buffers, where the branch arrives
         const int n_scan = !merged || ok ? n_my_tiles : 0;
@@ -583,7 +585,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
                 int nback;
                 if (ti < S) { h = f.h0 && exists ? f.h0[(size_t)b * D + d] : 0.0f; P = 1.0f; nback = ti; }
                 else { h = h_prev_own; P = P_prev_own; nback = S - 1; }
-                // The records are taken oldest first, up to eight at a time: all of a batch are requested at once, then polled
+                // The records are taken oldest first, a few at a time: all of a batch are requested at once, then polled
                 // until every lane sees this call's tag in both halves of each record (8-byte words are written atomically).
                 const uint4 *src = p.agg + ((size_t)group * p.tiles_total + gidx) * CH + c_own;
                 for (int jb = nback; jb > 0 && ok; jb -= LOOKBACK_BATCH) {
