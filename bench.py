@@ -38,7 +38,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # DRAM bytes per prefill launch on the bench workload (dram__bytes_read.sum + dram__bytes_write.sum of one ncu capture,
 # profiles/sm100_prefill_kernel_cfg1.md) together with the SHA-256 of the kernel source the capture was taken from:
 # the figure is reported only while the benched kernel source still has that hash, else null.
-NCU_TRAFFIC = {"bytes": 86779904 + 38424320, "kernel_sha256": "5a7c17c6514325df36dff701c430a409f52f42076cf00ff1d71408e8d6573fb3"}
+NCU_TRAFFIC = {"bytes": 86755328 + 38701824, "kernel_sha256": "a2734afb89a6f935973edc9757b9231be2746bc1cd3bcbf865044f0c71ebbe0f"}
 KERNEL_SOURCE = os.path.join(ROOT, "paper_2402_19427_b200", "csrc", "rglru_sm100.cu")
 
 
@@ -308,7 +308,7 @@ def run_ours(args):
 
     # The K timed steps are K calls of the public API captured once in a CUDA graph and replayed: the calls allocate nothing
     # (outputs and workspace are passed in), and a graph takes the host's launch cost and the gap between consecutive
-    # cooperative launches out of the measurement (measured: 86 against 91 us per step with plain stream launches, which are
+    # launches out of the measurement (measured: 86 against 91 us per step with plain stream launches, which are
     # timed as well and reported beside it).  Everything that costs host time (NVML set-up, event creation, the capture)
     # happens before the warm-up, so that the GPU does not sit idle between the warm-up and the timed region; the warm-up
     # itself is preceded by untimed launches of the same step for PREWARM_S seconds, which brings clocks and caches to their

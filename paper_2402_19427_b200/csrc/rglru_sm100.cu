@@ -165,6 +165,14 @@ __device__ __noinline__ bool stage_weights(const CUtensorMap *tm_wa, const CUten
     return w_ok;
 }
 
+// The failure path of every role, out of line: inlined at six places it cost the hot loops registers (eight-byte spills; B1 T65536
+// D4096 577 instead of 573 us, B1 T197 D2560 11.4 instead of 11.2).
+__device__ __noinline__ void set_timeout(volatile int *abort_flag, uint32_t peer_abort, uint32_t *status) {
+    *abort_flag = 1;
+    st_cluster_u32(peer_abort, 1u);   // the peer would otherwise run into its own limit waiting for this CTA
+    atomicExch(status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT);
+}
+
 // MERGED: the call has a gate branch and writes y_t = h_t GeLU(branch_t); a separate instantiation so that the plain forward
 // carries none of its code.  GeLU triples the scan warps' work per element, so there are eight of them, half a tile each (four
 // warps with whole tiles: 180 us on B8 T2048 D2560, twice the plain forward).
@@ -203,11 +211,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
     // the tensor), their weights are zero in both directions, and nothing of them is written.
     const int cbase = head * p.hstride, cvalid = min(p.cvalid, D - cbase);   // the layer's last group may hold fewer heads
     const uint32_t peer_abort = map_to_cta(base + SMEM_MISC + 4, rank ^ 1u);
-    auto record_timeout = [&]() {
-        *abort_flag = 1;
-        st_cluster_u32(peer_abort, 1u);   // the peer would otherwise run into its own limit waiting for this CTA
-        atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT);
-    };
+    auto record_timeout = [&]() { set_timeout(abort_flag, peer_abort, f.status); };
     // Work of this pair.  Sequences are dealt out whole where that keeps the S pairs of the head balanced: pair kcta
     // gets sequences kcta, kcta + S, ... of the first (B / S) * S ones and walks each from start to end, so a tile's
     // incoming state is simply the state the pair itself reached ("local" tiles: no record, no look-back).  The B % S
@@ -543,7 +547,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
         constexpr bool merged = MERGED;
         // carry records requested at once by the look-back: few, because their registers are live beside the tile's (eight for both:
         // B8 T2048 D2560 with the gate branch 126 instead of 122 us, B3 T1213 width 160 39.9 instead of 39.6)
-        constexpr int LOOKBACK_BATCH = MERGED ? 2 : 4;
+        constexpr int LOOKBACK_BATCH = MERGED ? 2 : 3;   // three: what four pairs of a head have to read
         bool ok = true;
         if constexpr (merged) ok = warp_wait(BAR_WDONE, 0, spin, abort_flag);   // and in the y buffers, where the branch arrives
         const int n_scan = !merged || ok ? n_my_tiles : 0;
