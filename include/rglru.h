@@ -26,6 +26,9 @@
  *  - `workspace` is caller-owned device scratch of at least rglru_workspace_bytes(...)
  *    bytes, 256-byte aligned.  Its contents need not be preserved between calls; calls
  *    that share a workspace must be ordered on one stream.
+ *  - A call may be captured in a CUDA graph and the graph replayed, on other contents of the same buffers.  Replays that share
+ *    a workspace must be ordered like calls.  After RGLRU_ERR_TIMEOUT, zero the workspace before a graph that uses it is
+ *    replayed: the replay looks for the records that the failed run left incomplete.
  *  - Shapes without a kernel return RGLRU_ERR_UNSUPPORTED.  There is no CPU fallback.
  *  - Kernels.  bf16 io with a head width D_h that is a multiple of 32 runs on tensor-core kernels: prefill and backward at any
  *    such width up to 1024, the decode step up to 256.  Section 4.1 fixes 16 blocks, so D_h is 256 only at D_RNN = 4096; it is 96

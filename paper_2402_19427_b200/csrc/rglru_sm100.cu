@@ -59,8 +59,9 @@ constexpr uint32_t SMEM_X = SMEM_U + US * U_STAGE_BYTES;
 constexpr uint32_t Y_BUF_BYTES = TILE * 32 * 2;            // 4096: one scan warp's 64 tokens x 32 channels
 constexpr uint32_t SMEM_Y = SMEM_X + XS * X_SLAB_BYTES;    // bf16 y_s[4 warps][2 buffers][64][32], staged for tiled stores
 constexpr uint32_t SMEM_AGG = SMEM_Y + 4 * 2 * Y_BUF_BYTES;   // float2 agg_s[2 buffers][2 half tiles][128 channels]
-constexpr uint32_t SMEM_BAR = SMEM_AGG + 2 * 2 * CH * 8;
-constexpr int NUM_BARS = 2 * XS + 2 * US + 4 + 8 + 1 + 8 + 2;
+constexpr uint32_t SMEM_EPOCH = SMEM_AGG + 2 * 2 * CH * 8;      // uint32 epoch_s[MAX_S - 1 time-split sequences][128 channels]
+constexpr uint32_t SMEM_BAR = SMEM_EPOCH + (MAX_S - 1) * CH * 4;
+constexpr int NUM_BARS = 2 * XS + 2 * US + 4 + 8 + 1 + 8 + 2 + 4;
 constexpr uint32_t SMEM_MISC = SMEM_BAR + NUM_BARS * 8;    // tmem base, abort flag
 constexpr uint32_t SMEM_TOTAL = SMEM_MISC + 16;
 constexpr uint32_t SMEM_ALLOC = SMEM_TOTAL + 1024;         // slack for 1024-byte alignment
@@ -100,10 +101,10 @@ struct Sm100Args {
     int cvalid;        // channel slots of a "head" that exist: k dh (fewer in the layer's last group when k does not divide H)
     int S;             // pairs per head (time split factor)
     int tps;           // tiles per sequence
-    int tiles_total;   // B * tps
+    int tiles_total;   // tiles of the sequence slots that can be split in time (record_slots * tps)
     uint32_t tag;      // validity tag of this call's aggregate records
     uint32_t tag_wait; // the tag the look-back waits for: `tag`, or a value nobody publishes under the failure-path test flag
-    uint4 *agg;        // [H*2][tiles_total][128] records {P, tag, h_loc, tag}
+    uint4 *agg;        // [H*2][tiles_total][128] records {P, tag + e, h_loc, tag + 2 e}, e: the sequence's epoch (see look-back records)
     unsigned long long spin_ns;
 };
 
@@ -165,6 +166,19 @@ __device__ __noinline__ bool stage_weights(const CUtensorMap *tm_wa, const CUten
     return w_ok;
 }
 
+// Look-back records.  The host's tag tells the records of one call from those of every other, but a CUDA graph replays a call with
+// the tag of its capture: the first replay's records would pass for the second's.  So a record also carries an epoch, one word per
+// time-split sequence and channel, that every execution advances.  It lives where nothing else is kept, in word x of the record of
+// the sequence's last tile (nobody looks back at that one): a pair reads it before it publishes anything, and the pair of the last
+// tile writes it back plus one after its look-back, which has by then seen a record of this execution from every other pair that
+// has a tile of the sequence.  Any starting value will do.  {tag + e, tag + 2 e} differs for every (tag, e), each half from epoch to
+// epoch as well.
+__device__ __forceinline__ uint32_t ld_volatile_u32(const void *ptr) {
+    uint32_t v;
+    asm volatile("ld.volatile.global.b32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
+    return v;
+}
+
 // The failure path of every role, out of line: inlined at six places it cost the hot loops registers (eight-byte spills; B1 T65536
 // D4096 577 instead of 573 us, B1 T197 D2560 11.4 instead of 11.2).
 __device__ __noinline__ void set_timeout(volatile int *abort_flag, uint32_t peer_abort, uint32_t *status) {
@@ -194,6 +208,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
     const uint32_t BAR_WREADY = bar0 + 8u * (2 * XS + 2 * US + 12);               // leader CTA only: both CTAs' weights are in tensor memory
     auto BAR_BRANCH = [&](int w) { return bar0 + 8u * (2 * XS + 2 * US + 13 + w); };   // scan warp w's block of the gate branch has landed
     const uint32_t BAR_WLOAD = bar0 + 8u * (2 * XS + 2 * US + 21), BAR_WDONE = BAR_WLOAD + 8;   // weights staged in shared memory; read out of it again
+    auto BAR_EPOCH = [&](int q) { return bar0 + 8u * (2 * XS + 2 * US + 23 + q); };   // merged: quarter q's epochs are in shared memory
     uint32_t *tmem_base_s = (uint32_t *)(smem + SMEM_MISC);
     volatile int *abort_flag = (volatile int *)(smem + SMEM_MISC + 4);
 
@@ -251,6 +266,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
         mbar_init(BAR_WREADY, 16);
         mbar_init(BAR_WLOAD, 1); mbar_init(BAR_WDONE, 8);
         for (int w = 0; w < 8; ++w) mbar_init(BAR_BRANCH(w), 1);
+        for (int q = 0; q < 4; ++q) mbar_init(BAR_EPOCH(q), 1);
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -549,7 +565,19 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
         // B8 T2048 D2560 with the gate branch 126 instead of 122 us, B3 T1213 width 160 39.9 instead of 39.6)
         constexpr int LOOKBACK_BATCH = MERGED ? 2 : 3;   // three: what four pairs of a head have to read
         bool ok = true;
-        if constexpr (merged) ok = warp_wait(BAR_WDONE, 0, spin, abort_flag);   // and in the y buffers, where the branch arrives
+        // the epochs of the time-split sequences, read before this pair publishes anything; with the gate branch the second half tile's
+        // warp, which publishes nothing, takes them from the first's
+        uint32_t *epoch_s = (uint32_t *)(smem + SMEM_EPOCH) + c_own;
+        if (n_shared > 0 && part == 0) {
+            for (int s = 0; s < f.B - B_whole; ++s)
+                epoch_s[s * CH] = ld_volatile_u32(p.agg + ((size_t)group * p.tiles_total + (size_t)(s + 1) * p.tps - 1) * CH + c_own);
+            __syncwarp();
+            if (merged && lane == 0) mbar_arrive(BAR_EPOCH(q));
+        }
+        if constexpr (merged) {
+            if (n_shared > 0 && part == 1) ok = warp_wait(BAR_EPOCH(q), 0, spin, abort_flag);
+            ok = ok && warp_wait(BAR_WDONE, 0, spin, abort_flag);   // the weights were staged in the y buffers too, where the branch arrives
+        }
         const int n_scan = !merged || ok ? n_my_tiles : 0;
         int b, ti;
         tile_first(b, ti);
@@ -581,17 +609,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
                 h = ti == 0 ? (f.h0 && exists ? f.h0[(size_t)b * D + d] : 0.0f) : h_prev_own;
                 P = ti == 0 ? 1.0f : P_prev_own;
             } else {
-                // publish the tile's aggregate before waiting for anyone
-                uint4 rec;
-                rec.x = __float_as_uint(e0.x * e1.x); rec.y = p.tag; rec.z = __float_as_uint(fmaf(e1.x, e0.y, e1.y)); rec.w = p.tag;
-                uint4 *dst = p.agg + ((size_t)group * p.tiles_total + gidx) * CH + c_own;
-                if (part == 0) asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(dst), "r"(rec.x), "r"(rec.y), "r"(rec.z), "r"(rec.w) : "memory");
+                // publish the tile's aggregate before waiting for anyone (nobody looks back at the last tile of a sequence)
+                const uint32_t ep = epoch_s[(b - B_whole) * CH];
+                uint4 *rec = p.agg + ((size_t)group * p.tiles_total + gidx) * CH + c_own;
+                if (part == 0 && ti + 1 < p.tps)
+                    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec), "r"(__float_as_uint(e0.x * e1.x)), "r"(p.tag + ep),
+                                 "r"(__float_as_uint(fmaf(e1.x, e0.y, e1.y))), "r"(p.tag + 2u * ep) : "memory");
                 int nback;
                 if (ti < S) { h = f.h0 && exists ? f.h0[(size_t)b * D + d] : 0.0f; P = 1.0f; nback = ti; }
                 else { h = h_prev_own; P = P_prev_own; nback = S - 1; }
-                // The records are taken oldest first, a few at a time: all of a batch are requested at once, then polled
-                // until every lane sees this call's tag in both halves of each record (8-byte words are written atomically).
-                const uint4 *src = p.agg + ((size_t)group * p.tiles_total + gidx) * CH + c_own;
+                // The records are taken oldest first, a few at a time: all of a batch are requested at once, then polled until every lane
+                // sees this execution's tag in both halves of each record (8-byte words are written atomically).
+                const uint32_t want_y = p.tag_wait + ep, want_w = p.tag_wait + 2u * ep;
                 for (int jb = nback; jb > 0 && ok; jb -= LOOKBACK_BATCH) {
                     const int cnt = jb < LOOKBACK_BATCH ? jb : LOOKBACK_BATCH;   // records jb, jb - 1, ..., jb - cnt + 1 tiles back
                     uint4 r[LOOKBACK_BATCH];
@@ -601,14 +630,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
 #pragma unroll
                         for (int k = 0; k < LOOKBACK_BATCH; ++k) {
                             if (k < cnt) {
-                                const uint4 *sj = src - (size_t)(jb - k) * CH;
+                                const uint4 *sj = rec - (size_t)(jb - k) * CH;
                                 asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];"
                                              : "=r"(r[k].x), "=r"(r[k].y), "=r"(r[k].z), "=r"(r[k].w) : "l"(sj) : "memory");
                             }
                         }
 #pragma unroll
                         for (int k = 0; k < LOOKBACK_BATCH; ++k)
-                            if (k < cnt) ready = ready && r[k].y == p.tag_wait && r[k].w == p.tag_wait;
+                            if (k < cnt) ready = ready && r[k].y == want_y && r[k].w == want_w;
                         if (__all_sync(0xffffffffu, ready)) break;
                         if ((npoll & 15u) == 15u) {
                             const uint64_t tnow = gtimer();
@@ -625,6 +654,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
                     }
                 }
                 if (!ok) break;
+                if (part == 0 && ti + 1 == p.tps) asm volatile("st.global.b32 [%0], %1;" ::"l"(rec), "r"(ep + 1u) : "memory");
             }
             const float h_mid = fmaf(e0.x, h, e0.y);      // state after the first half tile
             h_prev_own = fmaf(e1.x, h_mid, e1.y);         // state after the tile

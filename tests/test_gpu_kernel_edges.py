@@ -130,6 +130,36 @@ def test_replayed_graph_of_chained_chunks(oracle):
         assert_close("dx", to_np(g["x"]), gr["x"], io, scale=max(1.0, float(np.abs(gr["x"]).max())) if io == "f32" else 1.0)
 
 
+@pytest.mark.parametrize("B,T,Dh,H,merge,keep", [(1, 2000, 256, 1, False, True), (1, 2000, 256, 1, False, False), (1, 700, 96, 2, False, True),
+                                                (3, 130, 256, 2, True, True), (1, 1999, 256, 1, True, False), (2, 64, 256, 1, False, True)])
+def test_replayed_graph_of_a_time_split_forward(oracle, B, T, Dh, H, merge, keep):
+    """The fused prefill with sequences split in time over several CTA pairs: a replay of the captured call must not take the carry
+    records that the replay before it left in the workspace for its own.  Every replay works on other inputs."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    D = Dh * H
+    rounds = [synth.make_inputs(B, T, D, H, io="bf16", seed=80 + k, with_dy=True, with_state=True) for k in range(4)]
+    params = binding.Params.from_numpy(rounds[0]["params"], "bf16")
+    x, h0, branch = to_dev(rounds[0]["x"], "bf16"), to_dev(rounds[0]["h0"]), to_dev(rounds[0]["dy"], "bf16") if merge else None
+    ws = binding.alloc_workspace(binding.make_shape(B, T, D, H, x.dtype), binding.OP_PREFILL, x.device) if keep else None
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        binding.prefill(x, params, h0=h0, workspace=ws, gate_branch=branch)   # first use outside the capture
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            y, hT, _ = binding.prefill(x, params, h0=h0, workspace=ws, gate_branch=branch)
+        for inp in rounds:
+            x.copy_(to_dev(inp["x"], "bf16")); h0.copy_(to_dev(inp["h0"]))
+            if merge:
+                branch.copy_(to_dev(inp["dy"], "bf16"))
+            graph.replay()
+            stream.synchronize()
+            yr, hr, _ = oracle.prefill(inp["x"].astype(np.float64), f64(rounds[0]["params"]), H, h0=inp["h0"].astype(np.float64),
+                                       gate_branch=inp["dy"].astype(np.float64) if merge else None)
+            assert_close("y", to_np(y), yr, "bf16"); assert_close("h_T", to_np(hT), hr, "bf16")
+
+
 @pytest.mark.parametrize("change,error", [
     (dict(h0=lambda t: t.double()), ValueError), (dict(x=lambda t: t.transpose(0, 1)), ValueError), (dict(workspace=lambda t: t[:128]), RuntimeError),
     (dict(flags=lambda v: 1 << 40), RuntimeError), (dict(conv_state_in=lambda t: t.cpu()), ValueError)])
