@@ -190,7 +190,7 @@ __device__ __noinline__ void set_timeout(volatile int *abort_flag, uint32_t peer
 // MERGED: the call has a gate branch and writes y_t = h_t GeLU(branch_t); a separate instantiation so that the plain forward
 // carries none of its code.  GeLU triples the scan warps' work per element, so there are eight of them, half a tile each (four
 // warps with whole tiles: 180 us on B8 T2048 D2560, twice the plain forward).
-template <bool MERGED>
+template <bool MERGED, int LB>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THREADS : NUM_THREADS, 1) sm100_prefill_kernel(const __grid_constant__ Sm100Args p) {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -561,9 +561,6 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
         float h_prev_own = 0.0f;  // state at the end of this pair's previous tile
         float P_prev_own = 1.0f;  // prod of a_t from the start of the sequence to the end of this pair's previous tile
         constexpr bool merged = MERGED;
-        // carry records requested at once by the look-back: few, because their registers are live beside the tile's (eight for both:
-        // B8 T2048 D2560 with the gate branch 126 instead of 122 us, B3 T1213 width 160 39.9 instead of 39.6)
-        constexpr int LOOKBACK_BATCH = MERGED ? 2 : 3;   // three: what four pairs of a head have to read
         bool ok = true;
         // the epochs of the time-split sequences, read before this pair publishes anything; with the gate branch the second half tile's
         // warp, which publishes nothing, takes them from the first's
@@ -621,14 +618,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
                 // The records are taken oldest first, a few at a time: all of a batch are requested at once, then polled until every lane
                 // sees this execution's tag in both halves of each record (8-byte words are written atomically).
                 const uint32_t want_y = p.tag_wait + ep, want_w = p.tag_wait + 2u * ep;
-                for (int jb = nback; jb > 0 && ok; jb -= LOOKBACK_BATCH) {
-                    const int cnt = jb < LOOKBACK_BATCH ? jb : LOOKBACK_BATCH;   // records jb, jb - 1, ..., jb - cnt + 1 tiles back
-                    uint4 r[LOOKBACK_BATCH];
+                for (int jb = nback; jb > 0 && ok; jb -= LB) {
+                    const int cnt = jb < LB ? jb : LB;   // records jb, jb - 1, ..., jb - cnt + 1 tiles back
+                    uint4 r[LB];
                     uint64_t tstart = 0;
                     for (uint32_t npoll = 0;; ++npoll) {
                         bool ready = true;
 #pragma unroll
-                        for (int k = 0; k < LOOKBACK_BATCH; ++k) {
+                        for (int k = 0; k < LB; ++k) {
                             if (k < cnt) {
                                 const uint4 *sj = rec - (size_t)(jb - k) * CH;
                                 asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];"
@@ -636,7 +633,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
                             }
                         }
 #pragma unroll
-                        for (int k = 0; k < LOOKBACK_BATCH; ++k)
+                        for (int k = 0; k < LB; ++k)
                             if (k < cnt) ready = ready && r[k].y == want_y && r[k].w == want_w;
                         if (__all_sync(0xffffffffu, ready)) break;
                         if ((npoll & 15u) == 15u) {
@@ -649,7 +646,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
                     ok = __all_sync(0xffffffffu, ok);
                     if (ok) {
 #pragma unroll
-                        for (int k = 0; k < LOOKBACK_BATCH; ++k)
+                        for (int k = 0; k < LB; ++k)
                             if (k < cnt) { h = fmaf(__uint_as_float(r[k].x), h, __uint_as_float(r[k].z)); P *= __uint_as_float(r[k].x); }
                     }
                 }
@@ -754,6 +751,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
     if (warp == 5) tmem_dealloc2(tmem, 512);
 }
 
+// The instantiation for a call: with or without a gate branch, and with the look-back batch that suits the S - 1 records a time-split
+// tile has to read.  Batches are requested in turn, each a trip through L2, so many records want a large batch; but its registers are
+// live in the scan warps' loop, which costs every tile.  Three at once while that is one or two rounds (S <= 7), five from S = 8 on:
+// B8 T2048 D1024 (S = 16) 54.6 us with three, 48.8 with five, 50.0 with eight; D1536 in 16 heads (S = 8) 76.4 / 74.3 / 74.7; D2560 in
+// 10 heads (S = 7) 84.1 / 85.9 / 85.6; B1 T16384 D4096 (S = 4) 141.7 / 144.8 / 148.6.
+typedef void (*PrefillKernel)(Sm100Args);
+PrefillKernel prefill_kernel(bool merged, bool many) {
+    if (merged) return many ? sm100_prefill_kernel<true, 5> : sm100_prefill_kernel<true, 3>;
+    return many ? sm100_prefill_kernel<false, 5> : sm100_prefill_kernel<false, 3>;
+}
+
 // Per-device launch facts, looked up once per device with that device current.
 struct DeviceInfo {
     bool ready = false;
@@ -772,17 +780,17 @@ cudaError_t device_info(DeviceInfo *out) {
     DeviceInfo &di = g_dev[dev];
     if (!di.ready) {
         // opt in to the large dynamic shared memory once per device (function attributes are per context)
-        e = cudaFuncSetAttribute(sm100_prefill_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC);
-        if (e != cudaSuccess) return e;
-        e = cudaFuncSetAttribute(sm100_prefill_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC);
-        if (e != cudaSuccess) return e;
+        for (int v = 0; v < 4; ++v) {
+            e = cudaFuncSetAttribute(prefill_kernel(v & 1, v >> 1), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALLOC);
+            if (e != cudaSuccess) return e;
+        }
         int n = 0;
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) di.sms = n;
         cudaLaunchConfig_t q{};
         q.gridDim = dim3(2 * di.sms); q.blockDim = dim3(NUM_THREADS); q.dynamicSmemBytes = SMEM_ALLOC;
         int np = 0;
         // a pair needs two free SMs of one cluster-capable group, so fewer than sms / 2 pairs may fit
-        di.max_pairs = (cudaOccupancyMaxActiveClusters(&np, sm100_prefill_kernel<false>, &q) == cudaSuccess && np > 0) ? np : di.sms / 2 - 4;
+        di.max_pairs = (cudaOccupancyMaxActiveClusters(&np, sm100_prefill_kernel<false, 3>, &q) == cudaSuccess && np > 0) ? np : di.sms / 2 - 4;
         di.ready = true;
     }
     *out = di;
@@ -933,7 +941,7 @@ cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes,
         if ((e = cudaMemcpyAsync(cs_copy, a.cs_in, cs_bytes, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
         p.f.cs_in = cs_copy;
     }
-    return launch_dependent(a.gate_branch ? sm100_prefill_kernel<true> : sm100_prefill_kernel<false>, dim3(2 * G * S), dim3(a.gate_branch ? MERGED_THREADS : NUM_THREADS), SMEM_ALLOC, st, p);
+    return launch_dependent(prefill_kernel(a.gate_branch != nullptr, S > 7), dim3(2 * G * S), dim3(a.gate_branch ? MERGED_THREADS : NUM_THREADS), SMEM_ALLOC, st, p);
 }
 
 }  // namespace rglru
