@@ -239,7 +239,9 @@ int32_t rglru_prefill_static_scratch(const rglru_shape_t *shape, const rglru_par
  * Time limit of every device-side wait (a CTA waiting for another CTA's carry record, for a copy or for the tensor
  * core).  A wait that runs out makes the kernel record RGLRU_ERR_TIMEOUT in the workspace header, let work in flight
  * land, release its resources and return; nothing hangs and the context stays usable.  The default is 2 s, far above
- * any legitimate wait; ns = 0 restores it.  Process-wide; takes effect for calls issued afterwards.  Returns the
+ * any legitimate wait; ns = 0 restores it.  Blocks of one call that wait for one another's carry records need to be on the
+ * GPU together.  Where other work (another stream's kernel) keeps some of them off it, the limit counts from when the last of
+ * them has started; for that they are waited for up to 16 times the limit.  Process-wide; takes effect for calls issued afterwards.  Returns the
  * previous value.
  */
 uint64_t rglru_set_wait_limit_ns(uint64_t ns);

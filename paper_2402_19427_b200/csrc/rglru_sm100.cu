@@ -22,8 +22,9 @@
 // dealt out whole go to the S pairs of a head tile by tile, round-robin.  The scan warp folds such a tile to the
 // aggregate (prod a_t, h_end from zero state), publishes it, and obtains its incoming state from its own previous
 // tile plus the S-1 aggregates published by the other pairs (decoupled look-back); only then does it run the scan.
-// Waits are bounded and end in RGLRU_ERR_TIMEOUT.  With a time split the grid fits the SMs at once, and the pairs of a head are
-// neighbours in block order, so at most one head is partly dispatched while others still hold SMs, and those finish.
+// Waits are bounded and end in RGLRU_ERR_TIMEOUT.  With a time split the grid fits an idle GPU at once, and the pairs of a head are
+// neighbours in block order, so at most one head of a call is partly dispatched while others still hold SMs, and those finish.
+// Other work may keep the rest of that head off the SMs for as long as it likes: see carry_clock for what that does to the limits.
 // (A cooperative launch, which would ask for all SMs at once, measured the same but does not combine with dependent launch.)
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -104,6 +105,7 @@ struct Sm100Args {
     int tiles_total;   // tiles of the sequence slots that can be split in time (record_slots * tps)
     uint32_t tag;      // validity tag of this call's aggregate records
     uint32_t tag_wait; // the tag the look-back waits for: `tag`, or a value nobody publishes under the failure-path test flag
+    unsigned long long carry_ns;   // limit of a wait for carry records, from when the pairs waited for are running
     uint4 *agg;        // [H*2][tiles_total][128] records {P, tag + e, h_loc, tag + 2 e}, e: the sequence's epoch (see look-back records)
     unsigned long long spin_ns;
 };
@@ -177,6 +179,27 @@ __device__ __forceinline__ uint32_t ld_volatile_u32(const void *ptr) {
     uint32_t v;
     asm volatile("ld.volatile.global.b32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
     return v;
+}
+
+// A pair marks the record of its first time-split tile when it starts, with a word that no published record holds.  The limit of a
+// wait for records counts from when every pair waited for has left its mark: pairs that other work on the GPU keeps off the SMs are
+// no failure (with a limit of their own all the same, CARRY_START_LIMITS times as long, which the kernel's other waits share).
+constexpr uint32_t RUNNING = 0x80000000u;
+constexpr unsigned CARRY_START_LIMITS = 16;
+// One look at that clock, out of line because it is the rare path of the polls: `state` holds the time of the first look and of the
+// last one that missed a pair (units of 1024 ns), 0 before the first; the result is the next state, or ~0 when the wait is over.
+__device__ __noinline__ uint64_t carry_clock(uint64_t state, const uint4 *rec0, const uint32_t *epoch_s, int first, int count, int S, int tps, uint32_t tag, unsigned long long limit_ns) {
+    bool running = true;
+    for (int k = 0; k < count; ++k) {
+        const int pair = (first + k) % S;
+        const uint32_t mark = tag + epoch_s[(pair / tps) * CH], v = ld_volatile_u32(&rec0[(size_t)pair * CH].y);
+        running = running && (v == mark || v == (mark ^ RUNNING));
+    }
+    running = __all_sync(0xffffffffu, running);
+    const uint32_t now = (uint32_t)(gtimer() >> 10) | 1u, limit = (uint32_t)(limit_ns >> 10);
+    const uint32_t start = state == 0 ? now : (uint32_t)state, run = state == 0 || !running ? now : (uint32_t)(state >> 32);
+    if (now - run > limit || (now - start) / CARRY_START_LIMITS > limit) return ~0ull;
+    return ((uint64_t)run << 32) | start;
 }
 
 // The failure path of every role, out of line: inlined at six places it cost the hot loops registers (eight-byte spills; B1 T65536
@@ -568,6 +591,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
         if (n_shared > 0 && part == 0) {
             for (int s = 0; s < f.B - B_whole; ++s)
                 epoch_s[s * CH] = ld_volatile_u32(p.agg + ((size_t)group * p.tiles_total + (size_t)(s + 1) * p.tps - 1) * CH + c_own);
+            asm volatile("st.global.b32 [%0], %1;" ::"l"(&p.agg[((size_t)group * p.tiles_total + kcta) * CH + c_own].y), "r"((p.tag + epoch_s[(kcta / p.tps) * CH]) ^ RUNNING) : "memory");
             __syncwarp();
             if (merged && lane == 0) mbar_arrive(BAR_EPOCH(q));
         }
@@ -621,7 +645,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
                 for (int jb = nback; jb > 0 && ok; jb -= LB) {
                     const int cnt = jb < LB ? jb : LB;   // records jb, jb - 1, ..., jb - cnt + 1 tiles back
                     uint4 r[LB];
-                    uint64_t tstart = 0;
+                    uint64_t clock = 0;
                     for (uint32_t npoll = 0;; ++npoll) {
                         bool ready = true;
 #pragma unroll
@@ -637,9 +661,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(MERGED ? MERGED_THRE
                             if (k < cnt) ready = ready && r[k].y == want_y && r[k].w == want_w;
                         if (__all_sync(0xffffffffu, ready)) break;
                         if ((npoll & 15u) == 15u) {
-                            const uint64_t tnow = gtimer();
-                            if (tstart == 0) tstart = tnow;
-                            if (*abort_flag || tnow - tstart > spin) { ok = false; break; }
+                            clock = carry_clock(clock, rec - (size_t)gidx * CH, epoch_s, gidx - jb, cnt, S, p.tps, p.tag, p.carry_ns);
+                            if (*abort_flag || clock == ~0ull) { ok = false; break; }
                         }
                         __nanosleep(32);
                     }
@@ -929,7 +952,8 @@ cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes,
     p.tag = next_call_tag();
     p.tag_wait = (a.flags & RGLRU_FLAG_TEST_CARRY_NEVER_ARRIVES) ? ~p.tag : p.tag;
     p.agg = (uint4 *)ws_body;
-    p.spin_ns = g_spin_limit_ns;
+    p.carry_ns = g_spin_limit_ns;
+    p.spin_ns = S > 1 && a.B % S != 0 ? CARRY_START_LIMITS * g_spin_limit_ns : g_spin_limit_ns;   // behind a carry every role waits as long
     if (ws_body_bytes < sm100_prefill_workspace_bytes(a.B, a.T, a.D, a.H)) return cudaErrorInvalidValue;
     const size_t h_bytes = (size_t)a.B * a.D * sizeof(float), cs_bytes = (size_t)a.B * 3 * a.D * sizeof(__nv_bfloat16);
     char *h0_copy = (char *)ws_body + agg_bytes(a.B, a.T, G), *cs_copy = h0_copy + up256(h_bytes);

@@ -124,3 +124,75 @@ def test_head_shard_reproduces_the_full_run_bit_for_bit():
     torch.cuda.synchronize()
     chd = torch.from_numpy(ch).to(y.device)
     assert torch.equal(ys, y[:, :, chd]) and torch.equal(hs, hT[:, chd]) and torch.equal(cs, cso[:, :, chd])
+
+
+def _long_decode(binding, torch, blocks):
+    """A CUDA-core decode step of `blocks` blocks of 102 KB of shared memory that each hold an SM for some hundred microseconds."""
+    D = 1024
+    inp = synth.make_inputs(1, 1, D, 1, io="f32", seed=3)
+    params = binding.Params.from_numpy(inp["params"], "f32")
+    B = 16 * blocks
+    x, h, cs, y = torch.zeros(B, D, device="cuda"), torch.zeros(B, D, device="cuda"), torch.zeros(B, 3, D, device="cuda"), torch.empty(B, D, device="cuda")
+    ws = binding.alloc_workspace(binding.make_shape(B, 1, D, 1, torch.float32), binding.OP_DECODE, x.device)
+    return lambda: binding.decode_step(x, params, h, cs, y=y, workspace=ws)
+
+
+@pytest.mark.parametrize("merge", [False, True])
+def test_a_time_split_forward_waits_for_sms_that_other_work_holds(oracle, merge):
+    """Sequences split in time over CTA pairs that need 128 SMs, while a kernel on another stream keeps most of the 148 for several times the
+    wait limit: the pairs that run wait for those that cannot start yet, and the call ends as it would have done alone."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    B, T, H = 1, 2048, 4
+    inp = synth.make_inputs(B, T, 256 * H, H, io="bf16", seed=29, with_dy=True)
+    params = binding.Params.from_numpy(inp["params"], "bf16")
+    x, branch = to_dev(inp["x"], "bf16"), to_dev(inp["dy"], "bf16") if merge else None
+    ws = binding.alloc_workspace(binding.make_shape(B, T, 256 * H, H, torch.bfloat16), binding.OP_PREFILL, x.device)
+    hold = _long_decode(binding, torch, 140)
+    call = lambda: binding.prefill(x, params, workspace=ws, gate_branch=branch)
+    s0, s1 = torch.cuda.Stream(), torch.cuda.Stream()
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s0):
+        hold()
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record(); hold(); e1.record()
+    torch.cuda.synchronize()
+    held_ns = int(e0.elapsed_time(e1) * 1e6)
+    with torch.cuda.stream(s1):
+        call()
+    torch.cuda.synchronize()
+    prev = binding.set_wait_limit_ns(held_ns // 5)
+    try:
+        with torch.cuda.stream(s0):
+            hold()
+        with torch.cuda.stream(s1):
+            y, hT, _ = call()
+        torch.cuda.synchronize()
+        assert binding.query_status(ws) == binding.OK
+    finally:
+        binding.set_wait_limit_ns(prev)
+    yr, hr, _, _ = oracle.prefill(inp["x"].astype(np.float64), f64(inp["params"]), H, gate_branch=inp["dy"].astype(np.float64) if merge else None, with_a_prod=True)
+    assert_close("y", to_np(y), yr, "bf16"); assert_close("h_T", to_np(hT), hr, "bf16")
+
+
+def test_time_split_forwards_on_two_streams(oracle):
+    """Two time-split prefills in flight at once, each wanting most of the GPU, round after round: both finish and match the oracle."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    runs = []
+    for k, (T, H) in enumerate(((2048, 4), (1500, 5))):
+        inp = synth.make_inputs(1, T, 256 * H, H, io="bf16", seed=31 + k)
+        x = to_dev(inp["x"], "bf16")
+        ws = binding.alloc_workspace(binding.make_shape(1, T, 256 * H, H, torch.bfloat16), binding.OP_PREFILL, x.device)
+        runs.append((inp, binding.Params.from_numpy(inp["params"], "bf16"), x, ws, torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for _ in range(20):
+        out = []
+        for _, params, x, ws, st in runs:
+            with torch.cuda.stream(st):
+                out.append(binding.prefill(x, params, workspace=ws))
+    torch.cuda.synchronize()
+    for (inp, _, _, ws, _), (y, hT, _) in zip(runs, out):
+        assert binding.query_status(ws) == binding.OK
+        yr, hr, _ = oracle_prefill(oracle, inp)
+        assert_close("y", to_np(y), yr, "bf16"); assert_close("h_T", to_np(hT), hr, "bf16")
