@@ -76,7 +76,8 @@ __host__ __device__ constexpr uint32_t tm_acc(int bf, int gate) { return (uint32
 // 1 - erf(z) = t (a1 + t (a2 + t (a3 + t (a4 + t a5)))) exp(-z^2), t = 1 / (1 + p z), z >= 0,
 // used as 1 - Phi(|v|) = (1 - erf) / 2 (coefficients halved) and GeLU(v) = max(v, 0) - |v| (1 - Phi(|v|)), which needs no selects.
 __device__ __forceinline__ f32x2 gelu_times2(f32x2 y, float g0, float g1) {
-    const f32x2 g = pack2(g0, g1), ga = pack2(fabsf(g0), fabsf(g1));
+    // |v| beyond 64 is as good as 64 (the exponential is 0), and its product with that 0 stays 0 when v is infinite
+    const f32x2 g = pack2(g0, g1), ga = pack2(fminf(fabsf(g0), 64.0f), fminf(fabsf(g1), 64.0f));
     const f32x2 den = fma2(ga, pack2(0.3275911f * 0.70710678f, 0.3275911f * 0.70710678f), pack2(1.0f, 1.0f));
     const f32x2 t = pack2(rcp_approx(lo2(den)), rcp_approx(hi2(den)));
     const f32x2 ez = mul2(mul2(g, g), pack2(-0.72134752f, -0.72134752f));   // -v^2 / 2 log2 e

@@ -161,3 +161,27 @@ def test_time_shares_on_the_gpu_equal_the_uncut_prefill(oracle, world, with_stat
     assert_close("y", np.concatenate([to_np(o[0]) for o in out], 1), yr, "bf16")
     assert_close("h_T", to_np(out[-1][1]), hr, "bf16")
     assert np.array_equal(to_np(out[-1][2]), cr)
+
+
+@pytest.mark.parametrize("Dh,H", [(256, 1), (96, 2)])
+def test_gate_branch_of_extreme_values(Dh, H):
+    """GeLU(v) = v Phi(v) at the ends of the number range: v for large v (infinity included), 0 for very negative v, NaN for NaN."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    from util import to_dev
+    B, T, D = 1, 40, Dh * H
+    inp = synth.make_inputs(B, T, D, H, io="bf16", seed=17)
+    params = binding.Params.from_numpy(inp["params"], "bf16")
+    x = to_dev(inp["x"], "bf16")
+    h = binding.prefill(x, params)[0].float()
+    vals = torch.tensor([float("inf"), 3e38, 1e19, 100.0, 40.0, -40.0, -100.0, -1e19, -3e38, 0.0], device="cuda")
+    branch = vals.repeat(T * D // len(vals) + 1)[:T * D].view(B, T, D).to(torch.bfloat16)
+    branch[0, 7, 11] = float("nan")
+    y = binding.prefill(x, params, gate_branch=branch)[0].float()
+    torch.cuda.synchronize()
+    want = h * torch.where(branch.float() > 0, branch.float(), torch.zeros_like(h))
+    assert torch.isnan(y[0, 7, 11])
+    y[0, 7, 11] = want[0, 7, 11] = 0.0
+    big = torch.isinf(want) | (want.abs() > 1e38)   # h was rounded to bf16 before the product here, not there: overflow may differ
+    assert torch.equal(torch.sign(y[big]), torch.sign(want[big])) and not torch.isnan(y).any()
+    assert torch.allclose(y[~big], want[~big], rtol=2e-2, atol=1e-6)
