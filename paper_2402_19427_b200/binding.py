@@ -1,9 +1,9 @@
 """Thin binding over the C ABI in ``include/rglru.h``.
 
 ``prefill``, ``decode_step`` and ``backward`` go through the native extension ``_host`` (csrc/host_binding.cpp), which checks
-the arguments, allocates the outputs and calls the library; calls that it does not take, because an argument is wrong or
-unusual, go through the ctypes path below, which names what is wrong.  Argument marshalling only: every step of the path (Conv1D, gates, decay, scan, state hand-off,
-backward) runs inside the CUDA library.  PyTorch appears here for device memory and streams.
+the arguments, allocates the outputs and calls the library, whose status it raises; calls that it does not take, because an
+argument is wrong or unusual, go through the ctypes path below, which names what is wrong.  No call reaches the library twice.
+Argument marshalling only: every step of the path (Conv1D, gates, decay, scan, state hand-off, backward) runs inside the CUDA library.  PyTorch appears here for device memory and streams.
 There is no fallback: if the shared library is missing or a call fails, an exception is raised.
 """
 from __future__ import annotations
@@ -58,6 +58,7 @@ def _native():
         if not os.path.exists(HOST_PATH):
             raise RuntimeError(f"{HOST_PATH} is missing: build it with `python -m paper_2402_19427_b200.build`")
         from . import _host as ext
+        ext.set_error_type(RglruError)
         _host = ext
     return _host
 

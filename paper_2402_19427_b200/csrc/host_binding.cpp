@@ -2,8 +2,9 @@
 //
 // A decode step or a short prompt spends a few microseconds on the GPU; marshalling its arguments through ctypes and checking
 // them in Python took longer than that (decode step, B = 1: 12 us per call from Python, host-bound).  Each function here
-// handles the calls whose arguments pass every check and returns the outputs; for anything else it launches nothing and
-// returns None, and binding.py runs its checked path, which names the argument that is wrong or raises the library's status.
+// handles the calls whose arguments pass its checks and returns the outputs.  For anything else it does not call the library and
+// returns None, and binding.py runs its checked path, which names the argument that is wrong.  A status of the library is raised
+// here: the call may have launched kernels that update state in place, so it must not be made a second time.
 #define PY_SSIZE_T_CLEAN
 #include <Python.h>
 
@@ -39,6 +40,19 @@ at::Tensor fresh(at::IntArrayRef shape, at::ScalarType dtype, c10::Device dev) {
 }
 void *current_stream() { return (void *)c10::cuda::getCurrentCUDAStream().stream(); }
 PyObject *wrap(const at::Tensor &t) { return THPVariable_Wrap(t); }
+
+// binding.py's exception type for a status of the library, RglruError(code, where)
+PyObject *error_type = nullptr;
+PyObject *raise_status(int32_t rc, const char *where) {
+    PyObject *e = PyObject_CallFunction(error_type ? error_type : PyExc_RuntimeError, "is", (int)rc, where);
+    if (e) { PyErr_SetObject((PyObject *)Py_TYPE(e), e); Py_DECREF(e); }
+    return nullptr;
+}
+PyObject *set_error_type(PyObject *, PyObject *type) {
+    Py_INCREF(type);
+    Py_XSETREF(error_type, type);
+    Py_RETURN_NONE;
+}
 
 // Workspace of the call: the caller's, or scratch of this call (the library needs no particular contents)
 struct Workspace {
@@ -111,7 +125,7 @@ PyObject *prefill(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const rglru_prefill_extras_t ex{ptr(gb), (float *)ptr(ap)};
     const int32_t rc = rglru_prefill_ex(&k.s, &k.h->p, ptr(x), (const float *)ptr(h0), ptr(cs), yt.data_ptr(), (float *)ht.data_ptr(), ct.data_ptr(),
                                         gb || ap ? &ex : nullptr, w.p, w.n, current_stream());
-    if (rc != RGLRU_OK) Py_RETURN_NONE;
+    if (rc != RGLRU_OK) return raise_status(rc, "rglru_prefill");
     PyObject *out = PyTuple_New(3);
     PyTuple_SET_ITEM(out, 0, wrap(yt)); PyTuple_SET_ITEM(out, 1, wrap(ht)); PyTuple_SET_ITEM(out, 2, wrap(ct));
     return out;
@@ -133,7 +147,8 @@ PyObject *decode_step(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const at::Tensor yt = y ? *y : fresh({B, D}, io, dev);
     Workspace w;
     if (!w.take(ws, k.s, RGLRU_OP_DECODE, dev)) Py_RETURN_NONE;
-    if (rglru_decode_step(&k.s, &k.h->p, ptr(x), (float *)ptr(h), ptr(cs), yt.data_ptr(), w.p, w.n, current_stream()) != RGLRU_OK) Py_RETURN_NONE;
+    const int32_t rc = rglru_decode_step(&k.s, &k.h->p, ptr(x), (float *)ptr(h), ptr(cs), yt.data_ptr(), w.p, w.n, current_stream());
+    if (rc != RGLRU_OK) return raise_status(rc, "rglru_decode_step");
     if (y) { Py_INCREF(a[6]); return a[6]; }
     return wrap(yt);
     END_HANDLE_TH_ERRORS
@@ -166,7 +181,7 @@ PyObject *backward(PyObject *, PyObject *const *a, Py_ssize_t n) {
     auto f = [&](int i) { return (float *)g[i].data_ptr(); };
     const int32_t rc = rglru_backward(&k.s, &k.h->p, ptr(x), (const float *)ptr(h0), ptr(cs), ptr(y), ptr(dy), g[0].data_ptr(), f(1), f(2), f(3), f(4), f(5), f(6), f(7),
                                       want_state || dhT || dcs ? &sg : nullptr, w.p, w.n, current_stream());
-    if (rc != RGLRU_OK) Py_RETURN_NONE;
+    if (rc != RGLRU_OK) return raise_status(rc, "rglru_backward");
     PyObject *out = PyDict_New();
     for (int i = 0; i < count; ++i) {
         PyObject *t = wrap(g[i]);
@@ -178,6 +193,7 @@ PyObject *backward(PyObject *, PyObject *const *a, Py_ssize_t n) {
 }
 
 PyMethodDef methods[] = {
+    {"set_error_type", set_error_type, METH_O, nullptr},
     {"params_handle", (PyCFunction)(void (*)(void))params_handle, METH_FASTCALL, nullptr},
     {"prefill", (PyCFunction)(void (*)(void))prefill, METH_FASTCALL, nullptr},
     {"decode_step", (PyCFunction)(void (*)(void))decode_step, METH_FASTCALL, nullptr},

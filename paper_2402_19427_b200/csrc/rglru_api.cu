@@ -8,6 +8,8 @@
 
 using namespace rglru;
 
+#define CK(call) do { const cudaError_t ce = (call); if (ce != cudaSuccess) return call_status(ce); } while (0)
+
 namespace {
 
 inline bool aligned(const void *p, size_t a) { return (reinterpret_cast<uintptr_t>(p) & (a - 1)) == 0; }
@@ -165,7 +167,7 @@ int32_t rglru_prefill_ex(const rglru_shape_t *s, const rglru_params_t *p, const 
         e = sm100_wide_prefill(a, (char *)workspace + WS_HEADER_BYTES, workspace_bytes - WS_HEADER_BYTES, st);
     else
         e = generic_prefill(a, s->io, (char *)workspace + WS_HEADER_BYTES, st);
-    return e == cudaSuccess ? RGLRU_OK : RGLRU_ERR_CUDA;
+    return call_status(e);
 }
 
 int32_t rglru_decode_step(const rglru_shape_t *s, const rglru_params_t *p, const void *x, float *h, void *conv_state,
@@ -189,7 +191,7 @@ int32_t rglru_decode_step(const rglru_shape_t *s, const rglru_params_t *p, const
         e = sm100_decode(a, (cudaStream_t)cuda_stream);
     else
         e = generic_decode(a, s->io, (cudaStream_t)cuda_stream);
-    return e == cudaSuccess ? RGLRU_OK : RGLRU_ERR_CUDA;
+    return call_status(e);
 }
 
 int32_t rglru_backward(const rglru_shape_t *s, const rglru_params_t *p, const void *x, const float *h0,
@@ -226,7 +228,7 @@ int32_t rglru_backward(const rglru_shape_t *s, const rglru_params_t *p, const vo
                            (cudaStream_t)cuda_stream);
     else
         e = generic_backward(f, q, s->io, (char *)workspace + WS_HEADER_BYTES, (cudaStream_t)cuda_stream);
-    return e == cudaSuccess ? RGLRU_OK : RGLRU_ERR_CUDA;
+    return call_status(e);
 }
 
 size_t rglru_host_staging_bytes(const rglru_shape_t *s) {
@@ -260,16 +262,15 @@ int32_t rglru_prefill_host(const rglru_shape_t *s, const rglru_params_t *p, cons
     const bool splittable = hp != nullptr && s->B > 1 && seq_x % 16 == 0 && seq_h % 16 == 0 && seq_c % 16 == 0;
     const int nchunks = splittable ? (s->B < HostPipe::MAX_CHUNKS ? s->B : HostPipe::MAX_CHUNKS) : 1;
     if (nchunks == 1) {
-        if (cudaMemcpyAsync(sx, x_host, xbytes, cudaMemcpyHostToDevice, st) != cudaSuccess) return RGLRU_ERR_CUDA;
+        CK(cudaMemcpyAsync(sx, x_host, xbytes, cudaMemcpyHostToDevice, st));
         rc = rglru_prefill(s, p, sx, h0, conv_state_in, sy, (float *)sh, sc, workspace, workspace_bytes, cuda_stream);
         if (rc != RGLRU_OK) return rc;
-        if (cudaMemcpyAsync(y_host, sy, xbytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) return RGLRU_ERR_CUDA;
-        if (cudaMemcpyAsync(h_T_host, sh, hbytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) return RGLRU_ERR_CUDA;
-        if (cudaMemcpyAsync(conv_state_out_host, sc, cbytes, cudaMemcpyDeviceToHost, st) != cudaSuccess) return RGLRU_ERR_CUDA;
+        CK(cudaMemcpyAsync(y_host, sy, xbytes, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(h_T_host, sh, hbytes, cudaMemcpyDeviceToHost, st));
+        CK(cudaMemcpyAsync(conv_state_out_host, sc, cbytes, cudaMemcpyDeviceToHost, st));
         return RGLRU_OK;
     }
     std::lock_guard<std::mutex> lock(hp->mutex);
-#define CK(call) do { if ((call) != cudaSuccess) return RGLRU_ERR_CUDA; } while (0)
     CK(cudaEventRecord(hp->start, st));                      // everything below follows the work already on the stream
     CK(cudaStreamWaitEvent(hp->in, hp->start, 0));
     CK(cudaStreamWaitEvent(hp->out, hp->start, 0));
@@ -293,7 +294,6 @@ int32_t rglru_prefill_host(const rglru_shape_t *s, const rglru_params_t *p, cons
     CK(cudaMemcpyAsync(conv_state_out_host, sc, cbytes, cudaMemcpyDeviceToHost, hp->out));
     CK(cudaEventRecord(hp->done, hp->out));
     CK(cudaStreamWaitEvent(st, hp->done, 0));                // later work on the caller's stream sees the results
-#undef CK
     return RGLRU_OK;
 }
 
@@ -307,11 +307,11 @@ int32_t rglru_query_status(void *workspace, void *cuda_stream) {
     if (!workspace) return RGLRU_ERR_NULL;
     cudaStream_t st = (cudaStream_t)cuda_stream;
     uint32_t word = 0;
-    if (cudaMemcpyAsync(&word, workspace, sizeof(word), cudaMemcpyDeviceToHost, st) != cudaSuccess) return RGLRU_ERR_CUDA;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return RGLRU_ERR_CUDA;
+    CK(cudaMemcpyAsync(&word, workspace, sizeof(word), cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
     if ((word & 0xFFFFFF00u) != STATUS_MAGIC) return RGLRU_OK;  // nothing recorded
-    if (cudaMemsetAsync(workspace, 0, sizeof(word), st) != cudaSuccess) return RGLRU_ERR_CUDA;
-    if (cudaStreamSynchronize(st) != cudaSuccess) return RGLRU_ERR_CUDA;
+    CK(cudaMemsetAsync(workspace, 0, sizeof(word), st));
+    CK(cudaStreamSynchronize(st));
     return (int32_t)(word & 0xFFu);
 }
 

@@ -855,9 +855,8 @@ cudaError_t launch_forward(const FwdArgs &a, const Chain &ch, cudaStream_t st) {
     const int Dh = a.D / a.H, nchunk = ceil_div(a.T, BM), ntile = ceil_div(Dh, BM);
     const size_t grid = (size_t)nchunk * a.B * a.H * ntile;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    if (Dh % 4 == 0) launch_dependent(generic_forward_kernel<IOT, SAVE, BM, true>, dim3((unsigned)grid), dim3(MT), 0, st, a, ch, nchunk, ntile);
-    else launch_dependent(generic_forward_kernel<IOT, SAVE, BM, false>, dim3((unsigned)grid), dim3(MT), 0, st, a, ch, nchunk, ntile);
-    return cudaGetLastError();
+    return launch_dependent(Dh % 4 == 0 ? generic_forward_kernel<IOT, SAVE, BM, true> : generic_forward_kernel<IOT, SAVE, BM, false>, dim3((unsigned)grid), dim3(MT), 0, st,
+                            a, ch, nchunk, ntile);
 }
 template <typename IOT, bool SAVE>
 cudaError_t forward_any(const FwdArgs &a, const Chain &ch, cudaStream_t st) {
@@ -874,17 +873,13 @@ cudaError_t launch_du(const BwdArgs &q, cudaStream_t st) {
     const int Dh = q.D / q.H, ntile = ceil_div(Dh, 2 * BM);
     const size_t grid = (size_t)ceil_div((size_t)q.B * q.T, BM) * q.H * ntile;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    if (Dh % 4 == 0) launch_dependent(generic_bwd_du_kernel<IOT, BM, true>, dim3((unsigned)grid), dim3(MT), 0, st, q, ntile);
-    else launch_dependent(generic_bwd_du_kernel<IOT, BM, false>, dim3((unsigned)grid), dim3(MT), 0, st, q, ntile);
-    return cudaGetLastError();
+    return launch_dependent(Dh % 4 == 0 ? generic_bwd_du_kernel<IOT, BM, true> : generic_bwd_du_kernel<IOT, BM, false>, dim3((unsigned)grid), dim3(MT), 0, st, q, ntile);
 }
 template <int BM>
 cudaError_t launch_dw(const BwdArgs &q, cudaStream_t st) {
     const int Dh = q.D / q.H, mtile = ceil_div(Dh, BM), ntile = ceil_div(Dh, 2 * BM);
     const unsigned grid = (unsigned)((size_t)q.S * 2 * q.H * mtile * ntile);
-    if (Dh % 4 == 0) launch_dependent(generic_bwd_dw_kernel<BM, true>, grid, dim3(MT), 0, st, q, mtile, ntile);
-    else launch_dependent(generic_bwd_dw_kernel<BM, false>, grid, dim3(MT), 0, st, q, mtile, ntile);
-    return cudaGetLastError();
+    return launch_dependent(Dh % 4 == 0 ? generic_bwd_dw_kernel<BM, true> : generic_bwd_dw_kernel<BM, false>, dim3(grid), dim3(MT), 0, st, q, mtile, ntile);
 }
 }  // namespace
 
@@ -912,21 +907,18 @@ cudaError_t generic_decode(const FwdArgs &a, int io, cudaStream_t st) {
     cudaError_t e;
     if (io == RGLRU_F32) {
         if ((e = set_smem(generic_decode_kernel<float>, smem)) != cudaSuccess) return e;
-        launch_dependent(generic_decode_kernel<float>, grid, dim3(NT), smem, st, a);
-    } else {
-        if ((e = set_smem(generic_decode_kernel<__nv_bfloat16>, smem)) != cudaSuccess) return e;
-        launch_dependent(generic_decode_kernel<__nv_bfloat16>, grid, dim3(NT), smem, st, a);
+        return launch_dependent(generic_decode_kernel<float>, grid, dim3(NT), smem, st, a);
     }
-    return cudaGetLastError();
+    if ((e = set_smem(generic_decode_kernel<__nv_bfloat16>, smem)) != cudaSuccess) return e;
+    return launch_dependent(generic_decode_kernel<__nv_bfloat16>, grid, dim3(NT), smem, st, a);
 }
 
 cudaError_t state_conv_grads(const BwdArgs &q, int io, const void *du, bool du_is_half, cudaStream_t st) {
     if (!q.dcs_in && !q.dcs_out) return cudaSuccess;
     dim3 grid((q.D + NT - 1) / NT, q.B);
-    if (io == RGLRU_F32) launch_dependent(state_conv_grads_kernel<float, float>, grid, dim3(NT), 0, st, q, (const float *)du);
-    else if (du_is_half) launch_dependent(state_conv_grads_kernel<__nv_bfloat16, __half>, grid, dim3(NT), 0, st, q, (const __half *)du);
-    else launch_dependent(state_conv_grads_kernel<__nv_bfloat16, float>, grid, dim3(NT), 0, st, q, (const float *)du);
-    return cudaGetLastError();
+    if (io == RGLRU_F32) return launch_dependent(state_conv_grads_kernel<float, float>, grid, dim3(NT), 0, st, q, (const float *)du);
+    if (du_is_half) return launch_dependent(state_conv_grads_kernel<__nv_bfloat16, __half>, grid, dim3(NT), 0, st, q, (const __half *)du);
+    return launch_dependent(state_conv_grads_kernel<__nv_bfloat16, float>, grid, dim3(NT), 0, st, q, (const float *)du);
 }
 
 void add_reduce_job(ReduceJobs &jobs, const float *in, int nparts, size_t stride, float *out0, size_t n0, float *out1, size_t n1, float *out2, size_t n2) {
@@ -940,8 +932,7 @@ cudaError_t run_reduce_jobs(const ReduceJobs &jobs, cudaStream_t st) {
     int blocks = 0;
     for (int i = 0; i < jobs.n; ++i) blocks += jobs.job[i].blocks;
     if (blocks == 0) return cudaSuccess;
-    launch_dependent(reduce_jobs_kernel, dim3(blocks), dim3(256), 0, st, jobs);
-    return cudaGetLastError();
+    return launch_dependent(reduce_jobs_kernel, dim3(blocks), dim3(256), 0, st, jobs);
 }
 
 size_t generic_backward_workspace_bytes(int B, int T, int D, int H) {
@@ -982,8 +973,8 @@ cudaError_t generic_backward(const FwdArgs &fwd_in, BwdArgs &q, int io, void *ws
     const int ctiles = ceil_div(D, 32);
     const size_t g2 = (size_t)rchunks * B * ctiles;
     if (g2 > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    if (f32) launch_dependent(generic_bwd_scan_kernel<float>, dim3((unsigned)g2), dim3(NT), 0, st, q, chr, rchunks, ctiles);
-    else launch_dependent(generic_bwd_scan_kernel<__nv_bfloat16>, dim3((unsigned)g2), dim3(NT), 0, st, q, chr, rchunks, ctiles);
+    if ((e = launch_dependent(f32 ? generic_bwd_scan_kernel<float> : generic_bwd_scan_kernel<__nv_bfloat16>, dim3((unsigned)g2), dim3(NT), 0, st, q, chr, rchunks, ctiles)) != cudaSuccess)
+        return e;
     // 3. du += W^T dz
     const size_t blocks3 = (size_t)ceil_div((size_t)B * T, 64) * H * ceil_div(Dh, 128);
     if (tile_rows(blocks3) == 64) e = f32 ? launch_du<float, 64>(q, st) : launch_du<__nv_bfloat16, 64>(q, st);
@@ -994,8 +985,7 @@ cudaError_t generic_backward(const FwdArgs &fwd_in, BwdArgs &q, int io, void *ws
     if ((e = tile_rows(blocks4) == 64 ? launch_dw<64>(q, st) : launch_dw<32>(q, st)) != cudaSuccess) return e;
     // 5. Conv1D adjoint
     dim3 g5((D + NT - 1) / NT, q.nchunk, B);
-    if (f32) launch_dependent(generic_bwd_conv_kernel<float>, g5, dim3(NT), 0, st, q);
-    else launch_dependent(generic_bwd_conv_kernel<__nv_bfloat16>, g5, dim3(NT), 0, st, q);
+    if ((e = launch_dependent(f32 ? generic_bwd_conv_kernel<float> : generic_bwd_conv_kernel<__nv_bfloat16>, g5, dim3(NT), 0, st, q)) != cudaSuccess) return e;
     if ((e = state_conv_grads(q, io, q.hp, false, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
     // 6. deterministic reductions of the partial sums
     ReduceJobs jobs{};

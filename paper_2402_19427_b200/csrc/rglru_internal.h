@@ -49,6 +49,14 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+// A call's return code.  The error goes out in the code and is not left behind in the thread's runtime state, where a later call
+// (this library's or a caller's that links the same runtime) would take it for its own.
+inline int32_t call_status(cudaError_t e) {
+    if (e == cudaSuccess) return RGLRU_OK;
+    (void)cudaGetLastError();
+    return RGLRU_ERR_CUDA;
+}
+
 // The first 256 bytes of every workspace hold the device-side status: word 0 carries
 // STATUS_MAGIC | code once a kernel has recorded a condition.  A word without the magic
 // (fresh, uninitialised scratch) reads as "nothing recorded".

@@ -81,10 +81,10 @@ extern "C" int32_t rglru_prefill_static_scratch(const rglru_shape_t *s, const rg
 
     cudaError_t e;
     unsigned char *scratch = (unsigned char *)scratch_for_current_device(&e);
-    if (scratch == nullptr) return RGLRU_ERR_CUDA;
+    if (scratch == nullptr) return call_status(e);
     cudaStream_t st = (cudaStream_t)cuda_stream;
     // the status word must start at zero; everything else in the array is tagged per call
-    if (cudaMemsetAsync(scratch, 0, WS_HEADER_BYTES, st) != cudaSuccess) return RGLRU_ERR_CUDA;
+    if ((e = cudaMemsetAsync(scratch, 0, WS_HEADER_BYTES, st)) != cudaSuccess) return call_status(e);
 
     FwdArgs a{};
     a.B = s->B; a.T = s->T; a.D = s->D; a.H = s->H; a.c = s->c;
@@ -95,5 +95,5 @@ extern "C" int32_t rglru_prefill_static_scratch(const rglru_shape_t *s, const rg
     // rglru_query_status), else in the array's header, where nothing reads it back
     a.status = status_word ? (uint32_t *)status_word : (uint32_t *)scratch;
     e = sm100_prefill(a, scratch + WS_HEADER_BYTES, STATIC_SCRATCH_BYTES - WS_HEADER_BYTES, st);
-    return e == cudaSuccess ? RGLRU_OK : RGLRU_ERR_CUDA;
+    return call_status(e);
 }

@@ -179,3 +179,38 @@ def test_calls_the_native_path_does_not_take(change, error):
     with pytest.raises(error):
         binding.prefill(params=params, **dict(args, **{name: make(args[name])}))
     assert torch.equal(binding.prefill(params=params, **args)[0], good)
+
+
+def test_a_call_that_fails_in_the_library_is_not_made_twice(oracle, monkeypatch):
+    """A batch beyond the launch limits of one of the backward's kernels (more than 65535 sequences) fails after other kernels have been
+    launched.  The error is raised by the one call that met it: nothing is launched again, and the next call, which updates state in
+    place, neither reports that error nor runs twice."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    B, D = 65536, 32
+    inp = synth.make_inputs(1, 1, D, 1, io="bf16", seed=9)
+    params = binding.Params.from_numpy(inp["params"], "bf16")
+    x = torch.zeros(B, 1, D, dtype=torch.bfloat16, device="cuda")
+    ws = binding.alloc_workspace(binding.make_shape(B, 1, D, 1, x.dtype), binding.OP_BACKWARD, x.device)
+    step = synth.make_inputs(3, 1, 64, 2, io="f32", seed=10, with_state=True)
+    p32 = binding.Params.from_numpy(step["params"], "f32")
+    x32, h, cs = to_dev(step["x"][:, 0]), to_dev(step["h0"]), to_dev(step["conv_state"])
+    calls = []
+    real = binding.load()
+
+    class Counting:
+        def __getattr__(self, name):
+            if name in ("rglru_backward", "rglru_decode_step"):
+                calls.append(name)
+            return getattr(real, name)
+
+    monkeypatch.setattr(binding, "load", lambda: Counting())
+    with pytest.raises(binding.RglruError) as e:
+        binding.backward(x, params, x, workspace=ws)
+    assert e.value.code == binding.ERR_CUDA
+    y = binding.decode_step(x32, p32, h, cs)
+    torch.cuda.synchronize()
+    assert calls == []
+    yr, hr, cr = oracle_prefill(oracle, step, h0=step["h0"].astype(np.float64), cs=step["conv_state"].astype(np.float64))
+    assert_close("y", to_np(y), yr[:, 0], "f32"); assert_close("h", to_np(h), hr, "f32")
+    assert np.array_equal(to_np(cs), cr)
