@@ -69,6 +69,16 @@ struct Workspace {
     }
 };
 
+// The call into the library without the interpreter lock: a launch can block (a full queue, a first use that loads code), and other
+// Python threads go on meanwhile.  The tensors stay alive: the caller's arguments hold them.
+template <typename F> int32_t unlocked(F &&call) {
+    int32_t rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = call();
+    Py_END_ALLOW_THREADS
+    return rc;
+}
+
 struct Call {
     const ParamsHandle *h = nullptr;
     rglru_shape_t s{};
@@ -123,8 +133,11 @@ PyObject *prefill(PyObject *, PyObject *const *a, Py_ssize_t n) {
     Workspace w;
     if (!w.take(ws, k.s, RGLRU_OP_PREFILL, dev)) Py_RETURN_NONE;
     const rglru_prefill_extras_t ex{ptr(gb), (float *)ptr(ap)};
-    const int32_t rc = rglru_prefill_ex(&k.s, &k.h->p, ptr(x), (const float *)ptr(h0), ptr(cs), yt.data_ptr(), (float *)ht.data_ptr(), ct.data_ptr(),
-                                        gb || ap ? &ex : nullptr, w.p, w.n, current_stream());
+    void *const st = current_stream();
+    const int32_t rc = unlocked([&] {
+        return rglru_prefill_ex(&k.s, &k.h->p, ptr(x), (const float *)ptr(h0), ptr(cs), yt.data_ptr(), (float *)ht.data_ptr(), ct.data_ptr(),
+                                gb || ap ? &ex : nullptr, w.p, w.n, st);
+    });
     if (rc != RGLRU_OK) return raise_status(rc, "rglru_prefill");
     PyObject *out = PyTuple_New(3);
     PyTuple_SET_ITEM(out, 0, wrap(yt)); PyTuple_SET_ITEM(out, 1, wrap(ht)); PyTuple_SET_ITEM(out, 2, wrap(ct));
@@ -147,7 +160,8 @@ PyObject *decode_step(PyObject *, PyObject *const *a, Py_ssize_t n) {
     const at::Tensor yt = y ? *y : fresh({B, D}, io, dev);
     Workspace w;
     if (!w.take(ws, k.s, RGLRU_OP_DECODE, dev)) Py_RETURN_NONE;
-    const int32_t rc = rglru_decode_step(&k.s, &k.h->p, ptr(x), (float *)ptr(h), ptr(cs), yt.data_ptr(), w.p, w.n, current_stream());
+    void *const st = current_stream();
+    const int32_t rc = unlocked([&] { return rglru_decode_step(&k.s, &k.h->p, ptr(x), (float *)ptr(h), ptr(cs), yt.data_ptr(), w.p, w.n, st); });
     if (rc != RGLRU_OK) return raise_status(rc, "rglru_decode_step");
     if (y) { Py_INCREF(a[6]); return a[6]; }
     return wrap(yt);
@@ -179,8 +193,11 @@ PyObject *backward(PyObject *, PyObject *const *a, Py_ssize_t n) {
     if (want_state) { g[8] = fresh({B, D}, at::kFloat, dev); g[9] = fresh({B, 3, D}, io, dev); }
     const rglru_state_grads_t sg{(const float *)ptr(dhT), ptr(dcs), want_state ? (float *)g[8].data_ptr() : nullptr, want_state ? g[9].data_ptr() : nullptr};
     auto f = [&](int i) { return (float *)g[i].data_ptr(); };
-    const int32_t rc = rglru_backward(&k.s, &k.h->p, ptr(x), (const float *)ptr(h0), ptr(cs), ptr(y), ptr(dy), g[0].data_ptr(), f(1), f(2), f(3), f(4), f(5), f(6), f(7),
-                                      want_state || dhT || dcs ? &sg : nullptr, w.p, w.n, current_stream());
+    void *const st = current_stream();
+    const int32_t rc = unlocked([&] {
+        return rglru_backward(&k.s, &k.h->p, ptr(x), (const float *)ptr(h0), ptr(cs), ptr(y), ptr(dy), g[0].data_ptr(), f(1), f(2), f(3), f(4), f(5), f(6), f(7),
+                              want_state || dhT || dcs ? &sg : nullptr, w.p, w.n, st);
+    });
     if (rc != RGLRU_OK) return raise_status(rc, "rglru_backward");
     PyObject *out = PyDict_New();
     for (int i = 0; i < count; ++i) {

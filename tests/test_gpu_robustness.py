@@ -196,3 +196,43 @@ def test_time_split_forwards_on_two_streams(oracle):
         assert binding.query_status(ws) == binding.OK
         yr, hr, _ = oracle_prefill(oracle, inp)
         assert_close("y", to_np(y), yr, "bf16"); assert_close("h_T", to_np(hT), hr, "bf16")
+
+
+def test_other_python_threads_run_while_a_launch_blocks():
+    """A launch into a full queue blocks until the GPU has taken some of it.  The call has given up the interpreter lock by then, so a
+    second Python thread goes on at its own pace."""
+    import threading
+    import time
+    import torch
+    from paper_2402_19427_b200 import binding
+    inp = synth.make_inputs(2, 1, 64, 2, io="f32", seed=4, with_state=True)
+    params = binding.Params.from_numpy(inp["params"], "f32")
+    x, h, cs = to_dev(inp["x"][:, 0]), to_dev(inp["h0"]), to_dev(inp["conv_state"])
+    y = torch.empty_like(x)
+    ws = binding.alloc_workspace(binding.make_shape(2, 1, 64, 2, torch.float32), binding.OP_DECODE, x.device)
+    step = lambda: binding.decode_step(x, params, h, cs, y=y, workspace=ws)
+    step()
+    torch.cuda.synchronize()
+    gaps, stop = [], threading.Event()
+
+    def tick():
+        last = time.perf_counter()
+        while not stop.is_set():
+            time.sleep(0.002)
+            now = time.perf_counter()
+            gaps.append(now - last)
+            last = now
+
+    worker = threading.Thread(target=tick)
+    worker.start()
+    torch.cuda._sleep(1_000_000_000)   # about half a second of GPU time in front of the queue
+    longest = 0.0
+    for _ in range(4000):
+        t = time.perf_counter()
+        step()
+        longest = max(longest, time.perf_counter() - t)
+    stop.set()
+    worker.join()
+    torch.cuda.synchronize()
+    assert longest > 0.1, "no launch blocked: the queue took all of them"
+    assert max(gaps) < 0.5 * longest, (max(gaps), longest)
