@@ -3,6 +3,7 @@ from __future__ import annotations
 
 import os
 import subprocess
+import sys
 import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
@@ -44,6 +45,20 @@ def _host_command():
             "-lc10", "-lc10_cuda", "-Wl,-rpath,$ORIGIN"]
 
 
+def _host_against() -> str:
+    """What the host extension is compiled against besides its sources."""
+    import torch
+    return f"{sys.version}\n{torch.__version__}\n{os.path.abspath(torch.__file__)}\n"
+
+
+def _read(path: str) -> str:
+    try:
+        with open(path) as f:
+            return f.read()
+    except OSError:
+        return ""
+
+
 def _run(cmd):
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
@@ -80,9 +95,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError("link failed:\n" + r.stdout + r.stderr)
-    # the extension refers to the library by name only, so a rebuilt library does not make it stale
-    if force or _stale(HOST_PATH, [HOST_SOURCE, os.path.join(INCLUDE, "rglru.h")]):
+    # the extension refers to the library by name only, so a rebuilt library does not make it stale; another Python or torch does
+    stamp, against = os.path.join(objdir, "host.stamp"), _host_against()
+    if force or _stale(HOST_PATH, [HOST_SOURCE, os.path.join(INCLUDE, "rglru.h")]) or _read(stamp) != against:
         _run(_host_command())
+        with open(stamp, "w") as f:
+            f.write(against)
     return LIB_PATH
 
 

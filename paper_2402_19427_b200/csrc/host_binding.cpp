@@ -140,6 +140,7 @@ PyObject *prefill(PyObject *, PyObject *const *a, Py_ssize_t n) {
     });
     if (rc != RGLRU_OK) return raise_status(rc, "rglru_prefill");
     PyObject *out = PyTuple_New(3);
+    if (!out) return nullptr;
     PyTuple_SET_ITEM(out, 0, wrap(yt)); PyTuple_SET_ITEM(out, 1, wrap(ht)); PyTuple_SET_ITEM(out, 2, wrap(ct));
     return out;
     END_HANDLE_TH_ERRORS
@@ -200,6 +201,7 @@ PyObject *backward(PyObject *, PyObject *const *a, Py_ssize_t n) {
     });
     if (rc != RGLRU_OK) return raise_status(rc, "rglru_backward");
     PyObject *out = PyDict_New();
+    if (!out) return nullptr;
     for (int i = 0; i < count; ++i) {
         PyObject *t = wrap(g[i]);
         PyDict_SetItemString(out, names[i], t);

@@ -108,3 +108,21 @@ def test_binding_fails_loudly_without_library(monkeypatch):
     monkeypatch.setattr(binding, "LIB_PATH", "/nonexistent/librglru_b200.so")
     with pytest.raises(RuntimeError, match="no CPU fallback"):
         binding.load()
+
+
+def test_host_extension_is_rebuilt_for_another_python_or_torch(monkeypatch):
+    from paper_2402_19427_b200 import build
+    build.build()
+    ran = []
+    monkeypatch.setattr(build, "_run", lambda cmd: ran.append(cmd))
+    build.build()
+    assert not ran                       # up to date
+    monkeypatch.setattr(build, "_host_against", lambda: "another torch")
+    stamp = os.path.join(os.path.dirname(build.__file__), "_build", "host.stamp")
+    kept = open(stamp).read()
+    try:
+        build.build()
+        assert len(ran) == 1 and build.HOST_SOURCE in ran[0]
+    finally:
+        with open(stamp, "w") as f:
+            f.write(kept)
