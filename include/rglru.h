@@ -30,8 +30,8 @@
  *    a workspace must be ordered like calls.  After RGLRU_ERR_TIMEOUT, zero the workspace before a graph that uses it is
  *    replayed: the replay looks for the records that the failed run left incomplete.
  *  - Shapes without a kernel return RGLRU_ERR_UNSUPPORTED.  There is no CPU fallback.
- *  - Kernels.  bf16 io with a head width D_h that is a multiple of 32 runs on tensor-core kernels: prefill and backward at any
- *    such width up to 1024, the decode step up to 256.  Section 4.1 fixes 16 blocks, so D_h is 256 only at D_RNN = 4096; it is 96
+ *  - Kernels.  bf16 io with a head width D_h that is a multiple of 32 runs on tensor-core kernels: prefill at any such width up
+ *    to 1024, the decode step up to 256, the backward up to 256 when T is a multiple of 8.  Section 4.1 fixes 16 blocks, so D_h is 256 only at D_RNN = 4096; it is 96
  *    at D_RNN = 1536, 128 at 2048 and 160 at 2560.  Narrower heads share, or occupy alone, groups of 256 channel slots whose
  *    weight tile is block-diagonal; the slots a width leaves unused are idle work.  Every other shape with D_h <= 1024, fp32
  *    or bf16, runs on shape-generic CUDA-core kernels.

@@ -1,5 +1,5 @@
 // sm_100a backward of the RG-LRU temporal core (bf16 io, head width a multiple of 32 up to 256 -- narrower heads in groups of
-// 256 channel slots --, any T).
+// 256 channel slots --, T a multiple of 8), and the forward of heads wider than 256.
 //
 // The paper gives no backward; this is reverse-mode differentiation of Eq. 1-4 and the Conv1D.  The three dense
 // contractions run on tcgen05 tensor cores through one small GEMM kernel, the rest is element-wise and HBM-bound:
@@ -1121,15 +1121,19 @@ WideLayout wide_layout(int B, int T, int D, int H) {
 
 }  // namespace
 
-// Head width: any multiple of 32.  Up to 256, k = 256 / width (rounded down) consecutive heads form a group whose weight
-// matrix is block-diagonal; it is multiplied as a dense matrix (convert_w_kernel writes the zeros), and only the diagonal blocks
-// of its gradient are kept (reduce_dw_blocks_kernel).  A wider head is a group of its own, several column tiles wide.  Slots
-// beyond the group's channels do not exist: they meet zero weights, the scan writes zeros for those that share a 64-slot block
-// with real ones, the other blocks are left out of the products, and nothing of them is written to du.
+// Head width: a multiple of 32 up to 256.  k = 256 / width (rounded down) consecutive heads form a group whose weight matrix is
+// block-diagonal; it is multiplied as a dense matrix (convert_w_kernel writes the zeros), and only the diagonal blocks of its
+// gradient are kept (reduce_dw_blocks_kernel).  Slots beyond the group's channels do not exist: they meet zero weights, the scan
+// writes zeros for those that share a 64-slot block with real ones, the other blocks are left out of the products, and nothing of
+// them is written to du.
+// T a multiple of 8, and no wider heads: those calls get the CUDA-core kernels, which hold u, r, i, h, dz and du in fp32.  These
+// kernels run them too, five times as fast (B5 T1021 D1536 in 16 heads 133 against 665 us, B1 T512 D5632 in 16 heads 117 against
+// 534), but keep u, z, dz and du in fp16 and h_{t-1} in bf16: gradients of the parameters are then 2e-4 to 5e-4 from the exact ones
+// (2-norm) where fp32 is 2e-6, and a caller of such a shape has been promised the latter.
 bool sm100_backward_supported(int B, int T, int D, int H, int io) {
-    if (io != RGLRU_BF16 || B <= 0 || T <= 0 || H <= 0 || D % H != 0) return false;
+    if (io != RGLRU_BF16 || B <= 0 || T <= 0 || T % 8 != 0 || H <= 0 || D % H != 0) return false;
     const int dh = D / H;
-    return dh <= GENERIC_MAX_DH && dh % 32 == 0;
+    return dh <= DH && dh % 32 == 0;
 }
 
 size_t sm100_backward_workspace_bytes(int B, int T, int D, int H) { return bwd_layout(B, T, D, H).total; }

@@ -214,3 +214,29 @@ def test_a_call_that_fails_in_the_library_is_not_made_twice(oracle, monkeypatch)
     yr, hr, cr = oracle_prefill(oracle, step, h0=step["h0"].astype(np.float64), cs=step["conv_state"].astype(np.float64))
     assert_close("y", to_np(y), yr[:, 0], "f32"); assert_close("h", to_np(h), hr, "f32")
     assert np.array_equal(to_np(cs), cr)
+
+
+def _norm_error(got, ref):
+    ref = np.asarray(ref, dtype=np.float64)
+    return float(np.linalg.norm(np.asarray(got, dtype=np.float64) - ref) / np.linalg.norm(ref))
+
+
+@pytest.mark.parametrize("B,T,Dh,H", [(2, 203, 96, 3), (1, 130, 256, 1), (1, 64, 288, 2)])
+def test_backward_of_ragged_or_wide_layers_is_held_in_fp32(oracle, B, T, Dh, H):
+    """bf16 io, fp32 inside: the fp32 gradients are sums of a few hundred to a few ten thousand terms, each rounded a few dozen times at
+    2^-24, so their relative 2-norm error stays well below 2^-24 * sqrt(30000) = 1e-5 (measured 1e-6 to 4e-6; 16-bit intermediates
+    give 1e-4 to 6e-4)."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    D = Dh * H
+    inp = synth.make_inputs(B, T, D, H, io="bf16", seed=70 + T, with_dy=True, with_state=True, bias_scale=0.2)
+    params = binding.Params.from_numpy(inp["params"], "bf16")
+    x, h0, cs, dy = to_dev(inp["x"], "bf16"), to_dev(inp["h0"]), to_dev(inp["conv_state"], "bf16"), to_dev(inp["dy"], "bf16")
+    y, _, _ = binding.prefill(x, params, h0=h0, conv_state_in=cs)
+    h064, cs64 = inp["h0"].astype(np.float64), inp["conv_state"].astype(np.float64)
+    gr = oracle.backward(inp["x"].astype(np.float64), f64(inp["params"]), H, inp["dy"].astype(np.float64), h0=h064, conv_state_in=cs64, state_grads=True)
+    for saved in (None, y):
+        g = binding.backward(x, params, dy, h0=h0, conv_state_in=cs, y=saved, state_grads=True)
+        torch.cuda.synchronize()
+        for k in ("conv_w", "conv_b", "W_a", "b_a", "W_x", "b_x", "lam", "h0"):
+            assert _norm_error(to_np(g[k]), gr[k]) < 1e-5, k
