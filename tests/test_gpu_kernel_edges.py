@@ -240,3 +240,22 @@ def test_backward_of_ragged_or_wide_layers_is_held_in_fp32(oracle, B, T, Dh, H):
         torch.cuda.synchronize()
         for k in ("conv_w", "conv_b", "W_a", "b_a", "W_x", "b_x", "lam", "h0"):
             assert _norm_error(to_np(g[k]), gr[k]) < 1e-5, k
+
+
+@pytest.mark.parametrize("B,T,Dh,H,gain", [(2, 136, 256, 2, 1.0), (1, 2000, 96, 3, 8.0)])
+def test_backward_without_the_forward_output_uses_the_forward_kernel(B, T, Dh, H, gain):
+    """A forward output that the caller did not keep is the one that the forward would have given him, also where the gate
+    pre-activations are large: the gradients are the same bits with it and without it."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    inp = synth.make_inputs(B, T, Dh * H, H, io="bf16", seed=33, with_dy=True, with_state=True, bias_scale=0.2)
+    for k in ("W_a", "W_x"):
+        inp["params"][k] = inp["params"][k] * gain   # a power of two: still bf16 values
+    params = binding.Params.from_numpy(inp["params"], "bf16")
+    x, h0, cs, dy = to_dev(inp["x"], "bf16"), to_dev(inp["h0"]), to_dev(inp["conv_state"], "bf16"), to_dev(inp["dy"], "bf16")
+    y, _, _ = binding.prefill(x, params, h0=h0, conv_state_in=cs)
+    kept = binding.backward(x, params, dy, h0=h0, conv_state_in=cs, y=y, state_grads=True)
+    made = binding.backward(x, params, dy, h0=h0, conv_state_in=cs, state_grads=True)
+    torch.cuda.synchronize()
+    for k in kept:
+        assert torch.equal(kept[k], made[k]), k
