@@ -58,8 +58,9 @@ struct GemmArgs {
     int hstride;       // channels of a group that exist (fewer in a partial last group) = channels from one group to the next in [.., D] arrays
     int nx, ny;        // tile grid: nx x ny x H
     int kblocks;       // MODE_DW: 64-token K blocks of a split.  MODE_Z / MODE_DU: K runs over the existing 64-slot blocks of the group
+    int planes;        // MODE_Z: 1 (fp16 operands, z in fp16), or 3: A is a sum of three bf16 planes, B is bf16, z is fp32
     int rows_valid;    // MODE_Z / MODE_DU: number of tokens; MODE_DW: 2 NS
-    void *out;         // MODE_Z: __half z[tok][H][2][NS]; MODE_DU: __half du[tok][D] (+=); MODE_DW: float part[split][2][H][NS][NS]
+    void *out;         // MODE_Z: __half or float z[tok][H][2][NS]; MODE_DU: __half du[tok][D] (+=); MODE_DW: float part[split][2][H][NS][NS]
     uint32_t *status;
     unsigned long long spin_ns;
 };
@@ -68,7 +69,7 @@ struct GemmArgs {
 // layout, accumulate in tensor memory (fp32), and leave through the eight epilogue warps.  CTAs are persistent: each
 // walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... with two accumulators, so that the epilogue of one tile overlaps
 // the loads and MMAs of the next.  Tile number -> (x, y, z) with x fastest:
-//   MODE_Z : (token tiles, 2 gates x nt, H)   A = u[tok][h][k]        B = W_gate[h][out][k]
+//   MODE_Z : (token tiles, 2 gates x nt, H)   A = u[tok][h][k]        B = W_gate[h][out][k]; with three planes of u, smallest first
 //   MODE_DU: (token tiles, nt, H)             A = dz[tok][h][k=2 NS]  B = W[gate][h][k=out][in], MN-major
 //   MODE_DW: (2 NS / 128, splits x nt, H)     A = dz[tok][h][row]     B = u[tok][h][in], both MN-major, K = this split's tokens
 // 32-byte accesses: one whole DRAM sector per thread and instruction where a thread owns a row (pointers 32-byte aligned)
@@ -83,7 +84,7 @@ __device__ __forceinline__ void ld_global_v8(const void *ptr, uint32_t (&r)[8]) 
 
 // 64-slot blocks of group h that hold channels, and the number of K blocks of a tile of that group
 __device__ __forceinline__ int slot_blocks(const GemmArgs &p, int h) { return (min(p.hstride, p.D - h * p.hstride) + 63) / 64; }
-__device__ __forceinline__ int tile_kblocks(const GemmArgs &p, int h) { return p.mode == MODE_DW ? p.kblocks : (p.mode == MODE_DU ? 2 : 1) * slot_blocks(p, h); }
+__device__ __forceinline__ int tile_kblocks(const GemmArgs &p, int h) { return p.mode == MODE_DW ? p.kblocks : (p.mode == MODE_DU ? 2 : p.planes) * slot_blocks(p, h); }
 
 __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_constant__ GemmArgs p) {
     extern __shared__ uint8_t smem_raw[];
@@ -146,7 +147,11 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                         // u is read out of the layer's [tok][D] array at the group's first channel (channels past the group's own
                         // meet zero weights; past D they read as zero); dz has the groups' own [tok][group][2][NS] layout
                         const int kc = kb < kslots ? kb * 64 : p.NS + (kb - kslots) * 64;   // MODE_DU: the second gate's slots follow the first's
-                        if (p.mode == MODE_Z) {
+                        if (p.mode == MODE_Z && p.planes == 3) {   // u[head][plane][tok][width]: past the width both operands read as zero
+                            const int pl = 2 - kb / kslots, k0 = (kb % kslots) * 64;
+                            tma_load_3d(a_dst, &p.tm_a, k0, tx * 128, h * 3 + pl, BAR_FULL(s));
+                            tma_load_3d(b_dst, tb, k0, col0, h, BAR_FULL(s));
+                        } else if (p.mode == MODE_Z) {
                             tma_load_3d(a_dst, &p.tm_a, h * p.hstride + kb * 64, tx * 128, 0, BAR_FULL(s));
                             tma_load_3d(b_dst, tb, kb * 64, col0, h, BAR_FULL(s));
                         } else {
@@ -162,7 +167,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
     } else if (warp == 1) {
         // ---- MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = make_idesc_f16(128, p.NT), idesc_mn = make_idesc_f16_mn(128, p.NT), idesc_bmn = make_idesc_f16_bmn(128, p.NT);
+            const uint32_t idesc = p.planes == 3 ? make_idesc(128, p.NT) : make_idesc_f16(128, p.NT), idesc_mn = make_idesc_f16_mn(128, p.NT), idesc_bmn = make_idesc_f16_bmn(128, p.NT);
             int kbg = 0, it = 0;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
                 const int acc = it & 1;
@@ -253,7 +258,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                     tmem_ld32(tm_lane + c0, v);
                     tmem_ld_wait();
                     if (!valid) continue;
-                    if (p.mode == MODE_Z) {
+                    if (p.mode == MODE_Z && p.planes == 1) {
                         __half *dst = (__half *)p.out + (((size_t)row * p.H + h) * 2 + sel) * p.NS + col0 + c0;
 #pragma unroll
                         for (int j8 = 0; j8 < 2; ++j8) {
@@ -264,7 +269,8 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                         }
                     } else {
                         const int g = row >= p.NS, o_row = row - g * p.NS;
-                        float *dst = (float *)p.out + ((((size_t)sel * 2 + g) * p.H + h) * p.NS + o_row) * p.NS + col0 + c0;
+                        float *dst = (float *)p.out + (p.mode == MODE_Z ? (((size_t)row * p.H + h) * 2 + sel) * p.NS
+                                                                        : ((((size_t)sel * 2 + g) * p.H + h) * p.NS + o_row) * p.NS) + col0 + c0;
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             uint32_t w[8];
@@ -383,7 +389,8 @@ __device__ __forceinline__ f32x4 zero4() { return f32x4{pack2(0.f, 0.f), pack2(0
 __device__ __forceinline__ f32x4 fma4(const f32x4 &x, const f32x4 &y, const f32x4 &z) { return f32x4{fma2(x.a, y.a, z.a), fma2(x.b, y.b, z.b)}; }
 __device__ __forceinline__ f32x4 mul4(const f32x4 &x, const f32x4 &y) { return f32x4{mul2(x.a, y.a), mul2(x.b, y.b)}; }
 
-// u_t = b_c + sum_j w[j] x_{t-j} of tokens [tb, tb + n) of sequences b0, b0 + 1, ... as u[sequence][n][D]: one thread per
+// u_t = b_c + sum_j w[j] x_{t-j} of tokens [tb, tb + n) of sequences b0, b0 + 1, ... as fp16 u[sequence][n][D], or (PLANES) as
+// three bf16 values whose sum is the fp32 u exactly, u[head][plane][sequence][n][width]: one thread per
 // (sequence, 32 tokens, four adjacent channels), forward in time, eight tokens' loads in flight.  Bound by its 4 bytes per
 // element: with two channels per thread and a predicate on every token it executed 26 instructions per element (66 % of the issue
 // slots) and took 66 us on B4 T4096 D4096.  grid (ceil(D/256), ceil(n/128), sequences)
@@ -393,8 +400,18 @@ struct ConvArgs {
     const float *conv_b;
     __half *u;
     uint32_t *epoch;
+    int dh;               // PLANES: width of a head
 };
-__global__ void __launch_bounds__(256, 4) conv_forward_kernel(ConvArgs a) {
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+    return *(const uint32_t *)&v;
+}
+// what is left of (lo, hi) after the bf16 values in w: exact; nothing where w overflowed to infinity
+__device__ __forceinline__ f32x2 bf16_rest(f32x2 v, uint32_t w) {
+    const f32x2 t = bf2x(w);
+    return pack2(isinf(t.x) ? 0.0f : v.x - t.x, isinf(t.y) ? 0.0f : v.y - t.y);
+}
+template <bool PLANES> __global__ void __launch_bounds__(256, 4) conv_forward_kernel(ConvArgs a) {
     dependency_wait();
     const int d = blockIdx.x * CONV_CH + (threadIdx.x & 63) * 4, b = a.b0 + blockIdx.z;
     const int T = a.T, D = a.D, t0 = a.tb + blockIdx.y * CONV_CHUNK + (threadIdx.x >> 6) * CONV_SEG, t1 = min(a.tb + a.n, t0 + CONV_SEG);
@@ -412,12 +429,22 @@ __global__ void __launch_bounds__(256, 4) conv_forward_kernel(ConvArgs a) {
     f32x4 x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
     const uint32_t sD = (uint32_t)D / 4;   // token stride in groups of four channels
     const uint2 *px = (const uint2 *)(a.x + ((size_t)b * T + t0) * D + d);
-    uint2 *pu = (uint2 *)(a.u + ((size_t)blockIdx.z * a.n + (t0 - a.tb)) * D + d);
+    const size_t tok = (size_t)blockIdx.z * a.n + (t0 - a.tb), plane = (size_t)gridDim.z * a.n * a.dh / 4;   // plane: in uint2
+    uint2 *pu = (uint2 *)(PLANES ? a.u + (size_t)(d / a.dh) * 12 * plane + tok * a.dh + d % a.dh : a.u + tok * D + d);
+    const uint32_t su = PLANES ? (uint32_t)a.dh / 4 : sD;
     auto token = [&](uint2 xw) {
         const f32x4 x0 = bf4x(xw);
         const f32x4 uv = fma4(w[3], x3, fma4(w[2], x2, fma4(w[1], x1, fma4(w[0], x0, cb))));
-        *pu = make_uint2(pack_f16_sat(uv.a.x, uv.a.y), pack_f16_sat(uv.b.x, uv.b.y));
-        pu += sD;
+        if (PLANES) {
+            f32x4 v = uv;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                const uint2 w = make_uint2(pack_bf16(v.a.x, v.a.y), pack_bf16(v.b.x, v.b.y));
+                pu[q * plane] = w;
+                v = f32x4{bf16_rest(v.a, w.x), bf16_rest(v.b, w.y)};
+            }
+        } else *pu = make_uint2(pack_f16_sat(uv.a.x, uv.a.y), pack_f16_sat(uv.b.x, uv.b.y));
+        pu += su;
         x3 = x2; x2 = x1; x1 = x0;
     };
     int t = t0;
@@ -861,6 +888,7 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
 
 GemmArgs gemm_args(const Groups &gr, int D, uint32_t *status) {
     GemmArgs g{};
+    g.planes = 1;
     g.H = gr.G; g.D = D; g.NS = gr.NS; g.NT = gr.NT; g.nt = gr.nt; g.hstride = gr.hstride; g.status = status; g.spin_ns = g_spin_limit_ns;
     return g;
 }
@@ -892,12 +920,17 @@ cudaError_t gemm_z(const Groups &gr, int D, size_t ntok, const __half *u, const 
 
 // ------------------------------------------------------------------ forward of heads wider than 256
 // The fused prefill keeps a head's weights in the tensor memory of a CTA pair, which holds 256 channels.  A wider head runs as
-// conv_forward -> z product -> the kernel below, over at most WIDE_TOKENS tokens at a time so that the workspace stays small
-// (~7 bytes per element of a pass) and z mostly in L2; the state goes from pass to pass through h_T (and a_prod).
-// Forward scan: a block walks a 64-channel column forwards in chunks of 64 tokens, u, z_a, z_x (and the gate branch) of the
-// next chunk arriving by tiled TMA meanwhile; same shape as the reverse scan.  Bound by its 8 bytes per element.
+// conv_forward -> z product -> the kernel below, over at most WIDE_TOKENS tokens at a time so that the workspace stays small and z
+// mostly in L2; the state goes from pass to pass through h_T (and a_prod).
+// Everything between the kernels is fp32, as it is in the CUDA-core kernel that this path replaces: u goes to the tensor core as three
+// bf16 values that add up to it (24 bits) and meets the caller's bf16 weights as they are, z is fp32, the gates are libm-grade.
+// With u and z in fp16 the path took 69 us on B2 T777 D5632 in 16 heads where it takes 139 (Conv1D 15, product 56, scan 68) and the
+// CUDA cores 638, and h_T was 1e-4 from the exact one (relative 2-norm) where it is 3e-7 now and was 2e-6 on the CUDA cores.
+// Forward scan: a block walks a 64-channel column forwards in chunks of 32 tokens, four a warp, u, z_a, z_x (and the gate branch) of
+// the next chunk arriving by tiled TMA meanwhile; same shape as the reverse scan.
 struct WideScanArgs {
-    alignas(64) CUtensorMap tm_u, tm_z, tm_g;   // of the pass: [sequences][n][D], [sequences][n][G x 2 x NS]; the branch: [B][T][D]
+    alignas(64) CUtensorMap tm_u;        // [heads x 3 planes][sequences x n][width] of the pass, box 32 tokens x 64 channels
+    alignas(64) CUtensorMap tm_z, tm_g;  // z of the pass, [sequences][n][G x 2 x NS] fp32; the branch, [B][T][D]: the same box
     FwdArgs f;
     int G, hstride, NS, tiles, S, nchunk;
     int b0, nb, tb, n;                   // sequences b0 .. b0 + nb - 1, tokens tb .. tb + n - 1
@@ -906,36 +939,60 @@ struct WideScanArgs {
     uint32_t tag;
     unsigned long long spin_ns;
 };
-constexpr uint32_t WIDE_STAGE_BYTES = 4 * SCAN_TILE_BYTES;
+constexpr int WIDE_CHUNK = 32, WIDE_SEG = WIDE_CHUNK / 8;
+constexpr uint32_t WIDE_TILE_BYTES = WIDE_CHUNK * 128;   // of 64 channels of a 16-bit array; z takes two of them a gate
+constexpr uint32_t WIDE_STAGE_BYTES = 8 * WIDE_TILE_BYTES;
 constexpr uint32_t WIDE_SMEM_ALLOC = 2 * WIDE_STAGE_BYTES + 1024;
-constexpr size_t WIDE_TOKENS = 8192;
+constexpr size_t WIDE_TOKENS = 4096;
 
-template <bool POLY>
-__device__ __forceinline__ void wide_scan_column(const WideScanArgs &p, ScanShared &sh, const uint8_t *stage, uint32_t stage_addr, int bl, int k0, int group, int n0, f32x2 s2) {
-    const FwdArgs &f = p.f;
+// a_t and m_t i_t of Eq. 3-4 for one element, from 1 - a_t: eight independent chains a thread.  (As a call, with expm1f(2 L) for m
+// besides expf(L) for a: 150 instead of 139 us on B2 T777 D5632 in 16 heads, and h_T 2.0e-6 instead of 2.5e-7 from the exact one.)
+__device__ __forceinline__ float2 gates_acc(float za, float zx, float s) {
+    const float f = -expm1f(-s * sigmoid_acc(za));   // 1 - a_t; 1 - a_t^2 = f (2 - f)
+    return make_float2(1.0f - f, sqrtf(f * (2.0f - f)) * sigmoid_acc(zx));
+}
+
+__global__ void __launch_bounds__(256, 2) wide_scan_kernel(const __grid_constant__ WideScanArgs p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ ScanShared sh;
+    const uint32_t raw = smem_u32(smem_raw), stage_addr = (raw + 127u) & ~127u;
+    const uint8_t *stage = smem_raw + (stage_addr - raw);
     const int tid = threadIdx.x, lane = tid & 31, seg = tid >> 5;
+    if (tid == 0) {
+        mbar_init(smem_u32(&sh.full[0]), 1); mbar_init(smem_u32(&sh.full[1]), 1);
+        sh.abort = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    dependency_wait();
+    int bid = blockIdx.x;
+    const int k0 = bid % p.S; bid /= p.S;
+    const int n0 = (bid % p.tiles) * 64; bid /= p.tiles;
+    const int group = bid % p.G, bl = bid / p.G;
+    const FwdArgs &f = p.f;
     const int T = f.T, D = f.D, S = p.S, n = n0 + 2 * lane, d = group * p.hstride + n, b = p.b0 + bl;
     const bool cv = n < p.hstride && d < D, first = p.tb == 0, last = p.tb + p.n == T;
+    const f32x2 lam = cv ? ld2f(f.lambda + d) : pack2(0.f, 0.f);
+    const f32x2 s2 = pack2(decay_rate(lam.x, f.c), decay_rate(lam.y, f.c));
     const f32x2 ba = cv ? ld2f(f.b_a + d) : pack2(0.f, 0.f), bx = cv ? ld2f(f.b_x + d) : pack2(0.f, 0.f);
-    const f32x2 nba = mul2(ba, pack2(-LOG2E, -LOG2E)), nbx = mul2(bx, pack2(-LOG2E, -LOG2E));
-    const f32x2 ONE = pack2(1.0f, 1.0f), TWO = pack2(2.0f, 2.0f), NEG = pack2(-1.0f, -1.0f);
+    const f32x2 ONE = pack2(1.0f, 1.0f), ZERO = pack2(0.0f, 0.0f);
     const bool merged = f.gate_branch != nullptr;
     const uint32_t full0 = smem_u32(&sh.full[0]);
     auto issue = [&](int chunk, int st) {
-        const int t0 = chunk * SCAN_CHUNK, c = group * p.hstride + n0, zc = group * 2 * p.NS + n0;
+        const int t0 = chunk * WIDE_CHUNK, zc = 2 * (group * 2 * p.NS + n0);   // z in 16-bit units
         const uint32_t bar = full0 + 8u * st, dst = stage_addr + st * WIDE_STAGE_BYTES;
-        mbar_expect_tx(bar, (merged ? 4 : 3) * SCAN_TILE_BYTES);
+        mbar_expect_tx(bar, (merged ? 8 : 7) * WIDE_TILE_BYTES);
         tma_load_3d(dst, &p.tm_z, zc, t0, bl, bar);
-        tma_load_3d(dst + SCAN_TILE_BYTES, &p.tm_z, zc + p.NS, t0, bl, bar);
-        tma_load_3d(dst + 2 * SCAN_TILE_BYTES, &p.tm_u, c, t0, bl, bar);
-        if (merged) tma_load_3d(dst + 3 * SCAN_TILE_BYTES, &p.tm_g, c, p.tb + t0, b, bar);
+        tma_load_3d(dst + 2 * WIDE_TILE_BYTES, &p.tm_z, zc + 2 * p.NS, t0, bl, bar);
+        for (int q = 0; q < 3; ++q) tma_load_3d(dst + (4 + q) * WIDE_TILE_BYTES, &p.tm_u, n0, bl * p.n + t0, group * 3 + q, bar);
+        if (merged) tma_load_3d(dst + 7 * WIDE_TILE_BYTES, &p.tm_g, group * p.hstride + n0, p.tb + t0, b, bar);
     };
     if (tid == 0) {
         issue(k0, 0);
         if (k0 + S < p.nchunk) issue(k0 + S, 1);
     }
     const float *hin = first ? f.h0 : f.h_T;
-    f32x2 X = hin && cv ? ld2f(hin + (size_t)b * D + d) : pack2(0.f, 0.f);
+    f32x2 X = hin && cv ? ld2f(hin + (size_t)b * D + d) : ZERO;
     f32x2 Pc = !first && f.a_prod && cv ? ld2f(f.a_prod + (size_t)b * D + d) : ONE;   // product of a_t up to the chunk
     // through shared memory, so that the loads above have returned before this block publishes anything: the block that reaches
     // the end of the column overwrites h_T (and a_prod) once it has seen every other block's records
@@ -946,23 +1003,22 @@ __device__ __forceinline__ void wide_scan_column(const WideScanArgs &p, ScanShar
     bool ok = true;
     int it = 0;
     for (int chunk = k0; chunk < p.nchunk; chunk += S, ++it) {
-        const int st = it & 1, t0 = chunk * SCAN_CHUNK + seg * 8, nv = p.n - t0;
+        const int st = it & 1, t0 = chunk * WIDE_CHUNK + seg * WIDE_SEG, nv = p.n - t0;
         ok = warp_wait(full0 + 8u * st, (it >> 1) & 1, p.spin_ns, &sh.abort);
-        const uint32_t *sm = (const uint32_t *)(stage + st * WIDE_STAGE_BYTES) + seg * 8 * 32 + lane;
-        constexpr int TW = SCAN_TILE_BYTES / 4;
-        f32x2 P[8], h[8];
-        f32x2 Q = ONE, Hc = pack2(0.0f, 0.0f);
+        const uint8_t *sm = stage + st * WIDE_STAGE_BYTES;
+        const f32x2 *sz = (const f32x2 *)sm + seg * WIDE_SEG * 32 + lane;
+        const uint32_t *su = (const uint32_t *)(sm + 4 * WIDE_TILE_BYTES) + seg * WIDE_SEG * 32 + lane;
+        constexpr int TW = WIDE_TILE_BYTES / 4;
+        f32x2 P[WIDE_SEG], h[WIDE_SEG];
+        f32x2 Q = ONE, Hc = ZERO;
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            f32x2 r, fa;
-            gate_f2<POLY>(hf2x(sm[k * 32]), nba, s2, r, fa);
-            if (k >= nv) fa = pack2(0.f, 0.f);   // a token that does not exist holds the state: a = 1, m = 0
-            const f32x2 e = fma2(hf2x(sm[TW + k * 32]), pack2(-LOG2E, -LOG2E), nbx);
-            const f32x2 q = __fadd2_rn(pack2(ex2_approx(e.x), ex2_approx(e.y)), ONE);
-            const f32x2 gi = pack2(rcp_approx(q.x), rcp_approx(q.y));
-            const f32x2 at = fma2(fa, NEG, ONE), m2 = mul2(fa, fma2(fa, NEG, TWO));
-            const f32x2 m = pack2(sqrt_approx(m2.x), sqrt_approx(m2.y));
-            Hc = fma2(at, Hc, mul2(m, mul2(gi, hf2x(sm[2 * TW + k * 32]))));
+        for (int k = 0; k < WIDE_SEG; ++k) {
+            const f32x2 za = __fadd2_rn(sz[k * 32], ba), zx = __fadd2_rn(sz[TW + k * 32], bx);
+            const f32x2 u = __fadd2_rn(__fadd2_rn(bf2x(su[k * 32]), bf2x(su[TW + k * 32])), bf2x(su[2 * TW + k * 32]));
+            const float2 g0 = gates_acc(za.x, zx.x, s2.x), g1 = gates_acc(za.y, zx.y, s2.y);
+            // a token that does not exist holds the state (its row of u is the next sequence's)
+            const f32x2 at = k < nv ? pack2(g0.x, g1.x) : ONE, vt = k < nv ? mul2(pack2(g0.y, g1.y), u) : ZERO;
+            Hc = fma2(at, Hc, vt);
             Q = mul2(Q, at);
             P[k] = Q; h[k] = Hc;
         }
@@ -973,7 +1029,7 @@ __device__ __forceinline__ void wide_scan_column(const WideScanArgs &p, ScanShar
             if (seg == 0 && !sh.abort) {
                 uint4 *rec = p.rec + ((size_t)chunk * p.nb + bl) * D + d;
                 const size_t rstride = (size_t)p.nb * D;
-                f32x2 Qt = ONE, Gt = pack2(0.0f, 0.0f);
+                f32x2 Qt = ONE, Gt = ZERO;
 #pragma unroll
                 for (int k = 0; k < 8; ++k) { Gt = fma2(sh.agg[0][k][lane], Gt, sh.agg[1][k][lane]); Qt = mul2(Qt, sh.agg[0][k][lane]); }
                 if (cv) {
@@ -1010,16 +1066,13 @@ __device__ __forceinline__ void wide_scan_column(const WideScanArgs &p, ScanShar
         const uint32_t sD = (uint32_t)D / 2;
         uint32_t *p_y = (uint32_t *)((__nv_bfloat16 *)f.y + ((size_t)b * T + p.tb + t0) * D + d);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
+        for (int k = 0; k < WIDE_SEG; ++k) {
             f32x2 y = fma2(P[k], carry, h[k]);
             if (merged) {
-                const f32x2 g = bf2x(sm[3 * TW + k * 32]);   // y_t = h_t GeLU(branch_t), GeLU(v) = v Phi(v) (Section 2.3)
+                const f32x2 g = bf2x(su[3 * TW + k * 32]);   // y_t = h_t GeLU(branch_t), GeLU(v) = v Phi(v) (Section 2.3)
                 y = mul2(y, pack2(0.5f * g.x * (1.0f + erff(g.x * 0.70710678f)), 0.5f * g.y * (1.0f + erff(g.y * 0.70710678f))));
             }
-            if (cv && k < nv) {
-                const __nv_bfloat162 o = __floats2bfloat162_rn(y.x, y.y);
-                p_y[k * sD] = *(const uint32_t *)&o;
-            }
+            if (cv && k < nv) p_y[k * sD] = pack_bf16(y.x, y.y);
         }
         __syncthreads();   // everybody has read the stage and the segments' steps
         if (tid == 0 && chunk + 2 * S < p.nchunk) issue(chunk + 2 * S, st);
@@ -1047,50 +1100,31 @@ __device__ __forceinline__ void wide_scan_column(const WideScanArgs &p, ScanShar
     __syncthreads();
 }
 
-__global__ void __launch_bounds__(256, 2) wide_scan_kernel(const __grid_constant__ WideScanArgs p) {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ ScanShared sh;
-    const uint32_t raw = smem_u32(smem_raw), base = (raw + 127u) & ~127u;
-    if (threadIdx.x == 0) {
-        mbar_init(smem_u32(&sh.full[0]), 1); mbar_init(smem_u32(&sh.full[1]), 1);
-        sh.abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    dependency_wait();
-    int bid = blockIdx.x;
-    const int k0 = bid % p.S; bid /= p.S;
-    const int tile = bid % p.tiles; bid /= p.tiles;
-    const int group = bid % p.G, bl = bid / p.G;
-    const int n = tile * 64 + (threadIdx.x & 31) * 2, d = group * p.hstride + n;
-    const bool cv = n < p.hstride && d < p.f.D;
-    const f32x2 lam = cv ? ld2f(p.f.lambda + d) : pack2(0.f, 0.f);
-    const f32x2 s2 = cv ? pack2(decay_rate(lam.x, p.f.c), decay_rate(lam.y, p.f.c)) : pack2(0.f, 0.f);
-    uint8_t *stage = smem_raw + (base - raw);
-    if (__all_sync(0xffffffffu, s2.x <= S_POLY && s2.y <= S_POLY)) wide_scan_column<true>(p, sh, stage, base, bl, k0, group, tile * 64, s2);
-    else wide_scan_column<false>(p, sh, stage, base, bl, k0, group, tile * 64, s2);
-}
-
-WideScanArgs wide_scan_args(const Groups &gr, const FwdArgs &f, uint4 *rec, uint32_t *epoch) {
-    WideScanArgs p{};
-    p.f = f;
-    p.G = gr.G; p.hstride = gr.hstride; p.NS = gr.NS; p.tiles = (gr.hstride + 63) / 64;
-    p.rec = rec; p.epoch = epoch;
-    p.tag = next_call_tag(); p.spin_ns = g_spin_limit_ns;
-    return p;
+// z = u W^T of a pass of ntok tokens: u [head][plane][tok][width] in bf16, the caller's weights, z [tok][head][2][NS] in fp32.  The
+// tensor cores add the products of the smallest plane first, so that their roundings are small ones.
+cudaError_t wide_gemm_z(const Groups &gr, const FwdArgs &f, size_t ntok, const __half *u, float *z, cudaStream_t st) {
+    GemmArgs g = gemm_args(gr, f.D, f.status);
+    const uint64_t dh = gr.dh;
+    const uint64_t da[3] = {dh, ntok, 3 * (uint64_t)gr.G}, sa[2] = {dh * 2, dh * ntok * 2}, db[3] = {dh, dh, (uint64_t)gr.G}, sb[2] = {dh * 2, dh * dh * 2};
+    const uint32_t ba[3] = {64, 128, 1}, bb[3] = {64, (uint32_t)gr.NT, 1};
+    if (!encode_map16_3d(&g.tm_a, u, da, sa, ba, true) || !encode_map16_3d(&g.tm_b0, f.W_a, db, sb, bb, true) || !encode_map16_3d(&g.tm_b1, f.W_x, db, sb, bb, true))
+        return cudaErrorNotSupported;
+    g.mode = MODE_Z; g.planes = 3; g.rows_valid = (int)ntok; g.out = z;
+    g.nx = (int)((ntok + 127) / 128); g.ny = 2 * gr.nt;
+    return run_gemm(g, st);
 }
 // The scan of one pass (p.b0, nb, tb, n) over its u and z
-cudaError_t run_wide_scan(WideScanArgs &p, const __half *u, const __half *z, cudaStream_t st) {
+cudaError_t run_wide_scan(WideScanArgs &p, const __half *u, const float *z, cudaStream_t st) {
     static PerDeviceOptIn opt_in;
     cudaError_t e = opt_in.ensure(wide_scan_kernel, (int)WIDE_SMEM_ALLOC);
     if (e != cudaSuccess) return e;
-    const uint64_t D = p.f.D, n = p.n, wz = (uint64_t)p.G * 2 * p.NS;
-    const uint64_t du[3] = {D, n, (uint64_t)p.nb}, su[2] = {D * 2, D * n * 2};
-    const uint64_t dz[3] = {wz, n, (uint64_t)p.nb}, sz[2] = {wz * 2, wz * n * 2};
-    const uint32_t box[3] = {64, SCAN_CHUNK, 1};
-    if (!encode_map16_3d(&p.tm_u, u, du, su, box, false) || !encode_map16_3d(&p.tm_z, z, dz, sz, box, false)) return cudaErrorNotSupported;
-    if (p.f.gate_branch && !encode_bf16_map_3d(&p.tm_g, p.f.gate_branch, D, (uint64_t)p.f.T, (uint64_t)p.f.B, 64, SCAN_CHUNK, false)) return cudaErrorNotSupported;
-    p.nchunk = (p.n + SCAN_CHUNK - 1) / SCAN_CHUNK;
+    const uint64_t dh = p.hstride, n = p.n, ntok = n * p.nb, wz = (uint64_t)p.G * 2 * p.NS;
+    const uint64_t du[3] = {dh, ntok, 3 * (uint64_t)p.G}, su[2] = {dh * 2, dh * ntok * 2};
+    const uint64_t dz[3] = {2 * wz, n, (uint64_t)p.nb}, sz[2] = {wz * 4, wz * n * 4};   // fp32 as pairs of 16-bit elements
+    const uint32_t bu[3] = {64, WIDE_CHUNK, 1}, bz[3] = {128, WIDE_CHUNK, 1};
+    if (!encode_map16_3d(&p.tm_u, u, du, su, bu, false) || !encode_map16_3d(&p.tm_z, z, dz, sz, bz, false)) return cudaErrorNotSupported;
+    if (p.f.gate_branch && !encode_bf16_map_3d(&p.tm_g, p.f.gate_branch, p.f.D, (uint64_t)p.f.T, (uint64_t)p.f.B, 64, WIDE_CHUNK, false)) return cudaErrorNotSupported;
+    p.nchunk = (p.n + WIDE_CHUNK - 1) / WIDE_CHUNK;
     p.S = scan_split(p.nb * p.G * p.tiles, p.nchunk, 2 * num_sms());
     const size_t blocks = (size_t)p.nb * p.G * p.tiles * p.S;
     if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
@@ -1100,7 +1134,7 @@ cudaError_t run_wide_scan(WideScanArgs &p, const __half *u, const __half *z, cud
 // Passes over the batch: whole sequences while they fit WIDE_TOKENS, else one sequence in pieces of that length
 struct WideLayout {
     int nb, n;   // sequences and tokens of a pass, at most
-    size_t off_u, off_z, off_w16, off_rec, off_h0, total;
+    size_t off_u, off_z, off_rec, off_h0, total;
 };
 WideLayout wide_layout(int B, int T, int D, int H) {
     WideLayout L{};
@@ -1111,10 +1145,9 @@ WideLayout wide_layout(int B, int T, int D, int H) {
     const size_t tok = (size_t)L.nb * L.n;
     size_t o = 0;
     auto take = [&](size_t bytes) { const size_t at = o; o += up256(bytes); return at; };
-    L.off_u = take(tok * D * 2);
-    L.off_z = take(tok * gr.G * gr.NS * 2 * 2);
-    L.off_w16 = take(gr.W16_bytes());
-    L.off_rec = take((size_t)((L.n + SCAN_CHUNK - 1) / SCAN_CHUNK) * L.nb * D * sizeof(uint4) + 256);   // the records, then the launch counter
+    L.off_u = take(tok * D * 3 * 2);
+    L.off_z = take(tok * gr.G * gr.NS * 2 * 4);
+    L.off_rec = take((size_t)((L.n + WIDE_CHUNK - 1) / WIDE_CHUNK) * L.nb * D * sizeof(uint4) + 256);   // the records, then the launch counter
     L.off_h0 = take((size_t)B * D * 4);
     L.total = o;
     return L;
@@ -1175,7 +1208,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     // 1. fp16 weights, conv output
     if ((e = convert_w(gr, q.W_a, q.W_x, q.H, W16, st)) != cudaSuccess) return e;
     const dim3 grid_conv((D + CONV_CH - 1) / CONV_CH, L.nchunk_conv, B);
-    if ((e = launch_dependent(conv_forward_kernel, grid_conv, dim3(256), 0, st, ConvArgs{T, D, 0, 0, T, a.x, a.conv_w, a.cs_in, a.conv_b, u, a.epoch})) != cudaSuccess) return e;
+    if ((e = launch_dependent(conv_forward_kernel<false>, grid_conv, dim3(256), 0, st, ConvArgs{T, D, 0, 0, T, a.x, a.conv_w, a.cs_in, a.conv_b, u, a.epoch, gr.dh})) != cudaSuccess) return e;
 
     ReduceJobs jobs{};
     const uint64_t BT = L.BT;
@@ -1260,23 +1293,27 @@ cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_b
     const WideLayout L = wide_layout(B, T, D, a.H);
     if (ws_body_bytes < L.total) return cudaErrorInvalidValue;
     char *ws = (char *)ws_body;
-    __half *u = (__half *)(ws + L.off_u), *z = (__half *)(ws + L.off_z), *W16 = (__half *)(ws + L.off_w16);
+    __half *u = (__half *)(ws + L.off_u);
+    float *z = (float *)(ws + L.off_z);
     cudaError_t e;
-    WideScanArgs p = wide_scan_args(gr, a, (uint4 *)(ws + L.off_rec), nullptr);
-    p.epoch = (uint32_t *)(p.rec + (size_t)((L.n + SCAN_CHUNK - 1) / SCAN_CHUNK) * L.nb * D);
+    WideScanArgs p{};
+    p.f = a;
+    p.G = gr.G; p.hstride = gr.hstride; p.NS = gr.NS; p.tiles = (gr.hstride + 63) / 64;
+    p.tag = next_call_tag(); p.spin_ns = g_spin_limit_ns;
+    p.rec = (uint4 *)(ws + L.off_rec);
+    p.epoch = (uint32_t *)(p.rec + (size_t)((L.n + WIDE_CHUNK - 1) / WIDE_CHUNK) * L.nb * D);
     // blocks that share a column read the incoming state at unrelated times: an in-place update works on a copy
     const size_t hb = (size_t)B * D * sizeof(float);
     if (a.h0 && (uintptr_t)a.h0 < (uintptr_t)a.h_T + hb && (uintptr_t)a.h_T < (uintptr_t)a.h0 + hb) {
         if ((e = cudaMemcpyAsync(ws + L.off_h0, a.h0, hb, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
         p.f.h0 = (const float *)(ws + L.off_h0);
     }
-    if ((e = convert_w(gr, a.W_a, a.W_x, a.H, W16, st)) != cudaSuccess) return e;
     for (int b0 = 0; b0 < B; b0 += L.nb) {
         for (int tb = 0; tb < T; tb += L.n) {
             p.b0 = b0; p.nb = B - b0 < L.nb ? B - b0 : L.nb;
             p.tb = tb; p.n = T - tb < L.n ? T - tb : L.n;
-            if ((e = launch_dependent(conv_forward_kernel, dim3((D + CONV_CH - 1) / CONV_CH, (p.n + CONV_CHUNK - 1) / CONV_CHUNK, p.nb), dim3(256), 0, st, ConvArgs{T, D, b0, tb, p.n, (const __nv_bfloat16 *)a.x, (const __nv_bfloat16 *)a.conv_w, (const __nv_bfloat16 *)a.cs_in, a.conv_b, u, p.epoch})) != cudaSuccess) return e;
-            if ((e = gemm_z(gr, D, (size_t)p.nb * p.n, u, W16, z, a.status, st)) != cudaSuccess) return e;
+            if ((e = launch_dependent(conv_forward_kernel<true>, dim3((D + CONV_CH - 1) / CONV_CH, (p.n + CONV_CHUNK - 1) / CONV_CHUNK, p.nb), dim3(256), 0, st, ConvArgs{T, D, b0, tb, p.n, (const __nv_bfloat16 *)a.x, (const __nv_bfloat16 *)a.conv_w, (const __nv_bfloat16 *)a.cs_in, a.conv_b, u, p.epoch, gr.dh})) != cudaSuccess) return e;
+            if ((e = wide_gemm_z(gr, a, (size_t)p.nb * p.n, u, z, st)) != cudaSuccess) return e;
             if ((e = run_wide_scan(p, u, z, st)) != cudaSuccess) return e;
         }
     }

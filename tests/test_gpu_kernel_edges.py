@@ -259,3 +259,48 @@ def test_backward_without_the_forward_output_uses_the_forward_kernel(B, T, Dh, H
     torch.cuda.synchronize()
     for k in kept:
         assert torch.equal(kept[k], made[k]), k
+
+
+@pytest.mark.parametrize("B,T,Dh,H,gain", [(2, 203, 352, 2, 1.0), (1, 700, 288, 3, 8.0), (3, 33, 1024, 1, 8.0), (1, 4130, 288, 1, 1.0)])
+def test_forward_of_wide_heads_is_held_in_fp32(oracle, B, T, Dh, H, gain):
+    """Heads wider than 256, gate pre-activations of order one and of order ten, with channels of long memory: the fp32 outputs are as
+    close to the exact ones as fp32 arithmetic comes, 2^-24 * sqrt(30000) = 1e-5 over a thousand steps (measured 1e-6 to 3e-6; 16-bit
+    gate products give 1e-4 to 2e-4), and y is the rounded state.  Beyond a thousand steps the rounding of a_t = 0.99999 in the
+    channels of long memory adds up like a random walk: the CUDA-core kernel too is 9e-6 off after 9000."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    D = Dh * H
+    inp = synth.make_inputs(B, T, D, H, io="bf16", seed=44 + T, with_state=True, bias_scale=0.2)
+    p = inp["params"]
+    p["W_a"], p["W_x"] = p["W_a"] * gain, p["W_x"] * gain   # a power of two: still bf16 values
+    p["lam"][::20] = np.float32(np.log(0.9999 ** 0.125 / (1.0 - 0.9999 ** 0.125)))   # a^c = 0.9999
+    params = binding.Params.from_numpy(p, "bf16")
+    ap = torch.empty(B, D, dtype=torch.float32, device="cuda")
+    y, hT, cso = binding.prefill(to_dev(inp["x"], "bf16"), params, h0=to_dev(inp["h0"]), conv_state_in=to_dev(inp["conv_state"], "bf16"), a_prod=ap)
+    torch.cuda.synchronize()
+    yr, hr, cr, apr = oracle.prefill(inp["x"].astype(np.float64), f64(p), H, h0=inp["h0"].astype(np.float64), conv_state_in=inp["conv_state"].astype(np.float64), with_a_prod=True)
+    assert _norm_error(to_np(hT), hr) < 1e-5 * max(1.0, (T / 1000) ** 0.5)
+    assert _norm_error(to_np(y), yr) < 2.0 ** -9   # half a unit in the last of bf16's eight places, at most
+    # a product of T factors, each off by up to a few 2^-24: relative to the product itself
+    assert np.abs(to_np(ap) - apr).max() <= 4 * T * 2.0 ** -24 * np.abs(apr).max()
+    assert np.array_equal(to_np(cso), cr)
+
+
+def test_wide_heads_do_not_see_one_another(oracle):
+    """Block-diagonal gates: a NaN or an infinity in one head's inputs stays in that head, also where a head's width is no multiple of the
+    64 channels that the kernels load at once, and in its own sequence."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    B, T, Dh, H = 2, 70, 288, 3
+    inp = synth.make_inputs(B, T, Dh * H, H, io="bf16", seed=6)
+    params = binding.Params.from_numpy(inp["params"], "bf16")
+    x = to_dev(inp["x"], "bf16")
+    clean, hc, _ = binding.prefill(x, params)
+    bad = x.clone()
+    bad[1, 0, Dh] = float("nan"); bad[1, 5, 2 * Dh - 1] = float("inf")   # first and last channel of the middle head, second sequence
+    y, hT, _ = binding.prefill(bad, params)
+    torch.cuda.synchronize()
+    assert torch.isnan(y[1, 0, Dh])
+    for h in (0, 2):
+        assert torch.equal(y[:, :, h * Dh:(h + 1) * Dh], clean[:, :, h * Dh:(h + 1) * Dh]) and torch.equal(hT[:, h * Dh:(h + 1) * Dh], hc[:, h * Dh:(h + 1) * Dh])
+    assert torch.equal(y[0], clean[0]) and torch.equal(hT[0], hc[0])
