@@ -155,5 +155,7 @@ void add_reduce_job(ReduceJobs &jobs, const float *in, int nparts, size_t stride
 cudaError_t run_reduce_jobs(const ReduceJobs &jobs, cudaStream_t st);
 // A tag no other call uses: validity tag of the carry records a call publishes
 uint32_t next_call_tag();
+// Under the failure-path test flag waits look for the tag xor this, which nobody publishes
+inline uint32_t wait_flip(uint32_t flags) { return flags & RGLRU_FLAG_TEST_CARRY_NEVER_ARRIVES ? 0xFFFFFFFFu : 0u; }
 
 }  // namespace rglru

@@ -176,31 +176,15 @@ __device__ __noinline__ bool stage_weights(const CUtensorMap *tm_wa, const CUten
 // tile writes it back plus one after its look-back, which has by then seen a record of this execution from every other pair that
 // has a tile of the sequence.  Any starting value will do.  {tag + e, tag + 2 e} differs for every (tag, e), each half from epoch to
 // epoch as well.
-__device__ __forceinline__ uint32_t ld_volatile_u32(const void *ptr) {
-    uint32_t v;
-    asm volatile("ld.volatile.global.b32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
-    return v;
-}
-
-// A pair marks the record of its first time-split tile when it starts, with a word that no published record holds.  The limit of a
-// wait for records counts from when every pair waited for has left its mark: pairs that other work on the GPU keeps off the SMs are
-// no failure (with a limit of their own all the same, CARRY_START_LIMITS times as long, which the kernel's other waits share).
-constexpr uint32_t RUNNING = 0x80000000u;
-constexpr unsigned CARRY_START_LIMITS = 16;
-// One look at that clock, out of line because it is the rare path of the polls: `state` holds the time of the first look and of the
-// last one that missed a pair (units of 1024 ns), 0 before the first; the result is the next state, or ~0 when the wait is over.
+// Do the pairs of `count` time-split tiles from tile `first` on run?  See carry_clock_step; out of line because it is the rare path of the polls.
 __device__ __noinline__ uint64_t carry_clock(uint64_t state, const uint4 *rec0, const uint32_t *epoch_s, int first, int count, int S, int tps, uint32_t tag, unsigned long long limit_ns) {
     bool running = true;
     for (int k = 0; k < count; ++k) {
-        const int pair = (first + k) % S;
+        const int pair = (first + k) % S;   // whose first tile has the same number
         const uint32_t mark = tag + epoch_s[(pair / tps) * CH], v = ld_volatile_u32(&rec0[(size_t)pair * CH].y);
         running = running && (v == mark || v == (mark ^ RUNNING));
     }
-    running = __all_sync(0xffffffffu, running);
-    const uint32_t now = (uint32_t)(gtimer() >> 10) | 1u, limit = (uint32_t)(limit_ns >> 10);
-    const uint32_t start = state == 0 ? now : (uint32_t)state, run = state == 0 || !running ? now : (uint32_t)(state >> 32);
-    if (now - run > limit || (now - start) / CARRY_START_LIMITS > limit) return ~0ull;
-    return ((uint64_t)run << 32) | start;
+    return carry_clock_step(state, running, limit_ns);
 }
 
 // The failure path of every role, out of line: inlined at six places it cost the hot loops registers (eight-byte spills; B1 T65536

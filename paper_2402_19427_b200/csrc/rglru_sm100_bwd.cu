@@ -327,7 +327,7 @@ struct EwArgs {
     __half *du;                       // [tok][D]
     uint4 *rec;                       // [nchunk][B][D] carry records of the reverse scan
     uint32_t *epoch;                  // launch counter in the workspace (any starting value): part of the records' tag
-    uint32_t tag;
+    uint32_t tag, wait_flip;          // wait_flip: see rglru_internal.h
     unsigned long long spin_ns;
     uint32_t *status;
     float *part_vec;                  // [B*S][3][D]
@@ -490,7 +490,7 @@ template <bool POLY> __device__ __forceinline__ void gate_f2(f32x2 za, f32x2 nba
 // A column with idle SMs beside it is shared by S blocks that take its chunks round-robin: each chunk's step {Q, G} is
 // published before anyone waits, and a block forms its incoming carry from the one it reached S chunks ago and the S - 1
 // steps in between, in fixed order (run-to-run identical results).  The blocks of a column are neighbours in block order, so
-// with at most one partly dispatched column the resident ones always finish.
+// with at most one partly dispatched column the resident ones always finish; see carry_clock_step for other work on the GPU.
 struct ScanArgs {
     alignas(64) CUtensorMap tm_dy, tm_y, tm_u;   // [B][T][D], box 64 tokens x 64 channels
     alignas(64) CUtensorMap tm_z;                // [B][T][groups x 2 x NS], the same box
@@ -511,27 +511,54 @@ struct ScanShared {
     int abort;
 };
 
-// The first W of `left` records of a pair of channels (two adjacent ones), `stride` apart, polled until every lane sees this
-// launch's tag in both halves of each (8-byte words are written atomically: such a record is whole).  False if the wait ran out.
+// Carry records of one pair of channels (two adjacent ones) of a column whose links S blocks take round-robin; this lane's records of
+// link l are rec0 + l stride and the one behind it.
+struct Column {
+    uint4 *rec0;
+    ptrdiff_t stride;
+    int S;
+    bool cv;               // the channels exist
+    uint32_t tag, wait;    // this execution's tag, and the one waited for (another under the failure-path test flag)
+    unsigned long long limit_ns;
+};
+__device__ __forceinline__ void mark_running(const Column &c, int first_link) {
+    if (c.cv) asm volatile("st.global.b32 [%0], %1;" ::"l"(&(c.rec0 + (ptrdiff_t)first_link * c.stride)->y), "r"(c.tag ^ RUNNING) : "memory");
+}
+__device__ __forceinline__ void put_record(const Column &c, int link, f32x2 Q, f32x2 G) {
+    uint4 *rec = c.rec0 + (ptrdiff_t)link * c.stride;
+    if (!c.cv) return;
+    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec), "r"(__float_as_uint(Q.x)), "r"(c.tag), "r"(__float_as_uint(G.x)), "r"(c.tag) : "memory");
+    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec + 1), "r"(__float_as_uint(Q.y)), "r"(c.tag), "r"(__float_as_uint(G.y)), "r"(c.tag) : "memory");
+}
+// See carry_clock_step: do the blocks that write links first .. first + count - 1 run?
+__device__ __noinline__ uint64_t column_clock(uint64_t state, const uint4 *rec0, ptrdiff_t stride, int S, uint32_t tag, unsigned long long limit_ns, int first, int count) {
+    bool running = true;
+    for (int k = 0; k < count; ++k) {
+        const uint32_t v = ld_volatile_u32(&(rec0 + (ptrdiff_t)((first + k) % S) * stride)->y);
+        running = running && (v == tag || v == (tag ^ RUNNING));
+    }
+    return carry_clock_step(state, running, limit_ns);
+}
+// The first W of `left` records from link `first` on, polled until every lane sees this launch's tag in both halves of each (8-byte
+// words are written atomically: such a record is whole).  False if the wait ran out.
 template <int W>
-__device__ __forceinline__ bool read_records(const uint4 *rec, ptrdiff_t stride, int left, bool cv, uint32_t tag, unsigned long long spin_ns, uint4 (&w0)[W], uint4 (&w1)[W]) {
-    uint64_t tstart = 0;
+__device__ __forceinline__ bool read_records(const Column &c, int first, int left, uint4 (&w0)[W], uint4 (&w1)[W]) {
+    uint64_t clock = 0;
     for (uint32_t npoll = 0;; ++npoll) {
         bool ready = true;
 #pragma unroll
         for (int k = 0; k < W; ++k) {
-            if (k < left && cv) {
-                const uint4 *src = rec + (ptrdiff_t)k * stride;
+            if (k < left && c.cv) {
+                const uint4 *src = c.rec0 + (ptrdiff_t)(first + k) * c.stride;
                 asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w0[k].x), "=r"(w0[k].y), "=r"(w0[k].z), "=r"(w0[k].w) : "l"(src) : "memory");
                 asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w1[k].x), "=r"(w1[k].y), "=r"(w1[k].z), "=r"(w1[k].w) : "l"(src + 1) : "memory");
-                ready = ready && w0[k].y == tag && w0[k].w == tag && w1[k].y == tag && w1[k].w == tag;
+                ready = ready && w0[k].y == c.wait && w0[k].w == c.wait && w1[k].y == c.wait && w1[k].w == c.wait;
             }
         }
         if (__all_sync(0xffffffffu, ready)) return true;
         if ((npoll & 31u) == 31u) {
-            const uint64_t tnow = gtimer();
-            if (tstart == 0) tstart = tnow;
-            if (__any_sync(0xffffffffu, tnow - tstart > spin_ns)) return false;
+            clock = column_clock(clock, c.rec0, c.stride, c.S, c.tag, c.limit_ns, first, !c.cv ? 0 : left < W ? left : W);
+            if (clock == ~0ull) return false;
         }
     }
 }
@@ -566,6 +593,8 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
     f32x2 X = a.dh_T && cv ? ld2f(a.dh_T + (size_t)b * D + d) : pack2(0.f, 0.f);
     f32x2 s_lam = pack2(0.f, 0.f), s_ba = s_lam, s_bx = s_lam;
     const uint32_t tag = S > 1 ? a.tag + *a.epoch * 0x9E3779B1u : 0u;
+    auto column = [&]() { return Column{a.rec + ((size_t)(a.nchunk - 1) * a.B + b) * D + d, -(ptrdiff_t)a.B * D, S, cv, tag, tag ^ a.wait_flip, a.spin_ns}; };
+    if (S > 1 && seg == 0) mark_running(column(), k0);
     bool ok = true;
     int it = 0;
     for (int link = k0; link < a.nchunk; link += S, ++it) {
@@ -593,18 +622,14 @@ __device__ __forceinline__ void scan_column(const ScanArgs &p, ScanShared &sh, c
         __syncthreads();
         if (S > 1) {
             if (seg == 0 && !sh.abort) {
-                uint4 *rec = a.rec + ((size_t)chunk * a.B + b) * D + d;
-                const size_t rstride = (size_t)a.B * D;   // the next later chunk
                 f32x2 Qt = ONE, Gt = pack2(0.0f, 0.0f);
 #pragma unroll
                 for (int k = 7; k >= 0; --k) { Gt = fma2(sh.agg[0][k][lane], Gt, sh.agg[1][k][lane]); Qt = mul2(Qt, sh.agg[0][k][lane]); }
-                if (cv) {
-                    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec), "r"(__float_as_uint(Qt.x)), "r"(tag), "r"(__float_as_uint(Gt.x)), "r"(tag) : "memory");
-                    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec + 1), "r"(__float_as_uint(Qt.y)), "r"(tag), "r"(__float_as_uint(Gt.y)), "r"(tag) : "memory");
-                }
-                for (int jb = min(link, S - 1); jb > 0 && ok; jb -= SCAN_WINDOW) {   // records jb, jb - 1, ... chunks later, farthest first
+                const Column col = column();
+                put_record(col, link, Qt, Gt);
+                for (int jb = min(link, S - 1); jb > 0 && ok; jb -= SCAN_WINDOW) {   // links link - jb, link - jb + 1, ...
                     uint4 w0[SCAN_WINDOW], w1[SCAN_WINDOW];
-                    ok = read_records<SCAN_WINDOW>(rec + (size_t)jb * rstride, -(ptrdiff_t)rstride, jb, cv, tag, a.spin_ns, w0, w1);
+                    ok = read_records<SCAN_WINDOW>(col, link - jb, jb, w0, w1);
                     if (!ok) break;
 #pragma unroll
                     for (int k = 0; k < SCAN_WINDOW; ++k)
@@ -936,7 +961,7 @@ struct WideScanArgs {
     int b0, nb, tb, n;                   // sequences b0 .. b0 + nb - 1, tokens tb .. tb + n - 1
     uint4 *rec;                          // [nchunk][nb][D] carry records
     uint32_t *epoch;
-    uint32_t tag;
+    uint32_t tag, wait_flip;             // wait_flip: see rglru_internal.h
     unsigned long long spin_ns;
 };
 constexpr int WIDE_CHUNK = 32, WIDE_SEG = WIDE_CHUNK / 8;
@@ -1000,6 +1025,8 @@ __global__ void __launch_bounds__(256, 2) wide_scan_kernel(const __grid_constant
     __syncthreads();
     X = sh.xin[lane]; Pc = sh.pin[lane];
     const uint32_t tag = S > 1 ? p.tag + *p.epoch * 0x9E3779B1u : 0u;
+    auto column = [&]() { return Column{p.rec + (size_t)bl * D + d, (ptrdiff_t)p.nb * D, S, cv, tag, tag ^ p.wait_flip, p.spin_ns}; };
+    if (S > 1 && seg == 0) mark_running(column(), k0);
     bool ok = true;
     int it = 0;
     for (int chunk = k0; chunk < p.nchunk; chunk += S, ++it) {
@@ -1027,18 +1054,14 @@ __global__ void __launch_bounds__(256, 2) wide_scan_kernel(const __grid_constant
         __syncthreads();
         if (S > 1) {
             if (seg == 0 && !sh.abort) {
-                uint4 *rec = p.rec + ((size_t)chunk * p.nb + bl) * D + d;
-                const size_t rstride = (size_t)p.nb * D;
                 f32x2 Qt = ONE, Gt = ZERO;
 #pragma unroll
                 for (int k = 0; k < 8; ++k) { Gt = fma2(sh.agg[0][k][lane], Gt, sh.agg[1][k][lane]); Qt = mul2(Qt, sh.agg[0][k][lane]); }
-                if (cv) {
-                    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec), "r"(__float_as_uint(Qt.x)), "r"(tag), "r"(__float_as_uint(Gt.x)), "r"(tag) : "memory");
-                    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(rec + 1), "r"(__float_as_uint(Qt.y)), "r"(tag), "r"(__float_as_uint(Gt.y)), "r"(tag) : "memory");
-                }
+                const Column col = column();
+                put_record(col, chunk, Qt, Gt);
                 for (int jb = min(chunk, S - 1); jb > 0 && ok; jb -= SCAN_WINDOW) {   // records jb, jb - 1, ... chunks earlier, farthest first
                     uint4 w0[SCAN_WINDOW], w1[SCAN_WINDOW];
-                    ok = read_records<SCAN_WINDOW>(rec - (size_t)jb * rstride, rstride, jb, cv, tag, p.spin_ns, w0, w1);
+                    ok = read_records<SCAN_WINDOW>(col, chunk - jb, jb, w0, w1);
                     if (!ok) break;
 #pragma unroll
                     for (int k = 0; k < SCAN_WINDOW; ++k) {
@@ -1192,7 +1215,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     a.conv_b = fwd.conv_b; a.b_a = fwd.b_a; a.b_x = fwd.b_x; a.lambda = q.lambda; a.h0 = fwd.h0;
     a.u = u; a.dz = dz; a.z = z; a.du = du;
     a.rec = (uint4 *)(ws + L.off_rec); a.epoch = (uint32_t *)(a.rec + (size_t)B * L.nchunk * D);
-    a.tag = next_call_tag(); a.spin_ns = g_spin_limit_ns; a.status = status; a.part_vec = (float *)(ws + L.off_pvec);
+    a.tag = next_call_tag(); a.wait_flip = wait_flip(fwd.flags); a.spin_ns = g_spin_limit_ns; a.status = status; a.part_vec = (float *)(ws + L.off_pvec);
     a.dh_T = q.dh_T; a.dh0 = q.dh0;
 
     // 0. h_{t-1} comes from the forward output.  When the caller kept none the fused prefill makes it, whose gate products stay in fp32
@@ -1299,7 +1322,7 @@ cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_b
     WideScanArgs p{};
     p.f = a;
     p.G = gr.G; p.hstride = gr.hstride; p.NS = gr.NS; p.tiles = (gr.hstride + 63) / 64;
-    p.tag = next_call_tag(); p.spin_ns = g_spin_limit_ns;
+    p.tag = next_call_tag(); p.wait_flip = wait_flip(a.flags); p.spin_ns = g_spin_limit_ns;
     p.rec = (uint4 *)(ws + L.off_rec);
     p.epoch = (uint32_t *)(p.rec + (size_t)((L.n + WIDE_CHUNK - 1) / WIDE_CHUNK) * L.nb * D);
     // blocks that share a column read the incoming state at unrelated times: an in-place update works on a copy

@@ -126,6 +126,25 @@ __device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_
     asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}"
                  ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accum) : "memory");
 }
+// Blocks that wait for one another's carry records.  A block marks the record it will write first when it starts, with a word that no
+// published record holds.  The limit of a wait for records counts from when every block waited for has left its mark: blocks that
+// other work on the GPU keeps off the SMs are no failure (with a limit of their own all the same, CARRY_START_LIMITS times as long).
+constexpr uint32_t RUNNING = 0x80000000u;
+constexpr unsigned CARRY_START_LIMITS = 16;
+__device__ __forceinline__ uint32_t ld_volatile_u32(const void *ptr) {
+    uint32_t v;
+    asm volatile("ld.volatile.global.b32 %0, [%1];" : "=r"(v) : "l"(ptr) : "memory");
+    return v;
+}
+// One look at that clock: `state` holds the time of the first look and of the last one that missed a block (units of 1024 ns), 0
+// before the first; the result is the next state, or ~0 when the wait is over.  All lanes of the warp call it.
+__device__ __forceinline__ uint64_t carry_clock_step(uint64_t state, bool running, unsigned long long limit_ns) {
+    running = __all_sync(0xffffffffu, running);
+    const uint32_t now = (uint32_t)(gtimer() >> 10) | 1u, limit = (uint32_t)(limit_ns >> 10);
+    const uint32_t start = state == 0 ? now : (uint32_t)state, run = state == 0 || !running ? now : (uint32_t)(state >> 32);
+    if (now - run > limit || (now - start) / CARRY_START_LIMITS > limit) return ~0ull;
+    return ((uint64_t)run << 32) | start;
+}
 // Programmatic dependent launch (see launch_dependent): let the next kernel of the stream be scheduled; wait for the previous one
 __device__ __forceinline__ void dependency_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }

@@ -236,3 +236,38 @@ def test_other_python_threads_run_while_a_launch_blocks():
     torch.cuda.synchronize()
     assert longest > 0.1, "no launch blocked: the queue took all of them"
     assert max(gaps) < 0.5 * longest, (max(gaps), longest)
+
+
+@pytest.mark.parametrize("B,T,Dh,H,io,flags,backward", [
+    (1, 2000, 288, 1, "bf16", 0, False),                                        # blocks that share a column of the wide forward
+    (1, 2000, 256, 1, "bf16", 0, True), (1, 2000, 256, 1, "bf16", 0, "saved"),  # ... of the reverse scan; the forward in front of it
+])
+def test_every_wait_for_a_carry_is_bounded(oracle, B, T, Dh, H, io, flags, backward):
+    """As above for the other kernels that hand carries from block to block: the wait runs out, the status says so, once, and the next
+    call on the same workspace is right."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    D = Dh * H
+    inp = synth.make_inputs(B, T, D, H, io=io, seed=14, with_dy=True)
+    params = binding.Params.from_numpy(inp["params"], io)
+    x, dy = to_dev(inp["x"], io), to_dev(inp["dy"], io)
+    ws = binding.alloc_workspace(binding.make_shape(B, T, D, H, x.dtype, flags=flags), binding.OP_BACKWARD if backward else binding.OP_PREFILL, x.device)
+    y = binding.prefill(x, params, flags=flags)[0] if backward == "saved" else None
+
+    def call(f):
+        return binding.backward(x, params, dy, y=y, flags=f, workspace=ws)["x"] if backward else binding.prefill(x, params, flags=f, workspace=ws)[0]
+
+    call(flags)
+    prev = binding.set_wait_limit_ns(1_000_000)
+    try:
+        call(flags | binding.FLAG_TEST_CARRY_NEVER_ARRIVES)
+        torch.cuda.synchronize()
+        assert binding.query_status(ws) == binding.ERR_TIMEOUT
+        assert binding.query_status(ws) == binding.OK
+    finally:
+        binding.set_wait_limit_ns(prev)
+    out = call(flags)
+    torch.cuda.synchronize()
+    assert binding.query_status(ws) == binding.OK
+    ref = oracle.backward(inp["x"].astype(np.float64), f64(inp["params"]), H, inp["dy"].astype(np.float64))["x"] if backward else oracle_prefill(oracle, inp)[0]
+    assert_close("out", to_np(out), ref, io, scale=max(1.0, float(np.abs(ref).max())) if io == "f32" else 1.0)
