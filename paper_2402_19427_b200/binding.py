@@ -22,7 +22,7 @@ OK, ERR_NULL, ERR_SHAPE, ERR_UNSUPPORTED, ERR_ALIGN, ERR_WORKSPACE, ERR_CUDA, ER
 F32, BF16 = 0, 1
 OP_PREFILL, OP_DECODE, OP_BACKWARD = 0, 1, 2
 FLAG_NONE, FLAG_FORCE_GENERIC = 0, 1
-FLAG_TEST_CARRY_NEVER_ARRIVES = 0x40000000   # failure-path test hook of the tensor-core prefill (see include/rglru.h)
+FLAG_TEST_CARRY_NEVER_ARRIVES = 0x40000000   # failure-path test hook (see include/rglru.h)
 
 EXPORTED = ["rglru_abi_version", "rglru_status_string", "rglru_workspace_bytes", "rglru_prefill",
             "rglru_decode_step", "rglru_backward", "rglru_host_staging_bytes", "rglru_prefill_host",

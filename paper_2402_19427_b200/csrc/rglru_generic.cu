@@ -177,10 +177,10 @@ template <int E, bool VEC, typename T> __device__ __forceinline__ void fetch_k(c
 // One record {A, tag, B, tag2} per (sequence, channel): what the chunks so far hand to the next one.  Chunk c waits for the
 // tags of its predecessor and overwrites the record with its own; nobody else reads it, so one slot serves the whole chain.
 // The last chunk writes too: what a finished call leaves behind carries a tag that no chunk waits for, also when a CUDA graph
-// replays the call with the same tags.
+// replays the call with the same tags.  A chunk whose wait ran out says so to the next one, which gives up without a wait of its own.
 struct Chain {
     uint4 *slot;        // [B][D]
-    uint32_t tag, tag2;
+    uint32_t tag, tag2, flip;   // flip: see wait_flip
     unsigned long long spin_ns;
     uint32_t *status;
 };
@@ -190,11 +190,14 @@ __device__ __forceinline__ bool chain_wait(const Chain &ch, const uint4 *slot, b
     for (uint32_t n = 0;; ++n) {
         uint4 r = make_uint4(0u, 0u, 0u, 0u);
         if (need) asm volatile("ld.volatile.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(slot) : "memory");
-        const bool ready = !need || (r.y == ch.tag + (uint32_t)link && r.w == (ch.tag2 ^ (uint32_t)link));
+        const uint32_t ty = ch.tag + (uint32_t)link, tw = ch.tag2 ^ (uint32_t)link;
+        const bool ready = !need || (r.y == (ty ^ ch.flip) && r.w == (tw ^ ch.flip));
         if (__all_sync(0xffffffffu, ready)) {
             A = __uint_as_float(r.x); B = __uint_as_float(r.z);
             return true;
         }
+        // a failed link, whichever it is: blocks that gave up at once have overwritten one another's
+        if (__any_sync(0xffffffffu, need && r.w == ~(ch.tag2 ^ (r.y - ch.tag)))) return false;
         if ((n & 31u) == 31u) {
             const uint64_t t = ptx::gtimer();
             if (t0 == 0) t0 = t;
@@ -208,6 +211,10 @@ __device__ __forceinline__ bool chain_wait(const Chain &ch, const uint4 *slot, b
 __device__ __forceinline__ void chain_put(const Chain &ch, uint4 *slot, int link, float A, float B) {
     asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(slot), "r"(__float_as_uint(A)), "r"(ch.tag + (uint32_t)link), "r"(__float_as_uint(B)),
                  "r"(ch.tag2 ^ (uint32_t)link) : "memory");
+}
+
+__device__ __forceinline__ void chain_fail(const Chain &ch, uint4 *slot, int link) {
+    asm volatile("st.global.v4.b32 [%0], {%1, %2, %3, %4};" ::"l"(slot), "r"(0u), "r"(ch.tag + (uint32_t)link), "r"(0u), "r"(~(ch.tag2 ^ (uint32_t)link)) : "memory");
 }
 
 // ------------------------------------------------------------------ forward
@@ -370,7 +377,10 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(F
                 for (int q = 0; q < 3; ++q) cs_out[((size_t)b * 3 + q) * D + d] = keep[q];
             }
         }
-        if (!ok) ok_s = 0;
+        if (!ok) {
+            if (cv) chain_fail(ch, slot, chunk);
+            ok_s = 0;
+        }
     }
     __syncthreads();
     if (!ok_s) return;
@@ -543,7 +553,10 @@ __global__ void __launch_bounds__(NT) generic_bwd_scan_kernel(BwdArgs q, Chain c
         }
 #pragma unroll
         for (int k = 7; k >= 0; --k) { in_g[k][lane] = X; X = fmaf(agg_Q[k][lane], X, agg_g[k][lane]); }
-        if (!ok) ok_s = 0;
+        if (!ok) {
+            if (cv) chain_fail(ch, slot, link);
+            ok_s = 0;
+        }
     }
     __syncthreads();
     if (!ok_s) return;
@@ -864,9 +877,9 @@ cudaError_t forward_any(const FwdArgs &a, const Chain &ch, cudaStream_t st) {
     const size_t blocks64 = (size_t)ceil_div(a.T, 64) * a.B * a.H * ceil_div(Dh, 64);
     return tile_rows(blocks64) == 64 ? launch_forward<IOT, SAVE, 64>(a, ch, st) : launch_forward<IOT, SAVE, 32>(a, ch, st);
 }
-Chain make_chain(uint4 *slots, uint32_t *status) {
+Chain make_chain(uint4 *slots, const FwdArgs &f) {
     const uint32_t tag = next_call_tag();
-    return Chain{slots, tag, tag * 0x85EBCA6Bu + 0x27220A95u, g_spin_limit_ns, status};
+    return Chain{slots, tag, tag * 0x85EBCA6Bu + 0x27220A95u, wait_flip(f.flags), g_spin_limit_ns, f.status};
 }
 template <typename IOT, int BM>
 cudaError_t launch_du(const BwdArgs &q, cudaStream_t st) {
@@ -888,7 +901,7 @@ cudaError_t launch_dw(const BwdArgs &q, cudaStream_t st) {
 // (h0 needs none: the only block that reads a channel's h0 precedes the one that writes its h_T in the chain.)
 cudaError_t generic_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_t st) {
     FwdArgs f = a;
-    const Chain ch = make_chain((uint4 *)ws_body, a.status);
+    const Chain ch = make_chain((uint4 *)ws_body, a);
     const size_t cs_bytes = (size_t)a.B * 3 * a.D * (io == RGLRU_F32 ? 4 : 2);
     const uintptr_t ci = (uintptr_t)a.cs_in, co = (uintptr_t)a.cs_out;
     if (ci && ci < co + cs_bytes && co < ci + cs_bytes) {
@@ -966,7 +979,7 @@ cudaError_t generic_backward(const FwdArgs &fwd_in, BwdArgs &q, int io, void *ws
     // 1. forward sweep, keeping u, r, i and h_{t-1} in fp32
     FwdArgs f = fwd_in;
     f.save_u = q.u; f.save_r = q.r; f.save_i = q.gi; f.save_hprev = q.hp;
-    const Chain chf = make_chain(slots_f, fwd_in.status), chr = make_chain(slots_r, fwd_in.status);
+    const Chain chf = make_chain(slots_f, fwd_in), chr = make_chain(slots_r, fwd_in);
     cudaError_t e = f32 ? forward_any<float, true>(f, chf, st) : forward_any<__nv_bfloat16, true>(f, chf, st);
     if (e != cudaSuccess) return e;
     // 2. reverse-time scan + element-wise adjoints

@@ -239,6 +239,7 @@ def test_other_python_threads_run_while_a_launch_blocks():
 
 
 @pytest.mark.parametrize("B,T,Dh,H,io,flags,backward", [
+    (1, 700, 64, 2, "f32", 1, False), (1, 700, 64, 2, "f32", 1, True),          # chunk chains of the CUDA-core kernels
     (1, 2000, 288, 1, "bf16", 0, False),                                        # blocks that share a column of the wide forward
     (1, 2000, 256, 1, "bf16", 0, True), (1, 2000, 256, 1, "bf16", 0, "saved"),  # ... of the reverse scan; the forward in front of it
 ])
@@ -271,3 +272,30 @@ def test_every_wait_for_a_carry_is_bounded(oracle, B, T, Dh, H, io, flags, backw
     assert binding.query_status(ws) == binding.OK
     ref = oracle.backward(inp["x"].astype(np.float64), f64(inp["params"]), H, inp["dy"].astype(np.float64))["x"] if backward else oracle_prefill(oracle, inp)[0]
     assert_close("out", to_np(out), ref, io, scale=max(1.0, float(np.abs(ref).max())) if io == "f32" else 1.0)
+
+
+def test_a_failed_link_ends_the_chain_at_once():
+    """4000 chunks in a chain, of which the GPU holds less than a quarter at a time: a link that gives up tells the next, so the call ends
+    after one wait limit and not after one per wave of blocks."""
+    import time
+    import torch
+    from paper_2402_19427_b200 import binding
+    T, D = 128000, 64
+    inp = synth.make_inputs(1, 1, D, 1, io="f32", seed=15)
+    params = binding.Params.from_numpy(inp["params"], "f32")
+    x = torch.zeros(1, T, D, device="cuda")
+    ws = binding.alloc_workspace(binding.make_shape(1, T, D, 1, torch.float32), binding.OP_PREFILL, x.device)
+    y = torch.empty_like(x)
+    binding.prefill(x, params, y=y, workspace=ws)
+    torch.cuda.synchronize()
+    limit = 0.1
+    prev = binding.set_wait_limit_ns(int(limit * 1e9))
+    try:
+        t = time.perf_counter()
+        binding.prefill(x, params, y=y, workspace=ws, flags=binding.FLAG_TEST_CARRY_NEVER_ARRIVES)
+        torch.cuda.synchronize()
+        t = time.perf_counter() - t
+        assert binding.query_status(ws) == binding.ERR_TIMEOUT
+    finally:
+        binding.set_wait_limit_ns(prev)
+    assert limit < t < 2 * limit, t
