@@ -236,7 +236,9 @@ def prefill_static_scratch(x, params: Params, y, h_T, conv_state_out, h0=None, c
 
 
 def decode_step(x, params: Params, h, conv_state, c=8.0, flags=0, y=None, workspace=None):
-    """One token for B sequences; h[B,D] fp32 and conv_state[B,3,D] are updated in place; returns y[B,D]."""
+    """One token for B sequences; h[B,D] fp32 and conv_state[B,3,D] are updated in place; returns y[B,D].  The step may read the
+    parameters while the kernel before it on the stream still runs: after an in-place update of them (an optimiser step, a cast) put
+    other work or an event in between (see rglru_decode_step in include/rglru.h)."""
     out = params.native.decode_step(params.handle, x, h, conv_state, c, flags, y, workspace)
     if out is not None:
         return out

@@ -1,6 +1,6 @@
 // Shape-generic CUDA-core kernels for the RG-LRU temporal core: any head width up to
 // GENERIC_MAX_DH, fp32 or bf16 io, accurate libm-grade transcendental functions, fp32 throughout.
-// They serve the fp32 configurations, bf16 heads without a tensor-core kernel, and the backward of both.
+// They serve fp32 io, bf16 heads without a tensor-core kernel, and the backward of both, of heads wider than 256 and of ragged lengths.
 //
 // Every contraction (gate products W_a u, W_x u of Eq. 1-2; du = W^T dz; dW = dz^T u) is a register-blocked fp32 product on
 // packed FMAs: 128 threads own BM x 2 BM results, 2 TM NH = BM * BM / 64 each (64 for BM = 64), operands staged K-major
@@ -843,7 +843,8 @@ size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
 inline int ceil_div(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 
 // Rows per block of a contraction with `blocks64` blocks of 64 rows x 128 columns: three of those fit an SM, and below two per
-// SM the machine is better filled by four times as many blocks of 32 x 64 (config 0, B1 T256 D256 H2: 8 -> 64 blocks).
+// SM the machine is better filled by four times as many blocks of 32 x 64 (B1 T256 D256 in two heads: 8 -> 64 blocks).  Counted for
+// the 148 SMs of a B200 whatever the device, like the splits below, whose number the host-only workspace size has to agree with.
 constexpr int FILL_BLOCKS = 296;
 inline int tile_rows(size_t blocks64) { return blocks64 >= (size_t)FILL_BLOCKS ? 64 : 32; }
 

@@ -38,6 +38,8 @@ struct PerDeviceOptIn {
 // latency and the set-up overlap the tail of its predecessor.  A kernel lets its successor in (dependency_trigger) when its main
 // work is done, or simply by ending: triggered at the start, the successors of several small kernels came to sit beside them
 // (forward and backward of B1 T256 D256, seven launches: 81 us without, 84 us triggered at the start, 70 us at the end).
+// The exceptions are the two tensor-core decode kernels: both read the layer's parameters before they wait (rglru.h says what that
+// asks of a caller), and the one for many sequences, which fills an SM by itself, lets its successor in on entry.
 template <typename... P, typename... A>
 cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args) {
     cudaLaunchConfig_t cfg{};
@@ -113,11 +115,11 @@ cudaError_t generic_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_
 cudaError_t generic_decode(const FwdArgs &a, int io, cudaStream_t st);
 cudaError_t generic_backward(const FwdArgs &fwd, BwdArgs &b, int io, void *ws_body, cudaStream_t st);
 
-// ---- sm_100a tensor-core kernels (bf16 io, D_h = 256) ----
+// ---- sm_100a tensor-core kernels (bf16 io, D_h a multiple of 32 up to 256) ----
 bool sm100_prefill_supported(int B, int T, int D, int H, int io);
 size_t sm100_prefill_workspace_bytes(int B, int T, int D, int H);
 cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes, cudaStream_t st);
-// the same for heads wider than 256, as separate kernels
+// the same for heads wider than 256 (a multiple of 32 up to GENERIC_MAX_DH), as separate kernels
 bool sm100_wide_prefill_supported(int B, int T, int D, int H, int io);
 size_t sm100_wide_prefill_workspace_bytes(int B, int T, int D, int H);
 cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes, cudaStream_t st);
@@ -132,7 +134,7 @@ bool encode_bf16_map_3d(CUtensorMap *tm, const void *ptr, uint64_t d0, uint64_t 
 // The general form for any 16-bit element type: dims (innermost first), byte strides of dims 1 and 2, box extents.
 bool encode_map16_3d(CUtensorMap *tm, const void *ptr, const uint64_t dims[3], const uint64_t strides_bytes[2], const uint32_t box[3],
                      bool swizzle128);
-// ---- sm_100a backward (bf16 io, D_h a multiple of 32): tensor-core GEMMs around element-wise scan kernels
+// ---- sm_100a backward (bf16 io, D_h a multiple of 32 up to 256, T a multiple of 8): tensor-core GEMMs around element-wise scan kernels
 bool sm100_backward_supported(int B, int T, int D, int H, int io);
 size_t sm100_backward_workspace_bytes(int B, int T, int D, int H);
 cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &b, const void *y_saved, void *ws_body, size_t ws_body_bytes, uint32_t *status,

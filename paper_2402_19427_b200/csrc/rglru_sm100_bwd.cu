@@ -7,7 +7,7 @@
 //                        (every tensor-core operand here is fp16: 11 significant bits instead of bf16's 8 keep the
 //                        rounding of u and dz out of the gradients; finite overflow saturates at +-65504)
 //   2. GEMM              z_a | z_x = u W_a^T | u W_x^T per head (Eq. 1-2 before the sigmoid), fp16 out
-//   3. scan              reverse-time scan g_t = dy_t + a_{t+1} g_{t+1} over chunks of 64 tokens with decoupled look-back, and
+//   3. scan              reverse-time scan g_t = dy_t + a_{t+1} g_{t+1} over chunks of 64 tokens, and
 //                        the element-wise adjoints: dz_a, dz_x (fp16, token-major), the direct part of du (fp16), partial
 //                        sums of dLambda, db_a, db_x
 //   4. GEMM              du += dz_a W_a + dz_x W_x
@@ -840,8 +840,8 @@ unsigned gemm_grid(const GemmArgs &g) {
     return (unsigned)(ntiles < nsm ? ntiles : nsm);
 }
 
-// Groups of heads, the unit of the GEMMs and of the z / dz arrays: k = 256 / width (rounded down) consecutive heads, or one head
-// wider than 256.  Its NS channel slots (the channels rounded up) are nt column tiles of NT <= 256.
+// Groups of heads, the unit of the GEMMs and of the z / dz arrays: k = 256 / width (rounded down) consecutive heads, or (forward
+// only) one head wider than 256.  Its NS channel slots (the channels rounded up) are nt column tiles of NT <= 256.
 struct Groups {
     int dh, k, G, hstride, NS, NT, nt;
     size_t W16_bytes() const { return (size_t)2 * G * NS * NS * 2; }

@@ -299,3 +299,53 @@ def test_a_failed_link_ends_the_chain_at_once():
     finally:
         binding.set_wait_limit_ns(prev)
     assert limit < t < 2 * limit, t
+
+
+@pytest.mark.parametrize("B,T,Dh,H,io,merge", [
+    (2, 70, 96, 3, "bf16", False), (1, 130, 160, 3, "bf16", True), (3, 33, 32, 9, "bf16", False),   # partial last groups, unused channel slots
+    (2, 71, 288, 2, "bf16", True), (1, 4100, 288, 1, "bf16", False),                                # heads wider than 256; more than one pass
+    (2, 67, 34, 3, "bf16", False), (1, 97, 66, 2, "f32", True),                                     # CUDA-core kernels, odd widths
+])
+def test_prefill_of_other_widths_writes_only_its_outputs(oracle, B, T, Dh, H, io, merge):
+    import torch
+    from paper_2402_19427_b200 import binding
+    D, dt = Dh * H, torch.bfloat16 if io == "bf16" else torch.float32
+    inp = synth.make_inputs(B, T, D, H, io=io, seed=910 + T, with_state=True, with_dy=True)
+    params = binding.Params.from_numpy(inp["params"], io)
+    g = Guarded()
+    y, hT, cso, ap = g.empty((B, T, D), dt), g.empty((B, D), torch.float32), g.empty((B, 3, D), dt), g.empty((B, D), torch.float32)
+    ws = g.empty((binding.workspace_bytes(binding.make_shape(B, T, D, H, dt), binding.OP_PREFILL),), torch.uint8)
+    ws[:256].zero_()
+    binding.prefill(to_dev(inp["x"], io), params, h0=to_dev(inp["h0"]), conv_state_in=to_dev(inp["conv_state"], io), y=y, h_T=hT, conv_state_out=cso,
+                    workspace=ws, a_prod=ap, gate_branch=to_dev(inp["dy"], io) if merge else None)
+    g.check()
+    assert binding.query_status(ws) == binding.OK
+    yr, hr, cr, apr = oracle.prefill(inp["x"].astype(np.float64), f64(inp["params"]), H, h0=inp["h0"].astype(np.float64),
+                                     conv_state_in=inp["conv_state"].astype(np.float64), gate_branch=inp["dy"].astype(np.float64) if merge else None, with_a_prod=True)
+    assert_close("y", to_np(y), yr, io); assert_close("h_T", to_np(hT), hr, io); assert_close("a_prod", to_np(ap), apr, io)
+    assert np.array_equal(to_np(cso), cr)
+
+
+@pytest.mark.parametrize("B,T,Dh,H,io,saved", [
+    (2, 72, 96, 3, "bf16", True), (1, 136, 160, 3, "bf16", False), (3, 40, 32, 9, "bf16", True),   # tensor cores: partial groups, tails of a chunk
+    (2, 71, 96, 3, "bf16", True), (1, 64, 288, 2, "bf16", False), (2, 67, 34, 3, "f32", False),    # ragged, wide, odd widths
+])
+def test_backward_of_other_shapes_writes_only_its_outputs(B, T, Dh, H, io, saved):
+    import torch
+    from paper_2402_19427_b200 import binding
+    D, dt, f32 = Dh * H, torch.bfloat16 if io == "bf16" else torch.float32, torch.float32
+    inp = synth.make_inputs(B, T, D, H, io=io, seed=56, with_dy=True, with_state=True)
+    params = binding.Params.from_numpy(inp["params"], io)
+    x, dy, h0, cs = to_dev(inp["x"], io), to_dev(inp["dy"], io), to_dev(inp["h0"]), to_dev(inp["conv_state"], io)
+    y = binding.prefill(x, params, h0=h0, conv_state_in=cs)[0] if saved else None
+    g = Guarded()
+    out = dict(x=g.empty((B, T, D), dt), conv_w=g.empty((4, D), f32), conv_b=g.empty((D,), f32), W_a=g.empty((H, Dh, Dh), f32), b_a=g.empty((D,), f32),
+               W_x=g.empty((H, Dh, Dh), f32), b_x=g.empty((D,), f32), lam=g.empty((D,), f32), h0=g.empty((B, D), f32), conv_state=g.empty((B, 3, D), dt))
+    ws = g.empty((binding.workspace_bytes(binding.make_shape(B, T, D, H, dt), binding.OP_BACKWARD),), torch.uint8)
+    ws[:256].zero_()
+    binding.backward(x, params, dy, h0=h0, conv_state_in=cs, y=y, workspace=ws, out=out, state_grads=True, dh_T=h0, dconv_state_out=cs)
+    g.check()
+    ref = binding.backward(x, params, dy, h0=h0, conv_state_in=cs, y=y, state_grads=True, dh_T=h0, dconv_state_out=cs)
+    torch.cuda.synchronize()
+    for k, v in out.items():
+        assert torch.equal(v, ref[k]), k   # and every element of them is written: the guarded buffers started as 0xA5
