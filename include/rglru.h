@@ -35,6 +35,10 @@
  *    at D_RNN = 1536, 128 at 2048 and 160 at 2560.  Narrower heads share, or occupy alone, groups of 256 channel slots whose
  *    weight tile is block-diagonal; the slots a width leaves unused are idle work.  Every other shape with D_h <= 1024, fp32
  *    or bf16, runs on shape-generic CUDA-core kernels.
+ *  - Precision.  State and sums are fp32 everywhere.  Between their parts the CUDA-core kernels and the prefill of heads wider than
+ *    256 keep fp32 (fp32 outputs within a few 1e-6 of the exact ones, relative 2-norm).  The other tensor-core kernels use 16-bit
+ *    operands: the prefill keeps the Conv1D output and the weights in fp16 (finite overflow saturates at 65504; h_T within 1e-4), the
+ *    decode step in bf16, the backward its intermediates in fp16 and h_{t-1} in bf16 (parameter gradients within 5e-4).
  */
 #ifndef RGLRU_H_
 #define RGLRU_H_
