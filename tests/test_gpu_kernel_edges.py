@@ -304,3 +304,38 @@ def test_wide_heads_do_not_see_one_another(oracle):
     for h in (0, 2):
         assert torch.equal(y[:, :, h * Dh:(h + 1) * Dh], clean[:, :, h * Dh:(h + 1) * Dh]) and torch.equal(hT[:, h * Dh:(h + 1) * Dh], hc[:, h * Dh:(h + 1) * Dh])
     assert torch.equal(y[0], clean[0]) and torch.equal(hT[0], hc[0])
+
+
+@pytest.mark.parametrize("B,T,Dh,H", [
+    (2, 8, 256, 1), (1, 72, 256, 1), (1, 120, 96, 3),    # one chunk, tails of a chunk, a partial last group of heads
+    (1, 1208, 160, 2),                                  # a column shared by many blocks, channels beyond the last 64
+    (3, 1032, 64, 5),
+])
+def test_tensor_core_backward_at_the_edges_of_its_chunks(oracle, B, T, Dh, H):
+    """Lengths that are multiples of 8, which the tensor-core backward takes, and of no chunk of 64 tokens."""
+    forward_and_backward(oracle, B, T, Dh * H, H, "bf16", 0, seed=720 + T)
+
+
+def test_replayed_graph_of_the_tensor_core_backward(oracle):
+    """Columns shared by several blocks: a replay must not take the records that the replay before it left in the workspace."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    B, T, D, H = 1, 1208, 256, 1
+    rounds = [synth.make_inputs(B, T, D, H, io="bf16", seed=90 + k, with_dy=True) for k in range(3)]
+    params = binding.Params.from_numpy(rounds[0]["params"], "bf16")
+    x, dy = to_dev(rounds[0]["x"], "bf16"), to_dev(rounds[0]["dy"], "bf16")
+    ws = binding.alloc_workspace(binding.make_shape(B, T, D, H, x.dtype), binding.OP_BACKWARD, x.device)
+    stream = torch.cuda.Stream()
+    with torch.cuda.stream(stream):
+        binding.backward(x, params, dy, workspace=ws)   # first use outside the capture
+        stream.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            g = binding.backward(x, params, dy, workspace=ws)
+        for inp in rounds:
+            x.copy_(to_dev(inp["x"], "bf16")); dy.copy_(to_dev(inp["dy"], "bf16"))
+            graph.replay()
+            stream.synchronize()
+            gr = oracle.backward(inp["x"].astype(np.float64), f64(rounds[0]["params"]), H, inp["dy"].astype(np.float64))
+            for k in ("x", "W_a", "lam"):
+                assert_close("d" + k, to_np(g[k]), gr[k], "bf16")
