@@ -14,7 +14,7 @@ INCLUDE = os.path.join(_ROOT, "include")
 LIB_PATH = os.path.join(_PKG, "librglru_b200.so")
 HOST_PATH = os.path.join(_PKG, "_host.so")       # CPython extension behind binding.py (links against the library above)
 HOST_SOURCE = os.path.join(CSRC, "host_binding.cpp")
-SOURCES = ["rglru_api.cu", "rglru_generic.cu", "rglru_sm100.cu", "rglru_sm100_decode.cu", "rglru_sm100_bwd.cu", "rglru_static_scratch.cu"]
+SOURCES = ["rglru_api.cu", "rglru_generic.cu", "rglru_sm100.cu", "rglru_sm100_decode.cu", "rglru_sm100_bwd.cu", "rglru_sm100_split.cu", "rglru_static_scratch.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 

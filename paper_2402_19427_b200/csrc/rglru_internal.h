@@ -115,14 +115,17 @@ cudaError_t generic_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_
 cudaError_t generic_decode(const FwdArgs &a, int io, cudaStream_t st);
 cudaError_t generic_backward(const FwdArgs &fwd, BwdArgs &b, int io, void *ws_body, cudaStream_t st);
 
+// ---- fp32 products on the tensor cores (fp32 io, and bf16 calls that are fp32 between the kernels; D_h a multiple of 32) ----
+bool split_supported(int B, int T, int D, int H);
+size_t split_prefill_workspace_bytes(int B, int D, int H, int io);
+size_t split_backward_workspace_bytes(int B, int T, int D, int H, int io);
+cudaError_t split_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_t st);
+cudaError_t split_backward(const FwdArgs &fwd, BwdArgs &b, int io, void *ws_body, cudaStream_t st);
+
 // ---- sm_100a tensor-core kernels (bf16 io, D_h a multiple of 32 up to 256) ----
 bool sm100_prefill_supported(int B, int T, int D, int H, int io);
 size_t sm100_prefill_workspace_bytes(int B, int T, int D, int H);
 cudaError_t sm100_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes, cudaStream_t st);
-// the same for heads wider than 256 (a multiple of 32 up to GENERIC_MAX_DH), as separate kernels
-bool sm100_wide_prefill_supported(int B, int T, int D, int H, int io);
-size_t sm100_wide_prefill_workspace_bytes(int B, int T, int D, int H);
-cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes, cudaStream_t st);
 bool sm100_decode_supported(int B, int D, int H, int io);
 cudaError_t sm100_decode(const FwdArgs &a, cudaStream_t st);
 extern unsigned long long g_spin_limit_ns;  // every device-side wait gives up after this many nanoseconds
@@ -143,6 +146,10 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &b, const void *y_saved, 
 // on conv_state_out added to the rows it copies (dx_{T-3+k} is recomputed from du with the term added, so it is rounded once;
 // rows of conv_state_in when T < 3).  du is [B,T,D] of DUT (float or __half); io tensors are IOT.  No-op without dcs_in / dcs_out.
 cudaError_t state_conv_grads(const BwdArgs &q, int io, const void *du, bool du_is_half, cudaStream_t st);
+// Conv1D adjoint: dx, and the partial sums q.part_conv [B * conv_backward_chunks(B, T, D)][5][D] of dconv_w and dconv_b.  du is [B,T,D], fp16 beside
+// bf16 io or fp32; D a multiple of 4.
+int conv_backward_chunks(int B, int T, int D);
+cudaError_t conv_backward(const BwdArgs &q, int io, const void *du, bool du_is_half, cudaStream_t st);
 // Sums over partial results, all of a call in one launch: out[i] = sum over p of in[p * stride + i] in a fixed order (run-to-run
 // identical results), the row of n0 + n1 + n2 values being split over up to three output arrays (any may be null or empty).
 struct ReduceJob {

@@ -1,5 +1,5 @@
 // sm_100a backward of the RG-LRU temporal core (bf16 io, head width a multiple of 32 up to 256 -- narrower heads in groups of
-// 256 channel slots --, T a multiple of 8), and the forward of heads wider than 256.
+// 256 channel slots --, T a multiple of 8).
 //
 // The paper gives no backward; this is reverse-mode differentiation of Eq. 1-4 and the Conv1D.  The three dense
 // contractions run on tcgen05 tensor cores through one small GEMM kernel, the rest is element-wise and HBM-bound:
@@ -58,9 +58,8 @@ struct GemmArgs {
     int hstride;       // channels of a group that exist (fewer in a partial last group) = channels from one group to the next in [.., D] arrays
     int nx, ny;        // tile grid: nx x ny x H
     int kblocks;       // MODE_DW: 64-token K blocks of a split.  MODE_Z / MODE_DU: K runs over the existing 64-slot blocks of the group
-    int planes;        // MODE_Z: 1 (fp16 operands, z in fp16), or 3: A is a sum of three bf16 planes, B is bf16, z is fp32
     int rows_valid;    // MODE_Z / MODE_DU: number of tokens; MODE_DW: 2 NS
-    void *out;         // MODE_Z: __half or float z[tok][H][2][NS]; MODE_DU: __half du[tok][D] (+=); MODE_DW: float part[split][2][H][NS][NS]
+    void *out;         // MODE_Z: __half z[tok][H][2][NS]; MODE_DU: __half du[tok][D] (+=); MODE_DW: float part[split][2][H][NS][NS]
     uint32_t *status;
     unsigned long long spin_ns;
 };
@@ -69,7 +68,7 @@ struct GemmArgs {
 // layout, accumulate in tensor memory (fp32), and leave through the eight epilogue warps.  CTAs are persistent: each
 // walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... with two accumulators, so that the epilogue of one tile overlaps
 // the loads and MMAs of the next.  Tile number -> (x, y, z) with x fastest:
-//   MODE_Z : (token tiles, 2 gates x nt, H)   A = u[tok][h][k]        B = W_gate[h][out][k]; with three planes of u, smallest first
+//   MODE_Z : (token tiles, 2 gates x nt, H)   A = u[tok][h][k]        B = W_gate[h][out][k]
 //   MODE_DU: (token tiles, nt, H)             A = dz[tok][h][k=2 NS]  B = W[gate][h][k=out][in], MN-major
 //   MODE_DW: (2 NS / 128, splits x nt, H)     A = dz[tok][h][row]     B = u[tok][h][in], both MN-major, K = this split's tokens
 // 32-byte accesses: one whole DRAM sector per thread and instruction where a thread owns a row (pointers 32-byte aligned)
@@ -84,7 +83,7 @@ __device__ __forceinline__ void ld_global_v8(const void *ptr, uint32_t (&r)[8]) 
 
 // 64-slot blocks of group h that hold channels, and the number of K blocks of a tile of that group
 __device__ __forceinline__ int slot_blocks(const GemmArgs &p, int h) { return (min(p.hstride, p.D - h * p.hstride) + 63) / 64; }
-__device__ __forceinline__ int tile_kblocks(const GemmArgs &p, int h) { return p.mode == MODE_DW ? p.kblocks : (p.mode == MODE_DU ? 2 : p.planes) * slot_blocks(p, h); }
+__device__ __forceinline__ int tile_kblocks(const GemmArgs &p, int h) { return p.mode == MODE_DW ? p.kblocks : (p.mode == MODE_DU ? 2 : 1) * slot_blocks(p, h); }
 
 __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_constant__ GemmArgs p) {
     extern __shared__ uint8_t smem_raw[];
@@ -147,11 +146,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                         // u is read out of the layer's [tok][D] array at the group's first channel (channels past the group's own
                         // meet zero weights; past D they read as zero); dz has the groups' own [tok][group][2][NS] layout
                         const int kc = kb < kslots ? kb * 64 : p.NS + (kb - kslots) * 64;   // MODE_DU: the second gate's slots follow the first's
-                        if (p.mode == MODE_Z && p.planes == 3) {   // u[head][plane][tok][width]: past the width both operands read as zero
-                            const int pl = 2 - kb / kslots, k0 = (kb % kslots) * 64;
-                            tma_load_3d(a_dst, &p.tm_a, k0, tx * 128, h * 3 + pl, BAR_FULL(s));
-                            tma_load_3d(b_dst, tb, k0, col0, h, BAR_FULL(s));
-                        } else if (p.mode == MODE_Z) {
+                        if (p.mode == MODE_Z) {
                             tma_load_3d(a_dst, &p.tm_a, h * p.hstride + kb * 64, tx * 128, 0, BAR_FULL(s));
                             tma_load_3d(b_dst, tb, kb * 64, col0, h, BAR_FULL(s));
                         } else {
@@ -167,7 +162,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
     } else if (warp == 1) {
         // ---- MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = p.planes == 3 ? make_idesc(128, p.NT) : make_idesc_f16(128, p.NT), idesc_mn = make_idesc_f16_mn(128, p.NT), idesc_bmn = make_idesc_f16_bmn(128, p.NT);
+            const uint32_t idesc = make_idesc_f16(128, p.NT), idesc_mn = make_idesc_f16_mn(128, p.NT), idesc_bmn = make_idesc_f16_bmn(128, p.NT);
             int kbg = 0, it = 0;
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
                 const int acc = it & 1;
@@ -258,7 +253,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                     tmem_ld32(tm_lane + c0, v);
                     tmem_ld_wait();
                     if (!valid) continue;
-                    if (p.mode == MODE_Z && p.planes == 1) {
+                    if (p.mode == MODE_Z) {
                         __half *dst = (__half *)p.out + (((size_t)row * p.H + h) * 2 + sel) * p.NS + col0 + c0;
 #pragma unroll
                         for (int j8 = 0; j8 < 2; ++j8) {
@@ -269,8 +264,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                         }
                     } else {
                         const int g = row >= p.NS, o_row = row - g * p.NS;
-                        float *dst = (float *)p.out + (p.mode == MODE_Z ? (((size_t)row * p.H + h) * 2 + sel) * p.NS
-                                                                        : ((((size_t)sel * 2 + g) * p.H + h) * p.NS + o_row) * p.NS) + col0 + c0;
+                        float *dst = (float *)p.out + ((((size_t)sel * 2 + g) * p.H + h) * p.NS + o_row) * p.NS + col0 + c0;
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             uint32_t w[8];
@@ -389,32 +383,25 @@ __device__ __forceinline__ f32x4 zero4() { return f32x4{pack2(0.f, 0.f), pack2(0
 __device__ __forceinline__ f32x4 fma4(const f32x4 &x, const f32x4 &y, const f32x4 &z) { return f32x4{fma2(x.a, y.a, z.a), fma2(x.b, y.b, z.b)}; }
 __device__ __forceinline__ f32x4 mul4(const f32x4 &x, const f32x4 &y) { return f32x4{mul2(x.a, y.a), mul2(x.b, y.b)}; }
 
-// u_t = b_c + sum_j w[j] x_{t-j} of tokens [tb, tb + n) of sequences b0, b0 + 1, ... as fp16 u[sequence][n][D], or (PLANES) as
-// three bf16 values whose sum is the fp32 u exactly, u[head][plane][sequence][n][width]: one thread per
-// (sequence, 32 tokens, four adjacent channels), forward in time, eight tokens' loads in flight.  Bound by its 4 bytes per
-// element: with two channels per thread and a predicate on every token it executed 26 instructions per element (66 % of the issue
-// slots) and took 66 us on B4 T4096 D4096.  grid (ceil(D/256), ceil(n/128), sequences)
+// u_t = b_c + sum_j w[j] x_{t-j} as fp16 u[B][T][D]: one thread per (sequence, 32 tokens, four adjacent channels), forward in time,
+// eight tokens' loads in flight.  Bound by its 4 bytes per element: with two channels per thread and a predicate on every token it
+// executed 26 instructions per element (66 % of the issue slots) and took 66 us on B4 T4096 D4096.
+// grid (ceil(D/256), ceil(T/128), B)
 struct ConvArgs {
-    int T, D, b0, tb, n;
+    int T, D;
     const __nv_bfloat16 *x, *conv_w, *cs_in;
     const float *conv_b;
     __half *u;
     uint32_t *epoch;
-    int dh;               // PLANES: width of a head
 };
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
     return *(const uint32_t *)&v;
 }
-// what is left of (lo, hi) after the bf16 values in w: exact; nothing where w overflowed to infinity
-__device__ __forceinline__ f32x2 bf16_rest(f32x2 v, uint32_t w) {
-    const f32x2 t = bf2x(w);
-    return pack2(isinf(t.x) ? 0.0f : v.x - t.x, isinf(t.y) ? 0.0f : v.y - t.y);
-}
-template <bool PLANES> __global__ void __launch_bounds__(256, 4) conv_forward_kernel(ConvArgs a) {
+__global__ void __launch_bounds__(256, 4) conv_forward_kernel(ConvArgs a) {
     dependency_wait();
-    const int d = blockIdx.x * CONV_CH + (threadIdx.x & 63) * 4, b = a.b0 + blockIdx.z;
-    const int T = a.T, D = a.D, t0 = a.tb + blockIdx.y * CONV_CHUNK + (threadIdx.x >> 6) * CONV_SEG, t1 = min(a.tb + a.n, t0 + CONV_SEG);
+    const int d = blockIdx.x * CONV_CH + (threadIdx.x & 63) * 4, b = blockIdx.z;
+    const int T = a.T, D = a.D, t0 = blockIdx.y * CONV_CHUNK + (threadIdx.x >> 6) * CONV_SEG, t1 = min(T, t0 + CONV_SEG);
     // the scans' carry records are told apart from those an earlier launch with the same host tag (a graph replay) left behind
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) *a.epoch += 1u;
     if (d >= D || t0 >= t1) return;
@@ -429,22 +416,12 @@ template <bool PLANES> __global__ void __launch_bounds__(256, 4) conv_forward_ke
     f32x4 x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
     const uint32_t sD = (uint32_t)D / 4;   // token stride in groups of four channels
     const uint2 *px = (const uint2 *)(a.x + ((size_t)b * T + t0) * D + d);
-    const size_t tok = (size_t)blockIdx.z * a.n + (t0 - a.tb), plane = (size_t)gridDim.z * a.n * a.dh / 4;   // plane: in uint2
-    uint2 *pu = (uint2 *)(PLANES ? a.u + (size_t)(d / a.dh) * 12 * plane + tok * a.dh + d % a.dh : a.u + tok * D + d);
-    const uint32_t su = PLANES ? (uint32_t)a.dh / 4 : sD;
+    uint2 *pu = (uint2 *)(a.u + ((size_t)b * T + t0) * D + d);
     auto token = [&](uint2 xw) {
         const f32x4 x0 = bf4x(xw);
         const f32x4 uv = fma4(w[3], x3, fma4(w[2], x2, fma4(w[1], x1, fma4(w[0], x0, cb))));
-        if (PLANES) {
-            f32x4 v = uv;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) {
-                const uint2 w = make_uint2(pack_bf16(v.a.x, v.a.y), pack_bf16(v.b.x, v.b.y));
-                pu[q * plane] = w;
-                v = f32x4{bf16_rest(v.a, w.x), bf16_rest(v.b, w.y)};
-            }
-        } else *pu = make_uint2(pack_f16_sat(uv.a.x, uv.a.y), pack_f16_sat(uv.b.x, uv.b.y));
-        pu += su;
+        *pu = make_uint2(pack_f16_sat(uv.a.x, uv.a.y), pack_f16_sat(uv.b.x, uv.b.y));
+        pu += sD;
         x3 = x2; x2 = x1; x1 = x0;
     };
     int t = t0;
@@ -506,7 +483,7 @@ constexpr int SCAN_WINDOW = 4;   // records requested at once
 
 struct ScanShared {
     f32x2 agg[2][8][32];   // steps of the eight segments: Q, G
-    f32x2 xin[32], pin[32];
+    f32x2 xin[32];
     uint64_t full[2];
     int abort;
 };
@@ -758,56 +735,70 @@ int scan_split(int columns, int nchunk, int slots) {
 // thread, a predicate on every token and sums per 32 tokens: 104 us on B4 T4096 D4096).  grid (ceil(D/256), ceil(T/128), B)
 struct ConvBwdArgs {
     int B, T, D;
-    const __nv_bfloat16 *x, *conv_w, *cs_in;
-    const __half *du;
-    __nv_bfloat16 *dx;
+    const void *x, *conv_w, *cs_in, *du;
+    void *dx;
     float *part_conv;   // [B*chunks][5][D]
 };
+// four adjacent channels as they lie in memory
+template <typename T> struct Four { typedef uint2 raw; };
+template <> struct Four<float> { typedef float4 raw; };
+__device__ __forceinline__ f32x4 four(const __nv_bfloat16 *, uint2 w) { return bf4x(w); }
+__device__ __forceinline__ f32x4 four(const __half *, uint2 w) { return hf4x(w); }
+__device__ __forceinline__ f32x4 four(const float *, float4 w) { return f32x4{pack2(w.x, w.y), pack2(w.z, w.w)}; }
+__device__ __forceinline__ uint2 four_out(const __nv_bfloat16 *, const f32x4 &v) { return make_uint2(pack_bf16(v.a.x, v.a.y), pack_bf16(v.b.x, v.b.y)); }
+__device__ __forceinline__ float4 four_out(const float *, const f32x4 &v) { return make_float4(v.a.x, v.a.y, v.b.x, v.b.y); }
 
-__global__ void __launch_bounds__(256, 2) conv_backward_kernel(ConvBwdArgs a) {
+// LEN: tokens per thread
+template <typename IOT, typename DUT, int LEN> __global__ void __launch_bounds__(256, 2) conv_backward_kernel(ConvBwdArgs a) {
+    typedef typename Four<IOT>::raw XR;
+    typedef typename Four<DUT>::raw GR;
     __shared__ float4 red[3][5][64];
     dependency_wait();
     const int c = threadIdx.x & 63, sg = threadIdx.x >> 6, d = blockIdx.x * CONV_CH + c * 4, b = blockIdx.z;
-    const int T = a.T, D = a.D, t0 = blockIdx.y * CONV_CHUNK + sg * CONV_SEG, t1 = min(T, t0 + CONV_SEG);
+    const int T = a.T, D = a.D, t0 = (blockIdx.y * 4 + sg) * LEN, t1 = min(T, t0 + LEN);
+    const IOT *x = (const IOT *)a.x, *cs_in = (const IOT *)a.cs_in, *cw = (const IOT *)a.conv_w;
+    auto io4 = [](const IOT *p) { return four(p, *(const XR *)p); };
+    auto du4 = [](const GR *p) { return four((const DUT *)p, *p); };
     f32x4 sw[5];   // four taps, bias
 #pragma unroll
     for (int j = 0; j < 5; ++j) sw[j] = zero4();
     if (d < D && t0 < t1) {
         f32x4 w[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) w[j] = bf4x(*(const uint2 *)(a.conv_w + (size_t)j * D + d));
+        for (int j = 0; j < 4; ++j) w[j] = io4(cw + (size_t)j * D + d);
         auto xat = [&](int t) -> f32x4 {
-            if (t >= 0) return bf4x(*(const uint2 *)(a.x + ((size_t)b * T + t) * D + d));
-            return a.cs_in ? bf4x(*(const uint2 *)(a.cs_in + ((size_t)b * 3 + (3 + t)) * D + d)) : zero4();
+            if (t >= 0) return io4(x + ((size_t)b * T + t) * D + d);
+            return cs_in ? io4(cs_in + ((size_t)b * 3 + (3 + t)) * D + d) : zero4();
         };
         const uint32_t sD = (uint32_t)D / 4;
-        const uint2 *px = (const uint2 *)(a.x + ((size_t)b * T + t0) * D + d), *pg = (const uint2 *)(a.du + ((size_t)b * T + t0) * D + d);
-        uint2 *pdx = (uint2 *)(a.dx + ((size_t)b * T + t0) * D + d);
+        const XR *px = (const XR *)(x + ((size_t)b * T + t0) * D + d);
+        const GR *pg = (const GR *)((const DUT *)a.du + ((size_t)b * T + t0) * D + d);
+        XR *pdx = (XR *)((IOT *)a.dx + ((size_t)b * T + t0) * D + d);
         f32x4 x1 = xat(t0 - 1), x2 = xat(t0 - 2), x3 = xat(t0 - 3);
-        f32x4 g0 = hf4x(pg[0]), g1 = t0 + 1 < T ? hf4x(pg[sD]) : zero4(), g2 = t0 + 2 < T ? hf4x(pg[2 * sD]) : zero4();
+        f32x4 g0 = du4(pg), g1 = t0 + 1 < T ? du4(pg + sD) : zero4(), g2 = t0 + 2 < T ? du4(pg + 2 * sD) : zero4();
         pg += 3 * (size_t)sD;
-        auto token = [&](uint2 xw, uint2 gw) {   // gw: du_{t+3}, zero bits past the end
-            const f32x4 x0 = bf4x(xw), g3 = hf4x(gw);
-            const f32x4 o = fma4(w[3], g3, fma4(w[2], g2, fma4(w[1], g1, mul4(w[0], g0))));
-            const __nv_bfloat162 oa = __floats2bfloat162_rn(o.a.x, o.a.y), ob = __floats2bfloat162_rn(o.b.x, o.b.y);
-            *pdx = make_uint2(*(const uint32_t *)&oa, *(const uint32_t *)&ob);
+        auto token = [&](XR xw, GR gw) {   // gw: du_{t+3}, zero bits past the end
+            const f32x4 x0 = four((const IOT *)nullptr, xw), g3 = four((const DUT *)nullptr, gw);
+            *pdx = four_out((const IOT *)nullptr, fma4(w[3], g3, fma4(w[2], g2, fma4(w[1], g1, mul4(w[0], g0)))));
             pdx += sD;
             sw[0] = fma4(g0, x0, sw[0]); sw[1] = fma4(g0, x1, sw[1]); sw[2] = fma4(g0, x2, sw[2]); sw[3] = fma4(g0, x3, sw[3]);
             sw[4].a = __fadd2_rn(sw[4].a, g0.a); sw[4].b = __fadd2_rn(sw[4].b, g0.b);
             g0 = g1; g1 = g2; g2 = g3;
             x3 = x2; x2 = x1; x1 = x0;
         };
+        constexpr int BATCH = sizeof(XR) + sizeof(GR) <= 16 ? 8 : 4;   // tokens' loads in flight
         int t = t0;
 #pragma unroll 1
-        for (; t + 8 <= t1 && t + 11 <= T; t += 8) {
-            uint2 xs[8], gs[8];
+        for (; t + BATCH <= t1 && t + BATCH + 3 <= T; t += BATCH) {
+            XR xs[BATCH];
+            GR gs[BATCH];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) { xs[k] = *px; px += sD; gs[k] = *pg; pg += sD; }
+            for (int k = 0; k < BATCH; ++k) { xs[k] = *px; px += sD; gs[k] = *pg; pg += sD; }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) token(xs[k], gs[k]);
+            for (int k = 0; k < BATCH; ++k) token(xs[k], gs[k]);
         }
 #pragma unroll 1
-        for (; t < t1; ++t) { token(*px, t + 3 < T ? *pg : make_uint2(0u, 0u)); px += sD; pg += sD; }
+        for (; t < t1; ++t) { token(*px, t + 3 < T ? *pg : GR{}); px += sD; pg += sD; }
     }
     // segments added in order: run-to-run identical
     if (sg > 0) {
@@ -904,7 +895,7 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
     L.off_fws = take(sm100_prefill_workspace_bytes(B, T, D, Hl));
     L.off_rec = take((size_t)B * L.nchunk * D * sizeof(uint4) + 256);   // the records, then the launch counter
     L.off_pvec = take((size_t)B * (L.nchunk < SCAN_MAX_S ? L.nchunk : SCAN_MAX_S) * 3 * D * 4);
-    L.off_pconv = take((size_t)B * L.nchunk_conv * 5 * D * 4);
+    L.off_pconv = take((size_t)B * conv_backward_chunks(B, T, D) * 5 * D * 4);
     L.off_pdw = take((size_t)L.S * 2 * gr.G * gr.NS * gr.NS * 4);
     L.off_w16 = take(gr.W16_bytes());
     L.total = o;
@@ -913,7 +904,6 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
 
 GemmArgs gemm_args(const Groups &gr, int D, uint32_t *status) {
     GemmArgs g{};
-    g.planes = 1;
     g.H = gr.G; g.D = D; g.NS = gr.NS; g.NT = gr.NT; g.nt = gr.nt; g.hstride = gr.hstride; g.status = status; g.spin_ns = g_spin_limit_ns;
     return g;
 }
@@ -943,239 +933,6 @@ cudaError_t gemm_z(const Groups &gr, int D, size_t ntok, const __half *u, const 
     return run_gemm(g, st);
 }
 
-// ------------------------------------------------------------------ forward of heads wider than 256
-// The fused prefill keeps a head's weights in the tensor memory of a CTA pair, which holds 256 channels.  A wider head runs as
-// conv_forward -> z product -> the kernel below, over at most WIDE_TOKENS tokens at a time so that the workspace stays small and z
-// mostly in L2; the state goes from pass to pass through h_T (and a_prod).
-// Everything between the kernels is fp32, as it is in the CUDA-core kernel that this path replaces: u goes to the tensor core as three
-// bf16 values that add up to it (24 bits) and meets the caller's bf16 weights as they are, z is fp32, the gates are libm-grade.
-// With u and z in fp16 the path took 69 us on B2 T777 D5632 in 16 heads where it takes 139 (Conv1D 15, product 56, scan 68) and the
-// CUDA cores 638, and h_T was 1e-4 from the exact one (relative 2-norm) where it is 3e-7 now and was 2e-6 on the CUDA cores.
-// Forward scan: a block walks a 64-channel column forwards in chunks of 32 tokens, four a warp, u, z_a, z_x (and the gate branch) of
-// the next chunk arriving by tiled TMA meanwhile; same shape as the reverse scan.
-struct WideScanArgs {
-    alignas(64) CUtensorMap tm_u;        // [heads x 3 planes][sequences x n][width] of the pass, box 32 tokens x 64 channels
-    alignas(64) CUtensorMap tm_z, tm_g;  // z of the pass, [sequences][n][G x 2 x NS] fp32; the branch, [B][T][D]: the same box
-    FwdArgs f;
-    int G, hstride, NS, tiles, S, nchunk;
-    int b0, nb, tb, n;                   // sequences b0 .. b0 + nb - 1, tokens tb .. tb + n - 1
-    uint4 *rec;                          // [nchunk][nb][D] carry records
-    uint32_t *epoch;
-    uint32_t tag, wait_flip;             // wait_flip: see rglru_internal.h
-    unsigned long long spin_ns;
-};
-constexpr int WIDE_CHUNK = 32, WIDE_SEG = WIDE_CHUNK / 8;
-constexpr uint32_t WIDE_TILE_BYTES = WIDE_CHUNK * 128;   // of 64 channels of a 16-bit array; z takes two of them a gate
-constexpr uint32_t WIDE_STAGE_BYTES = 8 * WIDE_TILE_BYTES;
-constexpr uint32_t WIDE_SMEM_ALLOC = 2 * WIDE_STAGE_BYTES + 1024;
-constexpr size_t WIDE_TOKENS = 4096;
-
-// a_t and m_t i_t of Eq. 3-4 for one element, from 1 - a_t: eight independent chains a thread.  (As a call, with expm1f(2 L) for m
-// besides expf(L) for a: 150 instead of 139 us on B2 T777 D5632 in 16 heads, and h_T 2.0e-6 instead of 2.5e-7 from the exact one.)
-__device__ __forceinline__ float2 gates_acc(float za, float zx, float s) {
-    const float f = -expm1f(-s * sigmoid_acc(za));   // 1 - a_t; 1 - a_t^2 = f (2 - f)
-    return make_float2(1.0f - f, sqrtf(f * (2.0f - f)) * sigmoid_acc(zx));
-}
-
-__global__ void __launch_bounds__(256, 2) wide_scan_kernel(const __grid_constant__ WideScanArgs p) {
-    extern __shared__ uint8_t smem_raw[];
-    __shared__ ScanShared sh;
-    const uint32_t raw = smem_u32(smem_raw), stage_addr = (raw + 127u) & ~127u;
-    const uint8_t *stage = smem_raw + (stage_addr - raw);
-    const int tid = threadIdx.x, lane = tid & 31, seg = tid >> 5;
-    if (tid == 0) {
-        mbar_init(smem_u32(&sh.full[0]), 1); mbar_init(smem_u32(&sh.full[1]), 1);
-        sh.abort = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-    dependency_wait();
-    int bid = blockIdx.x;
-    const int k0 = bid % p.S; bid /= p.S;
-    const int n0 = (bid % p.tiles) * 64; bid /= p.tiles;
-    const int group = bid % p.G, bl = bid / p.G;
-    const FwdArgs &f = p.f;
-    const int T = f.T, D = f.D, S = p.S, n = n0 + 2 * lane, d = group * p.hstride + n, b = p.b0 + bl;
-    const bool cv = n < p.hstride && d < D, first = p.tb == 0, last = p.tb + p.n == T;
-    const f32x2 lam = cv ? ld2f(f.lambda + d) : pack2(0.f, 0.f);
-    const f32x2 s2 = pack2(decay_rate(lam.x, f.c), decay_rate(lam.y, f.c));
-    const f32x2 ba = cv ? ld2f(f.b_a + d) : pack2(0.f, 0.f), bx = cv ? ld2f(f.b_x + d) : pack2(0.f, 0.f);
-    const f32x2 ONE = pack2(1.0f, 1.0f), ZERO = pack2(0.0f, 0.0f);
-    const bool merged = f.gate_branch != nullptr;
-    const uint32_t full0 = smem_u32(&sh.full[0]);
-    auto issue = [&](int chunk, int st) {
-        const int t0 = chunk * WIDE_CHUNK, zc = 2 * (group * 2 * p.NS + n0);   // z in 16-bit units
-        const uint32_t bar = full0 + 8u * st, dst = stage_addr + st * WIDE_STAGE_BYTES;
-        mbar_expect_tx(bar, (merged ? 8 : 7) * WIDE_TILE_BYTES);
-        tma_load_3d(dst, &p.tm_z, zc, t0, bl, bar);
-        tma_load_3d(dst + 2 * WIDE_TILE_BYTES, &p.tm_z, zc + 2 * p.NS, t0, bl, bar);
-        for (int q = 0; q < 3; ++q) tma_load_3d(dst + (4 + q) * WIDE_TILE_BYTES, &p.tm_u, n0, bl * p.n + t0, group * 3 + q, bar);
-        if (merged) tma_load_3d(dst + 7 * WIDE_TILE_BYTES, &p.tm_g, group * p.hstride + n0, p.tb + t0, b, bar);
-    };
-    if (tid == 0) {
-        issue(k0, 0);
-        if (k0 + S < p.nchunk) issue(k0 + S, 1);
-    }
-    const float *hin = first ? f.h0 : f.h_T;
-    f32x2 X = hin && cv ? ld2f(hin + (size_t)b * D + d) : ZERO;
-    f32x2 Pc = !first && f.a_prod && cv ? ld2f(f.a_prod + (size_t)b * D + d) : ONE;   // product of a_t up to the chunk
-    // through shared memory, so that the loads above have returned before this block publishes anything: the block that reaches
-    // the end of the column overwrites h_T (and a_prod) once it has seen every other block's records
-    if (seg == 0) { sh.xin[lane] = X; sh.pin[lane] = Pc; }
-    __syncthreads();
-    X = sh.xin[lane]; Pc = sh.pin[lane];
-    const uint32_t tag = S > 1 ? p.tag + *p.epoch * 0x9E3779B1u : 0u;
-    auto column = [&]() { return Column{p.rec + (size_t)bl * D + d, (ptrdiff_t)p.nb * D, S, cv, tag, tag ^ p.wait_flip, p.spin_ns}; };
-    if (S > 1 && seg == 0) mark_running(column(), k0);
-    bool ok = true;
-    int it = 0;
-    for (int chunk = k0; chunk < p.nchunk; chunk += S, ++it) {
-        const int st = it & 1, t0 = chunk * WIDE_CHUNK + seg * WIDE_SEG, nv = p.n - t0;
-        ok = warp_wait(full0 + 8u * st, (it >> 1) & 1, p.spin_ns, &sh.abort);
-        const uint8_t *sm = stage + st * WIDE_STAGE_BYTES;
-        const f32x2 *sz = (const f32x2 *)sm + seg * WIDE_SEG * 32 + lane;
-        const uint32_t *su = (const uint32_t *)(sm + 4 * WIDE_TILE_BYTES) + seg * WIDE_SEG * 32 + lane;
-        constexpr int TW = WIDE_TILE_BYTES / 4;
-        f32x2 P[WIDE_SEG], h[WIDE_SEG];
-        f32x2 Q = ONE, Hc = ZERO;
-#pragma unroll
-        for (int k = 0; k < WIDE_SEG; ++k) {
-            const f32x2 za = __fadd2_rn(sz[k * 32], ba), zx = __fadd2_rn(sz[TW + k * 32], bx);
-            const f32x2 u = __fadd2_rn(__fadd2_rn(bf2x(su[k * 32]), bf2x(su[TW + k * 32])), bf2x(su[2 * TW + k * 32]));
-            const float2 g0 = gates_acc(za.x, zx.x, s2.x), g1 = gates_acc(za.y, zx.y, s2.y);
-            // a token that does not exist holds the state (its row of u is the next sequence's)
-            const f32x2 at = k < nv ? pack2(g0.x, g1.x) : ONE, vt = k < nv ? mul2(pack2(g0.y, g1.y), u) : ZERO;
-            Hc = fma2(at, Hc, vt);
-            Q = mul2(Q, at);
-            P[k] = Q; h[k] = Hc;
-        }
-        sh.agg[0][seg][lane] = Q; sh.agg[1][seg][lane] = Hc;
-        if (!ok) sh.abort = 1;
-        __syncthreads();
-        if (S > 1) {
-            if (seg == 0 && !sh.abort) {
-                f32x2 Qt = ONE, Gt = ZERO;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) { Gt = fma2(sh.agg[0][k][lane], Gt, sh.agg[1][k][lane]); Qt = mul2(Qt, sh.agg[0][k][lane]); }
-                const Column col = column();
-                put_record(col, chunk, Qt, Gt);
-                for (int jb = min(chunk, S - 1); jb > 0 && ok; jb -= SCAN_WINDOW) {   // records jb, jb - 1, ... chunks earlier, farthest first
-                    uint4 w0[SCAN_WINDOW], w1[SCAN_WINDOW];
-                    ok = read_records<SCAN_WINDOW>(col, chunk - jb, jb, w0, w1);
-                    if (!ok) break;
-#pragma unroll
-                    for (int k = 0; k < SCAN_WINDOW; ++k) {
-                        if (k < jb && cv) {
-                            const f32x2 q = pack2(__uint_as_float(w0[k].x), __uint_as_float(w1[k].x));
-                            X = fma2(q, X, pack2(__uint_as_float(w0[k].z), __uint_as_float(w1[k].z)));
-                            Pc = mul2(Pc, q);
-                        }
-                    }
-                }
-                sh.xin[lane] = X; sh.pin[lane] = Pc;
-                if (!ok) sh.abort = 1;
-            }
-            __syncthreads();
-            X = sh.xin[lane]; Pc = sh.pin[lane];
-        }
-        if (sh.abort) break;   // uniform: set before the barrier above
-        f32x2 carry = X;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            if (k == seg) carry = X;
-            X = fma2(sh.agg[0][k][lane], X, sh.agg[1][k][lane]);
-            Pc = mul2(Pc, sh.agg[0][k][lane]);
-        }
-        const uint32_t sD = (uint32_t)D / 2;
-        uint32_t *p_y = (uint32_t *)((__nv_bfloat16 *)f.y + ((size_t)b * T + p.tb + t0) * D + d);
-#pragma unroll
-        for (int k = 0; k < WIDE_SEG; ++k) {
-            f32x2 y = fma2(P[k], carry, h[k]);
-            if (merged) {
-                const f32x2 g = bf2x(su[3 * TW + k * 32]);   // y_t = h_t GeLU(branch_t), GeLU(v) = v Phi(v) (Section 2.3)
-                y = mul2(y, pack2(0.5f * g.x * (1.0f + erff(g.x * 0.70710678f)), 0.5f * g.y * (1.0f + erff(g.y * 0.70710678f))));
-            }
-            if (cv && k < nv) p_y[k * sD] = pack_bf16(y.x, y.y);
-        }
-        __syncthreads();   // everybody has read the stage and the segments' steps
-        if (tid == 0 && chunk + 2 * S < p.nchunk) issue(chunk + 2 * S, st);
-        if (chunk == p.nchunk - 1 && seg == 0 && cv) {
-            *(float2 *)(f.h_T + (size_t)b * D + d) = X;
-            if (f.a_prod) *(float2 *)(f.a_prod + (size_t)b * D + d) = Pc;
-            if (last) {   // the last three raw inputs of concat(conv_state_in, x), bit-exact
-                uint32_t keep[3];
-#pragma unroll
-                for (int kk = 0; kk < 3; ++kk) {
-                    const int t = T - 3 + kk;
-                    keep[kk] = t >= 0 ? *(const uint32_t *)((const __nv_bfloat16 *)f.x + ((size_t)b * T + t) * D + d)
-                                      : (f.cs_in ? *(const uint32_t *)((const __nv_bfloat16 *)f.cs_in + ((size_t)b * 3 + (3 + t)) * D + d) : 0u);
-                }
-#pragma unroll
-                for (int kk = 0; kk < 3; ++kk) *(uint32_t *)((__nv_bfloat16 *)f.cs_out + ((size_t)b * 3 + kk) * D + d) = keep[kk];
-            }
-        }
-    }
-    if (sh.abort && tid == 0) {
-        atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT);
-        const uint64_t tw = gtimer();   // let copies in flight land before shared memory is given back
-        while (gtimer() - tw < 50000ull) __nanosleep(1000);
-    }
-    __syncthreads();
-}
-
-// z = u W^T of a pass of ntok tokens: u [head][plane][tok][width] in bf16, the caller's weights, z [tok][head][2][NS] in fp32.  The
-// tensor cores add the products of the smallest plane first, so that their roundings are small ones.
-cudaError_t wide_gemm_z(const Groups &gr, const FwdArgs &f, size_t ntok, const __half *u, float *z, cudaStream_t st) {
-    GemmArgs g = gemm_args(gr, f.D, f.status);
-    const uint64_t dh = gr.dh;
-    const uint64_t da[3] = {dh, ntok, 3 * (uint64_t)gr.G}, sa[2] = {dh * 2, dh * ntok * 2}, db[3] = {dh, dh, (uint64_t)gr.G}, sb[2] = {dh * 2, dh * dh * 2};
-    const uint32_t ba[3] = {64, 128, 1}, bb[3] = {64, (uint32_t)gr.NT, 1};
-    if (!encode_map16_3d(&g.tm_a, u, da, sa, ba, true) || !encode_map16_3d(&g.tm_b0, f.W_a, db, sb, bb, true) || !encode_map16_3d(&g.tm_b1, f.W_x, db, sb, bb, true))
-        return cudaErrorNotSupported;
-    g.mode = MODE_Z; g.planes = 3; g.rows_valid = (int)ntok; g.out = z;
-    g.nx = (int)((ntok + 127) / 128); g.ny = 2 * gr.nt;
-    return run_gemm(g, st);
-}
-// The scan of one pass (p.b0, nb, tb, n) over its u and z
-cudaError_t run_wide_scan(WideScanArgs &p, const __half *u, const float *z, cudaStream_t st) {
-    static PerDeviceOptIn opt_in;
-    cudaError_t e = opt_in.ensure(wide_scan_kernel, (int)WIDE_SMEM_ALLOC);
-    if (e != cudaSuccess) return e;
-    const uint64_t dh = p.hstride, n = p.n, ntok = n * p.nb, wz = (uint64_t)p.G * 2 * p.NS;
-    const uint64_t du[3] = {dh, ntok, 3 * (uint64_t)p.G}, su[2] = {dh * 2, dh * ntok * 2};
-    const uint64_t dz[3] = {2 * wz, n, (uint64_t)p.nb}, sz[2] = {wz * 4, wz * n * 4};   // fp32 as pairs of 16-bit elements
-    const uint32_t bu[3] = {64, WIDE_CHUNK, 1}, bz[3] = {128, WIDE_CHUNK, 1};
-    if (!encode_map16_3d(&p.tm_u, u, du, su, bu, false) || !encode_map16_3d(&p.tm_z, z, dz, sz, bz, false)) return cudaErrorNotSupported;
-    if (p.f.gate_branch && !encode_bf16_map_3d(&p.tm_g, p.f.gate_branch, p.f.D, (uint64_t)p.f.T, (uint64_t)p.f.B, 64, WIDE_CHUNK, false)) return cudaErrorNotSupported;
-    p.nchunk = (p.n + WIDE_CHUNK - 1) / WIDE_CHUNK;
-    p.S = scan_split(p.nb * p.G * p.tiles, p.nchunk, 2 * num_sms());
-    const size_t blocks = (size_t)p.nb * p.G * p.tiles * p.S;
-    if (blocks > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    return launch_dependent(wide_scan_kernel, dim3((unsigned)blocks), dim3(256), WIDE_SMEM_ALLOC, st, p);
-}
-
-// Passes over the batch: whole sequences while they fit WIDE_TOKENS, else one sequence in pieces of that length
-struct WideLayout {
-    int nb, n;   // sequences and tokens of a pass, at most
-    size_t off_u, off_z, off_rec, off_h0, total;
-};
-WideLayout wide_layout(int B, int T, int D, int H) {
-    WideLayout L{};
-    const Groups gr = make_groups(D, H);
-    L.n = (size_t)T < WIDE_TOKENS ? T : (int)WIDE_TOKENS;
-    const size_t fit = WIDE_TOKENS / L.n;
-    L.nb = (size_t)B < fit ? B : (int)fit;
-    const size_t tok = (size_t)L.nb * L.n;
-    size_t o = 0;
-    auto take = [&](size_t bytes) { const size_t at = o; o += up256(bytes); return at; };
-    L.off_u = take(tok * D * 3 * 2);
-    L.off_z = take(tok * gr.G * gr.NS * 2 * 4);
-    L.off_rec = take((size_t)((L.n + WIDE_CHUNK - 1) / WIDE_CHUNK) * L.nb * D * sizeof(uint4) + 256);   // the records, then the launch counter
-    L.off_h0 = take((size_t)B * D * 4);
-    L.total = o;
-    return L;
-}
-
 }  // namespace
 
 // Head width: a multiple of 32 up to 256.  k = 256 / width (rounded down) consecutive heads form a group whose weight matrix is
@@ -1191,6 +948,28 @@ bool sm100_backward_supported(int B, int T, int D, int H, int io) {
     if (io != RGLRU_BF16 || B <= 0 || T <= 0 || T % 8 != 0 || H <= 0 || D % H != 0) return false;
     const int dh = D / H;
     return dh <= DH && dh % 32 == 0;
+}
+
+namespace {
+// Tokens per thread: 32, or 8 while 128-token blocks would leave SMs idle (B1 T256 D256, fp32: two blocks, 11 us)
+int conv_backward_len(int B, int T, int D) {
+    return (size_t)B * ((T + CONV_CHUNK - 1) / CONV_CHUNK) * ((D + CONV_CH - 1) / CONV_CH) >= 148 ? CONV_SEG : 8;
+}
+template <typename IOT, typename DUT>
+cudaError_t launch_conv_backward(const ConvBwdArgs &a, cudaStream_t st) {
+    const dim3 grid((a.D + CONV_CH - 1) / CONV_CH, conv_backward_chunks(a.B, a.T, a.D), a.B);
+    return launch_dependent(conv_backward_len(a.B, a.T, a.D) == CONV_SEG ? conv_backward_kernel<IOT, DUT, CONV_SEG> : conv_backward_kernel<IOT, DUT, 8>, grid, dim3(256), 0, st, a);
+}
+}  // namespace
+int conv_backward_chunks(int B, int T, int D) {
+    const int per_block = 4 * conv_backward_len(B, T, D);
+    return (T + per_block - 1) / per_block;
+}
+
+cudaError_t conv_backward(const BwdArgs &q, int io, const void *du, bool du_is_half, cudaStream_t st) {
+    const ConvBwdArgs a{q.B, q.T, q.D, q.x, q.conv_w, q.cs_in, du, q.dx, q.part_conv};
+    if (io == RGLRU_F32) return launch_conv_backward<float, float>(a, st);
+    return du_is_half ? launch_conv_backward<__nv_bfloat16, __half>(a, st) : launch_conv_backward<__nv_bfloat16, float>(a, st);
 }
 
 size_t sm100_backward_workspace_bytes(int B, int T, int D, int H) { return bwd_layout(B, T, D, H).total; }
@@ -1231,7 +1010,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     // 1. fp16 weights, conv output
     if ((e = convert_w(gr, q.W_a, q.W_x, q.H, W16, st)) != cudaSuccess) return e;
     const dim3 grid_conv((D + CONV_CH - 1) / CONV_CH, L.nchunk_conv, B);
-    if ((e = launch_dependent(conv_forward_kernel<false>, grid_conv, dim3(256), 0, st, ConvArgs{T, D, 0, 0, T, a.x, a.conv_w, a.cs_in, a.conv_b, u, a.epoch, gr.dh})) != cudaSuccess) return e;
+    if ((e = launch_dependent(conv_forward_kernel, grid_conv, dim3(256), 0, st, ConvArgs{T, D, a.x, a.conv_w, a.cs_in, a.conv_b, u, a.epoch})) != cudaSuccess) return e;
 
     ReduceJobs jobs{};
     const uint64_t BT = L.BT;
@@ -1291,56 +1070,11 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
     }
     // 6. per-channel sums, Conv1D adjoint
     add_reduce_job(jobs, a.part_vec, B * sc.S, (size_t)3 * D, q.dlambda, D, q.db_a, D, q.db_x, D);
-    ConvBwdArgs cb{};
-    cb.B = B; cb.T = T; cb.D = D;
-    cb.x = a.x; cb.conv_w = a.conv_w; cb.cs_in = a.cs_in; cb.du = du; cb.dx = (__nv_bfloat16 *)q.dx;
-    cb.part_conv = (float *)(ws + L.off_pconv);
-    if ((e = launch_dependent(conv_backward_kernel, grid_conv, dim3(256), 0, st, cb)) != cudaSuccess) return e;
+    q.part_conv = (float *)(ws + L.off_pconv);
+    if ((e = conv_backward(q, RGLRU_BF16, du, true, st)) != cudaSuccess) return e;
     if ((e = state_conv_grads(q, RGLRU_BF16, du, true, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
-    add_reduce_job(jobs, cb.part_conv, B * L.nchunk_conv, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
+    add_reduce_job(jobs, q.part_conv, B * conv_backward_chunks(B, T, D), (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
     return run_reduce_jobs(jobs, st);
-}
-
-// Heads wider than 256 (a multiple of 32): see wide_scan_kernel
-bool sm100_wide_prefill_supported(int B, int T, int D, int H, int io) {
-    if (io != RGLRU_BF16 || B <= 0 || T <= 0 || H <= 0 || D % H != 0) return false;
-    const int dh = D / H;
-    return dh > DH && dh <= GENERIC_MAX_DH && dh % 32 == 0;
-}
-
-size_t sm100_wide_prefill_workspace_bytes(int B, int T, int D, int H) { return wide_layout(B, T, D, H).total; }
-
-cudaError_t sm100_wide_prefill(const FwdArgs &a, void *ws_body, size_t ws_body_bytes, cudaStream_t st) {
-    const int B = a.B, T = a.T, D = a.D;
-    const Groups gr = make_groups(D, a.H);
-    const WideLayout L = wide_layout(B, T, D, a.H);
-    if (ws_body_bytes < L.total) return cudaErrorInvalidValue;
-    char *ws = (char *)ws_body;
-    __half *u = (__half *)(ws + L.off_u);
-    float *z = (float *)(ws + L.off_z);
-    cudaError_t e;
-    WideScanArgs p{};
-    p.f = a;
-    p.G = gr.G; p.hstride = gr.hstride; p.NS = gr.NS; p.tiles = (gr.hstride + 63) / 64;
-    p.tag = next_call_tag(); p.wait_flip = wait_flip(a.flags); p.spin_ns = g_spin_limit_ns;
-    p.rec = (uint4 *)(ws + L.off_rec);
-    p.epoch = (uint32_t *)(p.rec + (size_t)((L.n + WIDE_CHUNK - 1) / WIDE_CHUNK) * L.nb * D);
-    // blocks that share a column read the incoming state at unrelated times: an in-place update works on a copy
-    const size_t hb = (size_t)B * D * sizeof(float);
-    if (a.h0 && (uintptr_t)a.h0 < (uintptr_t)a.h_T + hb && (uintptr_t)a.h_T < (uintptr_t)a.h0 + hb) {
-        if ((e = cudaMemcpyAsync(ws + L.off_h0, a.h0, hb, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
-        p.f.h0 = (const float *)(ws + L.off_h0);
-    }
-    for (int b0 = 0; b0 < B; b0 += L.nb) {
-        for (int tb = 0; tb < T; tb += L.n) {
-            p.b0 = b0; p.nb = B - b0 < L.nb ? B - b0 : L.nb;
-            p.tb = tb; p.n = T - tb < L.n ? T - tb : L.n;
-            if ((e = launch_dependent(conv_forward_kernel<true>, dim3((D + CONV_CH - 1) / CONV_CH, (p.n + CONV_CHUNK - 1) / CONV_CHUNK, p.nb), dim3(256), 0, st, ConvArgs{T, D, b0, tb, p.n, (const __nv_bfloat16 *)a.x, (const __nv_bfloat16 *)a.conv_w, (const __nv_bfloat16 *)a.cs_in, a.conv_b, u, p.epoch, gr.dh})) != cudaSuccess) return e;
-            if ((e = wide_gemm_z(gr, a, (size_t)p.nb * p.n, u, z, st)) != cudaSuccess) return e;
-            if ((e = run_wide_scan(p, u, z, st)) != cudaSuccess) return e;
-        }
-    }
-    return cudaSuccess;
 }
 
 }  // namespace rglru

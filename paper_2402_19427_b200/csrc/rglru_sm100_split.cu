@@ -1,0 +1,951 @@
+// fp32 products on the sm_100a tensor cores, and the kernels around them: the forward and backward of fp32 io, the forward of bf16
+// heads wider than 256 and the backward of bf16 calls that are promised fp32 between the kernels (heads wider than 256, ragged
+// lengths).  Head widths that are multiples of 32.
+//
+// An fp32 value is the exact sum of three bf16 values ("planes": 8 + 8 + 8 significant bits, each the upper half of what the ones before
+// leave).  A product of two fp32 operands is the sum of the six plane products of at least 2^-16 of the first one's size -- the other
+// three are below 2^-24 --, and bf16 weights are a single plane, so that three products do.  They run on tcgen05 (kind::f16, bf16) and
+// accumulate in fp32 tensor memory.  The accumulation rounds towards zero: measured on 128 x 128 tiles of random numbers, relative
+// 2-norm error (bias) 5.5e-8 (-2.8e-8) after 64 products a result, 1.9e-7 (-1.2e-7) after 256, 8.6e-7 (-5.5e-7) after 1024, against
+// 4.5e-8, 0.9e-7 and 2.1e-7 of a chain of fp32 FMAs.  So the leading product of each pair of planes has an accumulator of its own,
+// which takes at most a few hundred terms, and the small ones another, whose roundings are 2^-8 smaller.
+//   1. split_weights      (fp32 io) the weights as planes
+//   2. split_forward      Conv1D, planes of u, both gate products, gates, scan, chain of chunks: y, or for the backward r, i, the
+//                         state before every eighth token, and the planes of u
+//   3. split_reverse      reverse scan and element-wise adjoints: planes of dz, the direct part of du in fp32
+//   4. split_products     du += W^T dz and dW = dz^T u, one launch
+//   5. Conv1D adjoint (rglru_sm100_bwd.cu) and reductions in fixed order (rglru_generic.cu)
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include "rglru_chain.cuh"
+#include "rglru_gates32.cuh"
+#include "rglru_internal.h"
+#include "sm100_ptx.cuh"
+
+namespace rglru {
+namespace {
+
+using namespace ptx;
+
+constexpr int PLANES = 3;
+constexpr int SEG = 8;                        // tokens between saved states = tokens of a thread of the reverse scan
+constexpr int FWD_THREADS = 320;              // eight warps of Conv1D and epilogue, one of copies, one of products
+constexpr uint32_t TILE_BYTES = 128 * 128;    // 128 rows (or 2 x 64 columns) of 64 bf16: one operand tile of a K block of 64
+constexpr int PROD_RING = 13;
+
+__device__ __forceinline__ f32x2 bf2x(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
+__device__ __forceinline__ float top16(float v) { return __uint_as_float(__float_as_uint(v) & 0xFFFF0000u); }
+__device__ __forceinline__ uint32_t tops(f32x2 v) { return __byte_perm(__float_as_uint(v.x), __float_as_uint(v.y), 0x7632); }   // the upper halves, v.x's below
+// The planes of two values, each the upper half of what is left: eight bits at a time and exact.  An infinity becomes the largest finite
+// value first (it would leave a NaN behind itself; as a factor of the products it is the same to the gates).
+__device__ __forceinline__ void split_planes(f32x2 v, uint32_t (&w)[PLANES]) {
+    v = pack2(clamp_nan(v.x, 3.402823466e38f), clamp_nan(v.y, 3.402823466e38f));
+#pragma unroll
+    for (int q = 0; q < PLANES; ++q) {
+        w[q] = tops(v);
+        if (q + 1 < PLANES) v = fma2(pack2(top16(v.x), top16(v.y)), pack2(-1.0f, -1.0f), v);
+    }
+}
+__device__ __forceinline__ f32x2 ld2f(const float *p) { return *(const float2 *)p; }
+__device__ __forceinline__ f32x2 ld2(const float *p) { return *(const float2 *)p; }
+__device__ __forceinline__ f32x2 ld2(const __nv_bfloat16 *p) { return bf2x(*(const uint32_t *)p); }
+__device__ __forceinline__ float ld1(const float *p) { return *p; }
+__device__ __forceinline__ float ld1(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
+__device__ __forceinline__ void st1(float *p, float v) { *p = v; }
+__device__ __forceinline__ void st1(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
+__device__ __forceinline__ void st_global_v8(void *ptr, const uint32_t (&r)[8]) {
+    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(ptr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]),
+                 "r"(r[6]), "r"(r[7]) : "memory");
+}
+__device__ __forceinline__ void ld_global_v8(const void *ptr, uint32_t (&r)[8]) {
+    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                 "=r"(r[6]), "=r"(r[7]) : "l"(ptr) : "memory");
+}
+
+// ------------------------------------------------------------------ weights as planes (fp32 io)
+// out[gate][plane][n], two values a thread
+__global__ void __launch_bounds__(256) split_weights_kernel(const float *Wa, const float *Wx, uint32_t *out, size_t n2) {
+    dependency_wait();
+    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+    dependency_trigger();
+    if (i >= 2 * n2) return;
+    const size_t gate = i >= n2, j = i - gate * n2;
+    uint32_t w[PLANES];
+    split_planes(ld2f((gate ? Wx : Wa) + 2 * j), w);
+#pragma unroll
+    for (int q = 0; q < PLANES; ++q) out[(gate * PLANES + q) * n2 + j] = w[q];
+}
+
+// One K block of 64 (four instructions, or two of its first half): the operands' descriptors advance by da and db 16-byte units an
+// instruction.  Straight-line code with nothing but additions: one thread issues it, and with the descriptors built in loops it needed
+// 240 cycles an instruction where the tensor core needs 49 to 65 (B4 T1024 D1024 in 4 heads, forward 72 us, products 75).
+__device__ __forceinline__ void mma_block(uint32_t d_tmem, uint64_t a, uint32_t da, uint64_t b, uint32_t db, uint32_t idesc, bool accumulate, bool full) {
+    mma_ss(d_tmem, a, b, idesc, accumulate);
+    mma_ss(d_tmem, a + da, b + db, idesc, 1);
+    if (full) {
+        mma_ss(d_tmem, a + 2 * da, b + 2 * db, idesc, 1);
+        mma_ss(d_tmem, a + 3 * da, b + 3 * db, idesc, 1);
+    }
+}
+
+// ------------------------------------------------------------------ forward
+// Block = (chunk of TOK tokens, sequence, head, 128 output channels).  Eight warps convolve 64 input channels at a time and write the
+// three planes of u as the B operand (K-major, 128-byte swizzle, two stages); weight tiles of 128 channels x 64 arrive by tiled TMA as
+// the A operand; z is left channel-per-lane in tensor memory, so that each of the eight warps then walks its 32 channels through half
+// of the chunk's tokens in registers.  Chunks are chained as in rglru_generic.cu (block order is chunk-major).
+// Two blocks fit an SM (64 tokens: 97 KB of shared memory, 256 columns of tensor memory), one's gates beside the other's products.
+struct SplitFwdArgs {
+    alignas(64) CUtensorMap tm_wa, tm_wx;   // [planes x H][dh][dh], box 64 x 128
+    FwdArgs f;
+    Chain ch;
+    uint32_t *u_planes;   // SAVE: [head][plane][B T][dh] bf16
+    float *h_seg;         // SAVE: [B][ceil(T / SEG)][D] state before every SEG-th token
+    int nchunk, mtiles;
+    int wplanes;          // 1 (bf16 weights) or 3
+};
+template <int TOK> struct FwdSmem {
+    static constexpr int SLOTS = TOK == 32 ? 5 : 3;   // weight tiles in flight, two blocks on an SM all the same
+    static constexpr uint32_t PLANE = TOK * 128, STAGE = PLANES * PLANE, RING = 2 * STAGE, BAR = RING + SLOTS * TILE_BYTES;
+    static constexpr uint32_t ALLOC = BAR + 256 + 1024;
+    static constexpr uint32_t COLS = 4 * TOK;   // z_a, z_x: leading product and the small ones
+};
+
+template <typename IOT, bool SAVE, int TOK, bool POLY>
+__device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t tmem, int b, int head, int mt, int chunk, float *xch, volatile int *abort_flag, float s) {
+    constexpr int HALF = TOK / 2;
+    const FwdArgs &f = p.f;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, half = warp >> 2;
+    const int T = f.T, D = f.D, dh = D / f.H, chl = q * 32 + lane, c = mt * 128 + chl;
+    const bool cv = c < dh;
+    const int d = head * dh + (cv ? c : 0), t0 = chunk * TOK + half * HALF;
+    const IOT *x = (const IOT *)f.x, *cw = (const IOT *)f.conv_w, *cs_in = (const IOT *)f.cs_in;
+    const IOT *xb = x + (size_t)b * T * D + d;
+    auto xat = [&](int t) -> float { return t >= 0 ? (t < T ? ld1(xb + (size_t)t * D) : 0.0f) : cs_in ? ld1(cs_in + ((size_t)b * 3 + (3 + t)) * D + d) : 0.0f; };
+    const float ba = f.b_a[d], bx = f.b_x[d], cb = f.conv_b ? f.conv_b[d] : 0.0f;
+    float w[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) w[j] = ld1(cw + (size_t)j * D + d);
+    float x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
+    const uint32_t tm = tmem + ((uint32_t)(q * 32) << 16) + half * HALF;
+    float P = 1.0f, h = 0.0f, segP[HALF / SEG], segH[HALF / SEG];
+#pragma unroll(SAVE ? HALF / SEG : 1)
+    for (int j = 0; j < HALF / SEG; ++j) {
+        f32x2 za[4], zx[4], la[4], lx[4];
+        const int tb = t0 + j * SEG;
+        tmem_ld8p(tm + j * SEG, za); tmem_ld8p(tm + TOK + j * SEG, la); tmem_ld8p(tm + 2 * TOK + j * SEG, zx); tmem_ld8p(tm + 3 * TOK + j * SEG, lx);
+        float xs[SEG];
+        const bool whole = tb + SEG <= T;
+        if (whole) {
+            const IOT *px = xb + (size_t)tb * D;
+#pragma unroll
+            for (int k = 0; k < SEG; ++k) { xs[k] = ld1(px); px += D; }
+        } else {
+#pragma unroll
+            for (int k = 0; k < SEG; ++k) xs[k] = xat(tb + k);
+        }
+        float *pr = nullptr, *pi = nullptr;
+        if (SAVE) { const size_t e = ((size_t)b * T + tb) * D + d; pr = f.save_r + e; pi = f.save_i + e; }
+        tmem_ld_wait();
+        if (SAVE) { segP[j] = P; segH[j] = h; }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const f32x2 r = sigmoid2_acc(__fadd2_rn(__fadd2_rn(za[k], la[k]), pack2(ba, ba)));
+            const f32x2 g = sigmoid2_acc(__fadd2_rn(__fadd2_rn(zx[k], lx[k]), pack2(bx, bx)));
+            const f32x2 fr = one_minus_decay2<POLY>(r, pack2(s, s));
+            f32x2 rm;
+            const f32x2 m = input_scale2(fr, rm);
+            float u[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const float x0 = xs[2 * k + e];
+                u[e] = fmaf(w[3], x3, fmaf(w[2], x2, fmaf(w[1], x1, fmaf(w[0], x0, cb))));
+                x3 = x2; x2 = x1; x1 = x0;
+            }
+            const f32x2 a = fma2(fr, pack2(-1.0f, -1.0f), pack2(1.0f, 1.0f)), v = mul2(m, mul2(g, pack2(u[0], u[1])));
+            const bool e0 = whole || tb + 2 * k < T, e1 = whole || tb + 2 * k + 1 < T;
+            if (SAVE) {
+                if (e0 && cv) { *pr = r.x; *pi = g.x; }
+                pr += D; pi += D;
+                if (e1 && cv) { *pr = r.y; *pi = g.y; }
+                pr += D; pi += D;
+            }
+            // a token that does not exist holds the state
+            const float a0 = e0 ? a.x : 1.0f, v0 = e0 ? v.x : 0.0f, a1 = e1 ? a.y : 1.0f, v1 = e1 ? v.y : 0.0f;
+            P *= a0; h = fmaf(a0, h, v0);
+            if (!SAVE) { za[k].x = P; zx[k].x = h; }
+            P *= a1; h = fmaf(a1, h, v1);
+            if (!SAVE) { za[k].y = P; zx[k].y = h; }
+        }
+        if (!SAVE) { tmem_st8p(tm + j * SEG, za); tmem_st8p(tm + 2 * TOK + j * SEG, zx); }
+    }
+    if (!SAVE) tmem_st_wait();
+    // ---- chain: the first half's thread of a channel takes the state that the previous chunk reached and hands its own on
+    float *xP = xch, *xh = xch + 128;
+    if (half == 1) { xP[chl] = P; xh[chl] = h; }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    float carry = 0.0f;
+    if (half == 0) {
+        uint4 *slot = p.ch.slot + (size_t)b * D + d;
+        const float P1 = xP[chl], h1 = xh[chl], cP = P * P1, cH = fmaf(P1, h, h1);
+        float P_in = 1.0f;
+        bool ok = !*abort_flag;
+        if (ok) {
+            if (chunk == 0) carry = f.h0 ? f.h0[(size_t)b * D + d] : 0.0f;
+            else ok = chain_wait(p.ch, slot, cv, chunk - 1, carry, P_in);
+        }
+        const float hs = fmaf(cP, carry, cH), Ps = cP * P_in;
+        if (ok && cv) {
+            chain_put(p.ch, slot, chunk, hs, Ps);
+            if (!SAVE && chunk + 1 == p.nchunk) {
+                f.h_T[(size_t)b * D + d] = hs;
+                if (f.a_prod) f.a_prod[(size_t)b * D + d] = Ps;
+                // the last three raw inputs of concat(conv_state_in, x), bit-exact
+                IOT keep[3];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const int t = T - 3 + k;
+                    keep[k] = t >= 0 ? xb[(size_t)t * D] : cs_in ? cs_in[((size_t)b * 3 + (3 + t)) * D + d] : IOT(0.0f);
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) ((IOT *)f.cs_out)[((size_t)b * 3 + k) * D + d] = keep[k];
+            }
+        }
+        if (!ok) {
+            if (cv) chain_fail(p.ch, slot, chunk);
+            *abort_flag = 1;
+        }
+        xP[chl] = fmaf(P, carry, h);   // the state that the second half starts from
+    }
+    asm volatile("bar.sync 1, 256;" ::: "memory");
+    if (*abort_flag) return;
+    if (half == 1) carry = xP[chl];
+    if (SAVE) {
+        const int nseg = (T + SEG - 1) / SEG;
+#pragma unroll
+        for (int j = 0; j < HALF / SEG; ++j)
+            if (cv && t0 + j * SEG < T) p.h_seg[((size_t)b * nseg + t0 / SEG + j) * D + d] = fmaf(segP[j], carry, segH[j]);
+        return;
+    }
+    const IOT *gb = (const IOT *)f.gate_branch;
+#pragma unroll 1
+    for (int j = 0; j < HALF / SEG; ++j) {
+        f32x2 Pv[4], hv[4];
+        tmem_ld8p(tm + j * SEG, Pv); tmem_ld8p(tm + 2 * TOK + j * SEG, hv);
+        tmem_ld_wait();
+        const int tb = t0 + j * SEG;
+        const size_t e = ((size_t)b * T + tb) * D + d;
+        IOT *y = (IOT *)f.y + e;
+#pragma unroll
+        for (int k = 0; k < SEG; ++k) {
+            if (tb + k < T && cv) {
+                float o = fmaf(k & 1 ? Pv[k / 2].y : Pv[k / 2].x, carry, k & 1 ? hv[k / 2].y : hv[k / 2].x);
+                if (gb) {   // merged output of the recurrent block (Section 2.3): v Phi(v) of the second branch, then the product
+                    const float g = ld1(gb + e + (size_t)k * D);
+                    o *= 0.5f * g * (1.0f + erff(g * 0.70710678f));
+                }
+                st1(y, o);
+            }
+            y += D;
+        }
+    }
+}
+
+template <typename IOT, bool SAVE, int TOK>
+__global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __grid_constant__ SplitFwdArgs p) {
+    using S = FwdSmem<TOK>;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ float xch[2 * 128];
+    __shared__ uint32_t tmem_s;
+    __shared__ volatile int abort_s;
+    const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
+    uint8_t *smem = smem_raw + (base - raw);
+    const uint32_t bar = base + S::BAR;
+    auto U_FULL = [&](int i) { return bar + 8u * i; };
+    auto U_EMPTY = [&](int i) { return bar + 16u + 8u * i; };
+    auto W_FULL = [&](int i) { return bar + 32u + 8u * i; };
+    auto W_EMPTY = [&](int i) { return bar + 32u + 8u * (S::SLOTS + i); };
+    const uint32_t ACC = bar + 32u + 16u * S::SLOTS;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const FwdArgs &f = p.f;
+    const int T = f.T, D = f.D, H = f.H, dh = D / H, nk = (dh + 63) / 64;
+    int bid = blockIdx.x;
+    const int mt = bid % p.mtiles; bid /= p.mtiles;
+    const int head = bid % H; bid /= H;
+    const int b = bid % f.B, chunk = bid / f.B;
+    if (tid == 0) {
+        for (int i = 0; i < 2; ++i) { mbar_init(U_FULL(i), 8); mbar_init(U_EMPTY(i), 1); }
+        for (int i = 0; i < S::SLOTS; ++i) { mbar_init(W_FULL(i), 1); mbar_init(W_EMPTY(i), 1); }
+        mbar_init(ACC, 1);
+        abort_s = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 8) { tmem_alloc(smem_u32(&tmem_s), S::COLS); tmem_relinquish(); }
+    if (warp == 9 && lane == 0) { prefetch_tensormap(&p.tm_wa); prefetch_tensormap(&p.tm_wx); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_s;
+    const unsigned long long spin = p.ch.spin_ns;
+    dependency_wait();
+    if (warp == 9) {
+        if (lane == 0) {
+            bool ok = true;
+            int it = 0;
+            for (int kc = 0; kc < nk && ok; ++kc) {
+                for (int g = 0; g < 2 && ok; ++g) {
+                    for (int q = p.wplanes - 1; q >= 0 && ok; --q, ++it) {
+                        const int s = it % S::SLOTS;
+                        ok = mbar_wait(W_EMPTY(s), ((it / S::SLOTS) & 1) ^ 1, spin, (volatile int *)&abort_s);
+                        if (!ok) break;
+                        mbar_expect_tx(W_FULL(s), TILE_BYTES);
+                        tma_load_3d(base + S::RING + s * TILE_BYTES, g ? &p.tm_wx : &p.tm_wa, kc * 64, mt * 128, q * H + head, W_FULL(s));
+                    }
+                }
+            }
+            if (!ok) { abort_s = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
+        }
+    } else if (warp == 8) {
+        if (lane == 0) {
+            constexpr uint32_t idesc = make_idesc(128, TOK);
+            constexpr int WP = sizeof(IOT) == 4 ? PLANES : 1;
+            bool ok = true;
+            int slot = 0, round = 0;
+            for (int kc = 0; kc < nk && ok; ++kc) {
+                const bool full = dh - kc * 64 >= 64;   // else the last half block
+                ok = mbar_wait(U_FULL(kc & 1), (kc >> 1) & 1, spin, (volatile int *)&abort_s);
+                if (!ok) break;
+                const uint64_t u_desc = make_desc_sw128(base + (kc & 1) * S::STAGE);
+#pragma unroll
+                for (int i = 0; i < 2 * WP; ++i) {
+                    const int g = i / WP, q = WP - 1 - i % WP;   // gate, plane of the weights: smallest first
+                    ok = ok && mbar_wait(W_FULL(slot), round & 1, spin, (volatile int *)&abort_s);
+                    if (!ok) break;
+                    tc_fence_after();
+                    const uint64_t w_desc = make_desc_sw128(base + S::RING + slot * TILE_BYTES);
+#pragma unroll
+                    for (int pl = 2 - q; pl >= 0; --pl)
+                        mma_block(tmem + (2 * g + (q + pl != 0)) * TOK, w_desc, 2, u_desc + pl * (S::PLANE >> 4), 2, idesc, kc > 0 || (q + pl != 0 && !(q == WP - 1 && pl == 2 - q)), full);
+                    tc_commit(W_EMPTY(slot));
+                    if (++slot == S::SLOTS) { slot = 0; ++round; }
+                }
+                if (ok) tc_commit(U_EMPTY(kc & 1));
+            }
+            if (ok) tc_commit(ACC);
+            else { abort_s = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
+        }
+    } else {
+        // ---- u of 64 channels x TOK tokens at a time: lane = two adjacent channels, warp = TOK / 8 tokens
+        constexpr int TW = TOK / 8;
+        const int ta = chunk * TOK + warp * TW;
+        const IOT *x = (const IOT *)f.x + (size_t)b * T * D + head * dh, *cw = (const IOT *)f.conv_w + head * dh, *cs = (const IOT *)f.cs_in;
+        if (cs) cs += (size_t)b * 3 * D + head * dh;
+        f32x2 xr[TW + 3];
+        const bool inside = ta >= 3 && ta + TW <= T;   // uniform over the warp
+        f32x2 w[4], cb;
+        auto fetch = [&](int kc) {
+            const int k = kc * 64 + 2 * lane;
+            const bool kv = k < dh;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) w[j] = kv ? ld2(cw + (size_t)j * D + k) : pack2(0.f, 0.f);
+            cb = kv && f.conv_b ? ld2f(f.conv_b + head * dh + k) : pack2(0.f, 0.f);
+            if (inside && kc * 64 + 64 <= dh) {
+                const IOT *px = x + (size_t)(ta - 3) * D + k;
+#pragma unroll
+                for (int i = 0; i < TW + 3; ++i) { xr[i] = ld2(px); px += D; }
+                return;
+            }
+#pragma unroll
+            for (int i = 0; i < TW + 3; ++i) {
+                const int t = ta - 3 + i;
+                xr[i] = pack2(0.f, 0.f);
+                if (k < dh) {
+                    if (t >= 0) { if (t < T) xr[i] = ld2(x + (size_t)t * D + k); }
+                    else if (cs) xr[i] = ld2(cs + (size_t)(3 + t) * D + k);
+                }
+            }
+        };
+        bool ok = true;
+        fetch(0);
+        for (int kc = 0; kc < nk; ++kc) {
+            const int k = kc * 64 + 2 * lane;
+            const bool kv = k < dh;
+            f32x2 u[TW];
+#pragma unroll
+            for (int i = 0; i < TW; ++i) u[i] = fma2(w[3], xr[i], fma2(w[2], xr[i + 1], fma2(w[1], xr[i + 2], fma2(w[0], xr[i + 3], cb))));
+            if (kc + 1 < nk) fetch(kc + 1);
+            ok = warp_wait(U_EMPTY(kc & 1), ((kc >> 1) & 1) ^ 1, spin, (volatile int *)&abort_s);
+            if (!ok) break;
+            uint8_t *st = smem + (kc & 1) * S::STAGE + warp * TW * 128 + (lane & 3) * 4;
+            const bool own = SAVE && (kc >> 1) == mt && kv;
+            const size_t plane = (size_t)f.B * T * dh / 2;
+            const uint32_t row_words = (uint32_t)dh / 2;
+            uint32_t *d0 = p.u_planes + (size_t)head * PLANES * plane + (((size_t)b * T + ta) * dh + k) / 2, *d1 = d0 + plane, *d2 = d1 + plane;
+#pragma unroll
+            for (int i = 0; i < TW; ++i) {
+                uint32_t pl[PLANES];
+                split_planes(u[i], pl);
+                const uint32_t off = i * 128 + (((lane >> 2) ^ ((warp * TW + i) & 7)) << 4);
+#pragma unroll
+                for (int q = 0; q < PLANES; ++q) *(uint32_t *)(st + q * S::PLANE + off) = pl[q];
+                if (SAVE) {
+                    if (own && ta + i < T) { *d0 = pl[0]; *d1 = pl[1]; *d2 = pl[2]; }
+                    d0 += row_words; d1 += row_words; d2 += row_words;
+                }
+            }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(U_FULL(kc & 1));
+        }
+        if (ok) ok = warp_wait(ACC, 0, spin, (volatile int *)&abort_s);
+        if (!ok && lane == 0) { abort_s = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
+        tc_fence_after();
+        dependency_trigger();
+        const int c = mt * 128 + (warp & 3) * 32 + lane;
+        const float s = c < dh ? decay_rate_acc(f.lambda[head * dh + c], f.c) : 0.0f;
+        if (__all_sync(0xffffffffu, s <= S_POLY)) forward_epilogue<IOT, SAVE, TOK, true>(p, tmem, b, head, mt, chunk, xch, &abort_s, s);
+        else forward_epilogue<IOT, SAVE, TOK, false>(p, tmem, b, head, mt, chunk, xch, &abort_s, s);
+        tc_fence_before();
+    }
+    __syncthreads();
+    if (abort_s) {   // let copies and MMAs in flight land before shared and tensor memory are given back
+        const uint64_t tw = gtimer();
+        while (gtimer() - tw < 50000ull) __nanosleep(1000);
+        __syncthreads();
+    }
+    if (warp == 8) tmem_dealloc(tmem, S::COLS);
+}
+
+// ------------------------------------------------------------------ reverse scan
+//   g_t = dy_t + a_{t+1} g_{t+1};  dL = g a (h_{t-1} - a v / m);  dv = g m;  di = dv u;  du = dv i;
+//   dr = -s dL;  dz_a = dr r (1-r);  dz_x = di i (1-i);  dLambda += dL c r sigmoid(-Lambda).
+// Block = (chunk of 64 tokens, sequence, 64 channels): a thread holds eight tokens x two adjacent channels.  h_{t-1} is run again from
+// the state before the thread's tokens, u convolved again from x, so that 8 bytes of fp32 an element (r and i) are what the forward
+// leaves behind.
+struct SplitRevArgs {
+    BwdArgs q;
+    const float *conv_b, *h_seg;
+    uint32_t *dz;         // [head][gate][plane][B T][dh] bf16
+    Chain ch;
+    int nchunk, ctiles;
+};
+constexpr int REV_CHUNK = 64;
+struct RevShared {
+    f32x2 agg[2][8][32], in_g[8][32], sums[3][8][32];
+    int ok;
+};
+
+template <typename IOT, bool POLY>
+__device__ __forceinline__ void reverse_chunk(const SplitRevArgs &p, RevShared &sh, int b, int link, int ct, f32x2 lam, f32x2 s) {
+    const BwdArgs &q = p.q;
+    const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5, chunk = p.nchunk - 1 - link;
+    const int T = q.T, D = q.D, dh = D / q.H, n = ct * 64 + 2 * lane;
+    const bool cv = n < D;
+    const int d = cv ? n : 0, t0 = chunk * REV_CHUNK + seg * SEG, nv = min(SEG, T - t0);   // nv may be <= 0
+    const f32x2 ONE = pack2(1.0f, 1.0f), ZERO = pack2(0.0f, 0.0f), NEG = pack2(-1.0f, -1.0f);
+    const IOT *dy = (const IOT *)q.dy, *x = (const IOT *)q.x, *cs = (const IOT *)q.cs_in, *cw = (const IOT *)q.conv_w;
+    const size_t e0 = ((size_t)b * T + t0) * D + d;
+    f32x2 r[SEG], f[SEG], dyv[SEG];
+    {
+        const float *pr = q.r + e0;
+        const IOT *pd = dy + e0;
+#pragma unroll
+        for (int i = 0; i < SEG; ++i) {
+            r[i] = i < nv ? ld2f(pr) : ZERO;
+            dyv[i] = i < nv ? ld2(pd) : ZERO;
+            pr += D; pd += D;
+        }
+    }
+    f32x2 Q = ONE, G = ZERO;
+#pragma unroll
+    for (int i = SEG - 1; i >= 0; --i) {   // r = 0 for a token that does not exist: it passes g through
+        f[i] = one_minus_decay2<POLY>(r[i], s);
+        const f32x2 a = fma2(f[i], NEG, ONE);
+        G = mul2(a, __fadd2_rn(dyv[i], G));
+        Q = mul2(Q, a);
+    }
+    sh.agg[0][seg][lane] = Q; sh.agg[1][seg][lane] = G;
+    __syncthreads();
+    if (seg == 0) {
+        uint4 *slot = p.ch.slot + (size_t)b * D + d;
+        f32x2 cQ = ONE, cG = ZERO;   // the chunk as one step, before the wait
+#pragma unroll
+        for (int k = 7; k >= 0; --k) { cG = fma2(sh.agg[0][k][lane], cG, sh.agg[1][k][lane]); cQ = mul2(cQ, sh.agg[0][k][lane]); }
+        f32x2 X = ZERO;
+        float unused;
+        bool ok = true;
+        // past the last token g holds the gradient arriving on h_T (h_T = h_{T-1}, so it is carried with factor 1)
+        if (link == 0) { if (q.dh_T) X = ld2f(q.dh_T + (size_t)b * D + d); }
+        else ok = chain_wait(p.ch, slot, cv, link - 1, X.x, unused) && chain_wait(p.ch, slot + 1, cv, link - 1, X.y, unused);
+        const f32x2 Xout = fma2(cQ, X, cG);
+        if (ok && cv) {
+            chain_put(p.ch, slot, link, Xout.x, 0.0f);
+            chain_put(p.ch, slot + 1, link, Xout.y, 0.0f);
+            if (chunk == 0 && q.dh0) *(float2 *)(q.dh0 + (size_t)b * D + d) = Xout;   // a_0 g_0: h0 enters Eq. 4 only at t = 0
+        }
+#pragma unroll
+        for (int k = 7; k >= 0; --k) { sh.in_g[k][lane] = X; X = fma2(sh.agg[0][k][lane], X, sh.agg[1][k][lane]); }
+        if (!ok) {
+            if (cv) { chain_fail(p.ch, slot, link); chain_fail(p.ch, slot + 1, link); }
+            sh.ok = 0;
+        }
+    }
+    // u, i and h_{t-1} of the thread's tokens (while the first warp waits for the chain)
+    f32x2 u[SEG], gi[SEG], hp[SEG];
+    if (nv > 0) {
+        f32x2 w[4], cb = p.conv_b ? ld2f(p.conv_b + d) : ZERO;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = ld2(cw + (size_t)j * D + d);
+        auto xat = [&](int t) -> f32x2 { return t >= 0 ? ld2(x + ((size_t)b * T + t) * D + d) : cs ? ld2(cs + ((size_t)b * 3 + (3 + t)) * D + d) : ZERO; };
+        f32x2 x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
+        f32x2 h = ld2f(p.h_seg + ((size_t)b * ((T + SEG - 1) / SEG) + t0 / SEG) * D + d);
+        const float *pg = q.gi + e0;
+        const IOT *px = x + e0;
+#pragma unroll
+        for (int i = 0; i < SEG; ++i) {
+            gi[i] = i < nv ? ld2f(pg) : ZERO;
+            u[i] = i < nv ? ld2(px) : ZERO;
+            pg += D; px += D;
+        }
+#pragma unroll
+        for (int i = 0; i < SEG; ++i) {
+            const f32x2 x0 = u[i];
+            u[i] = fma2(w[3], x3, fma2(w[2], x2, fma2(w[1], x1, fma2(w[0], x0, cb))));
+            x3 = x2; x2 = x1; x1 = x0;
+            f32x2 rm;
+            hp[i] = h;
+            h = fma2(fma2(f[i], NEG, ONE), h, mul2(input_scale2(f[i], rm), mul2(gi[i], u[i])));
+        }
+    }
+    __syncthreads();
+    if (!sh.ok) return;
+    dependency_trigger();
+    f32x2 carry = sh.in_g[seg][lane], s_lam = ZERO, s_ba = ZERO, s_bx = ZERO;
+    const size_t plane = (size_t)q.B * T * dh / 2;   // of pairs
+    const int head = d / dh;
+    // from the last token of the segment backwards
+    uint32_t *dz = p.dz + (size_t)head * 2 * PLANES * plane + (((size_t)b * T + t0 + SEG - 1) * dh + (d - head * dh)) / 2;
+    float *pdu = q.hp + e0 + (size_t)(SEG - 1) * D;
+    const f32x2 ns = mul2(s, NEG);
+#pragma unroll
+    for (int i = SEG - 1; i >= 0; --i) {
+        if (i < nv && cv) {
+            f32x2 rm;
+            const f32x2 a = fma2(f[i], NEG, ONE), m = input_scale2(f[i], rm);
+            const f32x2 g = __fadd2_rn(dyv[i], carry);
+            carry = mul2(a, g);
+            const f32x2 v = mul2(gi[i], u[i]);
+            const f32x2 dLr = mul2(mul2(carry, fma2(mul2(a, v), mul2(rm, NEG), hp[i])), r[i]);   // dL r
+            const f32x2 dv = mul2(g, m);
+            const f32x2 dza = mul2(mul2(dLr, ns), fma2(r[i], NEG, ONE)), dzx = mul2(mul2(mul2(dv, u[i]), gi[i]), fma2(gi[i], NEG, ONE));
+            s_lam = __fadd2_rn(s_lam, dLr);
+            s_ba = __fadd2_rn(s_ba, dza); s_bx = __fadd2_rn(s_bx, dzx);
+            uint32_t pa[PLANES], px[PLANES];
+            split_planes(dza, pa); split_planes(dzx, px);
+#pragma unroll
+            for (int k = 0; k < PLANES; ++k) { dz[k * plane] = pa[k]; dz[(PLANES + k) * plane] = px[k]; }
+            *(float2 *)pdu = mul2(dv, gi[i]);
+        }
+        dz -= dh / 2;
+        pdu -= D;
+    }
+    sh.sums[0][seg][lane] = s_lam; sh.sums[1][seg][lane] = s_ba; sh.sums[2][seg][lane] = s_bx;
+    __syncthreads();
+    if (seg < 3 && cv) {
+        f32x2 t = ZERO;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) t = __fadd2_rn(t, sh.sums[seg][k][lane]);
+        if (seg == 0) t = mul2(t, pack2(q.c / (1.0f + expf(lam.x)), q.c / (1.0f + expf(lam.y))));   // dL/dLambda = c r sigmoid(-Lambda)
+        *(float2 *)(q.part_vec + ((size_t)(b * p.nchunk + chunk) * 3 + seg) * D + d) = t;
+    }
+}
+
+template <typename IOT> __global__ void __launch_bounds__(256, 2) split_reverse_kernel(const SplitRevArgs p) {
+    __shared__ RevShared sh;
+    if (threadIdx.x == 0) sh.ok = 1;
+    dependency_wait();
+    int bid = blockIdx.x;
+    const int ct = bid % p.ctiles; bid /= p.ctiles;
+    const int b = bid % p.q.B, link = bid / p.q.B;   // last chunk first
+    const int n = ct * 64 + 2 * (threadIdx.x & 31);
+    const f32x2 lam = n < p.q.D ? ld2f(p.q.lambda + n) : pack2(100.0f, 100.0f);
+    const f32x2 s = pack2(decay_rate_acc(lam.x, p.q.c), decay_rate_acc(lam.y, p.q.c));
+    // uniform over the block: every warp holds the same channels
+    if (__all_sync(0xffffffffu, s.x <= S_POLY && s.y <= S_POLY)) reverse_chunk<IOT, true>(p, sh, b, link, ct, lam, s);
+    else reverse_chunk<IOT, false>(p, sh, b, link, ct, lam, s);
+}
+
+// ------------------------------------------------------------------ du and dW
+// Tiles of 128 x NT results, K in blocks of 64, in one launch:
+//   dW: part[split][gate][head][o][n] = sum over the split's tokens of dz[tok][o] u[tok][n]   A = dz, B = u, both MN-major, K = tokens
+//   du: du[tok][n] += sum over gates and o of dz[tok][o] W[o][n]                              A = dz, K-major; B = W, MN-major
+// Per K block the planes of A and B arrive as tiles of 16 KB in a ring of thirteen, in an order in which they also become free: A2 B0 A1 A0
+// B1 B2 with products A2 B0, A1 B0, A0 B0, A1 B1, A0 B1, A0 B2 (bf16 weights: A2 B0 A1 A0).  After every two K blocks the
+// epilogue warps add both accumulators to fp32 registers: 128 terms are what an accumulator takes (see the top of the file; with 256 dW of
+// B1 T256 D256 was 3.9e-7 from the exact one, where the CUDA cores are 3.4e-7).
+// Persistent blocks, one per SM, with two pairs of accumulators: a pair is drained while the products fill the other.
+struct SplitProdArgs {
+    alignas(64) CUtensorMap tm_dzk, tm_dzm;   // dz planes [6 H][B T][dh], boxes of 128 tokens x 64 and 64 tokens x 64
+    alignas(64) CUtensorMap tm_u;             // u planes [3 H][B T][dh], box 64 tokens x 64
+    alignas(64) CUtensorMap tm_wa, tm_wx;     // weights [planes x H][out][in], box 64 x 64
+    int H, dh, D, NT, nt, mt, wplanes;
+    int S, kb_split, dw_tiles, tiles;
+    size_t ntok;
+    float *du, *part;
+    uint32_t *status;
+    unsigned long long spin_ns;
+};
+constexpr uint32_t PROD_BAR = PROD_RING * TILE_BYTES, PROD_ALLOC = PROD_BAR + 256 + 1024;
+constexpr int PROD_DRAIN = 2;
+
+struct ProdTile { bool dw; int head, gate, split, m0, n0, kblocks; };
+__device__ __forceinline__ ProdTile prod_tile(const SplitProdArgs &p, int i) {
+    ProdTile t{};
+    t.dw = i < p.dw_tiles;
+    if (t.dw) {
+        t.n0 = (i % p.nt) * p.NT; i /= p.nt;
+        t.m0 = (i % p.mt) * 128; i /= p.mt;
+        t.head = i % p.H; i /= p.H;
+        t.gate = i & 1; t.split = i >> 1;
+        const int total = (int)((p.ntok + 63) / 64);
+        t.kblocks = min(p.kb_split, total - t.split * p.kb_split);
+    } else {
+        i -= p.dw_tiles;
+        t.n0 = (i % p.nt) * p.NT; i /= p.nt;
+        t.head = i % p.H; t.m0 = i / p.H * 128;
+        t.kblocks = 2 * ((p.dh + 63) / 64);
+    }
+    return t;
+}
+
+__global__ void __launch_bounds__(FWD_THREADS, 1) split_products_kernel(const __grid_constant__ SplitProdArgs p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint32_t tmem_s;
+    __shared__ volatile int abort_s;
+    const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
+    const uint32_t bar = base + PROD_BAR;
+    auto FULL = [&](int i) { return bar + 8u * i; };
+    auto EMPTY = [&](int i) { return bar + 8u * (PROD_RING + i); };
+    auto ACC_FULL = [&](int i) { return bar + 16u * PROD_RING + 8u * i; };
+    auto ACC_EMPTY = [&](int i) { return bar + 16u * PROD_RING + 16u + 8u * i; };
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid == 0) {
+        for (int i = 0; i < PROD_RING; ++i) { mbar_init(FULL(i), 1); mbar_init(EMPTY(i), 1); }
+        for (int i = 0; i < 2; ++i) { mbar_init(ACC_FULL(i), 1); mbar_init(ACC_EMPTY(i), 8); }
+        abort_s = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 8) { tmem_alloc(smem_u32(&tmem_s), 512); tmem_relinquish(); }
+    if (warp == 9 && lane == 0) { prefetch_tensormap(&p.tm_dzk); prefetch_tensormap(&p.tm_dzm); prefetch_tensormap(&p.tm_u); prefetch_tensormap(&p.tm_wa); prefetch_tensormap(&p.tm_wx); }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_s;
+    const int kslots = (p.dh + 63) / 64;
+    dependency_wait();
+    bool ok = true;
+    if (warp == 9) {
+        if (lane == 0) {
+            int s = 0, round = 0;
+            for (int i = blockIdx.x; i < p.tiles && ok; i += gridDim.x) {
+                const ProdTile t = prod_tile(p, i);
+                const int bplanes = t.dw ? PLANES : p.wplanes;
+                auto load = [&](int kb, bool a, int plane) {
+                    ok = ok && mbar_wait(EMPTY(s), (round & 1) ^ 1, p.spin_ns, (volatile int *)&abort_s);
+                    if (!ok) return;
+                    const uint32_t dst = base + s * TILE_BYTES, full = FULL(s);
+                    mbar_expect_tx(full, TILE_BYTES);
+                    if (t.dw) {
+                        const int k0 = (t.split * p.kb_split + kb) * 64, c = a ? t.m0 : t.n0, row = a ? (t.head * 2 + t.gate) * PLANES + plane : t.head * PLANES + plane;
+                        const CUtensorMap *tm = a ? &p.tm_dzm : &p.tm_u;
+                        tma_load_3d(dst, tm, c, k0, row, full);
+                        tma_load_3d(dst + TILE_BYTES / 2, tm, c + 64, k0, row, full);
+                    } else {
+                        const int gate = kb >= kslots, k0 = (kb - gate * kslots) * 64;
+                        if (a) tma_load_3d(dst, &p.tm_dzk, k0, t.m0, (t.head * 2 + gate) * PLANES + plane, full);
+                        else {
+                            const CUtensorMap *tm = gate ? &p.tm_wx : &p.tm_wa;
+                            tma_load_3d(dst, tm, t.n0, k0, plane * p.H + t.head, full);
+                            tma_load_3d(dst + TILE_BYTES / 2, tm, t.n0 + 64, k0, plane * p.H + t.head, full);
+                        }
+                    }
+                    if (++s == PROD_RING) { s = 0; ++round; }
+                };
+                for (int kb = 0; kb < t.kblocks && ok; ++kb) {
+                    load(kb, true, 2); load(kb, false, 0); load(kb, true, 1); load(kb, true, 0);
+                    if (bplanes == PLANES) { load(kb, false, 1); load(kb, false, 2); }
+                }
+            }
+        }
+    } else if (warp == 8) {
+        if (lane == 0) {
+            const uint32_t id_mn = make_idesc(128, p.NT) | (1u << 15) | (1u << 16), id_bmn = make_idesc(128, p.NT) | (1u << 16);
+            int s0 = 0, r0 = 0, drains = 0;   // ring slot of the K block's first tile and its round, accumulator pairs handed over
+            for (int i = blockIdx.x; i < p.tiles && ok; i += gridDim.x) {
+                const ProdTile t = prod_tile(p, i);
+                const bool six = t.dw || p.wplanes == PLANES;
+                const uint32_t da = t.dw ? 2048 >> 4 : 32 >> 4, db = 2048 >> 4, id = t.dw ? id_mn : id_bmn;
+                const uint64_t a_desc = t.dw ? make_desc_sw128_mn(base, TILE_BYTES / 2) : make_desc_sw128(base), b_desc = make_desc_sw128_mn(base, TILE_BYTES / 2);
+                int in_acc = 0;
+                for (int kb = 0; kb < t.kblocks && ok; ++kb) {
+                    const uint32_t acc = tmem + (drains & 1) * 256;
+                    if (in_acc == 0) ok = mbar_wait(ACC_EMPTY(drains & 1), ((drains >> 1) & 1) ^ 1, p.spin_ns, (volatile int *)&abort_s);
+                    // this block's tiles, in order: A2 B0 A1 A0 B1 B2
+                    auto slot = [&](int j) { const int v = s0 + j; return v >= PROD_RING ? v - PROD_RING : v; };
+                    auto need = [&](int j) { ok = ok && mbar_wait(FULL(slot(j)), (r0 + (s0 + j >= PROD_RING)) & 1, p.spin_ns, (volatile int *)&abort_s); tc_fence_after(); };
+                    const bool full = t.dw || p.dh - (kb >= kslots ? kb - kslots : kb) * 64 >= 64, more = in_acc > 0;
+                    auto multiply = [&](int ja, int jb, int small, bool accumulate) {
+                        if (ok) mma_block(acc + small * 128, a_desc + (uint32_t)slot(ja) * (TILE_BYTES >> 4), da, b_desc + (uint32_t)slot(jb) * (TILE_BYTES >> 4), db, id, accumulate, full);
+                    };
+                    auto release = [&](int j) { if (ok) tc_commit(EMPTY(slot(j))); };
+                    need(0); need(1);
+                    multiply(0, 1, 1, more);  release(0);
+                    need(2);
+                    multiply(2, 1, 1, true);
+                    need(3);
+                    multiply(3, 1, 0, more);  release(1);
+                    if (six) {
+                        need(4);
+                        multiply(2, 4, 1, true); multiply(3, 4, 1, true);
+                        release(4);
+                        need(5);
+                        multiply(3, 5, 1, true);
+                        release(5);
+                    }
+                    release(2); release(3);
+                    s0 += six ? 6 : 4;
+                    if (s0 >= PROD_RING) { s0 -= PROD_RING; ++r0; }
+                    if (++in_acc == PROD_DRAIN || kb == t.kblocks - 1) {
+                        if (ok) tc_commit(ACC_FULL(drains & 1));
+                        ++drains; in_acc = 0;
+                    }
+                }
+            }
+        }
+    } else {
+        const int q = warp & 3, half = warp >> 2;
+        int drains = 0;
+        for (int i = blockIdx.x; i < p.tiles && ok; i += gridDim.x) {
+            const ProdTile t = prod_tile(p, i);
+            const int row = t.m0 + q * 32 + lane, c0 = t.n0 + half * 64;
+            const bool valid = t.dw ? row < p.dh : (size_t)row < p.ntok;
+            float *dst = t.dw ? p.part + ((((size_t)t.split * 2 + t.gate) * p.H + t.head) * p.dh + row) * p.dh + c0 : p.du + (size_t)row * p.D + t.head * p.dh + c0;
+            f32x2 sum[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) sum[j] = pack2(0.f, 0.f);
+            if (!t.dw && valid) {   // the direct part of du, on its way while the products run
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    if (half * 64 + j * 8 < p.NT && c0 + j * 8 < p.dh) {
+                        uint32_t o[8];
+                        ld_global_v8(dst + 8 * j, o);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) sum[4 * j + e] = pack2(__uint_as_float(o[2 * e]), __uint_as_float(o[2 * e + 1]));
+                    }
+                }
+            }
+            const int rounds = (t.kblocks + PROD_DRAIN - 1) / PROD_DRAIN;
+            for (int r = 0; r < rounds; ++r, ++drains) {
+                const int acc = drains & 1;
+                ok = warp_wait(ACC_FULL(acc), (drains >> 1) & 1, p.spin_ns, (volatile int *)&abort_s);
+                if (!ok) break;
+                tc_fence_after();
+                const uint32_t tm = tmem + ((uint32_t)(q * 32) << 16) + acc * 256 + half * 64;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (half * 64 + j * 16 < p.NT) {
+                        f32x2 v[8], w[8];
+                        tmem_ld16(tm + j * 16, v); tmem_ld16(tm + 128 + j * 16, w);
+                        tmem_ld_wait();
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) sum[8 * j + e] = __fadd2_rn(sum[8 * j + e], __fadd2_rn(v[e], w[e]));
+                    }
+                }
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(ACC_EMPTY(acc));
+            }
+            if (valid && ok) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    if (half * 64 + j * 8 < p.NT && c0 + j * 8 < p.dh) {
+                        uint32_t o[8];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) { o[2 * e] = __float_as_uint(sum[4 * j + e].x); o[2 * e + 1] = __float_as_uint(sum[4 * j + e].y); }
+                        st_global_v8(dst + 8 * j, o);
+                    }
+                }
+            }
+        }
+    }
+    dependency_trigger();
+    if (!ok && lane == 0) { abort_s = 1; atomicExch(p.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
+    tc_fence_before();
+    __syncthreads();
+    if (abort_s) {   // let copies and MMAs in flight land before shared and tensor memory are given back
+        const uint64_t tw = gtimer();
+        while (gtimer() - tw < 50000ull) __nanosleep(1000);
+        __syncthreads();
+    }
+    if (warp == 8) tmem_dealloc(tmem, 512);
+}
+
+// ------------------------------------------------------------------ host side
+inline size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+inline int ceil_div(size_t a, size_t b) { return (int)((a + b - 1) / b); }
+int num_sms() {
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 148;
+    return nsm;
+}
+inline bool width_ok(int D, int H) { return H > 0 && D % H == 0 && (D / H) % 32 == 0 && D / H <= GENERIC_MAX_DH; }
+
+bool plane_map(CUtensorMap *tm, const void *ptr, uint64_t inner, uint64_t rows, uint64_t planes, uint32_t box0, uint32_t box1) {
+    const uint64_t dims[3] = {inner, rows, planes}, strides[2] = {inner * 2, inner * rows * 2};
+    const uint32_t box[3] = {box0, box1, 1};
+    return encode_map16_3d(tm, ptr, dims, strides, box, true);
+}
+
+// Tokens per block of the forward: 64, or 32 while that leaves SMs idle
+int fwd_tokens(int B, int T, int D, int H) {
+    const size_t blocks64 = (size_t)ceil_div(T, 64) * B * H * ceil_div(D / H, 128);
+    return blocks64 >= 148 ? 64 : 32;
+}
+
+template <typename IOT, bool SAVE, int TOK>
+cudaError_t launch_forward(SplitFwdArgs &p, cudaStream_t st) {
+    static PerDeviceOptIn opt_in;
+    cudaError_t e = opt_in.ensure(split_forward_kernel<IOT, SAVE, TOK>, (int)FwdSmem<TOK>::ALLOC);
+    if (e != cudaSuccess) return e;
+    p.nchunk = ceil_div(p.f.T, TOK);
+    const size_t grid = (size_t)p.nchunk * p.f.B * p.f.H * p.mtiles;
+    if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    return launch_dependent(split_forward_kernel<IOT, SAVE, TOK>, dim3((unsigned)grid), dim3(FWD_THREADS), FwdSmem<TOK>::ALLOC, st, p);
+}
+// The weights as the products read them: the caller's (bf16), or their planes (fp32), made here in `planes`
+cudaError_t weight_planes(const FwdArgs &f, int io, void *planes, const void *&wa, const void *&wx, cudaStream_t st) {
+    if (io == RGLRU_BF16) { wa = f.W_a; wx = f.W_x; return cudaSuccess; }
+    const size_t n = (size_t)f.D * (f.D / f.H), n2 = n / 2;
+    wa = planes; wx = (const char *)planes + PLANES * n * 2;
+    return launch_dependent(split_weights_kernel, dim3((unsigned)ceil_div(2 * n2, 256)), dim3(256), 0, st, (const float *)f.W_a, (const float *)f.W_x, (uint32_t *)planes, n2);
+}
+size_t weight_plane_bytes(int D, int H, int io) { return io == RGLRU_F32 ? up256((size_t)2 * PLANES * D * (D / H) * 2) : 0; }
+
+template <bool SAVE>
+cudaError_t forward(SplitFwdArgs &p, int io, const void *wa, const void *wx, cudaStream_t st) {
+    const int dh = p.f.D / p.f.H;
+    p.mtiles = ceil_div(dh, 128);
+    p.wplanes = io == RGLRU_F32 ? PLANES : 1;
+    if (!plane_map(&p.tm_wa, wa, dh, dh, (uint64_t)p.wplanes * p.f.H, 64, 128) || !plane_map(&p.tm_wx, wx, dh, dh, (uint64_t)p.wplanes * p.f.H, 64, 128)) return cudaErrorNotSupported;
+    const bool wide = fwd_tokens(p.f.B, p.f.T, p.f.D, p.f.H) == 64;
+    if (io == RGLRU_F32) return wide ? launch_forward<float, SAVE, 64>(p, st) : launch_forward<float, SAVE, 32>(p, st);
+    return wide ? launch_forward<__nv_bfloat16, SAVE, 64>(p, st) : launch_forward<__nv_bfloat16, SAVE, 32>(p, st);
+}
+
+// Token splits of dW: a split takes as long as a tile of du or less, at most 32 splits.  (One split beside the 640 tiles of du of B5 T1021
+// D1536 in 16 heads: 224 us.)
+int dw_split(size_t ntok, int &kb_split) {
+    const int total = ceil_div(ntok, 64);
+    kb_split = ceil_div(total, 32) > 4 ? ceil_div(total, 32) : 4;
+    return ceil_div(total, kb_split);
+}
+
+}  // namespace
+
+bool split_supported(int B, int T, int D, int H) { return B > 0 && T > 0 && width_ok(D, H); }
+
+// chain records | private copy of conv_state_in (see generic_prefill) | planes of the weights
+size_t split_prefill_workspace_bytes(int B, int D, int H, int io) {
+    return up256((size_t)B * D * sizeof(uint4)) + up256((size_t)B * 3 * D * (io == RGLRU_F32 ? 4 : 2)) + weight_plane_bytes(D, H, io);
+}
+
+cudaError_t split_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_t st) {
+    SplitFwdArgs p{};
+    p.f = a;
+    char *ws = (char *)ws_body, *copy = ws + up256((size_t)a.B * a.D * sizeof(uint4));
+    const size_t cs_bytes = (size_t)a.B * 3 * a.D * (io == RGLRU_F32 ? 4 : 2);
+    p.ch = make_chain((uint4 *)ws, a);
+    const uintptr_t ci = (uintptr_t)a.cs_in, co = (uintptr_t)a.cs_out;
+    cudaError_t e;
+    if (ci && ci < co + cs_bytes && co < ci + cs_bytes) {
+        if ((e = cudaMemcpyAsync(copy, a.cs_in, cs_bytes, cudaMemcpyDeviceToDevice, st)) != cudaSuccess) return e;
+        p.f.cs_in = copy;
+    }
+    const void *wa, *wx;
+    if ((e = weight_planes(a, io, copy + up256(cs_bytes), wa, wx, st)) != cudaSuccess) return e;
+    return forward<false>(p, io, wa, wx, st);
+}
+
+size_t split_backward_workspace_bytes(int B, int T, int D, int H, int io) {
+    const size_t ntok = (size_t)B * T, dh = D / H;
+    int kb;
+    const int S = dw_split(ntok, kb);
+    size_t bytes = 3 * up256(ntok * D * 4);                                    // r, i, du
+    bytes += up256(ntok * D * PLANES * 2) + up256(ntok * D * 2 * PLANES * 2);  // planes of u and dz
+    bytes += up256((size_t)B * ceil_div(T, SEG) * D * 4);
+    bytes += up256((size_t)B * ceil_div(T, REV_CHUNK) * 3 * D * 4) + up256((size_t)B * conv_backward_chunks(B, T, D) * 5 * D * 4);
+    bytes += up256((size_t)S * 2 * D * dh * 4) + 2 * up256((size_t)B * D * sizeof(uint4));
+    return bytes + weight_plane_bytes(D, H, io);
+}
+
+cudaError_t split_backward(const FwdArgs &fwd, BwdArgs &q, int io, void *ws_body, cudaStream_t st) {
+    const int B = q.B, T = q.T, D = q.D, H = q.H, dh = D / H;
+    const size_t ntok = (size_t)B * T, wsz = (size_t)D * dh;
+    char *at = (char *)ws_body;
+    auto take = [&](size_t bytes) { char *r = at; at += up256(bytes); return r; };
+    q.r = (float *)take(ntok * D * 4); q.gi = (float *)take(ntok * D * 4); q.hp = (float *)take(ntok * D * 4);
+    char *u_planes = take(ntok * D * PLANES * 2), *dz = take(ntok * D * 2 * PLANES * 2);
+    float *h_seg = (float *)take((size_t)B * ceil_div(T, SEG) * D * 4);
+    const int rchunks = ceil_div(T, REV_CHUNK);
+    q.nchunk = conv_backward_chunks(B, T, D);
+    SplitProdArgs g{};
+    g.S = dw_split(ntok, g.kb_split);
+    q.S = g.S;
+    q.part_vec = (float *)take((size_t)B * rchunks * 3 * D * 4);
+    q.part_conv = (float *)take((size_t)B * q.nchunk * 5 * D * 4);
+    q.part_dw = (float *)take((size_t)g.S * 2 * wsz * 4);
+    uint4 *slots_f = (uint4 *)take((size_t)B * D * sizeof(uint4)), *slots_r = (uint4 *)take((size_t)B * D * sizeof(uint4));
+    char *planes = take(weight_plane_bytes(D, H, io));
+    cudaError_t e;
+    const void *wa, *wx;
+    if ((e = weight_planes(fwd, io, planes, wa, wx, st)) != cudaSuccess) return e;
+    // forward sweep
+    SplitFwdArgs p{};
+    p.f = fwd;
+    p.f.save_r = q.r; p.f.save_i = q.gi;
+    p.f.gate_branch = nullptr;
+    p.u_planes = (uint32_t *)u_planes; p.h_seg = h_seg;
+    p.ch = make_chain(slots_f, fwd);
+    if ((e = forward<true>(p, io, wa, wx, st)) != cudaSuccess) return e;
+    // reverse scan and adjoints
+    SplitRevArgs r{};
+    r.q = q; r.conv_b = fwd.conv_b; r.h_seg = h_seg; r.dz = (uint32_t *)dz; r.ch = make_chain(slots_r, fwd);
+    r.nchunk = rchunks; r.ctiles = ceil_div(D, 64);
+    const size_t rgrid = (size_t)rchunks * B * r.ctiles;
+    if (rgrid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    if ((e = launch_dependent(io == RGLRU_F32 ? split_reverse_kernel<float> : split_reverse_kernel<__nv_bfloat16>, dim3((unsigned)rgrid), dim3(256), 0, st, r)) != cudaSuccess) return e;
+    // du += W^T dz, dW = dz^T u
+    const uint64_t w3 = io == RGLRU_F32 ? PLANES : 1;
+    if (!plane_map(&g.tm_dzk, dz, dh, ntok, (uint64_t)2 * PLANES * H, 64, 128) || !plane_map(&g.tm_dzm, dz, dh, ntok, (uint64_t)2 * PLANES * H, 64, 64) ||
+        !plane_map(&g.tm_u, u_planes, dh, ntok, (uint64_t)PLANES * H, 64, 64) || !plane_map(&g.tm_wa, wa, dh, dh, w3 * H, 64, 64) || !plane_map(&g.tm_wx, wx, dh, dh, w3 * H, 64, 64))
+        return cudaErrorNotSupported;
+    g.H = H; g.dh = dh; g.D = D; g.wplanes = (int)w3; g.ntok = ntok;
+    g.nt = ceil_div(dh, 128); g.mt = g.nt; g.NT = ceil_div(ceil_div(dh, g.nt), 32) * 32;
+    g.du = q.hp; g.part = q.part_dw; g.status = fwd.status; g.spin_ns = g_spin_limit_ns;
+    const size_t dw = (size_t)g.S * 2 * H * g.mt * g.nt, tiles = dw + (size_t)ceil_div(ntok, 128) * H * g.nt;
+    if (tiles > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+    g.dw_tiles = (int)dw; g.tiles = (int)tiles;
+    const int sms = num_sms();
+    static PerDeviceOptIn opt_in;
+    if ((e = opt_in.ensure(split_products_kernel, (int)PROD_ALLOC)) != cudaSuccess) return e;
+    if ((e = launch_dependent(split_products_kernel, dim3((unsigned)(tiles < (size_t)sms ? tiles : sms)), dim3(FWD_THREADS), PROD_ALLOC, st, g)) != cudaSuccess) return e;
+    if ((e = conv_backward(q, io, q.hp, false, st)) != cudaSuccess) return e;
+    if ((e = state_conv_grads(q, io, q.hp, false, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
+    ReduceJobs jobs{};
+    add_reduce_job(jobs, q.part_dw, q.S, 2 * wsz, q.dW_a, wsz, q.dW_x, wsz, nullptr, 0);
+    add_reduce_job(jobs, q.part_vec, B * rchunks, (size_t)3 * D, q.dlambda, D, q.db_a, D, q.db_x, D);
+    add_reduce_job(jobs, q.part_conv, B * q.nchunk, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
+    return run_reduce_jobs(jobs, st);
+}
+
+}  // namespace rglru

@@ -1,0 +1,40 @@
+"""GPU parity of the kernels that keep fp32 accuracy on the tensor cores (operands as sums of bf16 values), at the edges of their tiles:
+blocks of 32 or 64 tokens and 128 channels, K blocks of 64 (32 in a last half one), segments of eight tokens, splits of dW."""
+import numpy as np
+import pytest
+
+from paper_2402_19427_b200 import inputs as synth
+from test_gpu_kernel_edges import _norm_error, forward_and_backward
+from util import f64, to_dev, to_np
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B,T,Dh,H,io", [
+    (1, 1, 32, 1, "f32"), (2, 8, 64, 1, "f32"), (1, 31, 96, 2, "f32"), (3, 33, 128, 2, "f32"), (1, 65, 160, 3, "f32"),   # 32-token blocks
+    (4, 640, 256, 4, "f32"), (3, 641, 128, 8, "f32"), (16, 63, 96, 12, "f32"),                                           # 64-token blocks
+    (1, 70, 1024, 1, "f32"), (1, 40, 544, 2, "f32"),                                                                     # many channel and K blocks
+    (1, 3, 32, 3, "bf16"), (2, 129, 224, 2, "bf16"), (7, 321, 96, 16, "bf16"), (1, 90, 384, 2, "bf16"), (5, 64, 288, 16, "bf16"),
+])
+def test_split_products_at_the_edges_of_their_tiles(oracle, B, T, Dh, H, io):
+    forward_and_backward(oracle, B, T, Dh * H, H, io, 0, seed=300 + T)
+
+
+@pytest.mark.parametrize("io,B,T,Dh,H", [("f32", 2, 515, 256, 2), ("f32", 1, 1024, 96, 3), ("bf16", 2, 1021, 96, 4), ("bf16", 1, 300, 352, 2)])
+def test_split_products_are_as_exact_as_the_cuda_cores(oracle, io, B, T, Dh, H):
+    """No output is further from the exact one (relative 2-norm) than the CUDA-core kernels' own, beyond the 2^-22 that the roundings of
+    a few hundred accumulations towards zero (2^-24 each, on a growing sum) may add where theirs happens to be smaller."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    inp = synth.make_inputs(B, T, Dh * H, H, io=io, seed=81, with_dy=True, with_state=True, bias_scale=0.2)
+    params = binding.Params.from_numpy(inp["params"], io)
+    x, h0, cs, dy = to_dev(inp["x"], io), to_dev(inp["h0"]), to_dev(inp["conv_state"], io), to_dev(inp["dy"], io)
+    h064, cs64 = inp["h0"].astype(np.float64), inp["conv_state"].astype(np.float64)
+    ref = oracle.backward(inp["x"].astype(np.float64), f64(inp["params"]), H, inp["dy"].astype(np.float64), h0=h064, conv_state_in=cs64, state_grads=True)
+    err = []
+    for flags in (0, 1):   # 1: RGLRU_FLAG_FORCE_GENERIC
+        g = binding.backward(x, params, dy, h0=h0, conv_state_in=cs, state_grads=True, flags=flags)
+        torch.cuda.synchronize()
+        err.append({k: _norm_error(to_np(g[k]), ref[k]) for k in ref})
+    for k in ref:
+        assert err[0][k] <= err[1][k] + 2.0 ** -22, (k, err[0][k], err[1][k])
