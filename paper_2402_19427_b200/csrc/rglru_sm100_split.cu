@@ -32,7 +32,7 @@ constexpr int PLANES = 3;
 constexpr int SEG = 8;                        // tokens between saved states = tokens of a thread of the reverse scan
 constexpr int FWD_THREADS = 320;              // eight warps of Conv1D and epilogue, one of copies, one of products
 constexpr uint32_t TILE_BYTES = 128 * 128;    // 128 rows (or 2 x 64 columns) of 64 bf16: one operand tile of a K block of 64
-constexpr int PROD_RING = 13;
+constexpr int PROD_STAGES = 2, PROD_THREADS = 352;   // K blocks in flight; eight epilogue warps, one of products, two of copies
 
 __device__ __forceinline__ f32x2 bf2x(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
 __device__ __forceinline__ float top16(float v) { return __uint_as_float(__float_as_uint(v) & 0xFFFF0000u); }
@@ -579,10 +579,12 @@ template <typename IOT> __global__ void __launch_bounds__(256, 2) split_reverse_
 // Tiles of 128 x NT results, K in blocks of 64, in one launch:
 //   dW: part[split][gate][head][o][n] = sum over the split's tokens of dz[tok][o] u[tok][n]   A = dz, B = u, both MN-major, K = tokens
 //   du: du[tok][n] += sum over gates and o of dz[tok][o] W[o][n]                              A = dz, K-major; B = W, MN-major
-// Per K block the planes of A and B arrive as tiles of 16 KB in a ring of thirteen, in an order in which they also become free: A2 B0 A1 A0
-// B1 B2 with products A2 B0, A1 B0, A0 B0, A1 B1, A0 B1, A0 B2 (bf16 weights: A2 B0 A1 A0).  After every two K blocks the
-// epilogue warps add both accumulators to fp32 registers: 128 terms are what an accumulator takes (see the top of the file; with 256 dW of
-// B1 T256 D256 was 3.9e-7 from the exact one, where the CUDA cores are 3.4e-7).
+// Per K block the planes of A and B arrive as tiles of 16 KB, A2 B0 first, then A1 A0 B1 B2 (bf16 weights: A1 A0), one thread copying A
+// and one B, two K blocks in flight; the first two tiles are free again after A2 B0, A1 B0, A0 B0, the others after A1 B1, A0 B1, A0 B2.
+// (With a barrier a tile, thirteen of them in a ring, and one thread for all copies, copies and products each cost their thread more
+// than the tensor core: 72 us on B4 T1024 D1024 in 4 heads.)  After every two K blocks the epilogue warps add both accumulators to
+// fp32 registers: 128 terms are what an accumulator takes (see the top of the file; with 256 dW of B1 T256 D256 was 3.9e-7 from the
+// exact one, where the CUDA cores are 3.4e-7).
 // Persistent blocks, one per SM, with two pairs of accumulators: a pair is drained while the products fill the other.
 struct SplitProdArgs {
     alignas(64) CUtensorMap tm_dzk, tm_dzm;   // dz planes [6 H][B T][dh], boxes of 128 tokens x 64 and 64 tokens x 64
@@ -595,7 +597,7 @@ struct SplitProdArgs {
     uint32_t *status;
     unsigned long long spin_ns;
 };
-constexpr uint32_t PROD_BAR = PROD_RING * TILE_BYTES, PROD_ALLOC = PROD_BAR + 256 + 1024;
+constexpr uint32_t PROD_BAR = PROD_STAGES * 6 * TILE_BYTES, PROD_ALLOC = PROD_BAR + 256 + 1024;
 constexpr int PROD_DRAIN = 2;
 
 struct ProdTile { bool dw; int head, gate, split, m0, n0, kblocks; };
@@ -618,19 +620,20 @@ __device__ __forceinline__ ProdTile prod_tile(const SplitProdArgs &p, int i) {
     return t;
 }
 
-__global__ void __launch_bounds__(FWD_THREADS, 1) split_products_kernel(const __grid_constant__ SplitProdArgs p) {
+__global__ void __launch_bounds__(PROD_THREADS, 1) split_products_kernel(const __grid_constant__ SplitProdArgs p) {
     extern __shared__ uint8_t smem_raw[];
     __shared__ uint32_t tmem_s;
     __shared__ volatile int abort_s;
     const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
     const uint32_t bar = base + PROD_BAR;
-    auto FULL = [&](int i) { return bar + 8u * i; };
-    auto EMPTY = [&](int i) { return bar + 8u * (PROD_RING + i); };
-    auto ACC_FULL = [&](int i) { return bar + 16u * PROD_RING + 8u * i; };
-    auto ACC_EMPTY = [&](int i) { return bar + 16u * PROD_RING + 16u + 8u * i; };
+    // part 0: the tiles A2 B0 of a stage, part 1: the others
+    auto FULL = [&](int st, int part) { return bar + 8u * (2 * st + part); };
+    auto EMPTY = [&](int st, int part) { return bar + 8u * (2 * PROD_STAGES + 2 * st + part); };
+    auto ACC_FULL = [&](int i) { return bar + 8u * (4 * PROD_STAGES + i); };
+    auto ACC_EMPTY = [&](int i) { return bar + 8u * (4 * PROD_STAGES + 2 + i); };
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     if (tid == 0) {
-        for (int i = 0; i < PROD_RING; ++i) { mbar_init(FULL(i), 1); mbar_init(EMPTY(i), 1); }
+        for (int i = 0; i < 2 * PROD_STAGES; ++i) { mbar_init(FULL(i >> 1, i & 1), 2); mbar_init(EMPTY(i >> 1, i & 1), 1); }
         for (int i = 0; i < 2; ++i) { mbar_init(ACC_FULL(i), 1); mbar_init(ACC_EMPTY(i), 8); }
         abort_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -644,79 +647,75 @@ __global__ void __launch_bounds__(FWD_THREADS, 1) split_products_kernel(const __
     const int kslots = (p.dh + 63) / 64;
     dependency_wait();
     bool ok = true;
-    if (warp == 9) {
+    if (warp >= 9) {
         if (lane == 0) {
-            int s = 0, round = 0;
+            const bool is_a = warp == 9;
+            int kbg = 0;   // K blocks so far
             for (int i = blockIdx.x; i < p.tiles && ok; i += gridDim.x) {
                 const ProdTile t = prod_tile(p, i);
-                const int bplanes = t.dw ? PLANES : p.wplanes;
-                auto load = [&](int kb, bool a, int plane) {
-                    ok = ok && mbar_wait(EMPTY(s), (round & 1) ^ 1, p.spin_ns, (volatile int *)&abort_s);
-                    if (!ok) return;
-                    const uint32_t dst = base + s * TILE_BYTES, full = FULL(s);
-                    mbar_expect_tx(full, TILE_BYTES);
-                    if (t.dw) {
-                        const int k0 = (t.split * p.kb_split + kb) * 64, c = a ? t.m0 : t.n0, row = a ? (t.head * 2 + t.gate) * PLANES + plane : t.head * PLANES + plane;
-                        const CUtensorMap *tm = a ? &p.tm_dzm : &p.tm_u;
-                        tma_load_3d(dst, tm, c, k0, row, full);
-                        tma_load_3d(dst + TILE_BYTES / 2, tm, c + 64, k0, row, full);
-                    } else {
-                        const int gate = kb >= kslots, k0 = (kb - gate * kslots) * 64;
-                        if (a) tma_load_3d(dst, &p.tm_dzk, k0, t.m0, (t.head * 2 + gate) * PLANES + plane, full);
+                const bool six = t.dw || p.wplanes == PLANES;
+                for (int kb = 0; kb < t.kblocks && ok; ++kb, ++kbg) {
+                    const int st = kbg % PROD_STAGES;
+                    const uint32_t parity = ((kbg / PROD_STAGES) & 1) ^ 1, s0 = base + st * 6 * TILE_BYTES;
+                    const int gate = kb >= kslots, k0 = t.dw ? (t.split * p.kb_split + kb) * 64 : (kb - gate * kslots) * 64;
+                    auto load = [&](int tile, int plane, uint32_t full) {
+                        const uint32_t dst = s0 + tile * TILE_BYTES;
+                        if (is_a && !t.dw) tma_load_3d(dst, &p.tm_dzk, k0, t.m0, (t.head * 2 + gate) * PLANES + plane, full);
                         else {
-                            const CUtensorMap *tm = gate ? &p.tm_wx : &p.tm_wa;
-                            tma_load_3d(dst, tm, t.n0, k0, plane * p.H + t.head, full);
-                            tma_load_3d(dst + TILE_BYTES / 2, tm, t.n0 + 64, k0, plane * p.H + t.head, full);
+                            const CUtensorMap *tm = t.dw ? (is_a ? &p.tm_dzm : &p.tm_u) : gate ? &p.tm_wx : &p.tm_wa;
+                            const int c = is_a ? t.m0 : t.n0, row = !t.dw ? plane * p.H + t.head : (is_a ? t.head * 2 + t.gate : t.head) * PLANES + plane;
+                            tma_load_3d(dst, tm, c, k0, row, full);
+                            tma_load_3d(dst + TILE_BYTES / 2, tm, c + 64, k0, row, full);
                         }
-                    }
-                    if (++s == PROD_RING) { s = 0; ++round; }
-                };
-                for (int kb = 0; kb < t.kblocks && ok; ++kb) {
-                    load(kb, true, 2); load(kb, false, 0); load(kb, true, 1); load(kb, true, 0);
-                    if (bplanes == PLANES) { load(kb, false, 1); load(kb, false, 2); }
+                    };
+                    ok = mbar_wait(EMPTY(st, 0), parity, p.spin_ns, (volatile int *)&abort_s);
+                    if (!ok) break;
+                    mbar_expect_tx(FULL(st, 0), TILE_BYTES);
+                    load(is_a ? 0 : 1, is_a ? 2 : 0, FULL(st, 0));
+                    if (!is_a && !six) { mbar_arrive(FULL(st, 1)); continue; }   // its wait is covered by the part-0 one of the next round
+                    ok = mbar_wait(EMPTY(st, 1), parity, p.spin_ns, (volatile int *)&abort_s);
+                    if (!ok) break;
+                    mbar_expect_tx(FULL(st, 1), 2 * TILE_BYTES);
+                    load(is_a ? 2 : 4, 1, FULL(st, 1));
+                    load(is_a ? 3 : 5, is_a ? 0 : 2, FULL(st, 1));
                 }
             }
         }
     } else if (warp == 8) {
         if (lane == 0) {
             const uint32_t id_mn = make_idesc(128, p.NT) | (1u << 15) | (1u << 16), id_bmn = make_idesc(128, p.NT) | (1u << 16);
-            int s0 = 0, r0 = 0, drains = 0;   // ring slot of the K block's first tile and its round, accumulator pairs handed over
+            constexpr uint64_t TS = TILE_BYTES >> 4;
+            int kbg = 0, drains = 0;   // K blocks so far, accumulator pairs handed over
             for (int i = blockIdx.x; i < p.tiles && ok; i += gridDim.x) {
                 const ProdTile t = prod_tile(p, i);
                 const bool six = t.dw || p.wplanes == PLANES;
                 const uint32_t da = t.dw ? 2048 >> 4 : 32 >> 4, db = 2048 >> 4, id = t.dw ? id_mn : id_bmn;
                 const uint64_t a_desc = t.dw ? make_desc_sw128_mn(base, TILE_BYTES / 2) : make_desc_sw128(base), b_desc = make_desc_sw128_mn(base, TILE_BYTES / 2);
                 int in_acc = 0;
-                for (int kb = 0; kb < t.kblocks && ok; ++kb) {
-                    const uint32_t acc = tmem + (drains & 1) * 256;
-                    if (in_acc == 0) ok = mbar_wait(ACC_EMPTY(drains & 1), ((drains >> 1) & 1) ^ 1, p.spin_ns, (volatile int *)&abort_s);
-                    // this block's tiles, in order: A2 B0 A1 A0 B1 B2
-                    auto slot = [&](int j) { const int v = s0 + j; return v >= PROD_RING ? v - PROD_RING : v; };
-                    auto need = [&](int j) { ok = ok && mbar_wait(FULL(slot(j)), (r0 + (s0 + j >= PROD_RING)) & 1, p.spin_ns, (volatile int *)&abort_s); tc_fence_after(); };
+                for (int kb = 0; kb < t.kblocks; ++kb, ++kbg) {
+                    const int st = kbg % PROD_STAGES;
+                    const uint32_t parity = (kbg / PROD_STAGES) & 1, acc = tmem + (drains & 1) * 256;
+                    const uint64_t A = a_desc + st * 6 * TS, B = b_desc + st * 6 * TS;
                     const bool full = t.dw || p.dh - (kb >= kslots ? kb - kslots : kb) * 64 >= 64, more = in_acc > 0;
-                    auto multiply = [&](int ja, int jb, int small, bool accumulate) {
-                        if (ok) mma_block(acc + small * 128, a_desc + (uint32_t)slot(ja) * (TILE_BYTES >> 4), da, b_desc + (uint32_t)slot(jb) * (TILE_BYTES >> 4), db, id, accumulate, full);
-                    };
-                    auto release = [&](int j) { if (ok) tc_commit(EMPTY(slot(j))); };
-                    need(0); need(1);
-                    multiply(0, 1, 1, more);  release(0);
-                    need(2);
-                    multiply(2, 1, 1, true);
-                    need(3);
-                    multiply(3, 1, 0, more);  release(1);
+                    if (in_acc == 0) ok = mbar_wait(ACC_EMPTY(drains & 1), ((drains >> 1) & 1) ^ 1, p.spin_ns, (volatile int *)&abort_s);
+                    ok = ok && mbar_wait(FULL(st, 0), parity, p.spin_ns, (volatile int *)&abort_s);
+                    if (!ok) break;
+                    tc_fence_after();
+                    mma_block(acc + 128, A, da, B + TS, db, id, more, full);                 // A2 B0
+                    ok = mbar_wait(FULL(st, 1), parity, p.spin_ns, (volatile int *)&abort_s);
+                    if (!ok) break;
+                    tc_fence_after();
+                    mma_block(acc + 128, A + 2 * TS, da, B + TS, db, id, true, full);        // A1 B0
+                    mma_block(acc, A + 3 * TS, da, B + TS, db, id, more, full);              // A0 B0
+                    tc_commit(EMPTY(st, 0));
                     if (six) {
-                        need(4);
-                        multiply(2, 4, 1, true); multiply(3, 4, 1, true);
-                        release(4);
-                        need(5);
-                        multiply(3, 5, 1, true);
-                        release(5);
+                        mma_block(acc + 128, A + 2 * TS, da, B + 4 * TS, db, id, true, full);   // A1 B1
+                        mma_block(acc + 128, A + 3 * TS, da, B + 4 * TS, db, id, true, full);   // A0 B1
+                        mma_block(acc + 128, A + 3 * TS, da, B + 5 * TS, db, id, true, full);   // A0 B2
                     }
-                    release(2); release(3);
-                    s0 += six ? 6 : 4;
-                    if (s0 >= PROD_RING) { s0 -= PROD_RING; ++r0; }
+                    tc_commit(EMPTY(st, 1));
                     if (++in_acc == PROD_DRAIN || kb == t.kblocks - 1) {
-                        if (ok) tc_commit(ACC_FULL(drains & 1));
+                        tc_commit(ACC_FULL(drains & 1));
                         ++drains; in_acc = 0;
                     }
                 }
@@ -938,7 +937,7 @@ cudaError_t split_backward(const FwdArgs &fwd, BwdArgs &q, int io, void *ws_body
     const int sms = num_sms();
     static PerDeviceOptIn opt_in;
     if ((e = opt_in.ensure(split_products_kernel, (int)PROD_ALLOC)) != cudaSuccess) return e;
-    if ((e = launch_dependent(split_products_kernel, dim3((unsigned)(tiles < (size_t)sms ? tiles : sms)), dim3(FWD_THREADS), PROD_ALLOC, st, g)) != cudaSuccess) return e;
+    if ((e = launch_dependent(split_products_kernel, dim3((unsigned)(tiles < (size_t)sms ? tiles : sms)), dim3(PROD_THREADS), PROD_ALLOC, st, g)) != cudaSuccess) return e;
     if ((e = conv_backward(q, io, q.hp, false, st)) != cudaSuccess) return e;
     if ((e = state_conv_grads(q, io, q.hp, false, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
     ReduceJobs jobs{};
