@@ -30,14 +30,15 @@
  *    a workspace must be ordered like calls.  After RGLRU_ERR_TIMEOUT, zero the workspace before a graph that uses it is
  *    replayed: the replay looks for the records that the failed run left incomplete.
  *  - Shapes without a kernel return RGLRU_ERR_UNSUPPORTED.  There is no CPU fallback.
- *  - Kernels.  bf16 io with a head width D_h that is a multiple of 32 runs on tensor-core kernels: prefill at any such width up
- *    to 1024, the decode step up to 256, the backward up to 256 when T is a multiple of 8.  Section 4.1 fixes 16 blocks, so D_h is 256 only at D_RNN = 4096; it is 96
+ *  - Kernels.  Head widths D_h that are multiples of 32, up to 1024, run on tensor-core kernels: prefill and backward at any such
+ *    width, fp32 or bf16, the decode step of bf16 up to 256.  Section 4.1 fixes 16 blocks, so D_h is 256 only at D_RNN = 4096; it is 96
  *    at D_RNN = 1536, 128 at 2048 and 160 at 2560.  Narrower heads share, or occupy alone, groups of 256 channel slots whose
- *    weight tile is block-diagonal; the slots a width leaves unused are idle work.  Every other shape with D_h <= 1024, fp32
- *    or bf16, runs on shape-generic CUDA-core kernels.
- *  - Precision.  State and sums are fp32 everywhere.  Between their parts the CUDA-core kernels and the prefill of heads wider than
- *    256 keep fp32 (fp32 outputs within a few 1e-6 of the exact ones, relative 2-norm).  The other tensor-core kernels use 16-bit
- *    operands: the prefill keeps the Conv1D output and the weights in fp16 (finite overflow saturates at 65504; h_T within 1e-4), the
+ *    weight tile is block-diagonal; the slots a width leaves unused are idle work.  Every other shape with D_h <= 1024
+ *    runs on shape-generic CUDA-core kernels.
+ *  - Precision.  State and sums are fp32 everywhere.  fp32 io, the prefill and backward of heads wider than 256, the backward when T is
+ *    no multiple of 8, and the CUDA-core kernels keep fp32 between their parts (fp32 outputs within a few 1e-6 of the exact ones,
+ *    relative 2-norm; their tensor-core products split fp32 operands into bf16 values that add up to them).  The other tensor-core
+ *    kernels use 16-bit operands: the prefill keeps the Conv1D output and the weights in fp16 (finite overflow saturates at 65504; h_T within 1e-4), the
  *    decode step in bf16, the backward its intermediates in fp16 and h_{t-1} in bf16 (parameter gradients within 5e-4).
  */
 #ifndef RGLRU_H_

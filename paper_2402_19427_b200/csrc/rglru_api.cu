@@ -44,7 +44,7 @@ bool use_sm100_prefill(const rglru_shape_t *s) {
     return !(s->flags & RGLRU_FLAG_FORCE_GENERIC) && sm100_prefill_supported(s->B, s->T, s->D, s->H, s->io);
 }
 
-// Split products on the tensor cores, where neither the 16-bit kernels nor the CUDA-core ones are meant
+// Calls that are promised fp32 throughout, on the tensor cores: what the 16-bit kernels do not take, at widths that are multiples of 32
 bool use_split(const rglru_shape_t *s) { return !(s->flags & RGLRU_FLAG_FORCE_GENERIC) && split_supported(s->B, s->T, s->D, s->H); }
 
 // Two helper streams and the events that tie them to the caller's stream for rglru_prefill_host, one set per device,

@@ -831,8 +831,8 @@ unsigned gemm_grid(const GemmArgs &g) {
     return (unsigned)(ntiles < nsm ? ntiles : nsm);
 }
 
-// Groups of heads, the unit of the GEMMs and of the z / dz arrays: k = 256 / width (rounded down) consecutive heads, or (forward
-// only) one head wider than 256.  Its NS channel slots (the channels rounded up) are nt column tiles of NT <= 256.
+// Groups of heads, the unit of the GEMMs and of the z / dz arrays: k = 256 / width (rounded down) consecutive heads in
+// NS channel slots, their channels rounded up to K blocks of 64: one column tile (nt = 1, NT = NS).
 struct Groups {
     int dh, k, G, hstride, NS, NT, nt;
     size_t W16_bytes() const { return (size_t)2 * G * NS * NS * 2; }
@@ -840,13 +840,11 @@ struct Groups {
 Groups make_groups(int D, int H) {
     Groups g{};
     g.dh = D / H;
-    g.k = g.dh < DH ? DH / g.dh : 1;
+    g.k = DH / g.dh;
     g.G = (H + g.k - 1) / g.k;
     g.hstride = g.k * g.dh;
-    g.nt = (g.hstride + DH - 1) / DH;
-    const int unit = g.nt % 2 ? 64 : 32;   // NS has to be a multiple of 64, the K block
-    g.NT = (((g.hstride + g.nt - 1) / g.nt + unit - 1) / unit) * unit;
-    g.NS = g.nt * g.NT;
+    g.nt = 1;
+    g.NT = g.NS = (g.hstride + 63) / 64 * 64;
     return g;
 }
 
@@ -940,10 +938,10 @@ cudaError_t gemm_z(const Groups &gr, int D, size_t ntok, const __half *u, const 
 // gradient are kept (reduce_dw_blocks_kernel).  Slots beyond the group's channels do not exist: they meet zero weights, the scan
 // writes zeros for those that share a 64-slot block with real ones, the other blocks are left out of the products, and nothing of
 // them is written to du.
-// T a multiple of 8, and no wider heads: those calls get the CUDA-core kernels, which hold u, r, i, h, dz and du in fp32.  These
-// kernels run them too, five times as fast (B5 T1021 D1536 in 16 heads 133 against 665 us, B1 T512 D5632 in 16 heads 117 against
-// 534), but keep u, z, dz and du in fp16 and h_{t-1} in bf16: gradients of the parameters are then 2e-4 to 5e-4 from the exact ones
-// (2-norm) where fp32 is 2e-6, and a caller of such a shape has been promised the latter.
+// T a multiple of 8, and no wider heads: those calls get the kernels with split products (rglru_sm100_split.cu), which hold u, r, i,
+// h, dz and du in fp32.  These kernels run them too, twice as fast (B5 T1021 D1536 in 16 heads 133 us), but keep u, z, dz and du in
+// fp16 and h_{t-1} in bf16: gradients of the parameters are then 2e-4 to 5e-4 from the exact ones (2-norm) where fp32 is below
+// 1e-6, and a caller of such a shape has been promised the latter.
 bool sm100_backward_supported(int B, int T, int D, int H, int io) {
     if (io != RGLRU_BF16 || B <= 0 || T <= 0 || T % 8 != 0 || H <= 0 || D % H != 0) return false;
     const int dh = D / H;

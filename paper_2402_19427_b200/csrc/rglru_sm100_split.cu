@@ -294,7 +294,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
             int it = 0;
             for (int kc = 0; kc < nk && ok; ++kc) {
                 for (int g = 0; g < 2 && ok; ++g) {
-                    for (int q = p.wplanes - 1; q >= 0 && ok; --q, ++it) {
+                    for (int q = 0; q < p.wplanes && ok; ++q, ++it) {
                         const int s = it % S::SLOTS;
                         ok = mbar_wait(W_EMPTY(s), ((it / S::SLOTS) & 1) ^ 1, spin, (volatile int *)&abort_s);
                         if (!ok) break;
@@ -307,7 +307,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
         }
     } else if (warp == 8) {
         if (lane == 0) {
-            constexpr uint32_t idesc = make_idesc(128, TOK);
+            // the planes of u lie one behind the other, and so do a gate's two accumulators: the first two planes are one operand of twice the width
+            constexpr uint32_t idesc = make_idesc(128, TOK), idesc2 = make_idesc(128, 2 * TOK);
             constexpr int WP = sizeof(IOT) == 4 ? PLANES : 1;
             bool ok = true;
             int slot = 0, round = 0;
@@ -318,14 +319,19 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
                 const uint64_t u_desc = make_desc_sw128(base + (kc & 1) * S::STAGE);
 #pragma unroll
                 for (int i = 0; i < 2 * WP; ++i) {
-                    const int g = i / WP, q = WP - 1 - i % WP;   // gate, plane of the weights: smallest first
+                    const int g = i / WP, q = i % WP;   // gate, plane of the weights
+                    const uint32_t acc = tmem + 2 * g * TOK;
                     ok = ok && mbar_wait(W_FULL(slot), round & 1, spin, (volatile int *)&abort_s);
                     if (!ok) break;
                     tc_fence_after();
                     const uint64_t w_desc = make_desc_sw128(base + S::RING + slot * TILE_BYTES);
-#pragma unroll
-                    for (int pl = 2 - q; pl >= 0; --pl)
-                        mma_block(tmem + (2 * g + (q + pl != 0)) * TOK, w_desc, 2, u_desc + pl * (S::PLANE >> 4), 2, idesc, kc > 0 || (q + pl != 0 && !(q == WP - 1 && pl == 2 - q)), full);
+                    if (q == 0) {
+                        mma_block(acc, w_desc, 2, u_desc, 2, idesc2, kc > 0, full);
+                        mma_block(acc + TOK, w_desc, 2, u_desc + 2 * (S::PLANE >> 4), 2, idesc, true, full);
+                    } else {
+                        mma_block(acc + TOK, w_desc, 2, u_desc, 2, idesc, true, full);
+                        if (q == 1) mma_block(acc + TOK, w_desc, 2, u_desc + (S::PLANE >> 4), 2, idesc, true, full);
+                    }
                     tc_commit(W_EMPTY(slot));
                     if (++slot == S::SLOTS) { slot = 0; ++round; }
                 }
