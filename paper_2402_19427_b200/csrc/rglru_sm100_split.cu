@@ -112,7 +112,7 @@ template <int TOK> struct FwdSmem {
 };
 
 template <typename IOT, bool SAVE, int TOK, bool POLY>
-__device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t tmem, int b, int head, int mt, int chunk, float *xch, volatile int *abort_flag, float s) {
+__device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t tmem, int b, int head, int mt, int chunk, float *xch, volatile int *abort_flag, float s, uint32_t acc_bar, bool ok) {
     constexpr int HALF = TOK / 2;
     const FwdArgs &f = p.f;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, half = warp >> 2;
@@ -128,7 +128,23 @@ __device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t
     for (int j = 0; j < 4; ++j) w[j] = ld1(cw + (size_t)j * D + d);
     float x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
     const uint32_t tm = tmem + ((uint32_t)(q * 32) << 16) + half * HALF;
-    float P = 1.0f, h = 0.0f, segP[HALF / SEG], segH[HALF / SEG];
+    float P = 1.0f, h = 0.0f, segP[HALF / SEG], segH[HALF / SEG], xn[SEG];
+    auto fetch = [&](int tb) {
+        if (tb + SEG <= T) {
+            const IOT *px = xb + (size_t)tb * D;
+#pragma unroll
+            for (int k = 0; k < SEG; ++k) { xn[k] = ld1(px); px += D; }
+        } else {
+#pragma unroll
+            for (int k = 0; k < SEG; ++k) xn[k] = xat(tb + k);
+        }
+    };
+    fetch(t0);
+    // everything above is on its way while the products run
+    if (ok) ok = warp_wait(acc_bar, 0, p.ch.spin_ns, abort_flag);
+    if (!ok && lane == 0) { *abort_flag = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
+    tc_fence_after();
+    dependency_trigger();
 #pragma unroll(SAVE ? HALF / SEG : 1)
     for (int j = 0; j < HALF / SEG; ++j) {
         f32x2 za[4], zx[4], la[4], lx[4];
@@ -136,14 +152,10 @@ __device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t
         tmem_ld8p(tm + j * SEG, za); tmem_ld8p(tm + TOK + j * SEG, la); tmem_ld8p(tm + 2 * TOK + j * SEG, zx); tmem_ld8p(tm + 3 * TOK + j * SEG, lx);
         float xs[SEG];
         const bool whole = tb + SEG <= T;
-        if (whole) {
-            const IOT *px = xb + (size_t)tb * D;
+        if (SAVE && j > 0) fetch(tb);
 #pragma unroll
-            for (int k = 0; k < SEG; ++k) { xs[k] = ld1(px); px += D; }
-        } else {
-#pragma unroll
-            for (int k = 0; k < SEG; ++k) xs[k] = xat(tb + k);
-        }
+        for (int k = 0; k < SEG; ++k) xs[k] = xn[k];
+        if (!SAVE && j + 1 < HALF / SEG) fetch(tb + SEG);   // SAVE has no registers left for it
         float *pr = nullptr, *pi = nullptr;
         if (SAVE) { const size_t e = ((size_t)b * T + tb) * D + d; pr = f.save_r + e; pi = f.save_i + e; }
         tmem_ld_wait();
@@ -189,7 +201,7 @@ __device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t
         uint4 *slot = p.ch.slot + (size_t)b * D + d;
         const float P1 = xP[chl], h1 = xh[chl], cP = P * P1, cH = fmaf(P1, h, h1);
         float P_in = 1.0f;
-        bool ok = !*abort_flag;
+        ok = !*abort_flag;
         if (ok) {
             if (chunk == 0) carry = f.h0 ? f.h0[(size_t)b * D + d] : 0.0f;
             else ok = chain_wait(p.ch, slot, cv, chunk - 1, carry, P_in);
@@ -282,12 +294,43 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
     }
     if (warp == 8) { tmem_alloc(smem_u32(&tmem_s), S::COLS); tmem_relinquish(); }
     if (warp == 9 && lane == 0) { prefetch_tensormap(&p.tm_wa); prefetch_tensormap(&p.tm_wx); }
+    const unsigned long long spin = p.ch.spin_ns;
+    dependency_wait();
+    // u of 64 channels x TOK tokens at a time: lane = two adjacent channels, warp = TOK / 8 tokens.  The first loads are on their way
+    // while the block sets itself up.
+    constexpr int TW = TOK / 8;
+    const int ta = chunk * TOK + warp * TW;
+    const IOT *x = (const IOT *)f.x + (size_t)b * T * D + head * dh, *cw = (const IOT *)f.conv_w + head * dh, *cs = (const IOT *)f.cs_in;
+    if (cs) cs += (size_t)b * 3 * D + head * dh;
+    f32x2 xr[TW + 3], w[4], cb;
+    const bool inside = ta >= 3 && ta + TW <= T;   // uniform over the warp
+    auto fetch = [&](int kc) {
+        const int k = kc * 64 + 2 * lane;
+        const bool kv = k < dh;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) w[j] = kv ? ld2(cw + (size_t)j * D + k) : pack2(0.f, 0.f);
+        cb = kv && f.conv_b ? ld2f(f.conv_b + head * dh + k) : pack2(0.f, 0.f);
+        if (inside && kc * 64 + 64 <= dh) {
+            const IOT *px = x + (size_t)(ta - 3) * D + k;
+#pragma unroll
+            for (int i = 0; i < TW + 3; ++i) { xr[i] = ld2(px); px += D; }
+            return;
+        }
+#pragma unroll
+        for (int i = 0; i < TW + 3; ++i) {
+            const int t = ta - 3 + i;
+            xr[i] = pack2(0.f, 0.f);
+            if (kv) {
+                if (t >= 0) { if (t < T) xr[i] = ld2(x + (size_t)t * D + k); }
+                else if (cs) xr[i] = ld2(cs + (size_t)(3 + t) * D + k);
+            }
+        }
+    };
+    if (warp < 8) fetch(0);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_s;
-    const unsigned long long spin = p.ch.spin_ns;
-    dependency_wait();
     if (warp == 9) {
         if (lane == 0) {
             bool ok = true;
@@ -341,38 +384,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
             else { abort_s = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
         }
     } else {
-        // ---- u of 64 channels x TOK tokens at a time: lane = two adjacent channels, warp = TOK / 8 tokens
-        constexpr int TW = TOK / 8;
-        const int ta = chunk * TOK + warp * TW;
-        const IOT *x = (const IOT *)f.x + (size_t)b * T * D + head * dh, *cw = (const IOT *)f.conv_w + head * dh, *cs = (const IOT *)f.cs_in;
-        if (cs) cs += (size_t)b * 3 * D + head * dh;
-        f32x2 xr[TW + 3];
-        const bool inside = ta >= 3 && ta + TW <= T;   // uniform over the warp
-        f32x2 w[4], cb;
-        auto fetch = [&](int kc) {
-            const int k = kc * 64 + 2 * lane;
-            const bool kv = k < dh;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = kv ? ld2(cw + (size_t)j * D + k) : pack2(0.f, 0.f);
-            cb = kv && f.conv_b ? ld2f(f.conv_b + head * dh + k) : pack2(0.f, 0.f);
-            if (inside && kc * 64 + 64 <= dh) {
-                const IOT *px = x + (size_t)(ta - 3) * D + k;
-#pragma unroll
-                for (int i = 0; i < TW + 3; ++i) { xr[i] = ld2(px); px += D; }
-                return;
-            }
-#pragma unroll
-            for (int i = 0; i < TW + 3; ++i) {
-                const int t = ta - 3 + i;
-                xr[i] = pack2(0.f, 0.f);
-                if (k < dh) {
-                    if (t >= 0) { if (t < T) xr[i] = ld2(x + (size_t)t * D + k); }
-                    else if (cs) xr[i] = ld2(cs + (size_t)(3 + t) * D + k);
-                }
-            }
-        };
         bool ok = true;
-        fetch(0);
         for (int kc = 0; kc < nk; ++kc) {
             const int k = kc * 64 + 2 * lane;
             const bool kv = k < dh;
@@ -403,14 +415,10 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
             __syncwarp();
             if (lane == 0) mbar_arrive(U_FULL(kc & 1));
         }
-        if (ok) ok = warp_wait(ACC, 0, spin, (volatile int *)&abort_s);
-        if (!ok && lane == 0) { abort_s = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
-        tc_fence_after();
-        dependency_trigger();
         const int c = mt * 128 + (warp & 3) * 32 + lane;
         const float s = c < dh ? decay_rate_acc(f.lambda[head * dh + c], f.c) : 0.0f;
-        if (__all_sync(0xffffffffu, s <= S_POLY)) forward_epilogue<IOT, SAVE, TOK, true>(p, tmem, b, head, mt, chunk, xch, &abort_s, s);
-        else forward_epilogue<IOT, SAVE, TOK, false>(p, tmem, b, head, mt, chunk, xch, &abort_s, s);
+        if (__all_sync(0xffffffffu, s <= S_POLY)) forward_epilogue<IOT, SAVE, TOK, true>(p, tmem, b, head, mt, chunk, xch, &abort_s, s, ACC, ok);
+        else forward_epilogue<IOT, SAVE, TOK, false>(p, tmem, b, head, mt, chunk, xch, &abort_s, s, ACC, ok);
         tc_fence_before();
     }
     __syncthreads();
@@ -442,26 +450,16 @@ struct RevShared {
 };
 
 template <typename IOT, bool POLY>
-__device__ __forceinline__ void reverse_chunk(const SplitRevArgs &p, RevShared &sh, int b, int link, int ct, f32x2 lam, f32x2 s) {
+__device__ __forceinline__ void reverse_chunk(const SplitRevArgs &p, RevShared &sh, int b, int link, int ct, f32x2 lam, f32x2 s, f32x2 (&r)[SEG], f32x2 (&dyv)[SEG]) {
     const BwdArgs &q = p.q;
     const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5, chunk = p.nchunk - 1 - link;
     const int T = q.T, D = q.D, dh = D / q.H, n = ct * 64 + 2 * lane;
     const bool cv = n < D;
     const int d = cv ? n : 0, t0 = chunk * REV_CHUNK + seg * SEG, nv = min(SEG, T - t0);   // nv may be <= 0
     const f32x2 ONE = pack2(1.0f, 1.0f), ZERO = pack2(0.0f, 0.0f), NEG = pack2(-1.0f, -1.0f);
-    const IOT *dy = (const IOT *)q.dy, *x = (const IOT *)q.x, *cs = (const IOT *)q.cs_in, *cw = (const IOT *)q.conv_w;
+    const IOT *x = (const IOT *)q.x, *cs = (const IOT *)q.cs_in, *cw = (const IOT *)q.conv_w;
     const size_t e0 = ((size_t)b * T + t0) * D + d;
-    f32x2 r[SEG], f[SEG], dyv[SEG];
-    {
-        const float *pr = q.r + e0;
-        const IOT *pd = dy + e0;
-#pragma unroll
-        for (int i = 0; i < SEG; ++i) {
-            r[i] = i < nv ? ld2f(pr) : ZERO;
-            dyv[i] = i < nv ? ld2(pd) : ZERO;
-            pr += D; pd += D;
-        }
-    }
+    f32x2 f[SEG];
     f32x2 Q = ONE, G = ZERO;
 #pragma unroll
     for (int i = SEG - 1; i >= 0; --i) {   // r = 0 for a token that does not exist: it passes g through
@@ -573,12 +571,23 @@ template <typename IOT> __global__ void __launch_bounds__(256, 2) split_reverse_
     int bid = blockIdx.x;
     const int ct = bid % p.ctiles; bid /= p.ctiles;
     const int b = bid % p.q.B, link = bid / p.q.B;   // last chunk first
-    const int n = ct * 64 + 2 * (threadIdx.x & 31);
-    const f32x2 lam = n < p.q.D ? ld2f(p.q.lambda + n) : pack2(100.0f, 100.0f);
+    const int n = ct * 64 + 2 * (threadIdx.x & 31), D = p.q.D, t0 = (p.nchunk - 1 - link) * REV_CHUNK + (threadIdx.x >> 5) * SEG, nv = min(SEG, p.q.T - t0);
+    const bool cv = n < D;
+    const f32x2 lam = cv ? ld2f(p.q.lambda + n) : pack2(100.0f, 100.0f), ZERO = pack2(0.0f, 0.0f);
+    f32x2 r[SEG], dyv[SEG];   // on their way while the decay rates are computed
+    const size_t e0 = ((size_t)b * p.q.T + t0) * D + (cv ? n : 0);
+    const float *pr = p.q.r + e0;
+    const IOT *pd = (const IOT *)p.q.dy + e0;
+#pragma unroll
+    for (int i = 0; i < SEG; ++i) {
+        r[i] = i < nv ? ld2f(pr) : ZERO;
+        dyv[i] = i < nv ? ld2(pd) : ZERO;
+        pr += D; pd += D;
+    }
     const f32x2 s = pack2(decay_rate_acc(lam.x, p.q.c), decay_rate_acc(lam.y, p.q.c));
     // uniform over the block: every warp holds the same channels
-    if (__all_sync(0xffffffffu, s.x <= S_POLY && s.y <= S_POLY)) reverse_chunk<IOT, true>(p, sh, b, link, ct, lam, s);
-    else reverse_chunk<IOT, false>(p, sh, b, link, ct, lam, s);
+    if (__all_sync(0xffffffffu, s.x <= S_POLY && s.y <= S_POLY)) reverse_chunk<IOT, true>(p, sh, b, link, ct, lam, s, r, dyv);
+    else reverse_chunk<IOT, false>(p, sh, b, link, ct, lam, s, r, dyv);
 }
 
 // ------------------------------------------------------------------ du and dW
