@@ -37,10 +37,10 @@ constexpr int PROD_STAGES = 2, PROD_THREADS = 352;   // K blocks in flight; eigh
 __device__ __forceinline__ f32x2 bf2x(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
 __device__ __forceinline__ float top16(float v) { return __uint_as_float(__float_as_uint(v) & 0xFFFF0000u); }
 __device__ __forceinline__ uint32_t tops(f32x2 v) { return __byte_perm(__float_as_uint(v.x), __float_as_uint(v.y), 0x7632); }   // the upper halves, v.x's below
-// The planes of two values, each the upper half of what is left: eight bits at a time and exact.  An infinity becomes the largest finite
-// value first (it would leave a NaN behind itself; as a factor of the products it is the same to the gates).
-__device__ __forceinline__ void split_planes(f32x2 v, uint32_t (&w)[PLANES]) {
-    v = pack2(clamp_nan(v.x, 3.402823466e38f), clamp_nan(v.y, 3.402823466e38f));
+// The planes of two values, each the upper half of what is left: eight bits at a time and exact.  An infinity leaves a NaN behind itself:
+// right for gradients, which stay non-finite.  CLAMP: it becomes the largest finite value first, which is the same to the gates.
+template <bool CLAMP> __device__ __forceinline__ void split_planes(f32x2 v, uint32_t (&w)[PLANES]) {
+    if (CLAMP) v = pack2(clamp_nan(v.x, 3.402823466e38f), clamp_nan(v.y, 3.402823466e38f));
 #pragma unroll
     for (int q = 0; q < PLANES; ++q) {
         w[q] = tops(v);
@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) split_weights_kernel(const float *Wa, con
     if (i >= 2 * n2) return;
     const size_t gate = i >= n2, j = i - gate * n2;
     uint32_t w[PLANES];
-    split_planes(ld2f((gate ? Wx : Wa) + 2 * j), w);
+    split_planes<true>(ld2f((gate ? Wx : Wa) + 2 * j), w);
 #pragma unroll
     for (int q = 0; q < PLANES; ++q) out[(gate * PLANES + q) * n2 + j] = w[q];
 }
@@ -105,7 +105,7 @@ struct SplitFwdArgs {
     int wplanes;          // 1 (bf16 weights) or 3
 };
 template <int TOK> struct FwdSmem {
-    static constexpr int SLOTS = TOK == 32 ? 5 : 3;   // weight tiles in flight, two blocks on an SM all the same
+    static constexpr int SLOTS = TOK == 32 ? 10 : 3;   // weight tiles in flight: two blocks of 64 tokens share an SM, one of 32 has it to itself
     static constexpr uint32_t PLANE = TOK * 128, STAGE = PLANES * PLANE, RING = 2 * STAGE, BAR = RING + SLOTS * TILE_BYTES;
     static constexpr uint32_t ALLOC = BAR + 256 + 1024;
     static constexpr uint32_t COLS = 4 * TOK;   // z_a, z_x: leading product and the small ones
@@ -402,7 +402,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
 #pragma unroll
             for (int i = 0; i < TW; ++i) {
                 uint32_t pl[PLANES];
-                split_planes(u[i], pl);
+                split_planes<true>(u[i], pl);
                 const uint32_t off = i * 128 + (((lane >> 2) ^ ((warp * TW + i) & 7)) << 4);
 #pragma unroll
                 for (int q = 0; q < PLANES; ++q) *(uint32_t *)(st + q * S::PLANE + off) = pl[q];
@@ -545,7 +545,7 @@ __device__ __forceinline__ void reverse_chunk(const SplitRevArgs &p, RevShared &
             s_lam = __fadd2_rn(s_lam, dLr);
             s_ba = __fadd2_rn(s_ba, dza); s_bx = __fadd2_rn(s_bx, dzx);
             uint32_t pa[PLANES], px[PLANES];
-            split_planes(dza, pa); split_planes(dzx, px);
+            split_planes<false>(dza, pa); split_planes<false>(dzx, px);
 #pragma unroll
             for (int k = 0; k < PLANES; ++k) { dz[k * plane] = pa[k]; dz[(PLANES + k) * plane] = px[k]; }
             *(float2 *)pdu = mul2(dv, gi[i]);
@@ -820,10 +820,10 @@ bool plane_map(CUtensorMap *tm, const void *ptr, uint64_t inner, uint64_t rows, 
     return encode_map16_3d(tm, ptr, dims, strides, box, true);
 }
 
-// Tokens per block of the forward: 64, or 32 while that leaves SMs idle
+// Tokens per block of the forward: 64, or 32 while that gives every block an SM of its own
 int fwd_tokens(int B, int T, int D, int H) {
-    const size_t blocks64 = (size_t)ceil_div(T, 64) * B * H * ceil_div(D / H, 128);
-    return blocks64 >= 148 ? 64 : 32;
+    const size_t blocks32 = (size_t)ceil_div(T, 32) * B * H * ceil_div(D / H, 128);
+    return blocks32 <= 148 ? 32 : 64;
 }
 
 template <typename IOT, bool SAVE, int TOK>
