@@ -38,3 +38,19 @@ def test_split_products_are_as_exact_as_the_cuda_cores(oracle, io, B, T, Dh, H):
         err.append({k: _norm_error(to_np(g[k]), ref[k]) for k in ref})
     for k in ref:
         assert err[0][k] <= err[1][k] + 2.0 ** -22, (k, err[0][k], err[1][k])
+
+
+def test_split_backward_keeps_an_overflowed_gradient_non_finite():
+    """An infinite dy must not come out as finite weight gradients: loss scaling looks for it there.  It stays in its own head."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    T, Dh, H = 40, 64, 2
+    inp = synth.make_inputs(1, T, Dh * H, H, io="f32", seed=4, with_dy=True)
+    params = binding.Params.from_numpy(inp["params"], "f32")
+    dy = to_dev(inp["dy"])
+    dy[0, 20, 3] = float("inf")
+    g = binding.backward(to_dev(inp["x"]), params, dy)
+    torch.cuda.synchronize()
+    for k in ("W_a", "W_x"):
+        assert not bool(torch.isfinite(g[k][0, 3]).any()), k
+        assert bool(torch.isfinite(g[k][1]).all()), k
