@@ -55,4 +55,11 @@ __device__ __forceinline__ float decay_rate_acc(float lambda, float c) {
     return c * (z > 0.0f ? z + log1pf(expf(-z)) : log1pf(expf(z)));
 }
 
+// GeLU(v) = v Phi(v), the non-linearity on the second branch of the recurrent block (Section 2.3).  Below -64 Phi(v) is 0 in fp32, and
+// -64 stands in for v: -infinity times that 0 would be NaN
+__device__ __forceinline__ float gelu_acc(float v) {
+    v = v < -64.0f ? -64.0f : v;
+    return 0.5f * v * (1.0f + erff(v * 0.70710678f));
+}
+
 }  // namespace rglru

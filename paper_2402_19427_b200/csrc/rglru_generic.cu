@@ -14,6 +14,7 @@
 #include <cuda_fp16.h>
 
 #include "rglru_chain.cuh"
+#include "rglru_gates32.cuh"
 #include "rglru_internal.h"
 #include "sm100_ptx.cuh"
 
@@ -47,8 +48,6 @@ __device__ __forceinline__ void ld4(const __nv_bfloat16 *p, float *v) {
 }
 
 __device__ __forceinline__ float sigmoid_acc(float z) { return 1.0f / (1.0f + expf(-z)); }
-// GeLU(v) = v Phi(v), the non-linearity on the second branch of the recurrent block (Section 2.3)
-__device__ __forceinline__ float gelu(float v) { return 0.5f * v * (1.0f + erff(v * 0.70710678f)); }
 
 // s = c * softplus(-Lambda) = -c log sigmoid(Lambda)   (Appendix A, with a = sigmoid(Lambda))
 __device__ __forceinline__ float decay_rate(float lambda, float c) {
@@ -353,7 +352,7 @@ __global__ void __launch_bounds__(MT, BM == 64 ? 3 : 6) generic_forward_kernel(F
                 const float hv = fmaf(P[i][j], in_h[ty][tx * NH + j], h[i][j]);
                 if (SAVE) a.save_hprev[e + j] = hv;
                 // merged output of the recurrent block (Section 2.3): GeLU on the second branch, then the product
-                else stf((IOT *)a.y, e + j, gb ? hv * gelu(ldf(gb, e + j)) : hv);
+                else stf((IOT *)a.y, e + j, gb ? hv * gelu_acc(ldf(gb, e + j)) : hv);
             }
         }
     }

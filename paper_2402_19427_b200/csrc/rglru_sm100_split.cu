@@ -252,10 +252,7 @@ __device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t
         for (int k = 0; k < SEG; ++k) {
             if (tb + k < T && cv) {
                 float o = fmaf(k & 1 ? Pv[k / 2].y : Pv[k / 2].x, carry, k & 1 ? hv[k / 2].y : hv[k / 2].x);
-                if (gb) {   // merged output of the recurrent block (Section 2.3): v Phi(v) of the second branch, then the product
-                    const float g = ld1(gb + e + (size_t)k * D);
-                    o *= 0.5f * g * (1.0f + erff(g * 0.70710678f));
-                }
+                if (gb) o *= gelu_acc(ld1(gb + e + (size_t)k * D));   // merged output of the recurrent block (Section 2.3)
                 st1(y, o);
             }
             y += D;

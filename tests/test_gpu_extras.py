@@ -163,21 +163,25 @@ def test_time_shares_on_the_gpu_equal_the_uncut_prefill(oracle, world, with_stat
     assert np.array_equal(to_np(out[-1][2]), cr)
 
 
-@pytest.mark.parametrize("Dh,H", [(256, 1), (96, 2)])
-def test_gate_branch_of_extreme_values(Dh, H):
-    """GeLU(v) = v Phi(v) at the ends of the number range: v for large v (infinity included), 0 for very negative v, NaN for NaN."""
+@pytest.mark.parametrize("Dh,H,io,flags", [
+    (256, 1, "bf16", 0), (96, 2, "bf16", 0),                           # fused prefill
+    (96, 2, "f32", 0), (288, 1, "bf16", 0),                            # split products
+    (34, 2, "f32", 0), (96, 2, "f32", 1), (288, 1, "bf16", 1)])        # CUDA cores
+def test_gate_branch_of_extreme_values(Dh, H, io, flags):
+    """GeLU(v) = v Phi(v) at the ends of the number range: v for large v (infinity included), 0 for very negative v (infinity included),
+    NaN for NaN."""
     import torch
     from paper_2402_19427_b200 import binding
     from util import to_dev
     B, T, D = 1, 40, Dh * H
-    inp = synth.make_inputs(B, T, D, H, io="bf16", seed=17)
-    params = binding.Params.from_numpy(inp["params"], "bf16")
-    x = to_dev(inp["x"], "bf16")
-    h = binding.prefill(x, params)[0].float()
-    vals = torch.tensor([float("inf"), 3e38, 1e19, 100.0, 40.0, -40.0, -100.0, -1e19, -3e38, 0.0], device="cuda")
-    branch = vals.repeat(T * D // len(vals) + 1)[:T * D].view(B, T, D).to(torch.bfloat16)
+    inp = synth.make_inputs(B, T, D, H, io=io, seed=17)
+    params = binding.Params.from_numpy(inp["params"], io)
+    x = to_dev(inp["x"], io)
+    h = binding.prefill(x, params, flags=flags)[0].float()
+    vals = torch.tensor([float("inf"), 3e38, 1e19, 100.0, 40.0, -40.0, -100.0, -1e19, -3e38, float("-inf"), 0.0], device="cuda")
+    branch = vals.repeat(T * D // len(vals) + 1)[:T * D].view(B, T, D).to(x.dtype)
     branch[0, 7, 11] = float("nan")
-    y = binding.prefill(x, params, gate_branch=branch)[0].float()
+    y = binding.prefill(x, params, gate_branch=branch, flags=flags)[0].float()
     torch.cuda.synchronize()
     want = h * torch.where(branch.float() > 0, branch.float(), torch.zeros_like(h))
     assert torch.isnan(y[0, 7, 11])
