@@ -2,9 +2,10 @@
 // heads wider than 256 and the backward of bf16 calls that are promised fp32 between the kernels (heads wider than 256, ragged
 // lengths).  Head widths that are multiples of 32.
 //
-// An fp32 value is the exact sum of three bf16 values ("planes": 8 + 8 + 8 significant bits, each the upper half of what the ones before
-// leave).  A product of two fp32 operands is the sum of the six plane products of at least 2^-16 of the first one's size -- the other
-// three are below 2^-24 --, and bf16 weights are a single plane, so that three products do.  They run on tcgen05 (kind::f16, bf16) and
+// An fp32 value is the exact sum of three bf16 values ("planes": each the nearest to what the ones before leave, so that it is at most
+// 2^-8 and 2^-17 of the value).  A product of two fp32 operands is the sum of six plane products; the other three are at most 2^-24 of it
+// together, of either sign (planes cut off instead of rounded leave out up to 2^-21, always of the product's sign), and bf16 weights are
+// a single plane, so that three products do.  They run on tcgen05 (kind::f16, bf16) and
 // accumulate in fp32 tensor memory.  The accumulation rounds towards zero: measured on 128 x 128 tiles of random numbers, relative
 // 2-norm error (bias) 5.5e-8 (-2.8e-8) after 64 products a result, 1.9e-7 (-1.2e-7) after 256, 8.6e-7 (-5.5e-7) after 1024, against
 // 4.5e-8, 0.9e-7 and 2.1e-7 of a chain of fp32 FMAs.  So the leading product of each pair of planes has an accumulator of its own,
@@ -35,17 +36,27 @@ constexpr uint32_t TILE_BYTES = 128 * 128;    // 128 rows (or 2 x 64 columns) of
 constexpr int PROD_STAGES = 2, PROD_THREADS = 352;   // K blocks in flight; eight epilogue warps, one of products, two of copies
 
 __device__ __forceinline__ f32x2 bf2x(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
-__device__ __forceinline__ float top16(float v) { return __uint_as_float(__float_as_uint(v) & 0xFFFF0000u); }
 __device__ __forceinline__ uint32_t tops(f32x2 v) { return __byte_perm(__float_as_uint(v.x), __float_as_uint(v.y), 0x7632); }   // the upper halves, v.x's below
-// The planes of two values, each the upper half of what is left: eight bits at a time and exact.  An infinity leaves a NaN behind itself:
-// right for gradients, which stay non-finite.  CLAMP: it becomes the largest finite value first, which is the same to the gates.
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+    uint32_t r;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
+    return r;
+}
+__device__ __forceinline__ float bound_bf16(float v) {   // the largest finite bf16 value, with v's sign, for what would round up to infinity; a NaN stays one
+    float y;
+    asm("min.NaN.xorsign.abs.f32 %0, %1, %2;" : "=f"(y) : "f"(v), "f"(3.38953139e38f));
+    return y;
+}
+// The planes of two values: the nearest bf16 value to what is left, twice; what is left then (at most eight bits) is a bf16 value itself.
+// An infinity leaves a NaN behind itself: right for gradients, which stay non-finite.  CLAMP: it becomes the largest finite value first,
+// which is the same to the gates.
 template <bool CLAMP> __device__ __forceinline__ void split_planes(f32x2 v, uint32_t (&w)[PLANES]) {
     if (CLAMP) v = pack2(clamp_nan(v.x, 3.402823466e38f), clamp_nan(v.y, 3.402823466e38f));
-#pragma unroll
-    for (int q = 0; q < PLANES; ++q) {
-        w[q] = tops(v);
-        if (q + 1 < PLANES) v = fma2(pack2(top16(v.x), top16(v.y)), pack2(-1.0f, -1.0f), v);
-    }
+    w[0] = pack_bf16(bound_bf16(v.x), bound_bf16(v.y));
+    v = fma2(bf2x(w[0]), pack2(-1.0f, -1.0f), v);
+    w[1] = pack_bf16(v.x, v.y);
+    v = fma2(bf2x(w[1]), pack2(-1.0f, -1.0f), v);
+    w[2] = tops(v);
 }
 __device__ __forceinline__ f32x2 ld2f(const float *p) { return *(const float2 *)p; }
 __device__ __forceinline__ f32x2 ld2(const float *p) { return *(const float2 *)p; }

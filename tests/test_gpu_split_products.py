@@ -54,3 +54,25 @@ def test_split_backward_keeps_an_overflowed_gradient_non_finite():
     for k in ("W_a", "W_x"):
         assert not bool(torch.isfinite(g[k][0, 3]).any()), k
         assert bool(torch.isfinite(g[k][1]).all()), k
+
+
+def test_split_products_leave_out_no_more_than_a_rounding():
+    """One token, so that every dW[o][n] is one product dz[o] u[n], with dz the db of the same call and u = x (taps 1, 0, 0, 0) of values
+    whose lower sixteen bits are all ones.  The plane products that are left out come to at most 2^-24 of it, the sum of the two
+    accumulators is rounded once (2^-24), the small one five times at 2^-7 of the size."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    Dh, H = 128, 2
+    inp = synth.make_inputs(1, 1, Dh * H, H, io="f32", seed=12, with_dy=True)
+    p = inp["params"]
+    p["conv_w"][:] = 0.0
+    p["conv_w"][0] = 1.0
+    p["conv_b"][:] = 0.0
+    x = (inp["x"].view(np.uint32) | np.uint32(0xFFFF)).view(np.float32)
+    g = binding.backward(to_dev(x), binding.Params.from_numpy(p, "f32"), to_dev(inp["dy"]))
+    torch.cuda.synchronize()
+    u = x.astype(np.float64).reshape(H, 1, Dh)
+    for W, b in (("W_a", "b_a"), ("W_x", "b_x")):
+        want = to_np(g[b]).reshape(H, Dh, 1) * u
+        worst = (np.abs(to_np(g[W]) - want) / np.abs(want)).max()
+        assert worst <= 2.0 ** -23 + 5 * 2.0 ** -31, (W, worst * 2.0 ** 24)
