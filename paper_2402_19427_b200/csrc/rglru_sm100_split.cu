@@ -48,10 +48,9 @@ __device__ __forceinline__ float bound_bf16(float v) {   // the largest finite b
     return y;
 }
 // The planes of two values: the nearest bf16 value to what is left, twice; what is left then (at most eight bits) is a bf16 value itself.
-// An infinity leaves a NaN behind itself: right for gradients, which stay non-finite.  CLAMP: it becomes the largest finite value first,
-// which is the same to the gates.
-template <bool CLAMP> __device__ __forceinline__ void split_planes(f32x2 v, uint32_t (&w)[PLANES]) {
-    if (CLAMP) v = pack2(clamp_nan(v.x, 3.402823466e38f), clamp_nan(v.y, 3.402823466e38f));
+// An infinity leaves infinity and NaN behind itself, so that whatever it enters is NaN: gradients stay non-finite, and for the gates,
+// which an infinite sum saturates, see exact_walk.
+__device__ __forceinline__ void split_planes(f32x2 v, uint32_t (&w)[PLANES]) {
     w[0] = pack_bf16(bound_bf16(v.x), bound_bf16(v.y));
     v = fma2(bf2x(w[0]), pack2(-1.0f, -1.0f), v);
     w[1] = pack_bf16(v.x, v.y);
@@ -83,7 +82,7 @@ __global__ void __launch_bounds__(256) split_weights_kernel(const float *Wa, con
     if (i >= 2 * n2) return;
     const size_t gate = i >= n2, j = i - gate * n2;
     uint32_t w[PLANES];
-    split_planes<true>(ld2f((gate ? Wx : Wa) + 2 * j), w);
+    split_planes(ld2f((gate ? Wx : Wa) + 2 * j), w);
 #pragma unroll
     for (int q = 0; q < PLANES; ++q) out[(gate * PLANES + q) * n2 + j] = w[q];
 }
@@ -122,87 +121,119 @@ template <int TOK> struct FwdSmem {
     static constexpr uint32_t COLS = 4 * TOK;   // z_a, z_x: leading product and the small ones
 };
 
-template <typename IOT, bool SAVE, int TOK, bool POLY>
-__device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t tmem, int b, int head, int mt, int chunk, float *xch, volatile int *abort_flag, float s, uint32_t acc_bar, bool ok) {
+// A channel on its walk through the tokens from zero state: what the Conv1D needs of it and where it stands
+struct Walk {
+    float ba, bx, cb, w[4], s;
+    float P, h, x1, x2, x3;   // the step so far; the last three inputs
+};
+// Gates, decay and scan of the eight tokens from tb on: za, zx are the sums of Eq. 1 and 2 without their biases, and become the running
+// steps P and h.  SAVE: r and i go to pr and pi instead.
+template <bool SAVE, bool POLY>
+__device__ __forceinline__ void walk_segment(Walk &k, f32x2 (&za)[4], f32x2 (&zx)[4], const float (&xs)[SEG], int tb, int T, int D, bool cv, float *pr, float *pi) {
+    const bool whole = tb + SEG <= T;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const f32x2 r = sigmoid2_acc(__fadd2_rn(za[j], pack2(k.ba, k.ba)));
+        const f32x2 g = sigmoid2_acc(__fadd2_rn(zx[j], pack2(k.bx, k.bx)));
+        const f32x2 fr = one_minus_decay2<POLY>(r, pack2(k.s, k.s));
+        f32x2 rm;
+        const f32x2 m = input_scale2(fr, rm);
+        float u[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float x0 = xs[2 * j + e];
+            u[e] = fmaf(k.w[3], k.x3, fmaf(k.w[2], k.x2, fmaf(k.w[1], k.x1, fmaf(k.w[0], x0, k.cb))));
+            k.x3 = k.x2; k.x2 = k.x1; k.x1 = x0;
+        }
+        const f32x2 a = fma2(fr, pack2(-1.0f, -1.0f), pack2(1.0f, 1.0f)), v = mul2(m, mul2(g, pack2(u[0], u[1])));
+        const bool e0 = whole || tb + 2 * j < T, e1 = whole || tb + 2 * j + 1 < T;
+        if (SAVE) {
+            if (e0 && cv) { *pr = r.x; *pi = g.x; }
+            pr += D; pi += D;
+            if (e1 && cv) { *pr = r.y; *pi = g.y; }
+            pr += D; pi += D;
+        }
+        // a token that does not exist holds the state
+        const float a0 = e0 ? a.x : 1.0f, v0 = e0 ? v.x : 0.0f, a1 = e1 ? a.y : 1.0f, v1 = e1 ? v.y : 0.0f;
+        k.P *= a0; k.h = fmaf(a0, k.h, v0);
+        if (!SAVE) { za[j].x = k.P; zx[j].x = k.h; }
+        k.P *= a1; k.h = fmaf(a1, k.h, v1);
+        if (!SAVE) { za[j].y = k.P; zx[j].y = k.h; }
+    }
+}
+
+// The walk of a warp that ended in a NaN, once more, with the sums of the gates made term by term: an infinite factor is NaN in the
+// products of its planes, where a sum that ends in an infinity saturates its gate.  Slow (some hundred microseconds), and only for inputs
+// or weights that are not finite.  Out of line, so that it costs the walk that everybody takes no registers; leaves the step up to each
+// segment (SAVE) in tensor memory, where the running steps go otherwise, and returns the whole one.
+template <typename IOT, bool SAVE, int TOK>
+__device__ __noinline__ float2 exact_walk(const SplitFwdArgs &p, uint32_t tm, int b, int head, int c, int t0, float s) {
+    const FwdArgs &f = p.f;
+    const int T = f.T, D = f.D, dh = D / f.H;
+    const bool cv = c < dh;
+    const IOT *x = (const IOT *)f.x + (size_t)b * T * D + head * dh, *cw = (const IOT *)f.conv_w + head * dh, *cs = (const IOT *)f.cs_in;
+    if (cs) cs += (size_t)b * 3 * D + head * dh;
+    if (!cv) c = 0;
+    const size_t row = ((size_t)head * dh + c) * dh;
+    const IOT *wa = (const IOT *)f.W_a + row, *wx = (const IOT *)f.W_x + row;
+    auto xat = [&](int t, int k) -> float { return t >= 0 ? (t < T ? ld1(x + (size_t)t * D + k) : 0.0f) : cs ? ld1(cs + (size_t)(3 + t) * D + k) : 0.0f; };
+    auto bias = [&](int k) -> float { return f.conv_b ? f.conv_b[head * dh + k] : 0.0f; };
+    Walk k{f.b_a[head * dh + c], f.b_x[head * dh + c], bias(c), {}, s, 1.0f, 0.0f, xat(t0 - 1, c), xat(t0 - 2, c), xat(t0 - 3, c)};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) k.w[i] = ld1(cw + (size_t)i * D + c);
+    float segP[TOK / 2 / SEG], segH[TOK / 2 / SEG];
+#pragma unroll
+    for (int j = 0; j < TOK / 2 / SEG; ++j) {
+        const int tb = t0 + j * SEG;
+        f32x2 za[4], zx[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { za[i] = pack2(0.f, 0.f); zx[i] = pack2(0.f, 0.f); }
+#pragma unroll 1
+        for (int n = 0; n < dh; ++n) {
+            float xv[SEG + 3], u[SEG], w[4];
+            const float cb = bias(n), a = ld1(wa + n), g = ld1(wx + n);
+#pragma unroll
+            for (int i = 0; i < SEG + 3; ++i) xv[i] = xat(tb - 3 + i, n);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = ld1(cw + (size_t)i * D + n);
+#pragma unroll
+            for (int i = 0; i < SEG; ++i) u[i] = fmaf(w[3], xv[i], fmaf(w[2], xv[i + 1], fmaf(w[1], xv[i + 2], fmaf(w[0], xv[i + 3], cb))));
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                za[i] = fma2(pack2(a, a), pack2(u[2 * i], u[2 * i + 1]), za[i]);
+                zx[i] = fma2(pack2(g, g), pack2(u[2 * i], u[2 * i + 1]), zx[i]);
+            }
+        }
+        float xs[SEG];
+#pragma unroll
+        for (int i = 0; i < SEG; ++i) xs[i] = xat(tb + i, c);
+        segP[j] = k.P; segH[j] = k.h;
+        const size_t e = ((size_t)b * T + tb) * D + head * dh + c;
+        walk_segment<SAVE, false>(k, za, zx, xs, tb, T, D, cv, SAVE ? f.save_r + e : nullptr, SAVE ? f.save_i + e : nullptr);
+        if (!SAVE) { tmem_st8p(tm + j * SEG, za); tmem_st8p(tm + 2 * TOK + j * SEG, zx); }
+    }
+    if (SAVE) {
+        f32x2 v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = j < TOK / 2 / SEG ? pack2(segP[j], segH[j]) : pack2(0.f, 0.f);
+        tmem_st8p(tm, v);
+    }
+    tmem_st_wait();
+    return make_float2(k.P, k.h);
+}
+
+// Chain of the chunks, then the outputs: y, or (SAVE) the states before the segments
+template <typename IOT, bool SAVE, int TOK>
+__device__ __forceinline__ void forward_rest(const SplitFwdArgs &p, uint32_t tmem, int b, int head, int mt, int chunk, float *xch, volatile int *abort_flag, bool ok, float P, float h,
+                                             const float (&segP)[TOK / 2 / SEG], const float (&segH)[TOK / 2 / SEG]) {
     constexpr int HALF = TOK / 2;
     const FwdArgs &f = p.f;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, half = warp >> 2;
     const int T = f.T, D = f.D, dh = D / f.H, chl = q * 32 + lane, c = mt * 128 + chl;
     const bool cv = c < dh;
     const int d = head * dh + (cv ? c : 0), t0 = chunk * TOK + half * HALF;
-    const IOT *x = (const IOT *)f.x, *cw = (const IOT *)f.conv_w, *cs_in = (const IOT *)f.cs_in;
-    const IOT *xb = x + (size_t)b * T * D + d;
-    auto xat = [&](int t) -> float { return t >= 0 ? (t < T ? ld1(xb + (size_t)t * D) : 0.0f) : cs_in ? ld1(cs_in + ((size_t)b * 3 + (3 + t)) * D + d) : 0.0f; };
-    const float ba = f.b_a[d], bx = f.b_x[d], cb = f.conv_b ? f.conv_b[d] : 0.0f;
-    float w[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) w[j] = ld1(cw + (size_t)j * D + d);
-    float x3 = xat(t0 - 3), x2 = xat(t0 - 2), x1 = xat(t0 - 1);
+    const IOT *cs_in = (const IOT *)f.cs_in, *xb = (const IOT *)f.x + (size_t)b * T * D + d;
     const uint32_t tm = tmem + ((uint32_t)(q * 32) << 16) + half * HALF;
-    float P = 1.0f, h = 0.0f, segP[HALF / SEG], segH[HALF / SEG], xn[SEG];
-    auto fetch = [&](int tb) {
-        if (tb + SEG <= T) {
-            const IOT *px = xb + (size_t)tb * D;
-#pragma unroll
-            for (int k = 0; k < SEG; ++k) { xn[k] = ld1(px); px += D; }
-        } else {
-#pragma unroll
-            for (int k = 0; k < SEG; ++k) xn[k] = xat(tb + k);
-        }
-    };
-    fetch(t0);
-    // everything above is on its way while the products run
-    if (ok) ok = warp_wait(acc_bar, 0, p.ch.spin_ns, abort_flag);
-    if (!ok && lane == 0) { *abort_flag = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
-    tc_fence_after();
-    dependency_trigger();
-#pragma unroll(SAVE ? HALF / SEG : 1)
-    for (int j = 0; j < HALF / SEG; ++j) {
-        f32x2 za[4], zx[4], la[4], lx[4];
-        const int tb = t0 + j * SEG;
-        tmem_ld8p(tm + j * SEG, za); tmem_ld8p(tm + TOK + j * SEG, la); tmem_ld8p(tm + 2 * TOK + j * SEG, zx); tmem_ld8p(tm + 3 * TOK + j * SEG, lx);
-        float xs[SEG];
-        const bool whole = tb + SEG <= T;
-        if (SAVE && j > 0) fetch(tb);
-#pragma unroll
-        for (int k = 0; k < SEG; ++k) xs[k] = xn[k];
-        if (!SAVE && j + 1 < HALF / SEG) fetch(tb + SEG);   // SAVE has no registers left for it
-        float *pr = nullptr, *pi = nullptr;
-        if (SAVE) { const size_t e = ((size_t)b * T + tb) * D + d; pr = f.save_r + e; pi = f.save_i + e; }
-        tmem_ld_wait();
-        if (SAVE) { segP[j] = P; segH[j] = h; }
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const f32x2 r = sigmoid2_acc(__fadd2_rn(__fadd2_rn(za[k], la[k]), pack2(ba, ba)));
-            const f32x2 g = sigmoid2_acc(__fadd2_rn(__fadd2_rn(zx[k], lx[k]), pack2(bx, bx)));
-            const f32x2 fr = one_minus_decay2<POLY>(r, pack2(s, s));
-            f32x2 rm;
-            const f32x2 m = input_scale2(fr, rm);
-            float u[2];
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const float x0 = xs[2 * k + e];
-                u[e] = fmaf(w[3], x3, fmaf(w[2], x2, fmaf(w[1], x1, fmaf(w[0], x0, cb))));
-                x3 = x2; x2 = x1; x1 = x0;
-            }
-            const f32x2 a = fma2(fr, pack2(-1.0f, -1.0f), pack2(1.0f, 1.0f)), v = mul2(m, mul2(g, pack2(u[0], u[1])));
-            const bool e0 = whole || tb + 2 * k < T, e1 = whole || tb + 2 * k + 1 < T;
-            if (SAVE) {
-                if (e0 && cv) { *pr = r.x; *pi = g.x; }
-                pr += D; pi += D;
-                if (e1 && cv) { *pr = r.y; *pi = g.y; }
-                pr += D; pi += D;
-            }
-            // a token that does not exist holds the state
-            const float a0 = e0 ? a.x : 1.0f, v0 = e0 ? v.x : 0.0f, a1 = e1 ? a.y : 1.0f, v1 = e1 ? v.y : 0.0f;
-            P *= a0; h = fmaf(a0, h, v0);
-            if (!SAVE) { za[k].x = P; zx[k].x = h; }
-            P *= a1; h = fmaf(a1, h, v1);
-            if (!SAVE) { za[k].y = P; zx[k].y = h; }
-        }
-        if (!SAVE) { tmem_st8p(tm + j * SEG, za); tmem_st8p(tm + 2 * TOK + j * SEG, zx); }
-    }
-    if (!SAVE) tmem_st_wait();
     // ---- chain: the first half's thread of a channel takes the state that the previous chunk reached and hands its own on
     float *xP = xch, *xh = xch + 128;
     if (half == 1) { xP[chl] = P; xh[chl] = h; }
@@ -269,6 +300,74 @@ __device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t
             y += D;
         }
     }
+}
+
+template <typename IOT, bool SAVE, int TOK, bool POLY>
+__device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t tmem, int b, int head, int mt, int chunk, float *xch, volatile int *abort_flag, float s, uint32_t acc_bar, bool ok) {
+    constexpr int HALF = TOK / 2;
+    const FwdArgs &f = p.f;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = warp & 3, half = warp >> 2;
+    const int T = f.T, D = f.D, dh = D / f.H, chl = q * 32 + lane, c = mt * 128 + chl;
+    const bool cv = c < dh;
+    const int d = head * dh + (cv ? c : 0), t0 = chunk * TOK + half * HALF;
+    const IOT *x = (const IOT *)f.x, *cw = (const IOT *)f.conv_w, *cs_in = (const IOT *)f.cs_in;
+    const IOT *xb = x + (size_t)b * T * D + d;
+    auto xat = [&](int t) -> float { return t >= 0 ? (t < T ? ld1(xb + (size_t)t * D) : 0.0f) : cs_in ? ld1(cs_in + ((size_t)b * 3 + (3 + t)) * D + d) : 0.0f; };
+    Walk k{f.b_a[d], f.b_x[d], f.conv_b ? f.conv_b[d] : 0.0f, {}, s, 1.0f, 0.0f, xat(t0 - 1), xat(t0 - 2), xat(t0 - 3)};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) k.w[j] = ld1(cw + (size_t)j * D + d);
+    const uint32_t tm = tmem + ((uint32_t)(q * 32) << 16) + half * HALF;
+    float segP[HALF / SEG], segH[HALF / SEG], xn[SEG];
+    auto fetch = [&](int tb) {
+        if (tb + SEG <= T) {
+            const IOT *px = xb + (size_t)tb * D;
+#pragma unroll
+            for (int k = 0; k < SEG; ++k) { xn[k] = ld1(px); px += D; }
+        } else {
+#pragma unroll
+            for (int k = 0; k < SEG; ++k) xn[k] = xat(tb + k);
+        }
+    };
+    fetch(t0);
+    // everything above is on its way while the products run
+    if (ok) ok = warp_wait(acc_bar, 0, p.ch.spin_ns, abort_flag);
+    if (!ok && lane == 0) { *abort_flag = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
+    tc_fence_after();
+    dependency_trigger();
+#pragma unroll(SAVE ? HALF / SEG : 1)
+    for (int j = 0; j < HALF / SEG; ++j) {
+        f32x2 za[4], zx[4], la[4], lx[4];
+        const int tb = t0 + j * SEG;
+        tmem_ld8p(tm + j * SEG, za); tmem_ld8p(tm + TOK + j * SEG, la); tmem_ld8p(tm + 2 * TOK + j * SEG, zx); tmem_ld8p(tm + 3 * TOK + j * SEG, lx);
+        float xs[SEG];
+        if (SAVE && j > 0) fetch(tb);
+#pragma unroll
+        for (int i = 0; i < SEG; ++i) xs[i] = xn[i];
+        if (!SAVE && j + 1 < HALF / SEG) fetch(tb + SEG);   // SAVE has no registers left for it
+        tmem_ld_wait();
+        if (SAVE) { segP[j] = k.P; segH[j] = k.h; }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { za[i] = __fadd2_rn(za[i], la[i]); zx[i] = __fadd2_rn(zx[i], lx[i]); }
+        const size_t e = ((size_t)b * T + tb) * D + d;
+        walk_segment<SAVE, POLY>(k, za, zx, xs, tb, T, D, cv, SAVE ? f.save_r + e : nullptr, SAVE ? f.save_i + e : nullptr);
+        if (!SAVE) { tmem_st8p(tm + j * SEG, za); tmem_st8p(tm + 2 * TOK + j * SEG, zx); }
+    }
+    if (!SAVE) tmem_st_wait();
+    float P = k.P, h = k.h;
+    if (__any_sync(0xffffffffu, cv && (P != P || h != h))) {
+        const float2 step = exact_walk<IOT, SAVE, TOK>(p, tm, b, head, c, t0, s);
+        P = step.x; h = step.y;
+        if (SAVE) {
+            f32x2 v[4];
+            tmem_ld8p(tm, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < HALF / SEG; ++j) { segP[j] = v[j].x; segH[j] = v[j].y; }
+        }
+    }
+    // made again from here on: kept across the call above they would not fit the registers of the walk
+    asm volatile("" : "+r"(b), "+r"(head), "+r"(mt), "+r"(chunk));
+    forward_rest<IOT, SAVE, TOK>(p, tmem, b, head, mt, chunk, xch, abort_flag, ok, P, h, segP, segH);
 }
 
 template <typename IOT, bool SAVE, int TOK>
@@ -410,7 +509,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
 #pragma unroll
             for (int i = 0; i < TW; ++i) {
                 uint32_t pl[PLANES];
-                split_planes<true>(u[i], pl);
+                split_planes(u[i], pl);
                 const uint32_t off = i * 128 + (((lane >> 2) ^ ((warp * TW + i) & 7)) << 4);
 #pragma unroll
                 for (int q = 0; q < PLANES; ++q) *(uint32_t *)(st + q * S::PLANE + off) = pl[q];
@@ -553,7 +652,7 @@ __device__ __forceinline__ void reverse_chunk(const SplitRevArgs &p, RevShared &
             s_lam = __fadd2_rn(s_lam, dLr);
             s_ba = __fadd2_rn(s_ba, dza); s_bx = __fadd2_rn(s_bx, dzx);
             uint32_t pa[PLANES], px[PLANES];
-            split_planes<false>(dza, pa); split_planes<false>(dzx, px);
+            split_planes(dza, pa); split_planes(dzx, px);
 #pragma unroll
             for (int k = 0; k < PLANES; ++k) { dz[k * plane] = pa[k]; dz[(PLANES + k) * plane] = px[k]; }
             *(float2 *)pdu = mul2(dv, gi[i]);

@@ -76,3 +76,45 @@ def test_split_products_leave_out_no_more_than_a_rounding():
         want = to_np(g[b]).reshape(H, Dh, 1) * u
         worst = (np.abs(to_np(g[W]) - want) / np.abs(want)).max()
         assert worst <= 2.0 ** -23 + 5 * 2.0 ** -31, (W, worst * 2.0 ** 24)
+
+
+@pytest.mark.parametrize("io,B,T,Dh,H", [("f32", 2, 70, 96, 3), ("f32", 3, 770, 64, 4), ("bf16", 2, 70, 288, 3)])   # 32 and 64 tokens a block
+@pytest.mark.parametrize("what", ["x", "two x", "zero weight", "W_a", "W_x"])
+def test_split_products_do_not_lose_an_infinity(io, B, T, Dh, H, what):
+    """An infinite input or weight in one head: a gate whose sum is infinite saturates, one whose sum is not defined (infinities of both
+    signs, an infinity times zero) gives NaN, as on the CUDA cores; no gradient is finite that is not finite there, and the other heads
+    and (for an input) sequences do not see it."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    D = Dh * H
+    inp = synth.make_inputs(B, T, D, H, io=io, seed=18, with_dy=True, with_state=True, bias_scale=0.2)
+    p = inp["params"]
+    c0 = Dh + 5   # a channel of the second head
+    p["conv_w"][0, c0], p["conv_w"][0, c0 + 9] = 0.5, 0.5
+    if what in ("W_a", "W_x"):
+        p[what][1, 7, 5] = np.inf if what == "W_a" else -np.inf
+    else:
+        inp["x"][1, 20, c0] = np.inf
+        if what == "two x":
+            inp["x"][1, 20, c0 + 9] = -np.inf
+        if what == "zero weight":
+            p["W_a"][1, :40, 5] = 0.0
+    params = binding.Params.from_numpy(p, io)
+    x, h0, cs, dy = to_dev(inp["x"], io), to_dev(inp["h0"]), to_dev(inp["conv_state"], io), to_dev(inp["dy"], io)
+    got, want = [], []
+    for flags, out in ((0, got), (1, want)):   # 1: RGLRU_FLAG_FORCE_GENERIC
+        y, hT, _ = binding.prefill(x, params, h0=h0, conv_state_in=cs, flags=flags)
+        out += [y, hT, binding.backward(x, params, dy, h0=h0, conv_state_in=cs, state_grads=True, flags=flags)]
+    torch.cuda.synchronize()
+    for a, b in zip(got[:2], want[:2]):
+        ok = torch.isfinite(b)
+        assert torch.equal(torch.isfinite(a), ok)
+        assert what in ("W_a", "W_x") or bool((~ok).any())   # an infinite weight only saturates its gate
+        np.testing.assert_allclose(to_np(a[ok]), to_np(b[ok]), rtol=2e-2 if io == "bf16" else 1e-4, atol=1e-3 if io == "bf16" else 1e-5)
+    for k, b in want[2].items():
+        a = got[2][k]
+        assert not bool((torch.isfinite(a) & ~torch.isfinite(b)).any()), k
+        per_head = a.view(H, -1) if k in ("W_a", "W_x") else a.view(-1, H, Dh).transpose(0, 1)
+        assert bool(torch.isfinite(per_head[0]).all()) and bool(torch.isfinite(per_head[2]).all()), k
+    if what not in ("W_a", "W_x"):
+        assert bool(torch.isfinite(got[0][0]).all()) and bool(torch.isfinite(got[2]["x"][0]).all())
