@@ -8,8 +8,9 @@
 // a single plane, so that three products do.  They run on tcgen05 (kind::f16, bf16) and
 // accumulate in fp32 tensor memory.  The accumulation rounds towards zero: measured on 128 x 128 tiles of random numbers, relative
 // 2-norm error (bias) 5.5e-8 (-2.8e-8) after 64 products a result, 1.9e-7 (-1.2e-7) after 256, 8.6e-7 (-5.5e-7) after 1024, against
-// 4.5e-8, 0.9e-7 and 2.1e-7 of a chain of fp32 FMAs.  So the leading product of each pair of planes has an accumulator of its own,
-// which takes at most a few hundred terms, and the small ones another, whose roundings are 2^-8 smaller.
+// 4.5e-8, 0.9e-7 and 2.1e-7 of a chain of fp32 FMAs.  So the leading product of each pair of planes has accumulators of its own, which
+// take few enough terms that no output is further from the exact one than with such chains (128 in dW and du, see forward() for the
+// gates), and the small ones, whose roundings are 2^-8 smaller, others.
 //   1. split_weights      (fp32 io) the weights as planes
 //   2. split_forward      Conv1D, planes of u, both gate products, gates, scan, chain of chunks: y, or for the backward r, i, the
 //                         state before every eighth token, and the planes of u
@@ -113,12 +114,22 @@ struct SplitFwdArgs {
     float *h_seg;         // SAVE: [B][ceil(T / SEG)][D] state before every SEG-th token
     int nchunk, mtiles;
     int wplanes;          // 1 (bf16 weights) or 3
+    int sets;             // sets of accumulators, see KSet (more than one with LATE and 32 tokens only)
+    uint32_t cols;        // columns of tensor memory: those of the sets, rounded up to a power of two
 };
+// A set is two accumulators a gate, X and Y of TOK columns each, and the K blocks [k0, k1) that it takes.  Up to kb, leading products go to
+// X and the small ones to Y, the first two planes of u as one operand of twice the width.  With LATE, the small products of the blocks
+// from kb on, at most two, go to Y too, and then the leading ones: Y still is 2^-8 of the sum when they come.  See forward() for when.
+struct KSet { int k0, kb, k1; };
+template <bool LATE> __device__ __forceinline__ KSet k_set(int nk, int sets, int i) {
+    if (!LATE) return KSet{0, nk, nk};   // one set
+    const int k0 = nk * i / sets, k1 = nk * (i + 1) / sets;
+    return KSet{k0, k1 - max(0, min(2, k1 - k0 - 2)), k1};
+}
 template <int TOK> struct FwdSmem {
     static constexpr int SLOTS = TOK == 32 ? 10 : 3;   // weight tiles in flight: two blocks of 64 tokens share an SM, one of 32 has it to itself
     static constexpr uint32_t PLANE = TOK * 128, STAGE = PLANES * PLANE, RING = 2 * STAGE, BAR = RING + SLOTS * TILE_BYTES;
     static constexpr uint32_t ALLOC = BAR + 256 + 1024;
-    static constexpr uint32_t COLS = 4 * TOK;   // z_a, z_x: leading product and the small ones
 };
 
 // A channel on its walk through the tokens from zero state: what the Conv1D needs of it and where it stands
@@ -302,7 +313,7 @@ __device__ __forceinline__ void forward_rest(const SplitFwdArgs &p, uint32_t tme
     }
 }
 
-template <typename IOT, bool SAVE, int TOK, bool POLY>
+template <typename IOT, bool SAVE, bool LATE, int TOK, bool POLY>
 __device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t tmem, int b, int head, int mt, int chunk, float *xch, volatile int *abort_flag, float s, uint32_t acc_bar, bool ok) {
     constexpr int HALF = TOK / 2;
     const FwdArgs &f = p.f;
@@ -348,6 +359,22 @@ __device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t
         if (SAVE) { segP[j] = k.P; segH[j] = k.h; }
 #pragma unroll
         for (int i = 0; i < 4; ++i) { za[i] = __fadd2_rn(za[i], la[i]); zx[i] = __fadd2_rn(zx[i], lx[i]); }
+        if (LATE && TOK == 32) {
+#pragma unroll 1
+            for (int set = 1; set < p.sets; ++set) {
+#pragma unroll
+                for (int g = 0; g < 2; ++g) {
+                    f32x2 X[4], Y[4];
+                    tmem_ld8p(tm + (4 * set + 2 * g) * TOK + j * SEG, X); tmem_ld8p(tm + (4 * set + 2 * g + 1) * TOK + j * SEG, Y);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        if (g == 0) za[i] = __fadd2_rn(za[i], __fadd2_rn(X[i], Y[i]));
+                        else zx[i] = __fadd2_rn(zx[i], __fadd2_rn(X[i], Y[i]));
+                    }
+                }
+            }
+        }
         const size_t e = ((size_t)b * T + tb) * D + d;
         walk_segment<SAVE, POLY>(k, za, zx, xs, tb, T, D, cv, SAVE ? f.save_r + e : nullptr, SAVE ? f.save_i + e : nullptr);
         if (!SAVE) { tmem_st8p(tm + j * SEG, za); tmem_st8p(tm + 2 * TOK + j * SEG, zx); }
@@ -370,7 +397,7 @@ __device__ __forceinline__ void forward_epilogue(const SplitFwdArgs &p, uint32_t
     forward_rest<IOT, SAVE, TOK>(p, tmem, b, head, mt, chunk, xch, abort_flag, ok, P, h, segP, segH);
 }
 
-template <typename IOT, bool SAVE, int TOK>
+template <typename IOT, bool SAVE, bool LATE, int TOK>
 __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __grid_constant__ SplitFwdArgs p) {
     using S = FwdSmem<TOK>;
     extern __shared__ uint8_t smem_raw[];
@@ -399,7 +426,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
         abort_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 8) { tmem_alloc(smem_u32(&tmem_s), S::COLS); tmem_relinquish(); }
+    if (warp == 8) { tmem_alloc(smem_u32(&tmem_s), p.cols); tmem_relinquish(); }
     if (warp == 9 && lane == 0) { prefetch_tensormap(&p.tm_wa); prefetch_tensormap(&p.tm_wx); }
     const unsigned long long spin = p.ch.spin_ns;
     dependency_wait();
@@ -442,15 +469,23 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
         if (lane == 0) {
             bool ok = true;
             int it = 0;
-            for (int kc = 0; kc < nk && ok; ++kc) {
-                for (int g = 0; g < 2 && ok; ++g) {
-                    for (int q = 0; q < p.wplanes && ok; ++q, ++it) {
-                        const int s = it % S::SLOTS;
-                        ok = mbar_wait(W_EMPTY(s), ((it / S::SLOTS) & 1) ^ 1, spin, (volatile int *)&abort_s);
-                        if (!ok) break;
-                        mbar_expect_tx(W_FULL(s), TILE_BYTES);
-                        tma_load_3d(base + S::RING + s * TILE_BYTES, g ? &p.tm_wx : &p.tm_wa, kc * 64, mt * 128, q * H + head, W_FULL(s));
-                    }
+            auto load = [&](int kc, int g, int q) {
+                const int s = it % S::SLOTS;
+                ok = ok && mbar_wait(W_EMPTY(s), ((it / S::SLOTS) & 1) ^ 1, spin, (volatile int *)&abort_s);
+                if (!ok) return;
+                mbar_expect_tx(W_FULL(s), TILE_BYTES);
+                tma_load_3d(base + S::RING + s * TILE_BYTES, g ? &p.tm_wx : &p.tm_wa, kc * 64, mt * 128, q * H + head, W_FULL(s));
+                ++it;
+            };
+            for (int i = 0; i < (LATE ? p.sets : 1) && ok; ++i) {
+                const KSet r = k_set<LATE>(nk, p.sets, i);
+                for (int kc = r.k0; kc < r.kb; ++kc)
+                    for (int g = 0; g < 2; ++g)
+                        for (int q = 0; q < p.wplanes; ++q) load(kc, g, q);
+                for (int g = 0; LATE && g < 2 && r.kb < r.k1; ++g) {
+                    for (int kc = r.kb; kc < r.k1; ++kc)
+                        for (int q = p.wplanes - 1; q > 0; --q) load(kc, g, q);
+                    for (int kc = r.kb; kc < r.k1; ++kc) load(kc, g, 0);
                 }
             }
             if (!ok) { abort_s = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
@@ -462,30 +497,76 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
             constexpr int WP = sizeof(IOT) == 4 ? PLANES : 1;
             bool ok = true;
             int slot = 0, round = 0;
-            for (int kc = 0; kc < nk && ok; ++kc) {
-                const bool full = dh - kc * 64 >= 64;   // else the last half block
-                ok = mbar_wait(U_FULL(kc & 1), (kc >> 1) & 1, spin, (volatile int *)&abort_s);
-                if (!ok) break;
-                const uint64_t u_desc = make_desc_sw128(base + (kc & 1) * S::STAGE);
-#pragma unroll
-                for (int i = 0; i < 2 * WP; ++i) {
-                    const int g = i / WP, q = i % WP;   // gate, plane of the weights
-                    const uint32_t acc = tmem + 2 * g * TOK;
-                    ok = ok && mbar_wait(W_FULL(slot), round & 1, spin, (volatile int *)&abort_s);
+            auto u_full = [&](int kc) { ok = ok && mbar_wait(U_FULL(kc & 1), (kc >> 1) & 1, spin, (volatile int *)&abort_s); };
+            auto w_full = [&]() {
+                ok = ok && mbar_wait(W_FULL(slot), round & 1, spin, (volatile int *)&abort_s);
+                tc_fence_after();
+                return ok;
+            };
+            auto next_slot = [&]() { if (++slot == S::SLOTS) { slot = 0; ++round; } };
+            auto w_tile = [&](int s) { return make_desc_sw128(base + S::RING + s * TILE_BYTES); };
+            constexpr uint64_t B1 = S::PLANE >> 4, B2 = 2 * B1;
+            for (int set = 0; set < (LATE ? p.sets : 1) && ok; ++set) {
+                const KSet r = k_set<LATE>(nk, p.sets, set);
+                const uint32_t acc0 = tmem + 4 * set * TOK;
+                for (int kc = r.k0; kc < r.kb && ok; ++kc) {
+                    const bool full = dh - kc * 64 >= 64;   // else the last half block
+                    u_full(kc);
                     if (!ok) break;
-                    tc_fence_after();
-                    const uint64_t w_desc = make_desc_sw128(base + S::RING + slot * TILE_BYTES);
-                    if (q == 0) {
-                        mma_block(acc, w_desc, 2, u_desc, 2, idesc2, kc > 0, full);
-                        mma_block(acc + TOK, w_desc, 2, u_desc + 2 * (S::PLANE >> 4), 2, idesc, true, full);
-                    } else {
-                        mma_block(acc + TOK, w_desc, 2, u_desc, 2, idesc, true, full);
-                        if (q == 1) mma_block(acc + TOK, w_desc, 2, u_desc + (S::PLANE >> 4), 2, idesc, true, full);
+                    const uint64_t u_desc = make_desc_sw128(base + (kc & 1) * S::STAGE);
+#pragma unroll
+                    for (int i = 0; i < 2 * WP; ++i) {
+                        const int g = i / WP, q = i % WP;   // gate, plane of the weights
+                        const uint32_t acc = acc0 + 2 * g * TOK;
+                        if (!w_full()) break;
+                        const uint64_t w_desc = w_tile(slot);
+                        if (q == 0) {
+                            mma_block(acc, w_desc, 2, u_desc, 2, idesc2, kc > r.k0, full);
+                            mma_block(acc + TOK, w_desc, 2, u_desc + B2, 2, idesc, true, full);
+                        } else {
+                            mma_block(acc + TOK, w_desc, 2, u_desc, 2, idesc, true, full);
+                            if (q == 1) mma_block(acc + TOK, w_desc, 2, u_desc + B1, 2, idesc, true, full);
+                        }
+                        tc_commit(W_EMPTY(slot));
+                        next_slot();
                     }
-                    tc_commit(W_EMPTY(slot));
-                    if (++slot == S::SLOTS) { slot = 0; ++round; }
+                    if (ok) tc_commit(U_EMPTY(kc & 1));
                 }
-                if (ok) tc_commit(U_EMPTY(kc & 1));
+                if (!LATE || r.kb == r.k1) continue;
+                for (int g = 0; g < 2 && ok; ++g) {
+                    const uint32_t acc = acc0 + (2 * g + 1) * TOK;
+                    if (WP > 1) {
+                        for (int kc = r.kb; kc < r.k1 && ok; ++kc) {
+                            const bool full = dh - kc * 64 >= 64;
+                            const uint64_t u_desc = make_desc_sw128(base + (kc & 1) * S::STAGE);
+                            if (g == 0) u_full(kc);
+#pragma unroll
+                            for (int q = WP - 1; q > 0; --q) {
+                                if (!w_full()) break;
+                                mma_block(acc, w_tile(slot), 2, u_desc, 2, idesc, true, full);
+                                if (q == 1) mma_block(acc, w_tile(slot), 2, u_desc + B1, 2, idesc, true, full);
+                                tc_commit(W_EMPTY(slot));
+                                next_slot();
+                            }
+                        }
+                    }
+                    int first = slot;   // the tiles of the first plane stay until the leading products
+                    for (int kc = r.kb; kc < r.k1 && ok; ++kc) {
+                        const bool full = dh - kc * 64 >= 64;
+                        const uint64_t u_desc = make_desc_sw128(base + (kc & 1) * S::STAGE);
+                        if (WP == 1 && g == 0) u_full(kc);
+                        if (!w_full()) break;
+                        mma_block(acc, w_tile(slot), 2, u_desc + B1, 2, idesc, true, full);
+                        mma_block(acc, w_tile(slot), 2, u_desc + B2, 2, idesc, true, full);
+                        next_slot();
+                    }
+                    for (int kc = r.kb; kc < r.k1 && ok; ++kc) {
+                        mma_block(acc, w_tile(first), 2, make_desc_sw128(base + (kc & 1) * S::STAGE), 2, idesc, true, dh - kc * 64 >= 64);
+                        tc_commit(W_EMPTY(first));
+                        if (g == 1) tc_commit(U_EMPTY(kc & 1));
+                        if (++first == S::SLOTS) first = 0;
+                    }
+                }
             }
             if (ok) tc_commit(ACC);
             else { abort_s = 1; atomicExch(f.status, STATUS_MAGIC | (uint32_t)RGLRU_ERR_TIMEOUT); }
@@ -524,8 +605,8 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
         }
         const int c = mt * 128 + (warp & 3) * 32 + lane;
         const float s = c < dh ? decay_rate_acc(f.lambda[head * dh + c], f.c) : 0.0f;
-        if (__all_sync(0xffffffffu, s <= S_POLY)) forward_epilogue<IOT, SAVE, TOK, true>(p, tmem, b, head, mt, chunk, xch, &abort_s, s, ACC, ok);
-        else forward_epilogue<IOT, SAVE, TOK, false>(p, tmem, b, head, mt, chunk, xch, &abort_s, s, ACC, ok);
+        if (__all_sync(0xffffffffu, s <= S_POLY)) forward_epilogue<IOT, SAVE, LATE, TOK, true>(p, tmem, b, head, mt, chunk, xch, &abort_s, s, ACC, ok);
+        else forward_epilogue<IOT, SAVE, LATE, TOK, false>(p, tmem, b, head, mt, chunk, xch, &abort_s, s, ACC, ok);
         tc_fence_before();
     }
     __syncthreads();
@@ -534,7 +615,7 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
         while (gtimer() - tw < 50000ull) __nanosleep(1000);
         __syncthreads();
     }
-    if (warp == 8) tmem_dealloc(tmem, S::COLS);
+    if (warp == 8) tmem_dealloc(tmem, p.cols);
 }
 
 // ------------------------------------------------------------------ reverse scan
@@ -928,21 +1009,24 @@ bool plane_map(CUtensorMap *tm, const void *ptr, uint64_t inner, uint64_t rows, 
 }
 
 // Tokens per block of the forward: 64, or 32 while that gives every block an SM of its own.  fp32 step with 64 / 32 tokens, us: B2 T100
-// D1024 in 8 heads (64 blocks of 32) 58.3 / 53.3, B3 T190 D1024 in 4 (144) 83.5 / 78.8, B3 T250 (192) 91 / 107, B4 T250 (256) 108 / 124
-int fwd_tokens(int B, int T, int D, int H) {
+// D1024 in 8 heads (64 blocks of 32) 58.3 / 53.3, B3 T190 D1024 in 4 (144) 83.5 / 78.8, B3 T250 (192) 91 / 107, B4 T250 (256) 108 / 124.
+// Fp32 calls and backwards of heads wider than 640 too: see forward().
+int fwd_tokens(int B, int T, int D, int H, bool exact) {
     const size_t blocks32 = (size_t)ceil_div(T, 32) * B * H * ceil_div(D / H, 128);
-    return blocks32 <= 148 ? 32 : 64;
+    return blocks32 <= 148 || (exact && D / H > 640) ? 32 : 64;
 }
 
-template <typename IOT, bool SAVE, int TOK>
+template <typename IOT, bool SAVE, bool LATE, int TOK>
 cudaError_t launch_forward(SplitFwdArgs &p, cudaStream_t st) {
     static PerDeviceOptIn opt_in;
-    cudaError_t e = opt_in.ensure(split_forward_kernel<IOT, SAVE, TOK>, (int)FwdSmem<TOK>::ALLOC);
+    cudaError_t e = opt_in.ensure(split_forward_kernel<IOT, SAVE, LATE, TOK>, (int)FwdSmem<TOK>::ALLOC);
     if (e != cudaSuccess) return e;
     p.nchunk = ceil_div(p.f.T, TOK);
+    p.sets = TOK == 32 && LATE ? ceil_div(ceil_div(p.f.D / p.f.H, 64), 4) : 1;
+    for (p.cols = 4 * TOK; p.cols < (uint32_t)(4 * TOK * p.sets); p.cols *= 2) {}
     const size_t grid = (size_t)p.nchunk * p.f.B * p.f.H * p.mtiles;
     if (grid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    return launch_dependent(split_forward_kernel<IOT, SAVE, TOK>, dim3((unsigned)grid), dim3(FWD_THREADS), FwdSmem<TOK>::ALLOC, st, p);
+    return launch_dependent(split_forward_kernel<IOT, SAVE, LATE, TOK>, dim3((unsigned)grid), dim3(FWD_THREADS), FwdSmem<TOK>::ALLOC, st, p);
 }
 // The weights as the products read them: the caller's (bf16), or their planes (fp32), made here in `planes`
 cudaError_t weight_planes(const FwdArgs &f, int io, void *planes, const void *&wa, const void *&wx, cudaStream_t st) {
@@ -953,15 +1037,25 @@ cudaError_t weight_planes(const FwdArgs &f, int io, void *planes, const void *&w
 }
 size_t weight_plane_bytes(int D, int H, int io) { return io == RGLRU_F32 ? up256((size_t)2 * PLANES * D * (D / H) * 2) : 0; }
 
+// How many leading products an accumulator takes.  Fp32 calls and backwards are promised the accuracy of fp32 FMAs: no output may be
+// further from the exact one than the CUDA cores' own.  The worst one's share of theirs (fp32, B40 T64, where little else hides the
+// gates' error), all in one accumulator / the last two K blocks in Y / sets of at most four K blocks, 32 tokens: width 256 0.88 / 0.78 / -,
+// 352 0.94 / 0.83 / -, 512 1.07 / 0.88 / 0.82, 640 1.19 / 0.98 / 0.77, 768 1.31 / 1.08 / 0.73, 1024 1.61 / 1.35 / 0.80.  Forward and
+// backward of B4 T1024 D1024, us: width 256 249 / 254 / -, 512 334 / 356 / 551, 1024 526 / 540 / 931 (CUDA cores 1895).  The bf16 prefill
+// has always had the first: B3 T1213 D4096 of width 1024 311 / 317 us.
 template <bool SAVE>
 cudaError_t forward(SplitFwdArgs &p, int io, const void *wa, const void *wx, cudaStream_t st) {
     const int dh = p.f.D / p.f.H;
     p.mtiles = ceil_div(dh, 128);
     p.wplanes = io == RGLRU_F32 ? PLANES : 1;
     if (!plane_map(&p.tm_wa, wa, dh, dh, (uint64_t)p.wplanes * p.f.H, 64, 128) || !plane_map(&p.tm_wx, wx, dh, dh, (uint64_t)p.wplanes * p.f.H, 64, 128)) return cudaErrorNotSupported;
-    const bool wide = fwd_tokens(p.f.B, p.f.T, p.f.D, p.f.H) == 64;
-    if (io == RGLRU_F32) return wide ? launch_forward<float, SAVE, 64>(p, st) : launch_forward<float, SAVE, 32>(p, st);
-    return wide ? launch_forward<__nv_bfloat16, SAVE, 64>(p, st) : launch_forward<__nv_bfloat16, SAVE, 32>(p, st);
+    const bool wide = fwd_tokens(p.f.B, p.f.T, p.f.D, p.f.H, SAVE || io == RGLRU_F32) == 64, late = dh > 256;
+    if (io == RGLRU_F32) {
+        if (late) return wide ? launch_forward<float, SAVE, true, 64>(p, st) : launch_forward<float, SAVE, true, 32>(p, st);
+        return wide ? launch_forward<float, SAVE, false, 64>(p, st) : launch_forward<float, SAVE, false, 32>(p, st);
+    }
+    if (SAVE && late) return wide ? launch_forward<__nv_bfloat16, SAVE, SAVE, 64>(p, st) : launch_forward<__nv_bfloat16, SAVE, SAVE, 32>(p, st);
+    return wide ? launch_forward<__nv_bfloat16, SAVE, false, 64>(p, st) : launch_forward<__nv_bfloat16, SAVE, false, 32>(p, st);
 }
 
 // Token splits of dW: a split takes as long as a tile of du or less, at most 32 splits.  (One split beside the 640 tiles of du of B5 T1021

@@ -5,7 +5,7 @@ import pytest
 
 from paper_2402_19427_b200 import inputs as synth
 from test_gpu_kernel_edges import _norm_error, forward_and_backward
-from util import f64, to_dev, to_np
+from util import f64, oracle_prefill, to_dev, to_np
 
 pytestmark = pytest.mark.gpu
 
@@ -20,10 +20,13 @@ def test_split_products_at_the_edges_of_their_tiles(oracle, B, T, Dh, H, io):
     forward_and_backward(oracle, B, T, Dh * H, H, io, 0, seed=300 + T)
 
 
-@pytest.mark.parametrize("io,B,T,Dh,H", [("f32", 2, 515, 256, 2), ("f32", 1, 1024, 96, 3), ("bf16", 2, 1021, 96, 4), ("bf16", 1, 300, 352, 2)])
+@pytest.mark.parametrize("io,B,T,Dh,H", [
+    ("f32", 2, 515, 256, 2), ("f32", 1, 1024, 96, 3), ("bf16", 2, 1021, 96, 4), ("bf16", 1, 300, 352, 2),
+    ("f32", 2, 300, 160, 2), ("f32", 2, 300, 352, 2), ("f32", 1, 400, 544, 1), ("f32", 1, 400, 1024, 1), ("f32", 40, 64, 512, 2),
+    ("f32", 40, 64, 1024, 1), ("bf16", 1, 301, 512, 1), ("bf16", 1, 300, 1024, 1)])
 def test_split_products_are_as_exact_as_the_cuda_cores(oracle, io, B, T, Dh, H):
-    """No output is further from the exact one (relative 2-norm) than the CUDA-core kernels' own, beyond the 2^-22 that the roundings of
-    a few hundred accumulations towards zero (2^-24 each, on a growing sum) may add where theirs happens to be smaller."""
+    """No fp32 output is further from the exact one (relative 2-norm) than the CUDA-core kernels' own; the bf16 ones are roundings of such
+    values, of which a few fall to the other neighbour."""
     import torch
     from paper_2402_19427_b200 import binding
     inp = synth.make_inputs(B, T, Dh * H, H, io=io, seed=81, with_dy=True, with_state=True, bias_scale=0.2)
@@ -31,13 +34,16 @@ def test_split_products_are_as_exact_as_the_cuda_cores(oracle, io, B, T, Dh, H):
     x, h0, cs, dy = to_dev(inp["x"], io), to_dev(inp["h0"]), to_dev(inp["conv_state"], io), to_dev(inp["dy"], io)
     h064, cs64 = inp["h0"].astype(np.float64), inp["conv_state"].astype(np.float64)
     ref = oracle.backward(inp["x"].astype(np.float64), f64(inp["params"]), H, inp["dy"].astype(np.float64), h0=h064, conv_state_in=cs64, state_grads=True)
+    if io == "f32" or Dh > 256:   # narrower bf16 heads have another forward
+        ref["y"], ref["h_T"], _ = oracle_prefill(oracle, inp, h0=h064, cs=cs64)
     err = []
     for flags in (0, 1):   # 1: RGLRU_FLAG_FORCE_GENERIC
         g = binding.backward(x, params, dy, h0=h0, conv_state_in=cs, state_grads=True, flags=flags)
+        g["y"], g["h_T"], _ = binding.prefill(x, params, h0=h0, conv_state_in=cs, flags=flags)
         torch.cuda.synchronize()
         err.append({k: _norm_error(to_np(g[k]), ref[k]) for k in ref})
     for k in ref:
-        assert err[0][k] <= err[1][k] + 2.0 ** -22, (k, err[0][k], err[1][k])
+        assert err[0][k] <= err[1][k] * (1.001 if g[k].dtype == torch.bfloat16 else 1.0), (k, err[0][k], err[1][k])
 
 
 def test_split_backward_keeps_an_overflowed_gradient_non_finite():
