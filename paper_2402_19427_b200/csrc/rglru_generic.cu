@@ -891,9 +891,9 @@ void add_reduce_job(ReduceJobs &jobs, const float *in, int nparts, size_t stride
     const size_t n = n0 + n1 + n2;
     if (n == 0 || (out0 == nullptr && out1 == nullptr && out2 == nullptr)) return;
     ReduceJob &q = jobs.job[jobs.n++];
-    q = ReduceJob{in, stride, out0, out1, out2, n0, n1, n2, nparts, nparts > 16 && n < 65536, 0};
-    // Up to 16 parts are two rounds of loads for one thread; longer sums are cut into slices while there are few of them (20 parts of
-    // 295k sums in slices, 32 sums a block: 22 us)
+    // Up to 16 parts are two rounds of loads for one thread; longer sums are cut into slices.  Up to 32 parts (the splits of dW) are not
+    // where there are many of them: 20 parts of 295k sums in slices, 32 sums a block, took 22 us.
+    q = ReduceJob{in, stride, out0, out1, out2, n0, n1, n2, nparts, nparts > 16 && (n < 65536 || nparts > 32), 0};
     q.blocks = ceil_div(n, q.sliced ? 32 : 256);
 }
 cudaError_t run_reduce_jobs(const ReduceJobs &jobs, cudaStream_t st) {

@@ -339,3 +339,23 @@ def test_replayed_graph_of_the_tensor_core_backward(oracle):
             gr = oracle.backward(inp["x"].astype(np.float64), f64(rounds[0]["params"]), H, inp["dy"].astype(np.float64))
             for k in ("x", "W_a", "lam"):
                 assert_close("d" + k, to_np(g[k]), gr[k], "bf16")
+
+
+@pytest.mark.parametrize("flags", [0, GENERIC])
+def test_many_partial_sums_of_a_wide_layer_are_summed_in_slices(flags):
+    """One part for each of 1024 sequences, 5 D = 66560 sums of them.  With zero gate weights and the taps (1, 0, 0, 0) du is dx, so that
+    the exact sum is at hand.  All terms are positive: added one after the other they would be off by about 2^-25 sqrt(1024) / 3 = 3.2e-7
+    (relative 2-norm), in eight slices by 4e-8."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    B, Dh, H = 1024, 32, 416
+    D = Dh * H
+    p = synth.make_inputs(1, 1, D, H, io="f32", seed=2)["params"]
+    for k in ("W_a", "W_x", "conv_w"):
+        p[k][:] = 0.0
+    p["conv_w"][0] = 1.0
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    x, dy = torch.randn(B, 1, D, generator=gen, device="cuda"), torch.rand(B, 1, D, generator=gen, device="cuda")
+    g = binding.backward(x, binding.Params.from_numpy(p, "f32"), dy, flags=flags)
+    assert _norm_error(to_np(g["conv_b"]), g["x"].double().sum((0, 1)).cpu().numpy()) < 2.0 ** -23
