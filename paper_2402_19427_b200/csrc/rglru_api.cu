@@ -45,7 +45,10 @@ bool use_sm100_prefill(const rglru_shape_t *s) {
 }
 
 // Calls that are promised fp32 throughout, on the tensor cores: what the 16-bit kernels do not take, at widths that are multiples of 32
-bool use_split(const rglru_shape_t *s) { return !(s->flags & RGLRU_FLAG_FORCE_GENERIC) && split_supported(s->B, s->T, s->D, s->H); }
+bool use_split_prefill(const rglru_shape_t *s) {
+    return !(s->flags & RGLRU_FLAG_FORCE_GENERIC) && split_prefill_supported(s->B, s->T, s->D, s->H, s->io);
+}
+bool use_split_backward(const rglru_shape_t *s) { return !(s->flags & RGLRU_FLAG_FORCE_GENERIC) && split_backward_supported(s->D, s->H); }
 
 // Two helper streams and the events that tie them to the caller's stream for rglru_prefill_host, one set per device,
 // created on first use (streams and events are not device memory).  Calls on one device are serialised by the mutex.
@@ -117,15 +120,15 @@ size_t rglru_workspace_bytes(const rglru_shape_t *s, int32_t op) {
     size_t body = 0;
     switch (op) {
         case RGLRU_OP_PREFILL:
-            body = use_sm100_prefill(s) ? sm100_prefill_workspace_bytes(s->B, s->T, s->D, s->H)
-                   : use_split(s)       ? split_prefill_workspace_bytes(s->B, s->D, s->H, s->io)
-                                        : generic_prefill_workspace_bytes(s->B, s->D, s->io);
+            body = use_sm100_prefill(s)   ? sm100_prefill_workspace_bytes(s->B, s->T, s->D, s->H)
+                   : use_split_prefill(s) ? split_prefill_workspace_bytes(s->B, s->D, s->H, s->io)
+                                          : generic_prefill_workspace_bytes(s->B, s->D, s->io);
             break;
         case RGLRU_OP_DECODE: break;
         case RGLRU_OP_BACKWARD:
-            body = use_sm100_backward(s) ? sm100_backward_workspace_bytes(s->B, s->T, s->D, s->H)
-                   : use_split(s)        ? split_backward_workspace_bytes(s->B, s->T, s->D, s->H, s->io)
-                                         : generic_backward_workspace_bytes(s->B, s->T, s->D, s->H);
+            body = use_sm100_backward(s)   ? sm100_backward_workspace_bytes(s->B, s->T, s->D, s->H)
+                   : use_split_backward(s) ? split_backward_workspace_bytes(s->B, s->T, s->D, s->H, s->io)
+                                           : generic_backward_workspace_bytes(s->B, s->T, s->D, s->H);
             break;
         default: return 0;
     }
@@ -163,7 +166,7 @@ int32_t rglru_prefill_ex(const rglru_shape_t *s, const rglru_params_t *p, const 
     cudaError_t e;
     if (use_sm100_prefill(s))
         e = sm100_prefill(a, (char *)workspace + WS_HEADER_BYTES, workspace_bytes - WS_HEADER_BYTES, st);
-    else if (use_split(s))
+    else if (use_split_prefill(s))
         e = split_prefill(a, s->io, (char *)workspace + WS_HEADER_BYTES, st);
     else
         e = generic_prefill(a, s->io, (char *)workspace + WS_HEADER_BYTES, st);
@@ -226,7 +229,7 @@ int32_t rglru_backward(const rglru_shape_t *s, const rglru_params_t *p, const vo
     if (use_sm100_backward(s))
         e = sm100_backward(f, q, y, (char *)workspace + WS_HEADER_BYTES, workspace_bytes - WS_HEADER_BYTES, (uint32_t *)workspace,
                            (cudaStream_t)cuda_stream);
-    else if (use_split(s))
+    else if (use_split_backward(s))
         e = split_backward(f, q, s->io, (char *)workspace + WS_HEADER_BYTES, (cudaStream_t)cuda_stream);
     else
         e = generic_backward(f, q, s->io, (char *)workspace + WS_HEADER_BYTES, (cudaStream_t)cuda_stream);

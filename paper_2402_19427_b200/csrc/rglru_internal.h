@@ -116,7 +116,8 @@ cudaError_t generic_decode(const FwdArgs &a, int io, cudaStream_t st);
 cudaError_t generic_backward(const FwdArgs &fwd, BwdArgs &b, int io, void *ws_body, cudaStream_t st);
 
 // ---- fp32 products on the tensor cores (fp32 io, and bf16 calls that are fp32 between the kernels; D_h a multiple of 32) ----
-bool split_supported(int B, int T, int D, int H);
+bool split_prefill_supported(int B, int T, int D, int H, int io);
+bool split_backward_supported(int D, int H);
 size_t split_prefill_workspace_bytes(int B, int D, int H, int io);
 size_t split_backward_workspace_bytes(int B, int T, int D, int H, int io);
 cudaError_t split_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_t st);

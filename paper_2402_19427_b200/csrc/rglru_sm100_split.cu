@@ -1068,7 +1068,22 @@ int dw_split(size_t ntok, int &kb_split) {
 
 }  // namespace
 
-bool split_supported(int B, int T, int D, int H) { return B > 0 && T > 0 && width_ok(D, H); }
+// The fp32 forward of a few tokens is left to the CUDA cores: the weights as planes are a launch of their own and 1.5 times the bytes, and
+// while the blocks of 32 tokens x 32 channels of the other kernel have an SM each (two to an SM up to width 128) it takes no longer for all
+// of them than for one.  Split products / CUDA cores, us: B1 T1 D1024, widths 32 9.5 / 6.6, 128 12.1 / 10.2, 256 16.7 / 15.0, 1024 44.9 / 43.6;
+// D4096, width 256, T32 (128 blocks) 19.9 / 15.8, T64 (256) 20.6 / 27.4; width 128, T64 (256) 14.3 / 14.2, T128 (512) 15.6 / 24.8; width 32,
+// T64 (256) 12.6 / 8.5.  Beyond 128 tokens the two cross between 256 and 1024 (D256, width 32: T256 12.5 / 10.7, T1024 17.5 / 23.6), and
+// the state of the CUDA cores' kernel is further from the exact one with every token (y: 2 times as far as this one's after 64, 4 after 500),
+// so that those calls stay here; width 32, where three of four rows of a block have no channel, too (B8 T4096 D1024 755 / 717).
+// The backward of any size is faster here from 32 tokens on (width 32 of D4096 from 128: T64 40.2 / 37.1), before that within 10 %
+// (width 32: 8 us).
+bool split_prefill_supported(int B, int T, int D, int H, int io) {
+    if (!width_ok(D, H)) return false;
+    const int dh = D / H;
+    const size_t blocks = (size_t)B * H * ceil_div(T, 32) * ceil_div(dh, 32);
+    return io != RGLRU_F32 || T > 128 || blocks > (dh <= 128 ? 296 : 148);
+}
+bool split_backward_supported(int D, int H) { return width_ok(D, H); }
 
 // chain records | private copy of conv_state_in (see generic_prefill) | planes of the weights
 size_t split_prefill_workspace_bytes(int B, int D, int H, int io) {

@@ -5,7 +5,7 @@ import pytest
 
 from paper_2402_19427_b200 import inputs as synth
 from test_gpu_kernel_edges import _norm_error, forward_and_backward
-from util import f64, oracle_prefill, to_dev, to_np
+from util import assert_close, f64, oracle_prefill, to_dev, to_np
 
 pytestmark = pytest.mark.gpu
 
@@ -124,3 +124,46 @@ def test_split_products_do_not_lose_an_infinity(io, B, T, Dh, H, what):
         assert bool(torch.isfinite(per_head[0]).all()) and bool(torch.isfinite(per_head[2]).all()), k
     if what not in ("W_a", "W_x"):
         assert bool(torch.isfinite(got[0][0]).all()) and bool(torch.isfinite(got[2]["x"][0]).all())
+
+
+@pytest.mark.parametrize("B,T,Dh,H,few", [
+    (1, 1, 128, 8, True), (1, 128, 256, 4, True), (1, 129, 256, 4, False), (1, 32, 256, 18, True), (1, 32, 256, 19, False),
+    (37, 9, 32, 8, True), (38, 9, 32, 8, False), (1, 33, 1024, 2, True), (2, 33, 1024, 2, False)])
+def test_fp32_forward_of_few_tokens_is_left_to_the_cuda_cores(oracle, B, T, Dh, H, few):
+    """Both sides of the rule: the CUDA cores' own results, bit for bit, where they take the call, with a workspace as small as theirs;
+    the call is right on either side, state in place."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    D = Dh * H
+    inp = synth.make_inputs(B, T, D, H, io="f32", seed=400 + T, with_state=True, bias_scale=0.2)
+    params = binding.Params.from_numpy(inp["params"], "f32")
+    out, size = [], []
+    for flags in (0, 1):   # 1: RGLRU_FLAG_FORCE_GENERIC
+        h, c = to_dev(inp["h0"]), to_dev(inp["conv_state"])
+        shape = binding.make_shape(B, T, D, H, torch.float32, flags=flags)
+        size.append(binding.workspace_bytes(shape, binding.OP_PREFILL))
+        y, _, _ = binding.prefill(to_dev(inp["x"]), params, h0=h, conv_state_in=c, h_T=h, conv_state_out=c, flags=flags)
+        out.append((y, h, c))
+    torch.cuda.synchronize()
+    assert (size[0] == size[1]) == few
+    assert torch.equal(out[0][0], out[1][0]) == few and torch.equal(out[0][2], out[1][2])
+    yr, hr, cr = oracle_prefill(oracle, inp, h0=inp["h0"].astype(np.float64), cs=inp["conv_state"].astype(np.float64))
+    assert_close("y", to_np(out[0][0]), yr, "f32"); assert_close("h_T", to_np(out[0][1]), hr, "f32")
+    assert np.array_equal(to_np(out[0][2]), cr)
+
+
+def test_host_prefill_whose_shares_cross_that_rule(oracle):
+    """The whole batch is beyond the rule, the shares that the call cuts it into are not: a workspace for the whole serves them all."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    B, T, Dh, H = 6, 100, 128, 8
+    inp = synth.make_inputs(B, T, Dh * H, H, io="f32", seed=7)
+    D, params = Dh * H, binding.Params.from_numpy(inp["params"], "f32")
+    y, hT, cs = [torch.empty(*s, pin_memory=True) for s in ((B, T, D), (B, D), (B, 3, D))]
+    shape = binding.make_shape(B, T, D, H, torch.float32)
+    staging = torch.empty(binding.host_staging_bytes(shape), dtype=torch.uint8, device="cuda")
+    binding.prefill_host(torch.from_numpy(inp["x"]).pin_memory(), params, y, hT, cs, staging, binding.alloc_workspace(shape, binding.OP_PREFILL, staging.device))
+    torch.cuda.synchronize()
+    yr, hr, cr = oracle_prefill(oracle, inp)
+    assert_close("y", to_np(y), yr, "f32"); assert_close("h_T", to_np(hT), hr, "f32")
+    assert np.array_equal(to_np(cs), cr)
