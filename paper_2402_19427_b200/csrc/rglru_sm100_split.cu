@@ -1058,12 +1058,39 @@ cudaError_t forward(SplitFwdArgs &p, int io, const void *wa, const void *wx, cud
     return wide ? launch_forward<__nv_bfloat16, SAVE, false, 64>(p, st) : launch_forward<__nv_bfloat16, SAVE, false, 32>(p, st);
 }
 
-// Token splits of dW: a split takes as long as a tile of du or less, at most 32 splits.  (One split beside the 640 tiles of du of B5 T1021
-// D1536 in 16 heads: 224 us.)
-int dw_split(size_t ntok, int &kb_split) {
+// Token splits of dW: at least four K blocks each, at most `most` splits.  Up to 8192 tokens a split takes as long as a tile of du of a
+// 128-wide head; with more tokens it is longer, since the parts are memory.  (One split beside the 640 tiles of du of B5 T1021 D1536 in
+// 16 heads: 224 us, where the products take 96 now.)
+int dw_split(size_t ntok, int most, int &kb_split) {
     const int total = ceil_div(ntok, 64);
-    kb_split = ceil_div(total, 32) > 4 ? ceil_div(total, 32) : 4;
+    kb_split = ceil_div(total, most) > 4 ? ceil_div(total, most) : 4;
     return ceil_div(total, kb_split);
+}
+
+// The workspace of the backward holds r, i and du in fp32 and the planes of u and of dz, 30 bytes an element, where the CUDA cores'
+// backward has 16.  So a call that would need more than 4 GiB goes through its sequences in two passes or three, one after the other in
+// the same arrays, as many as it takes to need no more than they do.  Passes cost 1 to 8 % (B8 T2048 D4096 in 16 heads 2194 -> 2245 us,
+// B2 T16384 in 32 heads 3469 -> 3734), which smaller calls need not pay.  (r and i in the place of dz, 22 bytes in one pass: reverse scan
+// 78 -> 88 us, forward 90 -> 96 on B5 T1021 D1536 in 16 heads.)
+struct BwdPlan {
+    int seqs;            // of a pass
+    int passes, splits;  // splits of dW over all passes
+    size_t conv_rows;    // rows of part_conv over all passes
+};
+constexpr size_t ONE_PASS_BYTES = (size_t)4 << 30;
+BwdPlan bwd_plan(int B, int T, int D) {
+    BwdPlan L{};
+    L.passes = 1;
+    if ((size_t)B * T * D * 30 > ONE_PASS_BYTES)
+        while (L.passes < B && ceil_div(B, L.passes) * 30 > B * 16) ++L.passes;
+    L.seqs = ceil_div(B, L.passes);
+    for (int b0 = 0; b0 < B; b0 += L.seqs) {
+        const int n = B - b0 < L.seqs ? B - b0 : L.seqs;
+        int kb;
+        L.splits += dw_split((size_t)n * T, 32 / L.passes, kb);
+        L.conv_rows += (size_t)n * conv_backward_chunks(n, T, D);
+    }
+    return L;
 }
 
 }  // namespace
@@ -1108,74 +1135,90 @@ cudaError_t split_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_t 
 }
 
 size_t split_backward_workspace_bytes(int B, int T, int D, int H, int io) {
-    const size_t ntok = (size_t)B * T, dh = D / H;
-    int kb;
-    const int S = dw_split(ntok, kb);
+    const BwdPlan L = bwd_plan(B, T, D);
+    const size_t ntok = (size_t)L.seqs * T, dh = D / H;
     size_t bytes = 3 * up256(ntok * D * 4);                                    // r, i, du
     bytes += up256(ntok * D * PLANES * 2) + up256(ntok * D * 2 * PLANES * 2);  // planes of u and dz
-    bytes += up256((size_t)B * ceil_div(T, SEG) * D * 4);
-    bytes += up256((size_t)B * ceil_div(T, REV_CHUNK) * 3 * D * 4) + up256((size_t)B * conv_backward_chunks(B, T, D) * 5 * D * 4);
-    bytes += up256((size_t)S * 2 * D * dh * 4) + 2 * up256((size_t)B * D * sizeof(uint4));
+    bytes += up256((size_t)L.seqs * ceil_div(T, SEG) * D * 4);
+    bytes += up256((size_t)B * ceil_div(T, REV_CHUNK) * 3 * D * 4) + up256(L.conv_rows * 5 * D * 4);
+    bytes += up256((size_t)L.splits * 2 * D * dh * 4) + 2 * up256((size_t)L.seqs * D * sizeof(uint4));
     return bytes + weight_plane_bytes(D, H, io);
 }
 
-cudaError_t split_backward(const FwdArgs &fwd, BwdArgs &q, int io, void *ws_body, cudaStream_t st) {
-    const int B = q.B, T = q.T, D = q.D, H = q.H, dh = D / H;
-    const size_t ntok = (size_t)B * T, wsz = (size_t)D * dh;
+cudaError_t split_backward(const FwdArgs &fwd, BwdArgs &q_all, int io, void *ws_body, cudaStream_t st) {
+    const int T = fwd.T, D = fwd.D, H = fwd.H, dh = D / H, rchunks = ceil_div(T, REV_CHUNK);
+    const BwdPlan L = bwd_plan(fwd.B, T, D);
+    const size_t most = (size_t)L.seqs * T, wsz = (size_t)D * dh, iob = io == RGLRU_F32 ? 4 : 2;
     char *at = (char *)ws_body;
     auto take = [&](size_t bytes) { char *r = at; at += up256(bytes); return r; };
-    q.r = (float *)take(ntok * D * 4); q.gi = (float *)take(ntok * D * 4); q.hp = (float *)take(ntok * D * 4);
-    char *u_planes = take(ntok * D * PLANES * 2), *dz = take(ntok * D * 2 * PLANES * 2);
-    float *h_seg = (float *)take((size_t)B * ceil_div(T, SEG) * D * 4);
-    const int rchunks = ceil_div(T, REV_CHUNK);
-    q.nchunk = conv_backward_chunks(B, T, D);
-    SplitProdArgs g{};
-    g.S = dw_split(ntok, g.kb_split);
-    q.S = g.S;
-    q.part_vec = (float *)take((size_t)B * rchunks * 3 * D * 4);
-    q.part_conv = (float *)take((size_t)B * q.nchunk * 5 * D * 4);
-    q.part_dw = (float *)take((size_t)g.S * 2 * wsz * 4);
-    uint4 *slots_f = (uint4 *)take((size_t)B * D * sizeof(uint4)), *slots_r = (uint4 *)take((size_t)B * D * sizeof(uint4));
+    float *rr = (float *)take(most * D * 4), *gi = (float *)take(most * D * 4), *du = (float *)take(most * D * 4);
+    char *u_planes = take(most * D * PLANES * 2), *dz = take(most * D * 2 * PLANES * 2);
+    float *h_seg = (float *)take((size_t)L.seqs * ceil_div(T, SEG) * D * 4);
+    q_all.part_vec = (float *)take((size_t)fwd.B * rchunks * 3 * D * 4);
+    q_all.part_conv = (float *)take(L.conv_rows * 5 * D * 4);
+    q_all.part_dw = (float *)take((size_t)L.splits * 2 * wsz * 4);
+    uint4 *slots_f = (uint4 *)take((size_t)L.seqs * D * sizeof(uint4)), *slots_r = (uint4 *)take((size_t)L.seqs * D * sizeof(uint4));
     char *planes = take(weight_plane_bytes(D, H, io));
     cudaError_t e;
     const void *wa, *wx;
     if ((e = weight_planes(fwd, io, planes, wa, wx, st)) != cudaSuccess) return e;
-    // forward sweep
-    SplitFwdArgs p{};
-    p.f = fwd;
-    p.f.save_r = q.r; p.f.save_i = q.gi;
-    p.f.gate_branch = nullptr;
-    p.u_planes = (uint32_t *)u_planes; p.h_seg = h_seg;
-    p.ch = make_chain(slots_f, fwd);
-    if ((e = forward<true>(p, io, wa, wx, st)) != cudaSuccess) return e;
-    // reverse scan and adjoints
-    SplitRevArgs r{};
-    r.q = q; r.conv_b = fwd.conv_b; r.h_seg = h_seg; r.dz = (uint32_t *)dz; r.ch = make_chain(slots_r, fwd);
-    r.nchunk = rchunks; r.ctiles = ceil_div(D, 64);
-    const size_t rgrid = (size_t)rchunks * B * r.ctiles;
-    if (rgrid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    if ((e = launch_dependent(io == RGLRU_F32 ? split_reverse_kernel<float> : split_reverse_kernel<__nv_bfloat16>, dim3((unsigned)rgrid), dim3(256), 0, st, r)) != cudaSuccess) return e;
-    // du += W^T dz, dW = dz^T u
     const uint64_t w3 = io == RGLRU_F32 ? PLANES : 1;
-    if (!plane_map(&g.tm_dzk, dz, dh, ntok, (uint64_t)2 * PLANES * H, 64, 128) || !plane_map(&g.tm_dzm, dz, dh, ntok, (uint64_t)2 * PLANES * H, 64, 64) ||
-        !plane_map(&g.tm_u, u_planes, dh, ntok, (uint64_t)PLANES * H, 64, 64) || !plane_map(&g.tm_wa, wa, dh, dh, w3 * H, 64, 64) || !plane_map(&g.tm_wx, wx, dh, dh, w3 * H, 64, 64))
-        return cudaErrorNotSupported;
-    g.H = H; g.dh = dh; g.D = D; g.wplanes = (int)w3; g.ntok = ntok;
-    g.nt = ceil_div(dh, 128); g.mt = g.nt; g.NT = ceil_div(ceil_div(dh, g.nt), 32) * 32;
-    g.du = q.hp; g.part = q.part_dw; g.status = fwd.status; g.spin_ns = g_spin_limit_ns;
-    const size_t dw = (size_t)g.S * 2 * H * g.mt * g.nt, tiles = dw + (size_t)ceil_div(ntok, 128) * H * g.nt;
-    if (tiles > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
-    g.dw_tiles = (int)dw; g.tiles = (int)tiles;
-    const int sms = num_sms();
-    static PerDeviceOptIn opt_in;
-    if ((e = opt_in.ensure(split_products_kernel, (int)PROD_ALLOC)) != cudaSuccess) return e;
-    if ((e = launch_dependent(split_products_kernel, dim3((unsigned)(tiles < (size_t)sms ? tiles : sms)), dim3(PROD_THREADS), PROD_ALLOC, st, g)) != cudaSuccess) return e;
-    if ((e = conv_backward(q, io, q.hp, false, st)) != cudaSuccess) return e;
-    if ((e = state_conv_grads(q, io, q.hp, false, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
+    size_t splits = 0, conv_rows = 0;   // of the passes so far
+    for (int b0 = 0; b0 < fwd.B; b0 += L.seqs) {
+        const int B = fwd.B - b0 < L.seqs ? fwd.B - b0 : L.seqs;
+        const size_t ntok = (size_t)B * T, x0 = (size_t)b0 * T * D * iob, c0 = (size_t)b0 * 3 * D * iob, h0 = (size_t)b0 * D;
+        auto from = [](const void *ptr, size_t bytes) -> const void * { return ptr ? (const char *)ptr + bytes : nullptr; };
+        // this pass's share of what has a batch dimension
+        FwdArgs f = fwd;
+        f.B = B; f.x = from(f.x, x0); f.cs_in = from(f.cs_in, c0); f.h0 = (const float *)from(f.h0, h0 * 4);
+        f.gate_branch = nullptr;
+        BwdArgs q = q_all;
+        q.B = B; q.x = f.x; q.cs_in = f.cs_in; q.dy = from(q.dy, x0); q.dx = (void *)from(q.dx, x0);
+        q.dh_T = (const float *)from(q.dh_T, h0 * 4); q.dcs_out = from(q.dcs_out, c0);
+        q.dh0 = (float *)from(q.dh0, h0 * 4); q.dcs_in = (void *)from(q.dcs_in, c0);
+        q.r = rr; q.gi = gi; q.hp = du;
+        q.nchunk = conv_backward_chunks(B, T, D);
+        q.part_vec += (size_t)b0 * rchunks * 3 * D;
+        q.part_conv += conv_rows * 5 * D;
+        q.part_dw += splits * 2 * wsz;
+        SplitProdArgs g{};
+        g.S = dw_split(ntok, 32 / L.passes, g.kb_split);
+        splits += g.S; conv_rows += (size_t)B * q.nchunk;
+        // forward sweep
+        SplitFwdArgs p{};
+        p.f = f;
+        p.f.save_r = q.r; p.f.save_i = q.gi;
+        p.u_planes = (uint32_t *)u_planes; p.h_seg = h_seg;
+        p.ch = make_chain(slots_f, f);
+        if ((e = forward<true>(p, io, wa, wx, st)) != cudaSuccess) return e;
+        // reverse scan and adjoints
+        SplitRevArgs r{};
+        r.q = q; r.conv_b = f.conv_b; r.h_seg = h_seg; r.dz = (uint32_t *)dz; r.ch = make_chain(slots_r, f);
+        r.nchunk = rchunks; r.ctiles = ceil_div(D, 64);
+        const size_t rgrid = (size_t)rchunks * B * r.ctiles;
+        if (rgrid > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+        if ((e = launch_dependent(io == RGLRU_F32 ? split_reverse_kernel<float> : split_reverse_kernel<__nv_bfloat16>, dim3((unsigned)rgrid), dim3(256), 0, st, r)) != cudaSuccess) return e;
+        // du += W^T dz, dW = dz^T u
+        if (!plane_map(&g.tm_dzk, dz, dh, ntok, (uint64_t)2 * PLANES * H, 64, 128) || !plane_map(&g.tm_dzm, dz, dh, ntok, (uint64_t)2 * PLANES * H, 64, 64) ||
+            !plane_map(&g.tm_u, u_planes, dh, ntok, (uint64_t)PLANES * H, 64, 64) || !plane_map(&g.tm_wa, wa, dh, dh, w3 * H, 64, 64) || !plane_map(&g.tm_wx, wx, dh, dh, w3 * H, 64, 64))
+            return cudaErrorNotSupported;
+        g.H = H; g.dh = dh; g.D = D; g.wplanes = (int)w3; g.ntok = ntok;
+        g.nt = ceil_div(dh, 128); g.mt = g.nt; g.NT = ceil_div(ceil_div(dh, g.nt), 32) * 32;
+        g.du = q.hp; g.part = q.part_dw; g.status = f.status; g.spin_ns = g_spin_limit_ns;
+        const size_t dw = (size_t)g.S * 2 * H * g.mt * g.nt, tiles = dw + (size_t)ceil_div(ntok, 128) * H * g.nt;
+        if (tiles > 0x7FFFFFFFull) return cudaErrorInvalidConfiguration;
+        g.dw_tiles = (int)dw; g.tiles = (int)tiles;
+        const int sms = num_sms();
+        static PerDeviceOptIn opt_in;
+        if ((e = opt_in.ensure(split_products_kernel, (int)PROD_ALLOC)) != cudaSuccess) return e;
+        if ((e = launch_dependent(split_products_kernel, dim3((unsigned)(tiles < (size_t)sms ? tiles : sms)), dim3(PROD_THREADS), PROD_ALLOC, st, g)) != cudaSuccess) return e;
+        if ((e = conv_backward(q, io, q.hp, false, st)) != cudaSuccess) return e;
+        if ((e = state_conv_grads(q, io, q.hp, false, st)) != cudaSuccess) return e;   // after dx: it rewrites the rows conv_state_out copies
+    }
     ReduceJobs jobs{};
-    add_reduce_job(jobs, q.part_dw, q.S, 2 * wsz, q.dW_a, wsz, q.dW_x, wsz, nullptr, 0);
-    add_reduce_job(jobs, q.part_vec, B * rchunks, (size_t)3 * D, q.dlambda, D, q.db_a, D, q.db_x, D);
-    add_reduce_job(jobs, q.part_conv, B * q.nchunk, (size_t)5 * D, q.dconv_w, (size_t)4 * D, q.dconv_b, D, nullptr, 0);
+    add_reduce_job(jobs, q_all.part_dw, (int)splits, 2 * wsz, q_all.dW_a, wsz, q_all.dW_x, wsz, nullptr, 0);
+    add_reduce_job(jobs, q_all.part_vec, fwd.B * rchunks, (size_t)3 * D, q_all.dlambda, D, q_all.db_a, D, q_all.db_x, D);
+    add_reduce_job(jobs, q_all.part_conv, (int)conv_rows, (size_t)5 * D, q_all.dconv_w, (size_t)4 * D, q_all.dconv_b, D, nullptr, 0);
     return run_reduce_jobs(jobs, st);
 }
 

@@ -56,6 +56,16 @@ def test_workspace_bytes_host_only(lib):
     assert b.workspace_bytes(S(1, 0, 256, 2, b.F32, 8.0, 0), b.OP_DECODE) >= 256        # T ignored for decode
 
 
+@pytest.mark.parametrize("B,T,D,H,io", [(2, 32768, 4096, 16, 0), (3, 16385, 4096, 32, 1), (5, 8203, 4096, 16, 0), (7, 8203, 2560, 16, 0), (64, 2048, 2048, 16, 0),
+                                         (8, 4096, 5632, 16, 1)])
+def test_workspace_of_a_large_backward_is_what_the_cuda_cores_need(lib, B, T, D, H, io):
+    """The split products' arrays take 30 bytes an element of a pass, the CUDA cores' 16: from 4 GiB on the call makes as many passes over
+    its sequences as it takes.  The parts of dW come on top (up to 32, where the CUDA cores have few for wide layers)."""
+    from paper_2402_19427_b200 import binding as b
+    size = [b.workspace_bytes(b.Shape(B, T, D, H, io, 8.0, flags), b.OP_BACKWARD) for flags in (0, b.FLAG_FORCE_GENERIC)]
+    assert size[0] <= 1.1 * size[1], size
+
+
 def test_argument_errors_are_return_codes(lib):
     from paper_2402_19427_b200 import binding as b
     good = 0x7F0000001000  # aligned, never dereferenced: validation fails first in every call below

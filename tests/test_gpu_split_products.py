@@ -167,3 +167,27 @@ def test_host_prefill_whose_shares_cross_that_rule(oracle):
     yr, hr, cr = oracle_prefill(oracle, inp)
     assert_close("y", to_np(y), yr, "f32"); assert_close("h_T", to_np(hT), hr, "f32")
     assert np.array_equal(to_np(cs), cr)
+
+
+def test_backward_in_passes_over_the_sequences():
+    """A call whose arrays would take more than 4 GiB goes through its sequences in passes, three of two sequences at most here.  What
+    belongs to a sequence is bit for bit what a call of its pass alone gives, what is summed over them is the sum (in another order: 2^-22)."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    B, T, D, H = 5, 8203, 4096, 32
+    assert binding.workspace_bytes(binding.make_shape(B, T, D, H, torch.bfloat16), binding.OP_BACKWARD) < 20 * B * T * D
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    params = binding.Params.from_numpy(synth.make_inputs(1, 1, D, H, io="bf16", seed=6, bias_scale=0.2)["params"], "bf16")
+    f32 = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    bf16 = lambda *s: f32(*s).to(torch.bfloat16)
+    x, dy, h0, cs, dhT, dcs = bf16(B, T, D), bf16(B, T, D), f32(B, D), bf16(B, 3, D), f32(B, D), bf16(B, 3, D)
+    call = lambda s: binding.backward(x[s], params, dy[s], h0=h0[s], conv_state_in=cs[s], dh_T=dhT[s], dconv_state_out=dcs[s], state_grads=True)
+    whole, parts = call(slice(0, 5)), [call(slice(0, 2)), call(slice(2, 4)), call(slice(4, 5))]
+    torch.cuda.synchronize()
+    for k, v in whole.items():
+        if k in ("x", "h0", "conv_state"):
+            assert torch.equal(v, torch.cat([g[k] for g in parts])), k
+        else:
+            want = sum(g[k].double() for g in parts)
+            assert float((v.double() - want).norm() / want.norm()) < 2.0 ** -22, k
