@@ -1,5 +1,5 @@
 """GPU parity of the optional extras of the forward (rglru_prefill_ex) against the fp64 oracle, on the CUDA-core kernels
-(fp32 and bf16, any head width) and on the tensor-core kernel (bf16, head width 256): the merged output of the recurrent
+(fp32 and bf16, any head width), the split products and the fused tensor-core kernel (bf16): the merged output of the recurrent
 block, y_t = h_t * GeLU(branch_t) (Section 2.3), and the decay product of the call, prod_t a_t, which together with h_T from
 a zero state describes the call as one affine step of Eq. 4."""
 import numpy as np
@@ -46,9 +46,11 @@ def check_product(got, ref, io):
     assert np.all(got[~big] < 1e-25)
 
 
+@pytest.mark.parametrize("flags", [0, 1])   # 1: RGLRU_FLAG_FORCE_GENERIC
 @pytest.mark.parametrize("io,B,T,D,H", [("f32", 2, 37, 64, 2), ("f32", 1, 130, 96, 3), ("bf16", 2, 70, 128, 4)])
-def test_extras_on_the_cuda_core_kernels(oracle, io, B, T, D, H):
-    got, ref, _, _ = run_both(oracle, B, T, D, H, io, seed=600 + T)
+def test_extras_of_narrow_heads(oracle, io, B, T, D, H, flags):
+    """The CUDA-core kernel, and what takes the call otherwise: the same (few fp32 tokens), split products, the fused prefill."""
+    got, ref, _, _ = run_both(oracle, B, T, D, H, io, seed=600 + T, flags=flags)
     check_product(got, ref, io)
 
 

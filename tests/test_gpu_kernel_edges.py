@@ -48,7 +48,7 @@ def test_cuda_core_blocks_and_chunk_chain(oracle, B, T, D, H, io):
 
 @pytest.mark.parametrize("B,T,Dh,H", [
     (2, 1, 256, 1), (1, 63, 256, 1), (2, 65, 128, 3), (1, 127, 96, 3),   # one chunk, tails, a partial last group of heads
-    (1, 1203, 160, 2),    # a column shared by many blocks (look-back over their steps), channels beyond the last 64
+    (1, 1203, 160, 2),    # a long chain of chunks, channels beyond the last 128
     (3, 1030, 64, 5),
 ])
 def test_tensor_core_backward_of_ragged_sequences(oracle, B, T, Dh, H):
@@ -56,9 +56,9 @@ def test_tensor_core_backward_of_ragged_sequences(oracle, B, T, Dh, H):
 
 
 @pytest.mark.parametrize("B,T,Dh,H", [
-    (2, 77, 352, 2), (3, 1, 288, 1), (1, 64, 320, 3), (1, 200, 1024, 1),   # 2 x 192, 2 x 160 and 4 x 256 column tiles
-    (1, 515, 544, 1),      # 3 x 192; a column shared by several blocks
-    (2, 8300, 288, 1),     # more tokens than one pass of the wide forward: state carried from pass to pass
+    (2, 77, 352, 2), (3, 1, 288, 1), (1, 64, 320, 3), (1, 200, 1024, 1),   # 3 and 8 channel tiles of a head, the last one part empty
+    (1, 515, 544, 1),      # 5 tiles; nine K blocks, the last a half one
+    (2, 8300, 288, 1),     # 130 chunks in a chain
 ])
 def test_tensor_core_kernels_of_heads_wider_than_256(oracle, B, T, Dh, H):
     forward_and_backward(oracle, B, T, Dh * H, H, "bf16", 0, seed=300 + T)
@@ -102,7 +102,7 @@ def test_replayed_graph_of_chained_chunks(oracle):
     taken for those of the second, which works on other inputs."""
     import torch
     from paper_2402_19427_b200 import binding
-    for io, Dh, flags in (("f32", 64, GENERIC), ("bf16", 288, 0)):
+    for io, Dh, flags in (("f32", 64, GENERIC), ("bf16", 288, 0), ("f32", 96, 0), ("f32", 672, 0)):
         B, T, H = 1, 700, 1
         first, second = [synth.make_inputs(B, T, Dh * H, H, io=io, seed=60 + k, with_dy=True) for k in range(2)]
         params = binding.Params.from_numpy(first["params"], io)

@@ -240,8 +240,9 @@ def test_other_python_threads_run_while_a_launch_blocks():
 
 @pytest.mark.parametrize("B,T,Dh,H,io,flags,backward", [
     (1, 700, 64, 2, "f32", 1, False), (1, 700, 64, 2, "f32", 1, True),          # chunk chains of the CUDA-core kernels
-    (1, 2000, 288, 1, "bf16", 0, False),                                        # blocks that share a column of the wide forward
-    (1, 2000, 256, 1, "bf16", 0, True), (1, 2000, 256, 1, "bf16", 0, "saved"),  # ... of the reverse scan; the forward in front of it
+    (1, 2000, 288, 1, "bf16", 0, False), (1, 700, 64, 2, "f32", 0, False), (4, 1300, 64, 4, "f32", 0, False), (1, 200, 1024, 1, "f32", 0, False),   # split forwards
+    (1, 700, 64, 2, "f32", 0, True), (4, 1300, 64, 4, "f32", 0, True), (1, 701, 96, 2, "bf16", 0, True), (1, 300, 288, 2, "bf16", 0, "saved"),     # and backwards
+    (1, 2000, 256, 1, "bf16", 0, True), (1, 2000, 256, 1, "bf16", 0, "saved"),  # blocks that share a column of the 16-bit reverse scan; the forward in front of it
 ])
 def test_every_wait_for_a_carry_is_bounded(oracle, B, T, Dh, H, io, flags, backward):
     """As above for the other kernels that hand carries from block to block: the wait runs out, the status says so, once, and the next
@@ -274,8 +275,9 @@ def test_every_wait_for_a_carry_is_bounded(oracle, B, T, Dh, H, io, flags, backw
     assert_close("out", to_np(out), ref, io, scale=max(1.0, float(np.abs(ref).max())) if io == "f32" else 1.0)
 
 
-def test_a_failed_link_ends_the_chain_at_once():
-    """4000 chunks in a chain, of which the GPU holds less than a quarter at a time: a link that gives up tells the next, so the call ends
+@pytest.mark.parametrize("flags", [0, 1])   # split products, CUDA cores
+def test_a_failed_link_ends_the_chain_at_once(flags):
+    """2000 chunks in a chain, of which the GPU holds less than a quarter at a time: a link that gives up tells the next, so the call ends
     after one wait limit and not after one per wave of blocks."""
     import time
     import torch
@@ -284,15 +286,15 @@ def test_a_failed_link_ends_the_chain_at_once():
     inp = synth.make_inputs(1, 1, D, 1, io="f32", seed=15)
     params = binding.Params.from_numpy(inp["params"], "f32")
     x = torch.zeros(1, T, D, device="cuda")
-    ws = binding.alloc_workspace(binding.make_shape(1, T, D, 1, torch.float32), binding.OP_PREFILL, x.device)
+    ws = binding.alloc_workspace(binding.make_shape(1, T, D, 1, torch.float32, flags=flags), binding.OP_PREFILL, x.device)
     y = torch.empty_like(x)
-    binding.prefill(x, params, y=y, workspace=ws)
+    binding.prefill(x, params, y=y, workspace=ws, flags=flags)
     torch.cuda.synchronize()
     limit = 0.1
     prev = binding.set_wait_limit_ns(int(limit * 1e9))
     try:
         t = time.perf_counter()
-        binding.prefill(x, params, y=y, workspace=ws, flags=binding.FLAG_TEST_CARRY_NEVER_ARRIVES)
+        binding.prefill(x, params, y=y, workspace=ws, flags=flags | binding.FLAG_TEST_CARRY_NEVER_ARRIVES)
         torch.cuda.synchronize()
         t = time.perf_counter() - t
         assert binding.query_status(ws) == binding.ERR_TIMEOUT
@@ -303,7 +305,8 @@ def test_a_failed_link_ends_the_chain_at_once():
 
 @pytest.mark.parametrize("B,T,Dh,H,io,merge", [
     (2, 70, 96, 3, "bf16", False), (1, 130, 160, 3, "bf16", True), (3, 33, 32, 9, "bf16", False),   # partial last groups, unused channel slots
-    (2, 71, 288, 2, "bf16", True), (1, 4100, 288, 1, "bf16", False),                                # heads wider than 256; more than one pass
+    (2, 71, 288, 2, "bf16", True), (1, 4100, 288, 1, "bf16", False),                                # split products: heads wider than 256,
+    (2, 150, 96, 3, "f32", True), (3, 705, 64, 7, "f32", False), (1, 131, 672, 1, "f32", True),     # fp32, blocks of 32 and 64 tokens, three sets of accumulators
     (2, 67, 34, 3, "bf16", False), (1, 97, 66, 2, "f32", True),                                     # CUDA-core kernels, odd widths
 ])
 def test_prefill_of_other_widths_writes_only_its_outputs(oracle, B, T, Dh, H, io, merge):
@@ -329,6 +332,7 @@ def test_prefill_of_other_widths_writes_only_its_outputs(oracle, B, T, Dh, H, io
 @pytest.mark.parametrize("B,T,Dh,H,io,saved", [
     (2, 72, 96, 3, "bf16", True), (1, 136, 160, 3, "bf16", False), (3, 40, 32, 9, "bf16", True),   # tensor cores: partial groups, tails of a chunk
     (2, 71, 96, 3, "bf16", True), (1, 64, 288, 2, "bf16", False), (2, 67, 34, 3, "f32", False),    # ragged, wide, odd widths
+    (2, 67, 96, 3, "f32", True), (3, 705, 64, 7, "f32", False), (1, 131, 672, 1, "f32", False),    # fp32
 ])
 def test_backward_of_other_shapes_writes_only_its_outputs(B, T, Dh, H, io, saved):
     import torch
