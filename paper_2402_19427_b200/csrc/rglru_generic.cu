@@ -795,8 +795,6 @@ cudaError_t set_smem(K kernel, size_t bytes) {
     return cudaSuccess;
 }
 
-size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }
-inline int ceil_div(size_t a, size_t b) { return (int)((a + b - 1) / b); }
 
 // Rows per block of a contraction with `blocks64` blocks of 64 rows x 128 columns: three of those fit an SM, and below two per
 // SM the machine is better filled by four times as many blocks of 32 x 64 (B1 T256 D256 in two heads: 8 -> 64 blocks).  Counted for
@@ -816,7 +814,7 @@ int dw_splits(size_t ntok, int H, int Dh) {
 }  // namespace
 
 size_t generic_prefill_workspace_bytes(int B, int D, int io) {
-    return align256((size_t)B * D * sizeof(uint4)) + align256((size_t)B * 3 * D * (io == RGLRU_F32 ? 4 : 2));
+    return up256((size_t)B * D * sizeof(uint4)) + up256((size_t)B * 3 * D * (io == RGLRU_F32 ? 4 : 2));
 }
 
 namespace {
@@ -858,7 +856,7 @@ cudaError_t generic_prefill(const FwdArgs &a, int io, void *ws_body, cudaStream_
     const size_t cs_bytes = (size_t)a.B * 3 * a.D * (io == RGLRU_F32 ? 4 : 2);
     const uintptr_t ci = (uintptr_t)a.cs_in, co = (uintptr_t)a.cs_out;
     if (ci && ci < co + cs_bytes && co < ci + cs_bytes) {
-        void *copy = (char *)ws_body + align256((size_t)a.B * a.D * sizeof(uint4));
+        void *copy = (char *)ws_body + up256((size_t)a.B * a.D * sizeof(uint4));
         cudaError_t e = cudaMemcpyAsync(copy, a.cs_in, cs_bytes, cudaMemcpyDeviceToDevice, st);
         if (e != cudaSuccess) return e;
         f.cs_in = copy;
@@ -905,11 +903,11 @@ cudaError_t run_reduce_jobs(const ReduceJobs &jobs, cudaStream_t st) {
 
 size_t generic_backward_workspace_bytes(int B, int T, int D, int H) {
     const size_t btd = (size_t)B * T * D, Dh = D / H;
-    size_t bytes = 4 * align256(btd * sizeof(float));
-    bytes += align256((size_t)B * ceil_div(T, RCHUNK) * 3 * D * sizeof(float));
-    bytes += align256((size_t)B * ceil_div(T, GENERIC_BWD_CHUNK) * 5 * D * sizeof(float));
-    bytes += align256((size_t)dw_splits((size_t)B * T, H, (int)Dh) * 2 * H * Dh * Dh * sizeof(float));
-    bytes += 2 * align256((size_t)B * D * sizeof(uint4));
+    size_t bytes = 4 * up256(btd * sizeof(float));
+    bytes += up256((size_t)B * ceil_div(T, RCHUNK) * 3 * D * sizeof(float));
+    bytes += up256((size_t)B * ceil_div(T, GENERIC_BWD_CHUNK) * 5 * D * sizeof(float));
+    bytes += up256((size_t)dw_splits((size_t)B * T, H, (int)Dh) * 2 * H * Dh * Dh * sizeof(float));
+    bytes += 2 * up256((size_t)B * D * sizeof(uint4));
     return bytes;
 }
 
@@ -917,7 +915,7 @@ cudaError_t generic_backward(const FwdArgs &fwd_in, BwdArgs &q, int io, void *ws
     const int B = q.B, T = q.T, D = q.D, H = q.H, Dh = D / H;
     const size_t btd = (size_t)B * T * D, wsz = (size_t)H * Dh * Dh;
     char *p = (char *)ws_body;
-    auto take = [&](size_t bytes) { char *at = p; p += align256(bytes); return at; };
+    auto take = [&](size_t bytes) { char *at = p; p += up256(bytes); return at; };
     q.u = (float *)take(btd * sizeof(float));
     q.r = (float *)take(btd * sizeof(float));
     q.gi = (float *)take(btd * sizeof(float));

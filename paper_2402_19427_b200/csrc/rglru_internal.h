@@ -51,6 +51,14 @@ cudaError_t launch_dependent(void (*kernel)(P...), dim3 grid, dim3 block, size_t
     return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
 }
 
+inline size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
+inline int ceil_div(size_t a, size_t b) { return (int)((a + b - 1) / b); }
+inline int num_sms() {
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) return n;
+    return 148;
+}
+
 // A call's return code.  The error goes out in the code and is not left behind in the thread's runtime state, where a later call
 // (this library's or a caller's that links the same runtime) would take it for its own.
 inline int32_t call_status(cudaError_t e) {

@@ -872,7 +872,6 @@ bool sm100_prefill_supported(int B, int T, int D, int H, int io) {
 }
 
 namespace {
-inline size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 // Pairs that share a head's time axis: as many as fit beside the other heads, at most MAX_S.  The host-only workspace
 // size has to agree with the launch, so both count with at most MAX_PAIRS pairs whatever the device reports.
 constexpr int MAX_PAIRS = 74;

@@ -54,7 +54,7 @@ struct GemmArgs {
     alignas(64) CUtensorMap tm_b0;   // B rows (N side), K innermost
     alignas(64) CUtensorMap tm_b1;   // MODE_Z: the second gate's weights (grid.y selects)
     int mode, H, D;    // H: groups of heads
-    int NS, NT, nt;    // channel slots of a group; they are nt column tiles of NT
+    int NS, NT;        // channel slots of a group = columns of a tile
     int hstride;       // channels of a group that exist (fewer in a partial last group) = channels from one group to the next in [.., D] arrays
     int nx, ny;        // tile grid: nx x ny x H
     int kblocks;       // MODE_DW: 64-token K blocks of a split.  MODE_Z / MODE_DU: K runs over the existing 64-slot blocks of the group
@@ -68,18 +68,9 @@ struct GemmArgs {
 // layout, accumulate in tensor memory (fp32), and leave through the eight epilogue warps.  CTAs are persistent: each
 // walks tiles blockIdx.x, blockIdx.x + gridDim.x, ... with two accumulators, so that the epilogue of one tile overlaps
 // the loads and MMAs of the next.  Tile number -> (x, y, z) with x fastest:
-//   MODE_Z : (token tiles, 2 gates x nt, H)   A = u[tok][h][k]        B = W_gate[h][out][k]
-//   MODE_DU: (token tiles, nt, H)             A = dz[tok][h][k=2 NS]  B = W[gate][h][k=out][in], MN-major
-//   MODE_DW: (2 NS / 128, splits x nt, H)     A = dz[tok][h][row]     B = u[tok][h][in], both MN-major, K = this split's tokens
-// 32-byte accesses: one whole DRAM sector per thread and instruction where a thread owns a row (pointers 32-byte aligned)
-__device__ __forceinline__ void st_global_v8(void *ptr, const uint32_t (&r)[8]) {
-    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(ptr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]),
-                 "r"(r[6]), "r"(r[7]) : "memory");
-}
-__device__ __forceinline__ void ld_global_v8(const void *ptr, uint32_t (&r)[8]) {
-    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                 "=r"(r[6]), "=r"(r[7]) : "l"(ptr) : "memory");
-}
+//   MODE_Z : (token tiles, 2 gates, H)        A = u[tok][h][k]        B = W_gate[h][out][k]
+//   MODE_DU: (token tiles, 1, H)              A = dz[tok][h][k=2 NS]  B = W[gate][h][k=out][in], MN-major
+//   MODE_DW: (2 NS / 128, splits, H)          A = dz[tok][h][row]     B = u[tok][h][in], both MN-major, K = this split's tokens
 
 // 64-slot blocks of group h that hold channels, and the number of K blocks of a tile of that group
 __device__ __forceinline__ int slot_blocks(const GemmArgs &p, int h) { return (min(p.hstride, p.D - h * p.hstride) + 63) / 64; }
@@ -125,8 +116,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
             const int ncopies = (p.NT + 63) / 64;   // 64-channel copies of an MN-major B operand
             const uint32_t tx_bytes = A_STAGE_BYTES + (p.mode != MODE_Z ? (uint32_t)ncopies * MN_BLOCK_BYTES : (uint32_t)p.NT * 128u);
             for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x) {
-                const int tx = tile % p.nx, ty = (tile / p.nx) % p.ny, h = tile / (p.nx * p.ny);
-                const int col0 = (ty % p.nt) * p.NT, sel = ty / p.nt;   // sel: gate (MODE_Z), split (MODE_DW)
+                const int tx = tile % p.nx, sel = (tile / p.nx) % p.ny, h = tile / (p.nx * p.ny);   // sel: gate (MODE_Z), split (MODE_DW)
                 const CUtensorMap *tb = (p.mode == MODE_Z && sel == 1) ? &p.tm_b1 : &p.tm_b0;
                 const int kslots = slot_blocks(p, h), kblocks = tile_kblocks(p, h);
                 for (int kb = 0; kb < kblocks; ++kb, ++kbg) {
@@ -141,18 +131,18 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                         const int k0 = (sel * p.kblocks + kb) * 64;
 #pragma unroll
                         for (int j = 0; j < 2; ++j) tma_load_3d(a_dst + j * MN_BLOCK_BYTES, &p.tm_a, tx * 128 + j * 64, h, k0, BAR_FULL(s));
-                        for (int j = 0; j < ncopies; ++j) tma_load_3d(b_dst + j * MN_BLOCK_BYTES, tb, h * p.hstride + col0 + j * 64, k0, 0, BAR_FULL(s));
+                        for (int j = 0; j < ncopies; ++j) tma_load_3d(b_dst + j * MN_BLOCK_BYTES, tb, h * p.hstride + j * 64, k0, 0, BAR_FULL(s));
                     } else {
                         // u is read out of the layer's [tok][D] array at the group's first channel (channels past the group's own
                         // meet zero weights; past D they read as zero); dz has the groups' own [tok][group][2][NS] layout
                         const int kc = kb < kslots ? kb * 64 : p.NS + (kb - kslots) * 64;   // MODE_DU: the second gate's slots follow the first's
                         if (p.mode == MODE_Z) {
                             tma_load_3d(a_dst, &p.tm_a, h * p.hstride + kb * 64, tx * 128, 0, BAR_FULL(s));
-                            tma_load_3d(b_dst, tb, kb * 64, col0, h, BAR_FULL(s));
+                            tma_load_3d(b_dst, tb, kb * 64, 0, h, BAR_FULL(s));
                         } else {
                             tma_load_3d(a_dst, &p.tm_a, kc, h, tx * 128, BAR_FULL(s));
                             const int gate = kb >= kslots, o0 = (kb - gate * kslots) * 64;
-                            for (int j = 0; j < ncopies; ++j) tma_load_3d(b_dst + j * MN_BLOCK_BYTES, tb, col0 + j * 64, o0, gate * p.H + h, BAR_FULL(s));
+                            for (int j = 0; j < ncopies; ++j) tma_load_3d(b_dst + j * MN_BLOCK_BYTES, tb, j * 64, o0, gate * p.H + h, BAR_FULL(s));
                         }
                     }
                 }
@@ -203,8 +193,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
         const int q = warp & 3, half = (warp - 2) >> 2;
         int it = 0;
         for (int tile = blockIdx.x; tile < ntiles && ok; tile += gridDim.x, ++it) {
-            const int tx = tile % p.nx, ty = (tile / p.nx) % p.ny, h = tile / (p.nx * p.ny);
-            const int col0 = (ty % p.nt) * p.NT, sel = ty / p.nt;
+            const int tx = tile % p.nx, sel = (tile / p.nx) % p.ny, h = tile / (p.nx * p.ny);
             const int acc = it & 1;
             const int row = tx * 128 + q * 32 + lane;
             const bool valid = row < p.rows_valid;
@@ -213,12 +202,12 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
             auto wait_acc = [&]() { ok = warp_wait(BAR_ACCFULL(acc), (it >> 1) & 1, spin, abort_flag); tc_fence_after(); };
             if (p.mode == MODE_DU) {
                 // du is kept in fp16 like dz (bf16 failed the dx tolerance where the taps of the Conv1D adjoint cancel)
-                __half *dst0 = (__half *)p.out + (size_t)row * p.D + h * p.hstride + col0;
+                __half *dst0 = (__half *)p.out + (size_t)row * p.D + h * p.hstride;
                 uint32_t o[4][2][8];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int c0 = j * 64 + half * 32;
-                    if (valid && c0 < p.NT && col0 + c0 < cv) {   // a slot that does not exist: nothing of du belongs to it
+                    if (valid && c0 < p.NT && c0 < cv) {   // a slot that does not exist: nothing of du belongs to it
                         ld_global_v8(dst0 + c0, o[j][0]);
                         ld_global_v8(dst0 + c0 + 16, o[j][1]);
                     }
@@ -232,7 +221,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                         f32x2 v[16];
                         tmem_ld32(tm_lane + c0, v);
                         tmem_ld_wait();
-                        if (valid && col0 + c0 < cv) {
+                        if (valid && c0 < cv) {
 #pragma unroll
                             for (int e = 0; e < 8; ++e) {
                                 const float2 a0 = __half22float2(*(const __half2 *)&o[j][0][e]), a1 = __half22float2(*(const __half2 *)&o[j][1][e]);
@@ -254,7 +243,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                     tmem_ld_wait();
                     if (!valid) continue;
                     if (p.mode == MODE_Z) {
-                        __half *dst = (__half *)p.out + (((size_t)row * p.H + h) * 2 + sel) * p.NS + col0 + c0;
+                        __half *dst = (__half *)p.out + (((size_t)row * p.H + h) * 2 + sel) * p.NS + c0;
 #pragma unroll
                         for (int j8 = 0; j8 < 2; ++j8) {
                             uint32_t w[8];
@@ -264,7 +253,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) tc_gemm_kernel(const __grid_c
                         }
                     } else {
                         const int g = row >= p.NS, o_row = row - g * p.NS;
-                        float *dst = (float *)p.out + ((((size_t)sel * 2 + g) * p.H + h) * p.NS + o_row) * p.NS + col0 + c0;
+                        float *dst = (float *)p.out + ((((size_t)sel * 2 + g) * p.H + h) * p.NS + o_row) * p.NS + c0;
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
                             uint32_t w[8];
@@ -371,9 +360,7 @@ __global__ void reduce_dw_blocks_kernel(const float *part, int S, int G, int NS,
     (gate ? dWx : dWa)[i % per_gate] = acc;
 }
 
-__device__ __forceinline__ f32x2 bf2x(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
 __device__ __forceinline__ f32x2 hf2x(uint32_t w) { return __half22float2(*(const __half2 *)&w); }
-__device__ __forceinline__ f32x2 ld2f(const float *p) { return *(const float2 *)p; }
 
 // four adjacent channels
 struct f32x4 { f32x2 a, b; };
@@ -394,10 +381,6 @@ struct ConvArgs {
     __half *u;
     uint32_t *epoch;
 };
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *(const uint32_t *)&v;
-}
 __global__ void __launch_bounds__(256, 4) conv_forward_kernel(ConvArgs a) {
     dependency_wait();
     const int d = blockIdx.x * CONV_CH + (threadIdx.x & 63) * 4, b = blockIdx.z;
@@ -818,13 +801,7 @@ template <typename IOT, typename DUT, int LEN> __global__ void __launch_bounds__
     }
 }
 
-inline size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
 
-int num_sms() {
-    int dev = 0, nsm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 148;
-    return nsm;
-}
 unsigned gemm_grid(const GemmArgs &g) {
     const int nsm = num_sms();
     const int ntiles = g.nx * g.ny * g.H;
@@ -832,9 +809,9 @@ unsigned gemm_grid(const GemmArgs &g) {
 }
 
 // Groups of heads, the unit of the GEMMs and of the z / dz arrays: k = 256 / width (rounded down) consecutive heads in
-// NS channel slots, their channels rounded up to K blocks of 64: one column tile (nt = 1, NT = NS).
+// NS channel slots, their channels rounded up to K blocks of 64: one column tile (NT = NS).
 struct Groups {
-    int dh, k, G, hstride, NS, NT, nt;
+    int dh, k, G, hstride, NS, NT;
     size_t W16_bytes() const { return (size_t)2 * G * NS * NS * 2; }
 };
 Groups make_groups(int D, int H) {
@@ -843,7 +820,6 @@ Groups make_groups(int D, int H) {
     g.k = DH / g.dh;
     g.G = (H + g.k - 1) / g.k;
     g.hstride = g.k * g.dh;
-    g.nt = 1;
     g.NT = g.NS = (g.hstride + 63) / 64 * 64;
     return g;
 }
@@ -859,7 +835,7 @@ struct BwdLayout {
 // workspace size has to agree with the launch): 2 splits for 16 heads of 256 (64 tiles a split; eight of them took four rounds
 // and 67 MB of partial sums, dW and its reduction 110 us on B4 T4096).
 int dw_split(const Groups &gr, int kblocks) {
-    const int tiles = gr.G * gr.nt * (2 * gr.NS / 128), most = kblocks < 16 ? kblocks : 16;
+    const int tiles = gr.G * (2 * gr.NS / 128), most = kblocks < 16 ? kblocks : 16;
     const double part_us = 2.0 * 2 * gr.G * gr.NS * gr.NS * 4 / 5e6;
     int best = 1;
     double best_us = 1e30;
@@ -902,7 +878,7 @@ BwdLayout bwd_layout(int B, int T, int D, int Hl) {
 
 GemmArgs gemm_args(const Groups &gr, int D, uint32_t *status) {
     GemmArgs g{};
-    g.H = gr.G; g.D = D; g.NS = gr.NS; g.NT = gr.NT; g.nt = gr.nt; g.hstride = gr.hstride; g.status = status; g.spin_ns = g_spin_limit_ns;
+    g.H = gr.G; g.D = D; g.NS = gr.NS; g.NT = gr.NT; g.hstride = gr.hstride; g.status = status; g.spin_ns = g_spin_limit_ns;
     return g;
 }
 cudaError_t run_gemm(const GemmArgs &g, cudaStream_t st) {
@@ -927,7 +903,7 @@ cudaError_t gemm_z(const Groups &gr, int D, size_t ntok, const __half *u, const 
         !encode_map16_3d(&g.tm_b1, W16 + (size_t)gr.G * NS * NS, db, sb, bb, true))
         return cudaErrorNotSupported;
     g.mode = MODE_Z; g.rows_valid = (int)ntok; g.out = z;
-    g.nx = (int)((ntok + 127) / 128); g.ny = 2 * gr.nt;
+    g.nx = (int)((ntok + 127) / 128); g.ny = 2;
     return run_gemm(g, st);
 }
 
@@ -1044,7 +1020,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
         if (!encode_map16_3d(&g.tm_a, dz, ddz, sdz, ba, true) || !encode_map16_3d(&g.tm_b0, W16, db, sb, bb, true)) return cudaErrorNotSupported;
         g.tm_b1 = g.tm_b0;
         g.mode = MODE_DU; g.rows_valid = (int)BT; g.out = du;
-        g.nx = (int)mtiles; g.ny = gr.nt;
+        g.nx = (int)mtiles; g.ny = 1;
         if ((e = run_gemm(g, st)) != cudaSuccess) return e;
     }
     // 5. dW = dz^T u, split over the tokens, then a fixed-order sum of the splits
@@ -1056,7 +1032,7 @@ cudaError_t sm100_backward(const FwdArgs &fwd, BwdArgs &q, const void *y_saved, 
         g.tm_b1 = g.tm_b0;
         float *part = (float *)(ws + L.off_pdw);
         g.mode = MODE_DW; g.kblocks = L.kb_per_split; g.rows_valid = 2 * NS; g.out = part;
-        g.nx = 2 * NS / 128; g.ny = L.S * gr.nt;
+        g.nx = 2 * NS / 128; g.ny = L.S;
         if ((e = run_gemm(g, st)) != cudaSuccess) return e;
         const size_t wsz = (size_t)H * NS * NS;
         if (gr.dh == NS) {   // one head per group and every slot exists: the partial sums already have the layout of dW

@@ -62,10 +62,6 @@ struct DecArgs {
 
 __device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
 __device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-    return *(const uint32_t *)&v;
-}
 
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1) sm100_decode_kernel(const __grid_constant__ DecArgs p) {
     extern __shared__ uint8_t smem_raw[];
@@ -541,11 +537,6 @@ cudaError_t decode_few(const FwdArgs &a, int C, int NB, cudaStream_t st) {
     return NB == 8 ? cudaLaunchKernelEx(&cfg, sm100_decode_few_kernel<8>, a, dh, C) : cudaLaunchKernelEx(&cfg, sm100_decode_few_kernel<16>, a, dh, C);
 }
 
-int num_sms() {
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess && cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && n > 0) return n;
-    return 148;
-}
 
 }  // namespace
 

@@ -36,13 +36,7 @@ constexpr int FWD_THREADS = 320;              // eight warps of Conv1D and epilo
 constexpr uint32_t TILE_BYTES = 128 * 128;    // 128 rows (or 2 x 64 columns) of 64 bf16: one operand tile of a K block of 64
 constexpr int PROD_STAGES = 2, PROD_THREADS = 352;   // K blocks in flight; eight epilogue warps, one of products, two of copies
 
-__device__ __forceinline__ f32x2 bf2x(uint32_t w) { return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); }
 __device__ __forceinline__ uint32_t tops(f32x2 v) { return __byte_perm(__float_as_uint(v.x), __float_as_uint(v.y), 0x7632); }   // the upper halves, v.x's below
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-    uint32_t r;
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-    return r;
-}
 __device__ __forceinline__ float bound_bf16(float v) {   // the largest finite bf16 value, with v's sign, for what would round up to infinity; a NaN stays one
     float y;
     asm("min.NaN.xorsign.abs.f32 %0, %1, %2;" : "=f"(y) : "f"(v), "f"(3.38953139e38f));
@@ -58,21 +52,12 @@ __device__ __forceinline__ void split_planes(f32x2 v, uint32_t (&w)[PLANES]) {
     v = fma2(bf2x(w[1]), pack2(-1.0f, -1.0f), v);
     w[2] = tops(v);
 }
-__device__ __forceinline__ f32x2 ld2f(const float *p) { return *(const float2 *)p; }
-__device__ __forceinline__ f32x2 ld2(const float *p) { return *(const float2 *)p; }
+__device__ __forceinline__ f32x2 ld2(const float *p) { return ld2f(p); }
 __device__ __forceinline__ f32x2 ld2(const __nv_bfloat16 *p) { return bf2x(*(const uint32_t *)p); }
 __device__ __forceinline__ float ld1(const float *p) { return *p; }
 __device__ __forceinline__ float ld1(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
 __device__ __forceinline__ void st1(float *p, float v) { *p = v; }
 __device__ __forceinline__ void st1(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
-__device__ __forceinline__ void st_global_v8(void *ptr, const uint32_t (&r)[8]) {
-    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(ptr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]),
-                 "r"(r[6]), "r"(r[7]) : "memory");
-}
-__device__ __forceinline__ void ld_global_v8(const void *ptr, uint32_t (&r)[8]) {
-    asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];" : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
-                 "=r"(r[6]), "=r"(r[7]) : "l"(ptr) : "memory");
-}
 
 // ------------------------------------------------------------------ weights as planes (fp32 io)
 // out[gate][plane][n], two values a thread
@@ -993,13 +978,6 @@ __global__ void __launch_bounds__(PROD_THREADS, 1) split_products_kernel(const _
 }
 
 // ------------------------------------------------------------------ host side
-inline size_t up256(size_t v) { return (v + 255) & ~(size_t)255; }
-inline int ceil_div(size_t a, size_t b) { return (int)((a + b - 1) / b); }
-int num_sms() {
-    int dev = 0, nsm = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0) nsm = 148;
-    return nsm;
-}
 inline bool width_ok(int D, int H) { return H > 0 && D % H == 0 && (D / H) % 32 == 0 && D / H <= GENERIC_MAX_DH; }
 
 bool plane_map(CUtensorMap *tm, const void *ptr, uint64_t inner, uint64_t rows, uint64_t planes, uint32_t box0, uint32_t box1) {
@@ -1013,7 +991,7 @@ bool plane_map(CUtensorMap *tm, const void *ptr, uint64_t inner, uint64_t rows, 
 // Fp32 calls and backwards of heads wider than 640 too: see forward().
 int fwd_tokens(int B, int T, int D, int H, bool exact) {
     const size_t blocks32 = (size_t)ceil_div(T, 32) * B * H * ceil_div(D / H, 128);
-    return blocks32 <= 148 || (exact && D / H > 640) ? 32 : 64;
+    return blocks32 <= (size_t)num_sms() || (exact && D / H > 640) ? 32 : 64;
 }
 
 template <typename IOT, bool SAVE, bool LATE, int TOK>
