@@ -160,7 +160,8 @@ __device__ __forceinline__ void walk_segment(Walk &k, f32x2 (&za)[4], f32x2 (&zx
 
 // The walk of a warp that ended in a NaN, once more, with the sums of the gates made term by term: an infinite factor is NaN in the
 // products of its planes, where a sum that ends in an infinity saturates its gate.  Slow (some hundred microseconds), and only for inputs
-// or weights that are not finite.  Out of line, so that it costs the walk that everybody takes no registers; leaves the step up to each
+// or weights that are not finite (B2 T777 D5632, nothing but NaN: 1.6 ms; one infinite weight in every
+// channel: 19; finite: 0.12).  Out of line, so that it costs the walk that everybody takes no registers; leaves the step up to each
 // segment (SAVE) in tensor memory, where the running steps go otherwise, and returns the whole one.
 template <typename IOT, bool SAVE, int TOK>
 __device__ __noinline__ float2 exact_walk(const SplitFwdArgs &p, uint32_t tm, int b, int head, int c, int t0, float s) {
@@ -198,6 +199,12 @@ __device__ __noinline__ float2 exact_walk(const SplitFwdArgs &p, uint32_t tm, in
             for (int i = 0; i < 4; ++i) {
                 za[i] = fma2(pack2(a, a), pack2(u[2 * i], u[2 * i + 1]), za[i]);
                 zx[i] = fma2(pack2(g, g), pack2(u[2 * i], u[2 * i + 1]), zx[i]);
+            }
+            if ((n & 15) == 0) {   // where the inputs themselves are NaN there is nothing to find out
+                bool nan = true;
+#pragma unroll
+                for (int i = 0; i < 4; ++i) nan = nan && za[i].x != za[i].x && za[i].y != za[i].y && zx[i].x != zx[i].x && zx[i].y != zx[i].y;
+                if (__all_sync(0xffffffffu, nan)) break;
             }
         }
         float xs[SEG];
