@@ -191,3 +191,29 @@ def test_backward_in_passes_over_the_sequences():
         else:
             want = sum(g[k].double() for g in parts)
             assert float((v.double() - want).norm() / want.norm()) < 2.0 ** -22, k
+
+
+def test_gates_of_the_split_forward_are_good_to_their_last_places():
+    """Zero gate weights, so that r and i are the sigmoids of the biases, and an impulse: y_0 = m i u, y_1 = a y_0, for every channel another
+    r, i and decay.  i, m and the decay rate are within 2 units in the last place (4 x 2^-24), the error of r and of the rate enters m by
+    half (4), and there are two products (2): 14 x 2^-24 for y_0, and as much again for a, which is 1/2 at least."""
+    import torch
+    from paper_2402_19427_b200 import binding
+    T, Dh, H = 160, 256, 16
+    D = Dh * H
+    p = synth.make_inputs(1, 1, D, H, io="f32", seed=2)["params"]
+    rng = np.random.default_rng(8)
+    for k in ("W_a", "W_x", "conv_w", "conv_b"):
+        p[k][:] = 0.0
+    p["conv_w"][0] = 1.0
+    p["b_a"][:], p["b_x"][:] = rng.uniform(-12, 12, D), rng.uniform(-12, 12, D)
+    a_c = np.where(rng.random(D) < 0.5, rng.uniform(0.5, 0.999, D), 1.0 - 10.0 ** rng.uniform(-6, -3, D))
+    p["lam"][:] = np.log(a_c ** 0.125 / (1.0 - a_c ** 0.125))
+    x = torch.zeros(1, T, D, device="cuda")
+    x[0, 0] = torch.from_numpy(rng.standard_normal(D)).float()
+    y = to_np(binding.prefill(x, binding.Params.from_numpy(p, "f32"))[0])[0]
+    b_a, b_x, lam, u = p["b_a"].astype(np.float64), p["b_x"].astype(np.float64), p["lam"].astype(np.float64), to_np(x)[0, 0]
+    L = 8.0 * np.log1p(np.exp(-lam)) / (1.0 + np.exp(-b_a))
+    y0 = np.sqrt(-np.expm1(-2.0 * L)) * u / (1.0 + np.exp(-b_x))
+    assert (np.abs(y[0] - y0) / np.abs(y0)).max() <= 14 * 2.0 ** -24
+    assert (np.abs(y[1] - np.exp(-L) * y0) / np.abs(np.exp(-L) * y0)).max() <= 28 * 2.0 ** -24
