@@ -31,13 +31,14 @@
  *    replayed: the replay looks for the records that the failed run left incomplete.
  *  - Shapes without a kernel return RGLRU_ERR_UNSUPPORTED.  There is no CPU fallback.
  *  - Kernels.  Head widths D_h that are multiples of 32, up to 1024, run on tensor-core kernels: prefill and backward at any such
- *    width, fp32 or bf16, the decode step of bf16 up to 256.  Section 4.1 fixes 16 blocks, so D_h is 256 only at D_RNN = 4096; it is 96
+ *    width, fp32 or bf16 (but the fp32 prefill of few tokens on CUDA cores), the decode step of bf16 up to 256.  Section 4.1 fixes 16 blocks, so D_h is 256 only at D_RNN = 4096; it is 96
  *    at D_RNN = 1536, 128 at 2048 and 160 at 2560.  Narrower heads share, or occupy alone, groups of 256 channel slots whose
  *    weight tile is block-diagonal; the slots a width leaves unused are idle work.  Every other shape with D_h <= 1024
  *    runs on shape-generic CUDA-core kernels.
  *  - Precision.  State and sums are fp32 everywhere.  fp32 io, the prefill and backward of heads wider than 256, the backward when T is
  *    no multiple of 8, and the CUDA-core kernels keep fp32 between their parts (fp32 outputs within a few 1e-6 of the exact ones,
- *    relative 2-norm; their tensor-core products split fp32 operands into bf16 values that add up to them).  The other tensor-core
+ *    relative 2-norm; their tensor-core products split fp32 operands into bf16 values that add up to them, with no fp32 output
+ *    further from the exact one than on the CUDA cores).  The other tensor-core
  *    kernels use 16-bit operands: the prefill keeps the Conv1D output and the weights in fp16 (finite overflow saturates at 65504; h_T within 1e-4), the
  *    decode step in bf16, the backward its intermediates in fp16 and h_{t-1} in bf16 (parameter gradients within 5e-4).
  */
@@ -104,7 +105,9 @@ const char *rglru_status_string(int32_t status);
 /*
  * Device scratch needed by one call of `op` (rglru_op_t) on `shape`.  Host-only; returns 0
  * for an invalid or unsupported shape.  The value is at least 256 so that the status word
- * always has a home.
+ * always has a home.  The backward that is fp32 between its parts needs 30 bytes an element (B T D)
+ * up to 4 GiB, beyond that (with several sequences) about 16, which is what the CUDA-core kernels
+ * need (RGLRU_FLAG_FORCE_GENERIC).
  */
 size_t rglru_workspace_bytes(const rglru_shape_t *shape, int32_t op);
 

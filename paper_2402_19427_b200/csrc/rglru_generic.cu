@@ -1,6 +1,7 @@
 // Shape-generic CUDA-core kernels for the RG-LRU temporal core: any head width up to
 // GENERIC_MAX_DH, fp32 or bf16 io, accurate libm-grade transcendental functions, fp32 throughout.
-// They serve every shape without a tensor-core kernel: head widths that are no multiple of 32, and the decode step of fp32 io.
+// They serve every shape without a tensor-core kernel: head widths that are no multiple of 32, the decode step of fp32 io, and the fp32
+// prefill of few tokens.
 //
 // Every contraction (gate products W_a u, W_x u of Eq. 1-2; du = W^T dz; dW = dz^T u) is a register-blocked fp32 product on
 // packed FMAs: 128 threads own BM x 2 BM results, 2 TM NH = BM * BM / 64 each (64 for BM = 64), operands staged K-major

@@ -161,8 +161,8 @@ __device__ __forceinline__ void walk_segment(Walk &k, f32x2 (&za)[4], f32x2 (&zx
 // The walk of a warp that ended in a NaN, once more, with the sums of the gates made term by term: an infinite factor is NaN in the
 // products of its planes, where a sum that ends in an infinity saturates its gate.  Slow (some hundred microseconds), and only for inputs
 // or weights that are not finite (B2 T777 D5632, nothing but NaN: 1.6 ms; one infinite weight in every
-// channel: 19; finite: 0.12).  Out of line, so that it costs the walk that everybody takes no registers; leaves the step up to each
-// segment (SAVE) in tensor memory, where the running steps go otherwise, and returns the whole one.
+// channel: 19; finite: 0.12).  Out of line: the walk that everybody takes pays a vote and some 60 bytes of spills for it (backward of B5
+// T1021 D1536 in 16 heads 242.1 -> 245.5 us).  Leaves the step up to each segment (SAVE) in tensor memory, where the running steps go otherwise, and returns the whole one.
 template <typename IOT, bool SAVE, int TOK>
 __device__ __noinline__ float2 exact_walk(const SplitFwdArgs &p, uint32_t tm, int b, int head, int c, int t0, float s) {
     const FwdArgs &f = p.f;
@@ -615,7 +615,9 @@ __global__ void __launch_bounds__(FWD_THREADS, 2) split_forward_kernel(const __g
 //   dr = -s dL;  dz_a = dr r (1-r);  dz_x = di i (1-i);  dLambda += dL c r sigmoid(-Lambda).
 // Block = (chunk of 64 tokens, sequence, 64 channels): a thread holds eight tokens x two adjacent channels.  h_{t-1} is run again from
 // the state before the thread's tokens, u convolved again from x, so that 8 bytes of fp32 an element (r and i) are what the forward
-// leaves behind.
+// leaves behind.  At its 128 registers it spills some (56 and 68 bytes stored, 92 and 116 loaded, bf16 and fp32); with three blocks an SM
+// it spilled more and was slower (forward and backward of B4 T1024 D1024 in 4 heads 230 -> 243 us), and with dy read again after the chain
+// too (backward of B5 T1021 D1536 in 16 heads 242.6 -> 245.2).
 struct SplitRevArgs {
     BwdArgs q;
     const float *conv_b, *h_seg;
@@ -1043,9 +1045,10 @@ cudaError_t forward(SplitFwdArgs &p, int io, const void *wa, const void *wx, cud
     return wide ? launch_forward<__nv_bfloat16, SAVE, false, 64>(p, st) : launch_forward<__nv_bfloat16, SAVE, false, 32>(p, st);
 }
 
-// Token splits of dW: at least four K blocks each, at most `most` splits.  Up to 8192 tokens a split takes as long as a tile of du of a
-// 128-wide head; with more tokens it is longer, since the parts are memory.  (One split beside the 640 tiles of du of B5 T1021 D1536 in
-// 16 heads: 224 us, where the products take 96 now.)
+// Token splits of dW: at least four K blocks each, at most `most` splits.  Four blocks of six products are as long as a tile of du of an
+// fp32 head 128 wide; from 8192 tokens on a split is longer, since the parts are memory.  Neither the SMs nor the number of dW tiles
+// enter: one narrow head leaves most SMs without one.  (One split beside the 640 tiles of du of B5 T1021 D1536 in 16 heads: 224 us, where
+// the products take 61 now.)
 int dw_split(size_t ntok, int most, int &kb_split) {
     const int total = ceil_div(ntok, 64);
     kb_split = ceil_div(total, most) > 4 ? ceil_div(total, most) : 4;
