@@ -160,9 +160,10 @@ __device__ __forceinline__ void walk_segment(Walk &k, f32x2 (&za)[4], f32x2 (&zx
 
 // The walk of a warp that ended in a NaN, once more, with the sums of the gates made term by term: an infinite factor is NaN in the
 // products of its planes, where a sum that ends in an infinity saturates its gate.  Slow (some hundred microseconds), and only for inputs
-// or weights that are not finite (B2 T777 D5632, nothing but NaN: 1.6 ms; one infinite weight in every
-// channel: 19; finite: 0.12).  Out of line: the walk that everybody takes pays a vote and some 60 bytes of spills for it (backward of B5
-// T1021 D1536 in 16 heads 242.1 -> 245.5 us).  Leaves the step up to each segment (SAVE) in tensor memory, where the running steps go otherwise, and returns the whole one.
+// or weights that are not finite (every walk of B2 T777 D5632 made again: 19 ms; nothing but NaN, where the sums end at once: 1.6; finite:
+// 0.12).  Out of line: the walk that everybody takes pays a vote and some 60 bytes of spills for it (backward of B5 T1021 D1536 in 16
+// heads 242.1 -> 245.5 us).  Leaves the step up to each segment (SAVE) in tensor memory, where the running steps go otherwise, and returns
+// the whole one.
 template <typename IOT, bool SAVE, int TOK>
 __device__ __noinline__ float2 exact_walk(const SplitFwdArgs &p, uint32_t tm, int b, int head, int c, int t0, float s) {
     const FwdArgs &f = p.f;
